@@ -34,6 +34,8 @@ struct ScratchLayout {
   int64_t Kp;            // reduction length rounded up to the k-block of the kernel
   int64_t Co_pad;        // Co rounded up to the filter tile of the kernel
   size_t koff_off, filter_off, total;
+  size_t ffma_total;     // fp32 only: what the FFMA kernel alone needs
+  bool f32_split;        // fp32 only: the tensor-core kernel is used (filter images right after the status block)
   bool f16_shift;        // fp16 only: a shifted-view kernel (and its filter layout) is used
   bool f16_raw;          // fp16 only: the bulk-copy variant of the shifted-view kernel is used
   bool f16_mat;          // fp16 only: the matrix-transpose variant is used (own scratch layout)
@@ -117,6 +119,18 @@ struct F32Plan {
 };
 F32Plan plan_f32(const Geometry& g);
 
+// Tile shape of the fp32 kernel that runs on the tensor cores (see conv_f32_split.cu).
+struct F32SplitPlan {
+  bool eligible;
+  int32_t Wq, rows, halo, nsub, num_kb, nks_last, nstages;
+  int32_t bn, ntn, split, sb, nwork;   // channel tile and their number, CTAs per tile, filter slots, tiles
+  int32_t packed_rows;                 // most rows (ntn * bn) of any tile width: the filter area does not depend on N
+  int64_t VQ;
+  size_t filter_bytes;
+  double cost;                         // cycles, estimated
+};
+F32SplitPlan plan_f32_split(const Geometry& g);
+
 // Environment switches are testing aids: they are looked at only when IM2WIN_DEBUG is set in the
 // environment (checked once per process), so the default call path reads no environment.
 const char* debug_getenv(const char* name);
@@ -137,6 +151,8 @@ cudaError_t launch_pack_f16(const uint16_t* filter, void* scratch, const Geometr
                             const ScratchLayout& l, cudaStream_t stream);
 cudaError_t launch_conv_f32(const float* window, float* y, const void* scratch, const Geometry& g,
                             const ScratchLayout& l, cudaStream_t stream);
+cudaError_t launch_pack_f32_split(const float* filter, void* scratch, const Geometry& g, cudaStream_t stream);
+cudaError_t launch_conv_f32_split(const float* window, float* y, void* scratch, const Geometry& g, cudaStream_t stream);
 cudaError_t launch_pack_f16_shift(const uint16_t* filter, void* scratch, const Geometry& g,
                                   const ScratchLayout& l, cudaStream_t stream);
 cudaError_t launch_pack_f16_raw(const uint16_t* filter, void* scratch, const Geometry& g,

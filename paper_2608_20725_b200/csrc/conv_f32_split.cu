@@ -1,0 +1,746 @@
+// fp32 im2win convolution on the tensor cores: every fp32 operand is the exact sum of three bf16
+// pieces, and six bf16 products per term reproduce the fp32 product.
+//
+//     x = x1 + x2 + x3,  x1 = bf16(x), x2 = bf16(x - x1), x3 = x - x1 - x2        (24 = 8 + 8 + 8 bits)
+//     x w ~ x1 w1 + (x1 w2 + x2 w1) + (x1 w3 + x2 w2 + x3 w1)
+//
+// The three products left out are below 2^-26 |x w|.  What decides the accuracy is the accumulator: the
+// tensor core aligns the addends of an instruction to the largest one, cuts them two bits below fp32's
+// last and truncates the sum (measured), so a long chain in one accumulator drifts towards zero.  A chain
+// here is therefore short: the products of 64 k2 of one kernel column (a "unit") go into a fresh
+// accumulator, the small products first, and the epilogue warps add it to fp32 registers with rounded adds.
+// Error against 64 bits, relative 2-norm (round-to-nearest FFMA chain -> this kernel): K = 147 2.2e-7 ->
+// 0.8e-7, K = 576 4.3e-7 -> 1.0e-7, K = 4608 1.2e-6 -> 1.8e-7, on inputs of both signs and of one.
+// Values whose pieces or sums leave the finite range give a non-finite accumulator; such outputs (and
+// those below 2^-90, where pieces get lost under bf16's smallest value) are computed again with fp32 FMAs in
+// the order of the FFMA kernel (exact_output).
+//
+// The GEMM is the shifted-view one of conv_f16_shift.cu: the window tensor's columns are staged once,
+//     S[piece][row = virtual column q][k2 = c*Kh + u]     (64 k2 = 128 bytes per row, 128-byte swizzle),
+// and kernel column v multiplies the view that starts (v div s) rows further down; with stride s a stage
+// holds one column class t = v mod s.  Rows are the virtual positions q = (n*Ho + ho)*Wq + i, Wq = ceil(Wp/s).
+//
+// What bounds it: the tensor pipe, and next to it the shared-memory pipe the MMA reads its operands
+// through: an instruction of M = 128, K = 16 takes max(N/2, 32 + N/4) cycles.  Up to 80 channels the filter
+// pieces therefore lie side by side as one operand, [w1 | w2 | w3], and three instructions replace six
+// (x1 against all of it, x2 against [w1 | w2], x3 against w1, into three accumulators of one magnitude each).
+//
+// Roles (one persistent CTA per SM): one or two warpgroups of producers (thread = row; 32 loads in flight,
+// split, 16-byte stores), an MMA warp, a filter-copy warp (one untiled bulk copy per piece: the pack kernel
+// writes shared-memory images), eight epilogue warps that keep the tile's fp32 sums in registers.
+// A layer with few tiles is run by clusters of 2, 4 or 8 CTAs that share the stages of a tile and add their
+// registers through distributed shared memory, in rank order.
+#include <cuda_bf16.h>
+#include <stdlib.h>
+#include <string.h>
+
+#define IM2WIN_INLINE_SLOW_WAIT      // (a call cannot be compiled beside the 128 live sums of the epilogue warps)
+#include "common.cuh"
+#include "ptx_sm100.cuh"
+
+namespace im2win {
+namespace {
+
+using namespace ptx;
+
+constexpr int TILE_M = 128;
+constexpr int KB = 64;
+constexpr int A_STAGES = 2;
+constexpr int MAX_B = 16;
+constexpr int MAX_ACC = 4;
+constexpr int kSplitSmem = 226 * 1024;        // dynamic shared memory a CTA may use
+
+struct SplitParams {
+  const float* __restrict__ win;
+  const unsigned char* __restrict__ fp;       // packed filter: shared-memory images, see pack_f32_split_kernel
+  float* __restrict__ y;
+  uint32_t* status;
+  int64_t img_stride, strip, chan_stride;
+  uint32_t VQ;
+  int32_t K2, C, Wq, Wp, Ho, Wo, HoWo, Co, Kh, Kw, s, nsub, num_kb, nks_last;
+  int32_t rows, halo;                         // rows of a sub-tile (128 + halo rounded up to 8), halo
+  int32_t bn, ntn, nwork, nstages, split, sb, slot_bytes;
+};
+
+__device__ __forceinline__ void wait_for_previous_kernel() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+__device__ __forceinline__ float ld_if(const float* p, bool ok) {
+  float v = 0.f;
+  asm("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %2, 0;\n\t@p ld.global.nc.f32 %0, [%1];\n\t}"
+      : "+f"(v)
+      : "l"(p), "r"((int)ok));
+  return v;
+}
+__device__ __forceinline__ uint32_t cvt_bf16x2(float lo, float hi) {
+  uint32_t r;
+  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
+  return r;
+}
+// Two values -> their three pieces, packed (first value in the low half).
+__device__ __forceinline__ void split2(float a, float b, uint32_t& p1, uint32_t& p2, uint32_t& p3) {
+  p1 = cvt_bf16x2(a, b);
+  const float ra = a - __uint_as_float(p1 << 16), rb = b - __uint_as_float(p1 & 0xffff0000u);
+  p2 = cvt_bf16x2(ra, rb);
+  p3 = cvt_bf16x2(ra - __uint_as_float(p2 << 16), rb - __uint_as_float(p2 & 0xffff0000u));
+}
+__device__ __forceinline__ void st_shared16(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+  asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
+}
+__device__ __forceinline__ void tmem_ld16_issue(uint32_t taddr, uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr)
+      : "memory");
+}
+// The wait for loads into r[]: naming the registers keeps every use of them after it.
+__device__ __forceinline__ void tmem_wait16(uint32_t (&r)[16]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                 "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
+               :
+               : "memory");
+}
+__device__ __forceinline__ float ld_cluster(uint32_t addr) {
+  float v;
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
+  return v;
+}
+// bf16 operands, fp32 accumulator, both k-major.
+__host__ __device__ constexpr uint32_t instr_desc_bf16(int M, int N) {
+  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+}
+
+// An output that has to be computed again: not finite, or so small that pieces of its terms were lost.
+__device__ __forceinline__ bool suspicious(float v) {
+  const uint32_t u = __float_as_uint(v) << 1, lo = (uint32_t)(127 - 90) << 24;
+  return u != 0u && u - lo >= 0xff000000u - lo;
+}
+
+// v[e] -> base[e * stride] for e < count, over two address chains.
+__device__ __forceinline__ void store16(float* base, int stride, const float (&v)[16], int count, bool& again) {
+  float *p0 = base, *p1 = base + stride;
+  const int64_t step = 2 * (int64_t)stride;
+#pragma unroll
+  for (int e = 0; e < 16; e += 2) {
+    if (e < count) { *p0 = v[e]; again |= suspicious(v[e]); }
+    if (e + 1 < count) { *p1 = v[e + 1]; again |= suspicious(v[e + 1]); }
+    p0 += step; p1 += step;
+  }
+}
+
+template <int BNMAX> struct Form {
+  static constexpr bool CONCAT = BNMAX == 80;             // the filter pieces side by side in one operand
+  static constexpr int ACC_COLS = BNMAX == 128 ? 128 : 256;
+  static constexpr int NACC = 512 / ACC_COLS;
+  static constexpr int CH = BNMAX == 80 ? 3 : BNMAX / 32; // 16-channel chunks per epilogue warp
+  static constexpr int PWG = BNMAX == 256 ? 1 : 2;        // producer warpgroups
+  static constexpr int THREADS = 128 * (PWG + 3);
+  static constexpr int REGS_PRODUCER = 96;
+  static constexpr int REGS_MISC = 64;
+  static constexpr int REGS_EPILOGUE = BNMAX == 256 ? 176 : 112;
+  // (the launch holds 128 or 96 registers a thread: 96 + 64 + 2*176 = 4*128, 2*96 + 64 + 2*112 = 5*96)
+};
+
+// One output in fp32 FMAs, k ascending, for the values the split cannot hold.  The filter element is the sum of
+// its pieces (exact: the pack kernel keeps them finite for finite elements).
+__device__ __forceinline__ float exact_output(const SplitParams& q, bool concat, uint32_t n, int ho, int wo, int nt, int col) {
+  const float* wbase = q.win + (int64_t)n * q.img_stride + (int64_t)ho * q.strip + (int64_t)wo * q.s * q.Kh;
+  const unsigned char* frow = q.fp + (int64_t)nt * q.num_kb * q.Kw * 3 * q.bn * 128 + col * 128;
+  const int64_t piece = (int64_t)q.bn * 128;
+  float acc = 0.f;
+  for (int c = 0; c < q.C; ++c)
+    for (int v = 0; v < q.Kw; ++v)
+      for (int u = 0; u < q.Kh; ++u) {
+        const int k2 = c * q.Kh + u, kb = k2 / KB, e = k2 - kb * KB;
+        const unsigned char* f = frow + ((int64_t)kb * q.Kw + v) * 3 * piece + ((((e >> 3) ^ (col & 7)) << 4) | ((e & 7) * 2));
+        auto part = [&](int p) {
+          return __uint_as_float((uint32_t)*reinterpret_cast<const uint16_t*>(f + (concat ? p : 2 - p) * piece) << 16);
+        };
+        acc = fmaf(wbase[(int64_t)c * q.chan_stride + v * q.Kh + u], (part(0) + part(1)) + part(2), acc);
+      }
+  return acc;
+}
+
+template <int BNMAX>
+__global__ void __launch_bounds__(Form<BNMAX>::THREADS, 1) conv_f32_split_kernel(SplitParams q) {
+  using F = Form<BNMAX>;
+  extern __shared__ unsigned char smem_dyn[];
+  unsigned char* smem = reinterpret_cast<unsigned char*>(((uintptr_t)smem_dyn + 1023) & ~(uintptr_t)1023);
+  __shared__ __align__(8) uint64_t bars[2 * A_STAGES + 2 * MAX_B + 2 * MAX_ACC];
+  __shared__ uint32_t tmem_base_slot;
+  __shared__ volatile uint32_t abort_flag;
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int wg = warp >> 2;
+  const int sub_bytes = q.rows * 128, a_stage_bytes = 3 * sub_bytes;
+  const uint32_t a_ring = smem_u32(smem);
+  const uint32_t b_ring = a_ring + A_STAGES * a_stage_bytes;
+  const uint32_t a_full0 = smem_u32(&bars[0]), a_empty0 = a_full0 + 8 * A_STAGES;
+  const uint32_t b_full0 = a_empty0 + 8 * A_STAGES, b_empty0 = b_full0 + 8 * MAX_B;
+  const uint32_t acc_full0 = b_empty0 + 8 * MAX_B, acc_empty0 = acc_full0 + 8 * MAX_ACC;
+  int32_t* koff_s = reinterpret_cast<int32_t*>(smem + A_STAGES * a_stage_bytes + q.sb * q.slot_bytes);
+
+  if (threadIdx.x == 0) {
+    abort_flag = 0u;
+    for (int i = 0; i < A_STAGES; ++i) { mbar_init(a_full0 + 8 * i, 4); mbar_init(a_empty0 + 8 * i, 1); }
+    for (int i = 0; i < MAX_B; ++i) { mbar_init(b_full0 + 8 * i, 1); mbar_init(b_empty0 + 8 * i, 1); }
+    for (int i = 0; i < MAX_ACC; ++i) { mbar_init(acc_full0 + 8 * i, 1); mbar_init(acc_empty0 + 8 * i, 8); }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == F::PWG * 4 + 2) tmem_alloc(smem_u32(&tmem_base_slot), 512);
+  // k2 -> element offset inside the image (channel plane and row of the kernel), -1 for padded k2
+  for (int i = threadIdx.x; i < q.num_kb * KB; i += F::THREADS) {
+    const int c = i / q.Kh;
+    koff_s[i] = i < q.K2 ? (int32_t)(c * q.chan_stride + (i - c * q.Kh)) : -1;
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_acc = tmem_base_slot;
+  wait_for_previous_kernel();
+
+  // Work: tile w = position tile * channel tiles + channel tile.  split = 1: the CTA walks tiles w, w + grid, ...;
+  // otherwise the cluster has one tile and its CTA r the stages [S r / split, S (r + 1) / split).
+  const int rank = q.split > 1 ? (int)cluster_ctarank() : 0;
+  const int w_first = q.split > 1 ? (int)blockIdx.x / q.split : (int)blockIdx.x;
+  const int w_step = q.split > 1 ? q.nwork : (int)gridDim.x;
+  const int st0 = (int)((int64_t)q.nstages * rank / q.split), st1 = (int)((int64_t)q.nstages * (rank + 1) / q.split);
+  const int kb0 = st0 / q.nsub, t0 = st0 - kb0 * q.nsub;
+
+  if (wg < F::PWG) {
+    // ---------------- producers: thread = row ------------------------------------------------------
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(F::REGS_PRODUCER));
+    const int tid = threadIdx.x & 127;
+    bool ok = true;
+    uint32_t sc = 0;                                       // stages so far, of all producers
+    for (int w = w_first; w < q.nwork && ok; w += w_step) {
+      const uint32_t q0 = (uint32_t)(w / q.ntn) * TILE_M;
+      // Row -> window column (class 0) and the number of classes that exist there (0 beyond the tensor).
+      auto locate = [&](uint32_t vq, const float*& base, int& lim) {
+        base = q.win;
+        lim = 0;
+        if (vq < q.VQ) {
+          const uint32_t sg = vq / (uint32_t)q.Wq;
+          const int i = (int)(vq - sg * (uint32_t)q.Wq);
+          const uint32_t n = sg / (uint32_t)q.Ho;
+          const int ho = (int)(sg - n * (uint32_t)q.Ho);
+          base += (int64_t)n * q.img_stride + (int64_t)ho * q.strip + (int64_t)i * q.s * q.Kh;
+          lim = q.Wp - i * q.s;
+        }
+      };
+      const float *base, *hbase = q.win;
+      int lim, hlim = 0;
+      locate(q0 + tid, base, lim);
+      const int hrow = TILE_M + (tid >> 3), hch = tid & 7;  // halo item: a row below the tile, one chunk of it
+      const bool has_halo = tid < q.halo * 8;
+      if (has_halo) locate(q0 + hrow, hbase, hlim);
+      int kb = kb0, t = t0;
+      for (int st = st0; st < st1; ++st, ++sc) {
+        if (F::PWG == 1 || (int)(sc & 1) == wg) {
+          const int buf = sc & 1;
+          const uint32_t stage = a_ring + buf * a_stage_bytes;
+          const int nch = kb == q.num_kb - 1 ? 2 * q.nks_last : 8;      // the MMAs stop at the last step with real k2
+          const int4* kt = reinterpret_cast<const int4*>(koff_s + kb * KB);
+          auto load8 = [&](const float* src, bool row_ok, int ch, float (&v)[8]) {
+            const int4 o0 = kt[2 * ch], o1 = kt[2 * ch + 1];
+            const int32_t off[8] = {o0.x, o0.y, o0.z, o0.w, o1.x, o1.y, o1.z, o1.w};
+#pragma unroll
+            for (int e = 0; e < 8; ++e) v[e] = ld_if(src + off[e], row_ok && off[e] >= 0);
+          };
+          auto store8 = [&](int row, int ch, const float (&v)[8]) {
+            uint32_t p[3][4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) split2(v[2 * e], v[2 * e + 1], p[0][e], p[1][e], p[2][e]);
+            const uint32_t dst = stage + row * 128 + ((ch ^ (row & 7)) << 4);
+#pragma unroll
+            for (int i = 0; i < 3; ++i) st_shared16(dst + i * sub_bytes, p[i][0], p[i][1], p[i][2], p[i][3]);
+          };
+          const bool row_ok = t < lim;
+          const float* src = base + t * q.Kh;
+          float v[4][8], hv[8];
+#pragma unroll
+          for (int c = 0; c < 4; ++c) load8(src, row_ok && c < nch, c, v[c]);
+          const bool halo_now = has_halo && hch < nch;
+          if (halo_now) load8(hbase + t * q.Kh, t < hlim, hch, hv);
+          ok = mbar_wait(a_empty0 + 8 * buf, ((sc >> 1) & 1) ^ 1, &abort_flag, q.status);
+          ok = __all_sync(0xffffffffu, ok);
+          if (!ok) break;
+#pragma unroll
+          for (int c = 0; c < 4; ++c) if (c < nch) store8(tid, c, v[c]);
+          if (halo_now) store8(hrow, hch, hv);
+          if (nch > 4) {
+#pragma unroll
+            for (int c = 0; c < 4; ++c) load8(src, row_ok && 4 + c < nch, 4 + c, v[c]);
+#pragma unroll
+            for (int c = 0; c < 4; ++c) if (4 + c < nch) store8(tid, 4 + c, v[c]);
+          }
+          fence_proxy_async_smem();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(a_full0 + 8 * buf);
+        }
+        if (++t == q.nsub) { t = 0; ++kb; }
+      }
+    }
+  } else if (wg == F::PWG) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(F::REGS_MISC));
+    if ((warp & 3) == 0) {
+      // ---------------- MMA issuer -----------------------------------------------------------------
+      const bool leader = elect_one();
+      const uint32_t a_lo0 = smem_desc_lo(a_ring), b_lo0 = smem_desc_lo(b_ring);
+      const uint32_t sub_lo = (uint32_t)sub_bytes >> 4, bn_lo = (uint32_t)q.bn * 8;
+      const uint32_t id1 = instr_desc_bf16(TILE_M, q.bn), id2 = instr_desc_bf16(TILE_M, 2 * q.bn),
+                     id3 = instr_desc_bf16(TILE_M, 3 * q.bn);
+      bool ok = true;
+      uint32_t sc = 0, ac = 0;                             // stages and units so far
+      int slot = 0;
+      uint32_t bph = 0;
+      for (int w = w_first; w < q.nwork && ok; w += w_step) {
+        int kb = kb0, t = t0;
+        for (int st = st0; st < st1 && ok; ++st, ++sc) {
+          const int buf = sc & 1;
+          const int nks = kb == q.num_kb - 1 ? q.nks_last : KB / 16;
+          ok = mbar_wait(a_full0 + 8 * buf, (sc >> 1) & 1, &abort_flag, q.status);
+          ok = __all_sync(0xffffffffu, ok);
+          if (!ok) break;
+          uint32_t a_view = a_lo0 + (uint32_t)(buf * (a_stage_bytes >> 4));
+          for (int v = t; v < q.Kw; v += q.s, a_view += 8u, ++ac) {     // next view: one row (128 bytes) further down
+            const int ab = ac % F::NACC;
+            ok = mbar_wait(acc_empty0 + 8 * ab, ((ac / F::NACC) & 1) ^ 1, &abort_flag, q.status);
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok) break;
+            const uint32_t d = tmem_acc + ab * F::ACC_COLS;
+            if constexpr (F::CONCAT) {
+              ok = mbar_wait(b_full0 + 8 * slot, bph, &abort_flag, q.status);
+              ok = __all_sync(0xffffffffu, ok);
+              if (!ok) break;
+              tc_fence_after();
+              const uint32_t b_lo = b_lo0 + (uint32_t)(slot * (q.slot_bytes >> 4));
+              if (leader) {
+#pragma unroll
+                for (int j = 0; j < KB / 16; ++j)
+                  if (j < nks) umma_f16_lohi(d, a_view + 2 * j, b_lo + 2 * j, id3, (uint32_t)j);
+#pragma unroll
+                for (int j = 0; j < KB / 16; ++j)
+                  if (j < nks) umma_f16_lohi(d + q.bn, a_view + sub_lo + 2 * j, b_lo + 2 * j, id2, 1u);
+#pragma unroll
+                for (int j = 0; j < KB / 16; ++j)
+                  if (j < nks) umma_f16_lohi(d + 2 * q.bn, a_view + 2 * sub_lo + 2 * j, b_lo + 2 * j, id1, 1u);
+                umma_commit(b_empty0 + 8 * slot);
+              }
+              __syncwarp();
+              if (++slot == q.sb) { slot = 0; bph ^= 1u; }
+            } else {
+              // filter pieces arrive smallest first: w3 meets x1, w2 meets x2 and x1, w1 meets x3, x2 and x1
+#pragma unroll
+              for (int p = 0; p < 3; ++p) {
+                ok = mbar_wait(b_full0 + 8 * slot, bph, &abort_flag, q.status);
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) break;
+                tc_fence_after();
+                const uint32_t b_lo = b_lo0 + (uint32_t)(slot * (q.slot_bytes >> 4));
+                if (leader) {
+#pragma unroll
+                  for (int i = p; i >= 0; --i)
+#pragma unroll
+                    for (int j = 0; j < KB / 16; ++j)
+                      if (j < nks) umma_f16_lohi(d, a_view + i * sub_lo + 2 * j, b_lo + 2 * j, id1, (uint32_t)(p | j));
+                  umma_commit(b_empty0 + 8 * slot);
+                }
+                __syncwarp();
+                if (++slot == q.sb) { slot = 0; bph ^= 1u; }
+              }
+              if (!ok) break;
+            }
+            if (leader) umma_commit(acc_full0 + 8 * ab);
+            __syncwarp();
+          }
+          if (ok && leader) umma_commit(a_empty0 + 8 * buf);
+          __syncwarp();
+          if (++t == q.nsub) { t = 0; ++kb; }
+        }
+      }
+      (void)id2; (void)id3; (void)bn_lo;
+    } else if ((warp & 3) == 1) {
+      // ---------------- filter copies ----------------------------------------------------------------
+      const bool leader = elect_one();
+      bool ok = true;
+      int slot = 0;
+      uint32_t bph = 0;
+      const int per_unit = F::CONCAT ? 1 : 3;
+      for (int w = w_first; w < q.nwork && ok; w += w_step) {
+        const int nt = w % q.ntn;
+        const unsigned char* tile = q.fp + (int64_t)nt * q.num_kb * q.Kw * 3 * q.bn * 128;
+        int kb = kb0, t = t0;
+        for (int st = st0; st < st1 && ok; ++st) {
+          for (int v = t; v < q.Kw && ok; v += q.s) {
+            const unsigned char* src = tile + ((int64_t)kb * q.Kw + v) * 3 * q.bn * 128;
+            for (int p = 0; p < per_unit; ++p) {
+              ok = mbar_wait(b_empty0 + 8 * slot, bph ^ 1u, &abort_flag, q.status);
+              ok = __all_sync(0xffffffffu, ok);
+              if (!ok) break;
+              if (leader) {
+                mbar_arrive_expect_tx(b_full0 + 8 * slot, (uint32_t)q.slot_bytes);
+                bulk_load(b_ring + slot * q.slot_bytes, src + (int64_t)p * q.slot_bytes, (uint32_t)q.slot_bytes,
+                          b_full0 + 8 * slot);
+              }
+              __syncwarp();
+              if (++slot == q.sb) { slot = 0; bph ^= 1u; }
+            }
+          }
+          if (++t == q.nsub) { t = 0; ++kb; }
+        }
+      }
+      // copies in flight must land before the CTA gives its shared memory back (only after a wait that gave up)
+      if (!ok) for (int i = 0; i < 64; ++i) __nanosleep(1000);
+    }
+    __syncwarp();
+    if (q.split > 1) { cluster_sync_all(); cluster_sync_all(); }
+  } else {
+    // ---------------- epilogue: fp32 sums of the tile in registers -------------------------------------
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(F::REGS_EPILOGUE));
+    const int lq = warp & 3, h = (wg - F::PWG - 1);         // tensor-memory quadrant; which chunks of 16 channels
+    bool ok = true;
+    uint32_t ac = 0;
+    float acc[F::CH][16];
+    uint32_t n = 0;
+    int ho = 0, i0 = 0, nt = 0;
+    bool valid = false;
+    for (int w = w_first; w < q.nwork && ok; w += w_step) {
+      const int mt = w / q.ntn;
+      nt = w - mt * q.ntn;
+      const uint32_t vq = (uint32_t)mt * TILE_M + (uint32_t)(lq * 32 + lane);
+      valid = false;
+      if (vq < q.VQ) {
+        const uint32_t sg = vq / (uint32_t)q.Wq;
+        i0 = (int)(vq - sg * (uint32_t)q.Wq);
+        n = sg / (uint32_t)q.Ho;
+        ho = (int)(sg - n * (uint32_t)q.Ho);
+        valid = i0 < q.Wo;                                  // trailing columns of a strip are no output
+      }
+#pragma unroll
+      for (int j = 0; j < F::CH; ++j)
+#pragma unroll
+        for (int e = 0; e < 16; ++e) acc[j][e] = 0.f;
+      int t = t0;
+      for (int st = st0; st < st1 && ok; ++st) {
+        for (int v = t; v < q.Kw; v += q.s, ++ac) {
+          const int ab = ac % F::NACC;
+          ok = mbar_wait(acc_full0 + 8 * ab, (ac / F::NACC) & 1, &abort_flag, q.status);
+          ok = __all_sync(0xffffffffu, ok);
+          if (!ok) break;
+          tc_fence_after();
+          const uint32_t d = tmem_acc + ((uint32_t)(lq * 32) << 16) + ab * F::ACC_COLS + h * 16;
+          if constexpr (F::CONCAT) {
+#pragma unroll
+            for (int j = 0; j < F::CH; ++j) {
+              if ((h + 2 * j) * 16 >= q.bn) break;
+              uint32_t r0[16], r1[16], r2[16];
+              tmem_ld16_issue(d + 32 * j, r0);
+              tmem_ld16_issue(d + 32 * j + q.bn, r1);
+              tmem_ld16_issue(d + 32 * j + 2 * q.bn, r2);
+              tmem_wait16(r0);
+              tmem_wait16(r1);
+              tmem_wait16(r2);
+#pragma unroll
+              for (int e = 0; e < 16; ++e)
+                acc[j][e] += __uint_as_float(r0[e]) + (__uint_as_float(r1[e]) + __uint_as_float(r2[e]));
+            }
+          } else if constexpr (BNMAX == 256) {              // (one chunk in flight: 128 sums leave no more registers)
+#pragma unroll
+            for (int j = 0; j < F::CH; ++j) {
+              if ((h + 2 * j) * 16 >= q.bn) break;
+              uint32_t r0[16];
+              tmem_ld16_issue(d + 32 * j, r0);
+              tmem_wait16(r0);
+#pragma unroll
+              for (int e = 0; e < 16; ++e) acc[j][e] += __uint_as_float(r0[e]);
+            }
+          } else {
+#pragma unroll
+            for (int j = 0; j < F::CH; j += 2) {            // (columns beyond bn hold nothing and are not stored)
+              if ((h + 2 * j) * 16 >= q.bn) break;
+              uint32_t r0[16], r1[16];
+              tmem_ld16_issue(d + 32 * j, r0);
+              tmem_ld16_issue(d + 32 * j + 32, r1);
+              tmem_wait16(r0);
+              tmem_wait16(r1);
+#pragma unroll
+              for (int e = 0; e < 16; ++e) {
+                acc[j][e] += __uint_as_float(r0[e]);
+                acc[j + 1][e] += __uint_as_float(r1[e]);
+              }
+            }
+          }
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(acc_empty0 + 8 * ab);
+        }
+        if (++t == q.nsub) t = 0;
+      }
+      if (!ok || q.split > 1) break;
+      if (valid) {
+        const int co0 = nt * q.bn;
+        float* yrow = q.y + ((int64_t)n * q.Co + co0) * q.HoWo + (int64_t)ho * q.Wo + i0;
+        const int limit = q.Co - co0 < q.bn ? q.Co - co0 : q.bn;        // channels of this tile that exist
+        bool again = false;
+#pragma unroll
+        for (int j = 0; j < F::CH; ++j) {
+          const int c0 = (h + 2 * j) * 16;
+          store16(yrow + (int64_t)c0 * q.HoWo, q.HoWo, acc[j], limit - c0, again);
+        }
+        if (again) {
+          for (int c = h * 16; c < limit; c += (c & 15) == 15 ? 17 : 1)
+            if (suspicious(yrow[(int64_t)c * q.HoWo])) yrow[(int64_t)c * q.HoWo] = exact_output(q, F::CONCAT, n, ho, i0, nt, c);
+        }
+      }
+    }
+    if (q.split > 1) {
+      // All MMAs of this CTA have completed, so its rings are free: partial sums as P[channel][row], 4 bytes.
+      if (ok) {
+        float* part = reinterpret_cast<float*>(smem);
+#pragma unroll
+        for (int j = 0; j < F::CH; ++j)
+#pragma unroll
+          for (int e = 0; e < 16; ++e) {
+            const int c = (h + 2 * j) * 16 + e;
+            if (c < q.bn) part[c * TILE_M + lq * 32 + lane] = acc[j][e];
+          }
+      }
+      __syncwarp();
+      cluster_sync_all();
+      if (ok && valid) {
+        const int co0 = nt * q.bn;
+        const int limit = q.Co - co0 < q.bn ? q.Co - co0 : q.bn;
+        float* yrow = q.y + ((int64_t)n * q.Co + co0) * q.HoWo + (int64_t)ho * q.Wo + i0;
+        const int per = q.bn / q.split;                     // channels this CTA finishes (bn is a multiple of 16)
+        uint32_t peer[8];
+#pragma unroll
+        for (int r = 0; r < 8; ++r) peer[r] = mapa_shared(a_ring + (lq * 32 + lane) * 4, r < q.split ? r : 0);
+        for (int c = rank * per + h; c < (rank + 1) * per && c < limit; c += 2) {
+          float v[8];
+#pragma unroll
+          for (int r = 0; r < 8; ++r) v[r] = r < q.split ? ld_cluster(peer[r] + c * (TILE_M * 4)) : 0.f;
+          float sum = v[0];
+#pragma unroll
+          for (int r = 1; r < 8; ++r) sum += v[r];
+          if (suspicious(sum)) sum = exact_output(q, F::CONCAT, n, ho, i0, nt, c);
+          yrow[(int64_t)c * q.HoWo] = sum;
+        }
+      }
+      __syncwarp();
+      cluster_sync_all();
+    }
+  }
+  if (wg < F::PWG && q.split > 1) {
+    __syncwarp();
+    cluster_sync_all();
+    cluster_sync_all();
+  }
+
+  // ---------------- teardown -----------------------------------------------------------------------
+  tc_fence_before();
+  __syncthreads();
+  if (abort_flag) {
+    for (int i = 0; i < 64; ++i) __nanosleep(1000);
+    __syncthreads();
+  }
+  if (warp == F::PWG * 4 + 2) {
+    __syncwarp();
+    tc_fence_after();
+    tmem_dealloc(tmem_acc, 512);
+  }
+}
+
+// Filter -> the images the copy warp loads: for every (channel tile nt, k2-block kb, kernel column v) the three
+// pieces [bn channels][64 k2] in the 128-byte-swizzled order of shared memory, smallest first, or largest first
+// where they form one operand (bn <= 80).  One block: `rows` channels of one k2-block; its source is one
+// contiguous run of the OIHW filter per channel.  Channels beyond Co and k2 beyond C*Kh are zeros.
+__global__ void __launch_bounds__(256) pack_f32_split_kernel(const float* __restrict__ f, unsigned char* __restrict__ fp,
+                                                             uint32_t* __restrict__ status, int K2, int Kw, int Co, int bn,
+                                                             int num_kb, int rows, int concat) {
+  extern __shared__ float pack_f[];
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < kStatusBytes / 4) status[threadIdx.x] = 0u;
+  const int kb = blockIdx.x, row0 = blockIdx.y * rows;
+  const int nreal = K2 - kb * KB < KB ? K2 - kb * KB : KB;
+  const int run = nreal * Kw, pitch = KB * Kw;
+  for (int r = 0; r < rows; ++r) {
+    const int co = row0 + r;
+    const float* src = f + ((int64_t)co * K2 + (int64_t)kb * KB) * Kw;
+    for (int i = threadIdx.x; i < pitch; i += blockDim.x) pack_f[r * pitch + i] = (co < Co && i < run) ? __ldg(src + i) : 0.f;
+  }
+  __syncthreads();
+  const int items = rows * Kw * 8;
+  for (int it = threadIdx.x; it < items; it += blockDim.x) {
+    const int ch = it & 7, rv = it >> 3;
+    const int r = rv % rows, v = rv / rows;
+    const int row = row0 + r, nt = row / bn, rr = row - nt * bn;
+    const float* src = pack_f + r * pitch + ch * 8 * Kw + v;
+    uint32_t p[3][4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      float a[2] = {src[(2 * e) * Kw], src[(2 * e + 1) * Kw]};
+      uint32_t w[3] = {0u, 0u, 0u};
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        // The pieces of a finite element are finite (the first is cut where rounding would overflow); an
+        // infinity or NaN is its own first piece, the others are zero: the sum of the pieces is the element.
+        uint32_t b1 = cvt_bf16x2(a[k], 0.f) & 0xffffu, b2 = 0u, b3 = 0u;
+        const bool finite = (__float_as_uint(a[k]) & 0x7f800000u) != 0x7f800000u;
+        if (finite) {
+          if ((b1 & 0x7f80u) == 0x7f80u) b1 = __float_as_uint(a[k]) >> 16;
+          const float r1 = a[k] - __uint_as_float(b1 << 16);
+          b2 = cvt_bf16x2(r1, 0.f) & 0xffffu;
+          b3 = cvt_bf16x2(r1 - __uint_as_float(b2 << 16), 0.f) & 0xffffu;
+        }
+        w[0] |= b1 << (16 * k);
+        w[1] |= b2 << (16 * k);
+        w[2] |= b3 << (16 * k);
+      }
+      p[0][e] = w[0]; p[1][e] = w[1]; p[2][e] = w[2];
+    }
+    const int64_t piece = (int64_t)bn * 128;
+    unsigned char* dst = fp + (((int64_t)nt * num_kb + kb) * Kw + v) * 3 * piece + rr * 128 + ((ch ^ (rr & 7)) << 4);
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+      *reinterpret_cast<uint4*>(dst + (concat ? i : 2 - i) * piece) = make_uint4(p[i][0], p[i][1], p[i][2], p[i][3]);
+  }
+}
+
+int form_of(int bn) { return bn <= 80 ? 80 : (bn <= 128 ? 128 : 256); }
+int slot_bytes_of(int bn) { return (bn <= 80 ? 3 : 1) * bn * 128; }
+
+// Filter slots that fit beside the two S stages and the offset table.
+int slots_for(int bn, int rows, int num_kb) {
+  const int left = kSplitSmem - 1024 - A_STAGES * 3 * rows * 128 - num_kb * KB * 4;
+  const int n = left / slot_bytes_of(bn);
+  return n > MAX_B ? MAX_B : n;
+}
+
+// Cycles of the six products of a 128 x bn tile over 16 k (see the head of this file).
+double step_cycles(int bn) {
+  auto mma = [](int n) { const double pipe = n / 2.0, smem = 32 + n / 4.0; return pipe > smem ? pipe : smem; };
+  return bn <= 80 ? mma(3 * bn) + mma(2 * bn) + mma(bn) : 6 * mma(bn);
+}
+
+template <int BNMAX>
+cudaError_t launch_form(const SplitParams& q, int smem, cudaStream_t stream) {
+  static bool attr_done[64] = {};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+  if (!attr_done[dev]) {
+    cudaError_t e = cudaFuncSetAttribute(conv_f32_split_kernel<BNMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSplitSmem);
+    if (e != cudaSuccess) return e;
+    attr_done[dev] = true;
+  }
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = (unsigned)q.split; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+  const int grid = q.split > 1 ? q.nwork * q.split : (q.nwork < 148 ? q.nwork : 148);
+  cfg.gridDim = dim3((unsigned)grid, 1, 1);
+  cfg.blockDim = dim3(Form<BNMAX>::THREADS, 1, 1);
+  cfg.dynamicSmemBytes = (size_t)smem;
+  cfg.stream = stream;
+  cfg.attrs = attr;
+  cfg.numAttrs = q.split > 1 ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, conv_f32_split_kernel<BNMAX>, q);
+}
+
+}  // namespace
+
+F32SplitPlan plan_f32_split(const Geometry& g) {
+  F32SplitPlan p{};
+  p.eligible = false;
+  const int64_t K2 = (int64_t)g.C * g.Kh;
+  p.num_kb = (int32_t)((K2 + KB - 1) / KB);
+  p.halo = (g.Kw - 1) / g.s;
+  if (p.halo > 16 || g.Kw > 64 || K2 > 6144) return p;      // halo items, filter staging, offset table
+  p.rows = TILE_M + (p.halo + 7) / 8 * 8;
+  p.nsub = g.s < g.Kw ? g.s : g.Kw;
+  p.Wq = (g.Wp + g.s - 1) / g.s;
+  p.VQ = (int64_t)g.N * g.Ho * p.Wq;
+  if (p.VQ + 2 * TILE_M >= ((int64_t)1 << 31)) return p;
+  p.nks_last = (int32_t)((K2 - (int64_t)(p.num_kb - 1) * KB + 15) / 16);
+  p.nstages = p.num_kb * p.nsub;
+  const int64_t ntm = (p.VQ + TILE_M - 1) / TILE_M;
+  const double steps = ((p.num_kb - 1) * 4.0 + p.nks_last) * g.Kw;   // 16-wide steps of a tile
+  const char* force_bn = debug_getenv("IM2WIN_F32_SPLIT_BN");        // testing aids: channel tile, CTAs per tile
+  const char* force_z = debug_getenv("IM2WIN_F32_SPLIT_CTAS");
+  p.cost = 0;
+  p.packed_rows = 0;
+  const int most = (g.Co + 15) / 16;
+  for (int nt = (g.Co + 255) / 256; nt <= most && nt <= (g.Co + 255) / 256 + 32; ++nt) {
+    const int bn = ((g.Co + nt - 1) / nt + 15) / 16 * 16;
+    if (nt > 1 && (int64_t)(nt - 1) * bn >= g.Co) continue;          // fewer tiles of this width do
+    const int sb = slots_for(bn, p.rows, p.num_kb);
+    if (sb < (bn <= 80 ? 2 : 3)) continue;
+    if (nt * bn > p.packed_rows) p.packed_rows = nt * bn;
+    if (force_bn && bn != atoi(force_bn)) continue;
+    if (ntm * nt >= ((int64_t)1 << 30)) continue;
+    for (int z = 1; z <= 8; z *= 2) {
+      if (z > p.nstages || (z > 1 && ntm * nt * z > 128)) break;     // clusters: one tile each, all resident
+      if (force_z && z != atoi(force_z)) continue;
+      const int64_t rounds = z > 1 ? 1 : (ntm * nt + 147) / 148;
+      const double fill = 3.0 * bn * steps / 4 + 1200.0 * p.nstages; // shared-memory cycles of the copies and the staging
+      const double pipe = steps * step_cycles(bn), wave = pipe * 0.9 + fill;
+      const double tile = (pipe > wave ? pipe : wave) * ((p.nstages + z - 1) / z) / p.nstages + (z > 1 ? 5000 : 1500);
+      const double cost = rounds * tile + 6000;
+      if (!p.eligible || cost < p.cost) {
+        p.eligible = true;
+        p.cost = cost;
+        p.bn = bn; p.ntn = nt; p.split = z; p.sb = sb;
+        p.nwork = (int32_t)(ntm * nt);
+      }
+    }
+  }
+  if (!p.eligible) return p;
+  p.filter_bytes = (size_t)p.packed_rows * p.num_kb * KB * g.Kw * 6;
+  return p;
+}
+
+cudaError_t launch_pack_f32_split(const float* filter, void* scratch, const Geometry& g, cudaStream_t stream) {
+  const F32SplitPlan p = plan_f32_split(g);
+  if (!p.eligible) return cudaErrorInvalidValue;
+  unsigned char* base = static_cast<unsigned char*>(scratch);
+  int rows = 8;                                             // channels per block: staging within 40 KB
+  while (rows > 1 && (size_t)rows * KB * g.Kw * 4 > 40 * 1024) rows /= 2;
+  const size_t smem = (size_t)rows * KB * g.Kw * 4;
+  dim3 grid((unsigned)p.num_kb, (unsigned)(p.ntn * p.bn / rows));
+  if (grid.y > 65535) return cudaErrorInvalidValue;
+  pack_f32_split_kernel<<<grid, 256, smem, stream>>>(filter, base + kStatusBytes, reinterpret_cast<uint32_t*>(base), g.C * g.Kh,
+                                                     g.Kw, g.Co, p.bn, p.num_kb, rows, p.bn <= 80 ? 1 : 0);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_conv_f32_split(const float* window, float* y, void* scratch, const Geometry& g, cudaStream_t stream) {
+  const F32SplitPlan p = plan_f32_split(g);
+  if (!p.eligible) return cudaErrorInvalidValue;
+  unsigned char* base = static_cast<unsigned char*>(scratch);
+  SplitParams q;
+  q.win = window;
+  q.fp = base + kStatusBytes;
+  q.y = y;
+  q.status = reinterpret_cast<uint32_t*>(base);
+  q.img_stride = g.img_stride; q.strip = g.strip; q.chan_stride = g.chan_stride;
+  q.VQ = (uint32_t)p.VQ;
+  q.K2 = g.C * g.Kh; q.C = g.C; q.Wq = p.Wq; q.Wp = g.Wp; q.Ho = g.Ho; q.Wo = g.Wo; q.HoWo = g.Ho * g.Wo; q.Co = g.Co;
+  q.Kh = g.Kh; q.Kw = g.Kw; q.s = g.s; q.nsub = p.nsub; q.num_kb = p.num_kb; q.nks_last = p.nks_last;
+  q.rows = p.rows; q.halo = p.halo;
+  q.bn = p.bn; q.ntn = p.ntn; q.nwork = p.nwork; q.nstages = p.nstages; q.split = p.split;
+  q.sb = p.sb; q.slot_bytes = slot_bytes_of(p.bn);
+  const int rings = A_STAGES * 3 * p.rows * 128 + p.sb * q.slot_bytes + p.num_kb * KB * 4;
+  const int smem = 1024 + rings;
+  if (p.split > 1 && rings < p.bn * TILE_M * 4) return cudaErrorInvalidValue;
+  switch (form_of(p.bn)) {
+    case 80: return launch_form<80>(q, smem, stream);
+    case 128: return launch_form<128>(q, smem, stream);
+    default: return launch_form<256>(q, smem, stream);
+  }
+}
+
+}  // namespace im2win

@@ -61,8 +61,9 @@ extern "C" im2win_status im2win_conv_f32_static(const float* window, const float
   if ((reinterpret_cast<uintptr_t>(window) | reinterpret_cast<uintptr_t>(filter_oihw) |
        reinterpret_cast<uintptr_t>(y_nchw)) & 15u)
     return IM2WIN_ERR_MISALIGNED;
-  // The layer's scratch must fit the fixed array; nothing has touched CUDA yet.
-  if (l.total > (size_t)IM2WIN_STATIC_SCRATCH_BYTES) return IM2WIN_ERR_WORKSPACE_TOO_SMALL;
+  // This entry keeps to the FFMA kernel (the tensor-core kernel's filter images take half as much again);
+  // the layer's scratch must fit the fixed array; nothing has touched CUDA yet.
+  if (l.ffma_total > (size_t)IM2WIN_STATIC_SCRATCH_BYTES) return IM2WIN_ERR_WORKSPACE_TOO_SMALL;
   void* scratch = nullptr;
   if (static_scratch_address(&scratch) != cudaSuccess) return IM2WIN_ERR_CUDA;
   cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
