@@ -78,6 +78,7 @@ im2win_status scratch_layout(const Geometry& g, im2win_dtype dtype, ScratchLayou
     return IM2WIN_ERR_INVALID_ARG;
   }
   l->f32_split = false;
+  l->runs = false;
   l->f16_shift = false;
   l->f16_raw = false;
   l->f16_mat = false;
@@ -93,6 +94,13 @@ im2win_status scratch_layout(const Geometry& g, im2win_dtype dtype, ScratchLayou
     const int64_t wide = round_up((int64_t)kStatusBytes + 4 * round_up(g.K, 32), 256) + round_up(g.K, 32) * l->Co_pad * 4;
     int64_t most = round_up(wide, 256);
     if (split.eligible && kStatusBytes + (int64_t)split.filter_bytes > most) most = kStatusBytes + (int64_t)split.filter_bytes;
+    const RunsPlan runs = plan_runs(g, true);
+    if (runs.eligible) {
+      const char* force = debug_getenv("IM2WIN_F32_KERNEL");
+      l->runs = force && strcmp(force, "runs") == 0;
+      if (l->runs) l->f32_split = false;
+      if (kStatusBytes + (int64_t)runs.filter_bytes > most) most = kStatusBytes + (int64_t)runs.filter_bytes;
+    }
     l->ffma_total = l->total;
     l->total = (size_t)round_up(most, 256);
   }
@@ -130,6 +138,12 @@ im2win_status scratch_layout(const Geometry& g, im2win_dtype dtype, ScratchLayou
       const size_t mat_total = (size_t)round_up((int64_t)mat.scratch_bytes, 256);
       if (mat_total > l->total) l->total = mat_total;
     }
+    const RunsPlan runs = plan_runs(g, false);
+    if (runs.eligible) {
+      l->runs = force && strcmp(force, "runs") == 0;
+      const size_t runs_total = (size_t)round_up(kStatusBytes + (int64_t)runs.filter_bytes, 256);
+      if (runs_total > l->total) l->total = runs_total;
+    }
   }
   return IM2WIN_OK;
 }
@@ -157,7 +171,8 @@ static im2win_status conv_common(const void* window, const void* filter, float* 
   cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
   cudaError_t e = cudaSuccess;
   if (mode & kDoPack) {
-    if (l.f32_split) e = launch_pack_f32_split(static_cast<const float*>(filter), scratch, g, stream);
+    if (l.runs) e = launch_pack_runs(filter, scratch, g, dtype == IM2WIN_F32, stream);
+    else if (l.f32_split) e = launch_pack_f32_split(static_cast<const float*>(filter), scratch, g, stream);
     else if (dtype == IM2WIN_F32) e = launch_pack_f32(static_cast<const float*>(filter), scratch, g, l, stream);
     else if (l.f16_stem) e = launch_pack_f16_shift(static_cast<const uint16_t*>(filter), scratch, g, l, stream);
     else if (l.f16_mat) e = launch_pack_f16_mat(static_cast<const uint16_t*>(filter), scratch, g, stream);
@@ -168,7 +183,8 @@ static im2win_status conv_common(const void* window, const void* filter, float* 
     if (e != cudaSuccess) return IM2WIN_ERR_CUDA;
   }
   if (mode & kDoConv) {
-    if (l.f32_split) e = launch_conv_f32_split(static_cast<const float*>(window), y, scratch, g, stream);
+    if (l.runs) e = launch_conv_runs(window, y, scratch, g, dtype == IM2WIN_F32, stream);
+    else if (l.f32_split) e = launch_conv_f32_split(static_cast<const float*>(window), y, scratch, g, stream);
     else if (dtype == IM2WIN_F32) e = launch_conv_f32(static_cast<const float*>(window), y, scratch, g, l, stream);
     else if (l.f16_stem) e = launch_conv_f16_stem(static_cast<const uint16_t*>(window), y, scratch, g, l, stream);
     else if (l.f16_mat) e = launch_conv_f16_mat(static_cast<const uint16_t*>(window), y, scratch, g, stream);
@@ -203,6 +219,7 @@ const char* im2win_conv_kernel_name(const im2win_shape* shape, im2win_dtype dtyp
   Geometry g;
   ScratchLayout l;
   if (derive_geometry(shape, &g) != IM2WIN_OK || scratch_layout(g, dtype, &l) != IM2WIN_OK) return "none";
+  if (l.runs) return dtype == IM2WIN_F32 ? "f32-runs" : "f16-runs";
   if (dtype == IM2WIN_F32) return l.f32_split ? "f32-split" : "f32-ffma";
   if (l.f16_stem) return "f16-stem";
   if (l.f16_mat) return "f16-mat";

@@ -22,8 +22,10 @@
 //
 // What bounds it: the tensor pipe, and next to it the shared-memory pipe the MMA reads its operands
 // through: an instruction of M = 128, K = 16 takes max(N/2, 32 + N/4) cycles.  Up to 80 channels the filter
-// pieces therefore lie side by side as one operand, [w1 | w2 | w3], and three instructions replace six
-// (x1 against all of it, x2 against [w1 | w2], x3 against w1, into three accumulators of one magnitude each).
+// pieces therefore lie side by side as one operand, [w1 | w2 | w3], and three instructions replace six: x1
+// against all of it, x2 against [w1 | w2] one accumulator further, x3 against w1 two further, so that each of the
+// three accumulators holds products of one magnitude and their order is free.  A chain may then take several
+// units: `chain` steps of 16 k (12, or 8 on reductions below 288).
 //
 // Roles (one persistent CTA per SM): one or two warpgroups of producers (thread = row; 32 loads in flight,
 // split, 16-byte stores), an MMA warp, a filter-copy warp (one untiled bulk copy per piece: the pack kernel
@@ -59,14 +61,16 @@ struct SplitParams {
   uint32_t VQ;
   int32_t K2, C, Wq, Wp, Ho, Wo, HoWo, Co, Kh, Kw, s, nsub, num_kb, nks_last;
   int32_t rows, halo;                         // rows of a sub-tile (128 + halo rounded up to 8), halo
-  int32_t bn, ntn, nwork, nstages, split, sb, slot_bytes;
+  int32_t bn, ntn, nwork, nstages, split, sb, slot_bytes, chain;
 };
 
 __device__ __forceinline__ void wait_for_previous_kernel() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// (volatile: the loads of a batch stay together, ahead of the wait for the stage they are for; left to
+// itself the compiler moved them to their uses, one round trip per eight loads: 296 instead of XXX us)
 __device__ __forceinline__ float ld_if(const float* p, bool ok) {
   float v = 0.f;
-  asm("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %2, 0;\n\t@p ld.global.nc.f32 %0, [%1];\n\t}"
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %2, 0;\n\t@p ld.global.nc.f32 %0, [%1];\n\t}"
       : "+f"(v)
       : "l"(p), "r"((int)ok));
   return v;
@@ -133,15 +137,16 @@ __device__ __forceinline__ void store16(float* base, int stride, const float (&v
 
 template <int BNMAX> struct Form {
   static constexpr bool CONCAT = BNMAX == 80;             // the filter pieces side by side in one operand
-  static constexpr int ACC_COLS = BNMAX == 128 ? 128 : 256;
+  static constexpr int ACC_COLS = BNMAX == 128 ? 128 : 256; // tensor memory: a ring of accumulators (CONCAT: of triples)
   static constexpr int NACC = 512 / ACC_COLS;
+  static constexpr int ACC_LOG = BNMAX == 128 ? 2 : 1;
   static constexpr int CH = BNMAX == 80 ? 3 : BNMAX / 32; // 16-channel chunks per epilogue warp
   static constexpr int PWG = BNMAX == 256 ? 1 : 2;        // producer warpgroups
   static constexpr int THREADS = 128 * (PWG + 3);
-  static constexpr int REGS_PRODUCER = 96;
-  static constexpr int REGS_MISC = 64;
-  static constexpr int REGS_EPILOGUE = BNMAX == 256 ? 176 : 112;
-  // (the launch holds 128 or 96 registers a thread: 96 + 64 + 2*176 = 4*128, 2*96 + 64 + 2*112 = 5*96)
+  static constexpr int REGS_PRODUCER = 112;
+  static constexpr int REGS_MISC = BNMAX == 256 ? 64 : 48;
+  static constexpr int REGS_EPILOGUE = BNMAX == 256 ? 168 : 104;
+  // (the launch holds 128 or 96 registers a thread: 112 + 64 + 2*168 = 4*128, 2*112 + 48 + 2*104 = 5*96)
 };
 
 // One output in fp32 FMAs, k ascending, for the values the split cannot hold.  The filter element is the sum of
@@ -212,77 +217,94 @@ __global__ void __launch_bounds__(Form<BNMAX>::THREADS, 1) conv_f32_split_kernel
 
   if (wg < F::PWG) {
     // ---------------- producers: thread = row ------------------------------------------------------
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(F::REGS_PRODUCER));
+    if constexpr (BNMAX == 256) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(F::REGS_PRODUCER));
+    else asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(F::REGS_PRODUCER));
     const int tid = threadIdx.x & 127;
-    bool ok = true;
-    uint32_t sc = 0;                                       // stages so far, of all producers
-    for (int w = w_first; w < q.nwork && ok; w += w_step) {
-      const uint32_t q0 = (uint32_t)(w / q.ntn) * TILE_M;
-      // Row -> window column (class 0) and the number of classes that exist there (0 beyond the tensor).
-      auto locate = [&](uint32_t vq, const float*& base, int& lim) {
-        base = q.win;
-        lim = 0;
-        if (vq < q.VQ) {
-          const uint32_t sg = vq / (uint32_t)q.Wq;
-          const int i = (int)(vq - sg * (uint32_t)q.Wq);
-          const uint32_t n = sg / (uint32_t)q.Ho;
-          const int ho = (int)(sg - n * (uint32_t)q.Ho);
-          base += (int64_t)n * q.img_stride + (int64_t)ho * q.strip + (int64_t)i * q.s * q.Kh;
-          lim = q.Wp - i * q.s;
-        }
-      };
-      const float *base, *hbase = q.win;
-      int lim, hlim = 0;
-      locate(q0 + tid, base, lim);
-      const int hrow = TILE_M + (tid >> 3), hch = tid & 7;  // halo item: a row below the tile, one chunk of it
-      const bool has_halo = tid < q.halo * 8;
-      if (has_halo) locate(q0 + hrow, hbase, hlim);
-      int kb = kb0, t = t0;
-      for (int st = st0; st < st1; ++st, ++sc) {
-        if (F::PWG == 1 || (int)(sc & 1) == wg) {
-          const int buf = sc & 1;
-          const uint32_t stage = a_ring + buf * a_stage_bytes;
-          const int nch = kb == q.num_kb - 1 ? 2 * q.nks_last : 8;      // the MMAs stop at the last step with real k2
-          const int4* kt = reinterpret_cast<const int4*>(koff_s + kb * KB);
-          auto load8 = [&](const float* src, bool row_ok, int ch, float (&v)[8]) {
-            const int4 o0 = kt[2 * ch], o1 = kt[2 * ch + 1];
-            const int32_t off[8] = {o0.x, o0.y, o0.z, o0.w, o1.x, o1.y, o1.z, o1.w};
-#pragma unroll
-            for (int e = 0; e < 8; ++e) v[e] = ld_if(src + off[e], row_ok && off[e] >= 0);
-          };
-          auto store8 = [&](int row, int ch, const float (&v)[8]) {
-            uint32_t p[3][4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) split2(v[2 * e], v[2 * e + 1], p[0][e], p[1][e], p[2][e]);
-            const uint32_t dst = stage + row * 128 + ((ch ^ (row & 7)) << 4);
-#pragma unroll
-            for (int i = 0; i < 3; ++i) st_shared16(dst + i * sub_bytes, p[i][0], p[i][1], p[i][2], p[i][3]);
-          };
-          const bool row_ok = t < lim;
-          const float* src = base + t * q.Kh;
-          float v[4][8], hv[8];
-#pragma unroll
-          for (int c = 0; c < 4; ++c) load8(src, row_ok && c < nch, c, v[c]);
-          const bool halo_now = has_halo && hch < nch;
-          if (halo_now) load8(hbase + t * q.Kh, t < hlim, hch, hv);
-          ok = mbar_wait(a_empty0 + 8 * buf, ((sc >> 1) & 1) ^ 1, &abort_flag, q.status);
-          ok = __all_sync(0xffffffffu, ok);
-          if (!ok) break;
-#pragma unroll
-          for (int c = 0; c < 4; ++c) if (c < nch) store8(tid, c, v[c]);
-          if (halo_now) store8(hrow, hch, hv);
-          if (nch > 4) {
-#pragma unroll
-            for (int c = 0; c < 4; ++c) load8(src, row_ok && 4 + c < nch, 4 + c, v[c]);
-#pragma unroll
-            for (int c = 0; c < 4; ++c) if (4 + c < nch) store8(tid, 4 + c, v[c]);
-          }
-          fence_proxy_async_smem();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(a_full0 + 8 * buf);
-        }
-        if (++t == q.nsub) { t = 0; ++kb; }
+    const int hrow = TILE_M + (tid >> 3), hch = tid & 7;   // halo item: a row below the tile, one chunk of it
+    const bool has_halo = tid < q.halo * 8;
+    const float *base = q.win, *hbase = q.win;             // this thread's rows of the tile that is being loaded
+    int lim = 0, hlim = 0;                                 // ... and how many column classes exist there (0: no such row)
+    // The stage being loaded: tile, stage inside the CTA's range, its k2-block and column class, running number.
+    int w = w_first, st = st0, kb = kb0, t = t0;
+    uint32_t sc = 0;
+    auto advance = [&]() {
+      ++sc;
+      if (++t == q.nsub) { t = 0; ++kb; }
+      if (++st == st1) { st = st0; kb = kb0; t = t0; w += w_step; }
+    };
+    auto locate = [&](uint32_t vq, const float*& ptr, int& classes) {
+      ptr = q.win;
+      classes = 0;
+      if (vq < q.VQ) {
+        const uint32_t sg = vq / (uint32_t)q.Wq;
+        const int i = (int)(vq - sg * (uint32_t)q.Wq);
+        const uint32_t n = sg / (uint32_t)q.Ho;
+        const int ho = (int)(sg - n * (uint32_t)q.Ho);
+        ptr += (int64_t)n * q.img_stride + (int64_t)ho * q.strip + (int64_t)i * q.s * q.Kh;
+        classes = q.Wp - i * q.s;
       }
+    };
+    int here = -1;                                         // the position tile that base and hbase belong to
+    auto enter_tile = [&]() {
+      const int mt = w / q.ntn;
+      if (mt == here) return;
+      here = mt;
+      locate((uint32_t)mt * TILE_M + tid, base, lim);
+      if (has_halo) locate((uint32_t)mt * TILE_M + hrow, hbase, hlim);
+    };
+    auto chunks = [&]() { return kb == q.num_kb - 1 ? 2 * q.nks_last : 8; };   // the MMAs stop at the last step with real k2
+    auto load8 = [&](const float* src, bool row_ok, int ch, float (&v)[8]) {
+      const int4* kt = reinterpret_cast<const int4*>(koff_s + kb * KB);
+      const int4 o0 = kt[2 * ch], o1 = kt[2 * ch + 1];
+      const int32_t off[8] = {o0.x, o0.y, o0.z, o0.w, o1.x, o1.y, o1.z, o1.w};
+#pragma unroll
+      for (int e = 0; e < 8; ++e) v[e] = ld_if(src + off[e], row_ok && off[e] >= 0);
+    };
+    auto load_half = [&](int half, int nch, float (&v)[4][8]) {
+#pragma unroll
+      for (int c = 0; c < 4; ++c) load8(base + t * q.Kh, t < lim && 4 * half + c < nch, 4 * half + c, v[c]);
+    };
+    auto store8 = [&](uint32_t stage, int row, int ch, const float (&v)[8]) {
+      uint32_t p[3][4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) split2(v[2 * e], v[2 * e + 1], p[0][e], p[1][e], p[2][e]);
+      const uint32_t dst = stage + row * 128 + ((ch ^ (row & 7)) << 4);
+#pragma unroll
+      for (int i = 0; i < 3; ++i) st_shared16(dst + i * sub_bytes, p[i][0], p[i][1], p[i][2], p[i][3]);
+    };
+
+    // Half a stage (32 loads a thread) is on its way while the other half is split and stored; the first half
+    // of the warpgroup's next stage is requested before the second half of this one is stored.
+    bool ok = true;
+    float va[4][8], vb[4][8], vh[8];
+    if (F::PWG == 2 && wg == 1) advance();
+    if (w < q.nwork) {
+      enter_tile();
+      load_half(0, chunks(), va);
+      if (has_halo && hch < chunks()) load8(hbase + t * q.Kh, t < hlim, hch, vh);
+    }
+    while (w < q.nwork) {
+      const int buf = sc & 1, nch = chunks();
+      const uint32_t stage = a_ring + buf * a_stage_bytes, parity = ((sc >> 1) & 1) ^ 1;
+      load_half(1, nch, vb);
+      ok = mbar_wait(a_empty0 + 8 * buf, parity, &abort_flag, q.status);
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) break;
+#pragma unroll
+      for (int c = 0; c < 4; ++c) if (c < nch) store8(stage, tid, c, va[c]);
+      if (has_halo && hch < nch) store8(stage, hrow, hch, vh);
+#pragma unroll
+      for (int i = 0; i < F::PWG; ++i) advance();
+      if (w < q.nwork) {
+        enter_tile();
+        load_half(0, chunks(), va);
+        if (has_halo && hch < chunks()) load8(hbase + t * q.Kh, t < hlim, hch, vh);
+      }
+#pragma unroll
+      for (int c = 0; c < 4; ++c) if (4 + c < nch) store8(stage, tid, 4 + c, vb[c]);
+      fence_proxy_async_smem();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(a_full0 + 8 * buf);
     }
   } else if (wg == F::PWG) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(F::REGS_MISC));
@@ -290,11 +312,11 @@ __global__ void __launch_bounds__(Form<BNMAX>::THREADS, 1) conv_f32_split_kernel
       // ---------------- MMA issuer -----------------------------------------------------------------
       const bool leader = elect_one();
       const uint32_t a_lo0 = smem_desc_lo(a_ring), b_lo0 = smem_desc_lo(b_ring);
-      const uint32_t sub_lo = (uint32_t)sub_bytes >> 4, bn_lo = (uint32_t)q.bn * 8;
+      const uint32_t sub_lo = (uint32_t)sub_bytes >> 4;
       const uint32_t id1 = instr_desc_bf16(TILE_M, q.bn), id2 = instr_desc_bf16(TILE_M, 2 * q.bn),
                      id3 = instr_desc_bf16(TILE_M, 3 * q.bn);
       bool ok = true;
-      uint32_t sc = 0, ac = 0;                             // stages and units so far
+      uint32_t sc = 0, ac = 0;                             // stages and chains so far
       int slot = 0;
       uint32_t bph = 0;
       for (int w = w_first; w < q.nwork && ok; w += w_step) {
@@ -306,12 +328,17 @@ __global__ void __launch_bounds__(Form<BNMAX>::THREADS, 1) conv_f32_split_kernel
           ok = __all_sync(0xffffffffu, ok);
           if (!ok) break;
           uint32_t a_view = a_lo0 + (uint32_t)(buf * (a_stage_bytes >> 4));
-          for (int v = t; v < q.Kw; v += q.s, a_view += 8u, ++ac) {     // next view: one row (128 bytes) further down
-            const int ab = ac % F::NACC;
-            ok = mbar_wait(acc_empty0 + 8 * ab, ((ac / F::NACC) & 1) ^ 1, &abort_flag, q.status);
-            ok = __all_sync(0xffffffffu, ok);
-            if (!ok) break;
-            const uint32_t d = tmem_acc + ab * F::ACC_COLS;
+          int links = 0;                                   // steps in the open chain; 0: none is open
+          for (int v = t; v < q.Kw; v += q.s, a_view += 8u) {           // next view: one row (128 bytes) further down
+            const int ab = ac & (F::NACC - 1);
+            if (links == 0) {
+              ok = mbar_wait(acc_empty0 + 8 * ab, ((ac >> F::ACC_LOG) & 1) ^ 1, &abort_flag, q.status);
+              ok = __all_sync(0xffffffffu, ok);
+              if (!ok) break;
+            }
+            const uint32_t d = tmem_acc + ab * F::ACC_COLS, more = links > 0;
+            links += nks;
+            const bool last_link = !F::CONCAT || links + nks > q.chain || v + q.s >= q.Kw;
             if constexpr (F::CONCAT) {
               ok = mbar_wait(b_full0 + 8 * slot, bph, &abort_flag, q.status);
               ok = __all_sync(0xffffffffu, ok);
@@ -321,7 +348,7 @@ __global__ void __launch_bounds__(Form<BNMAX>::THREADS, 1) conv_f32_split_kernel
               if (leader) {
 #pragma unroll
                 for (int j = 0; j < KB / 16; ++j)
-                  if (j < nks) umma_f16_lohi(d, a_view + 2 * j, b_lo + 2 * j, id3, (uint32_t)j);
+                  if (j < nks) umma_f16_lohi(d, a_view + 2 * j, b_lo + 2 * j, id3, more | (uint32_t)j);
 #pragma unroll
                 for (int j = 0; j < KB / 16; ++j)
                   if (j < nks) umma_f16_lohi(d + q.bn, a_view + sub_lo + 2 * j, b_lo + 2 * j, id2, 1u);
@@ -354,7 +381,11 @@ __global__ void __launch_bounds__(Form<BNMAX>::THREADS, 1) conv_f32_split_kernel
               }
               if (!ok) break;
             }
-            if (leader) umma_commit(acc_full0 + 8 * ab);
+            if (last_link) {
+              if (leader) umma_commit(acc_full0 + 8 * ab);
+              ++ac;
+              links = 0;
+            }
             __syncwarp();
           }
           if (ok && leader) umma_commit(a_empty0 + 8 * buf);
@@ -362,7 +393,7 @@ __global__ void __launch_bounds__(Form<BNMAX>::THREADS, 1) conv_f32_split_kernel
           if (++t == q.nsub) { t = 0; ++kb; }
         }
       }
-      (void)id2; (void)id3; (void)bn_lo;
+      (void)id2; (void)id3;
     } else if ((warp & 3) == 1) {
       // ---------------- filter copies ----------------------------------------------------------------
       const bool leader = elect_one();
@@ -424,11 +455,13 @@ __global__ void __launch_bounds__(Form<BNMAX>::THREADS, 1) conv_f32_split_kernel
       for (int j = 0; j < F::CH; ++j)
 #pragma unroll
         for (int e = 0; e < 16; ++e) acc[j][e] = 0.f;
-      int t = t0;
+      int kb = kb0, t = t0;
       for (int st = st0; st < st1 && ok; ++st) {
-        for (int v = t; v < q.Kw; v += q.s, ++ac) {
-          const int ab = ac % F::NACC;
-          ok = mbar_wait(acc_full0 + 8 * ab, (ac / F::NACC) & 1, &abort_flag, q.status);
+        const int nks = kb == q.num_kb - 1 ? q.nks_last : KB / 16;
+        const int units = F::CONCAT ? (q.chain / nks) : 1;  // units of a chain
+        for (int v = t; v < q.Kw; v += q.s * units, ++ac) {
+          const int ab = ac & (F::NACC - 1);
+          ok = mbar_wait(acc_full0 + 8 * ab, (ac >> F::ACC_LOG) & 1, &abort_flag, q.status);
           ok = __all_sync(0xffffffffu, ok);
           if (!ok) break;
           tc_fence_after();
@@ -448,29 +481,20 @@ __global__ void __launch_bounds__(Form<BNMAX>::THREADS, 1) conv_f32_split_kernel
               for (int e = 0; e < 16; ++e)
                 acc[j][e] += __uint_as_float(r0[e]) + (__uint_as_float(r1[e]) + __uint_as_float(r2[e]));
             }
-          } else if constexpr (BNMAX == 256) {              // (one chunk in flight: 128 sums leave no more registers)
-#pragma unroll
-            for (int j = 0; j < F::CH; ++j) {
-              if ((h + 2 * j) * 16 >= q.bn) break;
-              uint32_t r0[16];
-              tmem_ld16_issue(d + 32 * j, r0);
-              tmem_wait16(r0);
-#pragma unroll
-              for (int e = 0; e < 16; ++e) acc[j][e] += __uint_as_float(r0[e]);
-            }
           } else {
+            constexpr int STEP = BNMAX == 256 ? 1 : 2;      // chunks in flight (128 sums leave registers for one)
 #pragma unroll
-            for (int j = 0; j < F::CH; j += 2) {            // (columns beyond bn hold nothing and are not stored)
+            for (int j = 0; j < F::CH; j += STEP) {         // (columns beyond bn hold nothing and are not stored)
               if ((h + 2 * j) * 16 >= q.bn) break;
               uint32_t r0[16], r1[16];
               tmem_ld16_issue(d + 32 * j, r0);
-              tmem_ld16_issue(d + 32 * j + 32, r1);
+              if (STEP == 2) tmem_ld16_issue(d + 32 * j + 32, r1);
               tmem_wait16(r0);
-              tmem_wait16(r1);
+              if (STEP == 2) tmem_wait16(r1);
 #pragma unroll
               for (int e = 0; e < 16; ++e) {
                 acc[j][e] += __uint_as_float(r0[e]);
-                acc[j + 1][e] += __uint_as_float(r1[e]);
+                if (STEP == 2) acc[j + STEP - 1][e] += __uint_as_float(r1[e]);
               }
             }
           }
@@ -478,9 +502,10 @@ __global__ void __launch_bounds__(Form<BNMAX>::THREADS, 1) conv_f32_split_kernel
           __syncwarp();
           if (lane == 0) mbar_arrive(acc_empty0 + 8 * ab);
         }
-        if (++t == q.nsub) t = 0;
+        if (++t == q.nsub) { t = 0; ++kb; }
       }
-      if (!ok || q.split > 1) break;
+      if (!ok) break;
+      if (q.split > 1) break;
       if (valid) {
         const int co0 = nt * q.bn;
         float* yrow = q.y + ((int64_t)n * q.Co + co0) * q.HoWo + (int64_t)ho * q.Wo + i0;
@@ -733,6 +758,7 @@ cudaError_t launch_conv_f32_split(const float* window, float* y, void* scratch, 
   q.rows = p.rows; q.halo = p.halo;
   q.bn = p.bn; q.ntn = p.ntn; q.nwork = p.nwork; q.nstages = p.nstages; q.split = p.split;
   q.sb = p.sb; q.slot_bytes = slot_bytes_of(p.bn);
+  q.chain = g.K >= 288 ? 12 : 8;
   const int rings = A_STAGES * 3 * p.rows * 128 + p.sb * q.slot_bytes + p.num_kb * KB * 4;
   const int smem = 1024 + rings;
   if (p.split > 1 && rings < p.bn * TILE_M * 4) return cudaErrorInvalidValue;

@@ -1,0 +1,795 @@
+// im2win convolution on the tensor cores with the window tensor brought in as contiguous runs.
+//
+// One kernel for two operand types: fp16 (one piece per operand, one product) and fp32 (three bf16 pieces, six
+// products, short accumulator chains; why and how accurate: conv_f32_split.cu).  It needs no alignment of planes,
+// strips or images and takes every stride.
+//
+// Columns.  In the im2win tensor the s*Kh elements of columns i*s .. i*s + s - 1 of a strip are contiguous, so a
+// convolution of stride s is one of stride 1 on columns s times as tall: virtual column i holds
+// e = t*Kh + u (t < min(s, Kw)), k2 = c*E + e with E = min(s, Kw)*Kh, and the kernel is G = ceil(Kw/s) virtual columns
+// wide; filter elements with g*s + t >= Kw are zeros (3x3 with stride 2: a third more products, but every element is
+// staged once and from one run).  A GEMM row is a virtual position q = (n*Ho + ho)*pitch + i; S[row][64 k2] is staged
+// once per k2-block and the MMAs of virtual kernel column g read the view that starts g rows further down.
+//
+// Staging.  The columns a tile needs of one channel are one contiguous run per image it touches: an untiled bulk
+// copy from the 16-byte boundary below to the one above brings it into a ring of raw slots (RK k2 each: the channels
+// of RK consecutive k2).  Eight warps then read the elements of their rows back (2- or 4-byte shared loads, the phase
+// of each channel's run added to the address), split them (fp32) and write 16-byte units of S.  Gathering with global
+// loads instead (conv_f16_shift.cu, conv_f32_split.cu) makes every load instruction touch 32 rows s*Kh elements apart:
+// three or more L1 wavefronts each, and a round trip to memory per batch.
+//
+// What bounds it: the shared-memory pipe, which carries the MMA's operand reads (32 + N/4 cycles per instruction of
+// M = 128, K = 16), the copies, the read-back and the S stores.
+#include <cuda_fp16.h>
+#include <stdlib.h>
+#include <string.h>
+
+#include <type_traits>
+
+#define IM2WIN_INLINE_SLOW_WAIT      // (a call beside the epilogue's live sums costs spills)
+#include "common.cuh"
+#include "ptx_sm100.cuh"
+
+namespace im2win {
+namespace {
+
+using namespace ptx;
+
+constexpr int TILE_M = 128;
+constexpr int KB = 64;
+constexpr int MAX_A = 4, MAX_RAW = 8, MAX_B = 16, MAX_ACC = 8;
+constexpr int MAX_SEG = 6;                    // images a tile may touch
+constexpr int kRunsSmem = 226 * 1024;
+constexpr int THREADS = 640;                  // 8 staging warps, 4 single-role warps, 8 epilogue warps
+
+struct RunsParams {
+  const unsigned char* __restrict__ win;
+  const unsigned char* __restrict__ fp;       // packed filter: shared-memory images, see pack_runs_kernel
+  float* __restrict__ y;
+  uint32_t* status;
+  int64_t img_bytes, chan_bytes, win_bytes;   // of one image, one channel plane, the whole window tensor
+  uint32_t VQ;
+  int32_t C, N, Wp, Wq, pitch, Ho, Wo, HoWo, Co, Kh, Kw, s;
+  int32_t E, G, K2, num_kb, nks_last;
+  int32_t col_bytes;                          // distance of neighbouring virtual columns: s*Kh elements
+  int32_t rows, halo, region, rk, raw_slot, a_stage;
+  int32_t bn, ntn, nwork, sa, sr, sb, slot_bytes, resident, chain;
+};
+
+__device__ __forceinline__ void wait_for_previous_kernel() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ uint32_t cvt_bf16x2(float lo, float hi) {
+  uint32_t r;
+  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
+  return r;
+}
+// Two values -> their three pieces, packed (first value in the low half).
+__device__ __forceinline__ void split2(float a, float b, uint32_t& p1, uint32_t& p2, uint32_t& p3) {
+  p1 = cvt_bf16x2(a, b);
+  const float ra = a - __uint_as_float(p1 << 16), rb = b - __uint_as_float(p1 & 0xffff0000u);
+  p2 = cvt_bf16x2(ra, rb);
+  p3 = cvt_bf16x2(ra - __uint_as_float(p2 << 16), rb - __uint_as_float(p2 & 0xffff0000u));
+}
+__device__ __forceinline__ void st_shared16(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+  asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
+}
+__device__ __forceinline__ uint32_t ld_shared_u16(uint32_t addr) {
+  uint16_t v;
+  asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(addr));
+  return v;
+}
+__device__ __forceinline__ float ld_shared_f32(uint32_t addr) {
+  float v;
+  asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr));
+  return v;
+}
+__device__ __forceinline__ void tmem_ld16_issue(uint32_t taddr, uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr)
+      : "memory");
+}
+// The wait for loads into r[]: naming the registers keeps every use of them after it.
+__device__ __forceinline__ void tmem_wait16(uint32_t (&r)[16]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                 "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
+               :
+               : "memory");
+}
+__host__ __device__ constexpr uint32_t instr_desc(bool bf16, int M, int N) {
+  return (1u << 4) | (bf16 ? (1u << 7) | (1u << 10) : 0u) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+}
+// An output that has to be computed again (see conv_f32_split.cu).
+__device__ __forceinline__ bool suspicious(float v) {
+  const uint32_t u = __float_as_uint(v) << 1, lo = (uint32_t)(127 - 90) << 24;
+  return u != 0u && u - lo >= 0xff000000u - lo;
+}
+
+template <bool F32, int BNMAX> struct Form {
+  static constexpr int ES = F32 ? 4 : 2;
+  static constexpr int ACC_COLS = F32 ? 256 : BNMAX;        // tensor memory: a ring of accumulators (fp32: of triples)
+  static constexpr int NACC = 512 / ACC_COLS;
+  static constexpr int ACC_LOG = NACC == 2 ? 1 : (NACC == 4 ? 2 : 3);
+  static constexpr int CH = (BNMAX + 31) / 32;              // 16-channel chunks per epilogue warp
+  static constexpr int REGS_STAGING = 80, REGS_MISC = 64, REGS_EPILOGUE = 128;   // 2*80 + 64 + 2*128 = 5*96
+};
+
+// Where the rows of a tile lie: image n0 + g of the tile is a run of its own, [start, end) in elements of a channel
+// plane, at byte seg_off(g) of a channel's region in a raw slot.
+struct TileRuns {
+  uint32_t n0, n1;
+  int32_t start0, end1;                                     // first element of image n0, end in image n1
+};
+__device__ __forceinline__ int run_size(int elems, int es) { return (elems * es + 30) & ~15; }
+__device__ __forceinline__ void split_q(const RunsParams& q, uint32_t vq, uint32_t& n, int& ho, int& i) {
+  const uint32_t sg = vq / (uint32_t)q.pitch;
+  i = (int)(vq - sg * (uint32_t)q.pitch);
+  n = sg / (uint32_t)q.Ho;
+  ho = (int)(sg - n * (uint32_t)q.Ho);
+}
+__device__ __forceinline__ TileRuns tile_runs(const RunsParams& q, uint32_t q0) {
+  TileRuns r;
+  int ho, i;
+  split_q(q, q0, r.n0, ho, i);
+  if (i > q.Wq - 1) i = q.Wq - 1;                           // (a dead row of a widened pitch: any column will do)
+  r.start0 = (ho * q.Wp + i * q.s) * q.Kh;
+  uint32_t ql = q0 + TILE_M + q.halo - 1;
+  if (ql >= q.VQ) ql = q.VQ - 1;
+  split_q(q, ql, r.n1, ho, i);
+  // (all s columns of the last virtual column: where s does not divide Wp some lie in the next strip or plane.  Only
+  // zero filter elements meet them, but they have to be numbers)
+  r.end1 = (ho * q.Wp + ((i < q.Wq - 1 ? i : q.Wq - 1) + 1) * q.s) * q.Kh;
+  return r;
+}
+
+// One output in fp32 FMAs, k ascending.  fp32: for the values the split cannot hold.  Both: where a column
+// outside the window, which meets zeros of the widened filter, holds an infinity or a NaN.
+template <bool F32>
+__device__ __forceinline__ float exact_output(const RunsParams& q, uint32_t n, int ho, int wo, int nt, int col) {
+  constexpr int ES = F32 ? 4 : 2, PIECES = F32 ? 3 : 1;
+  const unsigned char* wbase = q.win + (int64_t)n * q.img_bytes + ((int64_t)ho * q.Wp + (int64_t)wo * q.s) * q.Kh * ES;
+  const int64_t piece = (int64_t)q.bn * 128;
+  const unsigned char* frow = q.fp + (int64_t)nt * q.num_kb * q.G * PIECES * piece + col * 128;
+  float acc = 0.f;
+  for (int c = 0; c < q.C; ++c)
+    for (int v = 0; v < q.Kw; ++v)
+      for (int u = 0; u < q.Kh; ++u) {
+        const int g = v / q.s, k2 = c * q.E + (v - g * q.s) * q.Kh + u, kb = k2 / KB, e = k2 - kb * KB;
+        const unsigned char* f = frow + ((int64_t)kb * q.G + g) * PIECES * piece + ((((e >> 3) ^ (col & 7)) << 4) | ((e & 7) * 2));
+        const unsigned char* x = wbase + c * q.chan_bytes + (v * q.Kh + u) * ES;
+        if constexpr (F32) {
+          auto part = [&](int p) { return __uint_as_float((uint32_t)*reinterpret_cast<const uint16_t*>(f + p * piece) << 16); };
+          acc = fmaf(*reinterpret_cast<const float*>(x), (part(0) + part(1)) + part(2), acc);
+        } else {
+          acc = fmaf(__half2float(*reinterpret_cast<const __half*>(x)), __half2float(*reinterpret_cast<const __half*>(f)), acc);
+        }
+      }
+  return acc;
+}
+
+template <bool F32, int BNMAX, bool PHASED>
+__global__ void __launch_bounds__(THREADS, 1) conv_runs_kernel(RunsParams q) {
+  using F = Form<F32, BNMAX>;
+  constexpr int ES = F::ES;
+  extern __shared__ unsigned char smem_dyn[];
+  unsigned char* smem = reinterpret_cast<unsigned char*>(((uintptr_t)smem_dyn + 1023) & ~(uintptr_t)1023);
+  __shared__ __align__(8) uint64_t bars[2 * (MAX_A + MAX_RAW + MAX_B + MAX_ACC)];
+  __shared__ uint32_t tmem_base_slot;
+  __shared__ volatile uint32_t abort_flag;
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int sub_bytes = q.rows * 128;
+  const uint32_t a_ring = smem_u32(smem);
+  const uint32_t b_ring = a_ring + q.sa * q.a_stage;
+  const uint32_t raw_ring = b_ring + q.sb * q.slot_bytes;
+  int32_t* tab = reinterpret_cast<int32_t*>(smem + q.sa * q.a_stage + q.sb * q.slot_bytes + q.sr * q.raw_slot);
+  const uint32_t a_full0 = smem_u32(&bars[0]), a_empty0 = a_full0 + 8 * MAX_A;
+  const uint32_t raw_full0 = a_empty0 + 8 * MAX_A, raw_empty0 = raw_full0 + 8 * MAX_RAW;
+  const uint32_t b_full0 = raw_empty0 + 8 * MAX_RAW, b_empty0 = b_full0 + 8 * MAX_B;
+  const uint32_t acc_full0 = b_empty0 + 8 * MAX_B, acc_empty0 = acc_full0 + 8 * MAX_ACC;
+
+  if (threadIdx.x == 0) {
+    abort_flag = 0u;
+    for (int i = 0; i < MAX_A; ++i) { mbar_init(a_full0 + 8 * i, 8); mbar_init(a_empty0 + 8 * i, 1); }
+    for (int i = 0; i < MAX_RAW; ++i) { mbar_init(raw_full0 + 8 * i, 1); mbar_init(raw_empty0 + 8 * i, 8); }
+    for (int i = 0; i < MAX_B; ++i) { mbar_init(b_full0 + 8 * i, 1); mbar_init(b_empty0 + 8 * i, 1); }
+    for (int i = 0; i < MAX_ACC; ++i) { mbar_init(acc_full0 + 8 * i, 1); mbar_init(acc_empty0 + 8 * i, 8); }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 11) tmem_alloc(smem_u32(&tmem_base_slot), 512);
+  // k2 -> byte inside the raw slot that holds it (low half) and the phase its channel adds (high half); -1: padded k2
+  for (int k = threadIdx.x; k < q.num_kb * KB; k += THREADS) {
+    int32_t entry = -1;
+    if (k < q.K2) {
+      const int c = k / q.E, c_lo = (k / q.rk * q.rk) / q.E;
+      entry = (c - c_lo) * q.region + (k - c * q.E) * ES;
+      if (PHASED) entry |= (int32_t)((((int64_t)c * q.chan_bytes) & 15) << 16);
+    }
+    tab[k] = entry;
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_acc = tmem_base_slot;
+  wait_for_previous_kernel();
+
+  if (warp < 8) {
+    // ---------------- staging: raw runs -> S ------------------------------------------------------------
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(F::REGS_STAGING));
+    const int wg = warp >> 2, row = threadIdx.x & 127;
+    const int cps = q.rk >> 3;                               // 16-byte units per row and raw slot
+    const int hrow = TILE_M + (int)threadIdx.x / cps, hch = (int)threadIdx.x % cps;     // halo item of this thread
+    const bool has_halo = hrow < TILE_M + q.halo;
+    const int slots_per_kb = KB / q.rk;
+    bool ok = true;
+    int sa = 0, sr = 0;
+    uint32_t pa = 0, pr = 0;
+    for (int w = blockIdx.x; w < q.nwork && ok; w += gridDim.x) {
+      const uint32_t q0 = (uint32_t)(w / q.ntn) * TILE_M;
+      const TileRuns tr = tile_runs(q, q0);
+      const int plane = (q.Ho * q.Wp + q.Wq * q.s - q.Wp) * q.Kh;   // (up to the end of the last virtual column)
+      // Byte of row r's first element inside a channel's region, and the phase of its image's runs (channel 0).
+      auto locate = [&](int r, uint32_t& off, uint32_t& phase) {
+        off = 0; phase = 0;
+        const uint32_t vq = q0 + r;
+        if (vq >= q.VQ) return;                              // dead rows read whatever lies at the start: they are dropped
+        uint32_t n;
+        int ho, i;
+        split_q(q, vq, n, ho, i);
+        if (i >= q.Wq) return;
+        const int g = (int)(n - tr.n0), start = g == 0 ? tr.start0 : 0;
+        if (g > 0) off = run_size(plane - tr.start0, ES) + (g - 1) * run_size(plane, ES);
+        off += ((ho * q.Wp + i * q.s) * q.Kh - start) * ES;
+        phase = (uint32_t)(((int64_t)n * q.img_bytes + (int64_t)start * ES) & 15);
+        if (!PHASED) off += phase;
+      };
+      uint32_t off, ph, hoff = 0, hph = 0;
+      locate(row, off, ph);
+      if (has_halo) locate(hrow, hoff, hph);
+      for (int kb = 0; kb < q.num_kb && ok; ++kb) {
+        const int nch = kb == q.num_kb - 1 ? 2 * q.nks_last : 8;     // units of the k2-block; the MMAs stop there
+        const uint32_t stage = a_ring + sa * q.a_stage;
+        ok = mbar_wait(a_empty0 + 8 * sa, pa ^ 1u, &abort_flag, q.status);
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        for (int r = 0; r < slots_per_kb; ++r) {
+          if (r * cps >= nch) break;
+          ok = mbar_wait(raw_full0 + 8 * sr, pr, &abort_flag, q.status);
+          ok = __all_sync(0xffffffffu, ok);
+          if (!ok) break;
+          const uint32_t raw = raw_ring + sr * q.raw_slot;
+          // One unit: the eight k2 of `ch` of one row.
+          auto unit = [&](uint32_t o, uint32_t phase, int srow, int ch) {
+            const int4* kt = reinterpret_cast<const int4*>(tab + kb * KB) + 2 * ch;
+            const int4 t0 = kt[0], t1 = kt[1];
+            const int32_t ent[8] = {t0.x, t0.y, t0.z, t0.w, t1.x, t1.y, t1.z, t1.w};
+            const uint32_t src = raw + o;
+            uint32_t addr[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+              if (PHASED) addr[e] = src + (ent[e] & 0xffff) + ((phase + ((uint32_t)ent[e] >> 16)) & 15u);
+              else addr[e] = src + ent[e];
+            }
+            const bool padded = ent[7] < 0;                  // (uniform: only the last unit of the reduction)
+            if (padded) {
+#pragma unroll
+              for (int e = 0; e < 8; ++e) if (ent[e] < 0) addr[e] = raw;
+            }
+            const uint32_t dst = stage + srow * 128 + ((ch ^ (srow & 7)) << 4);
+            if constexpr (F32) {
+              float v[8];
+#pragma unroll
+              for (int e = 0; e < 8; ++e) v[e] = ld_shared_f32(addr[e]);
+              if (padded) {
+#pragma unroll
+                for (int e = 0; e < 8; ++e) if (ent[e] < 0) v[e] = 0.f;
+              }
+              uint32_t p[3][4];
+#pragma unroll
+              for (int e = 0; e < 4; ++e) split2(v[2 * e], v[2 * e + 1], p[0][e], p[1][e], p[2][e]);
+#pragma unroll
+              for (int i = 0; i < 3; ++i) st_shared16(dst + i * sub_bytes, p[i][0], p[i][1], p[i][2], p[i][3]);
+            } else {
+              uint32_t v[8];
+#pragma unroll
+              for (int e = 0; e < 8; ++e) v[e] = ld_shared_u16(addr[e]);
+              if (padded) {
+#pragma unroll
+                for (int e = 0; e < 8; ++e) if (ent[e] < 0) v[e] = 0u;
+              }
+              st_shared16(dst, v[0] | (v[1] << 16), v[2] | (v[3] << 16), v[4] | (v[5] << 16), v[6] | (v[7] << 16));
+            }
+          };
+          const int half = cps >> 1;
+#pragma unroll 2
+          for (int c = 0; c < half; ++c) {
+            const int ch = r * cps + wg * half + c;
+            if (ch < nch) unit(off, ph, row, ch);
+          }
+          if (has_halo && r * cps + hch < nch) unit(hoff, hph, hrow, r * cps + hch);
+          __syncwarp();
+          if (lane == 0) mbar_arrive(raw_empty0 + 8 * sr);
+          if (++sr == q.sr) { sr = 0; pr ^= 1u; }
+        }
+        if (!ok) break;
+        fence_proxy_async_smem();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(a_full0 + 8 * sa);
+        if (++sa == q.sa) { sa = 0; pa ^= 1u; }
+      }
+    }
+  } else if (warp < 12) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(F::REGS_MISC));
+    if (warp == 8) {
+      // ---------------- MMA issuer -----------------------------------------------------------------------
+      const bool leader = elect_one();
+      const uint32_t a_lo0 = smem_desc_lo(a_ring), b_lo0 = smem_desc_lo(b_ring);
+      const uint32_t sub_lo = (uint32_t)sub_bytes >> 4;
+      const uint32_t id1 = instr_desc(F32, TILE_M, q.bn), id2 = instr_desc(F32, TILE_M, 2 * q.bn),
+                     id3 = instr_desc(F32, TILE_M, 3 * q.bn);
+      bool ok = true;
+      int sa = 0, slot = 0;
+      uint32_t pa = 0, pb = 0, ac = 0;                       // ... chains (fp32) or tiles (fp16) so far
+      for (int w = blockIdx.x; w < q.nwork && ok; w += gridDim.x) {
+        int links = 0;                                       // steps in the open chain; 0: none is open
+        if (q.resident) slot = 0;
+        for (int kb = 0; kb < q.num_kb && ok; ++kb) {
+          const int nks = kb == q.num_kb - 1 ? q.nks_last : KB / 16;
+          ok = mbar_wait(a_full0 + 8 * sa, pa, &abort_flag, q.status);
+          ok = __all_sync(0xffffffffu, ok);
+          if (!ok) break;
+          uint32_t a_view = a_lo0 + (uint32_t)(sa * (q.a_stage >> 4));
+          for (int g = 0; g < q.G; ++g, a_view += 8u) {      // next view: one row (128 bytes) further down
+            const int ab = ac & (F::NACC - 1);
+            if (links == 0) {
+              ok = mbar_wait(acc_empty0 + 8 * ab, ((ac >> F::ACC_LOG) & 1) ^ 1, &abort_flag, q.status);
+              ok = __all_sync(0xffffffffu, ok);
+              if (!ok) break;
+            }
+            const uint32_t d = tmem_acc + ab * F::ACC_COLS, more = links > 0;
+            links += nks;
+            const bool last_link = F32 ? links + nks > q.chain || g + 1 == q.G : kb + 1 == q.num_kb && g + 1 == q.G;
+            ok = mbar_wait(b_full0 + 8 * slot, pb, &abort_flag, q.status);
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok) break;
+            tc_fence_after();
+            const uint32_t b_lo = b_lo0 + (uint32_t)(slot * (q.slot_bytes >> 4));
+            if (leader) {
+              if constexpr (F32) {
+#pragma unroll
+                for (int j = 0; j < KB / 16; ++j)
+                  if (j < nks) umma_f16_lohi(d, a_view + 2 * j, b_lo + 2 * j, id3, more | (uint32_t)j);
+#pragma unroll
+                for (int j = 0; j < KB / 16; ++j)
+                  if (j < nks) umma_f16_lohi(d + q.bn, a_view + sub_lo + 2 * j, b_lo + 2 * j, id2, 1u);
+#pragma unroll
+                for (int j = 0; j < KB / 16; ++j)
+                  if (j < nks) umma_f16_lohi(d + 2 * q.bn, a_view + 2 * sub_lo + 2 * j, b_lo + 2 * j, id1, 1u);
+              } else {
+#pragma unroll
+                for (int j = 0; j < KB / 16; ++j)
+                  if (j < nks) umma_f16_lohi(d, a_view + 2 * j, b_lo + 2 * j, id1, more | (uint32_t)j);
+              }
+              if (!q.resident) umma_commit(b_empty0 + 8 * slot);
+              if (last_link) umma_commit(acc_full0 + 8 * ab);
+            }
+            __syncwarp();
+            if (last_link) { ++ac; links = 0; }
+            if (++slot == q.sb) { slot = 0; if (!q.resident) pb ^= 1u; }
+          }
+          if (ok && leader) umma_commit(a_empty0 + 8 * sa);
+          __syncwarp();
+          if (++sa == q.sa) { sa = 0; pa ^= 1u; }
+        }
+      }
+      (void)id2; (void)id3; (void)sub_lo;
+    } else if (warp == 9) {
+      // ---------------- filter copies ----------------------------------------------------------------------
+      const bool leader = elect_one();
+      bool ok = true;
+      int slot = 0;
+      uint32_t pb = 0;
+      for (int w = blockIdx.x; w < q.nwork && ok; w += gridDim.x) {
+        const unsigned char* src = q.fp + (int64_t)(w % q.ntn) * q.num_kb * q.G * q.slot_bytes;
+        for (int u = 0; u < q.num_kb * q.G; ++u, src += q.slot_bytes) {
+          ok = mbar_wait(b_empty0 + 8 * slot, pb ^ 1u, &abort_flag, q.status);
+          ok = __all_sync(0xffffffffu, ok);
+          if (!ok) break;
+          if (leader) {
+            mbar_arrive_expect_tx(b_full0 + 8 * slot, (uint32_t)q.slot_bytes);
+            bulk_load(b_ring + slot * q.slot_bytes, src, (uint32_t)q.slot_bytes, b_full0 + 8 * slot);
+          }
+          __syncwarp();
+          if (++slot == q.sb) { slot = 0; pb ^= 1u; }
+        }
+        if (q.resident) break;                               // the whole filter is in place
+      }
+      if (!ok) for (int i = 0; i < 64; ++i) __nanosleep(1000);   // copies in flight must land first
+    } else if (warp == 10) {
+      // ---------------- raw copies --------------------------------------------------------------------------
+      bool ok = true;
+      int sr = 0;
+      uint32_t pr = 0;
+      const int plane = (q.Ho * q.Wp + q.Wq * q.s - q.Wp) * q.Kh;
+      const int nslots = (q.K2 + q.rk - 1) / q.rk;           // (slots beyond the last real k2 are not read either)
+      for (int w = blockIdx.x; w < q.nwork && ok; w += gridDim.x) {
+        const TileRuns tr = tile_runs(q, (uint32_t)(w / q.ntn) * TILE_M);
+        const int nseg = (int)(tr.n1 - tr.n0) + 1;
+        for (int sl = 0; sl < nslots; ++sl) {
+          ok = mbar_wait(raw_empty0 + 8 * sr, pr ^ 1u, &abort_flag, q.status);
+          ok = __all_sync(0xffffffffu, ok);
+          if (!ok) break;
+          const uint32_t bar = raw_full0 + 8 * sr;
+          const int c0 = sl * q.rk / q.E;
+          int k1 = sl * q.rk + q.rk - 1;
+          if (k1 > q.K2 - 1) k1 = q.K2 - 1;
+          const int nc = k1 / q.E - c0 + 1;
+          int seg_off = 0;
+          for (int g = 0; g < nseg; ++g) {
+            const int start = g == 0 ? tr.start0 : 0, end = g == nseg - 1 ? tr.end1 : plane;
+            for (int c = lane; c < nc; c += 32) {
+              const int64_t b0 = (int64_t)(tr.n0 + g) * q.img_bytes + (int64_t)(c0 + c) * q.chan_bytes + (int64_t)start * ES;
+              const int64_t from = b0 & ~(int64_t)15;
+              const int64_t stop = b0 + (int64_t)(end - start) * ES;
+              int64_t to = (stop + 15) & ~(int64_t)15;
+              const uint32_t dst = raw_ring + sr * q.raw_slot + c * q.region + seg_off;
+              if (to > q.win_bytes) {                        // the tensor ends here: its last bytes by hand, zeros beyond
+                to = q.win_bytes & ~(int64_t)15;
+                for (int64_t b = to; b < stop; b += 2)
+                  asm volatile("st.shared.u16 [%0], %1;" ::"r"(dst + (uint32_t)(b - from)),
+                               "h"(b < q.win_bytes ? *reinterpret_cast<const uint16_t*>(q.win + b) : (uint16_t)0) : "memory");
+              }
+              if (to > from) {
+                mbar_expect_tx(bar, (uint32_t)(to - from));
+                bulk_load(dst, q.win + from, (uint32_t)(to - from), bar);
+              }
+            }
+            seg_off += run_size(end - start, ES);
+          }
+          __syncwarp();
+          if (lane == 0) mbar_arrive(bar);
+          if (++sr == q.sr) { sr = 0; pr ^= 1u; }
+        }
+      }
+      if (!ok) for (int i = 0; i < 64; ++i) __nanosleep(1000);
+    }
+    __syncwarp();
+  } else {
+    // ---------------- epilogue ---------------------------------------------------------------------------------
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(F::REGS_EPILOGUE));
+    const int lq = warp & 3, h = (warp - 12) >> 2;           // tensor-memory quadrant; which channels
+    bool ok = true;
+    uint32_t ac = 0;
+    for (int w = blockIdx.x; w < q.nwork && ok; w += gridDim.x) {
+      const int mt = w / q.ntn, nt = w - mt * q.ntn;
+      const uint32_t vq = (uint32_t)mt * TILE_M + (uint32_t)(lq * 32 + lane);
+      const int co0 = nt * q.bn;
+      const int limit = q.Co - co0 < q.bn ? q.Co - co0 : q.bn;            // channels of this tile that exist
+      uint32_t n = 0;
+      int ho = 0, i0 = 0;
+      bool valid = false;
+      if (vq < q.VQ) {
+        split_q(q, vq, n, ho, i0);
+        valid = i0 < q.Wo;                                   // trailing columns of a strip are no output
+      }
+      float* yrow = q.y + ((int64_t)n * q.Co + co0) * q.HoWo + (int64_t)ho * q.Wo + i0;
+      if constexpr (F32) {
+        float acc[F::CH][16];
+#pragma unroll
+        for (int j = 0; j < F::CH; ++j)
+#pragma unroll
+          for (int e = 0; e < 16; ++e) acc[j][e] = 0.f;
+        for (int kb = 0; kb < q.num_kb && ok; ++kb) {
+          const int nks = kb == q.num_kb - 1 ? q.nks_last : KB / 16;
+          const int units = q.chain / nks;                   // of one chain
+          for (int g = 0; g < q.G; g += units, ++ac) {
+            const int ab = ac & (F::NACC - 1);
+            ok = mbar_wait(acc_full0 + 8 * ab, (ac >> F::ACC_LOG) & 1, &abort_flag, q.status);
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok) break;
+            tc_fence_after();
+            const uint32_t d = tmem_acc + ((uint32_t)(lq * 32) << 16) + ab * F::ACC_COLS + h * 16;
+#pragma unroll
+            for (int j = 0; j < F::CH; ++j) {
+              if ((h + 2 * j) * 16 >= q.bn) break;
+              uint32_t r0[16], r1[16], r2[16];
+              tmem_ld16_issue(d + 32 * j, r0);
+              tmem_ld16_issue(d + 32 * j + q.bn, r1);
+              tmem_ld16_issue(d + 32 * j + 2 * q.bn, r2);
+              tmem_wait16(r0);
+              tmem_wait16(r1);
+              tmem_wait16(r2);
+#pragma unroll
+              for (int e = 0; e < 16; ++e)
+                acc[j][e] += __uint_as_float(r0[e]) + (__uint_as_float(r1[e]) + __uint_as_float(r2[e]));
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(acc_empty0 + 8 * ab);
+          }
+        }
+        if (!ok) break;
+        if (valid) {
+          bool again = false;
+#pragma unroll
+          for (int j = 0; j < F::CH; ++j) {
+            const int c0 = (h + 2 * j) * 16;
+            float *p0 = yrow + (int64_t)c0 * q.HoWo, *p1 = p0 + q.HoWo;
+#pragma unroll
+            for (int e = 0; e < 16; e += 2) {
+              if (c0 + e < limit) { *p0 = acc[j][e]; again |= suspicious(acc[j][e]); }
+              if (c0 + e + 1 < limit) { *p1 = acc[j][e + 1]; again |= suspicious(acc[j][e + 1]); }
+              p0 += 2 * (int64_t)q.HoWo; p1 += 2 * (int64_t)q.HoWo;
+            }
+          }
+          if (again) {
+            for (int c = h * 16; c < limit; c += (c & 15) == 15 ? 17 : 1)
+              if (suspicious(yrow[(int64_t)c * q.HoWo])) yrow[(int64_t)c * q.HoWo] = exact_output<F32>(q, n, ho, i0, nt, c);
+          }
+        }
+      } else {
+        const int ab = ac & (F::NACC - 1);
+        ok = mbar_wait(acc_full0 + 8 * ab, (ac >> F::ACC_LOG) & 1, &abort_flag, q.status);
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        ++ac;
+        tc_fence_after();
+        const uint32_t d = tmem_acc + ((uint32_t)(lq * 32) << 16) + ab * F::ACC_COLS;
+#pragma unroll 1
+        for (int c0 = h * (BNMAX / 2); c0 < (h + 1) * (BNMAX / 2) && c0 < limit; c0 += 32) {
+          uint32_t v[32];
+          tmem_ld32(d + c0, v);
+          if (c0 + 32 >= (h + 1) * (BNMAX / 2) || c0 + 32 >= limit) {      // the last read of this accumulator
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(acc_empty0 + 8 * ab);
+          }
+          if (valid) {
+            store_strided32(yrow + (int64_t)c0 * q.HoWo, q.HoWo, v, limit - c0);
+            float zero = 0.f;
+#pragma unroll
+            for (int j = 0; j < 32; ++j) zero = fmaf(__uint_as_float(c0 + j < limit ? v[j] : 0u), 0.f, zero);
+            if (zero != 0.f) {                               // (a NaN: one of them is not finite)
+              for (int c = c0; c < c0 + 32 && c < limit; ++c) {
+                float* p = yrow + (int64_t)c * q.HoWo;
+                if (!(fabsf(*p) <= 3.4028234663852886e38f)) *p = exact_output<F32>(q, n, ho, i0, nt, c);
+              }
+            }
+          }
+        }
+        if (h * (BNMAX / 2) >= limit) {                      // (no channels for this warp)
+          __syncwarp();
+          if (lane == 0) mbar_arrive(acc_empty0 + 8 * ab);
+        }
+      }
+    }
+  }
+
+  // ---------------- teardown -----------------------------------------------------------------------
+  tc_fence_before();
+  __syncthreads();
+  if (abort_flag) {
+    for (int i = 0; i < 64; ++i) __nanosleep(1000);
+    __syncthreads();
+  }
+  if (warp == 11) {
+    __syncwarp();
+    tc_fence_after();
+    tmem_dealloc(tmem_acc, 512);
+  }
+}
+
+// Filter -> the images the copy warp loads: for every (channel tile nt, k2-block kb, virtual kernel column g) the
+// pieces [bn channels][64 k2] in the 128-byte-swizzled order of shared memory (fp32: the three pieces side by side,
+// largest first).  One block: `rows` channels of one k2-block; per channel its source is one contiguous run of the OIHW
+// filter (whole input channels).  Channels beyond Co, k2 beyond C*E and kernel columns beyond Kw are zeros.
+template <bool F32>
+__global__ void __launch_bounds__(256) pack_runs_kernel(const void* __restrict__ f, unsigned char* __restrict__ fp,
+                                                        uint32_t* __restrict__ status, int C, int Kh, int Kw, int s, int E, int G,
+                                                        int Co, int bn, int num_kb, int rows, int pitch) {
+  using T = typename std::conditional<F32, float, uint16_t>::type;
+  constexpr int PIECES = F32 ? 3 : 1;
+  extern __shared__ __align__(16) unsigned char pack_raw[];
+  T* stage = reinterpret_cast<T*>(pack_raw);
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < kStatusBytes / 4) status[threadIdx.x] = 0u;
+  const int kb = blockIdx.x, row0 = blockIdx.y * rows;
+  const int c0 = kb * KB / E;
+  int c1 = (kb * KB + KB - 1) / E;
+  if (c1 > C - 1) c1 = C - 1;
+  const int T2 = Kh * Kw, run = (c1 - c0 + 1) * T2;
+  for (int r = 0; r < rows; ++r) {
+    const int co = row0 + r;
+    if (co >= Co) break;
+    const T* src = static_cast<const T*>(f) + ((int64_t)co * C + c0) * T2;
+    for (int i = threadIdx.x; i < run; i += blockDim.x) stage[r * pitch + i] = __ldg(src + i);
+  }
+  __syncthreads();
+  const int items = rows * G * 8;
+  for (int it = threadIdx.x; it < items; it += blockDim.x) {
+    const int ch = it & 7, rg = it >> 3;
+    const int r = rg % rows, g = rg / rows;
+    const int row = row0 + r, nt = row / bn, rr = row - nt * bn;
+    uint32_t p[PIECES][4] = {};
+    int k2 = kb * KB + ch * 8;
+    int c = k2 / E, e = k2 - c * E, t = e / Kh, u = e - t * Kh;
+#pragma unroll
+    for (int x = 0; x < 8; ++x) {
+      const int v = g * s + t;
+      T a = 0;
+      if (row < Co && c < C && v < Kw) a = stage[r * pitch + (c - c0) * T2 + u * Kw + v];
+      if (++u == Kh) { u = 0; if ((++t) * Kh == E) { t = 0; ++c; } }
+      if constexpr (F32) {
+        // The pieces of a finite element are finite (the first is cut where rounding would overflow); an
+        // infinity or NaN is its own first piece, the others are zero: the sum of the pieces is the element.
+        uint32_t b1 = cvt_bf16x2(a, 0.f) & 0xffffu, b2 = 0u, b3 = 0u;
+        if ((__float_as_uint(a) & 0x7f800000u) != 0x7f800000u) {
+          if ((b1 & 0x7f80u) == 0x7f80u) b1 = __float_as_uint(a) >> 16;
+          const float r1 = a - __uint_as_float(b1 << 16);
+          b2 = cvt_bf16x2(r1, 0.f) & 0xffffu;
+          b3 = cvt_bf16x2(r1 - __uint_as_float(b2 << 16), 0.f) & 0xffffu;
+        }
+        p[0][x >> 1] |= b1 << (16 * (x & 1));
+        p[PIECES - 2][x >> 1] |= b2 << (16 * (x & 1));
+        p[PIECES - 1][x >> 1] |= b3 << (16 * (x & 1));
+      } else {
+        p[0][x >> 1] |= (uint32_t)a << (16 * (x & 1));
+      }
+    }
+    const int64_t piece = (int64_t)bn * 128;
+    unsigned char* dst = fp + (((int64_t)nt * num_kb + kb) * G + g) * PIECES * piece + rr * 128 + ((ch ^ (rr & 7)) << 4);
+#pragma unroll
+    for (int i = 0; i < PIECES; ++i) *reinterpret_cast<uint4*>(dst + i * piece) = make_uint4(p[i][0], p[i][1], p[i][2], p[i][3]);
+  }
+}
+
+template <bool F32, int BNMAX, bool PHASED>
+cudaError_t launch_form(const RunsParams& q, int smem, cudaStream_t stream) {
+  static bool attr_done[64] = {};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+  if (!attr_done[dev]) {
+    cudaError_t e = cudaFuncSetAttribute(conv_runs_kernel<F32, BNMAX, PHASED>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRunsSmem);
+    if (e != cudaSuccess) return e;
+    attr_done[dev] = true;
+  }
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.gridDim = dim3((unsigned)(q.nwork < 148 ? q.nwork : 148), 1, 1);
+  cfg.blockDim = dim3(THREADS, 1, 1);
+  cfg.dynamicSmemBytes = (size_t)smem;
+  cfg.stream = stream;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, conv_runs_kernel<F32, BNMAX, PHASED>, q);
+}
+
+}  // namespace
+
+RunsPlan plan_runs(const Geometry& g, bool f32) {
+  RunsPlan p{};
+  p.eligible = false;
+  const int es = f32 ? 4 : 2, pieces = f32 ? 3 : 1;
+  const int nsub = g.s < g.Kw ? g.s : g.Kw;
+  const int64_t E = (int64_t)nsub * g.Kh, K2 = g.C * E;
+  if (K2 > 6144 || E > 256 || g.chan_stride >= ((int64_t)1 << 30)) return p;
+  p.E = (int32_t)E;
+  p.G = (g.Kw + g.s - 1) / g.s;
+  p.num_kb = (int32_t)((K2 + KB - 1) / KB);
+  p.nks_last = (int32_t)((K2 - (int64_t)(p.num_kb - 1) * KB + 15) / 16);
+  p.halo = p.G - 1;
+  p.Wq = (g.Wp + g.s - 1) / g.s;
+  p.pitch = p.Wq;
+  // Rows of a strip start at multiples of eight where that puts every warp's stores on 32-byte sectors.
+  bool widen = g.Wo % 8 == 0;
+  if (const char* v = debug_getenv("IM2WIN_RUNS_PITCH")) widen = v[0] == '8';          // testing aid
+  if (widen) p.pitch = (p.Wq + 7) / 8 * 8;
+  p.VQ = (int64_t)g.N * g.Ho * p.pitch;
+  if (p.VQ + 2 * TILE_M >= ((int64_t)1 << 31)) return p;
+  p.rows = TILE_M + (p.halo + 7) / 8 * 8;
+  p.a_stage = pieces * p.rows * 128;
+  const int64_t per_img = (int64_t)g.Ho * p.pitch;
+  const int64_t segs = (TILE_M + p.halo - 2) / per_img + 2;
+  if (segs > MAX_SEG) return p;
+  // bytes a tile's columns of one channel take in a raw slot, whatever the tile
+  const int64_t region = (int64_t)(TILE_M + p.halo) * g.s * g.Kh * es + segs * 32;
+  p.region = (int32_t)((region + 15) / 16 * 16);
+  const int most = f32 ? 80 : 256;
+  p.ntn = (g.Co + most - 1) / most;
+  p.bn = ((g.Co + p.ntn - 1) / p.ntn + 15) / 16 * 16;
+  p.ntn = (g.Co + p.bn - 1) / p.bn;
+  p.slot_bytes = pieces * p.bn * 128;
+  const int64_t ntm = (p.VQ + TILE_M - 1) / TILE_M;
+  if (ntm * p.ntn >= ((int64_t)1 << 30)) return p;
+  p.nwork = (int32_t)(ntm * p.ntn);
+  const int units = p.num_kb * p.G;
+  const int budget = kRunsSmem - 1024 - p.num_kb * KB * 4;
+  // Rings: raw slots of 64, 32 or 16 k2, the largest of which three fit beside two S stages and the filter
+  // (resident where one channel tile's fits, else at least three units).
+  for (int pass = 0; pass < 4 && !p.eligible; ++pass) {
+    const bool resident = (pass & 1) == 0 && p.ntn == 1 && units <= MAX_B;
+    if ((pass & 1) == 0 && !resident) continue;
+    const int least_raw = pass < 2 ? 3 : 2;
+    const int least_b = resident ? units : (f32 ? 2 : 3);
+    for (int rk = 64; rk >= 16; rk /= 2) {
+      int64_t nch = (rk + E - 2) / E + 1;
+      if (nch > g.C) nch = g.C;
+      const int64_t raw = (nch * p.region + 127) / 128 * 128;
+      if (raw >= 65536 || (p.halo * (rk / 8)) > 256) continue;
+      if (2 * p.a_stage + least_b * p.slot_bytes + least_raw * raw > budget) continue;
+      p.rk = rk;
+      p.raw_slot = (int32_t)raw;
+      p.resident = resident;
+      p.sa = 2; p.sr = least_raw; p.sb = least_b;
+      auto fits = [&](int a, int r, int b) { return (int64_t)a * p.a_stage + (int64_t)r * raw + (int64_t)b * p.slot_bytes <= budget; };
+      if (!resident) while (p.sb < 4 && fits(p.sa, p.sr, p.sb + 1)) ++p.sb;
+      if (!f32 && fits(3, p.sr, p.sb)) p.sa = 3;
+      while (p.sr < MAX_RAW && fits(p.sa, p.sr + 1, p.sb)) ++p.sr;
+      if (!resident) while (p.sb < MAX_B && fits(p.sa, p.sr, p.sb + 1)) ++p.sb;
+      p.eligible = true;
+      break;
+    }
+  }
+  p.phased = (g.chan_stride * es) % 16 != 0;
+  p.filter_bytes = (size_t)p.ntn * p.bn * p.num_kb * KB * p.G * 2 * pieces;
+  return p;
+}
+
+cudaError_t launch_pack_runs(const void* filter, void* scratch, const Geometry& g, bool f32, cudaStream_t stream) {
+  const RunsPlan p = plan_runs(g, f32);
+  if (!p.eligible) return cudaErrorInvalidValue;
+  unsigned char* base = static_cast<unsigned char*>(scratch);
+  const int es = f32 ? 4 : 2;
+  int64_t nch = (KB + p.E - 2) / p.E + 1;
+  if (nch > g.C) nch = g.C;
+  const int64_t pitch = nch * g.T;
+  int rows = 8;                                             // channels per block: staging within 40 KB
+  while (rows > 1 && rows * pitch * es > 40 * 1024) rows /= 2;
+  const size_t smem = (size_t)(rows * pitch * es);
+  if (smem > 48 * 1024) return cudaErrorInvalidValue;
+  dim3 grid((unsigned)p.num_kb, (unsigned)(p.ntn * p.bn / rows));
+  if (grid.y > 65535) return cudaErrorInvalidValue;
+  uint32_t* status = reinterpret_cast<uint32_t*>(base);
+  if (f32)
+    pack_runs_kernel<true><<<grid, 256, smem, stream>>>(filter, base + kStatusBytes, status, g.C, g.Kh, g.Kw, g.s, p.E, p.G, g.Co,
+                                                        p.bn, p.num_kb, rows, (int)pitch);
+  else
+    pack_runs_kernel<false><<<grid, 256, smem, stream>>>(filter, base + kStatusBytes, status, g.C, g.Kh, g.Kw, g.s, p.E, p.G, g.Co,
+                                                         p.bn, p.num_kb, rows, (int)pitch);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_conv_runs(const void* window, float* y, void* scratch, const Geometry& g, bool f32, cudaStream_t stream) {
+  const RunsPlan p = plan_runs(g, f32);
+  if (!p.eligible) return cudaErrorInvalidValue;
+  unsigned char* base = static_cast<unsigned char*>(scratch);
+  const int64_t es = f32 ? 4 : 2;
+  RunsParams q;
+  q.win = static_cast<const unsigned char*>(window);
+  q.fp = base + kStatusBytes;
+  q.y = y;
+  q.status = reinterpret_cast<uint32_t*>(base);
+  q.img_bytes = g.img_stride * es; q.chan_bytes = g.chan_stride * es; q.win_bytes = g.window_elems * es;
+  q.VQ = (uint32_t)p.VQ;
+  q.C = g.C; q.N = g.N; q.Wp = g.Wp; q.Wq = p.Wq; q.pitch = p.pitch; q.Ho = g.Ho; q.Wo = g.Wo; q.HoWo = g.Ho * g.Wo;
+  q.Co = g.Co; q.Kh = g.Kh; q.Kw = g.Kw; q.s = g.s;
+  q.E = p.E; q.G = p.G; q.K2 = g.C * p.E; q.num_kb = p.num_kb; q.nks_last = p.nks_last;
+  q.col_bytes = (int32_t)(g.s * g.Kh * es);
+  q.rows = p.rows; q.halo = p.halo; q.region = p.region; q.rk = p.rk; q.raw_slot = p.raw_slot; q.a_stage = p.a_stage;
+  q.bn = p.bn; q.ntn = p.ntn; q.nwork = p.nwork; q.sa = p.sa; q.sr = p.sr; q.sb = p.sb;
+  q.slot_bytes = p.slot_bytes; q.resident = p.resident ? 1 : 0;
+  q.chain = g.K >= 288 ? 12 : 8;
+  const int smem = 1024 + p.sa * p.a_stage + p.sb * p.slot_bytes + p.sr * p.raw_slot + p.num_kb * KB * 4;
+#define IM2WIN_RUNS(F32_, BN_) (p.phased ? launch_form<F32_, BN_, true>(q, smem, stream) : launch_form<F32_, BN_, false>(q, smem, stream))
+  if (f32) return IM2WIN_RUNS(true, 80);
+  if (p.bn <= 64) return IM2WIN_RUNS(false, 64);
+  if (p.bn <= 128) return IM2WIN_RUNS(false, 128);
+  return IM2WIN_RUNS(false, 256);
+#undef IM2WIN_RUNS
+}
+
+}  // namespace im2win
