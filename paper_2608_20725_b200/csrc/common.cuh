@@ -134,9 +134,9 @@ F32SplitPlan plan_f32_split(const Geometry& g);
 
 // Tile and ring geometry of the run-staged kernel, fp16 or fp32 operands (see conv_runs.cu).
 struct RunsPlan {
-  bool eligible, resident, phased;     // phased: channel planes differ in their place inside 16 bytes
-  int32_t E, G, Wq, pitch, rows, halo, num_kb, nks_last;
-  int32_t region, rk, raw_slot, a_stage, slot_bytes;
+  bool eligible, resident, quad;       // quad: up to four channels, see the order of k2 there
+  int32_t units, octs, E, G, Wq, pitch, rows, halo, num_kb, nks_last;
+  int32_t region, raw_slot, a_stage, slot_bytes;
   int32_t bn, ntn, nwork, sa, sr, sb;
   int64_t VQ;
   size_t filter_bytes;

@@ -5,18 +5,25 @@
 // strips or images and takes every stride.
 //
 // Columns.  In the im2win tensor the s*Kh elements of columns i*s .. i*s + s - 1 of a strip are contiguous, so a
-// convolution of stride s is one of stride 1 on columns s times as tall: virtual column i holds
-// e = t*Kh + u (t < min(s, Kw)), k2 = c*E + e with E = min(s, Kw)*Kh, and the kernel is G = ceil(Kw/s) virtual columns
-// wide; filter elements with g*s + t >= Kw are zeros (3x3 with stride 2: a third more products, but every element is
-// staged once and from one run).  A GEMM row is a virtual position q = (n*Ho + ho)*pitch + i; S[row][64 k2] is staged
-// once per k2-block and the MMAs of virtual kernel column g read the view that starts g rows further down.
+// convolution of stride s is one of stride 1 on columns s times as tall: virtual column i holds e = t*Kh + u
+// (t < min(s, Kw)), E = min(s, Kw)*Kh of them, and the kernel is G = ceil(Kw/s) virtual columns wide; filter elements
+// with g*s + t >= Kw are zeros (3x3 with stride 2: a third more products, but every element is staged once and from
+// one run).  A GEMM row is a virtual position q = (n*Ho + ho)*pitch + i; S[row][64 k2] is staged once per k2-block and
+// the MMAs of virtual kernel column g read the view that starts g rows further down.
+//
+// Order of k2.  A unit of eight k2 (16 bytes of S) is eight channels at one e: unit j = octet * E + e (up to four
+// channels: four channels at two e).  The places of a row's elements in the eight channel planes are then the same
+// for every unit but for one uniform offset -- also where planes start at different phases of 16 bytes, because
+// eight planes further the phase repeats -- and a unit costs a thread eight 2- or 4-byte shared loads, four
+// packs and one store.  (With k2 = c*E + e and a table of offsets a unit took 225 instructions and the kernel was bound by
+// them: 114 us where this one takes XXX, 3x3 on 64 channels at 56x56, batch 128, fp16.)
 //
 // Staging.  The columns a tile needs of one channel are one contiguous run per image it touches: an untiled bulk
-// copy from the 16-byte boundary below to the one above brings it into a ring of raw slots (RK k2 each: the channels
-// of RK consecutive k2).  Eight warps then read the elements of their rows back (2- or 4-byte shared loads, the phase
-// of each channel's run added to the address), split them (fp32) and write 16-byte units of S.  Gathering with global
-// loads instead (conv_f16_shift.cu, conv_f32_split.cu) makes every load instruction touch 32 rows s*Kh elements apart:
-// three or more L1 wavefronts each, and a round trip to memory per batch.
+// copy from the 16-byte boundary below to the one above brings it into a ring of raw slots (`octs` octets of
+// channels each).  Four warpgroups take the units in turn, read the elements of their rows back (thread = row), split
+// them (fp32) and write the units of S.  Gathering with global loads instead (conv_f16_shift.cu, conv_f32_split.cu)
+// makes every load instruction touch 32 rows s*Kh elements apart: three or more L1 wavefronts each, and a round trip
+// to memory per batch.
 //
 // What bounds it: the shared-memory pipe, which carries the MMA's operand reads (32 + N/4 cycles per instruction of
 // M = 128, K = 16), the copies, the read-back and the S stores.
@@ -40,7 +47,19 @@ constexpr int KB = 64;
 constexpr int MAX_A = 4, MAX_RAW = 8, MAX_B = 16, MAX_ACC = 8;
 constexpr int MAX_SEG = 6;                    // images a tile may touch
 constexpr int kRunsSmem = 226 * 1024;
-constexpr int THREADS = 640;                  // 8 staging warps, 4 single-role warps, 8 epilogue warps
+constexpr int STAGING_WARPS = 16;
+constexpr int THREADS = 32 * (STAGING_WARPS + 4 + 8);   // staging; MMA, filter copies, two raw-copy warps; epilogue
+
+// n / d for n below 2^31: (n * mul) >> shift with mul = floor(2^shift / d) + 1, shift = 31 + ceil(log2 d).
+struct FastDiv {
+  uint32_t mul, shift;
+  __device__ __forceinline__ uint32_t operator()(uint32_t n) const { return (uint32_t)(((uint64_t)n * mul) >> shift); }
+};
+FastDiv fast_div(uint32_t d) {
+  uint32_t l = 0;
+  while (((uint64_t)1 << l) < d) ++l;
+  return {(uint32_t)((((uint64_t)1 << (31 + l)) / d) + 1), 31 + l};
+}
 
 struct RunsParams {
   const unsigned char* __restrict__ win;
@@ -49,10 +68,11 @@ struct RunsParams {
   uint32_t* status;
   int64_t img_bytes, chan_bytes, win_bytes;   // of one image, one channel plane, the whole window tensor
   uint32_t VQ;
+  FastDiv div_pitch, div_ho;
   int32_t C, N, Wp, Wq, pitch, Ho, Wo, HoWo, Co, Kh, Kw, s;
-  int32_t E, G, K2, num_kb, nks_last;
-  int32_t col_bytes;                          // distance of neighbouring virtual columns: s*Kh elements
-  int32_t rows, halo, region, rk, raw_slot, a_stage;
+  int32_t E, G, units, num_kb, nks_last;      // units: of eight k2
+  int32_t quad;                               // 1: up to four channels, a unit is four channels at two e
+  int32_t rows, halo, region, octs, raw_slot, a_stage;
   int32_t bn, ntn, nwork, sa, sr, sb, slot_bytes, resident, chain;
 };
 
@@ -74,12 +94,12 @@ __device__ __forceinline__ void st_shared16(uint32_t addr, uint32_t a, uint32_t 
 }
 __device__ __forceinline__ uint32_t ld_shared_u16(uint32_t addr) {
   uint16_t v;
-  asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(addr));
+  asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(addr) : "memory");
   return v;
 }
 __device__ __forceinline__ float ld_shared_f32(uint32_t addr) {
   float v;
-  asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr));
+  asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
   return v;
 }
 __device__ __forceinline__ void tmem_ld16_issue(uint32_t taddr, uint32_t (&r)[16]) {
@@ -114,7 +134,7 @@ template <bool F32, int BNMAX> struct Form {
   static constexpr int NACC = 512 / ACC_COLS;
   static constexpr int ACC_LOG = NACC == 2 ? 1 : (NACC == 4 ? 2 : 3);
   static constexpr int CH = (BNMAX + 31) / 32;              // 16-channel chunks per epilogue warp
-  static constexpr int REGS_STAGING = 80, REGS_MISC = 64, REGS_EPILOGUE = 128;   // 2*80 + 64 + 2*128 = 5*96
+  static constexpr int REGS_STAGING = 56, REGS_MISC = 56, REGS_EPILOGUE = 112;   // 4*56 + 56 + 2*112 = 7*72
 };
 
 // Where the rows of a tile lie: image n0 + g of the tile is a run of its own, [start, end) in elements of a channel
@@ -125,9 +145,9 @@ struct TileRuns {
 };
 __device__ __forceinline__ int run_size(int elems, int es) { return (elems * es + 30) & ~15; }
 __device__ __forceinline__ void split_q(const RunsParams& q, uint32_t vq, uint32_t& n, int& ho, int& i) {
-  const uint32_t sg = vq / (uint32_t)q.pitch;
+  const uint32_t sg = q.div_pitch(vq);
   i = (int)(vq - sg * (uint32_t)q.pitch);
-  n = sg / (uint32_t)q.Ho;
+  n = q.div_ho(sg);
   ho = (int)(sg - n * (uint32_t)q.Ho);
 }
 __device__ __forceinline__ TileRuns tile_runs(const RunsParams& q, uint32_t q0) {
@@ -157,8 +177,9 @@ __device__ __forceinline__ float exact_output(const RunsParams& q, uint32_t n, i
   for (int c = 0; c < q.C; ++c)
     for (int v = 0; v < q.Kw; ++v)
       for (int u = 0; u < q.Kh; ++u) {
-        const int g = v / q.s, k2 = c * q.E + (v - g * q.s) * q.Kh + u, kb = k2 / KB, e = k2 - kb * KB;
-        const unsigned char* f = frow + ((int64_t)kb * q.G + g) * PIECES * piece + ((((e >> 3) ^ (col & 7)) << 4) | ((e & 7) * 2));
+        const int g = v / q.s, e = (v - g * q.s) * q.Kh + u;
+        const int j = q.quad ? e >> 1 : (c >> 3) * q.E + e, at = q.quad ? (e & 1) * 4 + c : c & 7;      // unit, place in it
+        const unsigned char* f = frow + ((int64_t)(j >> 3) * q.G + g) * PIECES * piece + ((((j & 7) ^ (col & 7)) << 4) | (at * 2));
         const unsigned char* x = wbase + c * q.chan_bytes + (v * q.Kh + u) * ES;
         if constexpr (F32) {
           auto part = [&](int p) { return __uint_as_float((uint32_t)*reinterpret_cast<const uint16_t*>(f + p * piece) << 16); };
@@ -170,7 +191,7 @@ __device__ __forceinline__ float exact_output(const RunsParams& q, uint32_t n, i
   return acc;
 }
 
-template <bool F32, int BNMAX, bool PHASED>
+template <bool F32, int BNMAX>
 __global__ void __launch_bounds__(THREADS, 1) conv_runs_kernel(RunsParams q) {
   using F = Form<F32, BNMAX>;
   constexpr int ES = F::ES;
@@ -185,7 +206,6 @@ __global__ void __launch_bounds__(THREADS, 1) conv_runs_kernel(RunsParams q) {
   const uint32_t a_ring = smem_u32(smem);
   const uint32_t b_ring = a_ring + q.sa * q.a_stage;
   const uint32_t raw_ring = b_ring + q.sb * q.slot_bytes;
-  int32_t* tab = reinterpret_cast<int32_t*>(smem + q.sa * q.a_stage + q.sb * q.slot_bytes + q.sr * q.raw_slot);
   const uint32_t a_full0 = smem_u32(&bars[0]), a_empty0 = a_full0 + 8 * MAX_A;
   const uint32_t raw_full0 = a_empty0 + 8 * MAX_A, raw_empty0 = raw_full0 + 8 * MAX_RAW;
   const uint32_t b_full0 = raw_empty0 + 8 * MAX_RAW, b_empty0 = b_full0 + 8 * MAX_B;
@@ -193,137 +213,129 @@ __global__ void __launch_bounds__(THREADS, 1) conv_runs_kernel(RunsParams q) {
 
   if (threadIdx.x == 0) {
     abort_flag = 0u;
-    for (int i = 0; i < MAX_A; ++i) { mbar_init(a_full0 + 8 * i, 8); mbar_init(a_empty0 + 8 * i, 1); }
-    for (int i = 0; i < MAX_RAW; ++i) { mbar_init(raw_full0 + 8 * i, 1); mbar_init(raw_empty0 + 8 * i, 8); }
+    for (int i = 0; i < MAX_A; ++i) { mbar_init(a_full0 + 8 * i, STAGING_WARPS); mbar_init(a_empty0 + 8 * i, 1); }
+    for (int i = 0; i < MAX_RAW; ++i) { mbar_init(raw_full0 + 8 * i, 1); mbar_init(raw_empty0 + 8 * i, STAGING_WARPS); }
     for (int i = 0; i < MAX_B; ++i) { mbar_init(b_full0 + 8 * i, 1); mbar_init(b_empty0 + 8 * i, 1); }
     for (int i = 0; i < MAX_ACC; ++i) { mbar_init(acc_full0 + 8 * i, 1); mbar_init(acc_empty0 + 8 * i, 8); }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 11) tmem_alloc(smem_u32(&tmem_base_slot), 512);
-  // k2 -> byte inside the raw slot that holds it (low half) and the phase its channel adds (high half); -1: padded k2
-  for (int k = threadIdx.x; k < q.num_kb * KB; k += THREADS) {
-    int32_t entry = -1;
-    if (k < q.K2) {
-      const int c = k / q.E, c_lo = (k / q.rk * q.rk) / q.E;
-      entry = (c - c_lo) * q.region + (k - c * q.E) * ES;
-      if (PHASED) entry |= (int32_t)((((int64_t)c * q.chan_bytes) & 15) << 16);
-    }
-    tab[k] = entry;
-  }
+  if (warp == STAGING_WARPS) tmem_alloc(smem_u32(&tmem_base_slot), 512);
+  // The raw ring starts as zeros: places no copy fills (channels beyond C in the last octet) meet zero filter
+  // elements, but they have to be numbers.
+  for (int i = threadIdx.x * 16; i < q.sr * q.raw_slot; i += THREADS * 16) st_shared16(raw_ring + i, 0u, 0u, 0u, 0u);
+  fence_proxy_async_smem();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_acc = tmem_base_slot;
   wait_for_previous_kernel();
 
-  if (warp < 8) {
+  if (warp < STAGING_WARPS) {
     // ---------------- staging: raw runs -> S ------------------------------------------------------------
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(F::REGS_STAGING));
+    // Warpgroup wg takes the units j = wg mod 4 of a stage.  Every warp passes every stage and every slot in order, so
+    // no wait by phase parity can run ahead.
     const int wg = warp >> 2, row = threadIdx.x & 127;
-    const int cps = q.rk >> 3;                               // 16-byte units per row and raw slot
-    const int hrow = TILE_M + (int)threadIdx.x / cps, hch = (int)threadIdx.x % cps;     // halo item of this thread
-    const bool has_halo = hrow < TILE_M + q.halo;
-    const int slots_per_kb = KB / q.rk;
+    const int plane = (q.Ho * q.Wp + q.Wq * q.s - q.Wp) * q.Kh;   // (up to the end of the last virtual column)
+    const int per_slot = q.quad ? q.units : q.octs * q.E;
+    const uint32_t oct_step = 8u * q.region - (uint32_t)(q.E - 1) * ES, unit_step = q.quad ? 2u * ES : ES;
     bool ok = true;
     int sa = 0, sr = 0;
     uint32_t pa = 0, pr = 0;
     for (int w = blockIdx.x; w < q.nwork && ok; w += gridDim.x) {
       const uint32_t q0 = (uint32_t)(w / q.ntn) * TILE_M;
       const TileRuns tr = tile_runs(q, q0);
-      const int plane = (q.Ho * q.Wp + q.Wq * q.s - q.Wp) * q.Kh;   // (up to the end of the last virtual column)
-      // Byte of row r's first element inside a channel's region, and the phase of its image's runs (channel 0).
-      auto locate = [&](int r, uint32_t& off, uint32_t& phase) {
-        off = 0; phase = 0;
+      // Place of row r's first element in channel x of a slot's octet: byte inside the raw slot.
+      auto locate = [&](int r, uint32_t (&rb)[8]) {
+        uint32_t off = 0, phase = 0;
         const uint32_t vq = q0 + r;
-        if (vq >= q.VQ) return;                              // dead rows read whatever lies at the start: they are dropped
-        uint32_t n;
-        int ho, i;
-        split_q(q, vq, n, ho, i);
-        if (i >= q.Wq) return;
-        const int g = (int)(n - tr.n0), start = g == 0 ? tr.start0 : 0;
-        if (g > 0) off = run_size(plane - tr.start0, ES) + (g - 1) * run_size(plane, ES);
-        off += ((ho * q.Wp + i * q.s) * q.Kh - start) * ES;
-        phase = (uint32_t)(((int64_t)n * q.img_bytes + (int64_t)start * ES) & 15);
-        if (!PHASED) off += phase;
+        if (vq < q.VQ) {                                     // dead rows read whatever lies at the start: they are dropped
+          uint32_t n;
+          int ho, i;
+          split_q(q, vq, n, ho, i);
+          if (i < q.Wq) {
+            const int g = (int)(n - tr.n0), start = g == 0 ? tr.start0 : 0;
+            if (g > 0) off = run_size(plane - tr.start0, ES) + (g - 1) * run_size(plane, ES);
+            off += ((ho * q.Wp + i * q.s) * q.Kh - start) * ES;
+            phase = (uint32_t)((int64_t)n * q.img_bytes + (int64_t)start * ES);
+          }
+        }
+#pragma unroll
+        for (int x = 0; x < 8; ++x) rb[x] = off + x * q.region + ((phase + (uint32_t)x * (uint32_t)q.chan_bytes) & 15u);
+        if (q.quad) {
+#pragma unroll
+          for (int x = 0; x < 4; ++x) rb[4 + x] = rb[x] + ES;
+        }
       };
-      uint32_t off, ph, hoff = 0, hph = 0;
-      locate(row, off, ph);
-      if (has_halo) locate(hrow, hoff, hph);
+      uint32_t rb[8], hb[8];
+      locate(row, rb);
+      if (lane < q.halo) locate(TILE_M + lane, hb);
+      uint32_t src = 0;                                      // of the current unit; inside the slot: its number, and its e
+      int in_slot = 0, e = 0;
       for (int kb = 0; kb < q.num_kb && ok; ++kb) {
-        const int nch = kb == q.num_kb - 1 ? 2 * q.nks_last : 8;     // units of the k2-block; the MMAs stop there
-        const uint32_t stage = a_ring + sa * q.a_stage;
         ok = mbar_wait(a_empty0 + 8 * sa, pa ^ 1u, &abort_flag, q.status);
         ok = __all_sync(0xffffffffu, ok);
         if (!ok) break;
-        for (int r = 0; r < slots_per_kb; ++r) {
-          if (r * cps >= nch) break;
-          ok = mbar_wait(raw_full0 + 8 * sr, pr, &abort_flag, q.status);
-          ok = __all_sync(0xffffffffu, ok);
-          if (!ok) break;
-          const uint32_t raw = raw_ring + sr * q.raw_slot;
-          // One unit: the eight k2 of `ch` of one row.
-          auto unit = [&](uint32_t o, uint32_t phase, int srow, int ch) {
-            const int4* kt = reinterpret_cast<const int4*>(tab + kb * KB) + 2 * ch;
-            const int4 t0 = kt[0], t1 = kt[1];
-            const int32_t ent[8] = {t0.x, t0.y, t0.z, t0.w, t1.x, t1.y, t1.z, t1.w};
-            const uint32_t src = raw + o;
-            uint32_t addr[8];
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-              if (PHASED) addr[e] = src + (ent[e] & 0xffff) + ((phase + ((uint32_t)ent[e] >> 16)) & 15u);
-              else addr[e] = src + ent[e];
-            }
-            const bool padded = ent[7] < 0;                  // (uniform: only the last unit of the reduction)
-            if (padded) {
-#pragma unroll
-              for (int e = 0; e < 8; ++e) if (ent[e] < 0) addr[e] = raw;
-            }
-            const uint32_t dst = stage + srow * 128 + ((ch ^ (srow & 7)) << 4);
-            if constexpr (F32) {
-              float v[8];
-#pragma unroll
-              for (int e = 0; e < 8; ++e) v[e] = ld_shared_f32(addr[e]);
-              if (padded) {
-#pragma unroll
-                for (int e = 0; e < 8; ++e) if (ent[e] < 0) v[e] = 0.f;
-              }
-              uint32_t p[3][4];
-#pragma unroll
-              for (int e = 0; e < 4; ++e) split2(v[2 * e], v[2 * e + 1], p[0][e], p[1][e], p[2][e]);
-#pragma unroll
-              for (int i = 0; i < 3; ++i) st_shared16(dst + i * sub_bytes, p[i][0], p[i][1], p[i][2], p[i][3]);
-            } else {
-              uint32_t v[8];
-#pragma unroll
-              for (int e = 0; e < 8; ++e) v[e] = ld_shared_u16(addr[e]);
-              if (padded) {
-#pragma unroll
-                for (int e = 0; e < 8; ++e) if (ent[e] < 0) v[e] = 0u;
-              }
-              st_shared16(dst, v[0] | (v[1] << 16), v[2] | (v[3] << 16), v[4] | (v[5] << 16), v[6] | (v[7] << 16));
-            }
-          };
-          const int half = cps >> 1;
-#pragma unroll 2
-          for (int c = 0; c < half; ++c) {
-            const int ch = r * cps + wg * half + c;
-            if (ch < nch) unit(off, ph, row, ch);
+        const uint32_t stage = a_ring + sa * q.a_stage;
+        const int n_units = q.units - 8 * kb < 8 ? q.units - 8 * kb : 8;
+        for (int ch = 0; ch < n_units; ++ch) {
+          if (in_slot == 0) {
+            ok = mbar_wait(raw_full0 + 8 * sr, pr, &abort_flag, q.status);
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok) break;
+            src = raw_ring + sr * q.raw_slot;
+            e = 0;
           }
-          if (has_halo && r * cps + hch < nch) unit(hoff, hph, hrow, r * cps + hch);
-          __syncwarp();
-          if (lane == 0) mbar_arrive(raw_empty0 + 8 * sr);
-          if (++sr == q.sr) { sr = 0; pr ^= 1u; }
+          if ((ch & 3) == wg) {
+            auto unit = [&](const uint32_t (&at)[8], int srow) {
+              const uint32_t dst = stage + srow * 128 + ((ch ^ (srow & 7)) << 4);
+              if constexpr (F32) {
+                float v[8];
+#pragma unroll
+                for (int x = 0; x < 8; ++x) v[x] = ld_shared_f32(src + at[x]);
+                uint32_t p[3][4];
+#pragma unroll
+                for (int x = 0; x < 4; ++x) split2(v[2 * x], v[2 * x + 1], p[0][x], p[1][x], p[2][x]);
+#pragma unroll
+                for (int i = 0; i < 3; ++i) st_shared16(dst + i * sub_bytes, p[i][0], p[i][1], p[i][2], p[i][3]);
+              } else {
+                uint32_t v[8];
+#pragma unroll
+                for (int x = 0; x < 8; ++x) v[x] = ld_shared_u16(src + at[x]);
+                st_shared16(dst, v[0] | (v[1] << 16), v[2] | (v[3] << 16), v[4] | (v[5] << 16), v[6] | (v[7] << 16));
+              }
+            };
+            unit(rb, row);
+            // the rows below the tile: lanes of one of the warpgroup's warps, another one from unit to unit
+            if ((((8 * kb + ch) >> 2) & 3) == (warp & 3) && lane < q.halo) unit(hb, TILE_M + lane);
+          }
+          const bool last = 8 * kb + ch == q.units - 1;
+          if (++in_slot == per_slot || last) {
+            __syncwarp();
+            if (lane == 0) mbar_arrive(raw_empty0 + 8 * sr);
+            if (++sr == q.sr) { sr = 0; pr ^= 1u; }
+            in_slot = 0;
+          }
+          ++e;
+          src += e == q.E ? oct_step : unit_step;
+          if (e == q.E) e = 0;
         }
         if (!ok) break;
+        if ((n_units & 1) != 0 && (n_units & 3) == wg) {     // zeros up to the end of the MMA's last step
+          for (int i = 0; i < (F32 ? 3 : 1); ++i) {
+            st_shared16(stage + i * sub_bytes + row * 128 + ((n_units ^ (row & 7)) << 4), 0u, 0u, 0u, 0u);
+            if (lane < q.halo) st_shared16(stage + i * sub_bytes + (TILE_M + lane) * 128 + ((n_units ^ (lane & 7)) << 4), 0u, 0u, 0u, 0u);
+          }
+        }
         fence_proxy_async_smem();
         __syncwarp();
         if (lane == 0) mbar_arrive(a_full0 + 8 * sa);
         if (++sa == q.sa) { sa = 0; pa ^= 1u; }
       }
     }
-  } else if (warp < 12) {
+  } else if (warp < STAGING_WARPS + 4) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(F::REGS_MISC));
-    if (warp == 8) {
+    if (warp == STAGING_WARPS) {
       // ---------------- MMA issuer -----------------------------------------------------------------------
       const bool leader = elect_one();
       const uint32_t a_lo0 = smem_desc_lo(a_ring), b_lo0 = smem_desc_lo(b_ring);
@@ -386,7 +398,7 @@ __global__ void __launch_bounds__(THREADS, 1) conv_runs_kernel(RunsParams q) {
         }
       }
       (void)id2; (void)id3; (void)sub_lo;
-    } else if (warp == 9) {
+    } else if (warp == STAGING_WARPS + 1) {
       // ---------------- filter copies ----------------------------------------------------------------------
       const bool leader = elect_one();
       bool ok = true;
@@ -408,25 +420,26 @@ __global__ void __launch_bounds__(THREADS, 1) conv_runs_kernel(RunsParams q) {
         if (q.resident) break;                               // the whole filter is in place
       }
       if (!ok) for (int i = 0; i < 64; ++i) __nanosleep(1000);   // copies in flight must land first
-    } else if (warp == 10) {
-      // ---------------- raw copies --------------------------------------------------------------------------
+    } else {
+      // ---------------- raw copies: two warps, every second slot each --------------------------------------------------------------------------
       bool ok = true;
       int sr = 0;
-      uint32_t pr = 0;
+      uint32_t pr = 0, sc = warp & 1;
       const int plane = (q.Ho * q.Wp + q.Wq * q.s - q.Wp) * q.Kh;
-      const int nslots = (q.K2 + q.rk - 1) / q.rk;           // (slots beyond the last real k2 are not read either)
+      const int per_slot = q.quad ? 4 : 8 * q.octs, nslots = q.quad ? 1 : (q.C + per_slot - 1) / per_slot;
       for (int w = blockIdx.x; w < q.nwork && ok; w += gridDim.x) {
         const TileRuns tr = tile_runs(q, (uint32_t)(w / q.ntn) * TILE_M);
         const int nseg = (int)(tr.n1 - tr.n0) + 1;
-        for (int sl = 0; sl < nslots; ++sl) {
+        for (int sl = 0; sl < nslots; ++sl, ++sc) {
+          if (sc & 1) {
+            if (++sr == q.sr) { sr = 0; pr ^= 1u; }
+            continue;
+          }
           ok = mbar_wait(raw_empty0 + 8 * sr, pr ^ 1u, &abort_flag, q.status);
           ok = __all_sync(0xffffffffu, ok);
           if (!ok) break;
           const uint32_t bar = raw_full0 + 8 * sr;
-          const int c0 = sl * q.rk / q.E;
-          int k1 = sl * q.rk + q.rk - 1;
-          if (k1 > q.K2 - 1) k1 = q.K2 - 1;
-          const int nc = k1 / q.E - c0 + 1;
+          const int c0 = sl * per_slot, nc = q.C - c0 < per_slot ? q.C - c0 : per_slot;
           int seg_off = 0;
           for (int g = 0; g < nseg; ++g) {
             const int start = g == 0 ? tr.start0 : 0, end = g == nseg - 1 ? tr.end1 : plane;
@@ -460,7 +473,7 @@ __global__ void __launch_bounds__(THREADS, 1) conv_runs_kernel(RunsParams q) {
   } else {
     // ---------------- epilogue ---------------------------------------------------------------------------------
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(F::REGS_EPILOGUE));
-    const int lq = warp & 3, h = (warp - 12) >> 2;           // tensor-memory quadrant; which channels
+    const int lq = warp & 3, h = (warp - STAGING_WARPS - 4) >> 2;           // tensor-memory quadrant; which channels
     bool ok = true;
     uint32_t ac = 0;
     for (int w = blockIdx.x; w < q.nwork && ok; w += gridDim.x) {
@@ -575,7 +588,7 @@ __global__ void __launch_bounds__(THREADS, 1) conv_runs_kernel(RunsParams q) {
     for (int i = 0; i < 64; ++i) __nanosleep(1000);
     __syncthreads();
   }
-  if (warp == 11) {
+  if (warp == STAGING_WARPS) {
     __syncwarp();
     tc_fence_after();
     tmem_dealloc(tmem_acc, 512);
@@ -589,15 +602,15 @@ __global__ void __launch_bounds__(THREADS, 1) conv_runs_kernel(RunsParams q) {
 template <bool F32>
 __global__ void __launch_bounds__(256) pack_runs_kernel(const void* __restrict__ f, unsigned char* __restrict__ fp,
                                                         uint32_t* __restrict__ status, int C, int Kh, int Kw, int s, int E, int G,
-                                                        int Co, int bn, int num_kb, int rows, int pitch) {
+                                                        int Co, int bn, int num_kb, int rows, int pitch, int quad) {
   using T = typename std::conditional<F32, float, uint16_t>::type;
   constexpr int PIECES = F32 ? 3 : 1;
   extern __shared__ __align__(16) unsigned char pack_raw[];
   T* stage = reinterpret_cast<T*>(pack_raw);
   if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < kStatusBytes / 4) status[threadIdx.x] = 0u;
   const int kb = blockIdx.x, row0 = blockIdx.y * rows;
-  const int c0 = kb * KB / E;
-  int c1 = (kb * KB + KB - 1) / E;
+  const int c0 = quad ? 0 : kb * 8 / E * 8;
+  int c1 = quad ? C - 1 : (kb * 8 + 7) / E * 8 + 7;
   if (c1 > C - 1) c1 = C - 1;
   const int T2 = Kh * Kw, run = (c1 - c0 + 1) * T2;
   for (int r = 0; r < rows; ++r) {
@@ -613,14 +626,13 @@ __global__ void __launch_bounds__(256) pack_runs_kernel(const void* __restrict__
     const int r = rg % rows, g = rg / rows;
     const int row = row0 + r, nt = row / bn, rr = row - nt * bn;
     uint32_t p[PIECES][4] = {};
-    int k2 = kb * KB + ch * 8;
-    int c = k2 / E, e = k2 - c * E, t = e / Kh, u = e - t * Kh;
+    const int j = kb * 8 + ch;                               // unit: eight channels at one e, or four channels at two
 #pragma unroll
     for (int x = 0; x < 8; ++x) {
-      const int v = g * s + t;
+      const int o = j / E, e = quad ? 2 * j + (x >> 2) : j - o * E, c = quad ? (x & 3) : o * 8 + x;
+      const int t = e / Kh, u = e - t * Kh, v = g * s + t;
       T a = 0;
-      if (row < Co && c < C && v < Kw) a = stage[r * pitch + (c - c0) * T2 + u * Kw + v];
-      if (++u == Kh) { u = 0; if ((++t) * Kh == E) { t = 0; ++c; } }
+      if (row < Co && c < C && e < E && v < Kw) a = stage[r * pitch + (c - c0) * T2 + u * Kw + v];
       if constexpr (F32) {
         // The pieces of a finite element are finite (the first is cut where rounding would overflow); an
         // infinity or NaN is its own first piece, the others are zero: the sum of the pieces is the element.
@@ -645,13 +657,13 @@ __global__ void __launch_bounds__(256) pack_runs_kernel(const void* __restrict__
   }
 }
 
-template <bool F32, int BNMAX, bool PHASED>
+template <bool F32, int BNMAX>
 cudaError_t launch_form(const RunsParams& q, int smem, cudaStream_t stream) {
   static bool attr_done[64] = {};
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
   if (!attr_done[dev]) {
-    cudaError_t e = cudaFuncSetAttribute(conv_runs_kernel<F32, BNMAX, PHASED>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRunsSmem);
+    cudaError_t e = cudaFuncSetAttribute(conv_runs_kernel<F32, BNMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRunsSmem);
     if (e != cudaSuccess) return e;
     attr_done[dev] = true;
   }
@@ -665,23 +677,33 @@ cudaError_t launch_form(const RunsParams& q, int smem, cudaStream_t stream) {
   cfg.stream = stream;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, conv_runs_kernel<F32, BNMAX, PHASED>, q);
+  return cudaLaunchKernelEx(&cfg, conv_runs_kernel<F32, BNMAX>, q);
 }
 
 }  // namespace
+
+// Channels of the octets that a k2-block (8 units) can touch: what a block of the pack kernel stages.
+static int64_t pack_channels(int64_t E, int C) {
+  const int64_t n = ((8 + E - 2) / E + 1) * 8;
+  return n < C ? n : C;
+}
 
 RunsPlan plan_runs(const Geometry& g, bool f32) {
   RunsPlan p{};
   p.eligible = false;
   const int es = f32 ? 4 : 2, pieces = f32 ? 3 : 1;
   const int nsub = g.s < g.Kw ? g.s : g.Kw;
-  const int64_t E = (int64_t)nsub * g.Kh, K2 = g.C * E;
-  if (K2 > 6144 || E > 256 || g.chan_stride >= ((int64_t)1 << 30)) return p;
+  const int64_t E = (int64_t)nsub * g.Kh;
+  if (E > 256 || (int64_t)g.C * E > (1 << 20) || g.chan_stride >= ((int64_t)1 << 30)) return p;
+  if (pack_channels(E, g.C) * g.T * es > 48 * 1024) return p;
   p.E = (int32_t)E;
   p.G = (g.Kw + g.s - 1) / g.s;
-  p.num_kb = (int32_t)((K2 + KB - 1) / KB);
-  p.nks_last = (int32_t)((K2 - (int64_t)(p.num_kb - 1) * KB + 15) / 16);
+  p.quad = g.C <= 4;
+  p.units = (int32_t)(p.quad ? (E + 1) / 2 : (g.C + 7) / 8 * E);
+  p.num_kb = (p.units + 7) / 8;
+  p.nks_last = (p.units - 8 * (p.num_kb - 1) + 1) / 2;
   p.halo = p.G - 1;
+  if (p.halo > 31) return p;                                // (one lane per row below the tile)
   p.Wq = (g.Wp + g.s - 1) / g.s;
   p.pitch = p.Wq;
   // Rows of a strip start at multiples of eight where that puts every warp's stores on 32-byte sectors.
@@ -707,34 +729,26 @@ RunsPlan plan_runs(const Geometry& g, bool f32) {
   if (ntm * p.ntn >= ((int64_t)1 << 30)) return p;
   p.nwork = (int32_t)(ntm * p.ntn);
   const int units = p.num_kb * p.G;
-  const int budget = kRunsSmem - 1024 - p.num_kb * KB * 4;
-  // Rings: raw slots of 64, 32 or 16 k2, the largest of which three fit beside two S stages and the filter
-  // (resident where one channel tile's fits, else at least three units).
+  const int budget = kRunsSmem - 1024;
+  // A raw slot holds whole octets, at least three units; rings of two S stages, four slots (else two)
+  // and the filter (resident where one channel tile's fits, else at least three units).
+  p.octs = (int32_t)(E >= 3 ? 1 : (E == 2 ? 2 : 4));
+  const int64_t raw = ((p.quad ? 4 : 8 * p.octs) * (int64_t)p.region + 127) / 128 * 128;
   for (int pass = 0; pass < 4 && !p.eligible; ++pass) {
     const bool resident = (pass & 1) == 0 && p.ntn == 1 && units <= MAX_B;
     if ((pass & 1) == 0 && !resident) continue;
-    const int least_raw = pass < 2 ? 3 : 2;
-    const int least_b = resident ? units : (f32 ? 2 : 3);
-    for (int rk = 64; rk >= 16; rk /= 2) {
-      int64_t nch = (rk + E - 2) / E + 1;
-      if (nch > g.C) nch = g.C;
-      const int64_t raw = (nch * p.region + 127) / 128 * 128;
-      if (raw >= 65536 || (p.halo * (rk / 8)) > 256) continue;
-      if (2 * p.a_stage + least_b * p.slot_bytes + least_raw * raw > budget) continue;
-      p.rk = rk;
-      p.raw_slot = (int32_t)raw;
-      p.resident = resident;
-      p.sa = 2; p.sr = least_raw; p.sb = least_b;
-      auto fits = [&](int a, int r, int b) { return (int64_t)a * p.a_stage + (int64_t)r * raw + (int64_t)b * p.slot_bytes <= budget; };
-      if (!resident) while (p.sb < 4 && fits(p.sa, p.sr, p.sb + 1)) ++p.sb;
-      if (!f32 && fits(3, p.sr, p.sb)) p.sa = 3;
-      while (p.sr < MAX_RAW && fits(p.sa, p.sr + 1, p.sb)) ++p.sr;
-      if (!resident) while (p.sb < MAX_B && fits(p.sa, p.sr, p.sb + 1)) ++p.sb;
-      p.eligible = true;
-      break;
-    }
+    const int least_raw = pass < 2 ? 4 : 2, least_b = resident ? units : (f32 ? 2 : 3);
+    if (2 * p.a_stage + least_b * p.slot_bytes + least_raw * raw > budget) continue;
+    p.raw_slot = (int32_t)raw;
+    p.resident = resident;
+    p.sa = 2; p.sr = least_raw; p.sb = least_b;
+    auto fits = [&](int a, int r, int b) { return (int64_t)a * p.a_stage + (int64_t)r * raw + (int64_t)b * p.slot_bytes <= budget; };
+    if (!resident) while (p.sb < 4 && fits(p.sa, p.sr, p.sb + 1)) ++p.sb;
+    if (!f32 && fits(3, p.sr, p.sb)) p.sa = 3;
+    while (p.sr < MAX_RAW && fits(p.sa, p.sr + 2, p.sb)) p.sr += 2;   // (even: the two copy warps alternate)
+    if (!resident) while (p.sb < MAX_B && fits(p.sa, p.sr, p.sb + 1)) ++p.sb;
+    p.eligible = true;
   }
-  p.phased = (g.chan_stride * es) % 16 != 0;
   p.filter_bytes = (size_t)p.ntn * p.bn * p.num_kb * KB * p.G * 2 * pieces;
   return p;
 }
@@ -744,22 +758,19 @@ cudaError_t launch_pack_runs(const void* filter, void* scratch, const Geometry& 
   if (!p.eligible) return cudaErrorInvalidValue;
   unsigned char* base = static_cast<unsigned char*>(scratch);
   const int es = f32 ? 4 : 2;
-  int64_t nch = (KB + p.E - 2) / p.E + 1;
-  if (nch > g.C) nch = g.C;
-  const int64_t pitch = nch * g.T;
+  const int64_t pitch = pack_channels(p.E, g.C) * g.T;
   int rows = 8;                                             // channels per block: staging within 40 KB
   while (rows > 1 && rows * pitch * es > 40 * 1024) rows /= 2;
   const size_t smem = (size_t)(rows * pitch * es);
-  if (smem > 48 * 1024) return cudaErrorInvalidValue;
   dim3 grid((unsigned)p.num_kb, (unsigned)(p.ntn * p.bn / rows));
   if (grid.y > 65535) return cudaErrorInvalidValue;
   uint32_t* status = reinterpret_cast<uint32_t*>(base);
   if (f32)
     pack_runs_kernel<true><<<grid, 256, smem, stream>>>(filter, base + kStatusBytes, status, g.C, g.Kh, g.Kw, g.s, p.E, p.G, g.Co,
-                                                        p.bn, p.num_kb, rows, (int)pitch);
+                                                        p.bn, p.num_kb, rows, (int)pitch, p.quad);
   else
     pack_runs_kernel<false><<<grid, 256, smem, stream>>>(filter, base + kStatusBytes, status, g.C, g.Kh, g.Kw, g.s, p.E, p.G, g.Co,
-                                                         p.bn, p.num_kb, rows, (int)pitch);
+                                                         p.bn, p.num_kb, rows, (int)pitch, p.quad);
   return cudaGetLastError();
 }
 
@@ -775,21 +786,20 @@ cudaError_t launch_conv_runs(const void* window, float* y, void* scratch, const 
   q.status = reinterpret_cast<uint32_t*>(base);
   q.img_bytes = g.img_stride * es; q.chan_bytes = g.chan_stride * es; q.win_bytes = g.window_elems * es;
   q.VQ = (uint32_t)p.VQ;
+  q.div_pitch = fast_div((uint32_t)p.pitch);
+  q.div_ho = fast_div((uint32_t)g.Ho);
   q.C = g.C; q.N = g.N; q.Wp = g.Wp; q.Wq = p.Wq; q.pitch = p.pitch; q.Ho = g.Ho; q.Wo = g.Wo; q.HoWo = g.Ho * g.Wo;
   q.Co = g.Co; q.Kh = g.Kh; q.Kw = g.Kw; q.s = g.s;
-  q.E = p.E; q.G = p.G; q.K2 = g.C * p.E; q.num_kb = p.num_kb; q.nks_last = p.nks_last;
-  q.col_bytes = (int32_t)(g.s * g.Kh * es);
-  q.rows = p.rows; q.halo = p.halo; q.region = p.region; q.rk = p.rk; q.raw_slot = p.raw_slot; q.a_stage = p.a_stage;
+  q.E = p.E; q.G = p.G; q.units = p.units; q.quad = p.quad ? 1 : 0; q.num_kb = p.num_kb; q.nks_last = p.nks_last;
+  q.rows = p.rows; q.halo = p.halo; q.region = p.region; q.octs = p.octs; q.raw_slot = p.raw_slot; q.a_stage = p.a_stage;
   q.bn = p.bn; q.ntn = p.ntn; q.nwork = p.nwork; q.sa = p.sa; q.sr = p.sr; q.sb = p.sb;
   q.slot_bytes = p.slot_bytes; q.resident = p.resident ? 1 : 0;
   q.chain = g.K >= 288 ? 12 : 8;
-  const int smem = 1024 + p.sa * p.a_stage + p.sb * p.slot_bytes + p.sr * p.raw_slot + p.num_kb * KB * 4;
-#define IM2WIN_RUNS(F32_, BN_) (p.phased ? launch_form<F32_, BN_, true>(q, smem, stream) : launch_form<F32_, BN_, false>(q, smem, stream))
-  if (f32) return IM2WIN_RUNS(true, 80);
-  if (p.bn <= 64) return IM2WIN_RUNS(false, 64);
-  if (p.bn <= 128) return IM2WIN_RUNS(false, 128);
-  return IM2WIN_RUNS(false, 256);
-#undef IM2WIN_RUNS
+  const int smem = 1024 + p.sa * p.a_stage + p.sb * p.slot_bytes + p.sr * p.raw_slot;
+  if (f32) return launch_form<true, 80>(q, smem, stream);
+  if (p.bn <= 64) return launch_form<false, 64>(q, smem, stream);
+  if (p.bn <= 128) return launch_form<false, 128>(q, smem, stream);
+  return launch_form<false, 256>(q, smem, stream);
 }
 
 }  // namespace im2win
