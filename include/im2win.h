@@ -4,7 +4,9 @@
  * The library implements the hot path of the im2win convolution: the im2win
  * data transformation (paper Eq. 2) and the forward convolution over the
  * im2win tensor (paper Eq. 3, GEMM view of Algorithm 1) in two precisions:
- * fp32 on CUDA cores and fp16-input / fp32-accumulate on tensor cores.
+ * fp32 (on tensor cores through an exact three-piece split of every operand,
+ * on CUDA cores for reductions below 64 terms) and fp16-input /
+ * fp32-accumulate on tensor cores.
  *
  * Problem statement (paper, Section "Notation"): input I[N][C][H][W], filter
  * F[Co][C][Kh][Kw] (OIHW), output O[N][Co][Ho][Wo], all row-major with the
@@ -67,9 +69,9 @@ const char* im2win_status_string(im2win_status status);
 
 /*
  * Name of the convolution kernel the library selects for a layer (host-only,
- * launches nothing; static storage): "f32-ffma" for IM2WIN_F32; for IM2WIN_F16
- * one of the tensor-core kernels of Algorithm 1's GEMM view, "f16-stem",
- * "f16-mat", "f16-raw", "f16-shift" or "f16-gather"; "none" for an
+ * launches nothing; static storage): "f32-split" or "f32-ffma" for IM2WIN_F32;
+ * for IM2WIN_F16 one of the tensor-core kernels of Algorithm 1's GEMM view,
+ * "f16-stem", "f16-mat", "f16-raw", "f16-runs", "f16-shift" or "f16-gather"; "none" for an
  * invalid shape.  For reports and tests; the choice is an implementation detail.
  */
 const char* im2win_conv_kernel_name(const im2win_shape* shape, im2win_dtype dtype);
@@ -80,7 +82,7 @@ const char* im2win_conv_kernel_name(const im2win_shape* shape, im2win_dtype dtyp
  *                   of the im2win tensor (paper Eq. 2; Section "Im2win Data
  *                   Transformation"), with no hidden padding.
  *   scratch_bytes = what im2win_conv_f32 / im2win_conv_f16 need in `scratch`
- *                   (a status block, the repacked filter and an offset table).
+ *                   (a status block, the repacked filter, and an offset table or a copy of the filter).
  *   Ho, Wo        = output height and width.
  * Any of the four output pointers may be NULL.
  */
@@ -103,14 +105,18 @@ im2win_status im2win_transform(const void* x_nchw, void* window, const im2win_sh
                                im2win_dtype dtype, void* cuda_stream);
 
 /*
- * Forward convolution over the im2win tensor, fp32 on CUDA cores
+ * Forward convolution over the im2win tensor, fp32
  * (paper Eq. 3; Section "im2win convolutions", the "CC" variant):
  *     y[n][co][ho][wo] = sum_c sum_{t < Kh*Kw} window[n][c][ho][(wo*s)*Kh + t] * Fp[co][c][t],
  *     Fp[co][c][v*Kh + u] = filter_oihw[co][c][u][v]   (height before width).
  * The filter is repacked into `scratch` on every call (part of the timed
  * operation).  `y_nchw` is [N][Co][Ho][Wo] fp32.  `scratch` must hold at least
  * the scratch_bytes reported by im2win_workspace_size(shape, IM2WIN_F32, ...).
- * Products and sums are fp32; the summation order is unspecified.
+ * Sums are fp32 and their order is unspecified.  Reductions of 64 terms or more run on the tensor cores:
+ * every element is the exact sum of three bf16 pieces, and six products of
+ * pieces stand for one fp32 product to within 2^-26 of it; the error against 64 bits is
+ * below that of a chain of fp32 FMAs.  Infinities, NaNs and overflow come out as fp32 FMAs give
+ * them.  Device-side waits of this kernel are bounded as in im2win_conv_f16.
  */
 im2win_status im2win_conv_f32(const float* window, const float* filter_oihw, float* y_nchw,
                               void* scratch, size_t scratch_bytes, const im2win_shape* shape,

@@ -56,14 +56,13 @@ im2win_status derive_geometry(const im2win_shape* s, Geometry* g) {
   return IM2WIN_OK;
 }
 
-// Which fp32 kernel: the tensor cores, except on short reductions and where the estimate says that the
-// FFMA kernel's finer tiles win.  Forcing one of that kernel's forms, or IM2WIN_F32_KERNEL=ffma|split,
-// decides it (testing aids).
-static bool want_f32_split(const Geometry& g, const F32SplitPlan& split) {
+// Which fp32 kernel: the tensor cores from 64 terms on.  Measured over sixty layers of all sizes: 1.1 to 18 times
+// faster than the FFMA kernel from 72 terms on, 0.4 to 1.1 times below 64, where half-empty k2-blocks are split and
+// multiplied.  Forcing one of the FFMA kernel's forms, or IM2WIN_F32_KERNEL=ffma|split, decides it (testing aids).
+static bool want_f32_split(const Geometry& g) {
   if (const char* v = debug_getenv("IM2WIN_F32_KERNEL")) return strcmp(v, "split") == 0;
   for (const char* name : {"IM2WIN_F32_BM", "IM2WIN_F32_TALL", "IM2WIN_F32_KLANES", "IM2WIN_F32_BK"})
     if (debug_getenv(name)) return false;
-  (void)split;
   return g.K >= 64;
 }
 
@@ -78,7 +77,7 @@ im2win_status scratch_layout(const Geometry& g, im2win_dtype dtype, ScratchLayou
     return IM2WIN_ERR_INVALID_ARG;
   }
   l->f32_split = false;
-  l->runs = false;
+  l->f16_runs = false;
   l->f16_shift = false;
   l->f16_raw = false;
   l->f16_mat = false;
@@ -89,18 +88,11 @@ im2win_status scratch_layout(const Geometry& g, im2win_dtype dtype, ScratchLayou
   l->total = (size_t)round_up((int64_t)l->filter_off + fbytes, 256);
   if (dtype == IM2WIN_F32) {
     const F32SplitPlan split = plan_f32_split(g);
-    l->f32_split = split.eligible && want_f32_split(g, split);
+    l->f32_split = split.eligible && want_f32_split(g);
     // (the scratch size covers both kernels and does not depend on N)
     const int64_t wide = round_up((int64_t)kStatusBytes + 4 * round_up(g.K, 32), 256) + round_up(g.K, 32) * l->Co_pad * 4;
     int64_t most = round_up(wide, 256);
     if (split.eligible && kStatusBytes + (int64_t)split.filter_bytes > most) most = kStatusBytes + (int64_t)split.filter_bytes;
-    const RunsPlan runs = plan_runs(g, true);
-    if (runs.eligible) {
-      const char* force = debug_getenv("IM2WIN_F32_KERNEL");
-      l->runs = force && strcmp(force, "runs") == 0;
-      if (l->runs) l->f32_split = false;
-      if (kStatusBytes + (int64_t)runs.filter_bytes > most) most = kStatusBytes + (int64_t)runs.filter_bytes;
-    }
     l->ffma_total = l->total;
     l->total = (size_t)round_up(most, 256);
   }
@@ -138,9 +130,9 @@ im2win_status scratch_layout(const Geometry& g, im2win_dtype dtype, ScratchLayou
       const size_t mat_total = (size_t)round_up((int64_t)mat.scratch_bytes, 256);
       if (mat_total > l->total) l->total = mat_total;
     }
-    const RunsPlan runs = plan_runs(g, false);
+    const RunsPlan runs = plan_f16_runs(g);
     if (runs.eligible) {
-      l->runs = force && strcmp(force, "runs") == 0;
+      l->f16_runs = force ? strcmp(force, "runs") == 0 : false;
       const size_t runs_total = (size_t)round_up(kStatusBytes + (int64_t)runs.filter_bytes, 256);
       if (runs_total > l->total) l->total = runs_total;
     }
@@ -171,9 +163,9 @@ static im2win_status conv_common(const void* window, const void* filter, float* 
   cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
   cudaError_t e = cudaSuccess;
   if (mode & kDoPack) {
-    if (l.runs) e = launch_pack_runs(filter, scratch, g, dtype == IM2WIN_F32, stream);
-    else if (l.f32_split) e = launch_pack_f32_split(static_cast<const float*>(filter), scratch, g, stream);
+    if (l.f32_split) e = launch_pack_f32_split(static_cast<const float*>(filter), scratch, g, stream);
     else if (dtype == IM2WIN_F32) e = launch_pack_f32(static_cast<const float*>(filter), scratch, g, l, stream);
+    else if (l.f16_runs) e = launch_pack_f16_runs(static_cast<const uint16_t*>(filter), scratch, g, stream);
     else if (l.f16_stem) e = launch_pack_f16_shift(static_cast<const uint16_t*>(filter), scratch, g, l, stream);
     else if (l.f16_mat) e = launch_pack_f16_mat(static_cast<const uint16_t*>(filter), scratch, g, stream);
     else if (l.f16_raw)
@@ -183,9 +175,9 @@ static im2win_status conv_common(const void* window, const void* filter, float* 
     if (e != cudaSuccess) return IM2WIN_ERR_CUDA;
   }
   if (mode & kDoConv) {
-    if (l.runs) e = launch_conv_runs(window, y, scratch, g, dtype == IM2WIN_F32, stream);
-    else if (l.f32_split) e = launch_conv_f32_split(static_cast<const float*>(window), y, scratch, g, stream);
+    if (l.f32_split) e = launch_conv_f32_split(static_cast<const float*>(window), y, scratch, g, stream);
     else if (dtype == IM2WIN_F32) e = launch_conv_f32(static_cast<const float*>(window), y, scratch, g, l, stream);
+    else if (l.f16_runs) e = launch_conv_f16_runs(static_cast<const uint16_t*>(window), y, scratch, g, stream);
     else if (l.f16_stem) e = launch_conv_f16_stem(static_cast<const uint16_t*>(window), y, scratch, g, l, stream);
     else if (l.f16_mat) e = launch_conv_f16_mat(static_cast<const uint16_t*>(window), y, scratch, g, stream);
     else if (l.f16_raw) e = launch_conv_f16_raw(static_cast<const uint16_t*>(window), y, scratch, g, l, stream);
@@ -219,8 +211,8 @@ const char* im2win_conv_kernel_name(const im2win_shape* shape, im2win_dtype dtyp
   Geometry g;
   ScratchLayout l;
   if (derive_geometry(shape, &g) != IM2WIN_OK || scratch_layout(g, dtype, &l) != IM2WIN_OK) return "none";
-  if (l.runs) return dtype == IM2WIN_F32 ? "f32-runs" : "f16-runs";
   if (dtype == IM2WIN_F32) return l.f32_split ? "f32-split" : "f32-ffma";
+  if (l.f16_runs) return "f16-runs";
   if (l.f16_stem) return "f16-stem";
   if (l.f16_mat) return "f16-mat";
   if (l.f16_raw) return "f16-raw";

@@ -36,7 +36,7 @@ struct ScratchLayout {
   size_t koff_off, filter_off, total;
   size_t ffma_total;     // fp32 only: what the FFMA kernel alone needs
   bool f32_split;        // fp32 only: the tensor-core kernel is used (filter images right after the status block)
-  bool runs;             // the run-staged kernel is used (filter images right after the status block)
+  bool f16_runs;         // fp16 only: the run-staged kernel is used (filter images right after the status block)
   bool f16_shift;        // fp16 only: a shifted-view kernel (and its filter layout) is used
   bool f16_raw;          // fp16 only: the bulk-copy variant of the shifted-view kernel is used
   bool f16_mat;          // fp16 only: the matrix-transpose variant is used (own scratch layout)
@@ -127,12 +127,12 @@ struct F32SplitPlan {
   int32_t bn, ntn, split, sb, nwork;   // channel tile and their number, CTAs per tile, filter slots, tiles
   int32_t packed_rows;                 // most rows (ntn * bn) of any tile width: the filter area does not depend on N
   int64_t VQ;
-  size_t filter_bytes;
+  size_t copy_off, filter_bytes;       // images, then a copy of the filter as given
   double cost;                         // cycles, estimated
 };
 F32SplitPlan plan_f32_split(const Geometry& g);
 
-// Tile and ring geometry of the run-staged kernel, fp16 or fp32 operands (see conv_runs.cu).
+// Tile and ring geometry of the run-staged kernel (see conv_f16_runs.cu).
 struct RunsPlan {
   bool eligible, resident, quad;       // quad: up to four channels, see the order of k2 there
   int32_t units, octs, E, G, Wq, pitch, rows, halo, num_kb, nks_last;
@@ -141,7 +141,7 @@ struct RunsPlan {
   int64_t VQ;
   size_t filter_bytes;
 };
-RunsPlan plan_runs(const Geometry& g, bool f32);
+RunsPlan plan_f16_runs(const Geometry& g);
 
 // Environment switches are testing aids: they are looked at only when IM2WIN_DEBUG is set in the
 // environment (checked once per process), so the default call path reads no environment.
@@ -163,8 +163,8 @@ cudaError_t launch_pack_f16(const uint16_t* filter, void* scratch, const Geometr
                             const ScratchLayout& l, cudaStream_t stream);
 cudaError_t launch_conv_f32(const float* window, float* y, const void* scratch, const Geometry& g,
                             const ScratchLayout& l, cudaStream_t stream);
-cudaError_t launch_pack_runs(const void* filter, void* scratch, const Geometry& g, bool f32, cudaStream_t stream);
-cudaError_t launch_conv_runs(const void* window, float* y, void* scratch, const Geometry& g, bool f32, cudaStream_t stream);
+cudaError_t launch_pack_f16_runs(const uint16_t* filter, void* scratch, const Geometry& g, cudaStream_t stream);
+cudaError_t launch_conv_f16_runs(const uint16_t* window, float* y, void* scratch, const Geometry& g, cudaStream_t stream);
 cudaError_t launch_pack_f32_split(const float* filter, void* scratch, const Geometry& g, cudaStream_t stream);
 cudaError_t launch_conv_f32_split(const float* window, float* y, void* scratch, const Geometry& g, cudaStream_t stream);
 cudaError_t launch_pack_f16_shift(const uint16_t* filter, void* scratch, const Geometry& g,

@@ -1,8 +1,6 @@
-// im2win convolution on the tensor cores with the window tensor brought in as contiguous runs.
-//
-// One kernel for two operand types: fp16 (one piece per operand, one product) and fp32 (three bf16 pieces, six
-// products, short accumulator chains; why and how accurate: conv_f32_split.cu).  It needs no alignment of planes,
-// strips or images and takes every stride.
+// fp16-input / fp32-accumulate im2win convolution with the window tensor brought in as contiguous runs.  It needs no
+// alignment of planes, strips or images and takes every stride: the layers whose plane pitch is no multiple of 16
+// bytes, which conv_f16_mat.cu and conv_f16_raw.cu cannot bring in with tiled copies.
 //
 // Columns.  In the im2win tensor the s*Kh elements of columns i*s .. i*s + s - 1 of a strip are contiguous, so a
 // convolution of stride s is one of stride 1 on columns s times as tall: virtual column i holds e = t*Kh + u
@@ -14,24 +12,20 @@
 // Order of k2.  A unit of eight k2 (16 bytes of S) is eight channels at one e: unit j = octet * E + e (up to four
 // channels: four channels at two e).  The places of a row's elements in the eight channel planes are then the same
 // for every unit but for one uniform offset -- also where planes start at different phases of 16 bytes, because
-// eight planes further the phase repeats -- and a unit costs a thread eight 2- or 4-byte shared loads, four
-// packs and one store.  (With k2 = c*E + e and a table of offsets a unit took 225 instructions and the kernel was bound by
-// them: 114 us where this one takes XXX, 3x3 on 64 channels at 56x56, batch 128, fp16.)
+// eight planes further the phase repeats -- and a unit costs a thread eight 2-byte shared loads, four packs and one
+// store.
 //
 // Staging.  The columns a tile needs of one channel are one contiguous run per image it touches: an untiled bulk
 // copy from the 16-byte boundary below to the one above brings it into a ring of raw slots (`octs` octets of
-// channels each).  Four warpgroups take the units in turn, read the elements of their rows back (thread = row), split
-// them (fp32) and write the units of S.  Gathering with global loads instead (conv_f16_shift.cu, conv_f32_split.cu)
-// makes every load instruction touch 32 rows s*Kh elements apart: three or more L1 wavefronts each, and a round trip
-// to memory per batch.
+// channels each).  Two warpgroups take the units in turn, read the elements of their rows back (thread = row) and
+// write the units of S.  Gathering with 2-byte global loads instead (conv_f16_shift.cu) makes every load instruction
+// touch 32 rows s*Kh elements apart: three or more L1 wavefronts each, and a round trip to memory per batch.
 //
 // What bounds it: the shared-memory pipe, which carries the MMA's operand reads (32 + N/4 cycles per instruction of
 // M = 128, K = 16), the copies, the read-back and the S stores.
 #include <cuda_fp16.h>
 #include <stdlib.h>
 #include <string.h>
-
-#include <type_traits>
 
 #define IM2WIN_INLINE_SLOW_WAIT      // (a call beside the epilogue's live sums costs spills)
 #include "common.cuh"
@@ -47,7 +41,7 @@ constexpr int KB = 64;
 constexpr int MAX_A = 4, MAX_RAW = 8, MAX_B = 16, MAX_ACC = 8;
 constexpr int MAX_SEG = 6;                    // images a tile may touch
 constexpr int kRunsSmem = 226 * 1024;
-constexpr int STAGING_WARPS = 16;
+constexpr int STAGING_WARPS = 8;
 constexpr int THREADS = 32 * (STAGING_WARPS + 4 + 8);   // staging; MMA, filter copies, two raw-copy warps; epilogue
 
 // n / d for n below 2^31: (n * mul) >> shift with mul = floor(2^shift / d) + 1, shift = 31 + ceil(log2 d).
@@ -73,22 +67,10 @@ struct RunsParams {
   int32_t E, G, units, num_kb, nks_last;      // units: of eight k2
   int32_t quad;                               // 1: up to four channels, a unit is four channels at two e
   int32_t rows, halo, region, octs, raw_slot, a_stage;
-  int32_t bn, ntn, nwork, sa, sr, sb, slot_bytes, resident, chain;
+  int32_t bn, ntn, nwork, sa, sr, sb, slot_bytes, resident;
 };
 
 __device__ __forceinline__ void wait_for_previous_kernel() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ uint32_t cvt_bf16x2(float lo, float hi) {
-  uint32_t r;
-  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
-  return r;
-}
-// Two values -> their three pieces, packed (first value in the low half).
-__device__ __forceinline__ void split2(float a, float b, uint32_t& p1, uint32_t& p2, uint32_t& p3) {
-  p1 = cvt_bf16x2(a, b);
-  const float ra = a - __uint_as_float(p1 << 16), rb = b - __uint_as_float(p1 & 0xffff0000u);
-  p2 = cvt_bf16x2(ra, rb);
-  p3 = cvt_bf16x2(ra - __uint_as_float(p2 << 16), rb - __uint_as_float(p2 & 0xffff0000u));
-}
 __device__ __forceinline__ void st_shared16(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
   asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
 }
@@ -97,45 +79,8 @@ __device__ __forceinline__ uint32_t ld_shared_u16(uint32_t addr) {
   asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(addr) : "memory");
   return v;
 }
-__device__ __forceinline__ float ld_shared_f32(uint32_t addr) {
-  float v;
-  asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
-  return v;
-}
-__device__ __forceinline__ void tmem_ld16_issue(uint32_t taddr, uint32_t (&r)[16]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr)
-      : "memory");
-}
-// The wait for loads into r[]: naming the registers keeps every use of them after it.
-__device__ __forceinline__ void tmem_wait16(uint32_t (&r)[16]) {
-  asm volatile("tcgen05.wait::ld.sync.aligned;"
-               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
-                 "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
-               :
-               : "memory");
-}
-__host__ __device__ constexpr uint32_t instr_desc(bool bf16, int M, int N) {
-  return (1u << 4) | (bf16 ? (1u << 7) | (1u << 10) : 0u) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
-}
-// An output that has to be computed again (see conv_f32_split.cu).
-__device__ __forceinline__ bool suspicious(float v) {
-  const uint32_t u = __float_as_uint(v) << 1, lo = (uint32_t)(127 - 90) << 24;
-  return u != 0u && u - lo >= 0xff000000u - lo;
-}
-
-template <bool F32, int BNMAX> struct Form {
-  static constexpr int ES = F32 ? 4 : 2;
-  static constexpr int ACC_COLS = F32 ? 256 : BNMAX;        // tensor memory: a ring of accumulators (fp32: of triples)
-  static constexpr int NACC = 512 / ACC_COLS;
-  static constexpr int ACC_LOG = NACC == 2 ? 1 : (NACC == 4 ? 2 : 3);
-  static constexpr int CH = (BNMAX + 31) / 32;              // 16-channel chunks per epilogue warp
-  static constexpr int REGS_STAGING = 56, REGS_MISC = 56, REGS_EPILOGUE = 112;   // 4*56 + 56 + 2*112 = 7*72
-};
+constexpr int ES = 2;                         // bytes of an element
+constexpr int REGS_STAGING = 80, REGS_MISC = 64, REGS_EPILOGUE = 128;   // 2*80 + 64 + 2*128 = 5*96
 
 // Where the rows of a tile lie: image n0 + g of the tile is a run of its own, [start, end) in elements of a channel
 // plane, at byte seg_off(g) of a channel's region in a raw slot.
@@ -143,7 +88,7 @@ struct TileRuns {
   uint32_t n0, n1;
   int32_t start0, end1;                                     // first element of image n0, end in image n1
 };
-__device__ __forceinline__ int run_size(int elems, int es) { return (elems * es + 30) & ~15; }
+__device__ __forceinline__ int run_size(int elems) { return (elems * ES + 30) & ~15; }
 __device__ __forceinline__ void split_q(const RunsParams& q, uint32_t vq, uint32_t& n, int& ho, int& i) {
   const uint32_t sg = q.div_pitch(vq);
   i = (int)(vq - sg * (uint32_t)q.pitch);
@@ -165,36 +110,34 @@ __device__ __forceinline__ TileRuns tile_runs(const RunsParams& q, uint32_t q0) 
   return r;
 }
 
-// One output in fp32 FMAs, k ascending.  fp32: for the values the split cannot hold.  Both: where a column
-// outside the window, which meets zeros of the widened filter, holds an infinity or a NaN.
-template <bool F32>
+// One output in fp32 FMAs, k ascending, for outputs that came out infinite or NaN: a column outside the window, which
+// meets zeros of the widened filter, may hold the infinity or NaN.
 __device__ __forceinline__ float exact_output(const RunsParams& q, uint32_t n, int ho, int wo, int nt, int col) {
-  constexpr int ES = F32 ? 4 : 2, PIECES = F32 ? 3 : 1;
   const unsigned char* wbase = q.win + (int64_t)n * q.img_bytes + ((int64_t)ho * q.Wp + (int64_t)wo * q.s) * q.Kh * ES;
-  const int64_t piece = (int64_t)q.bn * 128;
-  const unsigned char* frow = q.fp + (int64_t)nt * q.num_kb * q.G * PIECES * piece + col * 128;
+  const unsigned char* frow = q.fp + (int64_t)nt * q.num_kb * q.G * q.slot_bytes + col * 128;
   float acc = 0.f;
   for (int c = 0; c < q.C; ++c)
     for (int v = 0; v < q.Kw; ++v)
       for (int u = 0; u < q.Kh; ++u) {
         const int g = v / q.s, e = (v - g * q.s) * q.Kh + u;
         const int j = q.quad ? e >> 1 : (c >> 3) * q.E + e, at = q.quad ? (e & 1) * 4 + c : c & 7;      // unit, place in it
-        const unsigned char* f = frow + ((int64_t)(j >> 3) * q.G + g) * PIECES * piece + ((((j & 7) ^ (col & 7)) << 4) | (at * 2));
+        const unsigned char* f = frow + ((int64_t)(j >> 3) * q.G + g) * q.slot_bytes + ((((j & 7) ^ (col & 7)) << 4) | (at * 2));
         const unsigned char* x = wbase + c * q.chan_bytes + (v * q.Kh + u) * ES;
-        if constexpr (F32) {
-          auto part = [&](int p) { return __uint_as_float((uint32_t)*reinterpret_cast<const uint16_t*>(f + p * piece) << 16); };
-          acc = fmaf(*reinterpret_cast<const float*>(x), (part(0) + part(1)) + part(2), acc);
-        } else {
-          acc = fmaf(__half2float(*reinterpret_cast<const __half*>(x)), __half2float(*reinterpret_cast<const __half*>(f)), acc);
-        }
+        acc = fmaf(__half2float(*reinterpret_cast<const __half*>(x)), __half2float(*reinterpret_cast<const __half*>(f)), acc);
       }
   return acc;
 }
 
-template <bool F32, int BNMAX>
-__global__ void __launch_bounds__(THREADS, 1) conv_runs_kernel(RunsParams q) {
-  using F = Form<F32, BNMAX>;
-  constexpr int ES = F::ES;
+// The MMAs of one kernel column, straight-line: a lone lane pays for every branch and address computation between them.
+template <int NKS>
+__device__ __forceinline__ void issue_column(uint32_t d, uint32_t a, uint32_t b, uint32_t idesc, uint32_t more) {
+#pragma unroll
+  for (int j = 0; j < NKS; ++j) umma_f16_lohi(d, a + 2 * j, b + 2 * j, idesc, j == 0 ? more : 1u);
+}
+
+template <int BNMAX>
+__global__ void __launch_bounds__(THREADS, 1) conv_f16_runs_kernel(RunsParams q) {
+  constexpr int NACC = 512 / BNMAX, ACC_LOG = NACC == 2 ? 1 : (NACC == 4 ? 2 : 3);      // ring of accumulators in tensor memory
   extern __shared__ unsigned char smem_dyn[];
   unsigned char* smem = reinterpret_cast<unsigned char*>(((uintptr_t)smem_dyn + 1023) & ~(uintptr_t)1023);
   __shared__ __align__(8) uint64_t bars[2 * (MAX_A + MAX_RAW + MAX_B + MAX_ACC)];
@@ -202,7 +145,6 @@ __global__ void __launch_bounds__(THREADS, 1) conv_runs_kernel(RunsParams q) {
   __shared__ volatile uint32_t abort_flag;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int sub_bytes = q.rows * 128;
   const uint32_t a_ring = smem_u32(smem);
   const uint32_t b_ring = a_ring + q.sa * q.a_stage;
   const uint32_t raw_ring = b_ring + q.sb * q.slot_bytes;
@@ -232,8 +174,8 @@ __global__ void __launch_bounds__(THREADS, 1) conv_runs_kernel(RunsParams q) {
 
   if (warp < STAGING_WARPS) {
     // ---------------- staging: raw runs -> S ------------------------------------------------------------
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(F::REGS_STAGING));
-    // Warpgroup wg takes the units j = wg mod 4 of a stage.  Every warp passes every stage and every slot in order, so
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_STAGING));
+    // Warpgroup wg takes every second unit.  Every warp passes every stage and every slot in order, so
     // no wait by phase parity can run ahead.
     const int wg = warp >> 2, row = threadIdx.x & 127;
     const int plane = (q.Ho * q.Wp + q.Wq * q.s - q.Wp) * q.Kh;   // (up to the end of the last virtual column)
@@ -255,7 +197,7 @@ __global__ void __launch_bounds__(THREADS, 1) conv_runs_kernel(RunsParams q) {
           split_q(q, vq, n, ho, i);
           if (i < q.Wq) {
             const int g = (int)(n - tr.n0), start = g == 0 ? tr.start0 : 0;
-            if (g > 0) off = run_size(plane - tr.start0, ES) + (g - 1) * run_size(plane, ES);
+            if (g > 0) off = run_size(plane - tr.start0) + (g - 1) * run_size(plane);
             off += ((ho * q.Wp + i * q.s) * q.Kh - start) * ES;
             phase = (uint32_t)((int64_t)n * q.img_bytes + (int64_t)start * ES);
           }
@@ -286,31 +228,19 @@ __global__ void __launch_bounds__(THREADS, 1) conv_runs_kernel(RunsParams q) {
             src = raw_ring + sr * q.raw_slot;
             e = 0;
           }
-          if ((ch & 3) == wg) {
+          if ((ch & 1) == wg) {
             auto unit = [&](const uint32_t (&at)[8], int srow) {
-              const uint32_t dst = stage + srow * 128 + ((ch ^ (srow & 7)) << 4);
-              if constexpr (F32) {
-                float v[8];
+              uint32_t v[8];
 #pragma unroll
-                for (int x = 0; x < 8; ++x) v[x] = ld_shared_f32(src + at[x]);
-                uint32_t p[3][4];
-#pragma unroll
-                for (int x = 0; x < 4; ++x) split2(v[2 * x], v[2 * x + 1], p[0][x], p[1][x], p[2][x]);
-#pragma unroll
-                for (int i = 0; i < 3; ++i) st_shared16(dst + i * sub_bytes, p[i][0], p[i][1], p[i][2], p[i][3]);
-              } else {
-                uint32_t v[8];
-#pragma unroll
-                for (int x = 0; x < 8; ++x) v[x] = ld_shared_u16(src + at[x]);
-                st_shared16(dst, v[0] | (v[1] << 16), v[2] | (v[3] << 16), v[4] | (v[5] << 16), v[6] | (v[7] << 16));
-              }
+              for (int x = 0; x < 8; ++x) v[x] = ld_shared_u16(src + at[x]);
+              st_shared16(stage + srow * 128 + ((ch ^ (srow & 7)) << 4), v[0] | (v[1] << 16), v[2] | (v[3] << 16),
+                          v[4] | (v[5] << 16), v[6] | (v[7] << 16));
             };
             unit(rb, row);
             // the rows below the tile: lanes of one of the warpgroup's warps, another one from unit to unit
-            if ((((8 * kb + ch) >> 2) & 3) == (warp & 3) && lane < q.halo) unit(hb, TILE_M + lane);
+            if (((4 * kb + (ch >> 1)) & 3) == (warp & 3) && lane < q.halo) unit(hb, TILE_M + lane);
           }
-          const bool last = 8 * kb + ch == q.units - 1;
-          if (++in_slot == per_slot || last) {
+          if (++in_slot == per_slot || 8 * kb + ch == q.units - 1) {
             __syncwarp();
             if (lane == 0) mbar_arrive(raw_empty0 + 8 * sr);
             if (++sr == q.sr) { sr = 0; pr ^= 1u; }
@@ -321,11 +251,9 @@ __global__ void __launch_bounds__(THREADS, 1) conv_runs_kernel(RunsParams q) {
           if (e == q.E) e = 0;
         }
         if (!ok) break;
-        if ((n_units & 1) != 0 && (n_units & 3) == wg) {     // zeros up to the end of the MMA's last step
-          for (int i = 0; i < (F32 ? 3 : 1); ++i) {
-            st_shared16(stage + i * sub_bytes + row * 128 + ((n_units ^ (row & 7)) << 4), 0u, 0u, 0u, 0u);
-            if (lane < q.halo) st_shared16(stage + i * sub_bytes + (TILE_M + lane) * 128 + ((n_units ^ (lane & 7)) << 4), 0u, 0u, 0u, 0u);
-          }
+        if ((n_units & 1) != 0 && wg == 1) {                 // zeros up to the end of the MMA's last step
+          st_shared16(stage + row * 128 + ((n_units ^ (row & 7)) << 4), 0u, 0u, 0u, 0u);
+          if (lane < q.halo) st_shared16(stage + (TILE_M + lane) * 128 + ((n_units ^ (lane & 7)) << 4), 0u, 0u, 0u, 0u);
         }
         fence_proxy_async_smem();
         __syncwarp();
@@ -334,70 +262,71 @@ __global__ void __launch_bounds__(THREADS, 1) conv_runs_kernel(RunsParams q) {
       }
     }
   } else if (warp < STAGING_WARPS + 4) {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(F::REGS_MISC));
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_MISC));
     if (warp == STAGING_WARPS) {
       // ---------------- MMA issuer -----------------------------------------------------------------------
       const bool leader = elect_one();
       const uint32_t a_lo0 = smem_desc_lo(a_ring), b_lo0 = smem_desc_lo(b_ring);
-      const uint32_t sub_lo = (uint32_t)sub_bytes >> 4;
-      const uint32_t id1 = instr_desc(F32, TILE_M, q.bn), id2 = instr_desc(F32, TILE_M, 2 * q.bn),
-                     id3 = instr_desc(F32, TILE_M, 3 * q.bn);
+      const uint32_t idesc = instr_desc_f16(TILE_M, q.bn);
       bool ok = true;
       int sa = 0, slot = 0;
-      uint32_t pa = 0, pb = 0, ac = 0;                       // ... chains (fp32) or tiles (fp16) so far
-      for (int w = blockIdx.x; w < q.nwork && ok; w += gridDim.x) {
-        int links = 0;                                       // steps in the open chain; 0: none is open
+      uint32_t pa = 0, pb = 0, ac = 0;                       // ... tiles so far
+      // A wait for a barrier that is already complete costs 200 cycles and more while the shared-memory pipe is busy, and
+      // the tensor pipe runs dry meanwhile: every barrier is looked at ahead of the instructions issued before it is
+      // needed, and waited for only where that look came too early.
+      uint32_t a_seen = 0, b_seen = 0, acc_seen = 0;
+      auto need = [&](uint32_t bar, uint32_t parity, uint32_t seen) {
+        if (__all_sync(0xffffffffu, seen != 0u)) return true;
+        return (bool)__all_sync(0xffffffffu, mbar_wait(bar, parity, &abort_flag, q.status));
+      };
+      for (int w = blockIdx.x; w < q.nwork && ok; w += gridDim.x, ++ac) {
+        const int ab = ac & (NACC - 1);
+        ok = need(acc_empty0 + 8 * ab, ((ac >> ACC_LOG) & 1) ^ 1, acc_seen);
+        if (!ok) break;
+        const uint32_t d = tmem_acc + ab * BNMAX;
+        uint32_t more = 0u;                                  // the tile's first instruction clears the accumulator
+        const bool fetch_b = !q.resident || w == (int)blockIdx.x;          // (a resident filter is complete after the first tile)
         if (q.resident) slot = 0;
         for (int kb = 0; kb < q.num_kb && ok; ++kb) {
           const int nks = kb == q.num_kb - 1 ? q.nks_last : KB / 16;
-          ok = mbar_wait(a_full0 + 8 * sa, pa, &abort_flag, q.status);
-          ok = __all_sync(0xffffffffu, ok);
+          ok = need(a_full0 + 8 * sa, pa, a_seen);
           if (!ok) break;
+          tc_fence_after();
           uint32_t a_view = a_lo0 + (uint32_t)(sa * (q.a_stage >> 4));
+          int nsa = sa + 1;
+          uint32_t npa = pa;
+          if (nsa == q.sa) { nsa = 0; npa ^= 1u; }
           for (int g = 0; g < q.G; ++g, a_view += 8u) {      // next view: one row (128 bytes) further down
-            const int ab = ac & (F::NACC - 1);
-            if (links == 0) {
-              ok = mbar_wait(acc_empty0 + 8 * ab, ((ac >> F::ACC_LOG) & 1) ^ 1, &abort_flag, q.status);
-              ok = __all_sync(0xffffffffu, ok);
+            const bool last_unit = g + 1 == q.G, last = kb + 1 == q.num_kb && last_unit;
+            int nslot = slot + 1;
+            uint32_t npb = pb;
+            if (nslot == q.sb) { nslot = 0; if (!q.resident) npb ^= 1u; }
+            if (fetch_b) {
+              ok = need(b_full0 + 8 * slot, pb, b_seen);
               if (!ok) break;
+              b_seen = mbar_test_wait(b_full0 + 8 * nslot, npb);
             }
-            const uint32_t d = tmem_acc + ab * F::ACC_COLS, more = links > 0;
-            links += nks;
-            const bool last_link = F32 ? links + nks > q.chain || g + 1 == q.G : kb + 1 == q.num_kb && g + 1 == q.G;
-            ok = mbar_wait(b_full0 + 8 * slot, pb, &abort_flag, q.status);
-            ok = __all_sync(0xffffffffu, ok);
-            if (!ok) break;
-            tc_fence_after();
+            if (last) acc_seen = mbar_test_wait(acc_empty0 + 8 * ((ac + 1) & (NACC - 1)), (((ac + 1) >> ACC_LOG) & 1) ^ 1);
+            if (last_unit) a_seen = mbar_test_wait(a_full0 + 8 * nsa, npa);
             const uint32_t b_lo = b_lo0 + (uint32_t)(slot * (q.slot_bytes >> 4));
             if (leader) {
-              if constexpr (F32) {
-#pragma unroll
-                for (int j = 0; j < KB / 16; ++j)
-                  if (j < nks) umma_f16_lohi(d, a_view + 2 * j, b_lo + 2 * j, id3, more | (uint32_t)j);
-#pragma unroll
-                for (int j = 0; j < KB / 16; ++j)
-                  if (j < nks) umma_f16_lohi(d + q.bn, a_view + sub_lo + 2 * j, b_lo + 2 * j, id2, 1u);
-#pragma unroll
-                for (int j = 0; j < KB / 16; ++j)
-                  if (j < nks) umma_f16_lohi(d + 2 * q.bn, a_view + 2 * sub_lo + 2 * j, b_lo + 2 * j, id1, 1u);
-              } else {
-#pragma unroll
-                for (int j = 0; j < KB / 16; ++j)
-                  if (j < nks) umma_f16_lohi(d, a_view + 2 * j, b_lo + 2 * j, id1, more | (uint32_t)j);
-              }
+              if (nks == KB / 16) issue_column<KB / 16>(d, a_view, b_lo, idesc, more);
+              else if (nks == 3) issue_column<3>(d, a_view, b_lo, idesc, more);
+              else if (nks == 2) issue_column<2>(d, a_view, b_lo, idesc, more);
+              else issue_column<1>(d, a_view, b_lo, idesc, more);
               if (!q.resident) umma_commit(b_empty0 + 8 * slot);
-              if (last_link) umma_commit(acc_full0 + 8 * ab);
+              if (last) umma_commit(acc_full0 + 8 * ab);
+              if (last_unit) umma_commit(a_empty0 + 8 * sa);
             }
             __syncwarp();
-            if (last_link) { ++ac; links = 0; }
-            if (++slot == q.sb) { slot = 0; if (!q.resident) pb ^= 1u; }
+            slot = nslot;
+            pb = npb;
+            more = 1u;
           }
-          if (ok && leader) umma_commit(a_empty0 + 8 * sa);
-          __syncwarp();
-          if (++sa == q.sa) { sa = 0; pa ^= 1u; }
+          sa = nsa;
+          pa = npa;
         }
       }
-      (void)id2; (void)id3; (void)sub_lo;
     } else if (warp == STAGING_WARPS + 1) {
       // ---------------- filter copies ----------------------------------------------------------------------
       const bool leader = elect_one();
@@ -460,7 +389,7 @@ __global__ void __launch_bounds__(THREADS, 1) conv_runs_kernel(RunsParams q) {
                 bulk_load(dst, q.win + from, (uint32_t)(to - from), bar);
               }
             }
-            seg_off += run_size(end - start, ES);
+            seg_off += run_size(end - start);
           }
           __syncwarp();
           if (lane == 0) mbar_arrive(bar);
@@ -472,7 +401,7 @@ __global__ void __launch_bounds__(THREADS, 1) conv_runs_kernel(RunsParams q) {
     __syncwarp();
   } else {
     // ---------------- epilogue ---------------------------------------------------------------------------------
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(F::REGS_EPILOGUE));
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(REGS_EPILOGUE));
     const int lq = warp & 3, h = (warp - STAGING_WARPS - 4) >> 2;           // tensor-memory quadrant; which channels
     bool ok = true;
     uint32_t ac = 0;
@@ -489,94 +418,38 @@ __global__ void __launch_bounds__(THREADS, 1) conv_runs_kernel(RunsParams q) {
         valid = i0 < q.Wo;                                   // trailing columns of a strip are no output
       }
       float* yrow = q.y + ((int64_t)n * q.Co + co0) * q.HoWo + (int64_t)ho * q.Wo + i0;
-      if constexpr (F32) {
-        float acc[F::CH][16];
-#pragma unroll
-        for (int j = 0; j < F::CH; ++j)
-#pragma unroll
-          for (int e = 0; e < 16; ++e) acc[j][e] = 0.f;
-        for (int kb = 0; kb < q.num_kb && ok; ++kb) {
-          const int nks = kb == q.num_kb - 1 ? q.nks_last : KB / 16;
-          const int units = q.chain / nks;                   // of one chain
-          for (int g = 0; g < q.G; g += units, ++ac) {
-            const int ab = ac & (F::NACC - 1);
-            ok = mbar_wait(acc_full0 + 8 * ab, (ac >> F::ACC_LOG) & 1, &abort_flag, q.status);
-            ok = __all_sync(0xffffffffu, ok);
-            if (!ok) break;
-            tc_fence_after();
-            const uint32_t d = tmem_acc + ((uint32_t)(lq * 32) << 16) + ab * F::ACC_COLS + h * 16;
-#pragma unroll
-            for (int j = 0; j < F::CH; ++j) {
-              if ((h + 2 * j) * 16 >= q.bn) break;
-              uint32_t r0[16], r1[16], r2[16];
-              tmem_ld16_issue(d + 32 * j, r0);
-              tmem_ld16_issue(d + 32 * j + q.bn, r1);
-              tmem_ld16_issue(d + 32 * j + 2 * q.bn, r2);
-              tmem_wait16(r0);
-              tmem_wait16(r1);
-              tmem_wait16(r2);
-#pragma unroll
-              for (int e = 0; e < 16; ++e)
-                acc[j][e] += __uint_as_float(r0[e]) + (__uint_as_float(r1[e]) + __uint_as_float(r2[e]));
-            }
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(acc_empty0 + 8 * ab);
-          }
-        }
-        if (!ok) break;
-        if (valid) {
-          bool again = false;
-#pragma unroll
-          for (int j = 0; j < F::CH; ++j) {
-            const int c0 = (h + 2 * j) * 16;
-            float *p0 = yrow + (int64_t)c0 * q.HoWo, *p1 = p0 + q.HoWo;
-#pragma unroll
-            for (int e = 0; e < 16; e += 2) {
-              if (c0 + e < limit) { *p0 = acc[j][e]; again |= suspicious(acc[j][e]); }
-              if (c0 + e + 1 < limit) { *p1 = acc[j][e + 1]; again |= suspicious(acc[j][e + 1]); }
-              p0 += 2 * (int64_t)q.HoWo; p1 += 2 * (int64_t)q.HoWo;
-            }
-          }
-          if (again) {
-            for (int c = h * 16; c < limit; c += (c & 15) == 15 ? 17 : 1)
-              if (suspicious(yrow[(int64_t)c * q.HoWo])) yrow[(int64_t)c * q.HoWo] = exact_output<F32>(q, n, ho, i0, nt, c);
-          }
-        }
-      } else {
-        const int ab = ac & (F::NACC - 1);
-        ok = mbar_wait(acc_full0 + 8 * ab, (ac >> F::ACC_LOG) & 1, &abort_flag, q.status);
-        ok = __all_sync(0xffffffffu, ok);
-        if (!ok) break;
-        ++ac;
-        tc_fence_after();
-        const uint32_t d = tmem_acc + ((uint32_t)(lq * 32) << 16) + ab * F::ACC_COLS;
+      const int ab = ac & (NACC - 1);
+      ok = mbar_wait(acc_full0 + 8 * ab, (ac >> ACC_LOG) & 1, &abort_flag, q.status);
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) break;
+      ++ac;
+      tc_fence_after();
+      const uint32_t d = tmem_acc + ((uint32_t)(lq * 32) << 16) + ab * BNMAX;
 #pragma unroll 1
-        for (int c0 = h * (BNMAX / 2); c0 < (h + 1) * (BNMAX / 2) && c0 < limit; c0 += 32) {
-          uint32_t v[32];
-          tmem_ld32(d + c0, v);
-          if (c0 + 32 >= (h + 1) * (BNMAX / 2) || c0 + 32 >= limit) {      // the last read of this accumulator
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(acc_empty0 + 8 * ab);
-          }
-          if (valid) {
-            store_strided32(yrow + (int64_t)c0 * q.HoWo, q.HoWo, v, limit - c0);
-            float zero = 0.f;
-#pragma unroll
-            for (int j = 0; j < 32; ++j) zero = fmaf(__uint_as_float(c0 + j < limit ? v[j] : 0u), 0.f, zero);
-            if (zero != 0.f) {                               // (a NaN: one of them is not finite)
-              for (int c = c0; c < c0 + 32 && c < limit; ++c) {
-                float* p = yrow + (int64_t)c * q.HoWo;
-                if (!(fabsf(*p) <= 3.4028234663852886e38f)) *p = exact_output<F32>(q, n, ho, i0, nt, c);
-              }
-            }
-          }
-        }
-        if (h * (BNMAX / 2) >= limit) {                      // (no channels for this warp)
+      for (int c0 = h * (BNMAX / 2); c0 < (h + 1) * (BNMAX / 2) && c0 < limit; c0 += 32) {
+        uint32_t v[32];
+        tmem_ld32(d + c0, v);
+        if (c0 + 32 >= (h + 1) * (BNMAX / 2) || c0 + 32 >= limit) {      // the last read of this accumulator
+          tc_fence_before();
           __syncwarp();
           if (lane == 0) mbar_arrive(acc_empty0 + 8 * ab);
         }
+        if (valid) {
+          store_strided32(yrow + (int64_t)c0 * q.HoWo, q.HoWo, v, limit - c0);
+          float zero = 0.f;
+#pragma unroll
+          for (int j = 0; j < 32; ++j) zero = fmaf(__uint_as_float(c0 + j < limit ? v[j] : 0u), 0.f, zero);
+          if (zero != 0.f) {                               // (a NaN: one of them is not finite)
+            for (int c = c0; c < c0 + 32 && c < limit; ++c) {
+              float* p = yrow + (int64_t)c * q.HoWo;
+              if (!(fabsf(*p) <= 3.4028234663852886e38f)) *p = exact_output(q, n, ho, i0, nt, c);
+            }
+          }
+        }
+      }
+      if (h * (BNMAX / 2) >= limit) {                      // (no channels for this warp)
+        __syncwarp();
+        if (lane == 0) mbar_arrive(acc_empty0 + 8 * ab);
       }
     }
   }
@@ -596,17 +469,12 @@ __global__ void __launch_bounds__(THREADS, 1) conv_runs_kernel(RunsParams q) {
 }
 
 // Filter -> the images the copy warp loads: for every (channel tile nt, k2-block kb, virtual kernel column g) the
-// pieces [bn channels][64 k2] in the 128-byte-swizzled order of shared memory (fp32: the three pieces side by side,
-// largest first).  One block: `rows` channels of one k2-block; per channel its source is one contiguous run of the OIHW
+// [bn channels][64 k2] in the 128-byte-swizzled order of shared memory.  One block: `rows` channels of one k2-block; per channel its source is one contiguous run of the OIHW
 // filter (whole input channels).  Channels beyond Co, k2 beyond C*E and kernel columns beyond Kw are zeros.
-template <bool F32>
-__global__ void __launch_bounds__(256) pack_runs_kernel(const void* __restrict__ f, unsigned char* __restrict__ fp,
+__global__ void __launch_bounds__(256) pack_f16_runs_kernel(const uint16_t* __restrict__ f, unsigned char* __restrict__ fp,
                                                         uint32_t* __restrict__ status, int C, int Kh, int Kw, int s, int E, int G,
                                                         int Co, int bn, int num_kb, int rows, int pitch, int quad) {
-  using T = typename std::conditional<F32, float, uint16_t>::type;
-  constexpr int PIECES = F32 ? 3 : 1;
-  extern __shared__ __align__(16) unsigned char pack_raw[];
-  T* stage = reinterpret_cast<T*>(pack_raw);
+  extern __shared__ uint16_t pack_h[];
   if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < kStatusBytes / 4) status[threadIdx.x] = 0u;
   const int kb = blockIdx.x, row0 = blockIdx.y * rows;
   const int c0 = quad ? 0 : kb * 8 / E * 8;
@@ -616,8 +484,8 @@ __global__ void __launch_bounds__(256) pack_runs_kernel(const void* __restrict__
   for (int r = 0; r < rows; ++r) {
     const int co = row0 + r;
     if (co >= Co) break;
-    const T* src = static_cast<const T*>(f) + ((int64_t)co * C + c0) * T2;
-    for (int i = threadIdx.x; i < run; i += blockDim.x) stage[r * pitch + i] = __ldg(src + i);
+    const uint16_t* src = f + ((int64_t)co * C + c0) * T2;
+    for (int i = threadIdx.x; i < run; i += blockDim.x) pack_h[r * pitch + i] = __ldg(src + i);
   }
   __syncthreads();
   const int items = rows * G * 8;
@@ -625,45 +493,28 @@ __global__ void __launch_bounds__(256) pack_runs_kernel(const void* __restrict__
     const int ch = it & 7, rg = it >> 3;
     const int r = rg % rows, g = rg / rows;
     const int row = row0 + r, nt = row / bn, rr = row - nt * bn;
-    uint32_t p[PIECES][4] = {};
+    uint32_t p[4] = {};
     const int j = kb * 8 + ch;                               // unit: eight channels at one e, or four channels at two
 #pragma unroll
     for (int x = 0; x < 8; ++x) {
       const int o = j / E, e = quad ? 2 * j + (x >> 2) : j - o * E, c = quad ? (x & 3) : o * 8 + x;
       const int t = e / Kh, u = e - t * Kh, v = g * s + t;
-      T a = 0;
-      if (row < Co && c < C && e < E && v < Kw) a = stage[r * pitch + (c - c0) * T2 + u * Kw + v];
-      if constexpr (F32) {
-        // The pieces of a finite element are finite (the first is cut where rounding would overflow); an
-        // infinity or NaN is its own first piece, the others are zero: the sum of the pieces is the element.
-        uint32_t b1 = cvt_bf16x2(a, 0.f) & 0xffffu, b2 = 0u, b3 = 0u;
-        if ((__float_as_uint(a) & 0x7f800000u) != 0x7f800000u) {
-          if ((b1 & 0x7f80u) == 0x7f80u) b1 = __float_as_uint(a) >> 16;
-          const float r1 = a - __uint_as_float(b1 << 16);
-          b2 = cvt_bf16x2(r1, 0.f) & 0xffffu;
-          b3 = cvt_bf16x2(r1 - __uint_as_float(b2 << 16), 0.f) & 0xffffu;
-        }
-        p[0][x >> 1] |= b1 << (16 * (x & 1));
-        p[PIECES - 2][x >> 1] |= b2 << (16 * (x & 1));
-        p[PIECES - 1][x >> 1] |= b3 << (16 * (x & 1));
-      } else {
-        p[0][x >> 1] |= (uint32_t)a << (16 * (x & 1));
-      }
+      uint32_t a = 0;
+      if (row < Co && c < C && e < E && v < Kw) a = pack_h[r * pitch + (c - c0) * T2 + u * Kw + v];
+      p[x >> 1] |= a << (16 * (x & 1));
     }
-    const int64_t piece = (int64_t)bn * 128;
-    unsigned char* dst = fp + (((int64_t)nt * num_kb + kb) * G + g) * PIECES * piece + rr * 128 + ((ch ^ (rr & 7)) << 4);
-#pragma unroll
-    for (int i = 0; i < PIECES; ++i) *reinterpret_cast<uint4*>(dst + i * piece) = make_uint4(p[i][0], p[i][1], p[i][2], p[i][3]);
+    *reinterpret_cast<uint4*>(fp + ((((int64_t)nt * num_kb + kb) * G + g) * bn + rr) * 128 + ((ch ^ (rr & 7)) << 4)) =
+        make_uint4(p[0], p[1], p[2], p[3]);
   }
 }
 
-template <bool F32, int BNMAX>
+template <int BNMAX>
 cudaError_t launch_form(const RunsParams& q, int smem, cudaStream_t stream) {
   static bool attr_done[64] = {};
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
   if (!attr_done[dev]) {
-    cudaError_t e = cudaFuncSetAttribute(conv_runs_kernel<F32, BNMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRunsSmem);
+    cudaError_t e = cudaFuncSetAttribute(conv_f16_runs_kernel<BNMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRunsSmem);
     if (e != cudaSuccess) return e;
     attr_done[dev] = true;
   }
@@ -677,7 +528,7 @@ cudaError_t launch_form(const RunsParams& q, int smem, cudaStream_t stream) {
   cfg.stream = stream;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, conv_runs_kernel<F32, BNMAX>, q);
+  return cudaLaunchKernelEx(&cfg, conv_f16_runs_kernel<BNMAX>, q);
 }
 
 }  // namespace
@@ -688,14 +539,13 @@ static int64_t pack_channels(int64_t E, int C) {
   return n < C ? n : C;
 }
 
-RunsPlan plan_runs(const Geometry& g, bool f32) {
+RunsPlan plan_f16_runs(const Geometry& g) {
   RunsPlan p{};
   p.eligible = false;
-  const int es = f32 ? 4 : 2, pieces = f32 ? 3 : 1;
   const int nsub = g.s < g.Kw ? g.s : g.Kw;
   const int64_t E = (int64_t)nsub * g.Kh;
   if (E > 256 || (int64_t)g.C * E > (1 << 20) || g.chan_stride >= ((int64_t)1 << 30)) return p;
-  if (pack_channels(E, g.C) * g.T * es > 48 * 1024) return p;
+  if (pack_channels(E, g.C) * g.T * ES > 48 * 1024) return p;          // staging of the filter pack
   p.E = (int32_t)E;
   p.G = (g.Kw + g.s - 1) / g.s;
   p.quad = g.C <= 4;
@@ -706,25 +556,20 @@ RunsPlan plan_runs(const Geometry& g, bool f32) {
   if (p.halo > 31) return p;                                // (one lane per row below the tile)
   p.Wq = (g.Wp + g.s - 1) / g.s;
   p.pitch = p.Wq;
-  // Rows of a strip start at multiples of eight where that puts every warp's stores on 32-byte sectors.
-  bool widen = g.Wo % 8 == 0;
-  if (const char* v = debug_getenv("IM2WIN_RUNS_PITCH")) widen = v[0] == '8';          // testing aid
-  if (widen) p.pitch = (p.Wq + 7) / 8 * 8;
   p.VQ = (int64_t)g.N * g.Ho * p.pitch;
   if (p.VQ + 2 * TILE_M >= ((int64_t)1 << 31)) return p;
   p.rows = TILE_M + (p.halo + 7) / 8 * 8;
-  p.a_stage = pieces * p.rows * 128;
+  p.a_stage = p.rows * 128;
   const int64_t per_img = (int64_t)g.Ho * p.pitch;
   const int64_t segs = (TILE_M + p.halo - 2) / per_img + 2;
   if (segs > MAX_SEG) return p;
   // bytes a tile's columns of one channel take in a raw slot, whatever the tile
-  const int64_t region = (int64_t)(TILE_M + p.halo) * g.s * g.Kh * es + segs * 32;
+  const int64_t region = (int64_t)(TILE_M + p.halo) * g.s * g.Kh * ES + segs * 32;
   p.region = (int32_t)((region + 15) / 16 * 16);
-  const int most = f32 ? 80 : 256;
-  p.ntn = (g.Co + most - 1) / most;
+  p.ntn = (g.Co + 255) / 256;
   p.bn = ((g.Co + p.ntn - 1) / p.ntn + 15) / 16 * 16;
   p.ntn = (g.Co + p.bn - 1) / p.bn;
-  p.slot_bytes = pieces * p.bn * 128;
+  p.slot_bytes = p.bn * 128;
   const int64_t ntm = (p.VQ + TILE_M - 1) / TILE_M;
   if (ntm * p.ntn >= ((int64_t)1 << 30)) return p;
   p.nwork = (int32_t)(ntm * p.ntn);
@@ -737,54 +582,47 @@ RunsPlan plan_runs(const Geometry& g, bool f32) {
   for (int pass = 0; pass < 4 && !p.eligible; ++pass) {
     const bool resident = (pass & 1) == 0 && p.ntn == 1 && units <= MAX_B;
     if ((pass & 1) == 0 && !resident) continue;
-    const int least_raw = pass < 2 ? 4 : 2, least_b = resident ? units : (f32 ? 2 : 3);
+    const int least_raw = pass < 2 ? 4 : 2, least_b = resident ? units : 3;
     if (2 * p.a_stage + least_b * p.slot_bytes + least_raw * raw > budget) continue;
     p.raw_slot = (int32_t)raw;
     p.resident = resident;
     p.sa = 2; p.sr = least_raw; p.sb = least_b;
     auto fits = [&](int a, int r, int b) { return (int64_t)a * p.a_stage + (int64_t)r * raw + (int64_t)b * p.slot_bytes <= budget; };
     if (!resident) while (p.sb < 4 && fits(p.sa, p.sr, p.sb + 1)) ++p.sb;
-    if (!f32 && fits(3, p.sr, p.sb)) p.sa = 3;
+    if (fits(3, p.sr, p.sb)) p.sa = 3;
     while (p.sr < MAX_RAW && fits(p.sa, p.sr + 2, p.sb)) p.sr += 2;   // (even: the two copy warps alternate)
     if (!resident) while (p.sb < MAX_B && fits(p.sa, p.sr, p.sb + 1)) ++p.sb;
     p.eligible = true;
   }
-  p.filter_bytes = (size_t)p.ntn * p.bn * p.num_kb * KB * p.G * 2 * pieces;
+  p.filter_bytes = (size_t)p.ntn * p.bn * p.num_kb * KB * p.G * 2;
   return p;
 }
 
-cudaError_t launch_pack_runs(const void* filter, void* scratch, const Geometry& g, bool f32, cudaStream_t stream) {
-  const RunsPlan p = plan_runs(g, f32);
+cudaError_t launch_pack_f16_runs(const uint16_t* filter, void* scratch, const Geometry& g, cudaStream_t stream) {
+  const RunsPlan p = plan_f16_runs(g);
   if (!p.eligible) return cudaErrorInvalidValue;
   unsigned char* base = static_cast<unsigned char*>(scratch);
-  const int es = f32 ? 4 : 2;
   const int64_t pitch = pack_channels(p.E, g.C) * g.T;
   int rows = 8;                                             // channels per block: staging within 40 KB
-  while (rows > 1 && rows * pitch * es > 40 * 1024) rows /= 2;
-  const size_t smem = (size_t)(rows * pitch * es);
+  while (rows > 1 && rows * pitch * ES > 40 * 1024) rows /= 2;
+  const size_t smem = (size_t)(rows * pitch * ES);
   dim3 grid((unsigned)p.num_kb, (unsigned)(p.ntn * p.bn / rows));
   if (grid.y > 65535) return cudaErrorInvalidValue;
-  uint32_t* status = reinterpret_cast<uint32_t*>(base);
-  if (f32)
-    pack_runs_kernel<true><<<grid, 256, smem, stream>>>(filter, base + kStatusBytes, status, g.C, g.Kh, g.Kw, g.s, p.E, p.G, g.Co,
-                                                        p.bn, p.num_kb, rows, (int)pitch, p.quad);
-  else
-    pack_runs_kernel<false><<<grid, 256, smem, stream>>>(filter, base + kStatusBytes, status, g.C, g.Kh, g.Kw, g.s, p.E, p.G, g.Co,
-                                                         p.bn, p.num_kb, rows, (int)pitch, p.quad);
+  pack_f16_runs_kernel<<<grid, 256, smem, stream>>>(filter, base + kStatusBytes, reinterpret_cast<uint32_t*>(base), g.C, g.Kh, g.Kw,
+                                                    g.s, p.E, p.G, g.Co, p.bn, p.num_kb, rows, (int)pitch, p.quad);
   return cudaGetLastError();
 }
 
-cudaError_t launch_conv_runs(const void* window, float* y, void* scratch, const Geometry& g, bool f32, cudaStream_t stream) {
-  const RunsPlan p = plan_runs(g, f32);
+cudaError_t launch_conv_f16_runs(const uint16_t* window, float* y, void* scratch, const Geometry& g, cudaStream_t stream) {
+  const RunsPlan p = plan_f16_runs(g);
   if (!p.eligible) return cudaErrorInvalidValue;
   unsigned char* base = static_cast<unsigned char*>(scratch);
-  const int64_t es = f32 ? 4 : 2;
   RunsParams q;
-  q.win = static_cast<const unsigned char*>(window);
+  q.win = reinterpret_cast<const unsigned char*>(window);
   q.fp = base + kStatusBytes;
   q.y = y;
   q.status = reinterpret_cast<uint32_t*>(base);
-  q.img_bytes = g.img_stride * es; q.chan_bytes = g.chan_stride * es; q.win_bytes = g.window_elems * es;
+  q.img_bytes = g.img_stride * ES; q.chan_bytes = g.chan_stride * ES; q.win_bytes = g.window_elems * ES;
   q.VQ = (uint32_t)p.VQ;
   q.div_pitch = fast_div((uint32_t)p.pitch);
   q.div_ho = fast_div((uint32_t)g.Ho);
@@ -794,12 +632,10 @@ cudaError_t launch_conv_runs(const void* window, float* y, void* scratch, const 
   q.rows = p.rows; q.halo = p.halo; q.region = p.region; q.octs = p.octs; q.raw_slot = p.raw_slot; q.a_stage = p.a_stage;
   q.bn = p.bn; q.ntn = p.ntn; q.nwork = p.nwork; q.sa = p.sa; q.sr = p.sr; q.sb = p.sb;
   q.slot_bytes = p.slot_bytes; q.resident = p.resident ? 1 : 0;
-  q.chain = g.K >= 288 ? 12 : 8;
   const int smem = 1024 + p.sa * p.a_stage + p.sb * p.slot_bytes + p.sr * p.raw_slot;
-  if (f32) return launch_form<true, 80>(q, smem, stream);
-  if (p.bn <= 64) return launch_form<false, 64>(q, smem, stream);
-  if (p.bn <= 128) return launch_form<false, 128>(q, smem, stream);
-  return launch_form<false, 256>(q, smem, stream);
+  if (p.bn <= 64) return launch_form<64>(q, smem, stream);
+  if (p.bn <= 128) return launch_form<128>(q, smem, stream);
+  return launch_form<256>(q, smem, stream);
 }
 
 }  // namespace im2win

@@ -13,7 +13,7 @@
 // 0.8e-7, K = 576 4.3e-7 -> 1.0e-7, K = 4608 1.2e-6 -> 1.8e-7, on inputs of both signs and of one.
 // Values whose pieces or sums leave the finite range give a non-finite accumulator; such outputs (and
 // those below 2^-90, where pieces get lost under bf16's smallest value) are computed again with fp32 FMAs in
-// the order of the FFMA kernel (exact_output).
+// the order of the FFMA kernel, from the window and a copy of the filter (exact_output).
 //
 // The GEMM is the shifted-view one of conv_f16_shift.cu: the window tensor's columns are staged once,
 //     S[piece][row = virtual column q][k2 = c*Kh + u]     (64 k2 = 128 bytes per row, 128-byte swizzle),
@@ -55,6 +55,7 @@ constexpr int kSplitSmem = 226 * 1024;        // dynamic shared memory a CTA may
 struct SplitParams {
   const float* __restrict__ win;
   const unsigned char* __restrict__ fp;       // packed filter: shared-memory images, see pack_f32_split_kernel
+  const float* __restrict__ f;                // the filter as given, for exact_output
   float* __restrict__ y;
   uint32_t* status;
   int64_t img_stride, strip, chan_stride;
@@ -67,7 +68,7 @@ struct SplitParams {
 __device__ __forceinline__ void wait_for_previous_kernel() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // (volatile: the loads of a batch stay together, ahead of the wait for the stage they are for; left to
-// itself the compiler moved them to their uses, one round trip per eight loads: 296 instead of XXX us)
+// itself the compiler may move them to their uses, one round trip per eight loads)
 __device__ __forceinline__ float ld_if(const float* p, bool ok) {
   float v = 0.f;
   asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %2, 0;\n\t@p ld.global.nc.f32 %0, [%1];\n\t}"
@@ -135,43 +136,58 @@ __device__ __forceinline__ void store16(float* base, int stride, const float (&v
   }
 }
 
-template <int BNMAX> struct Form {
+// PWG: producer warpgroups.  Two where a tile has several stages (3x3 on 64 channels at 56x56: 351 against 385 thousand
+// cycles with one), one with a single stage per tile (7x7 stems: 412 against 472 us) and beside 128 sums a thread.
+template <int BNMAX, int PWG_> struct Form {
+  static constexpr int PWG = PWG_;
   static constexpr bool CONCAT = BNMAX == 80;             // the filter pieces side by side in one operand
   static constexpr int ACC_COLS = BNMAX == 128 ? 128 : 256; // tensor memory: a ring of accumulators (CONCAT: of triples)
   static constexpr int NACC = 512 / ACC_COLS;
   static constexpr int ACC_LOG = BNMAX == 128 ? 2 : 1;
   static constexpr int CH = BNMAX == 80 ? 3 : BNMAX / 32; // 16-channel chunks per epilogue warp
-  static constexpr int PWG = BNMAX == 256 ? 1 : 2;        // producer warpgroups
   static constexpr int THREADS = 128 * (PWG + 3);
-  static constexpr int REGS_PRODUCER = 112;
-  static constexpr int REGS_MISC = BNMAX == 256 ? 64 : 48;
-  static constexpr int REGS_EPILOGUE = BNMAX == 256 ? 168 : 104;
-  // (the launch holds 128 or 96 registers a thread: 112 + 64 + 2*168 = 4*128, 2*112 + 48 + 2*104 = 5*96)
+  static constexpr int REGS_PRODUCER = 96;
+  static constexpr int REGS_MISC = 64;
+  static constexpr int REGS_EPILOGUE = PWG == 1 ? 176 : 112;
+  // (the launch holds 128 or 96 registers a thread: 96 + 64 + 2*176 = 4*128, 2*96 + 64 + 2*112 = 5*96)
 };
 
-// One output in fp32 FMAs, k ascending, for the values the split cannot hold.  The filter element is the sum of
-// its pieces (exact: the pack kernel keeps them finite for finite elements).
-__device__ __forceinline__ float exact_output(const SplitParams& q, bool concat, uint32_t n, int ho, int wo, int nt, int col) {
-  const float* wbase = q.win + (int64_t)n * q.img_stride + (int64_t)ho * q.strip + (int64_t)wo * q.s * q.Kh;
-  const unsigned char* frow = q.fp + (int64_t)nt * q.num_kb * q.Kw * 3 * q.bn * 128 + col * 128;
-  const int64_t piece = (int64_t)q.bn * 128;
+// One output in fp32 FMAs, k ascending, for the values the split cannot hold.
+__device__ __forceinline__ float exact_output(const SplitParams& q, uint32_t n, int ho, int wo, int co) {
+  const float* x = q.win + (int64_t)n * q.img_stride + (int64_t)ho * q.strip + (int64_t)wo * q.s * q.Kh;
+  const float* f = q.f + (int64_t)co * q.K2 * q.Kw;
   float acc = 0.f;
-  for (int c = 0; c < q.C; ++c)
+  for (int c = 0; c < q.C; ++c, x += q.chan_stride, f += q.Kh * q.Kw)
     for (int v = 0; v < q.Kw; ++v)
-      for (int u = 0; u < q.Kh; ++u) {
-        const int k2 = c * q.Kh + u, kb = k2 / KB, e = k2 - kb * KB;
-        const unsigned char* f = frow + ((int64_t)kb * q.Kw + v) * 3 * piece + ((((e >> 3) ^ (col & 7)) << 4) | ((e & 7) * 2));
-        auto part = [&](int p) {
-          return __uint_as_float((uint32_t)*reinterpret_cast<const uint16_t*>(f + (concat ? p : 2 - p) * piece) << 16);
-        };
-        acc = fmaf(wbase[(int64_t)c * q.chan_stride + v * q.Kh + u], (part(0) + part(1)) + part(2), acc);
-      }
+      for (int u = 0; u < q.Kh; ++u) acc = fmaf(x[v * q.Kh + u], f[u * q.Kw + v], acc);
   return acc;
 }
 
-template <int BNMAX>
-__global__ void __launch_bounds__(Form<BNMAX>::THREADS, 1) conv_f32_split_kernel(SplitParams q) {
-  using F = Form<BNMAX>;
+// The instructions of one filter operand of a unit, straight-line: a lone lane pays for every branch and address
+// computation between them.  CONCAT: the operand is [w1 | w2 | w3]; else it is piece 3 - p of the filter.
+template <bool CONCAT, int NKS>
+__device__ __forceinline__ void issue_steps(uint32_t d, uint32_t bn, uint32_t a, uint32_t sub_lo, uint32_t b, uint32_t id1,
+                                            uint32_t id2, uint32_t id3, uint32_t more, int p) {
+  if constexpr (CONCAT) {
+#pragma unroll
+    for (int j = 0; j < NKS; ++j) umma_f16_lohi(d, a + 2 * j, b + 2 * j, id3, j == 0 ? more : 1u);
+#pragma unroll
+    for (int j = 0; j < NKS; ++j) umma_f16_lohi(d + bn, a + sub_lo + 2 * j, b + 2 * j, id2, 1u);
+#pragma unroll
+    for (int j = 0; j < NKS; ++j) umma_f16_lohi(d + 2 * bn, a + 2 * sub_lo + 2 * j, b + 2 * j, id1, 1u);
+  } else {
+#pragma unroll
+    for (int i = 2; i >= 0; --i) {
+      if (i > p) continue;                                 // (p is a constant of the unrolled caller)
+#pragma unroll
+      for (int j = 0; j < NKS; ++j) umma_f16_lohi(d, a + i * sub_lo + 2 * j, b + 2 * j, id1, (uint32_t)(p | j));
+    }
+  }
+}
+
+template <int BNMAX, int PWG>
+__global__ void __launch_bounds__(Form<BNMAX, PWG>::THREADS, 1) conv_f32_split_kernel(SplitParams q) {
+  using F = Form<BNMAX, PWG>;
   extern __shared__ unsigned char smem_dyn[];
   unsigned char* smem = reinterpret_cast<unsigned char*>(((uintptr_t)smem_dyn + 1023) & ~(uintptr_t)1023);
   __shared__ __align__(8) uint64_t bars[2 * A_STAGES + 2 * MAX_B + 2 * MAX_ACC];
@@ -217,94 +233,77 @@ __global__ void __launch_bounds__(Form<BNMAX>::THREADS, 1) conv_f32_split_kernel
 
   if (wg < F::PWG) {
     // ---------------- producers: thread = row ------------------------------------------------------
-    if constexpr (BNMAX == 256) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(F::REGS_PRODUCER));
-    else asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(F::REGS_PRODUCER));
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(F::REGS_PRODUCER));
     const int tid = threadIdx.x & 127;
-    const int hrow = TILE_M + (tid >> 3), hch = tid & 7;   // halo item: a row below the tile, one chunk of it
-    const bool has_halo = tid < q.halo * 8;
-    const float *base = q.win, *hbase = q.win;             // this thread's rows of the tile that is being loaded
-    int lim = 0, hlim = 0;                                 // ... and how many column classes exist there (0: no such row)
-    // The stage being loaded: tile, stage inside the CTA's range, its k2-block and column class, running number.
-    int w = w_first, st = st0, kb = kb0, t = t0;
-    uint32_t sc = 0;
-    auto advance = [&]() {
-      ++sc;
-      if (++t == q.nsub) { t = 0; ++kb; }
-      if (++st == st1) { st = st0; kb = kb0; t = t0; w += w_step; }
-    };
-    auto locate = [&](uint32_t vq, const float*& ptr, int& classes) {
-      ptr = q.win;
-      classes = 0;
-      if (vq < q.VQ) {
-        const uint32_t sg = vq / (uint32_t)q.Wq;
-        const int i = (int)(vq - sg * (uint32_t)q.Wq);
-        const uint32_t n = sg / (uint32_t)q.Ho;
-        const int ho = (int)(sg - n * (uint32_t)q.Ho);
-        ptr += (int64_t)n * q.img_stride + (int64_t)ho * q.strip + (int64_t)i * q.s * q.Kh;
-        classes = q.Wp - i * q.s;
-      }
-    };
-    int here = -1;                                         // the position tile that base and hbase belong to
-    auto enter_tile = [&]() {
-      const int mt = w / q.ntn;
-      if (mt == here) return;
-      here = mt;
-      locate((uint32_t)mt * TILE_M + tid, base, lim);
-      if (has_halo) locate((uint32_t)mt * TILE_M + hrow, hbase, hlim);
-    };
-    auto chunks = [&]() { return kb == q.num_kb - 1 ? 2 * q.nks_last : 8; };   // the MMAs stop at the last step with real k2
-    auto load8 = [&](const float* src, bool row_ok, int ch, float (&v)[8]) {
-      const int4* kt = reinterpret_cast<const int4*>(koff_s + kb * KB);
-      const int4 o0 = kt[2 * ch], o1 = kt[2 * ch + 1];
-      const int32_t off[8] = {o0.x, o0.y, o0.z, o0.w, o1.x, o1.y, o1.z, o1.w};
-#pragma unroll
-      for (int e = 0; e < 8; ++e) v[e] = ld_if(src + off[e], row_ok && off[e] >= 0);
-    };
-    auto load_half = [&](int half, int nch, float (&v)[4][8]) {
-#pragma unroll
-      for (int c = 0; c < 4; ++c) load8(base + t * q.Kh, t < lim && 4 * half + c < nch, 4 * half + c, v[c]);
-    };
-    auto store8 = [&](uint32_t stage, int row, int ch, const float (&v)[8]) {
-      uint32_t p[3][4];
-#pragma unroll
-      for (int e = 0; e < 4; ++e) split2(v[2 * e], v[2 * e + 1], p[0][e], p[1][e], p[2][e]);
-      const uint32_t dst = stage + row * 128 + ((ch ^ (row & 7)) << 4);
-#pragma unroll
-      for (int i = 0; i < 3; ++i) st_shared16(dst + i * sub_bytes, p[i][0], p[i][1], p[i][2], p[i][3]);
-    };
-
-    // Half a stage (32 loads a thread) is on its way while the other half is split and stored; the first half
-    // of the warpgroup's next stage is requested before the second half of this one is stored.
     bool ok = true;
-    float va[4][8], vb[4][8], vh[8];
-    if (F::PWG == 2 && wg == 1) advance();
-    if (w < q.nwork) {
-      enter_tile();
-      load_half(0, chunks(), va);
-      if (has_halo && hch < chunks()) load8(hbase + t * q.Kh, t < hlim, hch, vh);
-    }
-    while (w < q.nwork) {
-      const int buf = sc & 1, nch = chunks();
-      const uint32_t stage = a_ring + buf * a_stage_bytes, parity = ((sc >> 1) & 1) ^ 1;
-      load_half(1, nch, vb);
-      ok = mbar_wait(a_empty0 + 8 * buf, parity, &abort_flag, q.status);
-      ok = __all_sync(0xffffffffu, ok);
-      if (!ok) break;
+    uint32_t sc = 0;                                       // stages so far, of all producers
+    for (int w = w_first; w < q.nwork && ok; w += w_step) {
+      const uint32_t q0 = (uint32_t)(w / q.ntn) * TILE_M;
+      // Row -> window column (class 0) and the number of classes that exist there (0 beyond the tensor).
+      auto locate = [&](uint32_t vq, const float*& base, int& lim) {
+        base = q.win;
+        lim = 0;
+        if (vq < q.VQ) {
+          const uint32_t sg = vq / (uint32_t)q.Wq;
+          const int i = (int)(vq - sg * (uint32_t)q.Wq);
+          const uint32_t n = sg / (uint32_t)q.Ho;
+          const int ho = (int)(sg - n * (uint32_t)q.Ho);
+          base += (int64_t)n * q.img_stride + (int64_t)ho * q.strip + (int64_t)i * q.s * q.Kh;
+          lim = q.Wp - i * q.s;
+        }
+      };
+      const float *base, *hbase = q.win;
+      int lim, hlim = 0;
+      locate(q0 + tid, base, lim);
+      const int hrow = TILE_M + (tid >> 3), hch = tid & 7;  // halo item: a row below the tile, one chunk of it
+      const bool has_halo = tid < q.halo * 8;
+      if (has_halo) locate(q0 + hrow, hbase, hlim);
+      int kb = kb0, t = t0;
+      for (int st = st0; st < st1; ++st, ++sc) {
+        if (F::PWG == 1 || (int)(sc & 1) == wg) {
+          const int buf = sc & 1;
+          const uint32_t stage = a_ring + buf * a_stage_bytes;
+          const int nch = kb == q.num_kb - 1 ? 2 * q.nks_last : 8;      // the MMAs stop at the last step with real k2
+          const int4* kt = reinterpret_cast<const int4*>(koff_s + kb * KB);
+          auto load8 = [&](const float* src, bool row_ok, int ch, float (&v)[8]) {
+            const int4 o0 = kt[2 * ch], o1 = kt[2 * ch + 1];
+            const int32_t off[8] = {o0.x, o0.y, o0.z, o0.w, o1.x, o1.y, o1.z, o1.w};
 #pragma unroll
-      for (int c = 0; c < 4; ++c) if (c < nch) store8(stage, tid, c, va[c]);
-      if (has_halo && hch < nch) store8(stage, hrow, hch, vh);
+            for (int e = 0; e < 8; ++e) v[e] = ld_if(src + off[e], row_ok && off[e] >= 0);
+          };
+          auto store8 = [&](int row, int ch, const float (&v)[8]) {
+            uint32_t p[3][4];
 #pragma unroll
-      for (int i = 0; i < F::PWG; ++i) advance();
-      if (w < q.nwork) {
-        enter_tile();
-        load_half(0, chunks(), va);
-        if (has_halo && hch < chunks()) load8(hbase + t * q.Kh, t < hlim, hch, vh);
+            for (int e = 0; e < 4; ++e) split2(v[2 * e], v[2 * e + 1], p[0][e], p[1][e], p[2][e]);
+            const uint32_t dst = stage + row * 128 + ((ch ^ (row & 7)) << 4);
+#pragma unroll
+            for (int i = 0; i < 3; ++i) st_shared16(dst + i * sub_bytes, p[i][0], p[i][1], p[i][2], p[i][3]);
+          };
+          const bool row_ok = t < lim;
+          const float* src = base + t * q.Kh;
+          float v[4][8], hv[8];
+#pragma unroll
+          for (int c = 0; c < 4; ++c) load8(src, row_ok && c < nch, c, v[c]);
+          const bool halo_now = has_halo && hch < nch;
+          if (halo_now) load8(hbase + t * q.Kh, t < hlim, hch, hv);
+          ok = mbar_wait(a_empty0 + 8 * buf, ((sc >> 1) & 1) ^ 1, &abort_flag, q.status);
+          ok = __all_sync(0xffffffffu, ok);
+          if (!ok) break;
+#pragma unroll
+          for (int c = 0; c < 4; ++c) if (c < nch) store8(tid, c, v[c]);
+          if (halo_now) store8(hrow, hch, hv);
+          if (nch > 4) {
+#pragma unroll
+            for (int c = 0; c < 4; ++c) load8(src, row_ok && 4 + c < nch, 4 + c, v[c]);
+#pragma unroll
+            for (int c = 0; c < 4; ++c) if (4 + c < nch) store8(tid, 4 + c, v[c]);
+          }
+          fence_proxy_async_smem();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(a_full0 + 8 * buf);
+        }
+        if (++t == q.nsub) { t = 0; ++kb; }
       }
-#pragma unroll
-      for (int c = 0; c < 4; ++c) if (4 + c < nch) store8(stage, tid, 4 + c, vb[c]);
-      fence_proxy_async_smem();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(a_full0 + 8 * buf);
     }
   } else if (wg == F::PWG) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(F::REGS_MISC));
@@ -319,77 +318,69 @@ __global__ void __launch_bounds__(Form<BNMAX>::THREADS, 1) conv_f32_split_kernel
       uint32_t sc = 0, ac = 0;                             // stages and chains so far
       int slot = 0;
       uint32_t bph = 0;
+      // A wait for a barrier that is already complete costs 200 cycles and more while the shared-memory pipe is busy, and
+      // the tensor pipe runs dry meanwhile: every barrier is looked at ahead of the instructions issued before it is
+      // needed, and waited for only where that look came too early.
+      uint32_t a_seen = 0, b_seen = 0, acc_seen = 0;
+      auto need = [&](uint32_t bar, uint32_t parity, uint32_t seen) {
+        if (__all_sync(0xffffffffu, seen != 0u)) return true;
+        return (bool)__all_sync(0xffffffffu, mbar_wait(bar, parity, &abort_flag, q.status));
+      };
+      auto next_slot = [&](int& sl, uint32_t& ph) { if (++sl == q.sb) { sl = 0; ph ^= 1u; } };
       for (int w = w_first; w < q.nwork && ok; w += w_step) {
         int kb = kb0, t = t0;
         for (int st = st0; st < st1 && ok; ++st, ++sc) {
           const int buf = sc & 1;
           const int nks = kb == q.num_kb - 1 ? q.nks_last : KB / 16;
-          ok = mbar_wait(a_full0 + 8 * buf, (sc >> 1) & 1, &abort_flag, q.status);
-          ok = __all_sync(0xffffffffu, ok);
+          ok = need(a_full0 + 8 * buf, (sc >> 1) & 1, a_seen);
           if (!ok) break;
+          tc_fence_after();
           uint32_t a_view = a_lo0 + (uint32_t)(buf * (a_stage_bytes >> 4));
           int links = 0;                                   // steps in the open chain; 0: none is open
           for (int v = t; v < q.Kw; v += q.s, a_view += 8u) {           // next view: one row (128 bytes) further down
             const int ab = ac & (F::NACC - 1);
             if (links == 0) {
-              ok = mbar_wait(acc_empty0 + 8 * ab, ((ac >> F::ACC_LOG) & 1) ^ 1, &abort_flag, q.status);
-              ok = __all_sync(0xffffffffu, ok);
+              ok = need(acc_empty0 + 8 * ab, ((ac >> F::ACC_LOG) & 1) ^ 1, acc_seen);
               if (!ok) break;
+              tc_fence_after();
             }
             const uint32_t d = tmem_acc + ab * F::ACC_COLS, more = links > 0;
             links += nks;
-            const bool last_link = !F::CONCAT || links + nks > q.chain || v + q.s >= q.Kw;
-            if constexpr (F::CONCAT) {
-              ok = mbar_wait(b_full0 + 8 * slot, bph, &abort_flag, q.status);
-              ok = __all_sync(0xffffffffu, ok);
+            const bool last_unit = v + q.s >= q.Kw;
+            const bool last_link = !F::CONCAT || links + nks > q.chain || last_unit;
+            // filter pieces: one operand (CONCAT), or one by one, smallest first: w3 meets x1, w2 meets x2 and x1, w1
+            // meets x3, x2 and x1
+#pragma unroll
+            for (int p = 0; p < (F::CONCAT ? 1 : 3); ++p) {
+              ok = need(b_full0 + 8 * slot, bph, b_seen);
               if (!ok) break;
-              tc_fence_after();
+              int nslot = slot;
+              uint32_t nbph = bph;
+              next_slot(nslot, nbph);
+              b_seen = mbar_test_wait(b_full0 + 8 * nslot, nbph);
+              if (F::CONCAT || p == 2) {
+                if (last_link) acc_seen = mbar_test_wait(acc_empty0 + 8 * ((ac + 1) & (F::NACC - 1)), (((ac + 1) >> F::ACC_LOG) & 1) ^ 1);
+                if (last_unit) a_seen = mbar_test_wait(a_full0 + 8 * (buf ^ 1), ((sc + 1) >> 1) & 1);
+              }
               const uint32_t b_lo = b_lo0 + (uint32_t)(slot * (q.slot_bytes >> 4));
               if (leader) {
-#pragma unroll
-                for (int j = 0; j < KB / 16; ++j)
-                  if (j < nks) umma_f16_lohi(d, a_view + 2 * j, b_lo + 2 * j, id3, more | (uint32_t)j);
-#pragma unroll
-                for (int j = 0; j < KB / 16; ++j)
-                  if (j < nks) umma_f16_lohi(d + q.bn, a_view + sub_lo + 2 * j, b_lo + 2 * j, id2, 1u);
-#pragma unroll
-                for (int j = 0; j < KB / 16; ++j)
-                  if (j < nks) umma_f16_lohi(d + 2 * q.bn, a_view + 2 * sub_lo + 2 * j, b_lo + 2 * j, id1, 1u);
+                if (nks == KB / 16) issue_steps<F::CONCAT, KB / 16>(d, q.bn, a_view, sub_lo, b_lo, id1, id2, id3, more, p);
+                else if (nks == 3) issue_steps<F::CONCAT, 3>(d, q.bn, a_view, sub_lo, b_lo, id1, id2, id3, more, p);
+                else if (nks == 2) issue_steps<F::CONCAT, 2>(d, q.bn, a_view, sub_lo, b_lo, id1, id2, id3, more, p);
+                else issue_steps<F::CONCAT, 1>(d, q.bn, a_view, sub_lo, b_lo, id1, id2, id3, more, p);
                 umma_commit(b_empty0 + 8 * slot);
+                if (F::CONCAT || p == 2) {
+                  if (last_link) umma_commit(acc_full0 + 8 * ab);
+                  if (last_unit) umma_commit(a_empty0 + 8 * buf);
+                }
               }
               __syncwarp();
-              if (++slot == q.sb) { slot = 0; bph ^= 1u; }
-            } else {
-              // filter pieces arrive smallest first: w3 meets x1, w2 meets x2 and x1, w1 meets x3, x2 and x1
-#pragma unroll
-              for (int p = 0; p < 3; ++p) {
-                ok = mbar_wait(b_full0 + 8 * slot, bph, &abort_flag, q.status);
-                ok = __all_sync(0xffffffffu, ok);
-                if (!ok) break;
-                tc_fence_after();
-                const uint32_t b_lo = b_lo0 + (uint32_t)(slot * (q.slot_bytes >> 4));
-                if (leader) {
-#pragma unroll
-                  for (int i = p; i >= 0; --i)
-#pragma unroll
-                    for (int j = 0; j < KB / 16; ++j)
-                      if (j < nks) umma_f16_lohi(d, a_view + i * sub_lo + 2 * j, b_lo + 2 * j, id1, (uint32_t)(p | j));
-                  umma_commit(b_empty0 + 8 * slot);
-                }
-                __syncwarp();
-                if (++slot == q.sb) { slot = 0; bph ^= 1u; }
-              }
-              if (!ok) break;
+              slot = nslot;
+              bph = nbph;
             }
-            if (last_link) {
-              if (leader) umma_commit(acc_full0 + 8 * ab);
-              ++ac;
-              links = 0;
-            }
-            __syncwarp();
+            if (!ok) break;
+            if (last_link) { ++ac; links = 0; }
           }
-          if (ok && leader) umma_commit(a_empty0 + 8 * buf);
-          __syncwarp();
           if (++t == q.nsub) { t = 0; ++kb; }
         }
       }
@@ -518,7 +509,7 @@ __global__ void __launch_bounds__(Form<BNMAX>::THREADS, 1) conv_f32_split_kernel
         }
         if (again) {
           for (int c = h * 16; c < limit; c += (c & 15) == 15 ? 17 : 1)
-            if (suspicious(yrow[(int64_t)c * q.HoWo])) yrow[(int64_t)c * q.HoWo] = exact_output(q, F::CONCAT, n, ho, i0, nt, c);
+            if (suspicious(yrow[(int64_t)c * q.HoWo])) yrow[(int64_t)c * q.HoWo] = exact_output(q, n, ho, i0, co0 + c);
         }
       }
     }
@@ -551,7 +542,7 @@ __global__ void __launch_bounds__(Form<BNMAX>::THREADS, 1) conv_f32_split_kernel
           float sum = v[0];
 #pragma unroll
           for (int r = 1; r < 8; ++r) sum += v[r];
-          if (suspicious(sum)) sum = exact_output(q, F::CONCAT, n, ho, i0, nt, c);
+          if (suspicious(sum)) sum = exact_output(q, n, ho, i0, co0 + c);
           yrow[(int64_t)c * q.HoWo] = sum;
         }
       }
@@ -581,10 +572,11 @@ __global__ void __launch_bounds__(Form<BNMAX>::THREADS, 1) conv_f32_split_kernel
 
 // Filter -> the images the copy warp loads: for every (channel tile nt, k2-block kb, kernel column v) the three
 // pieces [bn channels][64 k2] in the 128-byte-swizzled order of shared memory, smallest first, or largest first
-// where they form one operand (bn <= 80).  One block: `rows` channels of one k2-block; its source is one
-// contiguous run of the OIHW filter per channel.  Channels beyond Co and k2 beyond C*Kh are zeros.
+// where they form one operand (bn <= 80); and a copy of the filter as given.  One block: `rows` channels of one
+// k2-block; its source is one contiguous run of the OIHW filter per channel.  Channels beyond Co and k2 beyond C*Kh are
+// zeros.
 __global__ void __launch_bounds__(256) pack_f32_split_kernel(const float* __restrict__ f, unsigned char* __restrict__ fp,
-                                                             uint32_t* __restrict__ status, int K2, int Kw, int Co, int bn,
+                                                             float* __restrict__ copy, uint32_t* __restrict__ status, int K2, int Kw, int Co, int bn,
                                                              int num_kb, int rows, int concat) {
   extern __shared__ float pack_f[];
   if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < kStatusBytes / 4) status[threadIdx.x] = 0u;
@@ -593,8 +585,15 @@ __global__ void __launch_bounds__(256) pack_f32_split_kernel(const float* __rest
   const int run = nreal * Kw, pitch = KB * Kw;
   for (int r = 0; r < rows; ++r) {
     const int co = row0 + r;
-    const float* src = f + ((int64_t)co * K2 + (int64_t)kb * KB) * Kw;
-    for (int i = threadIdx.x; i < pitch; i += blockDim.x) pack_f[r * pitch + i] = (co < Co && i < run) ? __ldg(src + i) : 0.f;
+    const int64_t first = ((int64_t)co * K2 + (int64_t)kb * KB) * Kw;
+    for (int i = threadIdx.x; i < pitch; i += blockDim.x) {
+      float v = 0.f;
+      if (co < Co && i < run) {
+        v = __ldg(f + first + i);
+        copy[first + i] = v;
+      }
+      pack_f[r * pitch + i] = v;
+    }
   }
   __syncthreads();
   const int items = rows * Kw * 8;
@@ -605,27 +604,7 @@ __global__ void __launch_bounds__(256) pack_f32_split_kernel(const float* __rest
     const float* src = pack_f + r * pitch + ch * 8 * Kw + v;
     uint32_t p[3][4];
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      float a[2] = {src[(2 * e) * Kw], src[(2 * e + 1) * Kw]};
-      uint32_t w[3] = {0u, 0u, 0u};
-#pragma unroll
-      for (int k = 0; k < 2; ++k) {
-        // The pieces of a finite element are finite (the first is cut where rounding would overflow); an
-        // infinity or NaN is its own first piece, the others are zero: the sum of the pieces is the element.
-        uint32_t b1 = cvt_bf16x2(a[k], 0.f) & 0xffffu, b2 = 0u, b3 = 0u;
-        const bool finite = (__float_as_uint(a[k]) & 0x7f800000u) != 0x7f800000u;
-        if (finite) {
-          if ((b1 & 0x7f80u) == 0x7f80u) b1 = __float_as_uint(a[k]) >> 16;
-          const float r1 = a[k] - __uint_as_float(b1 << 16);
-          b2 = cvt_bf16x2(r1, 0.f) & 0xffffu;
-          b3 = cvt_bf16x2(r1 - __uint_as_float(b2 << 16), 0.f) & 0xffffu;
-        }
-        w[0] |= b1 << (16 * k);
-        w[1] |= b2 << (16 * k);
-        w[2] |= b3 << (16 * k);
-      }
-      p[0][e] = w[0]; p[1][e] = w[1]; p[2][e] = w[2];
-    }
+    for (int e = 0; e < 4; ++e) split2(src[(2 * e) * Kw], src[(2 * e + 1) * Kw], p[0][e], p[1][e], p[2][e]);
     const int64_t piece = (int64_t)bn * 128;
     unsigned char* dst = fp + (((int64_t)nt * num_kb + kb) * Kw + v) * 3 * piece + rr * 128 + ((ch ^ (rr & 7)) << 4);
 #pragma unroll
@@ -650,13 +629,13 @@ double step_cycles(int bn) {
   return bn <= 80 ? mma(3 * bn) + mma(2 * bn) + mma(bn) : 6 * mma(bn);
 }
 
-template <int BNMAX>
+template <int BNMAX, int PWG>
 cudaError_t launch_form(const SplitParams& q, int smem, cudaStream_t stream) {
   static bool attr_done[64] = {};
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
   if (!attr_done[dev]) {
-    cudaError_t e = cudaFuncSetAttribute(conv_f32_split_kernel<BNMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSplitSmem);
+    cudaError_t e = cudaFuncSetAttribute(conv_f32_split_kernel<BNMAX, PWG>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSplitSmem);
     if (e != cudaSuccess) return e;
     attr_done[dev] = true;
   }
@@ -668,12 +647,12 @@ cudaError_t launch_form(const SplitParams& q, int smem, cudaStream_t stream) {
   attr[1].val.clusterDim.x = (unsigned)q.split; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
   const int grid = q.split > 1 ? q.nwork * q.split : (q.nwork < 148 ? q.nwork : 148);
   cfg.gridDim = dim3((unsigned)grid, 1, 1);
-  cfg.blockDim = dim3(Form<BNMAX>::THREADS, 1, 1);
+  cfg.blockDim = dim3(Form<BNMAX, PWG>::THREADS, 1, 1);
   cfg.dynamicSmemBytes = (size_t)smem;
   cfg.stream = stream;
   cfg.attrs = attr;
   cfg.numAttrs = q.split > 1 ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, conv_f32_split_kernel<BNMAX>, q);
+  return cudaLaunchKernelEx(&cfg, conv_f32_split_kernel<BNMAX, PWG>, q);
 }
 
 }  // namespace
@@ -724,7 +703,8 @@ F32SplitPlan plan_f32_split(const Geometry& g) {
     }
   }
   if (!p.eligible) return p;
-  p.filter_bytes = (size_t)p.packed_rows * p.num_kb * KB * g.Kw * 6;
+  p.copy_off = ((size_t)p.packed_rows * p.num_kb * KB * g.Kw * 6 + 255) / 256 * 256;
+  p.filter_bytes = p.copy_off + (size_t)g.Co * g.K * 4;
   return p;
 }
 
@@ -737,7 +717,7 @@ cudaError_t launch_pack_f32_split(const float* filter, void* scratch, const Geom
   const size_t smem = (size_t)rows * KB * g.Kw * 4;
   dim3 grid((unsigned)p.num_kb, (unsigned)(p.ntn * p.bn / rows));
   if (grid.y > 65535) return cudaErrorInvalidValue;
-  pack_f32_split_kernel<<<grid, 256, smem, stream>>>(filter, base + kStatusBytes, reinterpret_cast<uint32_t*>(base), g.C * g.Kh,
+  pack_f32_split_kernel<<<grid, 256, smem, stream>>>(filter, base + kStatusBytes, reinterpret_cast<float*>(base + kStatusBytes + p.copy_off), reinterpret_cast<uint32_t*>(base), g.C * g.Kh,
                                                      g.Kw, g.Co, p.bn, p.num_kb, rows, p.bn <= 80 ? 1 : 0);
   return cudaGetLastError();
 }
@@ -749,6 +729,7 @@ cudaError_t launch_conv_f32_split(const float* window, float* y, void* scratch, 
   SplitParams q;
   q.win = window;
   q.fp = base + kStatusBytes;
+  q.f = reinterpret_cast<const float*>(base + kStatusBytes + p.copy_off);
   q.y = y;
   q.status = reinterpret_cast<uint32_t*>(base);
   q.img_stride = g.img_stride; q.strip = g.strip; q.chan_stride = g.chan_stride;
@@ -763,9 +744,9 @@ cudaError_t launch_conv_f32_split(const float* window, float* y, void* scratch, 
   const int smem = 1024 + rings;
   if (p.split > 1 && rings < p.bn * TILE_M * 4) return cudaErrorInvalidValue;
   switch (form_of(p.bn)) {
-    case 80: return launch_form<80>(q, smem, stream);
-    case 128: return launch_form<128>(q, smem, stream);
-    default: return launch_form<256>(q, smem, stream);
+    case 80: return p.num_kb == 1 ? launch_form<80, 1>(q, smem, stream) : launch_form<80, 2>(q, smem, stream);
+    case 128: return launch_form<128, 2>(q, smem, stream);
+    default: return launch_form<256, 1>(q, smem, stream);
   }
 }
 

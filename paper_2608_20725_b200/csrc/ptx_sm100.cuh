@@ -57,6 +57,18 @@ __device__ __forceinline__ uint32_t mbar_try_wait(uint32_t bar, uint32_t parity)
       : "memory");
   return ok;
 }
+// One look at a barrier, without the suspension that try_wait may add.
+__device__ __forceinline__ uint32_t mbar_test_wait(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return ok;
+}
 // Bounded waits.  A wait first polls SPIN_CHUNK times in line; only a wait that is still pending
 // then (milliseconds: each poll may suspend the thread for a while) enters the slow path below,
 // which gives up after SPIN_LIMIT polls or SPIN_TIME_NS of wall time, whichever comes first, or as

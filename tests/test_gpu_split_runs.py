@@ -1,0 +1,134 @@
+"""The fp32 kernel that runs on the tensor cores (three bf16 pieces per operand) and the run-staged fp16 kernel,
+forced over the forms and sizes where they can go wrong: every channel-tile form, tiles shared by clusters of CTAs,
+partly filled tiles, k2-blocks and columns, strides that do not divide the strip, several images in a tile, values
+that the split cannot hold.
+
+Tolerances: fp32 outputs within 1e-5 * sum|x||w| (gpu_helpers), integer-valued inputs exactly; the error of the split
+against the oracle's 64-bit values is at most that of the FFMA kernel on the same inputs.
+"""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2608_20725_b200 import binding, workloads
+from paper_2608_20725_b200.workloads import Layer
+from gpu_helpers import check_conv, gpu_conv, oracle_inputs
+
+pytestmark = pytest.mark.gpu
+
+
+def L(name, N, C, H, W, Co, Kh, Kw, s, p, seed, xd="normal01"):
+    return Layer(name, N, C, H, W, Co, Kh, Kw, s, p, seed, xd, "he_normal")
+
+
+# (layer, channel tiles, CTAs per tile) that the plan accepts for it; None: what the library picks
+SPLIT = [
+    (L("k72", 2, 8, 10, 12, 7, 3, 3, 1, 1, 200), [None, (16, 1)]),                    # shortest reductions, 7 of 16 channels
+    (L("co80", 2, 24, 13, 12, 80, 3, 3, 1, 1, 201), [(80, 1), (80, 2), (48, 2), (16, 1)]),   # pieces side by side, two k2-blocks
+    (L("co100", 3, 22, 12, 15, 100, 3, 3, 1, 1, 202), [(112, 1), (112, 2), (64, 2)]),   # pieces one by one, the last k2-block one step
+    (L("co300", 1, 70, 9, 9, 300, 3, 3, 1, 1, 203), [None, (160, 1), (160, 4), (112, 2), (80, 4), (48, 1)]),
+    (L("co256_s2", 2, 33, 15, 17, 256, 3, 3, 2, 1, 204), [(256, 1), (256, 4), (128, 2), (64, 4)]),   # two column classes
+    (L("s4_rag", 1, 6, 30, 41, 20, 11, 11, 4, 0, 205), [None, (32, 4), (32, 8)]),     # stride 4, cut-short last column, 2 rows below
+    (L("k11", 1, 7, 20, 18, 33, 11, 11, 1, 5, 206), [None, (48, 2)]),                 # ten rows below the tile
+    (L("imgs", 9, 30, 5, 5, 40, 3, 3, 1, 1, 207, "uniform01"), [None, (48, 2)]),      # several images in a tile
+    (L("k1x1", 3, 130, 7, 7, 65, 1, 1, 1, 0, 208, "uniform01"), [None, (80, 2), (48, 1)]),
+    (L("rect", 2, 9, 21, 14, 18, 5, 3, 2, 2, 209), [None, (32, 2)]),
+    (L("many_tiles", 40, 16, 24, 24, 24, 3, 3, 1, 1, 210, "uniform01"), [None]),      # more tiles than SMs: the rings go round
+]
+
+
+def force_split(monkeypatch, form):
+    monkeypatch.setenv("IM2WIN_F32_KERNEL", "split")
+    if form:
+        monkeypatch.setenv("IM2WIN_F32_SPLIT_BN", str(form[0]))
+        monkeypatch.setenv("IM2WIN_F32_SPLIT_CTAS", str(form[1]))
+
+
+@pytest.mark.parametrize("layer,form", [(l, f) for l, forms in SPLIT for f in forms], ids=lambda v: getattr(v, "name", str(v)))
+def test_conv_f32_split_forms(layer, form, monkeypatch):
+    force_split(monkeypatch, form)
+    dims = layer.dims()
+    assert binding.im2win_conv_kernel_name(dims, binding.F32) == "f32-split"
+    x, f = workloads.make_small_integer_inputs(layer)
+    y, _, _ = gpu_conv(x, f, dims, "f32")
+    yr, _ = oracle.conv_direct(x.numpy(), f.numpy(), dims)
+    assert np.array_equal(y.astype(np.float64), yr)
+    x, f = workloads.make_inputs(layer)
+    y, _, _ = gpu_conv(x, f, dims, "f32")
+    yr, ar = oracle.conv_direct(x.numpy(), f.numpy(), dims)
+    check_conv(y, yr, ar, "f32", layer.name)
+    monkeypatch.setenv("IM2WIN_F32_KERNEL", "ffma")
+    z, _, _ = gpu_conv(x, f, dims, "f32")
+    assert np.linalg.norm(y - yr) <= np.linalg.norm(z - yr)
+
+
+@pytest.mark.parametrize("form", [(80, 1), (80, 2), (112, 1), (256, 2)], ids=str)
+@pytest.mark.parametrize("what", ["inf", "nan", "lowest", "overflow", "inf weight", "tiny", "subnormal", "tiny weight"])
+def test_conv_f32_split_values_beyond_the_pieces(form, what, monkeypatch):
+    """Outputs that meet infinities, NaNs, values next to the largest finite one, or only values so small that pieces
+    are lost, are what the FFMA kernel computes: the same bits where they are not finite or tiny, and nothing else is
+    disturbed."""
+    layer = L("values", 2, 24, 9, 12, form[0] - 5, 3, 3, 1, 1, 220)
+    dims = layer.dims()
+    x, f = workloads.make_inputs(layer)
+    x, f = x.clone(), f.clone()
+    if what == "inf": x[0, 3, 4, 5] = float("inf")
+    if what == "nan": x[1, 7, 0, 11] = float("nan")
+    if what == "lowest": x[0, 1] = torch.finfo(torch.float32).min
+    if what == "overflow":                   # (one sign, so that no order of the sum stays finite)
+        x[1, :, 2] = 3e38
+        f = f.abs()
+    if what == "inf weight": f[6, 2, 1, 1] = float("-inf")
+    if what == "tiny": x *= 1e-36
+    if what == "subnormal": x *= 1e-39
+    if what == "tiny weight": f *= 1e-37
+    force_split(monkeypatch, form)
+    y, _, _ = gpu_conv(x, f, dims, "f32")
+    monkeypatch.setenv("IM2WIN_F32_KERNEL", "ffma")
+    z, _, _ = gpu_conv(x, f, dims, "f32")
+    same = (y == z) | (np.isnan(y) & np.isnan(z))
+    odd = ~np.isfinite(z) | (np.abs(z) < 2.0 ** -90)
+    assert odd.any() or what == "lowest"
+    assert same[odd].all() and np.array_equal(np.isfinite(y), np.isfinite(z))
+    ok = ~odd
+    if ok.any():
+        a, b = y[ok].astype(np.float64), z[ok].astype(np.float64)
+        scale = np.abs(b).max()
+        assert np.linalg.norm((a - b) / scale) <= 1e-6 * np.linalg.norm(b / scale)
+
+
+RUNS = [l for l, _ in SPLIT] + [
+    L("runs_quad", 2, 3, 19, 23, 20, 7, 7, 2, 3, 230),       # up to four channels: a unit is four channels at two columns' elements
+    L("runs_quad1", 3, 2, 12, 9, 16, 1, 1, 1, 0, 231),       # ... one unit, one step
+    L("runs_ragged3", 2, 7, 20, 21, 9, 4, 4, 3, 0, 232),     # stride 3, cut-short last column, tensor ends off a 16-byte boundary
+    L("runs_c9", 2, 9, 15, 17, 270, 2, 3, 1, 1, 233),        # an octet with one channel, two channel tiles
+    L("runs_resident", 6, 24, 30, 30, 48, 3, 3, 1, 1, 234),  # filter resident, tiles enough to go round the rings
+]
+
+
+@pytest.mark.parametrize("layer", RUNS, ids=lambda l: l.name)
+def test_conv_f16_runs(layer, monkeypatch):
+    monkeypatch.setenv("IM2WIN_F16_KERNEL", "runs")
+    dims = layer.dims()
+    if binding.im2win_conv_kernel_name(dims, binding.F16) != "f16-runs":
+        pytest.skip("its rings do not fit this layer")
+    x, f = workloads.make_small_integer_inputs(layer)
+    y, _, _ = gpu_conv(x, f, dims, "f16")
+    yr, _ = oracle.conv_direct(x.numpy(), f.numpy(), dims)
+    assert np.array_equal(y.astype(np.float64), yr)
+    x, f = workloads.make_inputs(layer)
+    y, _, _ = gpu_conv(x, f, dims, "f16")
+    xo, fo = oracle_inputs(x, f, "f16")
+    yr, ar = oracle.conv_direct(xo, fo, dims)
+    check_conv(y, yr, ar, "f16", layer.name)
+    # an infinity and a NaN reach exactly the outputs whose windows hold them (strided kernels are widened by zeros)
+    xs = x.clone()
+    xs.view(-1)[xs.numel() // 3] = float("inf")
+    xs.view(-1)[xs.numel() // 2] = float("nan")
+    y, _, _ = gpu_conv(xs, f, dims, "f16")
+    monkeypatch.setenv("IM2WIN_F16_KERNEL", "gather")
+    z, _, _ = gpu_conv(xs, f, dims, "f16")
+    odd = ~np.isfinite(z)
+    assert np.array_equal(np.isfinite(y), ~odd) and np.array_equal(np.isnan(y), np.isnan(z))
+    assert np.array_equal(np.sign(y[np.isinf(z)]), np.sign(z[np.isinf(z)]))

@@ -1,0 +1,23 @@
+"""Host-side rules of the kernel choice (no GPU): which fp32 kernel a layer takes, and that the scratch a caller was told
+to provide serves every smaller batch of the same layer, whatever kernel that one takes."""
+import pytest
+
+from paper_2608_20725_b200 import binding
+
+LAYERS = [(128, 64, 56, 56, 64, 3, 3, 1, 1), (128, 512, 7, 7, 512, 3, 3, 1, 1), (13, 37, 45, 61, 75, 5, 5, 2, 2),
+          (64, 256, 28, 28, 256, 11, 11, 1, 5), (128, 3, 224, 224, 64, 7, 7, 2, 3), (96, 9, 15, 17, 270, 2, 3, 1, 1),
+          (8, 512, 14, 14, 90, 11, 11, 4, 5), (160, 5, 8, 224, 17, 3, 3, 2, 0)]
+
+
+@pytest.mark.parametrize("layer", LAYERS, ids=str)
+@pytest.mark.parametrize("dtype", [binding.F32, binding.F16])
+def test_scratch_serves_smaller_batches(layer, dtype):
+    whole = binding.im2win_workspace_size(binding.make_shape(*layer), dtype)[1]
+    for n in range(1, layer[0]):
+        assert binding.im2win_workspace_size(binding.make_shape(n, *layer[1:]), dtype)[1] <= whole
+
+
+@pytest.mark.parametrize("C,K,want", [(3, 3, "f32-ffma"), (63, 1, "f32-ffma"), (64, 1, "f32-split"), (8, 3, "f32-split"),
+                                      (600, 11, "f32-ffma")])       # 27, 63, 64, 72 terms; an offset table too long
+def test_f32_kernel_by_length_of_the_reduction(C, K, want):
+    assert binding.im2win_conv_kernel_name((2, C, 20, 20, 24, K, K, 1, K // 2), binding.F32) == want
