@@ -130,9 +130,15 @@ im2win_status scratch_layout(const Geometry& g, im2win_dtype dtype, ScratchLayou
       const size_t mat_total = (size_t)round_up((int64_t)mat.scratch_bytes, 256);
       if (mat_total > l->total) l->total = mat_total;
     }
+    // Layers that neither the one-k-block kernel nor a tiled-copy kernel takes: kernels up to three virtual columns
+    // (Kw <= 3 s) go to the run-staged kernel where they are strided or have more than 64 output channels, and so does
+    // what the shifted-view kernel cannot stage.  Measured against the latter: 3x3 with stride 2 1.1 to 1.8 times faster
+    // (256 -> 512 channels at 28x28, batch 128: 140 -> 115 us), 3x3 with stride 1 on 128 to 379 channels 1.2 to 1.6;
+    // 0.8 to 1.0 on fewer channels, 0.5 to 0.9 on 5x5 to 11x11 with stride 1, whose tall tiles share filter stages.
     const RunsPlan runs = plan_f16_runs(g);
     if (runs.eligible) {
-      l->f16_runs = force ? strcmp(force, "runs") == 0 : false;
+      const bool rest = !l->f16_stem && !l->f16_mat && !l->f16_raw;
+      l->f16_runs = force ? strcmp(force, "runs") == 0 : rest && (!l->f16_shift || (runs.G <= 3 && (g.s > 1 || g.Co > 64)));
       const size_t runs_total = (size_t)round_up(kStatusBytes + (int64_t)runs.filter_bytes, 256);
       if (runs_total > l->total) l->total = runs_total;
     }
