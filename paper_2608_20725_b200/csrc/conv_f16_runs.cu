@@ -21,8 +21,11 @@
 // write the units of S.  Gathering with 2-byte global loads instead (conv_f16_shift.cu) makes every load instruction
 // touch 32 rows s*Kh elements apart: three or more L1 wavefronts each, and a round trip to memory per batch.
 //
-// What bounds it: the shared-memory pipe, which carries the MMA's operand reads (32 + N/4 cycles per instruction of
-// M = 128, K = 16), the copies, the read-back and the S stores.
+// What bounds it: the staging warps' read-back (without it 89 us where the whole takes 107) and the shared-memory pipe,
+// which carries the MMA's operand reads (32 + N/4 cycles per instruction of M = 128, K = 16), the copies, the read-back
+// and the S stores.  Measured against the gathering kernel: 3x3 stride 2 on 256 -> 512 channels at 28x28, batch 128,
+// 140 -> 115 us (515 TFLOP/s); 5x5 stride 2 on 37 -> 75 channels at 45x61, batch 13, 27 -> 17 us.  Eight staging warps and
+// not sixteen (128 us): more of them take issue slots from the MMA warp.
 #include <cuda_fp16.h>
 #include <stdlib.h>
 #include <string.h>
@@ -57,7 +60,7 @@ FastDiv fast_div(uint32_t d) {
 
 struct RunsParams {
   const unsigned char* __restrict__ win;
-  const unsigned char* __restrict__ fp;       // packed filter: shared-memory images, see pack_runs_kernel
+  const unsigned char* __restrict__ fp;       // packed filter: shared-memory images, see pack_f16_runs_kernel
   float* __restrict__ y;
   uint32_t* status;
   int64_t img_bytes, chan_bytes, win_bytes;   // of one image, one channel plane, the whole window tensor
