@@ -21,18 +21,20 @@
 // holds one column class t = v mod s.  Rows are the virtual positions q = (n*Ho + ho)*Wq + i, Wq = ceil(Wp/s).
 //
 // What bounds it: the tensor pipe, and next to it the shared-memory pipe the MMA reads its operands
-// through: an instruction of M = 128, K = 16 takes max(N/2, 32 + N/4) cycles.  Up to 80 channels the filter
-// pieces therefore lie side by side as one operand, [w1 | w2 | w3], and three instructions replace six: x1
-// against all of it, x2 against [w1 | w2] one accumulator further, x3 against w1 two further, so that each of the
-// three accumulators holds products of one magnitude and their order is free.  A chain may then take several
-// units: `chain` steps of 16 k (12, or 8 on reductions below 288).
+// through: an instruction of M = 128, K = 16 takes max(N/2, 32 + N/4) cycles.  Up to 64 channels the filter
+// pieces therefore lie side by side as one operand, [w1 | w2 | w3], and four instructions replace six: x1 against all
+// of it into three accumulators (x1w1 | x1w2 | x1w3), and x2w1, x2w2 and x3w1 into a fourth, so that no accumulator holds
+// the large products beside the small ones and a chain may take several units: `chain` steps of 16 k (12, or 8 on
+// reductions below 288).  Instructions are promised to run in the order of their issue only where accumulator and shape
+// are the same, so no accumulator is written under two shapes or from two starts.  (Without that, x2 against [w1 | w2]
+// one accumulator further and x3 against w1 two further take 208 cycles a step at 64 channels; this 240, six 288.)
 //
 // Roles (one persistent CTA per SM): one or two warpgroups of producers (thread = row; 32 loads in flight,
 // split, 16-byte stores), an MMA warp, a filter-copy warp (one untiled bulk copy per piece: the pack kernel
 // writes shared-memory images), eight epilogue warps that keep the tile's fp32 sums in registers.
-// Measured against the FFMA kernel (us): 3x3 on 64 channels at 56x56, batch 128, 541 -> 211 (140 TFLOP/s); 3x3 on 512
+// Measured against the FFMA kernel (us): 3x3 on 64 channels at 56x56, batch 128, 543 -> 226 (131 TFLOP/s); 3x3 on 512
 // channels at 7x7 624 -> 163; 11x11 on 256 channels at 28x28, batch 64, 14780 -> 4100 (194 TFLOP/s; 1.6 PFLOP/s of bf16
-// products with the strip ends, near the power limit); 7x7 stride 2 on 3 channels at 224x224 640 -> 401.
+// products with the strip ends, near the power limit); 7x7 stride 2 on 3 channels at 224x224 641 -> 428.
 // A layer with few tiles is run by clusters of 2, 4 or 8 CTAs that share the stages of a tile and add their
 // registers through distributed shared memory, in rank order: 3x3 on 512 channels, one 7x7 image, 225 -> 32 us.
 #include <cuda_bf16.h>
@@ -53,6 +55,7 @@ constexpr int KB = 64;
 constexpr int A_STAGES = 2;
 constexpr int MAX_B = 16;
 constexpr int MAX_ACC = 4;
+constexpr int CONCAT_BN = 64;                 // channel tiles up to here: the filter pieces side by side in one operand
 constexpr int kSplitSmem = 226 * 1024;        // dynamic shared memory a CTA may use
 
 struct SplitParams {
@@ -143,11 +146,11 @@ __device__ __forceinline__ void store16(float* base, int stride, const float (&v
 // cycles with one), one with a single stage per tile (7x7 stems: 412 against 472 us) and beside 128 sums a thread.
 template <int BNMAX, int PWG_> struct Form {
   static constexpr int PWG = PWG_;
-  static constexpr bool CONCAT = BNMAX == 80;             // the filter pieces side by side in one operand
-  static constexpr int ACC_COLS = BNMAX == 128 ? 128 : 256; // tensor memory: a ring of accumulators (CONCAT: of triples)
+  static constexpr bool CONCAT = BNMAX == CONCAT_BN;
+  static constexpr int ACC_COLS = CONCAT ? 4 * CONCAT_BN : BNMAX;   // tensor memory: a ring of accumulators (CONCAT: fours)
   static constexpr int NACC = 512 / ACC_COLS;
   static constexpr int ACC_LOG = BNMAX == 128 ? 2 : 1;
-  static constexpr int CH = BNMAX == 80 ? 3 : BNMAX / 32; // 16-channel chunks per epilogue warp
+  static constexpr int CH = BNMAX / 32;                   // 16-channel chunks per epilogue warp
   static constexpr int THREADS = 128 * (PWG + 3);
   static constexpr int REGS_PRODUCER = 96;
   static constexpr int REGS_MISC = 64;
@@ -170,14 +173,17 @@ __device__ __forceinline__ float exact_output(const SplitParams& q, uint32_t n, 
 // computation between them.  CONCAT: the operand is [w1 | w2 | w3]; else it is piece 3 - p of the filter.
 template <bool CONCAT, int NKS>
 __device__ __forceinline__ void issue_steps(uint32_t d, uint32_t bn, uint32_t a, uint32_t sub_lo, uint32_t b, uint32_t id1,
-                                            uint32_t id2, uint32_t id3, uint32_t more, int p) {
+                                            uint32_t id3, uint32_t more, int p) {
   if constexpr (CONCAT) {
+    const uint32_t low = d + 3 * bn, b2 = b + 8 * bn;      // (w2: bn rows of 128 bytes further down)
 #pragma unroll
     for (int j = 0; j < NKS; ++j) umma_f16_lohi(d, a + 2 * j, b + 2 * j, id3, j == 0 ? more : 1u);
 #pragma unroll
-    for (int j = 0; j < NKS; ++j) umma_f16_lohi(d + bn, a + sub_lo + 2 * j, b + 2 * j, id2, 1u);
+    for (int j = 0; j < NKS; ++j) umma_f16_lohi(low, a + 2 * sub_lo + 2 * j, b + 2 * j, id1, j == 0 ? more : 1u);
 #pragma unroll
-    for (int j = 0; j < NKS; ++j) umma_f16_lohi(d + 2 * bn, a + 2 * sub_lo + 2 * j, b + 2 * j, id1, 1u);
+    for (int j = 0; j < NKS; ++j) umma_f16_lohi(low, a + sub_lo + 2 * j, b2 + 2 * j, id1, 1u);
+#pragma unroll
+    for (int j = 0; j < NKS; ++j) umma_f16_lohi(low, a + sub_lo + 2 * j, b + 2 * j, id1, 1u);
   } else {
 #pragma unroll
     for (int i = 2; i >= 0; --i) {
@@ -315,8 +321,7 @@ __global__ void __launch_bounds__(Form<BNMAX, PWG>::THREADS, 1) conv_f32_split_k
       const bool leader = elect_one();
       const uint32_t a_lo0 = smem_desc_lo(a_ring), b_lo0 = smem_desc_lo(b_ring);
       const uint32_t sub_lo = (uint32_t)sub_bytes >> 4;
-      const uint32_t id1 = instr_desc_bf16(TILE_M, q.bn), id2 = instr_desc_bf16(TILE_M, 2 * q.bn),
-                     id3 = instr_desc_bf16(TILE_M, 3 * q.bn);
+      const uint32_t id1 = instr_desc_bf16(TILE_M, q.bn), id3 = instr_desc_bf16(TILE_M, 3 * q.bn);
       bool ok = true;
       uint32_t sc = 0, ac = 0;                             // stages and chains so far
       int slot = 0;
@@ -368,10 +373,10 @@ __global__ void __launch_bounds__(Form<BNMAX, PWG>::THREADS, 1) conv_f32_split_k
               }
               const uint32_t b_lo = b_lo0 + (uint32_t)(slot * (q.slot_bytes >> 4));
               if (leader) {
-                if (nks == KB / 16) issue_steps<F::CONCAT, KB / 16>(d, q.bn, a_view, sub_lo, b_lo, id1, id2, id3, more, p);
-                else if (nks == 3) issue_steps<F::CONCAT, 3>(d, q.bn, a_view, sub_lo, b_lo, id1, id2, id3, more, p);
-                else if (nks == 2) issue_steps<F::CONCAT, 2>(d, q.bn, a_view, sub_lo, b_lo, id1, id2, id3, more, p);
-                else issue_steps<F::CONCAT, 1>(d, q.bn, a_view, sub_lo, b_lo, id1, id2, id3, more, p);
+                if (nks == KB / 16) issue_steps<F::CONCAT, KB / 16>(d, q.bn, a_view, sub_lo, b_lo, id1, id3, more, p);
+                else if (nks == 3) issue_steps<F::CONCAT, 3>(d, q.bn, a_view, sub_lo, b_lo, id1, id3, more, p);
+                else if (nks == 2) issue_steps<F::CONCAT, 2>(d, q.bn, a_view, sub_lo, b_lo, id1, id3, more, p);
+                else issue_steps<F::CONCAT, 1>(d, q.bn, a_view, sub_lo, b_lo, id1, id3, more, p);
                 umma_commit(b_empty0 + 8 * slot);
                 if (F::CONCAT || p == 2) {
                   if (last_link) umma_commit(acc_full0 + 8 * ab);
@@ -388,7 +393,6 @@ __global__ void __launch_bounds__(Form<BNMAX, PWG>::THREADS, 1) conv_f32_split_k
           if (++t == q.nsub) { t = 0; ++kb; }
         }
       }
-      (void)id2; (void)id3;
     } else if ((warp & 3) == 1) {
       // ---------------- filter copies ----------------------------------------------------------------
       const bool leader = elect_one();
@@ -465,16 +469,18 @@ __global__ void __launch_bounds__(Form<BNMAX, PWG>::THREADS, 1) conv_f32_split_k
 #pragma unroll
             for (int j = 0; j < F::CH; ++j) {
               if ((h + 2 * j) * 16 >= q.bn) break;
-              uint32_t r0[16], r1[16], r2[16];
+              uint32_t r0[16], r1[16], r2[16], r3[16];
               tmem_ld16_issue(d + 32 * j, r0);
               tmem_ld16_issue(d + 32 * j + q.bn, r1);
               tmem_ld16_issue(d + 32 * j + 2 * q.bn, r2);
+              tmem_ld16_issue(d + 32 * j + 3 * q.bn, r3);
               tmem_wait16(r0);
               tmem_wait16(r1);
               tmem_wait16(r2);
+              tmem_wait16(r3);
 #pragma unroll
               for (int e = 0; e < 16; ++e)
-                acc[j][e] += __uint_as_float(r0[e]) + (__uint_as_float(r1[e]) + __uint_as_float(r2[e]));
+                acc[j][e] += __uint_as_float(r0[e]) + (__uint_as_float(r1[e]) + (__uint_as_float(r2[e]) + __uint_as_float(r3[e])));
             }
           } else {
             constexpr int STEP = BNMAX == 256 ? 1 : 2;      // chunks in flight (128 sums leave registers for one)
@@ -576,7 +582,7 @@ __global__ void __launch_bounds__(Form<BNMAX, PWG>::THREADS, 1) conv_f32_split_k
 
 // Filter -> the images the copy warp loads: for every (channel tile nt, k2-block kb, kernel column v) the three
 // pieces [bn channels][64 k2] in the 128-byte-swizzled order of shared memory, smallest first, or largest first
-// where they form one operand (bn <= 80); and a copy of the filter as given.  One block: `rows` channels of one
+// where they form one operand (bn <= CONCAT_BN); and a copy of the filter as given.  One block: `rows` channels of one
 // k2-block; its source is one contiguous run of the OIHW filter per channel.  Channels beyond Co and k2 beyond C*Kh are
 // zeros.
 __global__ void __launch_bounds__(256) pack_f32_split_kernel(const float* __restrict__ f, unsigned char* __restrict__ fp,
@@ -617,8 +623,8 @@ __global__ void __launch_bounds__(256) pack_f32_split_kernel(const float* __rest
   }
 }
 
-int form_of(int bn) { return bn <= 80 ? 80 : (bn <= 128 ? 128 : 256); }
-int slot_bytes_of(int bn) { return (bn <= 80 ? 3 : 1) * bn * 128; }
+int form_of(int bn) { return bn <= CONCAT_BN ? CONCAT_BN : (bn <= 128 ? 128 : 256); }
+int slot_bytes_of(int bn) { return (bn <= CONCAT_BN ? 3 : 1) * bn * 128; }
 
 // Filter slots that fit beside the two S stages and the offset table.
 int slots_for(int bn, int rows, int num_kb) {
@@ -630,7 +636,7 @@ int slots_for(int bn, int rows, int num_kb) {
 // Cycles of the six products of a 128 x bn tile over 16 k (see the head of this file).
 double step_cycles(int bn) {
   auto mma = [](int n) { const double pipe = n / 2.0, smem = 32 + n / 4.0; return pipe > smem ? pipe : smem; };
-  return bn <= 80 ? mma(3 * bn) + mma(2 * bn) + mma(bn) : 6 * mma(bn);
+  return bn <= CONCAT_BN ? mma(3 * bn) + 3 * mma(bn) : 6 * mma(bn);
 }
 
 template <int BNMAX, int PWG>
@@ -686,7 +692,7 @@ F32SplitPlan plan_f32_split(const Geometry& g) {
     const int bn = ((g.Co + nt - 1) / nt + 15) / 16 * 16;
     if (nt > 1 && (int64_t)(nt - 1) * bn >= g.Co) continue;          // fewer tiles of this width do
     const int sb = slots_for(bn, p.rows, p.num_kb);
-    if (sb < (bn <= 80 ? 2 : 3)) continue;
+    if (sb < (bn <= CONCAT_BN ? 2 : 3)) continue;
     if (nt * bn > p.packed_rows) p.packed_rows = nt * bn;
     if (force_bn && bn != atoi(force_bn)) continue;
     if (ntm * nt >= ((int64_t)1 << 30)) continue;
@@ -722,7 +728,7 @@ cudaError_t launch_pack_f32_split(const float* filter, void* scratch, const Geom
   dim3 grid((unsigned)p.num_kb, (unsigned)(p.ntn * p.bn / rows));
   if (grid.y > 65535) return cudaErrorInvalidValue;
   pack_f32_split_kernel<<<grid, 256, smem, stream>>>(filter, base + kStatusBytes, reinterpret_cast<float*>(base + kStatusBytes + p.copy_off), reinterpret_cast<uint32_t*>(base), g.C * g.Kh,
-                                                     g.Kw, g.Co, p.bn, p.num_kb, rows, p.bn <= 80 ? 1 : 0);
+                                                     g.Kw, g.Co, p.bn, p.num_kb, rows, p.bn <= CONCAT_BN ? 1 : 0);
   return cudaGetLastError();
 }
 
@@ -748,7 +754,7 @@ cudaError_t launch_conv_f32_split(const float* window, float* y, void* scratch, 
   const int smem = 1024 + rings;
   if (p.split > 1 && rings < p.bn * TILE_M * 4) return cudaErrorInvalidValue;
   switch (form_of(p.bn)) {
-    case 80: return p.num_kb == 1 ? launch_form<80, 1>(q, smem, stream) : launch_form<80, 2>(q, smem, stream);
+    case CONCAT_BN: return p.num_kb == 1 ? launch_form<CONCAT_BN, 1>(q, smem, stream) : launch_form<CONCAT_BN, 2>(q, smem, stream);
     case 128: return launch_form<128, 2>(q, smem, stream);
     default: return launch_form<256, 1>(q, smem, stream);
   }

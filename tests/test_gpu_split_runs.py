@@ -98,6 +98,26 @@ def test_conv_f32_split_values_beyond_the_pieces(form, what, monkeypatch):
         assert np.linalg.norm((a - b) / scale) <= 1e-6 * np.linalg.norm(b / scale)
 
 
+@pytest.mark.parametrize("co", [16, 33, 64, 80])
+def test_conv_f32_split_starts_from_clean_accumulators(co, monkeypatch):
+    """No output depends on what tensor memory held before: with NaNs left in all of its columns on every SM, a layer of
+    many tiles gives the same bits again and again, and the oracle's values."""
+    left = L("left", 40, 8, 24, 24, 256, 3, 3, 1, 1, 211)
+    layer = L("clean", 40, 40, 24, 24, co, 3, 3, 1, 1, 212)
+    x0, f0 = workloads.make_inputs(left)
+    x, f = workloads.make_inputs(layer)
+    yr, ar = oracle.conv_direct(x.numpy(), f.numpy(), layer.dims())
+    first = None
+    for _ in range(3):
+        force_split(monkeypatch, (256, 1))
+        gpu_conv(torch.full_like(x0, float("nan")), f0, left.dims(), "f32")
+        force_split(monkeypatch, ((co + 15) // 16 * 16, 1))
+        y, _, _ = gpu_conv(x, f, layer.dims(), "f32")
+        first = y if first is None else first
+        assert np.array_equal(y, first)
+    check_conv(first, yr, ar, "f32", layer.name)
+
+
 RUNS = [l for l, _ in SPLIT] + [
     L("runs_quad", 2, 3, 19, 23, 20, 7, 7, 2, 3, 230),       # up to four channels: a unit is four channels at two columns' elements
     L("runs_quad1", 3, 2, 12, 9, 16, 1, 1, 1, 0, 231),       # ... one unit, one step
