@@ -112,11 +112,13 @@ im2win_status im2win_transform(const void* x_nchw, void* window, const im2win_sh
  * The filter is repacked into `scratch` on every call (part of the timed
  * operation).  `y_nchw` is [N][Co][Ho][Wo] fp32.  `scratch` must hold at least
  * the scratch_bytes reported by im2win_workspace_size(shape, IM2WIN_F32, ...).
- * Sums are fp32 and their order is unspecified.  Reductions of 64 terms or more run on the tensor cores:
- * every element is the exact sum of three bf16 pieces, and six products of
+ * Sums are fp32 and their order is unspecified.  Reductions of 64 terms or more run on the tensor cores
+ * (im2win_conv_kernel_name: "f32-split"; a few shapes its tiles do not hold stay on CUDA cores):
+ * every element, subnormal ones included, is the exact sum of three scaled bf16 pieces, and six products of
  * pieces stand for one fp32 product to within 2^-26 of it; the error against 64 bits is
- * below that of a chain of fp32 FMAs.  Infinities, NaNs and overflow come out as fp32 FMAs give
- * them.  Device-side waits of this kernel are bounded as in im2win_conv_f16.
+ * below that of a chain of fp32 FMAs.  Outputs of 2^82 and more, outputs that meet an element of 2^104 or more, and
+ * non-zero outputs below 2^-90 are computed with fp32 FMAs, more slowly; infinities, NaNs and overflow therefore come
+ * out as fp32 FMAs give them.  Device-side waits of this kernel are bounded as in im2win_conv_f16.
  */
 im2win_status im2win_conv_f32(const float* window, const float* filter_oihw, float* y_nchw,
                               void* scratch, size_t scratch_bytes, const im2win_shape* shape,

@@ -1,8 +1,8 @@
 // fp32 im2win convolution on the tensor cores: every fp32 operand is the exact sum of three bf16
 // pieces, and six bf16 products per term reproduce the fp32 product.
 //
-//     x = x1 + x2 + x3,  x1 = bf16(x), x2 = bf16(x - x1), x3 = x - x1 - x2        (24 = 8 + 8 + 8 bits)
-//     x w ~ x1 w1 + (x1 w2 + x2 w1) + (x1 w3 + x2 w2 + x3 w1)
+//     2^23 x = x1 + x2 + x3,  x1 = bf16(2^23 x), x2 = bf16(2^23 x - x1), x3 = 2^23 x - x1 - x2   (24 = 8 + 8 + 8 bits)
+//     2^46 x w ~ x1 w1 + (x1 w2 + x2 w1) + (x1 w3 + x2 w2 + x3 w1)
 //
 // The three products left out are below 2^-26 |x w|.  What decides the accuracy is the accumulator: the
 // tensor core aligns the addends of an instruction to the largest one, cuts them two bits below fp32's
@@ -11,9 +11,12 @@
 // accumulator, the small products first, and the epilogue warps add it to fp32 registers with rounded adds.
 // Error against 64 bits, relative 2-norm (round-to-nearest FFMA chain -> this kernel): K = 147 2.2e-7 ->
 // 0.8e-7, K = 576 4.3e-7 -> 1.0e-7, K = 4608 1.2e-6 -> 1.8e-7, on inputs of both signs and of one.
-// Values whose pieces or sums leave the finite range give a non-finite accumulator; such outputs (and
-// those below 2^-90, where pieces get lost under bf16's smallest value) are computed again with fp32 FMAs in
-// the order of the FFMA kernel, from the window and a copy of the filter (exact_output).
+// The last bit of the smallest fp32 values, 2^-149, becomes bf16's smallest normal value, 2^-126, by the scaling: no piece
+// of any operand gets lost, or is a subnormal (by whose exponent the tensor core would align its addends: scaled by
+// 2^16, weights of 2^-145 gave six times the error).  Elements of 2^104 and sums of 2^82 and more give a non-finite
+// accumulator; such outputs (and non-zero ones below 2^-90, whose products the FFMA kernel rounds to fp32's subnormals)
+// are computed again with fp32 FMAs in the order of the FFMA kernel, from the window and a copy of the filter
+// (exact_output).
 //
 // The GEMM is the shifted-view one of conv_f16_shift.cu: the window tensor's columns are staged once,
 //     S[piece][row = virtual column q][k2 = c*Kh + u]     (64 k2 = 128 bytes per row, 128-byte swizzle),
@@ -87,12 +90,28 @@ __device__ __forceinline__ uint32_t cvt_bf16x2(float lo, float hi) {
   asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
   return r;
 }
-// Two values -> their three pieces, packed (first value in the low half).
+// Two values -> the three pieces of 2^23 times them, packed (first value in the low half).
+constexpr float kScale = 8388608.f, kUnscale = 1.f / (kScale * kScale);
+__device__ __forceinline__ uint64_t pair(float lo, float hi) {
+  return (uint64_t)__float_as_uint(lo) | ((uint64_t)__float_as_uint(hi) << 32);
+}
+// a - (the two bf16 of p), exact here.
+__device__ __forceinline__ uint64_t sub_pieces(uint64_t a, uint32_t p) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r)
+      : "l"(pair(__uint_as_float(p << 16), __uint_as_float(p & 0xffff0000u))), "l"(pair(-1.f, -1.f)), "l"(a));
+  return r;
+}
+__device__ __forceinline__ uint32_t cvt_pair(uint64_t v) {
+  return cvt_bf16x2(__uint_as_float((uint32_t)v), __uint_as_float((uint32_t)(v >> 32)));
+}
 __device__ __forceinline__ void split2(float a, float b, uint32_t& p1, uint32_t& p2, uint32_t& p3) {
-  p1 = cvt_bf16x2(a, b);
-  const float ra = a - __uint_as_float(p1 << 16), rb = b - __uint_as_float(p1 & 0xffff0000u);
-  p2 = cvt_bf16x2(ra, rb);
-  p3 = cvt_bf16x2(ra - __uint_as_float(p2 << 16), rb - __uint_as_float(p2 & 0xffff0000u));
+  uint64_t v;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(v) : "l"(pair(a, b)), "l"(pair(kScale, kScale)));
+  p1 = cvt_pair(v);
+  v = sub_pieces(v, p1);
+  p2 = cvt_pair(v);
+  p3 = cvt_pair(sub_pieces(v, p2));
 }
 __device__ __forceinline__ void st_shared16(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
   asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
@@ -124,20 +143,21 @@ __host__ __device__ constexpr uint32_t instr_desc_bf16(int M, int N) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
-// An output that has to be computed again: not finite, or so small that pieces of its terms were lost.
+// An output that has to be computed again: not finite, or so small that fp32 rounds its products.
 __device__ __forceinline__ bool suspicious(float v) {
   const uint32_t u = __float_as_uint(v) << 1, lo = (uint32_t)(127 - 90) << 24;
   return u != 0u && u - lo >= 0xff000000u - lo;
 }
 
-// v[e] -> base[e * stride] for e < count, over two address chains.
+// v[e] / 2^46 -> base[e * stride] for e < count, over two address chains.
 __device__ __forceinline__ void store16(float* base, int stride, const float (&v)[16], int count, bool& again) {
   float *p0 = base, *p1 = base + stride;
   const int64_t step = 2 * (int64_t)stride;
 #pragma unroll
   for (int e = 0; e < 16; e += 2) {
-    if (e < count) { *p0 = v[e]; again |= suspicious(v[e]); }
-    if (e + 1 < count) { *p1 = v[e + 1]; again |= suspicious(v[e + 1]); }
+    const float a = v[e] * kUnscale, b = v[e + 1] * kUnscale;
+    if (e < count) { *p0 = a; again |= suspicious(a); }
+    if (e + 1 < count) { *p1 = b; again |= suspicious(b); }
     p0 += step; p1 += step;
   }
 }
@@ -552,6 +572,7 @@ __global__ void __launch_bounds__(Form<BNMAX, PWG>::THREADS, 1) conv_f32_split_k
           float sum = v[0];
 #pragma unroll
           for (int r = 1; r < 8; ++r) sum += v[r];
+          sum *= kUnscale;
           if (suspicious(sum)) sum = exact_output(q, n, ho, i0, co0 + c);
           yrow[(int64_t)c * q.HoWo] = sum;
         }

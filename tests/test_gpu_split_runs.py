@@ -118,6 +118,26 @@ def test_conv_f32_split_starts_from_clean_accumulators(co, monkeypatch):
     check_conv(first, yr, ar, "f32", layer.name)
 
 
+@pytest.mark.parametrize("form", [(64, 1), (64, 2), (112, 1), (256, 2)], ids=str)
+@pytest.mark.parametrize("xs,fs", [(-100, 30), (-112, 40), (-124, 60), (-137, 60), (-145, 100), (40, -112), (60, -137),
+                                   (100, -145), (90, -50), (80, 5), (110, -120)])
+def test_conv_f32_split_holds_operands_of_any_size(form, xs, fs, monkeypatch):
+    """Small elements on one side and large ones on the other: the outputs are of ordinary size, and as close to the
+    64-bit values as the FFMA kernel's, although the operands' low bits lie far below bf16's range."""
+    layer = L("sizes", 2, 64, 9, 12, form[0] - 5, 3, 3, 1, 1, 221)
+    dims = layer.dims()
+    x, f = workloads.make_inputs(layer)
+    x, f = (x.double() * 2.0 ** xs).float(), (f.double() * 2.0 ** fs).float()
+    yr, ar = oracle.conv_direct(x.numpy(), f.numpy(), dims)
+    force_split(monkeypatch, form)
+    y, _, _ = gpu_conv(x, f, dims, "f32")
+    check_conv(y, yr, ar, "f32", layer.name)
+    monkeypatch.setenv("IM2WIN_F32_KERNEL", "ffma")
+    z, _, _ = gpu_conv(x, f, dims, "f32")
+    scale = 1.0 / np.abs(yr).max()
+    assert np.linalg.norm((y - yr) * scale) <= np.linalg.norm((z - yr) * scale)
+
+
 RUNS = [l for l, _ in SPLIT] + [
     L("runs_quad", 2, 3, 19, 23, 20, 7, 7, 2, 3, 230),       # up to four channels: a unit is four channels at two columns' elements
     L("runs_quad1", 3, 2, 12, 9, 16, 1, 1, 1, 0, 231),       # ... one unit, one step
