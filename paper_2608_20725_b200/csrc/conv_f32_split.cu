@@ -16,7 +16,7 @@
 // 2^16, weights of 2^-145 gave six times the error).  Elements of 2^104 and sums of 2^82 and more give a non-finite
 // accumulator; such outputs (and non-zero ones below 2^-90, whose products the FFMA kernel rounds to fp32's subnormals)
 // are computed again with fp32 FMAs in the order of the FFMA kernel, from the window and a copy of the filter
-// (exact_output).
+// (exact_outputs).
 //
 // The GEMM is the shifted-view one of conv_f16_shift.cu: the window tensor's columns are staged once,
 //     S[piece][row = virtual column q][k2 = c*Kh + u]     (64 k2 = 128 bytes per row, 128-byte swizzle),
@@ -64,7 +64,7 @@ constexpr int kSplitSmem = 226 * 1024;        // dynamic shared memory a CTA may
 struct SplitParams {
   const float* __restrict__ win;
   const unsigned char* __restrict__ fp;       // packed filter: shared-memory images, see pack_f32_split_kernel
-  const float* __restrict__ f;                // the filter as given, for exact_output
+  const float* __restrict__ f;                // the filter as given, for exact_outputs
   float* __restrict__ y;
   uint32_t* status;
   int64_t img_stride, strip, chan_stride;
@@ -178,15 +178,41 @@ template <int BNMAX, int PWG_> struct Form {
   // (the launch holds 128 or 96 registers a thread: 96 + 64 + 2*176 = 4*128, 2*96 + 64 + 2*112 = 5*96)
 };
 
-// One output in fp32 FMAs, k ascending, for the values the split cannot hold.
-__device__ __forceinline__ float exact_output(const SplitParams& q, uint32_t n, int ho, int wo, int co) {
-  const float* x = q.win + (int64_t)n * q.img_stride + (int64_t)ho * q.strip + (int64_t)wo * q.s * q.Kh;
-  const float* f = q.f + (int64_t)co * q.K2 * q.Kw;
-  float acc = 0.f;
-  for (int c = 0; c < q.C; ++c, x += q.chan_stride, f += q.Kh * q.Kw)
-    for (int v = 0; v < q.Kw; ++v)
-      for (int u = 0; u < q.Kh; ++u) acc = fmaf(x[v * q.Kh + u], f[u * q.Kw + v], acc);
-  return acc;
+// The suspicious ones among the outputs y[i * ystride], i < count <= 16, of the window at x and the filters f + i * fstep:
+// computed again in fp32 FMAs, k ascending.  Sixteen sums at a time share the loads of the window and keep the loads of
+// the filter (the same address in every lane) in flight; they end early once all are NaN, as in a tensor full of them.
+__device__ __noinline__ void exact_outputs(const float* __restrict__ x, const float* __restrict__ f, float* y, int64_t chan_stride,
+                                           int64_t fstep, int64_t ystride, int C, int Kh, int Kw, int count) {
+  bool any = false;
+  for (int i = 0; i < count; ++i) any |= suspicious(y[i * ystride]);
+  if (!any) return;
+  float acc[16];
+#pragma unroll
+  for (int i = 0; i < 16; ++i) acc[i] = 0.f;
+  bool open = true;
+#pragma unroll 1
+  for (int c = 0; c < C && open; ++c, x += chan_stride, f += Kh * Kw) {
+#pragma unroll 1
+    for (int v = 0; v < Kw; ++v)
+#pragma unroll 1
+      for (int u = 0; u < Kh; ++u) {
+        const float xv = x[v * Kh + u];
+        const float* fk = f + u * Kw + v;
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+          acc[i] = fmaf(xv, *fk, acc[i]);
+          if (i + 1 < count) fk += fstep;
+        }
+      }
+    open = false;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) open |= acc[i] == acc[i];
+  }
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    float* p = y + i * ystride;
+    if (i < count && suspicious(*p)) *p = acc[i];
+  }
 }
 
 // The instructions of one filter operand of a unit, straight-line: a lone lane pays for every branch and address
@@ -526,7 +552,19 @@ __global__ void __launch_bounds__(Form<BNMAX, PWG>::THREADS, 1) conv_f32_split_k
         if (++t == q.nsub) { t = 0; ++kb; }
       }
       if (!ok) break;
-      if (q.split > 1) break;
+      if (q.split > 1) {
+        // All MMAs of this CTA have completed, so its rings are free: partial sums as P[channel][row], 4 bytes.
+        // (here and not behind the loop, where the sums would have to be live over everything below)
+        float* part = reinterpret_cast<float*>(smem);
+#pragma unroll
+        for (int j = 0; j < F::CH; ++j)
+#pragma unroll
+          for (int e = 0; e < 16; ++e) {
+            const int c = (h + 2 * j) * 16 + e;
+            if (c < q.bn) part[c * TILE_M + lq * 32 + lane] = acc[j][e];
+          }
+        break;
+      }
       if (valid) {
         const int co0 = nt * q.bn;
         float* yrow = q.y + ((int64_t)n * q.Co + co0) * q.HoWo + (int64_t)ho * q.Wo + i0;
@@ -538,23 +576,15 @@ __global__ void __launch_bounds__(Form<BNMAX, PWG>::THREADS, 1) conv_f32_split_k
           store16(yrow + (int64_t)c0 * q.HoWo, q.HoWo, acc[j], limit - c0, again);
         }
         if (again) {
-          for (int c = h * 16; c < limit; c += (c & 15) == 15 ? 17 : 1)
-            if (suspicious(yrow[(int64_t)c * q.HoWo])) yrow[(int64_t)c * q.HoWo] = exact_output(q, n, ho, i0, co0 + c);
+          const float* x = q.win + (int64_t)n * q.img_stride + (int64_t)ho * q.strip + (int64_t)i0 * q.s * q.Kh;
+          const int64_t K = (int64_t)q.K2 * q.Kw;
+          for (int c = h * 16; c < limit; c += 32)
+            exact_outputs(x, q.f + (co0 + c) * K, yrow + (int64_t)c * q.HoWo, q.chan_stride, K, q.HoWo, q.C, q.Kh, q.Kw,
+                          limit - c < 16 ? limit - c : 16);
         }
       }
     }
     if (q.split > 1) {
-      // All MMAs of this CTA have completed, so its rings are free: partial sums as P[channel][row], 4 bytes.
-      if (ok) {
-        float* part = reinterpret_cast<float*>(smem);
-#pragma unroll
-        for (int j = 0; j < F::CH; ++j)
-#pragma unroll
-          for (int e = 0; e < 16; ++e) {
-            const int c = (h + 2 * j) * 16 + e;
-            if (c < q.bn) part[c * TILE_M + lq * 32 + lane] = acc[j][e];
-          }
-      }
       __syncwarp();
       cluster_sync_all();
       if (ok && valid) {
@@ -565,7 +595,9 @@ __global__ void __launch_bounds__(Form<BNMAX, PWG>::THREADS, 1) conv_f32_split_k
         uint32_t peer[8];
 #pragma unroll
         for (int r = 0; r < 8; ++r) peer[r] = mapa_shared(a_ring + (lq * 32 + lane) * 4, r < q.split ? r : 0);
-        for (int c = rank * per + h; c < (rank + 1) * per && c < limit; c += 2) {
+        const int c_end = (rank + 1) * per < limit ? (rank + 1) * per : limit;
+        bool again = false;
+        for (int c = rank * per + h; c < c_end; c += 2) {
           float v[8];
 #pragma unroll
           for (int r = 0; r < 8; ++r) v[r] = r < q.split ? ld_cluster(peer[r] + c * (TILE_M * 4)) : 0.f;
@@ -573,8 +605,17 @@ __global__ void __launch_bounds__(Form<BNMAX, PWG>::THREADS, 1) conv_f32_split_k
 #pragma unroll
           for (int r = 1; r < 8; ++r) sum += v[r];
           sum *= kUnscale;
-          if (suspicious(sum)) sum = exact_output(q, n, ho, i0, co0 + c);
+          again |= suspicious(sum);
           yrow[(int64_t)c * q.HoWo] = sum;
+        }
+        if (again) {
+          const float* x = q.win + (int64_t)n * q.img_stride + (int64_t)ho * q.strip + (int64_t)i0 * q.s * q.Kh;
+          const int64_t K = (int64_t)q.K2 * q.Kw;
+          for (int c = rank * per + h; c < c_end; c += 32) {
+            const int left = (c_end - c + 1) / 2;
+            exact_outputs(x, q.f + (co0 + c) * K, yrow + (int64_t)c * q.HoWo, q.chan_stride, 2 * K, 2 * (int64_t)q.HoWo, q.C,
+                          q.Kh, q.Kw, left < 16 ? left : 16);
+          }
         }
       }
       __syncwarp();

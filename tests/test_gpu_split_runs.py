@@ -138,6 +138,40 @@ def test_conv_f32_split_holds_operands_of_any_size(form, xs, fs, monkeypatch):
     assert np.linalg.norm((y - yr) * scale) <= np.linalg.norm((z - yr) * scale)
 
 
+def device_seconds(call):
+    start, stop = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    call()
+    start.record()
+    call()
+    stop.record()
+    stop.synchronize()
+    return start.elapsed_time(stop) / 1e3
+
+
+@pytest.mark.parametrize("what", ["nan", "inf", "tiny"])
+def test_conv_f32_split_recomputes_whole_tensors_in_bounded_time(what, monkeypatch):
+    """Every output of a long reduction computed again: the same values as the FFMA kernel, well inside the time after
+    which a device-side wait gives up (4 s), although one CTA has the whole tile.  Measured below 0.005 s (nan, inf) and 0.1 s
+    (tiny); one output at a time took 0.9 s by the count of its dependent steps."""
+    layer = L("long", 8, 96, 16, 40, 256, 16, 17, 1, 0, 222)
+    dims = layer.dims()
+    force_split(monkeypatch, (256, 1))
+    x, f = workloads.make_inputs(layer)
+    x, f = {"nan": (torch.full_like(x, float("nan")), f), "inf": (torch.full_like(x, float("inf")), f),
+            "tiny": (x * 1e-30, f * 1e-10)}[what]
+    window, scratch, y = binding.alloc_layer_buffers(dims, torch.float32)
+    xd, fd = x.cuda(), f.cuda()
+    binding.im2win_transform(xd, window, dims)
+    binding.im2win_pack_filter(fd, scratch, dims)
+    seconds = device_seconds(lambda: binding.im2win_conv_packed(window, y, scratch, dims))
+    binding.im2win_check_status(scratch)
+    monkeypatch.setenv("IM2WIN_F32_KERNEL", "ffma")
+    z, _, _ = gpu_conv(x, f, dims, "f32")
+    y = y.cpu().numpy()
+    assert ((y == z) | (np.isnan(y) & np.isnan(z))).all()
+    assert seconds < 0.25
+
+
 RUNS = [l for l, _ in SPLIT] + [
     L("runs_quad", 2, 3, 19, 23, 20, 7, 7, 2, 3, 230),       # up to four channels: a unit is four channels at two columns' elements
     L("runs_quad1", 3, 2, 12, 9, 16, 1, 1, 1, 0, 231),       # ... one unit, one step
