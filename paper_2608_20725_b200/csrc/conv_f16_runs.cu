@@ -69,6 +69,7 @@ struct RunsParams {
   int32_t C, N, Wp, Wq, pitch, Ho, Wo, HoWo, Co, Kh, Kw, s;
   int32_t E, G, units, num_kb, nks_last;      // units: of eight k2
   int32_t quad;                               // 1: up to four channels, a unit is four channels at two e
+  int32_t foreign;                            // 1: zero filter elements meet elements that are not of the window
   int32_t rows, halo, region, octs, raw_slot, a_stage;
   int32_t bn, ntn, nwork, sa, sr, sb, slot_bytes, resident;
 };
@@ -113,22 +114,47 @@ __device__ __forceinline__ TileRuns tile_runs(const RunsParams& q, uint32_t q0) 
   return r;
 }
 
-// One output in fp32 FMAs, k ascending, for outputs that came out infinite or NaN: a column outside the window, which
-// meets zeros of the widened filter, may hold the infinity or NaN.
-__device__ __forceinline__ float exact_output(const RunsParams& q, uint32_t n, int ho, int wo, int nt, int col) {
-  const unsigned char* wbase = q.win + (int64_t)n * q.img_bytes + ((int64_t)ho * q.Wp + (int64_t)wo * q.s) * q.Kh * ES;
-  const unsigned char* frow = q.fp + (int64_t)nt * q.num_kb * q.G * q.slot_bytes + col * 128;
-  float acc = 0.f;
-  for (int c = 0; c < q.C; ++c)
-    for (int v = 0; v < q.Kw; ++v)
-      for (int u = 0; u < q.Kh; ++u) {
-        const int g = v / q.s, e = (v - g * q.s) * q.Kh + u;
-        const int j = q.quad ? e >> 1 : (c >> 3) * q.E + e, at = q.quad ? (e & 1) * 4 + c : c & 7;      // unit, place in it
-        const unsigned char* f = frow + ((int64_t)(j >> 3) * q.G + g) * q.slot_bytes + ((((j & 7) ^ (col & 7)) << 4) | (at * 2));
-        const unsigned char* x = wbase + c * q.chan_bytes + (v * q.Kh + u) * ES;
-        acc = fmaf(__half2float(*reinterpret_cast<const __half*>(x)), __half2float(*reinterpret_cast<const __half*>(f)), acc);
+// The outputs y[i * ystride], i < count <= 16, that came out infinite or NaN although a zero filter element may have met an
+// infinity or NaN from outside their window (RunsParams::foreign): in fp32 FMAs, k ascending, from the window at x and
+// rows i of the filter image at f.  Sixteen sums at a time keep the loads of the filter (the same address in every lane) in
+// flight; they end early once all are NaN.  (A function of its own: expanded beside the epilogue it costs spills.)
+__device__ __noinline__ void exact_outputs(const unsigned char* __restrict__ x, const unsigned char* __restrict__ f, float* y,
+                                           int64_t ystride, int64_t chan_bytes, int C, int Kh, int Kw, int s, int E, int g_step,
+                                           int j_step, int quad, int count) {
+  auto not_finite = [](float v) { return !(fabsf(v) <= 3.4028234663852886e38f); };
+  bool any = false;
+  for (int i = 0; i < count; ++i) any |= not_finite(y[i * ystride]);
+  if (!any) return;
+  float acc[16];
+#pragma unroll
+  for (int i = 0; i < 16; ++i) acc[i] = 0.f;
+  bool open = true;
+#pragma unroll 1
+  for (int c = 0; c < C && open; ++c, x += chan_bytes) {
+    int g = 0, t = 0;                                      // kernel column v = g * s + t
+#pragma unroll 1
+    for (int v = 0; v < Kw; ++v) {
+#pragma unroll 1
+      for (int u = 0; u < Kh; ++u) {
+        const int e = t * Kh + u;
+        const int j = quad ? e >> 1 : (c >> 3) * E + e, at = quad ? (e & 1) * 4 + c : c & 7;      // unit, place in it
+        const unsigned char* fj = f + (int64_t)(j >> 3) * j_step + (int64_t)g * g_step + at * ES;
+        const float xv = __half2float(*reinterpret_cast<const __half*>(x + (v * Kh + u) * ES));
+#pragma unroll
+        for (int i = 0; i < 16; ++i)                       // (rows up to the next multiple of 16 exist)
+          acc[i] = fmaf(xv, __half2float(*reinterpret_cast<const __half*>(fj + i * 128 + (((j & 7) ^ (i & 7)) << 4))), acc[i]);
       }
-  return acc;
+      if (++t == s) { t = 0; ++g; }
+    }
+    open = false;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) open |= acc[i] == acc[i];
+  }
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    float* p = y + i * ystride;
+    if (i < count && not_finite(*p)) *p = acc[i];
+  }
 }
 
 // The MMAs of one kernel column, straight-line: a lone lane pays for every branch and address computation between them.
@@ -440,13 +466,16 @@ __global__ void __launch_bounds__(THREADS, 1) conv_f16_runs_kernel(RunsParams q)
         if (valid) {
           store_strided32(yrow + (int64_t)c0 * q.HoWo, q.HoWo, v, limit - c0);
           float zero = 0.f;
+          if (q.foreign) {
 #pragma unroll
-          for (int j = 0; j < 32; ++j) zero = fmaf(__uint_as_float(c0 + j < limit ? v[j] : 0u), 0.f, zero);
+            for (int j = 0; j < 32; ++j) zero = fmaf(__uint_as_float(c0 + j < limit ? v[j] : 0u), 0.f, zero);
+          }
           if (zero != 0.f) {                               // (a NaN: one of them is not finite)
-            for (int c = c0; c < c0 + 32 && c < limit; ++c) {
-              float* p = yrow + (int64_t)c * q.HoWo;
-              if (!(fabsf(*p) <= 3.4028234663852886e38f)) *p = exact_output(q, n, ho, i0, nt, c);
-            }
+            const unsigned char* x = q.win + (int64_t)n * q.img_bytes + ((int64_t)ho * q.Wp + (int64_t)i0 * q.s) * q.Kh * ES;
+            const unsigned char* f = q.fp + (int64_t)nt * q.num_kb * q.G * q.slot_bytes;
+            for (int c = c0; c < c0 + 32 && c < limit; c += 16)
+              exact_outputs(x, f + c * 128, yrow + (int64_t)c * q.HoWo, q.HoWo, q.chan_bytes, q.C, q.Kh, q.Kw, q.s, q.E,
+                            q.slot_bytes, q.G * q.slot_bytes, q.quad, limit - c < 16 ? limit - c : 16);
           }
         }
       }
@@ -631,6 +660,8 @@ cudaError_t launch_conv_f16_runs(const uint16_t* window, float* y, void* scratch
   q.div_ho = fast_div((uint32_t)g.Ho);
   q.C = g.C; q.N = g.N; q.Wp = g.Wp; q.Wq = p.Wq; q.pitch = p.pitch; q.Ho = g.Ho; q.Wo = g.Wo; q.HoWo = g.Ho * g.Wo;
   q.Co = g.Co; q.Kh = g.Kh; q.Kw = g.Kw; q.s = g.s;
+  // kernel columns beyond Kw, channels beyond C in the last octet, the element beyond an odd E
+  q.foreign = (g.Kw > g.s && g.Kw % g.s != 0) || (p.quad ? p.E % 2 != 0 : g.C % 8 != 0);
   q.E = p.E; q.G = p.G; q.units = p.units; q.quad = p.quad ? 1 : 0; q.num_kb = p.num_kb; q.nks_last = p.nks_last;
   q.rows = p.rows; q.halo = p.halo; q.region = p.region; q.octs = p.octs; q.raw_slot = p.raw_slot; q.a_stage = p.a_stage;
   q.bn = p.bn; q.ntn = p.ntn; q.nwork = p.nwork; q.sa = p.sa; q.sr = p.sr; q.sb = p.sb;

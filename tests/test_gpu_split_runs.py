@@ -151,8 +151,8 @@ def device_seconds(call):
 @pytest.mark.parametrize("what", ["nan", "inf", "tiny"])
 def test_conv_f32_split_recomputes_whole_tensors_in_bounded_time(what, monkeypatch):
     """Every output of a long reduction computed again: the same values as the FFMA kernel, well inside the time after
-    which a device-side wait gives up (4 s), although one CTA has the whole tile.  Measured below 0.005 s (nan, inf) and 0.1 s
-    (tiny); one output at a time took 0.9 s by the count of its dependent steps."""
+    which a device-side wait gives up (4 s), although one CTA has the whole tile.  (One output at a time: 128 x 26112
+    dependent steps of some 500 cycles, 0.9 s.)"""
     layer = L("long", 8, 96, 16, 40, 256, 16, 17, 1, 0, 222)
     dims = layer.dims()
     force_split(monkeypatch, (256, 1))
@@ -206,3 +206,33 @@ def test_conv_f16_runs(layer, monkeypatch):
     odd = ~np.isfinite(z)
     assert np.array_equal(np.isfinite(y), ~odd) and np.array_equal(np.isnan(y), np.isnan(z))
     assert np.array_equal(np.sign(y[np.isinf(z)]), np.sign(z[np.isinf(z)]))
+
+
+@pytest.mark.parametrize("layer", [L("down", 4, 256, 28, 28, 512, 3, 3, 2, 1, 240),       # columns beyond the kernel's width
+                                   L("c27", 4, 128, 27, 27, 128, 3, 3, 1, 1, 241),        # nothing foreign meets a zero
+                                   L("c9", 4, 129, 27, 27, 128, 3, 3, 1, 1, 242)],        # channels beyond the last
+                         ids=lambda l: l.name)
+@pytest.mark.parametrize("what", ["nan", "inf", "one nan"])
+def test_conv_f16_runs_not_finite_tensors_in_bounded_time(layer, what, monkeypatch):
+    """Tensors full of NaNs or infinities, and one NaN in a plain tensor: the classes the gather kernel gives.  A plain pass
+    takes 0.1 ms and less; one output at a time took 39 ms for a single NaN."""
+    dims = layer.dims()
+    monkeypatch.setenv("IM2WIN_F16_KERNEL", "runs")
+    assert binding.im2win_conv_kernel_name(dims, binding.F16) == "f16-runs"
+    x, f = workloads.make_inputs(layer)
+    if what == "one nan":
+        x = x.clone()
+        x[1, 3, 14, 13] = float("nan")
+    else:
+        x = torch.full_like(x, float(what))
+    window, scratch, y = binding.alloc_layer_buffers(dims, torch.float16)
+    xd, fd = x.half().cuda(), f.half().cuda()
+    binding.im2win_transform(xd, window, dims)
+    binding.im2win_pack_filter(fd, scratch, dims)
+    seconds = device_seconds(lambda: binding.im2win_conv_packed(window, y, scratch, dims))
+    binding.im2win_check_status(scratch)
+    z, _, _ = gpu_conv(x, f, dims, "f16-gather")
+    y = y.cpu().numpy()
+    assert np.array_equal(np.isnan(y), np.isnan(z)) and np.array_equal(np.isinf(y), np.isinf(z))
+    assert np.array_equal(np.sign(y[np.isinf(z)]), np.sign(z[np.isinf(z)]))
+    assert seconds < 5e-3
