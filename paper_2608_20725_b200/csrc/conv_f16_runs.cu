@@ -508,7 +508,7 @@ __global__ void __launch_bounds__(256) pack_f16_runs_kernel(const uint16_t* __re
                                                         int Co, int bn, int num_kb, int rows, int pitch, int quad) {
   extern __shared__ uint16_t pack_h[];
   if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < kStatusBytes / 4) status[threadIdx.x] = 0u;
-  const int kb = blockIdx.x, row0 = blockIdx.y * rows;
+  const int kb = blockIdx.y, row0 = blockIdx.x * rows;     // (channel blocks along x: any number of channels)
   const int c0 = quad ? 0 : kb * 8 / E * 8;
   int c1 = quad ? C - 1 : (kb * 8 + 7) / E * 8 + 7;
   if (c1 > C - 1) c1 = C - 1;
@@ -638,8 +638,7 @@ cudaError_t launch_pack_f16_runs(const uint16_t* filter, void* scratch, const Ge
   int rows = 8;                                             // channels per block: staging within 40 KB
   while (rows > 1 && rows * pitch * ES > 40 * 1024) rows /= 2;
   const size_t smem = (size_t)(rows * pitch * ES);
-  dim3 grid((unsigned)p.num_kb, (unsigned)(p.ntn * p.bn / rows));
-  if (grid.y > 65535) return cudaErrorInvalidValue;
+  dim3 grid((unsigned)(p.ntn * p.bn / rows), (unsigned)p.num_kb);   // (num_kb <= 2^14: C * E <= 2^20)
   pack_f16_runs_kernel<<<grid, 256, smem, stream>>>(filter, base + kStatusBytes, reinterpret_cast<uint32_t*>(base), g.C, g.Kh, g.Kw,
                                                     g.s, p.E, p.G, g.Co, p.bn, p.num_kb, rows, (int)pitch, p.quad);
   return cudaGetLastError();

@@ -652,7 +652,7 @@ __global__ void __launch_bounds__(256) pack_f32_split_kernel(const float* __rest
                                                              int num_kb, int rows, int concat) {
   extern __shared__ float pack_f[];
   if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < kStatusBytes / 4) status[threadIdx.x] = 0u;
-  const int kb = blockIdx.x, row0 = blockIdx.y * rows;
+  const int kb = blockIdx.y, row0 = blockIdx.x * rows;     // (channel blocks along x: any number of channels)
   const int nreal = K2 - kb * KB < KB ? K2 - kb * KB : KB;
   const int run = nreal * Kw, pitch = KB * Kw;
   for (int r = 0; r < rows; ++r) {
@@ -787,8 +787,7 @@ cudaError_t launch_pack_f32_split(const float* filter, void* scratch, const Geom
   int rows = 8;                                             // channels per block: staging within 40 KB
   while (rows > 1 && (size_t)rows * KB * g.Kw * 4 > 40 * 1024) rows /= 2;
   const size_t smem = (size_t)rows * KB * g.Kw * 4;
-  dim3 grid((unsigned)p.num_kb, (unsigned)(p.ntn * p.bn / rows));
-  if (grid.y > 65535) return cudaErrorInvalidValue;
+  dim3 grid((unsigned)(p.ntn * p.bn / rows), (unsigned)p.num_kb);
   pack_f32_split_kernel<<<grid, 256, smem, stream>>>(filter, base + kStatusBytes, reinterpret_cast<float*>(base + kStatusBytes + p.copy_off), reinterpret_cast<uint32_t*>(base), g.C * g.Kh,
                                                      g.Kw, g.Co, p.bn, p.num_kb, rows, p.bn <= CONCAT_BN ? 1 : 0);
   return cudaGetLastError();

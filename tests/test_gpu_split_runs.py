@@ -172,6 +172,22 @@ def test_conv_f32_split_recomputes_whole_tensors_in_bounded_time(what, monkeypat
     assert seconds < 0.25
 
 
+@pytest.mark.parametrize("precision,layer", [("f32", L("co524289", 1, 64, 4, 4, 524289, 1, 1, 1, 0, 250)),
+                                             ("f16", L("co524289", 1, 3, 9, 9, 524289, 3, 3, 2, 1, 251))], ids=["f32", "f16"])
+def test_filter_pack_takes_any_number_of_channels(precision, layer, monkeypatch):
+    """More channel blocks than the second axis of a grid has (65535)."""
+    monkeypatch.setenv("IM2WIN_F16_KERNEL", "runs")
+    dims = layer.dims()
+    code = binding.F32 if precision == "f32" else binding.F16
+    assert binding.im2win_conv_kernel_name(dims, code) == ("f32-split" if precision == "f32" else "f16-runs")
+    x, f = workloads.make_inputs(layer)
+    y, _, _ = gpu_conv(x, f, dims, precision)
+    for part in (slice(0, 40), slice(layer.Co - 40, layer.Co)):
+        xo, fo = oracle_inputs(x, f[part], precision)
+        yr, ar = oracle.conv_direct(xo, fo, dict(dims, Co=40))
+        check_conv(y[:, part], yr, ar, precision, layer.name)
+
+
 RUNS = [l for l, _ in SPLIT] + [
     L("runs_quad", 2, 3, 19, 23, 20, 7, 7, 2, 3, 230),       # up to four channels: a unit is four channels at two columns' elements
     L("runs_quad1", 3, 2, 12, 9, 16, 1, 1, 1, 0, 231),       # ... one unit, one step
