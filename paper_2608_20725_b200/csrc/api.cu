@@ -4,6 +4,7 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <algorithm>
 #include <mutex>
 
 #include "common.cuh"
@@ -66,6 +67,23 @@ static bool want_f32_split(const Geometry& g) {
   return g.K >= 64;
 }
 
+// The same layer with another batch.
+static Geometry with_batch(Geometry g, int32_t N) {
+  g.N = N;
+  g.P = (int64_t)N * g.Ho * g.Wo;
+  g.window_elems = (int64_t)N * g.img_stride;
+  g.out_elems = (int64_t)N * g.Co * g.Ho * g.Wo;
+  return g;
+}
+
+// What a kernel wants in scratch does not depend on the batch; whether it takes the layer does, and a kernel that takes a
+// batch takes every smaller one.  So the plan for one image sizes the scratch, which then serves each part of a batch
+// whichever kernel that part goes to.  `plan` is the plan for the whole batch (half the plans walk over many tiles).
+template <typename Plan>
+static Plan plan_for_any_batch(const Plan& plan, Plan (*make)(const Geometry&), const Geometry& g) {
+  return plan.eligible || g.N == 1 ? plan : make(with_batch(g, 1));
+}
+
 im2win_status scratch_layout(const Geometry& g, im2win_dtype dtype, ScratchLayout* l) {
   if (dtype == IM2WIN_F32) {
     l->Kp = round_up(g.K, plan_f32(g).bk);
@@ -86,25 +104,27 @@ im2win_status scratch_layout(const Geometry& g, im2win_dtype dtype, ScratchLayou
   l->filter_off = (size_t)round_up((int64_t)l->koff_off + 4 * l->Kp, 256);
   int64_t fbytes = l->Kp * l->Co_pad * (dtype == IM2WIN_F32 ? 4 : 2);
   l->total = (size_t)round_up((int64_t)l->filter_off + fbytes, 256);
+  int64_t most = (int64_t)l->total;                        // of all layouts, whichever kernel is picked or forced
   if (dtype == IM2WIN_F32) {
     const F32SplitPlan split = plan_f32_split(g);
     l->f32_split = split.eligible && want_f32_split(g);
-    // (the scratch size covers both kernels and does not depend on N)
-    const int64_t wide = round_up((int64_t)kStatusBytes + 4 * round_up(g.K, 32), 256) + round_up(g.K, 32) * l->Co_pad * 4;
-    int64_t most = round_up(wide, 256);
-    if (split.eligible && kStatusBytes + (int64_t)split.filter_bytes > most) most = kStatusBytes + (int64_t)split.filter_bytes;
     l->ffma_total = l->total;
-    l->total = (size_t)round_up(most, 256);
+    const int64_t Kp = round_up(g.K, 32);                  // (the widest k-block of the FFMA kernel)
+    most = round_up((int64_t)kStatusBytes + 4 * Kp, 256) + Kp * l->Co_pad * 4;
+    const F32SplitPlan any = plan_for_any_batch(split, plan_f32_split, g);
+    if (any.eligible) most = std::max(most, kStatusBytes + (int64_t)any.filter_bytes);
   }
   if (dtype == IM2WIN_F16) {
     // The shifted-view kernel is used whenever the layer is eligible; IM2WIN_F16_KERNEL=gather
-    // forces the general gather kernel (a testing aid).  The scratch size covers both layouts.
+    // forces the general gather kernel (a testing aid).
     const ShiftPlan plan = plan_f16_shift(g);
-    const bool stem_ok = plan_f16_stem(g).eligible;       // shares the filter layout of the shifted-view kernel
+    const StemPlan stem = plan_f16_stem(g);
+    const bool stem_ok = stem.eligible;                   // shares the filter layout of the shifted-view kernel
+    const int64_t K2p = round_up((int64_t)g.C * g.Kh, kF16KBlock);
+    const size_t shift_filter_off = (size_t)round_up((int64_t)kStatusBytes + 4 * K2p, 256);
+    if (plan_for_any_batch(plan, plan_f16_shift, g).eligible || plan_for_any_batch(stem, plan_f16_stem, g).eligible)
+      most = std::max(most, (int64_t)shift_filter_off + K2p * g.Co * g.Kw * 2);
     if (plan.eligible || stem_ok) {
-      const int64_t K2p = round_up((int64_t)g.C * g.Kh, kF16KBlock);
-      const size_t shift_filter_off = (size_t)round_up((int64_t)kStatusBytes + 4 * K2p, 256);
-      const size_t shift_total = (size_t)round_up((int64_t)shift_filter_off + K2p * g.Co * g.Kw * 2, 256);
       const char* force = debug_getenv("IM2WIN_F16_KERNEL");
       const bool use_shift = !(force && strcmp(force, "gather") == 0);
       if (use_shift) {
@@ -116,20 +136,16 @@ im2win_status scratch_layout(const Geometry& g, im2win_dtype dtype, ScratchLayou
         // layers with one k-block: their own kernel unless another one is forced
         l->f16_stem = stem_ok && (!force || strcmp(force, "stem") == 0);
       }
-      if (shift_total > l->total) l->total = shift_total;
     }
-    const MatPlan mat = plan_f16_mat(g);
+    const MatPlan mat = plan_f16_mat(g);                   // (takes its own scratch layout)
     const char* force = debug_getenv("IM2WIN_F16_KERNEL");
     // measured: the matrix-transpose kernel wins for strided layers (the others stage such layers
     // with 2-byte gathers) and for kernels up to 5 wide with 128 output channels or more (CTA pairs
     // above 128); IM2WIN_F16_KERNEL=mat forces it wherever it can run (a testing aid)
     const bool want = force ? strcmp(force, "mat") == 0 : (g.s > 1 || (g.Co >= 128 && g.Kw <= 5));
-    // (the scratch size covers every layout, whichever kernel is picked or forced)
-    if (mat.eligible) {
-      l->f16_mat = want && !l->f16_stem;
-      const size_t mat_total = (size_t)round_up((int64_t)mat.scratch_bytes, 256);
-      if (mat_total > l->total) l->total = mat_total;
-    }
+    l->f16_mat = mat.eligible && want && !l->f16_stem;
+    const MatPlan any_mat = plan_for_any_batch(mat, plan_f16_mat, g);
+    if (any_mat.eligible) most = std::max(most, (int64_t)any_mat.scratch_bytes);
     // Layers that neither the one-k-block kernel nor a tiled-copy kernel takes: kernels up to three virtual columns
     // (Kw <= 3 s) go to the run-staged kernel where they are strided or have more than 64 output channels, and so does
     // what the shifted-view kernel cannot stage.  Measured against the latter: 3x3 with stride 2 1.1 to 1.8 times faster
@@ -139,10 +155,11 @@ im2win_status scratch_layout(const Geometry& g, im2win_dtype dtype, ScratchLayou
     if (runs.eligible) {
       const bool rest = !l->f16_stem && !l->f16_mat && !l->f16_raw;
       l->f16_runs = force ? strcmp(force, "runs") == 0 : rest && (!l->f16_shift || (runs.G <= 3 && (g.s > 1 || g.Co > 64)));
-      const size_t runs_total = (size_t)round_up(kStatusBytes + (int64_t)runs.filter_bytes, 256);
-      if (runs_total > l->total) l->total = runs_total;
     }
+    const RunsPlan any_runs = plan_for_any_batch(runs, plan_f16_runs, g);
+    if (any_runs.eligible) most = std::max(most, kStatusBytes + (int64_t)any_runs.filter_bytes);
   }
+  l->total = (size_t)round_up(most, 256);
   return IM2WIN_OK;
 }
 

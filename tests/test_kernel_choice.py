@@ -17,6 +17,19 @@ def test_scratch_serves_smaller_batches(layer, dtype):
         assert binding.im2win_workspace_size(binding.make_shape(n, *layer[1:]), dtype)[1] <= whole
 
 
+# (image, kernel) of layers that a kernel no longer takes at the whole batch (2^31 virtual positions, boxes of a tile) but
+# takes at a part of it
+PARTS = [(8273, 2, 512, 512, 64, 6, 6, 1, 0), (16000, 1, 512, 512, 16, 1, 1, 1, 0), (8, 8, 13, 28, 1, 7, 3, 2, 0),
+         (7, 37, 13, 44, 96, 1, 17, 3, 2), (32, 2, 34, 8, 1, 5, 5, 3, 2)]
+
+
+@pytest.mark.parametrize("layer", PARTS, ids=str)
+@pytest.mark.parametrize("dtype", [binding.F32, binding.F16])
+def test_scratch_does_not_depend_on_the_batch(layer, dtype):
+    size = lambda n: binding.im2win_workspace_size(binding.make_shape(n, *layer[1:]), dtype)[1]
+    assert {size(n) for n in (1, 2, 3, layer[0] // 4, layer[0] // 2, layer[0] - 1)} == {size(layer[0])}
+
+
 @pytest.mark.parametrize("C,K,want", [(3, 3, "f32-ffma"), (63, 1, "f32-ffma"), (64, 1, "f32-split"), (8, 3, "f32-split"),
                                       (600, 11, "f32-ffma")])       # 27, 63, 64, 72 terms; an offset table too long
 def test_f32_kernel_by_length_of_the_reduction(C, K, want):
