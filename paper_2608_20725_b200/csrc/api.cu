@@ -54,6 +54,7 @@ im2win_status derive_geometry(const im2win_shape* s, Geometry* g) {
   if ((int64_t)s->Co * g->K >= lim * 16) return IM2WIN_ERR_UNSUPPORTED;
   g->window_elems = (int64_t)s->N * g->img_stride;
   g->out_elems = (int64_t)s->N * s->Co * g->Ho * g->Wo;
+  g->plan_N = s->N;
   return IM2WIN_OK;
 }
 
@@ -73,6 +74,7 @@ static Geometry with_batch(Geometry g, int32_t N) {
   g.P = (int64_t)N * g.Ho * g.Wo;
   g.window_elems = (int64_t)N * g.img_stride;
   g.out_elems = (int64_t)N * g.Co * g.Ho * g.Wo;
+  g.plan_N = N;
   return g;
 }
 
@@ -84,10 +86,12 @@ static Plan plan_for_any_batch(const Plan& plan, Plan (*make)(const Geometry&), 
   return plan.eligible || g.N == 1 ? plan : make(with_batch(g, 1));
 }
 
-im2win_status scratch_layout(const Geometry& g, im2win_dtype dtype, ScratchLayout* l) {
+// (The FFMA kernel's k-block is that of the images it runs on: its sums have one order in every form.)
+im2win_status scratch_layout(const Geometry& part, im2win_dtype dtype, ScratchLayout* l) {
+  const Geometry g = part.plan_N == part.N ? part : with_batch(part, part.plan_N);
   if (dtype == IM2WIN_F32) {
-    l->Kp = round_up(g.K, plan_f32(g).bk);
-    l->Co_pad = round_up(g.Co, plan_f32(g).bn);
+    l->Kp = round_up(g.K, plan_f32(part).bk);
+    l->Co_pad = round_up(g.Co, plan_f32(part).bn);
   } else if (dtype == IM2WIN_F16) {
     l->Kp = round_up(g.K, kF16KBlock);
     l->Co_pad = g.Co;
@@ -165,17 +169,19 @@ im2win_status scratch_layout(const Geometry& g, im2win_dtype dtype, ScratchLayou
 
 static inline bool misaligned(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) != 0; }
 
-// mode bit 0: pack the filter into scratch; bit 1: run the convolution on the packed filter.
+// mode bit 0: pack the filter into scratch; bit 1: run the convolution on the packed filter.  plan_N: the batch that the
+// shape's images are a part of (0: they are all of it).
 enum { kDoPack = 1, kDoConv = 2 };
 static im2win_status conv_common(const void* window, const void* filter, float* y, void* scratch,
                                  size_t scratch_bytes, const im2win_shape* shape, im2win_dtype dtype,
-                                 void* cuda_stream, int mode = kDoPack | kDoConv) {
+                                 void* cuda_stream, int mode = kDoPack | kDoConv, int32_t plan_N = 0) {
   if (!scratch || !shape) return IM2WIN_ERR_NULL_POINTER;
   if ((mode & kDoPack) && !filter) return IM2WIN_ERR_NULL_POINTER;
   if ((mode & kDoConv) && (!window || !y)) return IM2WIN_ERR_NULL_POINTER;
   Geometry g;
   im2win_status st = derive_geometry(shape, &g);
   if (st != IM2WIN_OK) return st;
+  if (plan_N) g.plan_N = plan_N;
   ScratchLayout l;
   st = scratch_layout(g, dtype, &l);
   if (st != IM2WIN_OK) return st;
@@ -504,15 +510,16 @@ im2win_status im2win_layer_forward_host(const void* x_host, const void* filter_h
     return ok;
   };
   const int per = ((g.N + nchunk - 1) / nchunk + unit - 1) / unit * unit;
+  // Chunks run the kernel that the whole batch would, with its order of the sums, so that the result is that of the whole.
   // Every distinct chunk size is validated before anything is queued: its geometry must derive and
-  // the scratch its kernels want (the kernel choice can depend on N) must fit the scratch that was
-  // sized for the whole batch.
+  // the scratch its kernels want must fit the scratch that was sized for the whole batch.
   for (int n0 = 0; n0 < g.N; n0 += per) {
     im2win_shape part = *shape;
     part.N = n0 + per < g.N ? per : g.N - n0;
     Geometry gp;
     ScratchLayout lp;
     st = derive_geometry(&part, &gp);
+    gp.plan_N = g.N;
     if (st == IM2WIN_OK) st = scratch_layout(gp, dtype, &lp);
     if (st != IM2WIN_OK) return st;
     if (lp.total > L.scratch_bytes) return IM2WIN_ERR_WORKSPACE_TOO_SMALL;
@@ -538,7 +545,7 @@ im2win_status im2win_layer_forward_host(const void* x_host, const void* filter_h
     result = im2win_transform(xd, wd, &part, dtype, cuda_stream);
     if (result != IM2WIN_OK) break;
     result = conv_common(wd, ws + L.f_off, reinterpret_cast<float*>(yd), ws + L.scratch_off, L.scratch_bytes, &part,
-                         dtype, cuda_stream);
+                         dtype, cuda_stream, kDoPack | kDoConv, g.N);
     if (result != IM2WIN_OK) break;
     if (!fence(stream, aux.out) ||
         cudaMemcpyAsync(reinterpret_cast<unsigned char*>(y_host) + (size_t)n0 * y_img, yd, (size_t)part.N * y_img,

@@ -24,6 +24,7 @@ struct Geometry {
   int64_t P;             // N*Ho*Wo
   int64_t window_elems;  // N*img_stride
   int64_t out_elems;     // N*Co*Ho*Wo
+  int32_t plan_N;        // batch the kernel and the order of its sums are chosen for: N, or what these N images are a part of
 };
 
 // Scratch layout shared by both precisions (offsets in bytes from `scratch`):
@@ -165,6 +166,7 @@ cudaError_t launch_conv_f32(const float* window, float* y, const void* scratch, 
                             const ScratchLayout& l, cudaStream_t stream);
 cudaError_t launch_pack_f16_runs(const uint16_t* filter, void* scratch, const Geometry& g, cudaStream_t stream);
 cudaError_t launch_conv_f16_runs(const uint16_t* window, float* y, void* scratch, const Geometry& g, cudaStream_t stream);
+// (both plan for g.plan_N images and run on g.N)
 cudaError_t launch_pack_f32_split(const float* filter, void* scratch, const Geometry& g, cudaStream_t stream);
 cudaError_t launch_conv_f32_split(const float* window, float* y, void* scratch, const Geometry& g, cudaStream_t stream);
 cudaError_t launch_pack_f16_shift(const uint16_t* filter, void* scratch, const Geometry& g,

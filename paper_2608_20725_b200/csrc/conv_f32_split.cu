@@ -740,10 +740,12 @@ F32SplitPlan plan_f32_split(const Geometry& g) {
   p.nsub = g.s < g.Kw ? g.s : g.Kw;
   p.Wq = (g.Wp + g.s - 1) / g.s;
   p.VQ = (int64_t)g.N * g.Ho * p.Wq;
-  if (p.VQ + 2 * TILE_M >= ((int64_t)1 << 31)) return p;
+  // Channel tile and split decide the order of the sums: they are chosen for the batch these images belong to.
+  const int64_t plan_VQ = (int64_t)g.plan_N * g.Ho * p.Wq;
+  if (plan_VQ + 2 * TILE_M >= ((int64_t)1 << 31)) return p;
   p.nks_last = (int32_t)((K2 - (int64_t)(p.num_kb - 1) * KB + 15) / 16);
   p.nstages = p.num_kb * p.nsub;
-  const int64_t ntm = (p.VQ + TILE_M - 1) / TILE_M;
+  const int64_t ntm = (plan_VQ + TILE_M - 1) / TILE_M;
   const double steps = ((p.num_kb - 1) * 4.0 + p.nks_last) * g.Kw;   // 16-wide steps of a tile
   const char* force_bn = debug_getenv("IM2WIN_F32_SPLIT_BN");        // testing aids: channel tile, CTAs per tile
   const char* force_z = debug_getenv("IM2WIN_F32_SPLIT_CTAS");
@@ -770,7 +772,7 @@ F32SplitPlan plan_f32_split(const Geometry& g) {
         p.eligible = true;
         p.cost = cost;
         p.bn = bn; p.ntn = nt; p.split = z; p.sb = sb;
-        p.nwork = (int32_t)(ntm * nt);
+        p.nwork = (int32_t)((p.VQ + TILE_M - 1) / TILE_M * nt);
       }
     }
   }

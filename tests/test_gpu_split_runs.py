@@ -188,6 +188,21 @@ def test_filter_pack_takes_any_number_of_channels(precision, layer, monkeypatch)
         check_conv(y[:, part], yr, ar, precision, layer.name)
 
 
+@pytest.mark.parametrize("layer", [L("host_tiles", 32, 256, 28, 28, 256, 3, 3, 1, 1, 260),    # the parts alone: other tiles, clusters
+                                   L("host_clusters", 40, 72, 28, 28, 64, 3, 3, 1, 1, 261),
+                                   L("host_ffma", 24, 7, 70, 70, 64, 3, 3, 1, 1, 262)], ids=lambda l: l.name)
+def test_layer_forward_host_in_parts_gives_the_bits_of_the_whole(layer):
+    dims = layer.dims()
+    x, f = workloads.make_inputs(layer)
+    assert (x.numel() + layer.N * layer.Co * layer.H * layer.W) * 4 >= 8 << 20      # large enough to go in four parts
+    y, _, _ = gpu_conv(x, f, dims, "f32")
+    out = torch.full(y.shape, float("nan")).pin_memory()
+    ws = torch.empty(binding.im2win_layer_workspace_size(dims, binding.F32), dtype=torch.uint8, device="cuda")
+    binding.im2win_layer_forward_host(x.pin_memory(), f.pin_memory(), out, ws, dims)
+    torch.cuda.synchronize()
+    assert np.array_equal(out.numpy(), y)
+
+
 RUNS = [l for l, _ in SPLIT] + [
     L("runs_quad", 2, 3, 19, 23, 20, 7, 7, 2, 3, 230),       # up to four channels: a unit is four channels at two columns' elements
     L("runs_quad1", 3, 2, 12, 9, 16, 1, 1, 1, 0, 231),       # ... one unit, one step
