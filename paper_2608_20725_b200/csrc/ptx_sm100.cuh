@@ -15,8 +15,9 @@ namespace ptx {
 constexpr uint32_t SPIN_LIMIT = 1u << 24;      // polls before a wait gives up (see mbar_wait)
 constexpr uint32_t SPIN_CHUNK = 1024;          // polls between looks at the abort flag and the clock
 constexpr uint64_t SPIN_TIME_NS = 4000000000ull;   // wall-time bound of one wait: 4 s
-// Word 2 of the status block: this marker makes the one-k-block kernel's copy warp leave out one
-// barrier arrival (the test of the bounded waits; nothing in the library writes it).
+// Word 2 of the status block: this marker makes the one-k-block kernel's copy warp, and the first CTA's MMA warp of the
+// run-staged and the fp32 tensor-core kernel, leave out one barrier arrival (the test of the bounded waits; nothing in the
+// library writes it).
 constexpr uint32_t kDebugDropArrive = 0x0d0a11feu;
 // Word 2 again: with this marker the NHWC shifted-view kernel's first K part of a tile does not raise
 // the tile's flag, so that the parts waiting for it run into their limit (same purpose).

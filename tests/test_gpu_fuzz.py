@@ -8,7 +8,7 @@ import numpy as np
 import pytest
 import torch
 
-from paper_2608_20725_b200 import workloads
+from paper_2608_20725_b200 import binding, workloads
 from gpu_helpers import check_conv, check_fused, gpu_conv, gpu_conv_nhwc, gpu_transform, gpu_transform_nhwc, oracle, oracle_inputs
 
 pytestmark = pytest.mark.gpu
@@ -102,3 +102,19 @@ def test_random_layer_nhwc_paths(layer, monkeypatch):
     y_pre, a2 = oracle.epilogue(yr, ar, dims, bias=bias, relu=True, out16=False, nhwc=True)
     y = gpu_conv_nhwc(x, f, dims, bias=bias, relu=True, out16=True, y_nhwc=True)
     check_fused(y, y_pre, a2, True, f"{layer.name} fused")
+
+
+@pytest.mark.parametrize("layer", FUZZ, ids=lambda l: l.name)
+def test_random_layer_split_and_runs(layer, monkeypatch):
+    """The fp32 tensor-core kernel and the run-staged fp16 kernel on every random layer they can take, also those that
+    the library gives to other kernels."""
+    dims = layer.dims()
+    x, f = workloads.make_inputs(layer)
+    monkeypatch.setenv("IM2WIN_F32_KERNEL", "split")
+    monkeypatch.setenv("IM2WIN_F16_KERNEL", "runs")
+    assert binding.im2win_conv_kernel_name(dims, binding.F32) == "f32-split"
+    for precision in ("f32",) + (("f16",) if binding.im2win_conv_kernel_name(dims, binding.F16) == "f16-runs" else ()):
+        xo, fo = oracle_inputs(x, f, precision)
+        yr, ar = oracle.conv_direct(xo, fo, dims)
+        y, _, _ = gpu_conv(x, f, dims, precision)
+        check_conv(y, yr, ar, precision, layer.name)
