@@ -68,6 +68,26 @@ static bool want_f32_split(const Geometry& g) {
   return g.K >= 64;
 }
 
+// Of the layers that neither the one-k-block kernel nor a tiled-copy kernel takes, and the shifted-view kernel could: which
+// ones the run-staged kernel gets.  Its copies are one per channel and image of a tile, so their number for each staged
+// element is (images of a tile) / E, with E elements per virtual column; the shifted-view kernel stages all s columns even
+// where the kernel has fewer (Kw < s).  Measured over 3090 layers (images of 5 to 35, kernels of 1 to 5, strides 1 to 3, 64
+// to 512 channels, batches 1 to 128), shifted-view time / run-staged time:
+//   stride 1, images / E up to 0.7: 1.3 with more than 148 tiles, 0.96 to 0.99 with fewer; above 0.7: 0.4 to 1.0
+//   stride 2 and more: 1.5 on average up to 0.7 (up to 2.1 with Kw < s); 0.5 to 1.3 above
+//   three virtual columns at stride 2 (5x5), more than 64 channels, at most 74 tiles: 0.9 to 1.1
+// On the 1565 layers taken 1.51 times as fast on average, 0.83 at the least (0.9 and less on 10 of them).  (256 -> 512
+// channels, 3x3 stride 2 at 28x28, batch 128: 140 -> 115 us; not taken: 3x3 on 512 channels at 7x7, batch 128, 44 us
+// against 72.)
+static bool prefer_runs(const Geometry& g, const RunsPlan& p) {
+  if (p.G > 3) return false;                               // (5x5 to 11x11 with stride 1: 0.5 to 0.9)
+  const int64_t per_img = (int64_t)g.Ho * p.Wq;
+  const double images = 1.0 + (128.0 + p.halo) / (double)per_img;
+  if (g.s == 1) return g.Co > 64 && images <= 0.7 * p.E && p.nwork > 148;
+  if (p.G == 3 && g.s == 2 && g.Co > 64 && p.nwork <= 74) return false;
+  return images <= (g.Kw < g.s ? 2.1 : 0.7) * p.E;
+}
+
 // The same layer with another batch.
 static Geometry with_batch(Geometry g, int32_t N) {
   g.N = N;
@@ -150,15 +170,10 @@ im2win_status scratch_layout(const Geometry& part, im2win_dtype dtype, ScratchLa
     l->f16_mat = mat.eligible && want && !l->f16_stem;
     const MatPlan any_mat = plan_for_any_batch(mat, plan_f16_mat, g);
     if (any_mat.eligible) most = std::max(most, (int64_t)any_mat.scratch_bytes);
-    // Layers that neither the one-k-block kernel nor a tiled-copy kernel takes: kernels up to three virtual columns
-    // (Kw <= 3 s) go to the run-staged kernel where they are strided or have more than 64 output channels, and so does
-    // what the shifted-view kernel cannot stage.  Measured against the latter: 3x3 with stride 2 1.1 to 1.8 times faster
-    // (256 -> 512 channels at 28x28, batch 128: 140 -> 115 us), 3x3 with stride 1 on 128 to 379 channels 1.2 to 1.6;
-    // 0.8 to 1.0 on fewer channels, 0.5 to 0.9 on 5x5 to 11x11 with stride 1, whose tall tiles share filter stages.
     const RunsPlan runs = plan_f16_runs(g);
     if (runs.eligible) {
       const bool rest = !l->f16_stem && !l->f16_mat && !l->f16_raw;
-      l->f16_runs = force ? strcmp(force, "runs") == 0 : rest && (!l->f16_shift || (runs.G <= 3 && (g.s > 1 || g.Co > 64)));
+      l->f16_runs = force ? strcmp(force, "runs") == 0 : rest && (!l->f16_shift || prefer_runs(g, runs));
     }
     const RunsPlan any_runs = plan_for_any_batch(runs, plan_f16_runs, g);
     if (any_runs.eligible) most = std::max(most, kStatusBytes + (int64_t)any_runs.filter_bytes);

@@ -34,3 +34,14 @@ def test_scratch_does_not_depend_on_the_batch(layer, dtype):
                                       (600, 11, "f32-ffma")])       # 27, 63, 64, 72 terms; an offset table too long
 def test_f32_kernel_by_length_of_the_reduction(C, K, want):
     assert binding.im2win_conv_kernel_name((2, C, 20, 20, 24, K, K, 1, K // 2), binding.F32) == want
+
+
+@pytest.mark.parametrize("layer,want", [
+    ((128, 256, 28, 28, 512, 3, 3, 2, 1), "f16-runs"), ((13, 37, 45, 61, 75, 5, 5, 2, 2), "f16-runs"),
+    ((64, 128, 27, 27, 128, 3, 3, 1, 1), "f16-runs"), ((64, 256, 15, 15, 130, 1, 1, 3, 0), "f16-shift"),
+    ((128, 512, 7, 7, 512, 3, 3, 1, 1), "f16-shift"),      # several images in a tile: a copy per image and channel
+    ((128, 512, 7, 7, 1024, 1, 1, 1, 0), "f16-shift"),     # one element per column and copy
+    ((1, 256, 27, 27, 256, 3, 3, 1, 1), "f16-shift"),      # few tiles
+    ((32, 64, 61, 45, 64, 3, 3, 1, 0), "f16-shift")])      # 64 channels
+def test_f16_kernel_on_odd_planes(layer, want):
+    assert binding.im2win_conv_kernel_name(layer, binding.F16) == want
