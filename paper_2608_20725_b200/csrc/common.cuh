@@ -136,7 +136,7 @@ F32SplitPlan plan_f32_split(const Geometry& g);
 // Tile and ring geometry of the run-staged kernel (see conv_f16_runs.cu).
 struct RunsPlan {
   bool eligible, resident, quad;       // quad: up to four channels, see the order of k2 there
-  int32_t units, octs, E, G, Wq, pitch, rows, halo, num_kb, nks_last;
+  int32_t units, octs, E, G, Wq, rows, halo, num_kb, nks_last;
   int32_t region, raw_slot, a_stage, slot_bytes;
   int32_t bn, ntn, nwork, sa, sr, sb;
   int64_t VQ;

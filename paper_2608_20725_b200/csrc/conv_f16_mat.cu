@@ -98,7 +98,6 @@ struct Segment {            // the part of a tile that lies in one image
 // the filter pack (the kernel before it in the stream) is still running; its barrier setup, tensor
 // memory allocation and descriptor fetches overlap the pack.  Every role that touches global memory
 // first waits for the preceding kernel to have completed (and its writes to be visible).
-__device__ __forceinline__ void wait_for_previous_kernel() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void let_next_kernel_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // Splits the rows of the tile starting at virtual position q0 by image: within an image the

@@ -6,7 +6,7 @@
 // convolution of stride s is one of stride 1 on columns s times as tall: virtual column i holds e = t*Kh + u
 // (t < min(s, Kw)), E = min(s, Kw)*Kh of them, and the kernel is G = ceil(Kw/s) virtual columns wide; filter elements
 // with g*s + t >= Kw are zeros (3x3 with stride 2: a third more products, but every element is staged once and from
-// one run).  A GEMM row is a virtual position q = (n*Ho + ho)*pitch + i; S[row][64 k2] is staged once per k2-block and
+// one run).  A GEMM row is a virtual position q = (n*Ho + ho)*Wq + i, Wq = ceil(Wp/s); S[row][64 k2] is staged once per k2-block and
 // the MMAs of virtual kernel column g read the view that starts g rows further down.
 //
 // Order of k2.  A unit of eight k2 (16 bytes of S) is eight channels at one e: unit j = octet * E + e (up to four
@@ -32,6 +32,7 @@
 
 #define IM2WIN_INLINE_SLOW_WAIT      // (a call beside the epilogue's live sums costs spills)
 #include "common.cuh"
+#include "launch.cuh"
 #include "ptx_sm100.cuh"
 
 namespace im2win {
@@ -65,19 +66,15 @@ struct RunsParams {
   uint32_t* status;
   int64_t img_bytes, chan_bytes, win_bytes;   // of one image, one channel plane, the whole window tensor
   uint32_t VQ;
-  FastDiv div_pitch, div_ho;
-  int32_t C, N, Wp, Wq, pitch, Ho, Wo, HoWo, Co, Kh, Kw, s;
+  FastDiv div_wq, div_ho;
+  int32_t C, Wp, Wq, Ho, Wo, HoWo, Co, Kh, Kw, s;
   int32_t E, G, units, num_kb, nks_last;      // units: of eight k2
   int32_t quad;                               // 1: up to four channels, a unit is four channels at two e
   int32_t foreign;                            // 1: zero filter elements meet elements that are not of the window
-  int32_t rows, halo, region, octs, raw_slot, a_stage;
+  int32_t halo, region, octs, raw_slot, a_stage;
   int32_t bn, ntn, nwork, sa, sr, sb, slot_bytes, resident;
 };
 
-__device__ __forceinline__ void wait_for_previous_kernel() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void st_shared16(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
-  asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
-}
 __device__ __forceinline__ uint32_t ld_shared_u16(uint32_t addr) {
   uint16_t v;
   asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(addr) : "memory");
@@ -94,8 +91,8 @@ struct TileRuns {
 };
 __device__ __forceinline__ int run_size(int elems) { return (elems * ES + 30) & ~15; }
 __device__ __forceinline__ void split_q(const RunsParams& q, uint32_t vq, uint32_t& n, int& ho, int& i) {
-  const uint32_t sg = q.div_pitch(vq);
-  i = (int)(vq - sg * (uint32_t)q.pitch);
+  const uint32_t sg = q.div_wq(vq);
+  i = (int)(vq - sg * (uint32_t)q.Wq);
   n = q.div_ho(sg);
   ho = (int)(sg - n * (uint32_t)q.Ho);
 }
@@ -103,14 +100,13 @@ __device__ __forceinline__ TileRuns tile_runs(const RunsParams& q, uint32_t q0) 
   TileRuns r;
   int ho, i;
   split_q(q, q0, r.n0, ho, i);
-  if (i > q.Wq - 1) i = q.Wq - 1;                           // (a dead row of a widened pitch: any column will do)
   r.start0 = (ho * q.Wp + i * q.s) * q.Kh;
   uint32_t ql = q0 + TILE_M + q.halo - 1;
   if (ql >= q.VQ) ql = q.VQ - 1;
   split_q(q, ql, r.n1, ho, i);
   // (all s columns of the last virtual column: where s does not divide Wp some lie in the next strip or plane.  Only
   // zero filter elements meet them, but they have to be numbers)
-  r.end1 = (ho * q.Wp + ((i < q.Wq - 1 ? i : q.Wq - 1) + 1) * q.s) * q.Kh;
+  r.end1 = (ho * q.Wp + (i + 1) * q.s) * q.Kh;
   return r;
 }
 
@@ -224,12 +220,10 @@ __global__ void __launch_bounds__(THREADS, 1) conv_f16_runs_kernel(RunsParams q)
           uint32_t n;
           int ho, i;
           split_q(q, vq, n, ho, i);
-          if (i < q.Wq) {
-            const int g = (int)(n - tr.n0), start = g == 0 ? tr.start0 : 0;
-            if (g > 0) off = run_size(plane - tr.start0) + (g - 1) * run_size(plane);
-            off += ((ho * q.Wp + i * q.s) * q.Kh - start) * ES;
-            phase = (uint32_t)((int64_t)n * q.img_bytes + (int64_t)start * ES);
-          }
+          const int g = (int)(n - tr.n0), start = g == 0 ? tr.start0 : 0;
+          if (g > 0) off = run_size(plane - tr.start0) + (g - 1) * run_size(plane);
+          off += ((ho * q.Wp + i * q.s) * q.Kh - start) * ES;
+          phase = (uint32_t)((int64_t)n * q.img_bytes + (int64_t)start * ES);
         }
 #pragma unroll
         for (int x = 0; x < 8; ++x) rb[x] = off + x * q.region + ((phase + (uint32_t)x * (uint32_t)q.chan_bytes) & 15u);
@@ -267,7 +261,7 @@ __global__ void __launch_bounds__(THREADS, 1) conv_f16_runs_kernel(RunsParams q)
             };
             unit(rb, row);
             // the rows below the tile: lanes of one of the warpgroup's warps, another one from unit to unit
-            if (((4 * kb + (ch >> 1)) & 3) == (warp & 3) && lane < q.halo) unit(hb, TILE_M + lane);
+            if ((ch >> 1) == (warp & 3) && lane < q.halo) unit(hb, TILE_M + lane);
           }
           if (++in_slot == per_slot || 8 * kb + ch == q.units - 1) {
             __syncwarp();
@@ -553,17 +547,7 @@ cudaError_t launch_form(const RunsParams& q, int smem, cudaStream_t stream) {
     if (e != cudaSuccess) return e;
     attr_done[dev] = true;
   }
-  cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.gridDim = dim3((unsigned)(q.nwork < 148 ? q.nwork : 148), 1, 1);
-  cfg.blockDim = dim3(THREADS, 1, 1);
-  cfg.dynamicSmemBytes = (size_t)smem;
-  cfg.stream = stream;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, conv_f16_runs_kernel<BNMAX>, q);
+  return launch_after_previous(conv_f16_runs_kernel<BNMAX>, q.nwork < 148 ? q.nwork : 148, 1, THREADS, smem, stream, q);
 }
 
 }  // namespace
@@ -590,12 +574,11 @@ RunsPlan plan_f16_runs(const Geometry& g) {
   p.halo = p.G - 1;
   if (p.halo > 31) return p;                                // (one lane per row below the tile)
   p.Wq = (g.Wp + g.s - 1) / g.s;
-  p.pitch = p.Wq;
-  p.VQ = (int64_t)g.N * g.Ho * p.pitch;
+  p.VQ = (int64_t)g.N * g.Ho * p.Wq;
   if (p.VQ + 2 * TILE_M >= ((int64_t)1 << 31)) return p;
   p.rows = TILE_M + (p.halo + 7) / 8 * 8;
   p.a_stage = p.rows * 128;
-  const int64_t per_img = (int64_t)g.Ho * p.pitch;
+  const int64_t per_img = (int64_t)g.Ho * p.Wq;
   const int64_t segs = (TILE_M + p.halo - 2) / per_img + 2;
   if (segs > MAX_SEG) return p;
   // bytes a tile's columns of one channel take in a raw slot, whatever the tile
@@ -658,14 +641,14 @@ cudaError_t launch_conv_f16_runs(const uint16_t* window, float* y, void* scratch
   q.status = reinterpret_cast<uint32_t*>(base);
   q.img_bytes = g.img_stride * ES; q.chan_bytes = g.chan_stride * ES; q.win_bytes = g.window_elems * ES;
   q.VQ = (uint32_t)p.VQ;
-  q.div_pitch = fast_div((uint32_t)p.pitch);
+  q.div_wq = fast_div((uint32_t)p.Wq);
   q.div_ho = fast_div((uint32_t)g.Ho);
-  q.C = g.C; q.N = g.N; q.Wp = g.Wp; q.Wq = p.Wq; q.pitch = p.pitch; q.Ho = g.Ho; q.Wo = g.Wo; q.HoWo = g.Ho * g.Wo;
+  q.C = g.C; q.Wp = g.Wp; q.Wq = p.Wq; q.Ho = g.Ho; q.Wo = g.Wo; q.HoWo = g.Ho * g.Wo;
   q.Co = g.Co; q.Kh = g.Kh; q.Kw = g.Kw; q.s = g.s;
   // kernel columns beyond Kw, channels beyond C in the last octet, the element beyond an odd E
   q.foreign = (g.Kw > g.s && g.Kw % g.s != 0) || (p.quad ? p.E % 2 != 0 : g.C % 8 != 0);
   q.E = p.E; q.G = p.G; q.units = p.units; q.quad = p.quad ? 1 : 0; q.num_kb = p.num_kb; q.nks_last = p.nks_last;
-  q.rows = p.rows; q.halo = p.halo; q.region = p.region; q.octs = p.octs; q.raw_slot = p.raw_slot; q.a_stage = p.a_stage;
+  q.halo = p.halo; q.region = p.region; q.octs = p.octs; q.raw_slot = p.raw_slot; q.a_stage = p.a_stage;
   q.bn = p.bn; q.ntn = p.ntn; q.nwork = p.nwork; q.sa = p.sa; q.sr = p.sr; q.sb = p.sb;
   q.slot_bytes = p.slot_bytes; q.resident = p.resident ? 1 : 0;
   const int smem = 1024 + p.sa * p.a_stage + p.sb * p.slot_bytes + p.sr * p.raw_slot;

@@ -46,6 +46,7 @@
 
 #define IM2WIN_INLINE_SLOW_WAIT      // (a call cannot be compiled beside the 128 live sums of the epilogue warps)
 #include "common.cuh"
+#include "launch.cuh"
 #include "ptx_sm100.cuh"
 
 namespace im2win {
@@ -74,7 +75,6 @@ struct SplitParams {
   int32_t bn, ntn, nwork, nstages, split, sb, slot_bytes, chain;
 };
 
-__device__ __forceinline__ void wait_for_previous_kernel() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // (volatile: the loads of a batch stay together, ahead of the wait for the stage they are for; left to
 // itself the compiler may move them to their uses, one round trip per eight loads)
@@ -112,9 +112,6 @@ __device__ __forceinline__ void split2(float a, float b, uint32_t& p1, uint32_t&
   v = sub_pieces(v, p1);
   p2 = cvt_pair(v);
   p3 = cvt_pair(sub_pieces(v, p2));
-}
-__device__ __forceinline__ void st_shared16(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
-  asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
 }
 __device__ __forceinline__ void tmem_ld16_issue(uint32_t taddr, uint32_t (&r)[16]) {
   asm volatile(
@@ -713,20 +710,8 @@ cudaError_t launch_form(const SplitParams& q, int smem, cudaStream_t stream) {
     if (e != cudaSuccess) return e;
     attr_done[dev] = true;
   }
-  cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute attr[2];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  attr[1].id = cudaLaunchAttributeClusterDimension;
-  attr[1].val.clusterDim.x = (unsigned)q.split; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
   const int grid = q.split > 1 ? q.nwork * q.split : (q.nwork < 148 ? q.nwork : 148);
-  cfg.gridDim = dim3((unsigned)grid, 1, 1);
-  cfg.blockDim = dim3(Form<BNMAX, PWG>::THREADS, 1, 1);
-  cfg.dynamicSmemBytes = (size_t)smem;
-  cfg.stream = stream;
-  cfg.attrs = attr;
-  cfg.numAttrs = q.split > 1 ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, conv_f32_split_kernel<BNMAX, PWG>, q);
+  return launch_after_previous(conv_f32_split_kernel<BNMAX, PWG>, grid, q.split, Form<BNMAX, PWG>::THREADS, smem, stream, q);
 }
 
 }  // namespace

@@ -92,7 +92,6 @@ struct NhwcParams {
 // (the filter pack) is still running, so that its barrier set-up, tensor-memory allocation and
 // descriptor fetches overlap that kernel; every role that touches global memory first waits for the
 // preceding kernel to have completed.
-__device__ __forceinline__ void wait_for_previous_kernel() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 __device__ __forceinline__ void red_add_f32(float* p, float v) {
   asm volatile("red.global.add.f32 [%0], %1;" ::"l"(p), "f"(v) : "memory");
