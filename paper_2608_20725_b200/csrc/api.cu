@@ -58,14 +58,19 @@ im2win_status derive_geometry(const im2win_shape* s, Geometry* g) {
   return IM2WIN_OK;
 }
 
-// Which fp32 kernel: the tensor cores from 64 terms on.  Measured over sixty layers of all sizes: 1.1 to 18 times
-// faster than the FFMA kernel from 72 terms on, 0.4 to 1.1 times below 64, where half-empty k2-blocks are split and
-// multiplied.  Forcing one of the FFMA kernel's forms, or IM2WIN_F32_KERNEL=ffma|split, decides it (testing aids).
-static bool want_f32_split(const Geometry& g) {
+// Which fp32 kernel: the tensor cores from 64 terms on, but up to 80 only where one stage holds them (not two k2-blocks or
+// column classes, the second nearly empty) and up to 256 channels, and below 160 only where 0.6 of the multiplied terms are
+// real (a kernel column's C * Kh terms are rounded up to 16).  Measured on 754 layers, FFMA time / time here: of the 345
+// with 64 terms and more that the rule takes 2.07 on average, 13 below 0.97, 0.85 at the least, up to 22; of the 169 it leaves
+// to the FFMA kernel 1.0 on average (0.62 to 1.47); 0.56 to 1.2 below 64 terms.  Forcing one of the FFMA kernel's forms, or
+// IM2WIN_F32_KERNEL=ffma|split, decides it (testing aids).
+static bool want_f32_split(const Geometry& g, const F32SplitPlan& p) {
   if (const char* v = debug_getenv("IM2WIN_F32_KERNEL")) return strcmp(v, "split") == 0;
   for (const char* name : {"IM2WIN_F32_BM", "IM2WIN_F32_TALL", "IM2WIN_F32_KLANES", "IM2WIN_F32_BK"})
     if (debug_getenv(name)) return false;
-  return g.K >= 64;
+  const int64_t multiplied = ((p.num_kb - 1) * 4 + p.nks_last) * (int64_t)16 * g.Kw;
+  if (g.K < 64 || (g.K < 160 && 10 * g.K < 6 * multiplied)) return false;
+  return g.K > 80 || (p.nstages == 1 && g.Co <= 256);
 }
 
 // Of the layers that neither the one-k-block kernel nor a tiled-copy kernel takes, and the shifted-view kernel could: which
@@ -131,7 +136,7 @@ im2win_status scratch_layout(const Geometry& part, im2win_dtype dtype, ScratchLa
   int64_t most = (int64_t)l->total;                        // of all layouts, whichever kernel is picked or forced
   if (dtype == IM2WIN_F32) {
     const F32SplitPlan split = plan_f32_split(g);
-    l->f32_split = split.eligible && want_f32_split(g);
+    l->f32_split = split.eligible && want_f32_split(g, split);
     l->ffma_total = l->total;
     const int64_t Kp = round_up(g.K, 32);                  // (the widest k-block of the FFMA kernel)
     most = round_up((int64_t)kStatusBytes + 4 * Kp, 256) + Kp * l->Co_pad * 4;

@@ -177,6 +177,7 @@ def test_conv_f32_split_recomputes_whole_tensors_in_bounded_time(what, monkeypat
 def test_filter_pack_takes_any_number_of_channels(precision, layer, monkeypatch):
     """More channel blocks than the second axis of a grid has (65535)."""
     monkeypatch.setenv("IM2WIN_F16_KERNEL", "runs")
+    monkeypatch.setenv("IM2WIN_F32_KERNEL", "split")
     dims = layer.dims()
     code = binding.F32 if precision == "f32" else binding.F16
     assert binding.im2win_conv_kernel_name(dims, code) == ("f32-split" if precision == "f32" else "f16-runs")

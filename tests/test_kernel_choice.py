@@ -45,3 +45,14 @@ def test_f32_kernel_by_length_of_the_reduction(C, K, want):
     ((32, 64, 61, 45, 64, 3, 3, 1, 0), "f16-shift")])      # 64 channels
 def test_f16_kernel_on_odd_planes(layer, want):
     assert binding.im2win_conv_kernel_name(layer, binding.F16) == want
+
+
+@pytest.mark.parametrize("layer,want", [
+    ((128, 64, 56, 56, 256, 1, 1, 1, 0), "f32-split"), ((128, 64, 56, 56, 300, 1, 1, 1, 0), "f32-ffma"),
+    ((8, 80, 28, 28, 128, 1, 1, 1, 0), "f32-ffma"),        # 80 terms in two k2-blocks
+    ((8, 81, 28, 28, 128, 1, 1, 1, 0), "f32-split"),
+    ((32, 3, 56, 56, 64, 5, 5, 2, 2), "f32-ffma"),         # 75 terms in two column classes
+    ((64, 8, 49, 20, 300, 1, 11, 2, 1), "f32-ffma"),       # 88 terms, half of the multiplied ones are zeros
+    ((128, 3, 224, 224, 64, 7, 7, 2, 3), "f32-split")])
+def test_f32_kernel_on_short_reductions(layer, want):
+    assert binding.im2win_conv_kernel_name(layer, binding.F32) == want
