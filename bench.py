@@ -3,13 +3,15 @@
 
 A step is one pass of the whole hot path over one batch of the headline layer
 (ResNet-style 3x3 layer, N=128 C=64 56x56 -> 64): im2win transform, filter
-pack and convolution, once in fp32 (CUDA cores) and once in fp16-in /
-fp32-accumulate (tensor cores).  The metric is convolution TFLOPS,
+pack and convolution, once in fp32 and once in fp16-in / fp32-accumulate
+(both on tensor cores).  The metric is convolution TFLOPS,
 2*N*Co*Ho*Wo*C*Kh*Kw per precision, over the device time of the whole step.
 
     python bench.py [--gpus N] [--steps K] [--warmup W] [--impl reference] [--report FILE]
 
-prints one JSON line (rank 0).  `--report FILE` additionally times every layer
+prints one JSON line (rank 0) on stdout, short enough for the tail of a log, and
+the call-by-call figures behind it (rooflines, memory, every benchmark layer) as
+a second JSON object on stderr.  `--report FILE` additionally times every layer
 of the workload table kernel by kernel and writes one JSON object per layer.
 """
 from __future__ import annotations
@@ -333,6 +335,15 @@ def time_cpu_oracle(layer, target_seconds=12.0):
                       f"{reps} passes ({dt:.1f} s)"}
 
 
+def rounded(v):
+    """Floats to six significant digits, through dicts and lists (a short line)."""
+    if isinstance(v, dict):
+        return {k: rounded(x) for k, x in v.items()}
+    if isinstance(v, (list, tuple)):
+        return [rounded(x) for x in v]
+    return float(f"{v:.6g}") if isinstance(v, float) else v
+
+
 def run_gpu_arm(args):
     from paper_2608_20725_b200 import binding
     rank = int(os.environ.get("RANK", "0"))
@@ -422,7 +433,10 @@ def run_gpu_arm(args):
     dominant = max(avg_ms, key=avg_ms.get)
     roof = dict(rooflines[dominant])
     roof["kernel"] = dominant
-    roof["traffic"] = traffic.get(f"{layer.name}:{dominant}")
+    if dominant.startswith("conv"):             # (measured per kernel: another kernel's bytes would say nothing)
+        kernel = binding.im2win_conv_kernel_name(runner.dims, binding.F32 if dominant == "conv_f32" else binding.F16)
+        roof["kernel"] = f"{dominant}:{kernel}"
+    roof["traffic"] = traffic.get(f"{layer.name}:{roof['kernel']}")
 
     out = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps, "warmup": args.warmup,
@@ -436,22 +450,22 @@ def run_gpu_arm(args):
         "tflops_with_transform": {p: runner.flops / ((avg_ms[f"conv_{p}"] + avg_ms[f"transform_{p}"]) * 1e-3) / 1e12
                                   for p in runner.precisions},
         "roofline": roof,
-        "kernels": rooflines,
-        "memory": dict(runner.memory_report(), torch_peak_allocated_bytes=peak_alloc),
         "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h,
                 "steps": e2e_steps, "ms_per_step": e2e_ms / e2e_steps},
         "gpu_launches": 6 * args.steps,
         "clocks": clocks,
     }
+    details = {"kernels": rooflines, "memory": dict(runner.memory_report(), torch_peak_allocated_bytes=peak_alloc)}
     if rank == 0:
         if world == 1 and not args.no_per_layer:
             # every BASELINE config, call by call (the metric is "per layer"): 20 launches each
             del runner, e2e_sets
             torch.cuda.empty_cache()
-            out["per_layer"] = per_layer_summary(layer_rows(peaks, peak_kind, iters=20, with_packed=False))
+            details["per_layer"] = per_layer_summary(layer_rows(peaks, peak_kind, iters=20, with_packed=False))
         if world == 1 and not args.no_cpu_baseline:
             out["cpu_baseline"] = time_cpu_oracle(layer)
-        print(json.dumps(out))
+        print(json.dumps(details), file=sys.stderr, flush=True)
+        print(json.dumps(rounded(out)), flush=True)
     if args.report and rank == 0:
         write_report(args.report, peaks, peak_kind,
                      names=args.report_layers.split(",") if args.report_layers else None)
@@ -599,7 +613,7 @@ def write_report(path, peaks, peak_kind, names=None, iters=20):
 
 
 def per_layer_summary(rows):
-    """The per-layer part of the bench line: for every BASELINE config and each of its calls the
+    """The per-layer part of the details: for every BASELINE config and each of its calls the
     device time, the bounding roofline and the fraction reached, plus the memory figures."""
     out = {}
     for row in rows:
