@@ -5,8 +5,8 @@
  * data transformation (paper Eq. 2) and the forward convolution over the
  * im2win tensor (paper Eq. 3, GEMM view of Algorithm 1) in two precisions:
  * fp32 (on tensor cores through an exact three-piece split of every operand,
- * on CUDA cores for reductions below 64 terms) and fp16-input /
- * fp32-accumulate on tensor cores.
+ * on CUDA cores for short reductions) and fp16-input / fp32-accumulate on
+ * tensor cores.
  *
  * Problem statement (paper, Section "Notation"): input I[N][C][H][W], filter
  * F[Co][C][Kh][Kw] (OIHW), output O[N][Co][Ho][Wo], all row-major with the
@@ -82,7 +82,8 @@ const char* im2win_conv_kernel_name(const im2win_shape* shape, im2win_dtype dtyp
  *                   of the im2win tensor (paper Eq. 2; Section "Im2win Data
  *                   Transformation"), with no hidden padding.
  *   scratch_bytes = what im2win_conv_f32 / im2win_conv_f16 need in `scratch`
- *                   (a status block, the repacked filter, and an offset table or a copy of the filter).
+ *                   (a status block, the repacked filter, and an offset table or a copy of the filter); the
+ *                   same for every N.  In fp32 about 2.7 times the filter's own bytes.
  *   Ho, Wo        = output height and width.
  * Any of the four output pointers may be NULL.
  */
@@ -112,8 +113,8 @@ im2win_status im2win_transform(const void* x_nchw, void* window, const im2win_sh
  * The filter is repacked into `scratch` on every call (part of the timed
  * operation).  `y_nchw` is [N][Co][Ho][Wo] fp32.  `scratch` must hold at least
  * the scratch_bytes reported by im2win_workspace_size(shape, IM2WIN_F32, ...).
- * Sums are fp32 and their order is unspecified.  Reductions of 64 terms or more run on the tensor cores
- * (im2win_conv_kernel_name: "f32-split"; a few shapes its tiles do not hold stay on CUDA cores):
+ * Sums are fp32 and their order is unspecified; it may depend on the batch.  Most reductions of 64 terms or more run
+ * on the tensor cores (im2win_conv_kernel_name: "f32-split"):
  * every element, subnormal ones included, is the exact sum of three scaled bf16 pieces, and six products of
  * pieces stand for one fp32 product to within 2^-26 of it; the error against 64 bits is
  * below that of a chain of fp32 FMAs.  Outputs of 2^82 and more, outputs that meet an element of 2^104 or more, and
@@ -312,12 +313,17 @@ const char* im2win_nhwc_kernel_name(const im2win_shape* shape, const im2win_epil
  * IM2WIN_STATIC_SCRATCH_BYTES that every GPU which loads the library holds until
  * the process exits.
  *
- * Same operation, arguments and results as im2win_conv_f32 (window, filter and
+ * Same operation and arguments as im2win_conv_f32 (window, filter and
  * y are the caller's device buffers).  Differences:
- *   - A layer whose scratch_bytes (im2win_workspace_size, IM2WIN_F32) exceed
+ *   - It always runs on CUDA cores (fp32 FMAs, the reduction in ascending order),
+ *     also where im2win_conv_f32 uses the tensor cores: results agree within the
+ *     accuracy of fp32 sums, not bit for bit, and long reductions are slower.
+ *   - A layer whose packed filter and offset table do not fit
  *     IM2WIN_STATIC_SCRATCH_BYTES is rejected with IM2WIN_ERR_WORKSPACE_TOO_SMALL
- *     before anything is launched (roughly: Co*C*Kh*Kw above one million filter
- *     elements does not fit).
+ *     before anything is launched: with Co rounded up to the channel tile (64; 96
+ *     or 128 above 64) and C*Kh*Kw to 16 or 32, four bytes per filter element
+ *     (roughly: above one million elements does not fit).  This is less than the
+ *     scratch_bytes of im2win_workspace_size, which cover both kernels.
  *   - The call allocates nothing: no cudaMalloc, no cudaFree, no allocating
  *     library routine.
  *   - The first call on each device looks up the device address of the array

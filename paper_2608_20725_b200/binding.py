@@ -214,8 +214,8 @@ def im2win_conv_f16(window, filter_oihw, y, scratch, shape, stream=None) -> None
 
 
 def im2win_conv_f32_static(window, filter_oihw, y, shape, stream=None) -> None:
-    """fp32 convolution for callers that cannot allocate device memory: same as im2win_conv_f32
-    but the scratch lives in a fixed array inside the library (layers needing more than
+    """fp32 convolution for callers that cannot allocate device memory: the operation of im2win_conv_f32,
+    always on CUDA cores, with the scratch in a fixed array inside the library (layers needing more than
     STATIC_SCRATCH_BYTES are rejected).  Calls that may overlap on the GPU must be serialised."""
     s = as_shape(shape)
     for t in (window, filter_oihw, y):

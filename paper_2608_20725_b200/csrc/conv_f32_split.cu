@@ -9,8 +9,9 @@
 // last and truncates the sum (measured), so a long chain in one accumulator drifts towards zero.  A chain
 // here is therefore short: the products of 64 k2 of one kernel column (a "unit") go into a fresh
 // accumulator, the small products first, and the epilogue warps add it to fp32 registers with rounded adds.
-// Error against 64 bits, relative 2-norm (round-to-nearest FFMA chain -> this kernel): K = 147 2.2e-7 ->
-// 0.8e-7, K = 576 4.3e-7 -> 1.0e-7, K = 4608 1.2e-6 -> 1.8e-7, on inputs of both signs and of one.
+// Error against 64 bits, relative 2-norm (round-to-nearest FFMA chain -> this kernel), inputs of both signs and of one:
+// K = 147 2.2e-7 -> 0.9e-7, K = 576 4.4e-7 -> 1.8e-7 with the long chains of the narrow tiles (below) and 1.0e-7 without,
+// K = 4608 1.1e-6 -> 1.7e-7 and 1.1e-7.
 // The last bit of the smallest fp32 values, 2^-149, becomes bf16's smallest normal value, 2^-126, by the scaling: no piece
 // of any operand gets lost, or is a subnormal (by whose exponent the tensor core would align its addends: scaled by
 // 2^16, weights of 2^-145 gave six times the error).  Elements of 2^104 and sums of 2^82 and more give a non-finite
@@ -23,7 +24,7 @@
 // and kernel column v multiplies the view that starts (v div s) rows further down; with stride s a stage
 // holds one column class t = v mod s.  Rows are the virtual positions q = (n*Ho + ho)*Wq + i, Wq = ceil(Wp/s).
 //
-// What bounds it: the tensor pipe, and next to it the shared-memory pipe the MMA reads its operands
+// What bounds it: the tensor pipe on wide tiles, and next to it the shared-memory pipe the MMA reads its operands
 // through: an instruction of M = 128, K = 16 takes max(N/2, 32 + N/4) cycles.  Up to 64 channels the filter
 // pieces therefore lie side by side as one operand, [w1 | w2 | w3], and four instructions replace six: x1 against all
 // of it into three accumulators (x1w1 | x1w2 | x1w3), and x2w1, x2w2 and x3w1 into a fourth, so that no accumulator holds
@@ -35,11 +36,12 @@
 // Roles (one persistent CTA per SM): one or two warpgroups of producers (thread = row; 32 loads in flight,
 // split, 16-byte stores), an MMA warp, a filter-copy warp (one untiled bulk copy per piece: the pack kernel
 // writes shared-memory images), eight epilogue warps that keep the tile's fp32 sums in registers.
-// Measured against the FFMA kernel (us): 3x3 on 64 channels at 56x56, batch 128, 543 -> 226 (131 TFLOP/s); 3x3 on 512
-// channels at 7x7 624 -> 163; 11x11 on 256 channels at 28x28, batch 64, 14780 -> 4100 (194 TFLOP/s; 1.6 PFLOP/s of bf16
-// products with the strip ends, near the power limit); 7x7 stride 2 on 3 channels at 224x224 641 -> 428.
+// Measured against the FFMA kernel (us, filter packed beforehand): 3x3 on 64 channels at 56x56, batch 128, 543 -> 221 (134
+// TFLOP/s; no pipe above 45 % of its rate: hand-offs over two stages); 3x3 on 512 channels at 7x7 627 -> 170; 11x11 on 256
+// channels at 28x28, batch 64, 14824 -> 4018 (198 TFLOP/s; 1.6 PFLOP/s of bf16 products with the strip ends, near the
+// power limit); 7x7 stride 2 on 3 channels at 224x224 642 -> 428.
 // A layer with few tiles is run by clusters of 2, 4 or 8 CTAs that share the stages of a tile and add their
-// registers through distributed shared memory, in rank order: 3x3 on 512 channels, one 7x7 image, 225 -> 32 us.
+// registers through distributed shared memory, in rank order: 3x3 on 512 channels, one 7x7 image, 225 -> 31 us.
 #include <cuda_bf16.h>
 #include <stdlib.h>
 #include <string.h>
