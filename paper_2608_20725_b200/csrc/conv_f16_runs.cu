@@ -301,8 +301,7 @@ __global__ void __launch_bounds__(THREADS, 1) conv_f16_runs_kernel(RunsParams q)
       // (testing aid: the commit of the first tile left out; looked up while its first stage is on its way)
       uint32_t drop = blockIdx.x == 0 ? *reinterpret_cast<volatile uint32_t*>(q.status + 2) : 0u;
       auto need = [&](uint32_t bar, uint32_t parity, uint32_t seen) {
-        if (__all_sync(0xffffffffu, seen != 0u)) return true;
-        return (bool)__all_sync(0xffffffffu, mbar_wait(bar, parity, &abort_flag, q.status));
+        return mbar_wait_unless_seen(bar, parity, seen, &abort_flag, q.status);
       };
       for (int w = blockIdx.x; w < q.nwork && ok; w += gridDim.x, ++ac) {
         const int ab = ac & (NACC - 1);

@@ -126,6 +126,12 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     if (mbar_try_wait(bar, parity)) return true;
   return mbar_wait_slow<false>(bar, parity, abort_flag, status);
 }
+// A warp's wait for a barrier that an earlier mbar_test_wait may have found complete already (the whole warp calls it).
+__device__ __forceinline__ bool mbar_wait_unless_seen(uint32_t bar, uint32_t parity, uint32_t seen, volatile uint32_t* abort_flag,
+                                                      uint32_t* status) {
+  if (__all_sync(0xffffffffu, seen != 0u)) return true;
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, status));
+}
 __device__ __forceinline__ void st_shared16(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
   asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
 }
