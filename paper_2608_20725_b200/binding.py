@@ -93,7 +93,9 @@ def lib() -> ctypes.CDLL:
     L.im2win_conv_kernel_name.restype = ctypes.c_char_p
     L.im2win_nhwc_kernel_name.argtypes = [P(Shape), P(Epilogue)]
     L.im2win_nhwc_kernel_name.restype = ctypes.c_char_p
+    # the library looks at IM2WIN_DEBUG in its first plan: here, so that both sides see the same
     _debug = bool(os.environ.get("IM2WIN_DEBUG"))
+    L.im2win_conv_kernel_name(ctypes.byref(Shape(1, 64, 1, 1, 1, 1, 1, 1, 0)), F32)
     _lib = L
     return L
 

@@ -1,7 +1,12 @@
 """Host-side rules of the kernel choice (no GPU): which fp32 kernel a layer takes, and that the scratch a caller was told
 to provide serves every smaller batch of the same layer, whatever kernel that one takes."""
+import os
+import subprocess
+import sys
+
 import pytest
 
+from conftest import ROOT
 from paper_2608_20725_b200 import binding
 
 LAYERS = [(128, 64, 56, 56, 64, 3, 3, 1, 1), (128, 512, 7, 7, 512, 3, 3, 1, 1), (13, 37, 45, 61, 75, 5, 5, 2, 2),
@@ -56,3 +61,16 @@ def test_f16_kernel_on_odd_planes(layer, want):
     ((128, 3, 224, 224, 64, 7, 7, 2, 3), "f32-split")])
 def test_f32_kernel_on_short_reductions(layer, want):
     assert binding.im2win_conv_kernel_name(layer, binding.F32) == want
+
+
+def test_switches_are_fixed_when_the_library_is_loaded():
+    """Testing-aid switches set after the library was loaded without IM2WIN_DEBUG change nothing: the library and the
+    binding, which then keeps sizes, look at it at the same moment."""
+    code = ("import os, sys; sys.path.insert(0, sys.argv[1])\n"
+            "from paper_2608_20725_b200 import binding\n"
+            "binding.lib()\n"
+            "os.environ.update(IM2WIN_DEBUG='1', IM2WIN_F32_KERNEL='ffma')\n"
+            "print(binding.im2win_conv_kernel_name((2, 64, 20, 20, 24, 3, 3, 1, 1), binding.F32))\n")
+    env = {k: v for k, v in os.environ.items() if not k.startswith("IM2WIN_")}
+    out = subprocess.run([sys.executable, "-c", code, ROOT], env=env, capture_output=True, text=True, check=True, timeout=300)
+    assert out.stdout.split() == ["f32-split"]
