@@ -458,7 +458,7 @@ def run_gpu_arm(args):
     details = {"kernels": rooflines, "memory": dict(runner.memory_report(), torch_peak_allocated_bytes=peak_alloc)}
     if rank == 0:
         if world == 1 and not args.no_per_layer:
-            # every BASELINE config, call by call (the metric is "per layer"): 20 launches each
+            # every benchmark layer, call by call (the metric is "per layer"): 20 launches each
             del runner, e2e_sets
             torch.cuda.empty_cache()
             details["per_layer"] = per_layer_summary(layer_rows(peaks, peak_kind, iters=20, with_packed=False))
@@ -537,7 +537,7 @@ def buffer_sets_for(layer):
 
 
 def layer_rows(peaks, peak_kind, names=None, iters=20, with_packed=True):
-    """Times every call of the named layers (default: all BASELINE configs) one by one: transform and
+    """Times every call of the named layers (default: all benchmark layers) one by one: transform and
     convolution (filter pack included) per precision, L2 flushed before each launch; then the same
     calls queued back to back over rotating buffer sets."""
     from paper_2608_20725_b200 import binding
@@ -613,7 +613,7 @@ def write_report(path, peaks, peak_kind, names=None, iters=20):
 
 
 def per_layer_summary(rows):
-    """The per-layer part of the details: for every BASELINE config and each of its calls the
+    """The per-layer part of the details: for every benchmark layer and each of its calls the
     device time, the bounding roofline and the fraction reached, plus the memory figures."""
     out = {}
     for row in rows:
