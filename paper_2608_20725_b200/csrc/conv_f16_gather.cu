@@ -59,7 +59,7 @@ conv_f16_gather_kernel(const __grid_constant__ CUtensorMap fmap, ConvF16Params q
   __shared__ uint32_t tmem_base_slot;
   __shared__ volatile uint32_t abort_flag;
 
-  const int warp = threadIdx.x >> 5;
+  const int warp = warp_index();
   const int lane = threadIdx.x & 31;
   const uint32_t smem_base = smem_u32(smem);
   const uint32_t full_bar0 = smem_u32(&bars[0]);

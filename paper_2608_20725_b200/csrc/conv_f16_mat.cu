@@ -154,7 +154,7 @@ __device__ __forceinline__ void conv_f16_mat_body(const CUtensorMap& fmap, const
   __shared__ Segment seg_s[NUM_WARPS][SEG_MAX];     // each warp keeps its own copy of the tile's segments
   __shared__ __align__(16) unsigned char trash[512];   // destination of matrix rows that belong to no S unit
 
-  const int warp = threadIdx.x >> 5;
+  const int warp = warp_index();
   const int lane = threadIdx.x & 31;
   // shared-memory map: filter ring (1024-byte aligned stages) | S ring | raw ring | k-block table
   const uint32_t b_ring = smem_u32(smem);

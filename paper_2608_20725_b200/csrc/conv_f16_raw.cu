@@ -127,7 +127,7 @@ conv_f16_raw_kernel(const __grid_constant__ CUtensorMap fmap, const __grid_const
   __shared__ volatile uint32_t abort_flag;
   __shared__ Segment seg_s[NUM_WARPS][SEG_MAX];     // each warp keeps its own copy of the tile's segments
 
-  const int warp = threadIdx.x >> 5;
+  const int warp = warp_index();
   const int lane = threadIdx.x & 31;
   // shared-memory map: S ring | filter ring | raw ring | k2 table
   const uint32_t a_ring = smem_u32(smem);

@@ -169,7 +169,7 @@ __global__ void __launch_bounds__(THREADS, 1) conv_f16_runs_kernel(RunsParams q)
   __shared__ uint32_t tmem_base_slot;
   __shared__ volatile uint32_t abort_flag;
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const uint32_t a_ring = smem_u32(smem);
   const uint32_t b_ring = a_ring + q.sa * q.a_stage;
   const uint32_t raw_ring = b_ring + q.sb * q.slot_bytes;

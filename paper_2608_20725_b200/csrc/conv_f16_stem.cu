@@ -187,7 +187,7 @@ conv_f16_stem_kernel(const __grid_constant__ CUtensorMap fmap, StemParams q) {
   __shared__ __align__(16) uint32_t tab_s[KB];           // k2 -> channel region + 2*u | (c*chan_stride mod 8) << 24
   __shared__ __align__(16) uint32_t zero_s[4];           // what padded k2 read
 
-  const int warp = threadIdx.x >> 5;
+  const int warp = warp_index();
   const int lane = threadIdx.x & 31;
   // shared-memory map: filter ring (1024-byte aligned stages) | S ring | raw ring
   const uint32_t b_ring = smem_u32(smem);

@@ -248,7 +248,7 @@ __global__ void __launch_bounds__(Form<BNMAX, PWG>::THREADS, 1) conv_f32_split_k
   __shared__ uint32_t tmem_base_slot;
   __shared__ volatile uint32_t abort_flag;
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const int wg = warp >> 2;
   const int sub_bytes = q.rows * 128, a_stage_bytes = 3 * sub_bytes;
   const uint32_t a_ring = smem_u32(smem);

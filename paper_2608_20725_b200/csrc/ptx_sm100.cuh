@@ -137,6 +137,12 @@ __device__ __forceinline__ void st_shared16(uint32_t addr, uint32_t a, uint32_t 
 }
 // In a kernel that may start before the one ahead of it in the stream is done: everything of that one is complete and visible.
 __device__ __forceinline__ void wait_for_previous_kernel() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// The warp's number, the same value in every lane as far as the compiler can see (a shuffle's result): the roles' branches
+// and loops then are uniform ones, and their counters and addresses stay in uniform registers instead of being handed over
+// lane by lane to every instruction that wants them uniform.  Against threadIdx.x >> 5: 7x7 stride 2 on 3 channels at 224x224,
+// fp16 135 -> 120 us, fp32 441 -> 408; 3x3 on 64 channels at 56x56 fp16 105 -> 97, fp32 218 -> 205; 3x3 on 512 channels at 7x7
+// fp32 166 -> 153 (batch 128).  The channel-innermost kernels, whose few busy warps leave the issue slots free, gain nothing.
+__device__ __forceinline__ int warp_index() { return (int)__shfl_sync(0xffffffffu, threadIdx.x >> 5, 0); }
 // True in exactly one lane of the (converged) warp.
 __device__ __forceinline__ bool elect_one() {
   uint32_t pred;
