@@ -125,7 +125,8 @@ F32Plan plan_f32(const Geometry& g);
 struct F32SplitPlan {
   bool eligible;
   int32_t Wq, rows, halo, nsub, num_kb, nks_last, nstages;
-  int32_t bn, ntn, split, sb, nwork;   // channel tile and their number, CTAs per tile, filter slots, tiles
+  int32_t bn, ntn, split, sb, nwork;   // channel tile and their number, CTAs per tile, filter slots, work items
+  int32_t n_main, parts;               // tiles from n_main on go out in parts of their channels
   int32_t packed_rows;                 // most rows (ntn * bn) of any tile width: the filter area does not depend on N
   int64_t VQ;
   size_t copy_off, filter_bytes;       // images, then a copy of the filter as given

@@ -75,8 +75,21 @@ struct SplitParams {
   int32_t K2, C, Wq, Wp, Ho, Wo, HoWo, Co, Kh, Kw, s, nsub, num_kb, nks_last;
   int32_t rows, halo;                         // rows of a sub-tile (128 + halo rounded up to 8), halo
   int32_t bn, ntn, nwork, nstages, split, sb, slot_bytes, chain;
+  int32_t n_main, parts;                      // tiles from n_main on are handed out in `parts` parts of their channels
 };
 
+
+// Work item w -> tile, first channel within it, channels.  The last round's tiles may go out in parts of their channels: no
+// sum changes.  (Pieces that lie side by side have no parts: PARTS is false.)
+struct Item {
+  int tile, first, bn;
+};
+template <bool PARTS>
+__device__ __forceinline__ Item work_item(const SplitParams& q, int w) {
+  if (!PARTS || w < q.n_main) return {w, 0, q.bn};
+  const int t = w - q.n_main, i = t / q.parts, bn = q.bn / q.parts;
+  return {q.n_main + i, (t - i * q.parts) * bn, bn};
+}
 
 // (volatile: the loads of a batch stay together, ahead of the wait for the stage they are for; left to
 // itself the compiler may move them to their uses, one round trip per eight loads)
@@ -292,7 +305,7 @@ __global__ void __launch_bounds__(Form<BNMAX, PWG>::THREADS, 1) conv_f32_split_k
     bool ok = true;
     uint32_t sc = 0;                                       // stages so far, of all producers
     for (int w = w_first; w < q.nwork && ok; w += w_step) {
-      const uint32_t q0 = (uint32_t)(w / q.ntn) * TILE_M;
+      const uint32_t q0 = (uint32_t)(work_item<!F::CONCAT>(q, w).tile / q.ntn) * TILE_M;
       // Row -> window column (class 0) and the number of classes that exist there (0 beyond the tensor).
       auto locate = [&](uint32_t vq, const float*& base, int& lim) {
         base = q.win;
@@ -366,7 +379,7 @@ __global__ void __launch_bounds__(Form<BNMAX, PWG>::THREADS, 1) conv_f32_split_k
       const bool leader = elect_one();
       const uint32_t a_lo0 = smem_desc_lo(a_ring), b_lo0 = smem_desc_lo(b_ring);
       const uint32_t sub_lo = (uint32_t)sub_bytes >> 4;
-      const uint32_t id1 = instr_desc_bf16(TILE_M, q.bn), id3 = instr_desc_bf16(TILE_M, 3 * q.bn);
+      const uint32_t id3 = instr_desc_bf16(TILE_M, 3 * q.bn);
       bool ok = true;
       uint32_t sc = 0, ac = 0;                             // stages and chains so far
       int slot = 0;
@@ -383,6 +396,7 @@ __global__ void __launch_bounds__(Form<BNMAX, PWG>::THREADS, 1) conv_f32_split_k
       };
       auto next_slot = [&](int& sl, uint32_t& ph) { if (++sl == q.sb) { sl = 0; ph ^= 1u; } };
       for (int w = w_first; w < q.nwork && ok; w += w_step) {
+        const uint32_t id1 = instr_desc_bf16(TILE_M, work_item<!F::CONCAT>(q, w).bn);
         int kb = kb0, t = t0;
         for (int st = st0; st < st1 && ok; ++st, ++sc) {
           const int buf = sc & 1;
@@ -447,8 +461,10 @@ __global__ void __launch_bounds__(Form<BNMAX, PWG>::THREADS, 1) conv_f32_split_k
       uint32_t bph = 0;
       const int per_unit = F::CONCAT ? 1 : 3;
       for (int w = w_first; w < q.nwork && ok; w += w_step) {
-        const int nt = w % q.ntn;
-        const unsigned char* tile = q.fp + (int64_t)nt * q.num_kb * q.Kw * 3 * q.bn * 128;
+        const Item it = work_item<!F::CONCAT>(q, w);
+        const int nt = it.tile % q.ntn;
+        const unsigned char* tile = q.fp + (int64_t)nt * q.num_kb * q.Kw * 3 * q.bn * 128 + (int64_t)it.first * 128;
+        const uint32_t bytes = F::CONCAT ? (uint32_t)q.slot_bytes : (uint32_t)it.bn * 128u;
         int kb = kb0, t = t0;
         for (int st = st0; st < st1 && ok; ++st) {
           for (int v = t; v < q.Kw && ok; v += q.s) {
@@ -458,9 +474,8 @@ __global__ void __launch_bounds__(Form<BNMAX, PWG>::THREADS, 1) conv_f32_split_k
               ok = __all_sync(0xffffffffu, ok);
               if (!ok) break;
               if (leader) {
-                mbar_arrive_expect_tx(b_full0 + 8 * slot, (uint32_t)q.slot_bytes);
-                bulk_load(b_ring + slot * q.slot_bytes, src + (int64_t)p * q.slot_bytes, (uint32_t)q.slot_bytes,
-                          b_full0 + 8 * slot);
+                mbar_arrive_expect_tx(b_full0 + 8 * slot, bytes);
+                bulk_load(b_ring + slot * q.slot_bytes, src + (int64_t)p * q.slot_bytes, bytes, b_full0 + 8 * slot);
               }
               __syncwarp();
               if (++slot == q.sb) { slot = 0; bph ^= 1u; }
@@ -485,8 +500,9 @@ __global__ void __launch_bounds__(Form<BNMAX, PWG>::THREADS, 1) conv_f32_split_k
     int ho = 0, i0 = 0, nt = 0;
     bool valid = false;
     for (int w = w_first; w < q.nwork && ok; w += w_step) {
-      const int mt = w / q.ntn;
-      nt = w - mt * q.ntn;
+      const Item it = work_item<!F::CONCAT>(q, w);
+      const int mt = it.tile / q.ntn;
+      nt = it.tile - mt * q.ntn;
       const uint32_t vq = (uint32_t)mt * TILE_M + (uint32_t)(lq * 32 + lane);
       valid = false;
       if (vq < q.VQ) {
@@ -532,7 +548,7 @@ __global__ void __launch_bounds__(Form<BNMAX, PWG>::THREADS, 1) conv_f32_split_k
             constexpr int STEP = BNMAX == 256 ? 1 : 2;      // chunks in flight (128 sums leave registers for one)
 #pragma unroll
             for (int j = 0; j < F::CH; j += STEP) {         // (columns beyond bn hold nothing and are not stored)
-              if ((h + 2 * j) * 16 >= q.bn) break;
+              if ((h + 2 * j) * 16 >= it.bn) break;
               uint32_t r0[16], r1[16];
               tmem_ld16_issue(d + 32 * j, r0);
               if (STEP == 2) tmem_ld16_issue(d + 32 * j + 32, r1);
@@ -566,9 +582,9 @@ __global__ void __launch_bounds__(Form<BNMAX, PWG>::THREADS, 1) conv_f32_split_k
         break;
       }
       if (valid) {
-        const int co0 = nt * q.bn;
+        const int co0 = nt * q.bn + it.first;
         float* yrow = q.y + ((int64_t)n * q.Co + co0) * q.HoWo + (int64_t)ho * q.Wo + i0;
-        const int limit = q.Co - co0 < q.bn ? q.Co - co0 : q.bn;        // channels of this tile that exist
+        const int limit = q.Co - co0 < it.bn ? q.Co - co0 : it.bn;      // channels of this item that exist
         bool again = false;
 #pragma unroll
         for (int j = 0; j < F::CH; ++j) {
@@ -695,10 +711,19 @@ int slots_for(int bn, int rows, int num_kb) {
   return n > MAX_B ? MAX_B : n;
 }
 
-// Cycles of the six products of a 128 x bn tile over 16 k (see the head of this file).
-double step_cycles(int bn) {
-  auto mma = [](int n) { const double pipe = n / 2.0, smem = 32 + n / 4.0; return pipe > smem ? pipe : smem; };
-  return bn <= CONCAT_BN ? mma(3 * bn) + 3 * mma(bn) : 6 * mma(bn);
+// Cycles of an instruction of N = n, and of the six products of a 128 x bn tile over 16 k (see the head of this file).
+double mma_cycles(int n) { const double pipe = n / 2.0, smem = 32 + n / 4.0; return pipe > smem ? pipe : smem; }
+double step_cycles(int bn) { return bn <= CONCAT_BN ? mma_cycles(3 * bn) + 3 * mma_cycles(bn) : 6 * mma_cycles(bn); }
+
+// Parts of its channels that a tile of the last round goes out in, where that round leaves half of the SMs or more idle: an
+// instruction of N = 64 takes 3/8 of the time of N = 256, so quarters save 5/8 of a round.  (5x5 on 256 channels at 28x28,
+// batch 64, 3.03 rounds of tiles: 966 -> 756 us; 7x7, 3.2 rounds: 1909 -> 1462.)
+int channel_parts(int64_t tiles, int bn) {
+  const int64_t last = tiles % 148;
+  if (last == 0 || bn <= CONCAT_BN) return 1;
+  for (int parts = 4; parts > 1; parts /= 2)
+    if (last * parts <= 148 && bn % (16 * parts) == 0) return parts;
+  return 1;
 }
 
 template <int BNMAX, int PWG>
@@ -751,16 +776,26 @@ F32SplitPlan plan_f32_split(const Geometry& g) {
     for (int z = 1; z <= 8; z *= 2) {
       if (z > p.nstages || (z > 1 && ntm * nt * z > 128)) break;     // clusters: one tile each, all resident
       if (force_z && z != atoi(force_z)) continue;
-      const int64_t rounds = z > 1 ? 1 : (ntm * nt + 147) / 148;
-      const double fill = 3.0 * bn * steps / 4 + 1200.0 * p.nstages; // shared-memory cycles of the copies and the staging
-      const double pipe = steps * step_cycles(bn), wave = pipe * 0.9 + fill;
-      const double tile = (pipe > wave ? pipe : wave) * ((p.nstages + z - 1) / z) / p.nstages + (z > 1 ? 5000 : 1500);
-      const double cost = rounds * tile + 6000;
+      auto tile_cycles = [&](int cols) {
+        // The tensor pipe, or the shared-memory pipe: operands, copies and staging.  (11x11 on 256 channels, a unit of four
+        // steps: 3126 cycles in tiles of 256 channels, 2185 in tiles of 128.)
+        const double fill = 3.0 * cols * steps / 4 + 1200.0 * p.nstages;
+        const double pipe = steps * (bn <= CONCAT_BN ? step_cycles(bn) : 6 * mma_cycles(cols));
+        const double wave = (bn <= CONCAT_BN ? pipe * 0.9 : steps * 6 * (32 + cols / 4.0)) + fill;
+        return (pipe > wave ? pipe : wave) * ((p.nstages + z - 1) / z) / p.nstages + (z > 1 ? 5000 : 1500);
+      };
+      const int64_t tiles = ntm * nt;
+      const int parts = channel_parts(tiles, bn);
+      const double cost = 6000 + (z > 1 ? tile_cycles(bn)
+                                        : (double)(tiles / 148) * tile_cycles(bn) + (tiles % 148 != 0 ? tile_cycles(bn / parts) : 0.0));
       if (!p.eligible || cost < p.cost) {
         p.eligible = true;
         p.cost = cost;
         p.bn = bn; p.ntn = nt; p.split = z; p.sb = sb;
-        p.nwork = (int32_t)((p.VQ + TILE_M - 1) / TILE_M * nt);
+        const int64_t mine = (p.VQ + TILE_M - 1) / TILE_M * nt;      // tiles of these N images
+        p.parts = z > 1 ? 1 : channel_parts(mine, bn);
+        p.n_main = (int32_t)(p.parts > 1 ? mine - mine % 148 : mine);
+        p.nwork = (int32_t)(p.n_main + (mine - p.n_main) * p.parts);
       }
     }
   }
@@ -797,7 +832,7 @@ cudaError_t launch_conv_f32_split(const float* window, float* y, void* scratch, 
   q.VQ = (uint32_t)p.VQ;
   q.K2 = g.C * g.Kh; q.C = g.C; q.Wq = p.Wq; q.Wp = g.Wp; q.Ho = g.Ho; q.Wo = g.Wo; q.HoWo = g.Ho * g.Wo; q.Co = g.Co;
   q.Kh = g.Kh; q.Kw = g.Kw; q.s = g.s; q.nsub = p.nsub; q.num_kb = p.num_kb; q.nks_last = p.nks_last;
-  q.rows = p.rows; q.halo = p.halo;
+  q.rows = p.rows; q.halo = p.halo; q.n_main = p.n_main; q.parts = p.parts;
   q.bn = p.bn; q.ntn = p.ntn; q.nwork = p.nwork; q.nstages = p.nstages; q.split = p.split;
   q.sb = p.sb; q.slot_bytes = slot_bytes_of(p.bn);
   q.chain = g.K >= 288 ? 12 : 8;
