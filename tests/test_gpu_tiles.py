@@ -1,5 +1,5 @@
 """Tiles and rounds of the convolution kernels at the sizes where their rules change: a last round in parts of the channels
-(fp32 on the tensor cores)."""
+(fp32 on the tensor cores), tiles of parts of strips (channel-innermost kernel)."""
 import numpy as np
 import pytest
 import torch
@@ -7,7 +7,7 @@ import torch
 import oracle
 from paper_2608_20725_b200 import binding, workloads
 from paper_2608_20725_b200.workloads import Layer
-from gpu_helpers import check_conv, gpu_conv
+from gpu_helpers import check_conv, gpu_conv, gpu_conv_nhwc, oracle_inputs
 
 pytestmark = pytest.mark.gpu
 
@@ -40,3 +40,23 @@ def test_f32_last_round_in_parts_of_the_channels(layer, bn, monkeypatch):
     assert np.array_equal(y[-1:], one)
     yr, ar = oracle.conv_direct(x[-1:].numpy(), f.numpy(), dict(dims, N=1))
     check_conv(one, yr, ar, "f32", layer.name)
+
+
+# reductions of 128 k-blocks of 64 and more, up to 256: strips of 28 in halves, 9 strips a tile; 27 and 30 do not divide
+@pytest.mark.parametrize("layer", [
+    L("k128", 1, 168, 28, 28, 72, 7, 7, 1, 3, 410), L("odd", 2, 165, 19, 27, 40, 7, 7, 1, 3, 411),
+    L("thirds", 1, 120, 21, 30, 130, 9, 9, 1, 4, 412), L("wide", 1, 168, 9, 60, 64, 7, 7, 1, 3, 413),
+    L("k256", 1, 256, 14, 28, 24, 8, 8, 1, 3, 414),
+    L("short", 1, 160, 28, 28, 72, 7, 7, 1, 3, 415), L("strided", 1, 168, 28, 56, 72, 7, 7, 2, 3, 416)], ids=lambda l: l.name)
+@pytest.mark.parametrize("layout", ["nchw", "nhwc"])
+def test_nhwc_tiles_of_parts_of_strips(layer, layout, monkeypatch):
+    monkeypatch.setenv("IM2WIN_NHWC_KERNEL", "overlap")
+    dims = layer.dims()
+    x, f = workloads.make_small_integer_inputs(layer)
+    yr, _ = oracle.conv_direct(x.numpy(), f.numpy(), dims)
+    y = gpu_conv_nhwc(x, f, dims, x_layout=layout)
+    assert np.array_equal(np.asarray(y).astype(np.float64), yr)
+    x, f = workloads.make_inputs(layer)
+    y = gpu_conv_nhwc(x, f, dims, x_layout=layout)
+    yr, ar = oracle.conv_direct(*oracle_inputs(x, f, "f16"), dims)
+    check_conv(y, yr, ar, "f16", layer.name)
