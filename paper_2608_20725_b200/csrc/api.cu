@@ -74,23 +74,36 @@ static bool want_f32_split(const Geometry& g, const F32SplitPlan& p) {
 }
 
 // Of the layers that neither the one-k-block kernel nor a tiled-copy kernel takes, and the shifted-view kernel could: which
-// ones the run-staged kernel gets.  Its copies are one per channel and image of a tile, so their number for each staged
+// ones the run-staged kernel gets.  Its copies are at most one per channel and image of a tile, so their number for each staged
 // element is (images of a tile) / E, with E elements per virtual column; the shifted-view kernel stages all s columns even
-// where the kernel has fewer (Kw < s).  Measured over 3090 layers (images of 5 to 35, kernels of 1 to 5, strides 1 to 3, 64
-// to 512 channels, batches 1 to 128), shifted-view time / run-staged time:
-//   stride 1, images / E up to 0.7: 1.3 with more than 148 tiles, 0.96 to 0.99 with fewer; above 0.7: 0.4 to 1.0
-//   stride 2 and more: 1.5 on average up to 0.7 (up to 2.1 with Kw < s); 0.5 to 1.3 above
-//   three virtual columns at stride 2 (5x5), more than 64 channels, at most 74 tiles: 0.9 to 1.1
-// On the 1565 layers taken 1.51 times as fast on average, 0.83 at the least (0.9 and less on 10 of them).  (256 -> 512
-// channels, 3x3 stride 2 at 28x28, batch 128: 140 -> 115 us; not taken: 3x3 on 512 channels at 7x7, batch 128, 44 us
-// against 72.)
+// where the kernel has fewer (Kw < s).  Measured over 400 layers (images of 7 to 160, kernels of 1 to 7, strides 1 and 2, 5 to
+// 512 channels, batches 1 to 128), shifted-view time / run-staged time:
+//   3x3 stride 1, images / E up to 0.7: 65 to 128 channels 1.22 to 1.66, more channels 0.92 to 1.1 with up to 148 tiles and
+//   1.1 to 1.6 with more; up to 64 channels 1.43 (1.14 at the least) where rows are staged in pairs, 1.1 (0.94) where not
+//   5x5 stride 1: 1.09 to 1.47 with more than 296 tiles, 0.7 to 1.2 with fewer; 7x7 0.84
+//   stride 2, up to 0.9: 3x3 1.62; 5x5 and 7x7 1.03 to 2.2 up to 128 channels, 0.9 to 1.1 on more with few tiles
+// (256 -> 512 channels, 3x3 stride 2 at 28x28, batch 128: 140 -> 97 us; not taken: 3x3 on 512 channels at 7x7, batch 128, 44 us
+// against 55.)
 static bool prefer_runs(const Geometry& g, const RunsPlan& p) {
-  if (p.G > 3) return false;                               // (5x5 to 11x11 with stride 1: 0.5 to 0.9)
   const int64_t per_img = (int64_t)g.Ho * p.Wq;
   const double images = 1.0 + (128.0 + p.halo) / (double)per_img;
-  if (g.s == 1) return g.Co > 64 && images <= 0.7 * p.E && p.nwork > 148;
-  if (p.G == 3 && g.s == 2 && g.Co > 64 && p.nwork <= 74) return false;
-  return images <= (g.Kw < g.s ? 2.1 : 0.7) * p.E;
+  const int64_t tiles = (int64_t)p.ntm * p.ntn;
+  if (g.s == 1) {
+    if (p.G == 5) return tiles > 296;
+    if (p.G > 3 || images > 0.7 * p.E) return false;
+    if (g.Co > 64) return g.Co <= 128 || tiles > 148;
+    return p.E == 3 && (int64_t)g.Ho * g.Wp % 2 == 0;
+  }
+  if (p.G > 4 || (p.G > 2 && g.s == 2 && g.Co > 128 && (p.G > 3 || tiles <= 74))) return false;
+  return images <= (g.Kw < g.s ? 2.1 : 0.9) * p.E;
+}
+
+// 3x3 layers of stride 1 that the tiled-copy kernels could take: the run-staged kernel below 128 channels (1.29 times as fast on
+// 23 such layers, 1.02 at the least: 3x3 on 32 channels at 112x112, batch 64, 134 -> 127 us), and from two and a half rounds
+// of tiles on also above (1.05 to 1.13 on ten layers; 0.83 to 1.07 on 19 of fewer tiles.  256 channels at 28x28, batch 64,
+// 61 -> 58 us; 64 -> 128 channels at 112x112 223 -> 194).
+static bool runs_before_tiled(const Geometry& g, const RunsPlan& p) {
+  return g.s == 1 && g.Kh == 3 && g.Kw == 3 && (g.Co < 128 || (int64_t)p.ntm * p.ntn > 370);
 }
 
 // The same layer with another batch.
@@ -160,8 +173,6 @@ im2win_status scratch_layout(const Geometry& part, im2win_dtype dtype, ScratchLa
         l->f16_shift = plan.eligible;
         l->Kp = K2p;
         l->filter_off = shift_filter_off;
-        // the bulk-copy variant shares the filter layout; IM2WIN_F16_KERNEL=shift keeps the gathering one
-        l->f16_raw = plan.eligible && plan_f16_raw(g).eligible && !(force && strcmp(force, "shift") == 0);
         // layers with one k-block: their own kernel unless another one is forced
         l->f16_stem = stem_ok && (!force || strcmp(force, "stem") == 0);
       }
@@ -173,10 +184,19 @@ im2win_status scratch_layout(const Geometry& part, im2win_dtype dtype, ScratchLa
     // above 128); IM2WIN_F16_KERNEL=mat forces it wherever it can run (a testing aid)
     const bool want = force ? strcmp(force, "mat") == 0 : (g.s > 1 || (g.Co >= 128 && g.Kw <= 5));
     l->f16_mat = mat.eligible && want && !l->f16_stem;
+    const RunsPlan runs = plan_f16_runs(g);
+    // (planes that are a multiple of 16 bytes: what the tiled-copy kernels need)
+    if (!force && runs.eligible && !l->f16_stem && (g.chan_stride * 2) % 16 == 0 && runs_before_tiled(g, runs)) {
+      l->f16_runs = true;
+      l->f16_mat = false;
+    }
+    // the bulk-copy variant shares the filter layout of the shifted-view kernel; IM2WIN_F16_KERNEL=shift keeps the gathering one
+    // (its plan walks over the tiles of an image: last)
+    if (l->f16_shift && !l->f16_stem && !l->f16_mat && !l->f16_runs && !(force && strcmp(force, "shift") == 0))
+      l->f16_raw = plan_f16_raw(g).eligible;
     const MatPlan any_mat = plan_for_any_batch(mat, plan_f16_mat, g);
     if (any_mat.eligible) most = std::max(most, (int64_t)any_mat.scratch_bytes);
-    const RunsPlan runs = plan_f16_runs(g);
-    if (runs.eligible) {
+    if (runs.eligible && !l->f16_runs) {
       const bool rest = !l->f16_stem && !l->f16_mat && !l->f16_raw;
       l->f16_runs = force ? strcmp(force, "runs") == 0 : rest && (!l->f16_shift || prefer_runs(g, runs));
     }

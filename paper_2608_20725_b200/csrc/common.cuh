@@ -136,10 +136,10 @@ F32SplitPlan plan_f32_split(const Geometry& g);
 
 // Tile and ring geometry of the run-staged kernel (see conv_f16_runs.cu).
 struct RunsPlan {
-  bool eligible, resident, quad;       // quad: up to four channels, see the order of k2 there
+  bool eligible, resident, quad, pair; // quad: up to four channels, see the order of k2 there; pair: CTA pairs
   int32_t units, octs, E, G, Wq, rows, halo, num_kb, nks_last;
-  int32_t region, raw_slot, a_stage, slot_bytes;
-  int32_t bn, ntn, nwork, sa, sr, sb;
+  int32_t region, raw_slot, a_stage, slot_bytes, cols, planes, seg_bytes;
+  int32_t bn, ntn, ntm, nwork, sa, sr, sb;
   int64_t VQ;
   size_t filter_bytes;
 };

@@ -1,6 +1,7 @@
 // fp16-input / fp32-accumulate im2win convolution with the window tensor brought in as contiguous runs.  It needs no
 // alignment of planes, strips or images and takes every stride: the layers whose plane pitch is no multiple of 16
-// bytes, which conv_f16_mat.cu and conv_f16_raw.cu cannot bring in with tiled copies.
+// bytes, which conv_f16_mat.cu and conv_f16_raw.cu cannot bring in with tiled copies, and the 3x3 layers of stride 1 on which it
+// is the faster one (runs_before_tiled in api.cu).
 //
 // Columns.  In the im2win tensor the s*Kh elements of columns i*s .. i*s + s - 1 of a strip are contiguous, so a
 // convolution of stride s is one of stride 1 on columns s times as tall: virtual column i holds e = t*Kh + u
@@ -15,18 +16,25 @@
 // eight planes further the phase repeats -- and a unit costs a thread eight 2-byte shared loads, four packs and one
 // store.
 //
-// Staging.  The columns a tile needs of one channel are one contiguous run per image it touches: an untiled bulk
-// copy from the 16-byte boundary below to the one above brings it into a ring of raw slots (`octs` octets of
-// channels each).  Two warpgroups take the units in turn, read the elements of their rows back (thread = row) and
-// write the units of S.  Gathering with 2-byte global loads instead (conv_f16_shift.cu) makes every load instruction
+// Raw copies.  The columns a tile needs of one channel are one contiguous run per image it touches.  An untiled bulk copy
+// brings a run from the 16-byte boundary below to the one above into a ring of raw slots (`octs` octets of channels
+// each); or, where 1, 2 or 4 channel planes are a multiple of 16 bytes and a tile touches at most two images, a tiled copy brings
+// the same run of every first, second or fourth channel of an octet (a copy costs the copy engine about 100 cycles, whatever
+// its size).  Gathering with 2-byte global loads instead (conv_f16_shift.cu) makes every load instruction
 // touch 32 rows s*Kh elements apart: three or more L1 wavefronts each, and a round trip to memory per batch.
 //
-// What bounds it: the staging warps' read-back (without it 89 us where the whole takes 107) and the shared-memory pipe,
-// which carries the MMA's operand reads (32 + N/4 cycles per instruction of M = 128, K = 16), the copies, the read-back
-// and the S stores.  Measured against the gathering kernel: 3x3 stride 2 on 256 -> 512 channels at 28x28, batch 128,
-// 140 -> 115 us (515 TFLOP/s); 5x5 stride 2 on 37 -> 75 channels at 45x61, batch 13, 27 -> 17 us.  Eight staging warps and
-// not sixteen (128 us): more of them take issue slots from the MMA warp.
+// Above 128 channels two CTAs form a pair (M = 256, cta_group::2): each stages its own position tile and half of the filter,
+// and the second CTA's MMA warp tells the leader that its half of a filter slot has arrived.
+//
+// What bounds it: no single pipe.  With the read-back, the S stores, the MMAs and the output stores all left out, what remains
+// (copies, hand-offs, the staging warps' arithmetic) still takes four fifths of the time: 86 of 109 us for 3x3 on 64 channels at
+// 56x56, batch 128.  Measured: 3x3 stride 2 on 256 -> 512 channels at 28x28, batch 128, 140 us with the gathering kernel,
+// 112 with a unit at a time, no pairs and two S stages, now 97 (610 TFLOP/s); 3x3 on 256 channels at 28x28, batch 64, 70 -> 58;
+// 64 -> 128 channels at 112x112, batch 64, 256 -> 194; 5x5 stride 2 on 37 -> 75 channels at 45x61, batch 13, 27 (gathering) and 15.
+// Eight staging warps: twelve or sixteen, with four epilogue warps, gave 111 and 117 us where eight gave 113, and 115 and 125 us
+// where eight gave 103.
 #include <cuda_fp16.h>
+#include <cuda.h>
 #include <stdlib.h>
 #include <string.h>
 
@@ -59,7 +67,8 @@ FastDiv fast_div(uint32_t d) {
   return {(uint32_t)((((uint64_t)1 << (31 + l)) / d) + 1), 31 + l};
 }
 
-struct RunsParams {
+struct alignas(64) RunsParams {
+  CUtensorMap map;                            // window tensor in rows of `planes` channel planes (tiled raw copies)
   const unsigned char* __restrict__ win;
   const unsigned char* __restrict__ fp;       // packed filter: shared-memory images, see pack_f16_runs_kernel
   float* __restrict__ y;
@@ -70,9 +79,14 @@ struct RunsParams {
   int32_t C, Wp, Wq, Ho, Wo, HoWo, Co, Kh, Kw, s;
   int32_t E, G, units, num_kb, nks_last;      // units: of eight k2
   int32_t quad;                               // 1: up to four channels, a unit is four channels at two e
+  int32_t mode;                               // how the staging warps read the raw runs (StagingMode)
   int32_t foreign;                            // 1: zero filter elements meet elements that are not of the window
   int32_t halo, region, octs, raw_slot, a_stage;
   int32_t bn, ntn, nwork, sa, sr, sb, slot_bytes, resident;
+  int32_t cols;                               // kernel columns in a filter slot
+  int32_t ntm;                                // position tiles
+  int32_t planes;                             // the least number of channel planes that is a multiple of 16 bytes; 0: bulk copies
+  int32_t seg_bytes;                          // tiled copies: from image to image of a tile in a raw slot
 };
 
 __device__ __forceinline__ uint32_t ld_shared_u16(uint32_t addr) {
@@ -80,8 +94,13 @@ __device__ __forceinline__ uint32_t ld_shared_u16(uint32_t addr) {
   asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(addr) : "memory");
   return v;
 }
+__device__ __forceinline__ uint32_t ld_shared_u32(uint32_t addr) {
+  uint32_t v;
+  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+  return v;
+}
 constexpr int ES = 2;                         // bytes of an element
-constexpr int REGS_STAGING = 80, REGS_MISC = 64, REGS_EPILOGUE = 128;   // 2*80 + 64 + 2*128 = 5*96
+constexpr int REGS_STAGING = 96, REGS_MISC = 64, REGS_EPILOGUE = 112;   // 2*96 + 64 + 2*112 = 5*96
 
 // Where the rows of a tile lie: image n0 + g of the tile is a run of its own, [start, end) in elements of a channel
 // plane, at byte seg_off(g) of a channel's region in a raw slot.
@@ -153,15 +172,238 @@ __device__ __noinline__ void exact_outputs(const unsigned char* __restrict__ x, 
   }
 }
 
-// The MMAs of one kernel column, straight-line: a lone lane pays for every branch and address computation between them.
-template <int NKS>
-__device__ __forceinline__ void issue_column(uint32_t d, uint32_t a, uint32_t b, uint32_t idesc, uint32_t more) {
+// The MMAs of COLS kernel columns, straight-line: a lone lane pays for every branch and address computation between them.
+template <int NKS, int COLS, bool PAIR>
+__device__ __forceinline__ void issue_columns(uint32_t d, uint32_t a, uint32_t b, uint32_t b_step, uint32_t idesc, uint32_t more) {
 #pragma unroll
-  for (int j = 0; j < NKS; ++j) umma_f16_lohi(d, a + 2 * j, b + 2 * j, idesc, j == 0 ? more : 1u);
+  for (int g = 0; g < COLS; ++g, b += b_step)              // next view: one row (128 bytes) further down
+#pragma unroll
+    for (int j = 0; j < NKS; ++j) {
+      const uint32_t acc = g == 0 && j == 0 ? more : 1u;
+      if (PAIR) umma_f16_ab_pair(d, a + 8 * g + 2 * j, kSmemDescHiSw128, b + 2 * j, kSmemDescHiSw128, idesc, acc);
+      else umma_f16_lohi(d, a + 8 * g + 2 * j, b + 2 * j, idesc, acc);
+    }
+}
+template <int COLS, bool PAIR>
+__device__ __forceinline__ void issue_slot(int nks, uint32_t d, uint32_t a, uint32_t b, uint32_t b_step, uint32_t idesc, uint32_t more) {
+  if (nks == KB / 16) issue_columns<KB / 16, COLS, PAIR>(d, a, b, b_step, idesc, more);
+  else if (nks == 3) issue_columns<3, COLS, PAIR>(d, a, b, b_step, idesc, more);
+  else if (nks == 2) issue_columns<2, COLS, PAIR>(d, a, b, b_step, idesc, more);
+  else issue_columns<1, COLS, PAIR>(d, a, b, b_step, idesc, more);
 }
 
-template <int BNMAX>
-__global__ void __launch_bounds__(THREADS, 1) conv_f16_runs_kernel(RunsParams q) {
+// The work items of a CTA: items first, first + step, ...; an item is a channel tile of one position tile, or of two for a
+// CTA pair (of an odd number of position tiles the last is staged by both and stored by one).
+struct Walk {
+  int first, step, rank, pair;
+  __device__ __forceinline__ int tile(const RunsParams& q, int w) const { return pair ? 2 * (w / q.ntn) + rank : w / q.ntn; }
+  __device__ __forceinline__ uint32_t start(const RunsParams& q, int w) const {
+    const int mt = tile(q, w);
+    return (uint32_t)(mt < q.ntm ? mt : q.ntm - 1) * TILE_M;
+  }
+};
+
+// The staging warps: raw runs -> S, thread = row (or two neighbouring rows).
+//   HALVES     an element at a time: any alignment
+//   QUAD       the same with units of four channels at two e (up to four channels)
+//   WORDS      two elements of a row at a time: E even and every row on a 4-byte boundary (strides of 2)
+//   ROW_PAIRS  rows 2t and 2t + 1 of a 3-high kernel at stride 1 are six neighbouring elements, read as three words: images
+//              of an even number of virtual columns, so that no pair lies in two images
+// A team of warps covers the rows of the tile and takes every TEAMS-th slot as a whole; all loads of up to GROUP units
+// are in flight together, and the slot is given back before the wait for a free S stage.  (A unit at a time, both
+// warpgroups on every slot, took 87 instructions and 560 cycles a unit: 3x3 stride 2 on 256 -> 512 channels at 28x28, batch
+// 128, 121 us.)
+// Where channel x of an octet lies in a raw slot: tiled copies bring every `planes`-th channel at a time.
+__device__ __forceinline__ int slot_row(const RunsParams& q, int x) {
+  if (q.planes <= 1) return x;
+  return q.planes == 2 ? (x & 1) * 4 + (x >> 1) : (x & 3) * 2 + (x >> 2);
+}
+
+enum StagingMode { HALVES, QUAD, WORDS, ROW_PAIRS };
+
+struct StagingBarriers {
+  uint32_t a_full0, a_empty0, raw_full0, raw_empty0;        // (a_full0 in a pair: the leader's, wherever it lies)
+};
+
+template <int MODE, bool PAIR>
+__device__ __forceinline__ void stage_tiles(const RunsParams& q, const Walk& walk, uint32_t a_ring, uint32_t raw_ring,
+                                            const StagingBarriers& b, int warp, int lane, volatile uint32_t* abort_flag) {
+  auto arrive_full = [&](int stage) {
+    if (PAIR) mbar_arrive_cluster(b.a_full0 + 8 * stage);
+    else mbar_arrive(b.a_full0 + 8 * stage);
+  };
+  constexpr int ROWS = MODE == ROW_PAIRS ? 2 : 1;
+  constexpr int TEAM = 4 / ROWS, TEAMS = STAGING_WARPS / TEAM;
+  constexpr int GROUP = MODE == WORDS ? 6 : 3;              // units in flight
+  constexpr uint32_t STEP = MODE == QUAD ? 2 * ES : ES;     // from unit to unit of an octet, in a channel plane
+  const int team = warp / TEAM, row = ((warp % TEAM) * 32 + lane) * ROWS;
+  const int plane = (q.Ho * q.Wp + q.Wq * q.s - q.Wp) * q.Kh;     // (up to the end of the last virtual column)
+  const int per_oct = MODE == QUAD ? q.units : q.E;
+  const int nocts = MODE == QUAD ? 1 : q.units / q.E, octs = MODE == QUAD ? 1 : q.octs;
+  const int nslots = (nocts + octs - 1) / octs;
+  auto swizzled = [](int r) { return (uint32_t)(r * 128 + ((r & 7) << 4)); };
+  // (lanes 4 to 7 of eight store the second row of a pair first: the eight meet eight bank groups)
+  const int second = ROWS == 2 ? (lane >> 2) & 1 : 0;
+  const uint32_t dst0 = swizzled(row + second), dst1 = ROWS == 2 ? swizzled(row + 1 - second) : 0u;
+  // rows below the tile: lane -> (row, unit of the group); one warp of the team has them, another one from slot to slot
+  const bool halo_fits = q.halo * GROUP <= 32;
+  bool ok = true;
+  // No more teams than raw slots: a team's next slot then reuses a buffer that was filled, for another team, before its last
+  // one was, and the parity it waits for is not that of two fills ago.
+  const int teams = q.sr < TEAMS ? q.sr : TEAMS;
+  int sa = 0, sr = team, next = team < teams ? team : 1 << 30;    // (next: this team's next slot of the tile)
+  uint32_t pa = 0, pr = 0;
+  uint32_t turn = 0;
+  for (int w = walk.first; w < q.nwork && ok; w += walk.step) {
+    const uint32_t q0 = walk.start(q, w);
+    const TileRuns tr = tile_runs(q, q0);
+    // Place of row r's first element in channel x of a slot's octet: byte inside the raw slot.
+    auto locate = [&](int r, uint32_t (&rb)[8]) {
+      uint32_t off = 0, phase = 0;
+      const uint32_t vq = q0 + r;
+      if (vq < q.VQ) {                                       // dead rows read whatever lies at the start: they are dropped
+        uint32_t n;
+        int ho, i;
+        split_q(q, vq, n, ho, i);
+        const int g = (int)(n - tr.n0), start = g == 0 ? tr.start0 : 0;
+        if (q.planes) off = g * q.seg_bytes;
+        else if (g > 0) off = run_size(plane - tr.start0) + (g - 1) * run_size(plane);
+        off += ((ho * q.Wp + i * q.s) * q.Kh - start) * ES;
+        phase = (uint32_t)((int64_t)n * q.img_bytes + (int64_t)start * ES);
+      }
+#pragma unroll
+      for (int x = 0; x < 8; ++x) rb[x] = off + slot_row(q, x) * q.region + ((phase + (uint32_t)x * (uint32_t)q.chan_bytes) & 15u);
+      if (MODE == QUAD) {
+#pragma unroll
+        for (int x = 0; x < 4; ++x) rb[4 + x] = rb[x] + ES;
+      }
+    };
+    uint32_t rb[8], hb[8];
+    locate(row, rb);
+    const int he = q.halo > 0 && halo_fits ? lane / q.halo : GROUP, hrow = TILE_M + lane - he * q.halo;
+    if (he < GROUP) {
+      locate(hrow, hb);
+#pragma unroll
+      for (int x = 0; x < 8; ++x) hb[x] += he * STEP;
+    }
+    int kb = 0;                                              // S stage this warp is at, and whether it may write to it
+    bool held = false;
+    auto go_to = [&](int target) {
+      while (ok && !(held && kb == target)) {
+        if (!held) {
+          ok = mbar_wait(b.a_empty0 + 8 * sa, pa ^ 1u, abort_flag, q.status);
+          ok = __all_sync(0xffffffffu, ok);
+          held = true;
+        } else {
+          fence_proxy_async_smem();
+          __syncwarp();
+          if (lane == 0) arrive_full(sa);
+          if (++sa == q.sa) { sa = 0; pa ^= 1u; }
+          ++kb;
+          held = false;
+        }
+      }
+    };
+    for (; next < nslots && ok; next += teams, ++turn) {
+      ok = mbar_wait(b.raw_full0 + 8 * sr, pr, abort_flag, q.status);
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) break;
+      uint32_t src = raw_ring + sr * q.raw_slot;
+      const bool halo_turn = q.halo > 0 && (int)(turn % TEAM) == warp % TEAM;
+      const int here = nocts - next * octs < octs ? nocts - next * octs : octs;
+      int j = next * octs * per_oct;                         // unit
+      for (int o = 0; o < here && ok; ++o, src += 8u * q.region) {
+        for (int e0 = 0; e0 < per_oct && ok; e0 += GROUP) {
+          const int n = per_oct - e0 < GROUP ? per_oct - e0 : GROUP;
+          const uint32_t at = src + e0 * STEP;
+          uint32_t p[GROUP * ROWS][4], hp[4] = {};
+          if constexpr (MODE == WORDS || MODE == ROW_PAIRS) {
+            uint32_t v[3][8];                                // (beyond the octet's last unit: place 0 again)
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+              const uint32_t from = MODE == ROW_PAIRS || 2 * i < n ? at + 4 * i : at;
+#pragma unroll
+              for (int x = 0; x < 8; ++x) v[i][x] = ld_shared_u32(from + rb[x]);
+            }
+#pragma unroll
+            for (int i = 0; i < 6; ++i)
+#pragma unroll
+              for (int x = 0; x < 4; ++x)
+                p[i][x] = __byte_perm(v[i / 2][2 * x], v[i / 2][2 * x + 1], (i & 1) ? 0x7632 : 0x5410);
+          } else {
+            uint32_t v[GROUP][8];
+#pragma unroll
+            for (int i = 0; i < GROUP; ++i) {
+              const uint32_t from = i < n ? at + i * STEP : at;
+#pragma unroll
+              for (int x = 0; x < 8; ++x) v[i][x] = ld_shared_u16(from + rb[x]);
+            }
+#pragma unroll
+            for (int i = 0; i < GROUP; ++i)
+#pragma unroll
+              for (int x = 0; x < 4; ++x) p[i][x] = __byte_perm(v[i][2 * x], v[i][2 * x + 1], 0x5410);
+          }
+          if (halo_turn && he < n) {
+#pragma unroll
+            for (int x = 0; x < 4; ++x)
+              hp[x] = __byte_perm(ld_shared_u16(at + hb[2 * x]), ld_shared_u16(at + hb[2 * x + 1]), 0x5410);
+          }
+          if (halo_turn && !halo_fits) {                     // many rows below the tile: unit by unit, lane = row
+            for (int i = 0; i < n && ok; ++i) {
+              go_to((j + i) >> 3);
+              if (!ok || lane >= q.halo) continue;
+              uint32_t lb[8], lp[4];
+              locate(TILE_M + lane, lb);
+#pragma unroll
+              for (int x = 0; x < 4; ++x)
+                lp[x] = __byte_perm(ld_shared_u16(at + i * STEP + lb[2 * x]), ld_shared_u16(at + i * STEP + lb[2 * x + 1]), 0x5410);
+              st_shared16(a_ring + sa * q.a_stage + (swizzled(TILE_M + lane) ^ (((j + i) & 7) << 4)), lp[0], lp[1], lp[2], lp[3]);
+            }
+            __syncwarp();
+          }
+          if (o == here - 1 && e0 + GROUP >= per_oct) {      // everything of the slot is in registers
+            __syncwarp();
+            if (lane == 0) mbar_arrive(b.raw_empty0 + 8 * sr);
+          }
+#pragma unroll
+          for (int i = 0; i < GROUP; ++i) {
+            if (i >= n) break;
+            go_to((j + i) >> 3);
+            if (!ok) break;
+            const uint32_t stage = a_ring + sa * q.a_stage, ch = (uint32_t)((j + i) & 7) << 4;
+            if constexpr (ROWS == 2) {
+              const uint32_t (&r0)[4] = p[i], (&r1)[4] = p[3 + i];
+              st_shared16(stage + (dst0 ^ ch), second ? r1[0] : r0[0], second ? r1[1] : r0[1], second ? r1[2] : r0[2], second ? r1[3] : r0[3]);
+              st_shared16(stage + (dst1 ^ ch), second ? r0[0] : r1[0], second ? r0[1] : r1[1], second ? r0[2] : r1[2], second ? r0[3] : r1[3]);
+            } else {
+              st_shared16(stage + (dst0 ^ ch), p[i][0], p[i][1], p[i][2], p[i][3]);
+            }
+            if (halo_turn && he == i) st_shared16(stage + (swizzled(hrow) ^ ch), hp[0], hp[1], hp[2], hp[3]);
+          }
+          j += n;
+        }
+      }
+      sr += teams;
+      if (sr >= q.sr) { sr -= q.sr; pr ^= 1u; }
+    }
+    if (team < teams) next -= nslots;
+    go_to(q.num_kb - 1);
+    if (!ok) break;
+    if ((q.units & 1) != 0 && team == 0) {                   // zeros up to the end of the MMA's last step
+      const uint32_t stage = a_ring + sa * q.a_stage, ch = (uint32_t)(q.units & 7) << 4;
+      st_shared16(stage + (dst0 ^ ch), 0u, 0u, 0u, 0u);
+      if (ROWS == 2) st_shared16(stage + (dst1 ^ ch), 0u, 0u, 0u, 0u);
+      if (warp == 0 && lane < q.halo) st_shared16(stage + (swizzled(TILE_M + lane) ^ ch), 0u, 0u, 0u, 0u);
+    }
+    fence_proxy_async_smem();
+    __syncwarp();
+    if (lane == 0) arrive_full(sa);
+    if (++sa == q.sa) { sa = 0; pa ^= 1u; }
+  }
+}
+
+template <int BNMAX, bool PAIR>
+__global__ void __launch_bounds__(THREADS, 1) conv_f16_runs_kernel(const __grid_constant__ RunsParams q) {
   constexpr int NACC = 512 / BNMAX, ACC_LOG = NACC == 2 ? 1 : (NACC == 4 ? 2 : 3);      // ring of accumulators in tensor memory
   extern __shared__ unsigned char smem_dyn[];
   unsigned char* smem = reinterpret_cast<unsigned char*>(((uintptr_t)smem_dyn + 1023) & ~(uintptr_t)1023);
@@ -177,22 +419,34 @@ __global__ void __launch_bounds__(THREADS, 1) conv_f16_runs_kernel(RunsParams q)
   const uint32_t raw_full0 = a_empty0 + 8 * MAX_A, raw_empty0 = raw_full0 + 8 * MAX_RAW;
   const uint32_t b_full0 = raw_empty0 + 8 * MAX_RAW, b_empty0 = b_full0 + 8 * MAX_B;
   const uint32_t acc_full0 = b_empty0 + 8 * MAX_B, acc_empty0 = acc_full0 + 8 * MAX_ACC;
+  const int rank = PAIR ? (int)cluster_ctarank() : 0;
+  const Walk walk = {PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x, PAIR ? (int)(gridDim.x >> 1) : (int)gridDim.x, rank, PAIR};
+  // the leader's barriers that both CTAs of a pair arrive on
+  const uint32_t a_full_dst = PAIR ? mapa_shared(a_full0, 0) : a_full0;
+  const uint32_t b_full_dst = PAIR ? mapa_shared(b_full0, 0) : b_full0;
+  const uint32_t acc_empty_dst = PAIR ? mapa_shared(acc_empty0, 0) : acc_empty0;
+  const int b_rows = PAIR ? q.bn / 2 : q.bn;               // filter rows (channels) this CTA holds of a kernel column
 
   if (threadIdx.x == 0) {
     abort_flag = 0u;
-    for (int i = 0; i < MAX_A; ++i) { mbar_init(a_full0 + 8 * i, STAGING_WARPS); mbar_init(a_empty0 + 8 * i, 1); }
-    for (int i = 0; i < MAX_RAW; ++i) { mbar_init(raw_full0 + 8 * i, 1); mbar_init(raw_empty0 + 8 * i, STAGING_WARPS); }
-    for (int i = 0; i < MAX_B; ++i) { mbar_init(b_full0 + 8 * i, 1); mbar_init(b_empty0 + 8 * i, 1); }
-    for (int i = 0; i < MAX_ACC; ++i) { mbar_init(acc_full0 + 8 * i, 1); mbar_init(acc_empty0 + 8 * i, 8); }
+    for (int i = 0; i < MAX_A; ++i) { mbar_init(a_full0 + 8 * i, PAIR ? 2 * STAGING_WARPS : STAGING_WARPS); mbar_init(a_empty0 + 8 * i, 1); }
+    for (int i = 0; i < MAX_RAW; ++i) { mbar_init(raw_full0 + 8 * i, 1); mbar_init(raw_empty0 + 8 * i, q.mode == ROW_PAIRS ? 2 : 4); }
+    // (the leader's b_full: its own copy and word from the other CTA's)
+    for (int i = 0; i < MAX_B; ++i) { mbar_init(b_full0 + 8 * i, PAIR && rank == 0 ? 2 : 1); mbar_init(b_empty0 + 8 * i, 1); }
+    for (int i = 0; i < MAX_ACC; ++i) { mbar_init(acc_full0 + 8 * i, 1); mbar_init(acc_empty0 + 8 * i, PAIR ? 16 : 8); }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == STAGING_WARPS) tmem_alloc(smem_u32(&tmem_base_slot), 512);
+  if (warp == STAGING_WARPS) {
+    if (PAIR) tmem_alloc_pair(smem_u32(&tmem_base_slot), 512);
+    else tmem_alloc(smem_u32(&tmem_base_slot), 512);
+  }
   // The raw ring starts as zeros: places no copy fills (channels beyond C in the last octet) meet zero filter
   // elements, but they have to be numbers.
   for (int i = threadIdx.x * 16; i < q.sr * q.raw_slot; i += THREADS * 16) st_shared16(raw_ring + i, 0u, 0u, 0u, 0u);
   fence_proxy_async_smem();
   tc_fence_before();
   __syncthreads();
+  if (PAIR) cluster_sync_all();                             // the peer's barriers exist before anything arrives on them
   tc_fence_after();
   const uint32_t tmem_acc = tmem_base_slot;
   wait_for_previous_kernel();
@@ -200,97 +454,18 @@ __global__ void __launch_bounds__(THREADS, 1) conv_f16_runs_kernel(RunsParams q)
   if (warp < STAGING_WARPS) {
     // ---------------- staging: raw runs -> S ------------------------------------------------------------
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_STAGING));
-    // Warpgroup wg takes every second unit.  Every warp passes every stage and every slot in order, so
-    // no wait by phase parity can run ahead.
-    const int wg = warp >> 2, row = threadIdx.x & 127;
-    const int plane = (q.Ho * q.Wp + q.Wq * q.s - q.Wp) * q.Kh;   // (up to the end of the last virtual column)
-    const int per_slot = q.quad ? q.units : q.octs * q.E;
-    const uint32_t oct_step = 8u * q.region - (uint32_t)(q.E - 1) * ES, unit_step = q.quad ? 2u * ES : ES;
-    bool ok = true;
-    int sa = 0, sr = 0;
-    uint32_t pa = 0, pr = 0;
-    for (int w = blockIdx.x; w < q.nwork && ok; w += gridDim.x) {
-      const uint32_t q0 = (uint32_t)(w / q.ntn) * TILE_M;
-      const TileRuns tr = tile_runs(q, q0);
-      // Place of row r's first element in channel x of a slot's octet: byte inside the raw slot.
-      auto locate = [&](int r, uint32_t (&rb)[8]) {
-        uint32_t off = 0, phase = 0;
-        const uint32_t vq = q0 + r;
-        if (vq < q.VQ) {                                     // dead rows read whatever lies at the start: they are dropped
-          uint32_t n;
-          int ho, i;
-          split_q(q, vq, n, ho, i);
-          const int g = (int)(n - tr.n0), start = g == 0 ? tr.start0 : 0;
-          if (g > 0) off = run_size(plane - tr.start0) + (g - 1) * run_size(plane);
-          off += ((ho * q.Wp + i * q.s) * q.Kh - start) * ES;
-          phase = (uint32_t)((int64_t)n * q.img_bytes + (int64_t)start * ES);
-        }
-#pragma unroll
-        for (int x = 0; x < 8; ++x) rb[x] = off + x * q.region + ((phase + (uint32_t)x * (uint32_t)q.chan_bytes) & 15u);
-        if (q.quad) {
-#pragma unroll
-          for (int x = 0; x < 4; ++x) rb[4 + x] = rb[x] + ES;
-        }
-      };
-      uint32_t rb[8], hb[8];
-      locate(row, rb);
-      if (lane < q.halo) locate(TILE_M + lane, hb);
-      uint32_t src = 0;                                      // of the current unit; inside the slot: its number, and its e
-      int in_slot = 0, e = 0;
-      for (int kb = 0; kb < q.num_kb && ok; ++kb) {
-        ok = mbar_wait(a_empty0 + 8 * sa, pa ^ 1u, &abort_flag, q.status);
-        ok = __all_sync(0xffffffffu, ok);
-        if (!ok) break;
-        const uint32_t stage = a_ring + sa * q.a_stage;
-        const int n_units = q.units - 8 * kb < 8 ? q.units - 8 * kb : 8;
-        for (int ch = 0; ch < n_units; ++ch) {
-          if (in_slot == 0) {
-            ok = mbar_wait(raw_full0 + 8 * sr, pr, &abort_flag, q.status);
-            ok = __all_sync(0xffffffffu, ok);
-            if (!ok) break;
-            src = raw_ring + sr * q.raw_slot;
-            e = 0;
-          }
-          if ((ch & 1) == wg) {
-            auto unit = [&](const uint32_t (&at)[8], int srow) {
-              uint32_t v[8];
-#pragma unroll
-              for (int x = 0; x < 8; ++x) v[x] = ld_shared_u16(src + at[x]);
-              st_shared16(stage + srow * 128 + ((ch ^ (srow & 7)) << 4), v[0] | (v[1] << 16), v[2] | (v[3] << 16),
-                          v[4] | (v[5] << 16), v[6] | (v[7] << 16));
-            };
-            unit(rb, row);
-            // the rows below the tile: lanes of one of the warpgroup's warps, another one from unit to unit
-            if ((ch >> 1) == (warp & 3) && lane < q.halo) unit(hb, TILE_M + lane);
-          }
-          if (++in_slot == per_slot || 8 * kb + ch == q.units - 1) {
-            __syncwarp();
-            if (lane == 0) mbar_arrive(raw_empty0 + 8 * sr);
-            if (++sr == q.sr) { sr = 0; pr ^= 1u; }
-            in_slot = 0;
-          }
-          ++e;
-          src += e == q.E ? oct_step : unit_step;
-          if (e == q.E) e = 0;
-        }
-        if (!ok) break;
-        if ((n_units & 1) != 0 && wg == 1) {                 // zeros up to the end of the MMA's last step
-          st_shared16(stage + row * 128 + ((n_units ^ (row & 7)) << 4), 0u, 0u, 0u, 0u);
-          if (lane < q.halo) st_shared16(stage + (TILE_M + lane) * 128 + ((n_units ^ (lane & 7)) << 4), 0u, 0u, 0u, 0u);
-        }
-        fence_proxy_async_smem();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(a_full0 + 8 * sa);
-        if (++sa == q.sa) { sa = 0; pa ^= 1u; }
-      }
-    }
+    const StagingBarriers b = {a_full_dst, a_empty0, raw_full0, raw_empty0};
+    if (q.mode == ROW_PAIRS) stage_tiles<ROW_PAIRS, PAIR>(q, walk, a_ring, raw_ring, b, warp, lane, &abort_flag);
+    else if (q.mode == WORDS) stage_tiles<WORDS, PAIR>(q, walk, a_ring, raw_ring, b, warp, lane, &abort_flag);
+    else if (q.mode == QUAD) stage_tiles<QUAD, PAIR>(q, walk, a_ring, raw_ring, b, warp, lane, &abort_flag);
+    else stage_tiles<HALVES, PAIR>(q, walk, a_ring, raw_ring, b, warp, lane, &abort_flag);
   } else if (warp < STAGING_WARPS + 4) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_MISC));
-    if (warp == STAGING_WARPS) {
-      // ---------------- MMA issuer -----------------------------------------------------------------------
+    if (warp == STAGING_WARPS && rank == 0) {
+      // ---------------- MMA issuer (the leader of a pair) -----------------------------------------------------------------------
       const bool leader = elect_one();
       const uint32_t a_lo0 = smem_desc_lo(a_ring), b_lo0 = smem_desc_lo(b_ring);
-      const uint32_t idesc = instr_desc_f16(TILE_M, q.bn);
+      const uint32_t idesc = instr_desc_f16(PAIR ? 2 * TILE_M : TILE_M, q.bn), b_step = (uint32_t)b_rows * 8u;
       bool ok = true;
       int sa = 0, slot = 0;
       uint32_t pa = 0, pb = 0, ac = 0;                       // ... tiles so far
@@ -303,13 +478,17 @@ __global__ void __launch_bounds__(THREADS, 1) conv_f16_runs_kernel(RunsParams q)
       auto need = [&](uint32_t bar, uint32_t parity, uint32_t seen) {
         return mbar_wait_unless_seen(bar, parity, seen, &abort_flag, q.status);
       };
-      for (int w = blockIdx.x; w < q.nwork && ok; w += gridDim.x, ++ac) {
+      auto commit = [&](uint32_t bar) {
+        if (PAIR) umma_commit_pair(bar);
+        else umma_commit(bar);
+      };
+      for (int w = walk.first; w < q.nwork && ok; w += walk.step, ++ac) {
         const int ab = ac & (NACC - 1);
         ok = need(acc_empty0 + 8 * ab, ((ac >> ACC_LOG) & 1) ^ 1, acc_seen);
         if (!ok) break;
         const uint32_t d = tmem_acc + ab * BNMAX;
         uint32_t more = 0u;                                  // the tile's first instruction clears the accumulator
-        const bool fetch_b = !q.resident || w == (int)blockIdx.x;          // (a resident filter is complete after the first tile)
+        const bool fetch_b = !q.resident || w == walk.first;          // (a resident filter is complete after the first tile)
         if (q.resident) slot = 0;
         for (int kb = 0; kb < q.num_kb && ok; ++kb) {
           const int nks = kb == q.num_kb - 1 ? q.nks_last : KB / 16;
@@ -320,8 +499,8 @@ __global__ void __launch_bounds__(THREADS, 1) conv_f16_runs_kernel(RunsParams q)
           int nsa = sa + 1;
           uint32_t npa = pa;
           if (nsa == q.sa) { nsa = 0; npa ^= 1u; }
-          for (int g = 0; g < q.G; ++g, a_view += 8u) {      // next view: one row (128 bytes) further down
-            const bool last_unit = g + 1 == q.G, last = kb + 1 == q.num_kb && last_unit;
+          for (int g = 0; g < q.G; g += q.cols, a_view += 8u * q.cols) {
+            const bool last_unit = g + q.cols == q.G, last = kb + 1 == q.num_kb && last_unit;
             int nslot = slot + 1;
             uint32_t npb = pb;
             if (nslot == q.sb) { nslot = 0; if (!q.resident) npb ^= 1u; }
@@ -334,13 +513,12 @@ __global__ void __launch_bounds__(THREADS, 1) conv_f16_runs_kernel(RunsParams q)
             if (last_unit) a_seen = mbar_test_wait(a_full0 + 8 * nsa, npa);
             const uint32_t b_lo = b_lo0 + (uint32_t)(slot * (q.slot_bytes >> 4));
             if (leader) {
-              if (nks == KB / 16) issue_column<KB / 16>(d, a_view, b_lo, idesc, more);
-              else if (nks == 3) issue_column<3>(d, a_view, b_lo, idesc, more);
-              else if (nks == 2) issue_column<2>(d, a_view, b_lo, idesc, more);
-              else issue_column<1>(d, a_view, b_lo, idesc, more);
-              if (!q.resident) umma_commit(b_empty0 + 8 * slot);
-              if (last && drop != kDebugDropArrive) umma_commit(acc_full0 + 8 * ab);
-              if (last_unit) umma_commit(a_empty0 + 8 * sa);
+              if (q.cols == 3) issue_slot<3, PAIR>(nks, d, a_view, b_lo, b_step, idesc, more);
+              else if (q.cols == 2) issue_slot<2, PAIR>(nks, d, a_view, b_lo, b_step, idesc, more);
+              else issue_slot<1, PAIR>(nks, d, a_view, b_lo, b_step, idesc, more);
+              if (!q.resident) commit(b_empty0 + 8 * slot);
+              if (last_unit) commit(a_empty0 + 8 * sa);
+              if (last && drop != kDebugDropArrive) commit(acc_full0 + 8 * ab);
             }
             __syncwarp();
             slot = nslot;
@@ -352,21 +530,44 @@ __global__ void __launch_bounds__(THREADS, 1) conv_f16_runs_kernel(RunsParams q)
         }
         drop = 0u;
       }
+    } else if (warp == STAGING_WARPS) {
+      // ---------------- the pair's other CTA: word to the leader that its half of a filter slot has arrived --------
+      bool ok = true;
+      int slot = 0;
+      uint32_t pb = 0;
+      const int slots = q.num_kb * q.G / q.cols;
+      for (int w = walk.first; w < q.nwork && ok; w += walk.step) {
+        for (int u = 0; u < slots; ++u) {
+          ok = mbar_wait(b_full0 + 8 * slot, pb, &abort_flag, q.status);
+          ok = __all_sync(0xffffffffu, ok);
+          if (!ok) break;
+          if (lane == 0) mbar_arrive_cluster(b_full_dst + 8 * slot);
+          __syncwarp();
+          if (++slot == q.sb) { slot = 0; pb ^= 1u; }
+        }
+        if (q.resident) break;
+      }
     } else if (warp == STAGING_WARPS + 1) {
       // ---------------- filter copies ----------------------------------------------------------------------
       const bool leader = elect_one();
       bool ok = true;
       int slot = 0;
       uint32_t pb = 0;
-      for (int w = blockIdx.x; w < q.nwork && ok; w += gridDim.x) {
-        const unsigned char* src = q.fp + (int64_t)(w % q.ntn) * q.num_kb * q.G * q.slot_bytes;
-        for (int u = 0; u < q.num_kb * q.G; ++u, src += q.slot_bytes) {
+      const int slots = q.num_kb * q.G / q.cols, column = q.bn * 128;       // bytes of a kernel column's image
+      for (int w = walk.first; w < q.nwork && ok; w += walk.step) {
+        const unsigned char* src = q.fp + (int64_t)(w % q.ntn) * slots * q.cols * column + rank * b_rows * 128;
+        for (int u = 0; u < slots; ++u, src += q.cols * column) {
           ok = mbar_wait(b_empty0 + 8 * slot, pb ^ 1u, &abort_flag, q.status);
           ok = __all_sync(0xffffffffu, ok);
           if (!ok) break;
           if (leader) {
             mbar_arrive_expect_tx(b_full0 + 8 * slot, (uint32_t)q.slot_bytes);
-            bulk_load(b_ring + slot * q.slot_bytes, src, (uint32_t)q.slot_bytes, b_full0 + 8 * slot);
+            if (PAIR) {
+              for (int c = 0; c < q.cols; ++c)
+                bulk_load(b_ring + slot * q.slot_bytes + c * b_rows * 128, src + c * column, (uint32_t)b_rows * 128u, b_full0 + 8 * slot);
+            } else {
+              bulk_load(b_ring + slot * q.slot_bytes, src, (uint32_t)q.slot_bytes, b_full0 + 8 * slot);
+            }
           }
           __syncwarp();
           if (++slot == q.sb) { slot = 0; pb ^= 1u; }
@@ -381,9 +582,44 @@ __global__ void __launch_bounds__(THREADS, 1) conv_f16_runs_kernel(RunsParams q)
       uint32_t pr = 0, sc = warp & 1;
       const int plane = (q.Ho * q.Wp + q.Wq * q.s - q.Wp) * q.Kh;
       const int per_slot = q.quad ? 4 : 8 * q.octs, nslots = q.quad ? 1 : (q.C + per_slot - 1) / per_slot;
-      for (int w = blockIdx.x; w < q.nwork && ok; w += gridDim.x) {
-        const TileRuns tr = tile_runs(q, (uint32_t)(w / q.ntn) * TILE_M);
+      for (int w = walk.first; w < q.nwork && ok; w += walk.step) {
+        const TileRuns tr = tile_runs(q, walk.start(q, w));
         const int nseg = (int)(tr.n1 - tr.n0) + 1;
+        // Copy `it` of a slot: one channel of one image.  From slot to slot only its source moves: per_slot planes further a
+        // run starts at the same phase of 16 bytes.  (Worked out per slot, a slot's eight copies cost their warp 1270 cycles.)
+        const int items = nseg * per_slot;
+        auto run_of = [&](int it, int64_t& from, uint32_t& size, uint32_t& to) {
+          const int g = it / per_slot, c = it - g * per_slot;
+          const int start = g == 0 ? tr.start0 : 0, end = g == nseg - 1 ? tr.end1 : plane;
+          const int64_t b0 = (int64_t)(tr.n0 + g) * q.img_bytes + (int64_t)c * q.chan_bytes + (int64_t)start * ES;
+          from = b0 & ~(int64_t)15;
+          size = (uint32_t)(((b0 + (int64_t)(end - start) * ES + 15) & ~(int64_t)15) - from);
+          to = raw_ring + c * q.region + (g == 0 ? 0 : run_size(plane - tr.start0) + (g - 1) * run_size(plane));
+        };
+        int64_t from0 = 0;
+        uint32_t size0 = 0, to0 = 0, total = 0;
+        // Tiled copies: lane -> image, octet of the slot and class of its channels; from slot to slot only the row moves.
+        int tx = 0, ty = 0, to = 0, oct = 0;
+        const int boxes = nseg * q.octs * q.planes;
+        if (q.planes) {
+          const int g = lane / (q.octs * q.planes), rest = lane - g * q.octs * q.planes, o = rest / q.planes, r = rest - o * q.planes;
+          tx = (int)((r * q.chan_bytes + (int64_t)(g == 0 ? tr.start0 : 0) * ES) >> 4) * 2;         // in 8-byte elements, even
+          ty = (int)(((int64_t)(tr.n0 + g) * q.C + 8 * o) / q.planes);
+          to = o < q.octs ? g * q.seg_bytes + (8 * o + r * (8 / q.planes)) * q.region : 0;
+          oct = o;
+        } else if (lane < items) {
+          run_of(lane, from0, size0, to0);
+          total = size0;
+        }
+        for (int it = lane + 32; it < items && q.planes == 0; it += 32) {
+          int64_t from;
+          uint32_t size, to;
+          run_of(it, from, size, to);
+          total += size;
+        }
+        total = __reduce_add_sync(0xffffffffu, total);
+        // bytes behind the first slot's last run, up to the next 16-byte boundary, that are still of the tensor
+        const int64_t spare = q.win_bytes - 15 - ((int64_t)tr.n1 * q.img_bytes + (per_slot - 1) * q.chan_bytes + (int64_t)tr.end1 * ES);
         for (int sl = 0; sl < nslots; ++sl, ++sc) {
           if (sc & 1) {
             if (++sr == q.sr) { sr = 0; pr ^= 1u; }
@@ -392,6 +628,34 @@ __global__ void __launch_bounds__(THREADS, 1) conv_f16_runs_kernel(RunsParams q)
           ok = mbar_wait(raw_empty0 + 8 * sr, pr ^ 1u, &abort_flag, q.status);
           ok = __all_sync(0xffffffffu, ok);
           if (!ok) break;
+          if (q.planes) {
+            const int here = (q.C + 7) / 8 - sl * q.octs < q.octs ? (q.C + 7) / 8 - sl * q.octs : q.octs;     // octets
+            if (lane == 0) mbar_arrive_expect_tx(raw_full0 + 8 * sr, (uint32_t)(nseg * here * 8 * q.region));
+            __syncwarp();
+            if (lane < boxes && oct < here)
+              tma_load_2d(raw_ring + sr * q.raw_slot + to, &q.map, tx, ty + sl * q.octs * (8 / q.planes), raw_full0 + 8 * sr);
+            __syncwarp();
+            if (++sr == q.sr) { sr = 0; pr ^= 1u; }
+            continue;
+          }
+          const int64_t ahead = (int64_t)sl * per_slot * q.chan_bytes;
+          if ((sl + 1) * per_slot <= q.C && ahead <= spare) {
+            const uint32_t bar = raw_full0 + 8 * sr, slot = sr * q.raw_slot;
+            const unsigned char* win = q.win + ahead;
+            if (lane == 0) mbar_arrive_expect_tx(bar, total);
+            __syncwarp();
+            if (lane < items) bulk_load(to0 + slot, win + from0, size0, bar);
+            for (int it = lane + 32; it < items; it += 32) {
+              int64_t from;
+              uint32_t size, to;
+              run_of(it, from, size, to);
+              bulk_load(to + slot, win + from, size, bar);
+            }
+            __syncwarp();
+            if (++sr == q.sr) { sr = 0; pr ^= 1u; }
+            continue;
+          }
+          // a slot that is not full, or may reach the end of the tensor
           const uint32_t bar = raw_full0 + 8 * sr;
           const int c0 = sl * per_slot, nc = q.C - c0 < per_slot ? q.C - c0 : per_slot;
           int seg_off = 0;
@@ -430,8 +694,12 @@ __global__ void __launch_bounds__(THREADS, 1) conv_f16_runs_kernel(RunsParams q)
     const int lq = warp & 3, h = (warp - STAGING_WARPS - 4) >> 2;           // tensor-memory quadrant; which channels
     bool ok = true;
     uint32_t ac = 0;
-    for (int w = blockIdx.x; w < q.nwork && ok; w += gridDim.x) {
-      const int mt = w / q.ntn, nt = w - mt * q.ntn;
+    auto arrive_empty = [&](int ab) {
+      if (PAIR) mbar_arrive_cluster(acc_empty_dst + 8 * ab);
+      else mbar_arrive(acc_empty0 + 8 * ab);
+    };
+    for (int w = walk.first; w < q.nwork && ok; w += walk.step) {
+      const int mt = walk.tile(q, w), nt = w % q.ntn;        // (a position tile beyond the last: nothing to store)
       const uint32_t vq = (uint32_t)mt * TILE_M + (uint32_t)(lq * 32 + lane);
       const int co0 = nt * q.bn;
       const int limit = q.Co - co0 < q.bn ? q.Co - co0 : q.bn;            // channels of this tile that exist
@@ -457,7 +725,7 @@ __global__ void __launch_bounds__(THREADS, 1) conv_f16_runs_kernel(RunsParams q)
         if (c0 + 32 >= (h + 1) * (BNMAX / 2) || c0 + 32 >= limit) {      // the last read of this accumulator
           tc_fence_before();
           __syncwarp();
-          if (lane == 0) mbar_arrive(acc_empty0 + 8 * ab);
+          if (lane == 0) arrive_empty(ab);
         }
         if (valid) {
           store_strided32(yrow + (int64_t)c0 * q.HoWo, q.HoWo, v, limit - c0);
@@ -468,16 +736,17 @@ __global__ void __launch_bounds__(THREADS, 1) conv_f16_runs_kernel(RunsParams q)
           }
           if (zero != 0.f) {                               // (a NaN: one of them is not finite)
             const unsigned char* x = q.win + (int64_t)n * q.img_bytes + ((int64_t)ho * q.Wp + (int64_t)i0 * q.s) * q.Kh * ES;
-            const unsigned char* f = q.fp + (int64_t)nt * q.num_kb * q.G * q.slot_bytes;
+            const int column = q.bn * 128;                 // bytes of a filter column's image
+            const unsigned char* f = q.fp + (int64_t)nt * q.num_kb * q.G * column;
             for (int c = c0; c < c0 + 32 && c < limit; c += 16)
               exact_outputs(x, f + c * 128, yrow + (int64_t)c * q.HoWo, q.HoWo, q.chan_bytes, q.C, q.Kh, q.Kw, q.s, q.E,
-                            q.slot_bytes, q.G * q.slot_bytes, q.quad, limit - c < 16 ? limit - c : 16);
+                            column, q.G * column, q.quad, limit - c < 16 ? limit - c : 16);
           }
         }
       }
       if (h * (BNMAX / 2) >= limit) {                      // (no channels for this warp)
         __syncwarp();
-        if (lane == 0) mbar_arrive(acc_empty0 + 8 * ab);
+        if (lane == 0) arrive_empty(ab);
       }
     }
   }
@@ -489,10 +758,12 @@ __global__ void __launch_bounds__(THREADS, 1) conv_f16_runs_kernel(RunsParams q)
     for (int i = 0; i < 64; ++i) __nanosleep(1000);
     __syncthreads();
   }
+  if (PAIR) cluster_sync_all();                             // no CTA leaves while its peer may still signal or read it
   if (warp == STAGING_WARPS) {
     __syncwarp();
     tc_fence_after();
-    tmem_dealloc(tmem_acc, 512);
+    if (PAIR) tmem_dealloc_pair(tmem_acc, 512);
+    else tmem_dealloc(tmem_acc, 512);
   }
 }
 
@@ -536,20 +807,43 @@ __global__ void __launch_bounds__(256) pack_f16_runs_kernel(const uint16_t* __re
   }
 }
 
-template <int BNMAX>
+template <int BNMAX, bool PAIR>
 cudaError_t launch_form(const RunsParams& q, int smem, cudaStream_t stream) {
   static bool attr_done[64] = {};
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
   if (!attr_done[dev]) {
-    cudaError_t e = cudaFuncSetAttribute(conv_f16_runs_kernel<BNMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRunsSmem);
+    cudaError_t e = cudaFuncSetAttribute(conv_f16_runs_kernel<BNMAX, PAIR>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRunsSmem);
     if (e != cudaSuccess) return e;
     attr_done[dev] = true;
   }
-  return launch_after_previous(conv_f16_runs_kernel<BNMAX>, q.nwork < 148 ? q.nwork : 148, 1, THREADS, smem, stream, q);
+  const int most = PAIR ? 74 : 148, grid = (q.nwork < most ? q.nwork : most) * (PAIR ? 2 : 1);
+  return launch_after_previous(conv_f16_runs_kernel<BNMAX, PAIR>, grid, PAIR ? 2 : 1, THREADS, smem, stream, q);
 }
 
 }  // namespace
+
+// The window tensor in rows of p.planes channel planes, 8-byte elements (a box may be 256 of them wide).
+static bool encode_window_rows(CUtensorMap* map, const uint16_t* window, const Geometry& g, const RunsPlan& p) {
+  typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
+                                    const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
+                                    CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+  static EncodeTiledFn encode = nullptr;
+  if (!encode) {
+    void* fn = nullptr;
+    cudaDriverEntryPointQueryResult found;
+    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &found) != cudaSuccess ||
+        found != cudaDriverEntryPointSuccess)
+      return false;
+    encode = reinterpret_cast<EncodeTiledFn>(fn);
+  }
+  const cuuint64_t row = (cuuint64_t)p.planes * g.chan_stride * ES;
+  const cuuint64_t dims[2] = {row / 8, (cuuint64_t)g.N * g.C / p.planes}, strides[1] = {row};
+  const cuuint32_t box[2] = {(cuuint32_t)(p.region / 8), (cuuint32_t)(8 / p.planes)}, ones[2] = {1, 1};
+  return encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 2, const_cast<uint16_t*>(window), dims, strides, box, ones,
+                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
 
 // Channels of the octets that a k2-block (8 units) can touch: what a block of the pack kernel stages.
 static int64_t pack_channels(int64_t E, int C) {
@@ -585,29 +879,60 @@ RunsPlan plan_f16_runs(const Geometry& g) {
   p.region = (int32_t)((region + 15) / 16 * 16);
   p.ntn = (g.Co + 255) / 256;
   p.bn = ((g.Co + p.ntn - 1) / p.ntn + 15) / 16 * 16;
+  if (p.bn > 128) p.bn = (p.bn + 31) / 32 * 32;             // (of a pair's instruction)
   p.ntn = (g.Co + p.bn - 1) / p.bn;
-  p.slot_bytes = p.bn * 128;
   const int64_t ntm = (p.VQ + TILE_M - 1) / TILE_M;
   if (ntm * p.ntn >= ((int64_t)1 << 30)) return p;
-  p.nwork = (int32_t)(ntm * p.ntn);
-  const int units = p.num_kb * p.G;
+  // CTA pairs above 128 channels: each CTA stages its own position tile and half of the filter.  The shared-memory pipe bounds
+  // those tiles (an instruction of N = 256 reads 12 KB of operands in 128 cycles, one of a pair 8 KB an SM), and the
+  // filter's copies, twice the bytes of all else, halve.
+  p.pair = p.bn > 128 && ntm > 1;
+  if (const char* v = debug_getenv("IM2WIN_F16_PAIR")) p.pair = p.pair && v[0] != '0';     // testing aid
+  p.ntm = (int32_t)ntm;
+  p.nwork = (int32_t)((p.pair ? (ntm + 1) / 2 : ntm) * p.ntn);
   const int budget = kRunsSmem - 1024;
-  // A raw slot holds whole octets, at least three units; rings of two S stages, four slots (else two)
-  // and the filter (resident where one channel tile's fits, else at least three units).
+  // A raw slot holds whole octets, at least three units; rings of two S stages, four slots (else two) and the filter:
+  // resident where one channel tile's fits, else two slots of all (up to three) kernel columns of a k2-block, so that the MMA
+  // warp waits and commits once a k2-block, else at least three of one column.
   p.octs = (int32_t)(E >= 3 ? 1 : (E == 2 ? 2 : 4));
-  const int64_t raw = ((p.quad ? 4 : 8 * p.octs) * (int64_t)p.region + 127) / 128 * 128;
-  for (int pass = 0; pass < 4 && !p.eligible; ++pass) {
-    const bool resident = (pass & 1) == 0 && p.ntn == 1 && units <= MAX_B;
-    if ((pass & 1) == 0 && !resident) continue;
-    const int least_raw = pass < 2 ? 4 : 2, least_b = resident ? units : 3;
-    if (2 * p.a_stage + least_b * p.slot_bytes + least_raw * raw > budget) continue;
+  int64_t raw = ((p.quad ? 4 : 8 * p.octs) * (int64_t)p.region + 127) / 128 * 128;
+  // Raw copies.  A bulk copy takes the copy engine 100 to 130 cycles whatever its size (3x3 on 64 channels at 56x56: 86 of 109 us
+  // with all else left out), a tiled one that brings 8 / planes channels at once hardly more; `planes` channel planes are a
+  // multiple of 16 bytes.  A box is as wide as a whole tile's columns, for every image of the tile: two images at most.
+  p.planes = 1;
+  while (p.planes < 8 && (p.planes * g.chan_stride * ES) % 16 != 0) p.planes *= 2;
+  // (every box starts on 128 bytes of shared memory: its 8 / planes rows are a multiple of that)
+  const int64_t wide = (int64_t)(TILE_M + p.halo) * g.s * g.Kh * ES + 15;
+  const int64_t box = (wide + 16 * p.planes - 1) / (16 * p.planes) * (16 * p.planes);
+  if (p.planes == 8 || p.quad || g.C % p.planes != 0 || box > 2048 || segs > 2 || segs * p.octs * p.planes > 32 ||
+      (int64_t)g.N * g.C >= ((int64_t)1 << 31))
+    p.planes = 0;
+  if (const char* v = debug_getenv("IM2WIN_F16_RUNS_TILED")) if (v[0] == '0') p.planes = 0;           // testing aid
+  const int64_t tiled_raw = segs * p.octs * 8 * box;
+  if (2 * (int64_t)p.a_stage + 3 * (int64_t)(p.pair ? p.bn / 2 : p.bn) * 128 + 4 * ((tiled_raw + 127) / 128 * 128) > budget) p.planes = 0;
+  if (p.planes) {
+    p.region = (int32_t)box;
+    p.seg_bytes = (int32_t)(p.octs * 8 * box);
+    raw = (tiled_raw + 127) / 128 * 128;
+  }
+  for (int pass = 0; pass < 6 && !p.eligible; ++pass) {
+    const int kind = pass % 3;                               // resident, whole k2-blocks, columns
+    p.cols = kind < 2 && p.G <= 3 ? p.G : 1;
+    p.slot_bytes = p.cols * (p.pair ? p.bn / 2 : p.bn) * 128;
+    const int units = p.num_kb * p.G / p.cols;
+    const bool resident = kind == 0 && p.ntn == 1 && units <= MAX_B;
+    if (kind == 0 && !resident) continue;
+    if (kind == 1 && p.cols == 1) continue;
+    const int least_raw = pass < 3 ? 4 : 2, least_b = resident ? units : (kind == 1 ? 2 : 3);
+    if (2 * (int64_t)p.a_stage + (int64_t)least_b * p.slot_bytes + least_raw * raw > budget) continue;
     p.raw_slot = (int32_t)raw;
     p.resident = resident;
     p.sa = 2; p.sr = least_raw; p.sb = least_b;
     auto fits = [&](int a, int r, int b) { return (int64_t)a * p.a_stage + (int64_t)r * raw + (int64_t)b * p.slot_bytes <= budget; };
+    if (!resident && p.sb < 3 && fits(p.sa, p.sr, 3)) p.sb = 3;
+    if (fits(3, p.sr, p.sb)) p.sa = 3;                       // (before a fourth filter slot: 120 -> 107 us on a pair's tiles)
     if (!resident) while (p.sb < 4 && fits(p.sa, p.sr, p.sb + 1)) ++p.sb;
-    if (fits(3, p.sr, p.sb)) p.sa = 3;
-    while (p.sr < MAX_RAW && fits(p.sa, p.sr + 2, p.sb)) p.sr += 2;   // (even: the two copy warps alternate)
+    while (p.sr + 2 <= MAX_RAW && fits(p.sa, p.sr + 2, p.sb)) p.sr += 2;   // (even: the two copy warps alternate)
     if (!resident) while (p.sb < MAX_B && fits(p.sa, p.sr, p.sb + 1)) ++p.sb;
     p.eligible = true;
   }
@@ -646,14 +971,21 @@ cudaError_t launch_conv_f16_runs(const uint16_t* window, float* y, void* scratch
   q.Co = g.Co; q.Kh = g.Kh; q.Kw = g.Kw; q.s = g.s;
   // kernel columns beyond Kw, channels beyond C in the last octet, the element beyond an odd E
   q.foreign = (g.Kw > g.s && g.Kw % g.s != 0) || (p.quad ? p.E % 2 != 0 : g.C % 8 != 0);
+  const bool words = p.E % 2 == 0 && g.s * g.Kh % 2 == 0 && (int64_t)g.Wp * g.Kh % 2 == 0;
+  const bool pairs = p.E == 3 && g.s == 1 && (int64_t)g.Ho * g.Wp % 2 == 0;
+  q.mode = p.quad ? QUAD : (words ? WORDS : (pairs ? ROW_PAIRS : HALVES));
   q.E = p.E; q.G = p.G; q.units = p.units; q.quad = p.quad ? 1 : 0; q.num_kb = p.num_kb; q.nks_last = p.nks_last;
   q.halo = p.halo; q.region = p.region; q.octs = p.octs; q.raw_slot = p.raw_slot; q.a_stage = p.a_stage;
   q.bn = p.bn; q.ntn = p.ntn; q.nwork = p.nwork; q.sa = p.sa; q.sr = p.sr; q.sb = p.sb;
-  q.slot_bytes = p.slot_bytes; q.resident = p.resident ? 1 : 0;
+  q.planes = p.planes; q.seg_bytes = p.seg_bytes;
+  if (p.planes) {
+    if (!encode_window_rows(&q.map, window, g, p)) return cudaErrorInvalidValue;
+  }
+  q.slot_bytes = p.slot_bytes; q.cols = p.cols; q.ntm = p.ntm; q.resident = p.resident ? 1 : 0;
   const int smem = 1024 + p.sa * p.a_stage + p.sb * p.slot_bytes + p.sr * p.raw_slot;
-  if (p.bn <= 64) return launch_form<64>(q, smem, stream);
-  if (p.bn <= 128) return launch_form<128>(q, smem, stream);
-  return launch_form<256>(q, smem, stream);
+  if (p.bn <= 64) return launch_form<64, false>(q, smem, stream);
+  if (p.bn <= 128) return launch_form<128, false>(q, smem, stream);
+  return p.pair ? launch_form<256, true>(q, smem, stream) : launch_form<256, false>(q, smem, stream);
 }
 
 }  // namespace im2win

@@ -1,5 +1,6 @@
 """Tiles and rounds of the convolution kernels at the sizes where their rules change: a last round in parts of the channels
-(fp32 on the tensor cores), tiles of parts of strips (channel-innermost kernel)."""
+(fp32 on the tensor cores), tiles of parts of strips (channel-innermost kernel), the ways the run-staged kernel brings
+its columns in."""
 import numpy as np
 import pytest
 import torch
@@ -60,3 +61,41 @@ def test_nhwc_tiles_of_parts_of_strips(layer, layout, monkeypatch):
     y = gpu_conv_nhwc(x, f, dims, x_layout=layout)
     yr, ar = oracle.conv_direct(*oracle_inputs(x, f, "f16"), dims)
     check_conv(y, yr, ar, "f16", layer.name)
+
+
+# the columns of the run-staged kernel: elements, words of two, pairs of rows; copies of one, two, four and eight channels
+@pytest.mark.parametrize("layer", [
+    L("pairs_1", 2, 24, 20, 14, 130, 3, 3, 1, 1, 420),       # plane a multiple of 16 bytes, CTA pairs, 5 position tiles
+    L("pairs_4", 3, 12, 14, 11, 33, 3, 3, 1, 1, 421),        # four planes are, half an octet, two images in a tile
+    L("pairs_8", 2, 16, 13, 12, 70, 3, 3, 1, 1, 422),        # eight planes: bulk copies
+    L("pairs_s", 5, 40, 9, 8, 16, 3, 3, 1, 0, 423),          # several images in a tile: bulk copies
+    L("words_2", 2, 16, 28, 28, 136, 3, 3, 2, 1, 424),       # two planes, stride 2, CTA pairs
+    L("words_c9", 2, 9, 28, 28, 264, 3, 3, 2, 1, 425),       # an odd number of channels: bulk copies, two channel tiles
+    L("words_10", 1, 16, 30, 30, 40, 5, 5, 2, 1, 426),       # ten elements a column, boxes too wide
+    L("words_2el", 1, 24, 30, 28, 40, 1, 2, 2, 0, 427),      # two elements, two octets a slot
+    L("halves_5", 2, 16, 16, 12, 48, 5, 5, 1, 2, 428),       # five elements, four rows below the tile
+    L("halves_1", 2, 72, 16, 16, 200, 1, 1, 1, 0, 429),      # one element, four octets a slot, the last slot not full
+    L("halves_odd", 2, 16, 13, 15, 48, 3, 3, 1, 1, 430),     # an odd number of columns in an image
+    L("last_pair", 9, 32, 16, 14, 256, 3, 3, 1, 1, 431),     # 18 position tiles
+    L("rounds", 40, 16, 26, 30, 200, 3, 3, 1, 1, 432)], ids=lambda l: l.name)      # more pairs than the GPU holds
+@pytest.mark.parametrize("tiled,pair", [("1", "1"), ("0", "1"), ("1", "0")])
+def test_f16_runs_columns_and_copies(layer, tiled, pair, monkeypatch):
+    monkeypatch.setenv("IM2WIN_F16_KERNEL", "runs")
+    monkeypatch.setenv("IM2WIN_F16_RUNS_TILED", tiled)
+    monkeypatch.setenv("IM2WIN_F16_PAIR", pair)
+    dims = layer.dims()
+    assert binding.im2win_conv_kernel_name(dims, binding.F16) == "f16-runs"
+    x, f = workloads.make_small_integer_inputs(layer)
+    y, _, _ = gpu_conv(x, f, dims, "f16")
+    yr, _ = oracle.conv_direct(x.numpy(), f.numpy(), dims)
+    assert np.array_equal(y.astype(np.float64), yr)
+    x, f = workloads.make_inputs(layer)
+    y, _, _ = gpu_conv(x, f, dims, "f16")
+    yr, ar = oracle.conv_direct(*oracle_inputs(x, f, "f16"), dims)
+    check_conv(y, yr, ar, "f16", layer.name)
+    # an infinity and a NaN reach exactly the outputs whose windows hold them
+    x.view(-1)[x.numel() // 3] = float("inf")
+    x.view(-1)[x.numel() // 2] = float("nan")
+    y, _, _ = gpu_conv(x, f, dims, "f16")
+    ref = torch.nn.functional.conv2d(x.half().double(), f.half().double(), stride=layer.stride, padding=layer.pad).numpy()
+    assert np.array_equal(np.isfinite(y), np.isfinite(ref)) and np.array_equal(np.isnan(y), np.isnan(ref))
