@@ -98,7 +98,7 @@ struct Segment {            // the part of a tile that lies in one image
 // the filter pack (the kernel before it in the stream) is still running; its barrier setup, tensor
 // memory allocation and descriptor fetches overlap the pack.  Every role that touches global memory
 // first waits for the preceding kernel to have completed (and its writes to be visible).
-__device__ __forceinline__ void let_next_kernel_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// (let_next_kernel_start in the pack, wait_for_previous_kernel here.)
 
 // Splits the rows of the tile starting at virtual position q0 by image: within an image the
 // columns of one channel are contiguous in the window tensor.  Returns the number of segments

@@ -774,6 +774,7 @@ __global__ void __launch_bounds__(256) pack_f16_runs_kernel(const uint16_t* __re
                                                         uint32_t* __restrict__ status, int C, int Kh, int Kw, int s, int E, int G,
                                                         int Co, int bn, int num_kb, int rows, int pitch, int quad) {
   extern __shared__ uint16_t pack_h[];
+  let_next_kernel_start();                                 // (the convolution sets itself up meanwhile)
   if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < kStatusBytes / 4) status[threadIdx.x] = 0u;
   const int kb = blockIdx.y, row0 = blockIdx.x * rows;     // (channel blocks along x: any number of channels)
   const int c0 = quad ? 0 : kb * 8 / E * 8;
@@ -945,8 +946,10 @@ cudaError_t launch_pack_f16_runs(const uint16_t* filter, void* scratch, const Ge
   if (!p.eligible) return cudaErrorInvalidValue;
   unsigned char* base = static_cast<unsigned char*>(scratch);
   const int64_t pitch = pack_channels(p.E, g.C) * g.T;
-  int rows = 8;                                             // channels per block: staging within 40 KB
-  while (rows > 1 && rows * pitch * ES > 40 * 1024) rows /= 2;
+  // Channels per block: staging within 40 KB, and two blocks an SM where the filter has them (a block's channels are loaded one
+  // after another, a round trip each: 3x3 on 64 -> 64 channels in 24 blocks took as long as ten times the filter)
+  int rows = 8;
+  while (rows > 1 && (rows * pitch * ES > 40 * 1024 || (int64_t)p.ntn * p.bn / rows * p.num_kb < 2 * 148)) rows /= 2;
   const size_t smem = (size_t)(rows * pitch * ES);
   dim3 grid((unsigned)(p.ntn * p.bn / rows), (unsigned)p.num_kb);   // (num_kb <= 2^14: C * E <= 2^20)
   pack_f16_runs_kernel<<<grid, 256, smem, stream>>>(filter, base + kStatusBytes, reinterpret_cast<uint32_t*>(base), g.C, g.Kh, g.Kw,

@@ -667,6 +667,7 @@ __global__ void __launch_bounds__(256) pack_f32_split_kernel(const float* __rest
                                                              float* __restrict__ copy, uint32_t* __restrict__ status, int K2, int Kw, int Co, int bn,
                                                              int num_kb, int rows, int concat) {
   extern __shared__ float pack_f[];
+  let_next_kernel_start();                                 // (the convolution sets itself up meanwhile)
   if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < kStatusBytes / 4) status[threadIdx.x] = 0u;
   const int kb = blockIdx.y, row0 = blockIdx.x * rows;     // (channel blocks along x: any number of channels)
   const int nreal = K2 - kb * KB < KB ? K2 - kb * KB : KB;
@@ -809,8 +810,10 @@ cudaError_t launch_pack_f32_split(const float* filter, void* scratch, const Geom
   const F32SplitPlan p = plan_f32_split(g);
   if (!p.eligible) return cudaErrorInvalidValue;
   unsigned char* base = static_cast<unsigned char*>(scratch);
-  int rows = 8;                                             // channels per block: staging within 40 KB
-  while (rows > 1 && (size_t)rows * KB * g.Kw * 4 > 40 * 1024) rows /= 2;
+  // Channels per block: staging within 40 KB, and two blocks an SM where the filter has them (a block's channels are loaded one
+  // after another, a round trip each)
+  int rows = 8;
+  while (rows > 1 && ((size_t)rows * KB * g.Kw * 4 > 40 * 1024 || (int64_t)p.ntn * p.bn / rows * p.num_kb < 2 * 148)) rows /= 2;
   const size_t smem = (size_t)rows * KB * g.Kw * 4;
   dim3 grid((unsigned)(p.ntn * p.bn / rows), (unsigned)p.num_kb);
   pack_f32_split_kernel<<<grid, 256, smem, stream>>>(filter, base + kStatusBytes, reinterpret_cast<float*>(base + kStatusBytes + p.copy_off), reinterpret_cast<uint32_t*>(base), g.C * g.Kh,

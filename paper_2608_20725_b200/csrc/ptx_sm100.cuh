@@ -137,6 +137,8 @@ __device__ __forceinline__ void st_shared16(uint32_t addr, uint32_t a, uint32_t 
 }
 // In a kernel that may start before the one ahead of it in the stream is done: everything of that one is complete and visible.
 __device__ __forceinline__ void wait_for_previous_kernel() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// A kernel after this one in the stream that waits that way may start as soon as every block here has come this far.
+__device__ __forceinline__ void let_next_kernel_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 // The warp's number, the same value in every lane as far as the compiler can see (a shuffle's result): the roles' branches
 // and loops then are uniform ones, and their counters and addresses stay in uniform registers instead of being handed over
 // lane by lane to every instruction that wants them uniform.  Against threadIdx.x >> 5: 7x7 stride 2 on 3 channels at 224x224,
