@@ -880,14 +880,14 @@ RunsPlan plan_f16_runs(const Geometry& g) {
   p.region = (int32_t)((region + 15) / 16 * 16);
   p.ntn = (g.Co + 255) / 256;
   p.bn = ((g.Co + p.ntn - 1) / p.ntn + 15) / 16 * 16;
-  if (p.bn > 128) p.bn = (p.bn + 31) / 32 * 32;             // (of a pair's instruction)
   p.ntn = (g.Co + p.bn - 1) / p.bn;
   const int64_t ntm = (p.VQ + TILE_M - 1) / TILE_M;
   if (ntm * p.ntn >= ((int64_t)1 << 30)) return p;
   // CTA pairs above 128 channels: each CTA stages its own position tile and half of the filter.  The shared-memory pipe bounds
   // those tiles (an instruction of N = 256 reads 12 KB of operands in 128 cycles, one of a pair 8 KB an SM), and the
   // filter's copies, twice the bytes of all else, halve.
-  p.pair = p.bn > 128 && ntm > 1;
+  // (N of a pair's instruction: a multiple of 32.  Wider tiles for the others would want more scratch)
+  p.pair = p.bn > 128 && p.bn % 32 == 0 && ntm > 1;
   if (const char* v = debug_getenv("IM2WIN_F16_PAIR")) p.pair = p.pair && v[0] != '0';     // testing aid
   p.ntm = (int32_t)ntm;
   p.nwork = (int32_t)((p.pair ? (ntm + 1) / 2 : ntm) * p.ntn);
@@ -897,6 +897,10 @@ RunsPlan plan_f16_runs(const Geometry& g) {
   // warp waits and commits once a k2-block, else at least three of one column.
   p.octs = (int32_t)(E >= 3 ? 1 : (E == 2 ? 2 : 4));
   int64_t raw = ((p.quad ? 4 : 8 * p.octs) * (int64_t)p.region + 127) / 128 * 128;
+  // Layers whose whole filter columns and bulk copies would not fit stay out, also where a pair's halves would: their scratch is
+  // not sized for this kernel's filter.
+  const int columns = p.num_kb * p.G, fewest = p.ntn == 1 && columns < 3 ? columns : 3;
+  if (2 * (int64_t)p.a_stage + (int64_t)fewest * p.bn * 128 + 2 * raw > budget) return p;
   // Raw copies.  A bulk copy takes the copy engine 100 to 130 cycles whatever its size (3x3 on 64 channels at 56x56: 86 of 109 us
   // with all else left out), a tiled one that brings 8 / planes channels at once hardly more; `planes` channel planes are a
   // multiple of 16 bytes.  A box is as wide as a whole tile's columns, for every image of the tile: two images at most.

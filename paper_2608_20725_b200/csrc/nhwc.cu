@@ -2011,20 +2011,14 @@ NhwcPlan plan_nhwc(const Geometry& g) {
   if ((int64_t)g.s * g.Kh * p.Cp * 2 >= ((int64_t)1 << 40) || p.strip * 2 >= ((int64_t)1 << 40)) return p;
   // the transform from NCHW stages at least eight columns of Cp + 2 channels in 48 KB of shared memory
   if ((int64_t)(p.Cp + 2) * 2 * 8 > 48 * 1024) return p;
-  // position tiles: G strips x bw output columns, tw of them along a strip (one when the strip fits 128 rows).  Whole strips
-  // of 28 fill 112 of a tile's 128 rows, halves of nine strips 126: stride 1 reductions of 128 to 256 k-blocks, whose tiles
-  // are long against their loads and stores, take the fewest tiles (7x7 on 256 channels at 28x28, batch 64, 254 -> 225 us,
-  // with bias, ReLU and binary16 stores 255 -> 221).  Beyond, the power limit decides and the gain does not hold (11x11, 480
-  // k-blocks: 617 to 636 -> 579 to 710).
-  p.ntm = lim;
-  for (int tw = (g.Wo + TILE_M - 1) / TILE_M, tries = 0; tries < 8 && tw <= g.Wo; ++tw, ++tries) {
-    const int bw = (g.Wo + tw - 1) / tw;
-    if (tries > 0 && (bw < 7 || p.num_kb < 128 || p.num_kb > 256 || g.s > 1)) break;
-    const int G = TILE_M / bw < 256 ? TILE_M / bw : 256;
-    const int64_t ntm = ((int64_t)g.N * g.Ho + G - 1) / G * tw;
-    if (tries > 0 && 100 * ntm > 97 * p.ntm) continue;       // (a few per cent are not worth shorter runs of stores)
-    p.tw = tw; p.bw = bw; p.G = G; p.ntm = ntm;
-  }
+  // position tiles: tw tiles along a strip of bw columns each (one when the strip fits 128 rows),
+  // G whole strips per tile when a strip is short
+  p.tw = (g.Wo + TILE_M - 1) / TILE_M;
+  p.bw = (g.Wo + p.tw - 1) / p.tw;
+  p.G = p.tw > 1 ? 1 : TILE_M / p.bw;
+  if (p.G > 256) p.G = 256;
+  const int64_t groups = ((int64_t)g.N * g.Ho + p.G - 1) / p.G;
+  p.ntm = groups * p.tw;
   // channel tile: the narrowest MMA N that covers Co, at most 256; CTA pairs (cta_group::2, M = 256)
   p.bn = g.Co <= 64 ? 64 : (g.Co <= 128 ? 128 : 256);
   p.pair = p.ntm >= 2;       // pairs at every width: half the filter bytes per CTA and half the MMA instructions per flop
@@ -2188,6 +2182,21 @@ struct NhwcChoice {
   bool runs;                 // overlapping-row kernel: the last round of tiles goes out as runs of its reduction
 };
 
+// Tiles of parts of strips for the overlapping-row kernel.  Whole strips of 28 fill 112 of a tile's 128 rows, halves of nine
+// strips 126: stride 1 reductions of 128 to 256 k-blocks, whose tiles are long against their loads and stores, take the fewest
+// tiles (7x7 on 256 channels at 28x28, batch 64, 254 -> 225 us, with bias, ReLU and binary16 stores 255 -> 221).  Beyond, the power
+// limit decides and the gain does not hold (11x11, 480 k-blocks: 617 to 636 -> 579 to 710).
+void part_strips(const Geometry& g, NhwcPlan& p) {
+  if (p.num_kb < 128 || p.num_kb > 256 || g.s > 1) return;
+  for (int tw = p.tw + 1; tw <= p.tw + 7 && (g.Wo + tw - 1) / tw >= 7; ++tw) {
+    const int bw = (g.Wo + tw - 1) / tw, G = TILE_M / bw;
+    const int64_t ntm = ((int64_t)g.N * g.Ho + G - 1) / G * tw;
+    if (100 * ntm > 97 * p.ntm) continue;                  // (a few per cent are not worth shorter runs of stores)
+    p.tw = tw; p.bw = bw; p.G = G; p.ntm = ntm;
+    break;
+  }
+}
+
 NhwcChoice choose_nhwc(const Geometry& g, const EpilogueArgs& epi) {
   NhwcChoice c{};
   NhwcPlan& plan = c.plan;
@@ -2254,6 +2263,7 @@ NhwcChoice choose_nhwc(const Geometry& g, const EpilogueArgs& epi) {
     const double r_split = (double)((it_s * plan.ksplit + slots - 1) / slots) / plan.ksplit + 0.1;
     if (r_tail <= r_split) { split = false; plan.ksplit = 1; }
   }
+  if (!use_shift) part_strips(g, plan);
   if (!use_shift && plan.partial_bytes > 0) {
     // Overlapping-row kernel: a short last round handed out as runs of its reduction (plan_runs), against
     // a K split of every tile (cleared output, atomics).  Measured: 7x7 on 256 channels 250 against 261 us,

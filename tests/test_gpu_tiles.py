@@ -43,12 +43,12 @@ def test_f32_last_round_in_parts_of_the_channels(layer, bn, monkeypatch):
     check_conv(one, yr, ar, "f32", layer.name)
 
 
-# reductions of 128 k-blocks of 64 and more, up to 256: strips of 28 in halves, 9 strips a tile; 27 and 30 do not divide
+# reductions of 128 k-blocks of 64 and more, up to 256: strips of 28 in halves, 9 strips a tile; 27 and 50 do not divide
 @pytest.mark.parametrize("layer", [
-    L("k128", 1, 168, 28, 28, 72, 7, 7, 1, 3, 410), L("odd", 2, 165, 19, 27, 40, 7, 7, 1, 3, 411),
-    L("thirds", 1, 120, 21, 30, 130, 9, 9, 1, 4, 412), L("wide", 1, 168, 9, 60, 64, 7, 7, 1, 3, 413),
-    L("k256", 1, 256, 14, 28, 24, 8, 8, 1, 3, 414),
-    L("short", 1, 160, 28, 28, 72, 7, 7, 1, 3, 415), L("strided", 1, 168, 28, 56, 72, 7, 7, 2, 3, 416)], ids=lambda l: l.name)
+    L("k128", 5, 168, 28, 28, 72, 7, 7, 1, 3, 410), L("odd", 5, 165, 19, 27, 40, 7, 7, 1, 3, 411),
+    L("w36", 4, 120, 21, 36, 130, 9, 9, 1, 4, 412), L("w50", 4, 168, 9, 50, 64, 7, 7, 1, 3, 413),
+    L("k256", 5, 256, 14, 28, 24, 8, 8, 1, 3, 414),
+    L("short", 5, 160, 28, 28, 24, 7, 7, 1, 3, 415), L("strided", 5, 168, 28, 56, 24, 7, 7, 2, 3, 416)], ids=lambda l: l.name)
 @pytest.mark.parametrize("layout", ["nchw", "nhwc"])
 def test_nhwc_tiles_of_parts_of_strips(layer, layout, monkeypatch):
     monkeypatch.setenv("IM2WIN_NHWC_KERNEL", "overlap")
