@@ -36,10 +36,10 @@
 // Roles (one persistent CTA per SM): one or two warpgroups of producers (thread = row; 32 loads in flight,
 // split, 16-byte stores), an MMA warp, a filter-copy warp (one untiled bulk copy per piece: the pack kernel
 // writes shared-memory images), eight epilogue warps that keep the tile's fp32 sums in registers.
-// Measured against the FFMA kernel (us, filter packed beforehand): 3x3 on 64 channels at 56x56, batch 128, 543 -> 221 (134
-// TFLOP/s; no pipe above 45 % of its rate: hand-offs over two stages); 3x3 on 512 channels at 7x7 627 -> 170; 11x11 on 256
-// channels at 28x28, batch 64, 14824 -> 4018 (198 TFLOP/s; 1.6 PFLOP/s of bf16 products with the strip ends, near the
-// power limit); 7x7 stride 2 on 3 channels at 224x224 642 -> 428.
+// Measured against the FFMA kernel (us, filter packed beforehand): 3x3 on 64 channels at 56x56, batch 128, 543 -> 201 (147
+// TFLOP/s; no pipe above 45 % of its rate: hand-offs over two stages); 3x3 on 512 channels at 7x7 627 -> 155; 11x11 on 256
+// channels at 28x28, batch 64, 14824 -> 3930 (202 TFLOP/s; 1.6 PFLOP/s of bf16 products with the strip ends, near the
+// power limit); 7x7 stride 2 on 3 channels at 224x224 642 -> 408.
 // A layer with few tiles is run by clusters of 2, 4 or 8 CTAs that share the stages of a tile and add their
 // registers through distributed shared memory, in rank order: 3x3 on 512 channels, one 7x7 image, 225 -> 31 us.
 #include <cuda_bf16.h>
