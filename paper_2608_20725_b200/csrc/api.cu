@@ -289,6 +289,16 @@ const char* im2win_conv_kernel_name(const im2win_shape* shape, im2win_dtype dtyp
   return "f16-gather";
 }
 
+// A testing aid, not part of the interface: how the run-staged kernel would run a layer.  Returns whether it can.
+int32_t im2win_f16_runs_form(const im2win_shape* shape, int32_t form[12]) {
+  Geometry g;
+  if (derive_geometry(shape, &g) != IM2WIN_OK) return 0;
+  const RunsPlan p = plan_f16_runs(g);
+  const int32_t v[12] = {p.mode, p.pair, p.planes, p.resident, p.teams, p.sr, p.octs, p.E, p.halo, p.bn, p.ntn, p.ntm};
+  for (int i = 0; i < 12; ++i) form[i] = v[i];
+  return p.eligible;
+}
+
 im2win_status im2win_workspace_size(const im2win_shape* shape, im2win_dtype dtype, size_t* window_bytes,
                                     size_t* scratch_bytes, int32_t* Ho, int32_t* Wo) {
   Geometry g;

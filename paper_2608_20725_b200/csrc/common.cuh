@@ -140,6 +140,7 @@ struct RunsPlan {
   int32_t units, octs, E, G, Wq, rows, halo, num_kb, nks_last;
   int32_t region, raw_slot, a_stage, slot_bytes, cols, planes, seg_bytes;
   int32_t bn, ntn, ntm, nwork, sa, sr, sb;
+  int32_t mode, teams;                 // how the staging warps read the raw slots, and how many teams they form
   int64_t VQ;
   size_t filter_bytes;
 };

@@ -83,6 +83,7 @@ struct alignas(64) RunsParams {
   int32_t foreign;                            // 1: zero filter elements meet elements that are not of the window
   int32_t halo, region, octs, raw_slot, a_stage;
   int32_t bn, ntn, nwork, sa, sr, sb, slot_bytes, resident;
+  int32_t teams;                              // of staging warps, a divisor of sr
   int32_t cols;                               // kernel columns in a filter slot
   int32_t ntm;                                // position tiles
   int32_t planes;                             // the least number of channel planes that is a multiple of 16 bytes; 0: bulk copies
@@ -209,7 +210,7 @@ struct Walk {
 //   WORDS      two elements of a row at a time: E even and every row on a 4-byte boundary (strides of 2)
 //   ROW_PAIRS  rows 2t and 2t + 1 of a 3-high kernel at stride 1 are six neighbouring elements, read as three words: images
 //              of an even number of virtual columns, so that no pair lies in two images
-// A team of warps covers the rows of the tile and takes every TEAMS-th slot as a whole; all loads of up to GROUP units
+// A team of warps covers the rows of the tile and takes every `teams`-th slot as a whole; all loads of up to GROUP units
 // are in flight together, and the slot is given back before the wait for a free S stage.  (A unit at a time, both
 // warpgroups on every slot, took 87 instructions and 560 cycles a unit: 3x3 stride 2 on 256 -> 512 channels at 28x28, batch
 // 128, 121 us.)
@@ -233,7 +234,7 @@ __device__ __forceinline__ void stage_tiles(const RunsParams& q, const Walk& wal
     else mbar_arrive(b.a_full0 + 8 * stage);
   };
   constexpr int ROWS = MODE == ROW_PAIRS ? 2 : 1;
-  constexpr int TEAM = 4 / ROWS, TEAMS = STAGING_WARPS / TEAM;
+  constexpr int TEAM = 4 / ROWS;
   constexpr int GROUP = MODE == WORDS ? 6 : 3;              // units in flight
   constexpr uint32_t STEP = MODE == QUAD ? 2 * ES : ES;     // from unit to unit of an octet, in a channel plane
   const int team = warp / TEAM, row = ((warp % TEAM) * 32 + lane) * ROWS;
@@ -248,9 +249,10 @@ __device__ __forceinline__ void stage_tiles(const RunsParams& q, const Walk& wal
   // rows below the tile: lane -> (row, unit of the group); one warp of the team has them, another one from slot to slot
   const bool halo_fits = q.halo * GROUP <= 32;
   bool ok = true;
-  // No more teams than raw slots: a team's next slot then reuses a buffer that was filled, for another team, before its last
-  // one was, and the parity it waits for is not that of two fills ago.
-  const int teams = q.sr < TEAMS ? q.sr : TEAMS;
+  // The number of teams divides the number of slots, so that a slot's fills all belong to one team.  It has waited for the one
+  // before when it waits for the next, whose parity then is not that of two fills ago.  (With slots that go from team to team
+  // that one may not have landed yet: copies of different slots land in any order.)
+  const int teams = q.teams;
   int sa = 0, sr = team, next = team < teams ? team : 1 << 30;    // (next: this team's next slot of the tile)
   uint32_t pa = 0, pr = 0;
   uint32_t turn = 0;
@@ -862,6 +864,9 @@ RunsPlan plan_f16_runs(const Geometry& g) {
   p.E = (int32_t)E;
   p.G = (g.Kw + g.s - 1) / g.s;
   p.quad = g.C <= 4;
+  const bool words = E % 2 == 0 && g.s * g.Kh % 2 == 0 && (int64_t)g.Wp * g.Kh % 2 == 0;
+  const bool pairs = E == 3 && g.s == 1 && (int64_t)g.Ho * g.Wp % 2 == 0;
+  p.mode = p.quad ? QUAD : (words ? WORDS : (pairs ? ROW_PAIRS : HALVES));
   p.units = (int32_t)(p.quad ? (E + 1) / 2 : (g.C + 7) / 8 * E);
   p.num_kb = (p.units + 7) / 8;
   p.nks_last = (p.units - 8 * (p.num_kb - 1) + 1) / 2;
@@ -937,7 +942,10 @@ RunsPlan plan_f16_runs(const Geometry& g) {
     if (!resident && p.sb < 3 && fits(p.sa, p.sr, 3)) p.sb = 3;
     if (fits(3, p.sr, p.sb)) p.sa = 3;                       // (before a fourth filter slot: 120 -> 107 us on a pair's tiles)
     if (!resident) while (p.sb < 4 && fits(p.sa, p.sr, p.sb + 1)) ++p.sb;
-    while (p.sr + 2 <= MAX_RAW && fits(p.sa, p.sr + 2, p.sb)) p.sr += 2;   // (even: the two copy warps alternate)
+    p.teams = p.mode == ROW_PAIRS && p.sr == 4 ? 4 : 2;
+    // (even: the two copy warps alternate; a multiple of the teams, see stage_tiles.  Four teams on four slots against three on
+    // six: 3x3 on 256 channels at 28x28, batch 64, 61 and 68 us, 64 -> 128 channels at 112x112 220 and 246)
+    while (p.sr + p.teams <= MAX_RAW && fits(p.sa, p.sr + p.teams, p.sb)) p.sr += p.teams;
     if (!resident) while (p.sb < MAX_B && fits(p.sa, p.sr, p.sb + 1)) ++p.sb;
     p.eligible = true;
   }
@@ -978,9 +986,7 @@ cudaError_t launch_conv_f16_runs(const uint16_t* window, float* y, void* scratch
   q.Co = g.Co; q.Kh = g.Kh; q.Kw = g.Kw; q.s = g.s;
   // kernel columns beyond Kw, channels beyond C in the last octet, the element beyond an odd E
   q.foreign = (g.Kw > g.s && g.Kw % g.s != 0) || (p.quad ? p.E % 2 != 0 : g.C % 8 != 0);
-  const bool words = p.E % 2 == 0 && g.s * g.Kh % 2 == 0 && (int64_t)g.Wp * g.Kh % 2 == 0;
-  const bool pairs = p.E == 3 && g.s == 1 && (int64_t)g.Ho * g.Wp % 2 == 0;
-  q.mode = p.quad ? QUAD : (words ? WORDS : (pairs ? ROW_PAIRS : HALVES));
+  q.mode = p.mode; q.teams = p.teams;
   q.E = p.E; q.G = p.G; q.units = p.units; q.quad = p.quad ? 1 : 0; q.num_kb = p.num_kb; q.nks_last = p.nks_last;
   q.halo = p.halo; q.region = p.region; q.octs = p.octs; q.raw_slot = p.raw_slot; q.a_stage = p.a_stage;
   q.bn = p.bn; q.ntn = p.ntn; q.nwork = p.nwork; q.sa = p.sa; q.sr = p.sr; q.sb = p.sb;

@@ -1,6 +1,8 @@
 """Helpers of the GPU parity tests: run the CUDA path through the C ABI with guard bands
 around every output buffer, and compare with the CPU oracle."""
+import ctypes
 import os
+from collections import namedtuple
 
 import numpy as np
 import torch
@@ -26,6 +28,21 @@ def assert_guards_intact(whole, numel, fill):
     ref = torch.full((GUARD,), fill, dtype=whole.dtype)
     assert torch.equal(head.view(torch.uint8), ref.view(torch.uint8)), "write before the buffer"
     assert torch.equal(tail.view(torch.uint8), ref.view(torch.uint8)), "write past the buffer"
+
+
+# How the run-staged fp16 kernel runs a layer: staging mode (0 to 3: elements, four channels, words of two, pairs of rows),
+# CTA pairs, channel planes in a row of the tiled copies (0: bulk copies), whether the filter stays in shared memory, teams of
+# staging warps and raw slots, octets of channels in a slot, elements of a virtual column, rows below a tile, channel tile
+# and number of channel and position tiles.
+RunsForm = namedtuple("RunsForm", "mode pair planes resident teams slots octs E halo bn ntn ntm")
+
+
+def runs_form(dims):
+    """The RunsForm of a layer (None: the kernel cannot take it).  Needs no GPU."""
+    fn = binding.lib().im2win_f16_runs_form
+    fn.argtypes, fn.restype = [ctypes.POINTER(binding.Shape), ctypes.POINTER(ctypes.c_int32)], ctypes.c_int32
+    form = (ctypes.c_int32 * 12)()
+    return RunsForm(*form) if fn(ctypes.byref(binding.as_shape(dims)), form) else None
 
 
 def gpu_transform(x_cpu: torch.Tensor, dims: dict) -> np.ndarray:

@@ -1,6 +1,8 @@
 """Tiles and rounds of the convolution kernels at the sizes where their rules change: a last round in parts of the channels
 (fp32 on the tensor cores), tiles of parts of strips (channel-innermost kernel), the ways the run-staged kernel brings
 its columns in."""
+from dataclasses import replace
+
 import numpy as np
 import pytest
 import torch
@@ -8,7 +10,7 @@ import torch
 import oracle
 from paper_2608_20725_b200 import binding, workloads
 from paper_2608_20725_b200.workloads import Layer
-from gpu_helpers import check_conv, gpu_conv, gpu_conv_nhwc, oracle_inputs
+from gpu_helpers import check_conv, gpu_conv, gpu_conv_nhwc, oracle_inputs, runs_form
 
 pytestmark = pytest.mark.gpu
 
@@ -99,3 +101,20 @@ def test_f16_runs_columns_and_copies(layer, tiled, pair, monkeypatch):
     y, _, _ = gpu_conv(x, f, dims, "f16")
     ref = torch.nn.functional.conv2d(x.half().double(), f.half().double(), stride=layer.stride, padding=layer.pad).numpy()
     assert np.array_equal(np.isfinite(y), np.isfinite(ref)) and np.array_equal(np.isnan(y), np.isnan(ref))
+
+
+# Four teams of staging warps on rings of four raw slots and of eight, which go round two to eight times in a tile
+@pytest.mark.parametrize("layer,slots", [
+    (L("teams_128", 3, 128, 28, 28, 128, 3, 3, 1, 1, 440), 4), (L("teams_64", 1, 64, 48, 50, 128, 3, 3, 1, 0, 441), 4),
+    (L("teams_pair", 2, 256, 20, 20, 256, 3, 3, 1, 1, 442), 4), (L("teams_to_64", 2, 128, 56, 30, 64, 3, 3, 1, 1, 443), 4),
+    (L("teams_eight", 2, 160, 30, 30, 16, 3, 3, 1, 1, 444), 8)], ids=lambda v: getattr(v, "name", str(v)))
+def test_f16_runs_teams_on_their_slots(layer, slots, monkeypatch):
+    monkeypatch.setenv("IM2WIN_F16_KERNEL", "runs")
+    dims = layer.dims()
+    form = runs_form(dims)
+    assert (form.mode, form.teams, form.slots) == (3, 4, slots) and layer.C // 8 >= 2 * slots
+    for seed in range(3):                                    # (new buffers every time: cold copies)
+        x, f = workloads.make_small_integer_inputs(replace(layer, seed=layer.seed + 100 * seed))
+        y, _, _ = gpu_conv(x, f, dims, "f16")
+        yr, _ = oracle.conv_direct(x.numpy(), f.numpy(), dims)
+        assert np.array_equal(y.astype(np.float64), yr)

@@ -1,12 +1,14 @@
 """Host-side rules of the kernel choice (no GPU): which fp32 kernel a layer takes, and that the scratch a caller was told
 to provide serves every smaller batch of the same layer, whatever kernel that one takes."""
 import os
+import random
 import subprocess
 import sys
 
 import pytest
 
 from conftest import ROOT
+from gpu_helpers import runs_form
 from paper_2608_20725_b200 import binding
 
 LAYERS = [(128, 64, 56, 56, 64, 3, 3, 1, 1), (128, 512, 7, 7, 512, 3, 3, 1, 1), (13, 37, 45, 61, 75, 5, 5, 2, 2),
@@ -74,3 +76,24 @@ def test_switches_are_fixed_when_the_library_is_loaded():
     env = {k: v for k, v in os.environ.items() if not k.startswith("IM2WIN_")}
     out = subprocess.run([sys.executable, "-c", code, ROOT], env=env, capture_output=True, text=True, check=True, timeout=300)
     assert out.stdout.split() == ["f32-split"]
+
+
+def test_run_staged_slots_keep_to_one_team():
+    """The team that takes a fill of a raw slot of the run-staged kernel has taken the fill before it too (it waits by the
+    parity of the fills): the number of teams divides the number of slots."""
+    rng = random.Random(7)
+    log = lambda lo, hi: round(lo * (hi / lo) ** rng.random())
+    seen = set()
+    layers = [(64, 256, 28, 28, 256, 3, 3, 1, 1), (64, 64, 112, 112, 128, 3, 3, 1, 0), (128, 128, 28, 28, 128, 3, 3, 1, 0),
+              (64, 128, 56, 56, 64, 3, 3, 1, 1)]
+    for _ in range(20000):
+        k, st = rng.choice([1, 2, 3, 3, 3, 4, 5, 7, 11]), rng.choice([1, 1, 1, 2, 2, 3, 4])
+        layers.append((log(1, 160), log(1, 600), log(7, 224), log(7, 224), log(1, 600), k,
+                       rng.choice([k, k, k, 1, 2, 3, 5]), st, rng.choice([0, k // 2])))
+    for layer in layers:
+        f = runs_form(layer)
+        if f is None:
+            continue
+        assert f.slots % f.teams == 0 and f.teams in (2, 4) and f.slots % 2 == 0, (layer, f)
+        seen.add((f.mode, f.teams))
+    assert {m for m, _ in seen} == {0, 1, 2, 3} and {t for _, t in seen} == {2, 4}
