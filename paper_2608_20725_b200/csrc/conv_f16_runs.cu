@@ -221,12 +221,16 @@ __device__ __forceinline__ int slot_row(const RunsParams& q, int x) {
 }
 
 enum StagingMode { HALVES, QUAD, WORDS, ROW_PAIRS };
+__host__ __device__ constexpr int group_of(int mode) { return mode == WORDS ? 6 : 3; }
+// Whether one warp reads the rows below a tile for a whole group of units at once; where they are more, HALVES and QUAD have
+// a form (MANY) that reads them unit by unit.
+__host__ __device__ constexpr bool halo_fits(int mode, int halo) { return halo * group_of(mode) <= 32; }
 
 struct StagingBarriers {
   uint32_t a_full0, a_empty0, raw_full0, raw_empty0;        // (a_full0 in a pair: the leader's, wherever it lies)
 };
 
-template <int MODE, bool PAIR>
+template <int MODE, bool MANY, bool PAIR>
 __device__ __forceinline__ void stage_tiles(const RunsParams& q, const Walk& walk, uint32_t a_ring, uint32_t raw_ring,
                                             const StagingBarriers& b, int warp, int lane, volatile uint32_t* abort_flag) {
   auto arrive_full = [&](int stage) {
@@ -235,7 +239,7 @@ __device__ __forceinline__ void stage_tiles(const RunsParams& q, const Walk& wal
   };
   constexpr int ROWS = MODE == ROW_PAIRS ? 2 : 1;
   constexpr int TEAM = 4 / ROWS;
-  constexpr int GROUP = MODE == WORDS ? 6 : 3;              // units in flight
+  constexpr int GROUP = group_of(MODE);                     // units in flight
   constexpr uint32_t STEP = MODE == QUAD ? 2 * ES : ES;     // from unit to unit of an octet, in a channel plane
   const int team = warp / TEAM, row = ((warp % TEAM) * 32 + lane) * ROWS;
   const int plane = (q.Ho * q.Wp + q.Wq * q.s - q.Wp) * q.Kh;     // (up to the end of the last virtual column)
@@ -246,8 +250,8 @@ __device__ __forceinline__ void stage_tiles(const RunsParams& q, const Walk& wal
   // (lanes 4 to 7 of eight store the second row of a pair first: the eight meet eight bank groups)
   const int second = ROWS == 2 ? (lane >> 2) & 1 : 0;
   const uint32_t dst0 = swizzled(row + second), dst1 = ROWS == 2 ? swizzled(row + 1 - second) : 0u;
-  // rows below the tile: lane -> (row, unit of the group); one warp of the team has them, another one from slot to slot
-  const bool halo_fits = q.halo * GROUP <= 32;
+  // rows below the tile: lane -> (row, unit of the group), with MANY lane -> row; one warp of the team has them, another one
+  // from slot to slot
   bool ok = true;
   // The number of teams divides the number of slots, so that a slot's fills all belong to one team.  It has waited for the one
   // before when it waits for the next, whose parity then is not that of two fills ago.  (With slots that go from team to team
@@ -282,7 +286,7 @@ __device__ __forceinline__ void stage_tiles(const RunsParams& q, const Walk& wal
     };
     uint32_t rb[8], hb[8];
     locate(row, rb);
-    const int he = q.halo > 0 && halo_fits ? lane / q.halo : GROUP, hrow = TILE_M + lane - he * q.halo;
+    const int he = MANY ? (lane < q.halo ? 0 : GROUP) : (q.halo > 0 ? lane / q.halo : GROUP), hrow = TILE_M + lane - he * q.halo;
     if (he < GROUP) {
       locate(hrow, hb);
 #pragma unroll
@@ -312,6 +316,10 @@ __device__ __forceinline__ void stage_tiles(const RunsParams& q, const Walk& wal
       if (!ok) break;
       uint32_t src = raw_ring + sr * q.raw_slot;
       const bool halo_turn = q.halo > 0 && (int)(turn % TEAM) == warp % TEAM;
+      auto give_back = [&]() {                               // everything of the slot is in registers
+        __syncwarp();
+        if (lane == 0) mbar_arrive(b.raw_empty0 + 8 * sr);
+      };
       const int here = nocts - next * octs < octs ? nocts - next * octs : octs;
       int j = next * octs * per_oct;                         // unit
       for (int o = 0; o < here && ok; ++o, src += 8u * q.region) {
@@ -345,28 +353,14 @@ __device__ __forceinline__ void stage_tiles(const RunsParams& q, const Walk& wal
 #pragma unroll
               for (int x = 0; x < 4; ++x) p[i][x] = __byte_perm(v[i][2 * x], v[i][2 * x + 1], 0x5410);
           }
-          if (halo_turn && he < n) {
+          auto read_low = [&](uint32_t from) {
 #pragma unroll
             for (int x = 0; x < 4; ++x)
-              hp[x] = __byte_perm(ld_shared_u16(at + hb[2 * x]), ld_shared_u16(at + hb[2 * x + 1]), 0x5410);
-          }
-          if (halo_turn && !halo_fits) {                     // many rows below the tile: unit by unit, lane = row
-            for (int i = 0; i < n && ok; ++i) {
-              go_to((j + i) >> 3);
-              if (!ok || lane >= q.halo) continue;
-              uint32_t lb[8], lp[4];
-              locate(TILE_M + lane, lb);
-#pragma unroll
-              for (int x = 0; x < 4; ++x)
-                lp[x] = __byte_perm(ld_shared_u16(at + i * STEP + lb[2 * x]), ld_shared_u16(at + i * STEP + lb[2 * x + 1]), 0x5410);
-              st_shared16(a_ring + sa * q.a_stage + (swizzled(TILE_M + lane) ^ (((j + i) & 7) << 4)), lp[0], lp[1], lp[2], lp[3]);
-            }
-            __syncwarp();
-          }
-          if (o == here - 1 && e0 + GROUP >= per_oct) {      // everything of the slot is in registers
-            __syncwarp();
-            if (lane == 0) mbar_arrive(b.raw_empty0 + 8 * sr);
-          }
+              hp[x] = __byte_perm(ld_shared_u16(from + hb[2 * x]), ld_shared_u16(from + hb[2 * x + 1]), 0x5410);
+          };
+          if (!MANY && halo_turn && he < n) read_low(at);
+          const bool last = o == here - 1 && e0 + GROUP >= per_oct;
+          if (last && !(MANY && halo_turn)) give_back();
 #pragma unroll
           for (int i = 0; i < GROUP; ++i) {
             if (i >= n) break;
@@ -380,8 +374,13 @@ __device__ __forceinline__ void stage_tiles(const RunsParams& q, const Walk& wal
             } else {
               st_shared16(stage + (dst0 ^ ch), p[i][0], p[i][1], p[i][2], p[i][3]);
             }
-            if (halo_turn && he == i) st_shared16(stage + (swizzled(hrow) ^ ch), hp[0], hp[1], hp[2], hp[3]);
+            if (MANY && halo_turn && he == 0) {              // (with its unit: the next one may belong to another stage)
+              read_low(at + i * STEP);
+              st_shared16(stage + (swizzled(hrow) ^ ch), hp[0], hp[1], hp[2], hp[3]);
+            }
+            if (!MANY && halo_turn && he == i) st_shared16(stage + (swizzled(hrow) ^ ch), hp[0], hp[1], hp[2], hp[3]);
           }
+          if (last && MANY && halo_turn && ok) give_back();
           j += n;
         }
       }
@@ -457,10 +456,13 @@ __global__ void __launch_bounds__(THREADS, 1) conv_f16_runs_kernel(const __grid_
     // ---------------- staging: raw runs -> S ------------------------------------------------------------
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_STAGING));
     const StagingBarriers b = {a_full_dst, a_empty0, raw_full0, raw_empty0};
-    if (q.mode == ROW_PAIRS) stage_tiles<ROW_PAIRS, PAIR>(q, walk, a_ring, raw_ring, b, warp, lane, &abort_flag);
-    else if (q.mode == WORDS) stage_tiles<WORDS, PAIR>(q, walk, a_ring, raw_ring, b, warp, lane, &abort_flag);
-    else if (q.mode == QUAD) stage_tiles<QUAD, PAIR>(q, walk, a_ring, raw_ring, b, warp, lane, &abort_flag);
-    else stage_tiles<HALVES, PAIR>(q, walk, a_ring, raw_ring, b, warp, lane, &abort_flag);
+    const bool many = !halo_fits(q.mode, q.halo);
+    if (q.mode == ROW_PAIRS) stage_tiles<ROW_PAIRS, false, PAIR>(q, walk, a_ring, raw_ring, b, warp, lane, &abort_flag);
+    else if (q.mode == WORDS) stage_tiles<WORDS, false, PAIR>(q, walk, a_ring, raw_ring, b, warp, lane, &abort_flag);
+    else if (q.mode == QUAD && many) stage_tiles<QUAD, true, PAIR>(q, walk, a_ring, raw_ring, b, warp, lane, &abort_flag);
+    else if (q.mode == QUAD) stage_tiles<QUAD, false, PAIR>(q, walk, a_ring, raw_ring, b, warp, lane, &abort_flag);
+    else if (many) stage_tiles<HALVES, true, PAIR>(q, walk, a_ring, raw_ring, b, warp, lane, &abort_flag);
+    else stage_tiles<HALVES, false, PAIR>(q, walk, a_ring, raw_ring, b, warp, lane, &abort_flag);
   } else if (warp < STAGING_WARPS + 4) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_MISC));
     if (warp == STAGING_WARPS && rank == 0) {
@@ -864,8 +866,8 @@ RunsPlan plan_f16_runs(const Geometry& g) {
   p.E = (int32_t)E;
   p.G = (g.Kw + g.s - 1) / g.s;
   p.quad = g.C <= 4;
-  const bool words = E % 2 == 0 && g.s * g.Kh % 2 == 0 && (int64_t)g.Wp * g.Kh % 2 == 0;
-  const bool pairs = E == 3 && g.s == 1 && (int64_t)g.Ho * g.Wp % 2 == 0;
+  const bool words = E % 2 == 0 && g.s * g.Kh % 2 == 0 && (int64_t)g.Wp * g.Kh % 2 == 0 && halo_fits(WORDS, p.G - 1);
+  const bool pairs = E == 3 && g.s == 1 && (int64_t)g.Ho * g.Wp % 2 == 0 && halo_fits(ROW_PAIRS, p.G - 1);
   p.mode = p.quad ? QUAD : (words ? WORDS : (pairs ? ROW_PAIRS : HALVES));
   p.units = (int32_t)(p.quad ? (E + 1) / 2 : (g.C + 7) / 8 * E);
   p.num_kb = (p.units + 7) / 8;
