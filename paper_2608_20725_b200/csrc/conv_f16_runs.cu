@@ -479,9 +479,11 @@ __global__ void __launch_bounds__(THREADS, 1) conv_f16_runs_kernel(const __grid_
       uint32_t a_seen = 0, b_seen = 0, acc_seen = 0;
       // (testing aid: the commit of the first tile left out; looked up while its first stage is on its way)
       uint32_t drop = blockIdx.x == 0 ? *reinterpret_cast<volatile uint32_t*>(q.status + 2) : 0u;
+      // (in a pair the other CTA arrives on all three kinds: cluster scope)
       auto need = [&](uint32_t bar, uint32_t parity, uint32_t seen) {
-        return mbar_wait_unless_seen(bar, parity, seen, &abort_flag, q.status);
+        return mbar_wait_unless_seen<PAIR>(bar, parity, seen, &abort_flag, q.status);
       };
+      auto look = [&](uint32_t bar, uint32_t parity) { return PAIR ? mbar_test_wait_cluster(bar, parity) : mbar_test_wait(bar, parity); };
       auto commit = [&](uint32_t bar) {
         if (PAIR) umma_commit_pair(bar);
         else umma_commit(bar);
@@ -511,10 +513,10 @@ __global__ void __launch_bounds__(THREADS, 1) conv_f16_runs_kernel(const __grid_
             if (fetch_b) {
               ok = need(b_full0 + 8 * slot, pb, b_seen);
               if (!ok) break;
-              b_seen = mbar_test_wait(b_full0 + 8 * nslot, npb);
+              b_seen = look(b_full0 + 8 * nslot, npb);
             }
-            if (last) acc_seen = mbar_test_wait(acc_empty0 + 8 * ((ac + 1) & (NACC - 1)), (((ac + 1) >> ACC_LOG) & 1) ^ 1);
-            if (last_unit) a_seen = mbar_test_wait(a_full0 + 8 * nsa, npa);
+            if (last) acc_seen = look(acc_empty0 + 8 * ((ac + 1) & (NACC - 1)), (((ac + 1) >> ACC_LOG) & 1) ^ 1);
+            if (last_unit) a_seen = look(a_full0 + 8 * nsa, npa);
             const uint32_t b_lo = b_lo0 + (uint32_t)(slot * (q.slot_bytes >> 4));
             if (leader) {
               if (q.cols == 3) issue_slot<3, PAIR>(nks, d, a_view, b_lo, b_step, idesc, more);

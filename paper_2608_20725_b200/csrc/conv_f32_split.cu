@@ -392,7 +392,7 @@ __global__ void __launch_bounds__(Form<BNMAX, PWG>::THREADS, 1) conv_f32_split_k
       // (testing aid: the first commit of an accumulator left out; looked up while the first stage is on its way)
       uint32_t drop = blockIdx.x == 0 ? *reinterpret_cast<volatile uint32_t*>(q.status + 2) : 0u;
       auto need = [&](uint32_t bar, uint32_t parity, uint32_t seen) {
-        return mbar_wait_unless_seen(bar, parity, seen, &abort_flag, q.status);
+        return mbar_wait_unless_seen<false>(bar, parity, seen, &abort_flag, q.status);
       };
       auto next_slot = [&](int& sl, uint32_t& ph) { if (++sl == q.sb) { sl = 0; ph ^= 1u; } };
       for (int w = w_first; w < q.nwork && ok; w += w_step) {

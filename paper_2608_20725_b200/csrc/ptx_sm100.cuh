@@ -126,12 +126,6 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     if (mbar_try_wait(bar, parity)) return true;
   return mbar_wait_slow<false>(bar, parity, abort_flag, status);
 }
-// A warp's wait for a barrier that an earlier mbar_test_wait may have found complete already (the whole warp calls it).
-__device__ __forceinline__ bool mbar_wait_unless_seen(uint32_t bar, uint32_t parity, uint32_t seen, volatile uint32_t* abort_flag,
-                                                      uint32_t* status) {
-  if (__all_sync(0xffffffffu, seen != 0u)) return true;
-  return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, status));
-}
 __device__ __forceinline__ void st_shared16(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
   asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
 }
@@ -365,6 +359,26 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity,
   for (uint32_t i = 0; i < SPIN_CHUNK; ++i)
     if (mbar_try_wait_cluster(bar, parity)) return true;
   return mbar_wait_slow<true>(bar, parity, abort_flag, status);
+}
+// One look at such a barrier.
+__device__ __forceinline__ uint32_t mbar_test_wait_cluster(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.test_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return ok;
+}
+// A warp's wait for a barrier that an earlier mbar_test_wait (CLUSTER: mbar_test_wait_cluster) may have found complete already
+// (the whole warp calls it).
+template <bool CLUSTER>
+__device__ __forceinline__ bool mbar_wait_unless_seen(uint32_t bar, uint32_t parity, uint32_t seen, volatile uint32_t* abort_flag,
+                                                      uint32_t* status) {
+  if (__all_sync(0xffffffffu, seen != 0u)) return true;
+  return __all_sync(0xffffffffu, CLUSTER ? mbar_wait_cluster(bar, parity, abort_flag, status) : mbar_wait(bar, parity, abort_flag, status));
 }
 __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
