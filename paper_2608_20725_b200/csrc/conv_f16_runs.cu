@@ -29,8 +29,8 @@
 // What bounds it: no single pipe.  With the read-back, the S stores, the MMAs and the output stores all left out, what remains
 // (copies, hand-offs, the staging warps' arithmetic) still takes four fifths of the time: 86 of 109 us for 3x3 on 64 channels at
 // 56x56, batch 128.  Measured: 3x3 stride 2 on 256 -> 512 channels at 28x28, batch 128, 140 us with the gathering kernel,
-// 112 with a unit at a time, no pairs and two S stages, now 97 (610 TFLOP/s); 3x3 on 256 channels at 28x28, batch 64, 70 -> 58;
-// 64 -> 128 channels at 112x112, batch 64, 256 -> 194; 5x5 stride 2 on 37 -> 75 channels at 45x61, batch 13, 27 (gathering) and 15.
+// 112 with a unit at a time, no pairs and two S stages, now 88 (670 TFLOP/s); 3x3 on 256 channels at 28x28, batch 64, 70 -> 58;
+// 64 -> 128 channels at 112x112, batch 64, 256 -> 194; 5x5 stride 2 on 37 -> 75 channels at 45x61, batch 13, 27 (gathering) and 13.
 // Eight staging warps: twelve or sixteen, with four epilogue warps, gave 111 and 117 us where eight gave 113, and 115 and 125 us
 // where eight gave 103.
 #include <cuda_fp16.h>
@@ -79,7 +79,6 @@ struct alignas(64) RunsParams {
   int32_t C, Wp, Wq, Ho, Wo, HoWo, Co, Kh, Kw, s;
   int32_t E, G, units, num_kb, nks_last;      // units: of eight k2
   int32_t quad;                               // 1: up to four channels, a unit is four channels at two e
-  int32_t mode;                               // how the staging warps read the raw runs (StagingMode)
   int32_t foreign;                            // 1: zero filter elements meet elements that are not of the window
   int32_t halo, region, octs, raw_slot, a_stage;
   int32_t bn, ntn, nwork, sa, sr, sb, slot_bytes, resident;
@@ -204,33 +203,53 @@ struct Walk {
   }
 };
 
-// The staging warps: raw runs -> S, thread = row (or two neighbouring rows).
-//   HALVES     an element at a time: any alignment
-//   QUAD       the same with units of four channels at two e (up to four channels)
-//   WORDS      two elements of a row at a time: E even and every row on a 4-byte boundary (strides of 2)
-//   ROW_PAIRS  rows 2t and 2t + 1 of a 3-high kernel at stride 1 are six neighbouring elements, read as three words: images
-//              of an even number of virtual columns, so that no pair lies in two images
-// A team of warps covers the rows of the tile and takes every `teams`-th slot as a whole; all loads of up to GROUP units
-// are in flight together, and the slot is given back before the wait for a free S stage.  (A unit at a time, both
-// warpgroups on every slot, took 87 instructions and 560 cycles a unit: 3x3 stride 2 on 256 -> 512 channels at 28x28, batch
-// 128, 121 us.)
 // Where channel x of an octet lies in a raw slot: tiled copies bring every `planes`-th channel at a time.
 __device__ __forceinline__ int slot_row(const RunsParams& q, int x) {
   if (q.planes <= 1) return x;
   return q.planes == 2 ? (x & 1) * 4 + (x >> 1) : (x & 3) * 2 + (x >> 2);
 }
 
-enum StagingMode { HALVES, QUAD, WORDS, ROW_PAIRS };
-__host__ __device__ constexpr int group_of(int mode) { return mode == WORDS ? 6 : 3; }
-// Whether one warp reads the rows below a tile for a whole group of units at once; where they are more, HALVES and QUAD have
-// a form (MANY) that reads them unit by unit.
-__host__ __device__ constexpr bool halo_fits(int mode, int halo) { return halo * group_of(mode) <= 32; }
+// The staging warps: raw runs -> S, thread = row (or two neighbouring rows).
+//   HALVES     an element at a time: any alignment
+//   WORDS      two elements of a row at a time: E even and every row on a 4-byte boundary (strides of 2)
+//   ROW_PAIRS  rows 2t and 2t + 1 of a 3-high kernel at stride 1 are six neighbouring elements, read as three words: images
+//              of an even number of virtual columns, so that no pair lies in two images
+//   UNITS      an element and a unit at a time, both warpgroups on every slot: any layer (stage_units)
+// The kernel is compiled for each by itself: small layers pay for code that is skipped (in one kernel for all, 8 to 9 us where
+// a kernel of UNITS alone takes 6 to 7).
+enum StagingMode { HALVES, WORDS, ROW_PAIRS, UNITS };
+constexpr int group_of(int mode) { return mode == WORDS ? 6 : 3; }
 
 struct StagingBarriers {
   uint32_t a_full0, a_empty0, raw_full0, raw_empty0;        // (a_full0 in a pair: the leader's, wherever it lies)
 };
 
-template <int MODE, bool MANY, bool PAIR>
+// Place of the first element of virtual position vq in channel x of a slot's octet: byte inside the raw slot.
+__device__ __forceinline__ void locate_row(const RunsParams& q, const TileRuns& tr, int plane, uint32_t vq, bool quad, uint32_t (&rb)[8]) {
+  uint32_t off = 0, phase = 0;
+  if (vq < q.VQ) {                                           // dead rows read whatever lies at the start: they are dropped
+    uint32_t n;
+    int ho, i;
+    split_q(q, vq, n, ho, i);
+    const int g = (int)(n - tr.n0), start = g == 0 ? tr.start0 : 0;
+    if (q.planes) off = g * q.seg_bytes;
+    else if (g > 0) off = run_size(plane - tr.start0) + (g - 1) * run_size(plane);
+    off += ((ho * q.Wp + i * q.s) * q.Kh - start) * ES;
+    phase = (uint32_t)((int64_t)n * q.img_bytes + (int64_t)start * ES);
+  }
+#pragma unroll
+  for (int x = 0; x < 8; ++x) rb[x] = off + slot_row(q, x) * q.region + ((phase + (uint32_t)x * (uint32_t)q.chan_bytes) & 15u);
+  if (quad) {
+#pragma unroll
+    for (int x = 0; x < 4; ++x) rb[4 + x] = rb[x] + ES;
+  }
+}
+
+// A team of warps covers the rows of the tile and takes every `teams`-th slot as a whole; all loads of up to GROUP units
+// are in flight together, and the slot is given back before the wait for a free S stage.  (A unit at a time, both
+// warpgroups on every slot, took 87 instructions and 560 cycles a unit: 3x3 stride 2 on 256 -> 512 channels at 28x28, batch
+// 128, 121 us.)
+template <int MODE, bool PAIR>
 __device__ __forceinline__ void stage_tiles(const RunsParams& q, const Walk& walk, uint32_t a_ring, uint32_t raw_ring,
                                             const StagingBarriers& b, int warp, int lane, volatile uint32_t* abort_flag) {
   auto arrive_full = [&](int stage) {
@@ -239,19 +258,16 @@ __device__ __forceinline__ void stage_tiles(const RunsParams& q, const Walk& wal
   };
   constexpr int ROWS = MODE == ROW_PAIRS ? 2 : 1;
   constexpr int TEAM = 4 / ROWS;
-  constexpr int GROUP = group_of(MODE);                     // units in flight
-  constexpr uint32_t STEP = MODE == QUAD ? 2 * ES : ES;     // from unit to unit of an octet, in a channel plane
+  constexpr int GROUP = MODE == WORDS ? 6 : 3;              // units in flight
   const int team = warp / TEAM, row = ((warp % TEAM) * 32 + lane) * ROWS;
   const int plane = (q.Ho * q.Wp + q.Wq * q.s - q.Wp) * q.Kh;     // (up to the end of the last virtual column)
-  const int per_oct = MODE == QUAD ? q.units : q.E;
-  const int nocts = MODE == QUAD ? 1 : q.units / q.E, octs = MODE == QUAD ? 1 : q.octs;
+  const int per_oct = q.E, nocts = q.units / q.E, octs = q.octs;
   const int nslots = (nocts + octs - 1) / octs;
   auto swizzled = [](int r) { return (uint32_t)(r * 128 + ((r & 7) << 4)); };
   // (lanes 4 to 7 of eight store the second row of a pair first: the eight meet eight bank groups)
   const int second = ROWS == 2 ? (lane >> 2) & 1 : 0;
   const uint32_t dst0 = swizzled(row + second), dst1 = ROWS == 2 ? swizzled(row + 1 - second) : 0u;
-  // rows below the tile: lane -> (row, unit of the group), with MANY lane -> row; one warp of the team has them, another one
-  // from slot to slot
+  // rows below the tile: lane -> (row, unit of the group); one warp of the team has them, another one from slot to slot
   bool ok = true;
   // The number of teams divides the number of slots, so that a slot's fills all belong to one team.  It has waited for the one
   // before when it waits for the next, whose parity then is not that of two fills ago.  (With slots that go from team to team
@@ -263,34 +279,14 @@ __device__ __forceinline__ void stage_tiles(const RunsParams& q, const Walk& wal
   for (int w = walk.first; w < q.nwork && ok; w += walk.step) {
     const uint32_t q0 = walk.start(q, w);
     const TileRuns tr = tile_runs(q, q0);
-    // Place of row r's first element in channel x of a slot's octet: byte inside the raw slot.
-    auto locate = [&](int r, uint32_t (&rb)[8]) {
-      uint32_t off = 0, phase = 0;
-      const uint32_t vq = q0 + r;
-      if (vq < q.VQ) {                                       // dead rows read whatever lies at the start: they are dropped
-        uint32_t n;
-        int ho, i;
-        split_q(q, vq, n, ho, i);
-        const int g = (int)(n - tr.n0), start = g == 0 ? tr.start0 : 0;
-        if (q.planes) off = g * q.seg_bytes;
-        else if (g > 0) off = run_size(plane - tr.start0) + (g - 1) * run_size(plane);
-        off += ((ho * q.Wp + i * q.s) * q.Kh - start) * ES;
-        phase = (uint32_t)((int64_t)n * q.img_bytes + (int64_t)start * ES);
-      }
-#pragma unroll
-      for (int x = 0; x < 8; ++x) rb[x] = off + slot_row(q, x) * q.region + ((phase + (uint32_t)x * (uint32_t)q.chan_bytes) & 15u);
-      if (MODE == QUAD) {
-#pragma unroll
-        for (int x = 0; x < 4; ++x) rb[4 + x] = rb[x] + ES;
-      }
-    };
+    auto locate = [&](int r, uint32_t (&at)[8]) { locate_row(q, tr, plane, q0 + r, false, at); };
     uint32_t rb[8], hb[8];
     locate(row, rb);
-    const int he = MANY ? (lane < q.halo ? 0 : GROUP) : (q.halo > 0 ? lane / q.halo : GROUP), hrow = TILE_M + lane - he * q.halo;
+    const int he = q.halo > 0 ? lane / q.halo : GROUP, hrow = TILE_M + lane - he * q.halo;
     if (he < GROUP) {
       locate(hrow, hb);
 #pragma unroll
-      for (int x = 0; x < 8; ++x) hb[x] += he * STEP;
+      for (int x = 0; x < 8; ++x) hb[x] += he * ES;
     }
     int kb = 0;                                              // S stage this warp is at, and whether it may write to it
     bool held = false;
@@ -316,16 +312,12 @@ __device__ __forceinline__ void stage_tiles(const RunsParams& q, const Walk& wal
       if (!ok) break;
       uint32_t src = raw_ring + sr * q.raw_slot;
       const bool halo_turn = q.halo > 0 && (int)(turn % TEAM) == warp % TEAM;
-      auto give_back = [&]() {                               // everything of the slot is in registers
-        __syncwarp();
-        if (lane == 0) mbar_arrive(b.raw_empty0 + 8 * sr);
-      };
       const int here = nocts - next * octs < octs ? nocts - next * octs : octs;
       int j = next * octs * per_oct;                         // unit
       for (int o = 0; o < here && ok; ++o, src += 8u * q.region) {
         for (int e0 = 0; e0 < per_oct && ok; e0 += GROUP) {
           const int n = per_oct - e0 < GROUP ? per_oct - e0 : GROUP;
-          const uint32_t at = src + e0 * STEP;
+          const uint32_t at = src + e0 * ES;
           uint32_t p[GROUP * ROWS][4], hp[4] = {};
           if constexpr (MODE == WORDS || MODE == ROW_PAIRS) {
             uint32_t v[3][8];                                // (beyond the octet's last unit: place 0 again)
@@ -344,7 +336,7 @@ __device__ __forceinline__ void stage_tiles(const RunsParams& q, const Walk& wal
             uint32_t v[GROUP][8];
 #pragma unroll
             for (int i = 0; i < GROUP; ++i) {
-              const uint32_t from = i < n ? at + i * STEP : at;
+              const uint32_t from = i < n ? at + i * ES : at;
 #pragma unroll
               for (int x = 0; x < 8; ++x) v[i][x] = ld_shared_u16(from + rb[x]);
             }
@@ -353,14 +345,15 @@ __device__ __forceinline__ void stage_tiles(const RunsParams& q, const Walk& wal
 #pragma unroll
               for (int x = 0; x < 4; ++x) p[i][x] = __byte_perm(v[i][2 * x], v[i][2 * x + 1], 0x5410);
           }
-          auto read_low = [&](uint32_t from) {
+          if (halo_turn && he < n) {
 #pragma unroll
             for (int x = 0; x < 4; ++x)
-              hp[x] = __byte_perm(ld_shared_u16(from + hb[2 * x]), ld_shared_u16(from + hb[2 * x + 1]), 0x5410);
-          };
-          if (!MANY && halo_turn && he < n) read_low(at);
-          const bool last = o == here - 1 && e0 + GROUP >= per_oct;
-          if (last && !(MANY && halo_turn)) give_back();
+              hp[x] = __byte_perm(ld_shared_u16(at + hb[2 * x]), ld_shared_u16(at + hb[2 * x + 1]), 0x5410);
+          }
+          if (o == here - 1 && e0 + GROUP >= per_oct) {      // everything of the slot is in registers
+            __syncwarp();
+            if (lane == 0) mbar_arrive(b.raw_empty0 + 8 * sr);
+          }
 #pragma unroll
           for (int i = 0; i < GROUP; ++i) {
             if (i >= n) break;
@@ -374,13 +367,8 @@ __device__ __forceinline__ void stage_tiles(const RunsParams& q, const Walk& wal
             } else {
               st_shared16(stage + (dst0 ^ ch), p[i][0], p[i][1], p[i][2], p[i][3]);
             }
-            if (MANY && halo_turn && he == 0) {              // (with its unit: the next one may belong to another stage)
-              read_low(at + i * STEP);
-              st_shared16(stage + (swizzled(hrow) ^ ch), hp[0], hp[1], hp[2], hp[3]);
-            }
-            if (!MANY && halo_turn && he == i) st_shared16(stage + (swizzled(hrow) ^ ch), hp[0], hp[1], hp[2], hp[3]);
+            if (halo_turn && he == i) st_shared16(stage + (swizzled(hrow) ^ ch), hp[0], hp[1], hp[2], hp[3]);
           }
-          if (last && MANY && halo_turn && ok) give_back();
           j += n;
         }
       }
@@ -403,7 +391,80 @@ __device__ __forceinline__ void stage_tiles(const RunsParams& q, const Walk& wal
   }
 }
 
-template <int BNMAX, bool PAIR>
+// The form for layers that give the teams too little to share out (see plan_f16_runs) or have more rows below a tile than a warp
+// can read for a group of units.  Warpgroup wg takes every second unit; every warp passes every stage and every slot in order, so no wait by phase
+// parity can run ahead.
+template <bool PAIR>
+__device__ __forceinline__ void stage_units(const RunsParams& q, const Walk& walk, uint32_t a_ring, uint32_t raw_ring,
+                                            const StagingBarriers& b, int warp, int lane, volatile uint32_t* abort_flag) {
+  const int wg = warp >> 2, row = (warp & 3) * 32 + lane;
+  const int plane = (q.Ho * q.Wp + q.Wq * q.s - q.Wp) * q.Kh;     // (up to the end of the last virtual column)
+  const int per_slot = q.quad ? q.units : q.octs * q.E;
+  const uint32_t oct_step = 8u * q.region - (uint32_t)(q.E - 1) * ES, unit_step = q.quad ? 2u * ES : ES;
+  bool ok = true;
+  int sa = 0, sr = 0;
+  uint32_t pa = 0, pr = 0;
+  for (int w = walk.first; w < q.nwork && ok; w += walk.step) {
+    const uint32_t q0 = walk.start(q, w);
+    const TileRuns tr = tile_runs(q, q0);
+    uint32_t rb[8], hb[8];
+    locate_row(q, tr, plane, q0 + row, q.quad, rb);
+    if (lane < q.halo) locate_row(q, tr, plane, q0 + TILE_M + lane, q.quad, hb);
+    uint32_t src = 0;                                        // of the current unit; inside the slot: its number, and its e
+    int in_slot = 0, e = 0;
+    for (int kb = 0; kb < q.num_kb && ok; ++kb) {
+      ok = mbar_wait(b.a_empty0 + 8 * sa, pa ^ 1u, abort_flag, q.status);
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) break;
+      const uint32_t stage = a_ring + sa * q.a_stage;
+      const int n_units = q.units - 8 * kb < 8 ? q.units - 8 * kb : 8;
+      for (int ch = 0; ch < n_units; ++ch) {
+        if (in_slot == 0) {
+          ok = mbar_wait(b.raw_full0 + 8 * sr, pr, abort_flag, q.status);
+          ok = __all_sync(0xffffffffu, ok);
+          if (!ok) break;
+          src = raw_ring + sr * q.raw_slot;
+          e = 0;
+        }
+        if ((ch & 1) == wg) {
+          auto unit = [&](const uint32_t (&at)[8], int srow) {
+            uint32_t v[8];
+#pragma unroll
+            for (int x = 0; x < 8; ++x) v[x] = ld_shared_u16(src + at[x]);
+            st_shared16(stage + srow * 128 + ((ch ^ (srow & 7)) << 4), v[0] | (v[1] << 16), v[2] | (v[3] << 16),
+                        v[4] | (v[5] << 16), v[6] | (v[7] << 16));
+          };
+          unit(rb, row);
+          // the rows below the tile: lanes of one of the warpgroup's warps, another one from unit to unit
+          if ((ch >> 1) == (warp & 3) && lane < q.halo) unit(hb, TILE_M + lane);
+        }
+        if (++in_slot == per_slot || 8 * kb + ch == q.units - 1) {
+          __syncwarp();
+          if (lane == 0) mbar_arrive(b.raw_empty0 + 8 * sr);
+          if (++sr == q.sr) { sr = 0; pr ^= 1u; }
+          in_slot = 0;
+        }
+        ++e;
+        src += e == q.E ? oct_step : unit_step;
+        if (e == q.E) e = 0;
+      }
+      if (!ok) break;
+      if ((n_units & 1) != 0 && wg == 1) {                   // zeros up to the end of the MMA's last step
+        st_shared16(stage + row * 128 + ((n_units ^ (row & 7)) << 4), 0u, 0u, 0u, 0u);
+        if (lane < q.halo) st_shared16(stage + (TILE_M + lane) * 128 + ((n_units ^ (lane & 7)) << 4), 0u, 0u, 0u, 0u);
+      }
+      fence_proxy_async_smem();
+      __syncwarp();
+      if (lane == 0) {
+        if (PAIR) mbar_arrive_cluster(b.a_full0 + 8 * sa);
+        else mbar_arrive(b.a_full0 + 8 * sa);
+      }
+      if (++sa == q.sa) { sa = 0; pa ^= 1u; }
+    }
+  }
+}
+
+template <int BNMAX, bool PAIR, int MODE>
 __global__ void __launch_bounds__(THREADS, 1) conv_f16_runs_kernel(const __grid_constant__ RunsParams q) {
   constexpr int NACC = 512 / BNMAX, ACC_LOG = NACC == 2 ? 1 : (NACC == 4 ? 2 : 3);      // ring of accumulators in tensor memory
   extern __shared__ unsigned char smem_dyn[];
@@ -431,7 +492,7 @@ __global__ void __launch_bounds__(THREADS, 1) conv_f16_runs_kernel(const __grid_
   if (threadIdx.x == 0) {
     abort_flag = 0u;
     for (int i = 0; i < MAX_A; ++i) { mbar_init(a_full0 + 8 * i, PAIR ? 2 * STAGING_WARPS : STAGING_WARPS); mbar_init(a_empty0 + 8 * i, 1); }
-    for (int i = 0; i < MAX_RAW; ++i) { mbar_init(raw_full0 + 8 * i, 1); mbar_init(raw_empty0 + 8 * i, q.mode == ROW_PAIRS ? 2 : 4); }
+    for (int i = 0; i < MAX_RAW; ++i) { mbar_init(raw_full0 + 8 * i, 1); mbar_init(raw_empty0 + 8 * i, MODE == UNITS ? STAGING_WARPS : (MODE == ROW_PAIRS ? 2 : 4)); }
     // (the leader's b_full: its own copy and word from the other CTA's)
     for (int i = 0; i < MAX_B; ++i) { mbar_init(b_full0 + 8 * i, PAIR && rank == 0 ? 2 : 1); mbar_init(b_empty0 + 8 * i, 1); }
     for (int i = 0; i < MAX_ACC; ++i) { mbar_init(acc_full0 + 8 * i, 1); mbar_init(acc_empty0 + 8 * i, PAIR ? 16 : 8); }
@@ -456,13 +517,8 @@ __global__ void __launch_bounds__(THREADS, 1) conv_f16_runs_kernel(const __grid_
     // ---------------- staging: raw runs -> S ------------------------------------------------------------
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_STAGING));
     const StagingBarriers b = {a_full_dst, a_empty0, raw_full0, raw_empty0};
-    const bool many = !halo_fits(q.mode, q.halo);
-    if (q.mode == ROW_PAIRS) stage_tiles<ROW_PAIRS, false, PAIR>(q, walk, a_ring, raw_ring, b, warp, lane, &abort_flag);
-    else if (q.mode == WORDS) stage_tiles<WORDS, false, PAIR>(q, walk, a_ring, raw_ring, b, warp, lane, &abort_flag);
-    else if (q.mode == QUAD && many) stage_tiles<QUAD, true, PAIR>(q, walk, a_ring, raw_ring, b, warp, lane, &abort_flag);
-    else if (q.mode == QUAD) stage_tiles<QUAD, false, PAIR>(q, walk, a_ring, raw_ring, b, warp, lane, &abort_flag);
-    else if (many) stage_tiles<HALVES, true, PAIR>(q, walk, a_ring, raw_ring, b, warp, lane, &abort_flag);
-    else stage_tiles<HALVES, false, PAIR>(q, walk, a_ring, raw_ring, b, warp, lane, &abort_flag);
+    if constexpr (MODE == UNITS) stage_units<PAIR>(q, walk, a_ring, raw_ring, b, warp, lane, &abort_flag);
+    else stage_tiles<MODE, PAIR>(q, walk, a_ring, raw_ring, b, warp, lane, &abort_flag);
   } else if (warp < STAGING_WARPS + 4) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_MISC));
     if (warp == STAGING_WARPS && rank == 0) {
@@ -613,17 +669,19 @@ __global__ void __launch_bounds__(THREADS, 1) conv_f16_runs_kernel(const __grid_
           ty = (int)(((int64_t)(tr.n0 + g) * q.C + 8 * o) / q.planes);
           to = o < q.octs ? g * q.seg_bytes + (8 * o + r * (8 / q.planes)) * q.region : 0;
           oct = o;
-        } else if (lane < items) {
-          run_of(lane, from0, size0, to0);
-          total = size0;
+        } else if (MODE != UNITS) {
+          if (lane < items) {
+            run_of(lane, from0, size0, to0);
+            total = size0;
+          }
+          for (int it = lane + 32; it < items; it += 32) {
+            int64_t from;
+            uint32_t size, to;
+            run_of(it, from, size, to);
+            total += size;
+          }
+          total = __reduce_add_sync(0xffffffffu, total);
         }
-        for (int it = lane + 32; it < items && q.planes == 0; it += 32) {
-          int64_t from;
-          uint32_t size, to;
-          run_of(it, from, size, to);
-          total += size;
-        }
-        total = __reduce_add_sync(0xffffffffu, total);
         // bytes behind the first slot's last run, up to the next 16-byte boundary, that are still of the tensor
         const int64_t spare = q.win_bytes - 15 - ((int64_t)tr.n1 * q.img_bytes + (per_slot - 1) * q.chan_bytes + (int64_t)tr.end1 * ES);
         for (int sl = 0; sl < nslots; ++sl, ++sc) {
@@ -645,7 +703,7 @@ __global__ void __launch_bounds__(THREADS, 1) conv_f16_runs_kernel(const __grid_
             continue;
           }
           const int64_t ahead = (int64_t)sl * per_slot * q.chan_bytes;
-          if ((sl + 1) * per_slot <= q.C && ahead <= spare) {
+          if (MODE != UNITS && (sl + 1) * per_slot <= q.C && ahead <= spare) {
             const uint32_t bar = raw_full0 + 8 * sr, slot = sr * q.raw_slot;
             const unsigned char* win = q.win + ahead;
             if (lane == 0) mbar_arrive_expect_tx(bar, total);
@@ -661,7 +719,7 @@ __global__ void __launch_bounds__(THREADS, 1) conv_f16_runs_kernel(const __grid_
             if (++sr == q.sr) { sr = 0; pr ^= 1u; }
             continue;
           }
-          // a slot that is not full, or may reach the end of the tensor
+          // a slot that is not full or may reach the end of the tensor, or one of few (UNITS: not worth working out ahead)
           const uint32_t bar = raw_full0 + 8 * sr;
           const int c0 = sl * per_slot, nc = q.C - c0 < per_slot ? q.C - c0 : per_slot;
           int seg_off = 0;
@@ -814,18 +872,26 @@ __global__ void __launch_bounds__(256) pack_f16_runs_kernel(const uint16_t* __re
   }
 }
 
-template <int BNMAX, bool PAIR>
-cudaError_t launch_form(const RunsParams& q, int smem, cudaStream_t stream) {
+template <int BNMAX, bool PAIR, int MODE>
+cudaError_t launch_mode(const RunsParams& q, int smem, cudaStream_t stream) {
   static bool attr_done[64] = {};
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
   if (!attr_done[dev]) {
-    cudaError_t e = cudaFuncSetAttribute(conv_f16_runs_kernel<BNMAX, PAIR>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRunsSmem);
+    cudaError_t e = cudaFuncSetAttribute(conv_f16_runs_kernel<BNMAX, PAIR, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRunsSmem);
     if (e != cudaSuccess) return e;
     attr_done[dev] = true;
   }
   const int most = PAIR ? 74 : 148, grid = (q.nwork < most ? q.nwork : most) * (PAIR ? 2 : 1);
-  return launch_after_previous(conv_f16_runs_kernel<BNMAX, PAIR>, grid, PAIR ? 2 : 1, THREADS, smem, stream, q);
+  return launch_after_previous(conv_f16_runs_kernel<BNMAX, PAIR, MODE>, grid, PAIR ? 2 : 1, THREADS, smem, stream, q);
+}
+
+template <int BNMAX, bool PAIR>
+cudaError_t launch_form(int mode, const RunsParams& q, int smem, cudaStream_t stream) {
+  if (mode == HALVES) return launch_mode<BNMAX, PAIR, HALVES>(q, smem, stream);
+  if (mode == WORDS) return launch_mode<BNMAX, PAIR, WORDS>(q, smem, stream);
+  if (mode == ROW_PAIRS) return launch_mode<BNMAX, PAIR, ROW_PAIRS>(q, smem, stream);
+  return launch_mode<BNMAX, PAIR, UNITS>(q, smem, stream);
 }
 
 }  // namespace
@@ -868,9 +934,10 @@ RunsPlan plan_f16_runs(const Geometry& g) {
   p.E = (int32_t)E;
   p.G = (g.Kw + g.s - 1) / g.s;
   p.quad = g.C <= 4;
-  const bool words = E % 2 == 0 && g.s * g.Kh % 2 == 0 && (int64_t)g.Wp * g.Kh % 2 == 0 && halo_fits(WORDS, p.G - 1);
-  const bool pairs = E == 3 && g.s == 1 && (int64_t)g.Ho * g.Wp % 2 == 0 && halo_fits(ROW_PAIRS, p.G - 1);
-  p.mode = p.quad ? QUAD : (words ? WORDS : (pairs ? ROW_PAIRS : HALVES));
+  p.octs = (int32_t)(E >= 3 ? 1 : (E == 2 ? 2 : 4));
+  const bool words = E % 2 == 0 && g.s * g.Kh % 2 == 0 && (int64_t)g.Wp * g.Kh % 2 == 0 && (p.G - 1) * group_of(WORDS) <= 32;
+  const bool pairs = E == 3 && g.s == 1 && (int64_t)g.Ho * g.Wp % 2 == 0;
+  p.mode = words ? WORDS : (pairs ? ROW_PAIRS : HALVES);
   p.units = (int32_t)(p.quad ? (E + 1) / 2 : (g.C + 7) / 8 * E);
   p.num_kb = (p.units + 7) / 8;
   p.nks_last = (p.units - 8 * (p.num_kb - 1) + 1) / 2;
@@ -895,8 +962,9 @@ RunsPlan plan_f16_runs(const Geometry& g) {
   // CTA pairs above 128 channels: each CTA stages its own position tile and half of the filter.  The shared-memory pipe bounds
   // those tiles (an instruction of N = 256 reads 12 KB of operands in 128 cycles, one of a pair 8 KB an SM), and the
   // filter's copies, twice the bytes of all else, halve.
-  // (N of a pair's instruction: a multiple of 32.  Wider tiles for the others would want more scratch)
-  p.pair = p.bn > 128 && p.bn % 32 == 0 && ntm > 1;
+  // (Not for the shortest reductions, which setting up and meeting makes longer: 1.05 to 1.16 times with up to 128 k2 on 15 layers,
+  // 0.92 to 1.15 with up to 256 on 13.  N of a pair's instruction: a multiple of 32.  Wider tiles for the others would want more scratch)
+  p.pair = p.bn > 128 && p.bn % 32 == 0 && ntm > 1 && p.num_kb * p.G >= 8;
   if (const char* v = debug_getenv("IM2WIN_F16_PAIR")) p.pair = p.pair && v[0] != '0';     // testing aid
   p.ntm = (int32_t)ntm;
   p.nwork = (int32_t)((p.pair ? (ntm + 1) / 2 : ntm) * p.ntn);
@@ -904,7 +972,6 @@ RunsPlan plan_f16_runs(const Geometry& g) {
   // A raw slot holds whole octets, at least three units; rings of two S stages, four slots (else two) and the filter:
   // resident where one channel tile's fits, else two slots of all (up to three) kernel columns of a k2-block, so that the MMA
   // warp waits and commits once a k2-block, else at least three of one column.
-  p.octs = (int32_t)(E >= 3 ? 1 : (E == 2 ? 2 : 4));
   int64_t raw = ((p.quad ? 4 : 8 * p.octs) * (int64_t)p.region + 127) / 128 * 128;
   // Layers whose whole filter columns and bulk copies would not fit stay out, also where a pair's halves would: their scratch is
   // not sized for this kernel's filter.
@@ -953,6 +1020,13 @@ RunsPlan plan_f16_runs(const Geometry& g) {
     if (!resident) while (p.sb < MAX_B && fits(p.sa, p.sr, p.sb + 1)) ++p.sb;
     p.eligible = true;
   }
+  // Teams or unit by unit, measured both ways on 750 layers (time of the teams / unit by unit): rows in pairs 0.70 to 1.05, words of
+  // two 0.75 to 1.07; by single elements 0.97 for columns of 3, 6 and 9, 1.02 to 1.16 for one element and the numbers that three
+  // does not divide, 0.85 to 1.13 above nine.  1.05 to 1.1 with up to two slots in a tile, 1.1 to 1.4 with rings of one for each team.
+  const int slots = ((g.C + 7) / 8 + p.octs - 1) / p.octs;
+  bool by_units = slots <= 2 || p.sr == 2 || E <= 2 || (p.mode == HALVES && (E % 3 != 0 || E > 9));
+  if (const char* v = debug_getenv("IM2WIN_F16_RUNS_UNITS")) by_units = v[0] != '0';       // testing aid
+  if (by_units || p.quad || p.halo * group_of(p.mode) > 32) { p.mode = UNITS; p.teams = 1; }
   p.filter_bytes = (size_t)p.ntn * p.bn * p.num_kb * KB * p.G * 2;
   return p;
 }
@@ -990,7 +1064,7 @@ cudaError_t launch_conv_f16_runs(const uint16_t* window, float* y, void* scratch
   q.Co = g.Co; q.Kh = g.Kh; q.Kw = g.Kw; q.s = g.s;
   // kernel columns beyond Kw, channels beyond C in the last octet, the element beyond an odd E
   q.foreign = (g.Kw > g.s && g.Kw % g.s != 0) || (p.quad ? p.E % 2 != 0 : g.C % 8 != 0);
-  q.mode = p.mode; q.teams = p.teams;
+  q.teams = p.teams;
   q.E = p.E; q.G = p.G; q.units = p.units; q.quad = p.quad ? 1 : 0; q.num_kb = p.num_kb; q.nks_last = p.nks_last;
   q.halo = p.halo; q.region = p.region; q.octs = p.octs; q.raw_slot = p.raw_slot; q.a_stage = p.a_stage;
   q.bn = p.bn; q.ntn = p.ntn; q.nwork = p.nwork; q.sa = p.sa; q.sr = p.sr; q.sb = p.sb;
@@ -1000,9 +1074,9 @@ cudaError_t launch_conv_f16_runs(const uint16_t* window, float* y, void* scratch
   }
   q.slot_bytes = p.slot_bytes; q.cols = p.cols; q.ntm = p.ntm; q.resident = p.resident ? 1 : 0;
   const int smem = 1024 + p.sa * p.a_stage + p.sb * p.slot_bytes + p.sr * p.raw_slot;
-  if (p.bn <= 64) return launch_form<64, false>(q, smem, stream);
-  if (p.bn <= 128) return launch_form<128, false>(q, smem, stream);
-  return p.pair ? launch_form<256, true>(q, smem, stream) : launch_form<256, false>(q, smem, stream);
+  if (p.bn <= 64) return launch_form<64, false>(p.mode, q, smem, stream);
+  if (p.bn <= 128) return launch_form<128, false>(p.mode, q, smem, stream);
+  return p.pair ? launch_form<256, true>(p.mode, q, smem, stream) : launch_form<256, false>(p.mode, q, smem, stream);
 }
 
 }  // namespace im2win

@@ -30,7 +30,7 @@ def assert_guards_intact(whole, numel, fill):
     assert torch.equal(tail.view(torch.uint8), ref.view(torch.uint8)), "write past the buffer"
 
 
-# How the run-staged fp16 kernel runs a layer: staging mode (0 to 3: elements, four channels, words of two, pairs of rows),
+# How the run-staged fp16 kernel runs a layer: staging mode (0 to 3: elements, words of two, pairs of rows, unit by unit),
 # CTA pairs, channel planes in a row of the tiled copies (0: bulk copies), whether the filter stays in shared memory, teams of
 # staging warps and raw slots, octets of channels in a slot, elements of a virtual column, rows below a tile, channel tile
 # and number of channel and position tiles.

@@ -112,7 +112,7 @@ def test_f16_runs_teams_on_their_slots(layer, slots, monkeypatch):
     monkeypatch.setenv("IM2WIN_F16_KERNEL", "runs")
     dims = layer.dims()
     form = runs_form(dims)
-    assert (form.mode, form.teams, form.slots) == (3, 4, slots) and layer.C // 8 >= 2 * slots
+    assert (form.mode, form.teams, form.slots) == (2, 4, slots) and layer.C // 8 >= 2 * slots
     for seed in range(3):                                    # (new buffers every time: cold copies)
         x, f = workloads.make_small_integer_inputs(replace(layer, seed=layer.seed + 100 * seed))
         y, _, _ = gpu_conv(x, f, dims, "f16")
@@ -120,17 +120,18 @@ def test_f16_runs_teams_on_their_slots(layer, slots, monkeypatch):
         assert np.array_equal(y.astype(np.float64), yr)
 
 
-# Rows below the tile: as many as a warp reads for a whole group of three or six units (ten, five), and more, which it reads unit
-# by unit: a group then lies in two k2-blocks wherever its units are no divisor of eight
+# Rows below the tile: as many as a warp reads for a whole group of three or six units (ten, five), and more, which only the form
+# that goes unit by unit takes
 @pytest.mark.parametrize("layer,mode,halo", [
-    (L("low_13", 1, 24, 16, 20, 24, 13, 13, 1, 6, 450), 0, 12), (L("low_pair", 2, 40, 14, 17, 150, 13, 14, 1, 3, 451), 0, 13),
-    (L("low_quad", 1, 3, 18, 21, 16, 12, 12, 1, 2, 452), 1, 11), (L("low_31", 1, 72, 6, 40, 16, 1, 32, 1, 0, 457), 0, 31),
-    (L("low_11", 1, 20, 15, 20, 20, 12, 12, 1, 3, 458), 0, 11), (L("low_3x12", 1, 40, 14, 20, 48, 3, 12, 1, 2, 456), 0, 11),
-    (L("low_3x11", 1, 40, 14, 20, 48, 3, 11, 1, 2, 459), 3, 10), (L("low_10", 2, 24, 14, 16, 33, 10, 10, 1, 4, 453), 0, 9),
-    (L("low_6", 1, 20, 20, 15, 150, 10, 7, 1, 3, 454), 0, 6), (L("low_5", 1, 20, 20, 15, 150, 10, 6, 1, 3, 460), 2, 5),
+    (L("low_13", 1, 24, 16, 20, 24, 13, 13, 1, 6, 450), 3, 12), (L("low_pair", 2, 40, 14, 17, 150, 13, 14, 1, 3, 451), 3, 13),
+    (L("low_quad", 1, 3, 18, 21, 16, 12, 12, 1, 2, 452), 3, 11), (L("low_31", 1, 72, 6, 40, 16, 1, 32, 1, 0, 457), 3, 31),
+    (L("low_11", 1, 20, 15, 20, 20, 12, 12, 1, 3, 458), 3, 11), (L("low_3x12", 1, 40, 14, 20, 48, 3, 12, 1, 2, 456), 3, 11),
+    (L("low_3x11", 1, 40, 14, 20, 48, 3, 11, 1, 2, 459), 2, 10), (L("low_10", 2, 24, 14, 16, 33, 10, 10, 1, 4, 453), 0, 9),
+    (L("low_6", 1, 20, 20, 15, 150, 10, 7, 1, 3, 454), 0, 6), (L("low_5", 1, 20, 20, 15, 150, 10, 6, 1, 3, 460), 1, 5),
     (L("low_s2", 1, 24, 15, 32, 20, 5, 15, 2, 2, 455), 0, 7)], ids=lambda v: getattr(v, "name", str(v)))
 def test_f16_runs_rows_below_the_tile(layer, mode, halo, monkeypatch):
     monkeypatch.setenv("IM2WIN_F16_KERNEL", "runs")
+    monkeypatch.setenv("IM2WIN_F16_RUNS_UNITS", "0")
     dims = layer.dims()
     form = runs_form(dims)
     assert (form.mode, form.halo) == (mode, halo)

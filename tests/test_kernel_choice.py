@@ -94,6 +94,6 @@ def test_run_staged_slots_keep_to_one_team():
         f = runs_form(layer)
         if f is None:
             continue
-        assert f.slots % f.teams == 0 and f.teams in (2, 4) and f.slots % 2 == 0, (layer, f)
+        assert f.slots % f.teams == 0 and f.teams in ((1,) if f.mode == 3 else (2, 4)) and f.slots % 2 == 0, (layer, f)
         seen.add((f.mode, f.teams))
-    assert {m for m, _ in seen} == {0, 1, 2, 3} and {t for _, t in seen} == {2, 4}
+    assert {m for m, _ in seen} == {0, 1, 2, 3} and {t for _, t in seen} == {1, 2, 4}
