@@ -65,28 +65,37 @@ def test_nhwc_tiles_of_parts_of_strips(layer, layout, monkeypatch):
     check_conv(y, yr, ar, "f16", layer.name)
 
 
-# the columns of the run-staged kernel: elements, words of two, pairs of rows; copies of one, two, four and eight channels
-@pytest.mark.parametrize("layer", [
-    L("pairs_1", 2, 24, 20, 14, 130, 3, 3, 1, 1, 420),       # plane a multiple of 16 bytes, CTA pairs, 5 position tiles
-    L("pairs_4", 3, 12, 14, 11, 33, 3, 3, 1, 1, 421),        # four planes are, half an octet, two images in a tile
-    L("pairs_8", 2, 16, 13, 12, 70, 3, 3, 1, 1, 422),        # eight planes: bulk copies
-    L("pairs_s", 5, 40, 9, 8, 16, 3, 3, 1, 0, 423),          # several images in a tile: bulk copies
-    L("words_2", 2, 16, 28, 28, 136, 3, 3, 2, 1, 424),       # two planes, stride 2, CTA pairs
-    L("words_c9", 2, 9, 28, 28, 264, 3, 3, 2, 1, 425),       # an odd number of channels: bulk copies, two channel tiles
-    L("words_10", 1, 16, 30, 30, 40, 5, 5, 2, 1, 426),       # ten elements a column, boxes too wide
-    L("words_2el", 1, 24, 30, 28, 40, 1, 2, 2, 0, 427),      # two elements, two octets a slot
-    L("halves_5", 2, 16, 16, 12, 48, 5, 5, 1, 2, 428),       # five elements, four rows below the tile
-    L("halves_1", 2, 72, 16, 16, 200, 1, 1, 1, 0, 429),      # one element, four octets a slot, the last slot not full
-    L("halves_odd", 2, 16, 13, 15, 48, 3, 3, 1, 1, 430),     # an odd number of columns in an image
-    L("last_pair", 9, 32, 16, 14, 256, 3, 3, 1, 1, 431),     # 18 position tiles
-    L("rounds", 40, 16, 26, 30, 200, 3, 3, 1, 1, 432)], ids=lambda l: l.name)      # more pairs than the GPU holds
-@pytest.mark.parametrize("tiled,pair", [("1", "1"), ("0", "1"), ("1", "0")])
-def test_f16_runs_columns_and_copies(layer, tiled, pair, monkeypatch):
+# the columns of the run-staged kernel: elements, words of two, pairs of rows, unit by unit; copies of one, two, four and eight
+# channels; CTA pairs.  (form: staging mode, pairs, planes of a tiled copy's row)
+@pytest.mark.parametrize("layer,form", [
+    (L("pairs_1", 2, 48, 20, 14, 150, 3, 3, 1, 1, 420), (2, 1, 1)),    # CTA pairs, an odd number of position tiles
+    (L("pairs_4", 3, 28, 14, 11, 33, 3, 3, 1, 1, 421), (2, 0, 4)),     # half an octet in the last slot, two images in a tile
+    (L("pairs_18", 2, 18, 13, 12, 70, 3, 3, 1, 1, 422), (2, 0, 0)),    # four planes, but no multiple of four channels: bulk copies
+    (L("pairs_s", 5, 40, 9, 8, 16, 3, 3, 1, 0, 423), (2, 0, 0)),       # several images in a tile: bulk copies
+    (L("words_2", 3, 40, 28, 28, 150, 3, 3, 2, 1, 424), (1, 1, 2)),    # stride 2, CTA pairs, an odd number of position tiles
+    (L("words_c33", 2, 33, 28, 28, 300, 3, 3, 2, 1, 425), (1, 1, 0)),  # an odd number of channels; pairs, two channel tiles, the last not full
+    (L("words_10", 1, 24, 30, 30, 40, 5, 5, 2, 1, 426), (1, 0, 0)),    # ten elements a column, boxes too wide
+    (L("words_2el", 1, 24, 30, 28, 40, 1, 2, 2, 0, 427), (3, 0, 2)),   # two elements, two octets a slot
+    (L("halves_5", 2, 16, 16, 12, 48, 5, 5, 1, 2, 428), (3, 0, 1)),    # five elements, four rows below the tile
+    (L("halves_1", 2, 520, 16, 16, 220, 1, 1, 1, 0, 429), (3, 1, 1)),  # one element, four octets a slot, the last slot not full; pairs
+    (L("halves_odd", 2, 40, 13, 15, 48, 3, 3, 1, 1, 430), (0, 0, 0)),  # an odd number of columns in an image; eight planes
+    (L("halves_9", 3, 64, 30, 31, 180, 3, 3, 3, 0, 433), (0, 1, 0)),   # stride 3, CTA pairs, an odd number of position tiles
+    (L("last_pair", 9, 48, 16, 14, 256, 3, 3, 1, 1, 431), (2, 1, 1)),  # 18 position tiles
+    (L("rounds", 32, 48, 20, 30, 250, 3, 3, 1, 1, 432), (2, 1, 1))],   # more pairs than the GPU holds, the channel tile not full
+    ids=lambda v: getattr(v, "name", None))
+@pytest.mark.parametrize("tiled,pair,units", [("1", "1", None), ("0", "1", None), ("1", "0", None), ("1", "1", "1"), ("1", "1", "0")])
+def test_f16_runs_columns_and_copies(layer, form, tiled, pair, units, monkeypatch):
     monkeypatch.setenv("IM2WIN_F16_KERNEL", "runs")
     monkeypatch.setenv("IM2WIN_F16_RUNS_TILED", tiled)
     monkeypatch.setenv("IM2WIN_F16_PAIR", pair)
+    if units:
+        monkeypatch.setenv("IM2WIN_F16_RUNS_UNITS", units)
     dims = layer.dims()
     assert binding.im2win_conv_kernel_name(dims, binding.F16) == "f16-runs"
+    got = runs_form(dims)
+    assert (got.mode == 3) == (form[0] == 3 if units is None else units == "1") and (units or got.mode == form[0])
+    assert got.pair == form[1] * int(pair) and got.planes == form[2] * int(tiled)
+    assert layer.name != "rounds" or got.ntm > 148
     x, f = workloads.make_small_integer_inputs(layer)
     y, _, _ = gpu_conv(x, f, dims, "f16")
     yr, _ = oracle.conv_direct(x.numpy(), f.numpy(), dims)
