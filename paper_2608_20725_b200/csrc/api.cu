@@ -73,37 +73,46 @@ static bool want_f32_split(const Geometry& g, const F32SplitPlan& p) {
   return g.K > 80 || (p.nstages == 1 && g.Co <= 256);
 }
 
+// Images that a tile of the run-staged kernel touches, on average.
+static double images_of_a_tile(const Geometry& g, const RunsPlan& p) { return 1.0 + (128.0 + p.halo) / (double)((int64_t)g.Ho * p.Wq); }
+
 // Of the layers that neither the one-k-block kernel nor a tiled-copy kernel takes, and the shifted-view kernel could: which
 // ones the run-staged kernel gets.  Its copies are at most one per channel and image of a tile, so their number for each staged
 // element is (images of a tile) / E, with E elements per virtual column; the shifted-view kernel stages all s columns even
-// where the kernel has fewer (Kw < s).  Measured over 400 layers (images of 7 to 160, kernels of 1 to 7, strides 1 and 2, 5 to
-// 512 channels, batches 1 to 128), shifted-view time / run-staged time:
+// where the kernel has fewer (Kw < s).  Measured over 400 layers (images of 7 to 160, square kernels of 1 to 7, strides 1 and 2, 5
+// to 512 channels, batches 1 to 128), shifted-view time / run-staged time:
 //   3x3 stride 1, images / E up to 0.7: 65 to 128 channels 1.22 to 1.66, more channels 0.92 to 1.1 with up to 148 tiles and
 //   1.1 to 1.6 with more; up to 64 channels 1.43 (1.14 at the least) where rows are staged in pairs, 1.1 (0.94) where not
 //   5x5 stride 1: 1.09 to 1.47 with more than 296 tiles, 0.7 to 1.2 with fewer; 7x7 0.84
 //   stride 2, up to 0.9: 3x3 1.62; 5x5 and 7x7 1.03 to 2.2 up to 128 channels, 0.9 to 1.1 on more with few tiles
-// (256 -> 512 channels, 3x3 stride 2 at 28x28, batch 128: 140 -> 97 us; not taken: 3x3 on 512 channels at 7x7, batch 128, 44 us
+// and over 220 layers that are not square or have larger strides (images of 4 to 100, with the forms the kernel has now):
+//   five wide, stride 1, more than 296 tiles: one to four high 1.06 to 1.8 at every images / E; six and seven high 1.1 to 1.7 up to
+//   128 channels, 0.93 to 1.5 on more
+//   strides 3 and 4, images / E of 0.7 to 0.9 1.4 to 2.1; four virtual columns (11 wide at stride 3) 1.45 to 2.3 up to 128
+//   channels, 1.02 to 1.5 on more from three tiles on, 0.92 and 0.99 with fewer
+// (256 -> 512 channels, 3x3 stride 2 at 28x28, batch 128: 140 -> 88 us; not taken: 3x3 on 512 channels at 7x7, batch 128, 44 us
 // against 55.)
 static bool prefer_runs(const Geometry& g, const RunsPlan& p) {
-  const int64_t per_img = (int64_t)g.Ho * p.Wq;
-  const double images = 1.0 + (128.0 + p.halo) / (double)per_img;
+  const double images = images_of_a_tile(g, p);
   const int64_t tiles = (int64_t)p.ntm * p.ntn;
   if (g.s == 1) {
-    if (p.G == 5) return tiles > 296;
+    if (p.G == 5) return tiles > 296 && (g.Kh <= 5 || g.Co <= 128);
     if (p.G > 3 || images > 0.7 * p.E) return false;
     if (g.Co > 64) return g.Co <= 128 || tiles > 148;
     return p.E == 3 && (int64_t)g.Ho * g.Wp % 2 == 0;
   }
   if (p.G > 4 || (p.G > 2 && g.s == 2 && g.Co > 128 && (p.G > 3 || tiles <= 74))) return false;
+  if (p.G == 4 && g.Co > 128 && tiles < 3) return false;
   return images <= (g.Kw < g.s ? 2.1 : 0.9) * p.E;
 }
 
 // 3x3 layers of stride 1 that the tiled-copy kernels could take: the run-staged kernel below 128 channels (1.29 times as fast on
 // 23 such layers, 1.02 at the least: 3x3 on 32 channels at 112x112, batch 64, 134 -> 127 us), and from two and a half rounds
 // of tiles on also above (1.05 to 1.13 on ten layers; 0.83 to 1.07 on 19 of fewer tiles.  256 channels at 28x28, batch 64,
-// 61 -> 58 us; 64 -> 128 channels at 112x112 223 -> 194).
+// 61 -> 58 us; 64 -> 128 channels at 112x112 223 -> 194).  Not the smallest images: 1.03 to 1.9 on 97 layers of 3 to 12 rows with
+// up to 1.25 images / E, 0.84 to 1.2 on 13 above (4x6 images, padded).
 static bool runs_before_tiled(const Geometry& g, const RunsPlan& p) {
-  return g.s == 1 && g.Kh == 3 && g.Kw == 3 && (g.Co < 128 || (int64_t)p.ntm * p.ntn > 370);
+  return g.s == 1 && g.Kh == 3 && g.Kw == 3 && images_of_a_tile(g, p) <= 1.25 * p.E && (g.Co < 128 || (int64_t)p.ntm * p.ntn > 370);
 }
 
 // The same layer with another batch.

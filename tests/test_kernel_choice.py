@@ -49,7 +49,11 @@ def test_f32_kernel_by_length_of_the_reduction(C, K, want):
     ((128, 512, 7, 7, 512, 3, 3, 1, 1), "f16-shift"),      # several images in a tile: a copy per image and channel
     ((128, 512, 7, 7, 1024, 1, 1, 1, 0), "f16-shift"),     # one element per column and copy
     ((1, 256, 27, 27, 256, 3, 3, 1, 1), "f16-shift"),      # few tiles
-    ((32, 64, 61, 45, 64, 3, 3, 1, 0), "f16-shift")])      # 64 channels
+    ((32, 64, 61, 45, 64, 3, 3, 1, 0), "f16-shift"),       # 64 channels
+    ((128, 128, 35, 9, 128, 7, 5, 1, 3), "f16-runs"), ((128, 128, 35, 9, 129, 7, 5, 1, 3), "f16-shift"),   # five wide, seven high
+    ((64, 128, 35, 19, 129, 5, 5, 1, 2), "f16-runs"), ((8, 128, 35, 19, 129, 5, 5, 1, 2), "f16-shift"),    # ... 380 tiles, 48
+    ((2, 256, 53, 7, 262, 11, 11, 3, 5), "f16-runs"), ((1, 256, 24, 9, 256, 5, 11, 3, 2), "f16-shift"),    # four virtual columns
+    ((16, 256, 8, 8, 64, 3, 3, 1, 1), "f16-runs"), ((16, 256, 4, 6, 64, 3, 3, 1, 1), "f16-shift")])        # images of a tile: 2.6, 5.1
 def test_f16_kernel_on_odd_planes(layer, want):
     assert binding.im2win_conv_kernel_name(layer, binding.F16) == want
 
