@@ -308,6 +308,15 @@ int32_t im2win_f16_runs_form(const im2win_shape* shape, int32_t form[12]) {
   return p.eligible;
 }
 
+// The same for the fp32 tensor-core kernel: channel tile, CTAs of a tile, parts of the last round's tiles.
+int32_t im2win_f32_split_form(const im2win_shape* shape, int32_t form[3]) {
+  Geometry g;
+  if (derive_geometry(shape, &g) != IM2WIN_OK) return 0;
+  const F32SplitPlan p = plan_f32_split(g);
+  form[0] = p.bn; form[1] = p.split; form[2] = p.parts;
+  return p.eligible;
+}
+
 im2win_status im2win_workspace_size(const im2win_shape* shape, im2win_dtype dtype, size_t* window_bytes,
                                     size_t* scratch_bytes, int32_t* Ho, int32_t* Wo) {
   Geometry g;

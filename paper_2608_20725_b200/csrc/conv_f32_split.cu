@@ -718,7 +718,7 @@ double step_cycles(int bn) { return bn <= CONCAT_BN ? mma_cycles(3 * bn) + 3 * m
 
 // Parts of its channels that a tile of the last round goes out in, where that round leaves half of the SMs or more idle: an
 // instruction of N = 64 takes 3/8 of the time of N = 256, so quarters save 5/8 of a round.  (5x5 on 256 channels at 28x28,
-// batch 64, 3.03 rounds of tiles: 966 -> 756 us; 7x7, 3.2 rounds: 1909 -> 1462.)
+// batch 64, 3.03 rounds of tiles: 966 -> 766 us; 7x7, 3.2 rounds: 1909 -> 1493.)
 int channel_parts(int64_t tiles, int bn) {
   const int64_t last = tiles % 148;
   if (last == 0 || bn <= CONCAT_BN) return 1;
@@ -777,18 +777,30 @@ F32SplitPlan plan_f32_split(const Geometry& g) {
     for (int z = 1; z <= 8; z *= 2) {
       if (z > p.nstages || (z > 1 && ntm * nt * z > 128)) break;     // clusters: one tile each, all resident
       if (force_z && z != atoi(force_z)) continue;
+      const int64_t tiles = ntm * nt;
+      // The estimate: the tensor pipe, or the shared-memory pipe with operands, copies and staging.  For clusters and reductions of one
+      // k2-block the latter is nine tenths of the former, and what is staged.  Else the operands are counted (11x11 on 256
+      // channels, a unit of four steps: 3126 cycles in tiles of 256 channels, 2185 in tiles of 128), for layers of one round up to
+      // nine tenths; in more rounds the last may go out in parts.  Against nine tenths for all 1.17 times as fast on average on 223
+      // layers that choose other tiles for it, 0.97 at the least.  Counted for all, with parts for all: too wide tiles, 0.72 at the
+      // least (3x3 stride 2 on 64 -> 256 channels at 14x14, batch 95: 42 tiles of 256 channels in pairs of CTAs 31.6 us, 126 of 96
+      // 23.4; 3x3 on 16 -> 256 channels at 16x140: halves of 62 tiles of 256 15.2, 124 of 128 13.4; 5x5 on 8 -> 372 channels at
+      // 47x47 26.5 and 22.9).
+      const bool counted = z == 1 && p.num_kb > 1 && bn > CONCAT_BN, rounds = z == 1 && p.num_kb > 1 && tiles > 148;
       auto tile_cycles = [&](int cols) {
-        // The tensor pipe, or the shared-memory pipe: operands, copies and staging.  (11x11 on 256 channels, a unit of four
-        // steps: 3126 cycles in tiles of 256 channels, 2185 in tiles of 128.)
         const double fill = 3.0 * cols * steps / 4 + 1200.0 * p.nstages;
         const double pipe = steps * (bn <= CONCAT_BN ? step_cycles(bn) : 6 * mma_cycles(cols));
-        const double wave = (bn <= CONCAT_BN ? pipe * 0.9 : steps * 6 * (32 + cols / 4.0)) + fill;
+        double wave = pipe * 0.9;
+        if (counted) {
+          const double operands = steps * 6 * (32 + cols / 4.0);
+          wave = rounds || operands < wave ? operands : wave;
+        }
+        wave += fill;
         return (pipe > wave ? pipe : wave) * ((p.nstages + z - 1) / z) / p.nstages + (z > 1 ? 5000 : 1500);
       };
-      const int64_t tiles = ntm * nt;
-      const int parts = channel_parts(tiles, bn);
-      const double cost = 6000 + (z > 1 ? tile_cycles(bn)
-                                        : (double)(tiles / 148) * tile_cycles(bn) + (tiles % 148 != 0 ? tile_cycles(bn / parts) : 0.0));
+      const int parts = rounds ? channel_parts(tiles, bn) : 1;
+      const double last = tiles % 148 == 0 ? 0.0 : tile_cycles(bn / parts);
+      const double cost = 6000 + (z > 1 ? tile_cycles(bn) : (double)(tiles / 148) * tile_cycles(bn) + last);
       if (!p.eligible || cost < p.cost) {
         p.eligible = true;
         p.cost = cost;

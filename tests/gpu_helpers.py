@@ -45,6 +45,14 @@ def runs_form(dims):
     return RunsForm(*form) if fn(ctypes.byref(binding.as_shape(dims)), form) else None
 
 
+def split_form(dims):
+    """(channel tile, CTAs of a tile, parts of the last round's tiles) of the fp32 tensor-core kernel.  Needs no GPU."""
+    fn = binding.lib().im2win_f32_split_form
+    fn.argtypes, fn.restype = [ctypes.POINTER(binding.Shape), ctypes.POINTER(ctypes.c_int32)], ctypes.c_int32
+    form = (ctypes.c_int32 * 3)()
+    return tuple(form) if fn(ctypes.byref(binding.as_shape(dims)), form) else None
+
+
 def gpu_transform(x_cpu: torch.Tensor, dims: dict) -> np.ndarray:
     """x (float32/float16/int32/int16 CPU tensor) -> window tensor as a numpy array of the same dtype."""
     code = binding.F32 if x_cpu.element_size() == 4 else binding.F16

@@ -8,7 +8,7 @@ import sys
 import pytest
 
 from conftest import ROOT
-from gpu_helpers import runs_form
+from gpu_helpers import runs_form, split_form
 from paper_2608_20725_b200 import binding
 
 LAYERS = [(128, 64, 56, 56, 64, 3, 3, 1, 1), (128, 512, 7, 7, 512, 3, 3, 1, 1), (13, 37, 45, 61, 75, 5, 5, 2, 2),
@@ -101,3 +101,13 @@ def test_run_staged_slots_keep_to_one_team():
         assert f.slots % f.teams == 0 and f.teams in ((1,) if f.mode == 3 else (2, 4)) and f.slots % 2 == 0, (layer, f)
         seen.add((f.mode, f.teams))
     assert {m for m, _ in seen} == {0, 1, 2, 3} and {t for _, t in seen} == {1, 2, 4}
+
+
+@pytest.mark.parametrize("layer,want", [
+    ((64, 256, 28, 28, 256, 5, 5, 1, 2), (256, 1, 4)),      # three rounds of tiles and four: the last in quarters
+    ((95, 64, 14, 14, 256, 3, 3, 2, 1), (96, 1, 1)),        # one round: narrow tiles, no pairs of CTAs on wide ones
+    ((4, 16, 16, 140, 256, 3, 3, 1, 0), (128, 1, 1)),       # ... and no halves of wide ones
+    ((32, 128, 20, 20, 256, 3, 7, 1, 1), (256, 1, 1)),      # one round of wide tiles, not two with the last in halves
+    ((4, 8, 47, 47, 372, 5, 5, 1, 2), (128, 1, 1))])        # one k2-block: two rounds of narrow tiles
+def test_f32_tiles(layer, want):
+    assert split_form(layer) == want
