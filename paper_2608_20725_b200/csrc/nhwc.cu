@@ -2183,9 +2183,11 @@ struct NhwcChoice {
 };
 
 // Tiles of parts of strips for the overlapping-row kernel.  Whole strips of 28 fill 112 of a tile's 128 rows, halves of nine
-// strips 126: stride 1 reductions of 128 to 256 k-blocks, whose tiles are long against their loads and stores, take the fewest
-// tiles (7x7 on 256 channels at 28x28, batch 64, 254 -> 225 us, with bias, ReLU and binary16 stores 255 -> 221).  Beyond, the power
-// limit decides and the gain does not hold (11x11, 480 k-blocks: 617 to 636 -> 579 to 710).
+// strips 126: stride 1 reductions of 128 to 256 k-blocks, whose tiles are long against their loads and stores, take the widest
+// parts that save 3 % of the tiles (7x7 on 256 channels at 28x28, batch 64, 254 -> 225 us, with bias, ReLU and binary16 stores
+// 255 -> 221).  Measured with and without on layers where such parts exist: 1.11 times as fast on average on 45 of 128 to 256
+// k-blocks, 0.96 at the least, one below 0.97.  Outside it gains too, but less surely: 1.13 on 45 of 64 to 127 with five below
+// 0.97, 1.07 on 45 of 24 to 63 with eleven, 1.09 on 45 of more, where the power limit decides, 0.92 at the least.
 void part_strips(const Geometry& g, NhwcPlan& p) {
   if (p.num_kb < 128 || p.num_kb > 256 || g.s > 1) return;
   for (int tw = p.tw + 1; tw <= p.tw + 7 && (g.Wo + tw - 1) / tw >= 7; ++tw) {
