@@ -1,7 +1,7 @@
 // fp16-input / fp32-accumulate im2win convolution on the sm_100a tensor cores:
 // shifted-view kernel with bulk-copied window runs (stride 1, 128-position tiles).
-// (3x3 layers go to conv_f16_runs.cu, which is 1.29 times as fast on them on average; this one is left the other kernels up
-// to four wide: a 1x1 on 128 -> 64 channels at 80x80, batch 16, takes 19 us here and 34 there.)
+// (3x3 layers go to conv_f16_runs.cu, which is 1.29 times as fast on them on average; this one is left those of the smallest
+// images, see runs_before_tiled, and the other kernels up to four wide: a 1x1 on 128 -> 64 channels at 80x80, batch 16, takes 19 us here and 34 there.)
 //
 // Same GEMM formulation as conv_f16_shift.cu (paper Algorithm 1 with the S tile
 // of im2win columns and Kw row-shifted views of it), but the S tile is no longer
