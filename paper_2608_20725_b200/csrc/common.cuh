@@ -27,6 +27,18 @@ struct Geometry {
   int32_t plan_N;        // batch the kernel and the order of its sums are chosen for: N, or what these N images are a part of
 };
 
+// Clusters of z CTAs, each CTA an SM to itself, that a B200 holds at once: they lie within a GPC, so that wide ones leave SMs over.
+// (What cudaOccupancyMaxActiveClusters says of 226 KB of shared memory a CTA; 16 clusters of 8 CTAs run in two rounds: 7x7 on
+// 256 -> 78 channels at 35x35, batch 2, 87 us in clusters of 8, 47 in clusters of 4.)
+constexpr int kMaxCtas = 16;       // of a cluster (above 8: the non-portable sizes)
+// Longest reduction of an fp16 layer whose tiles are shared.  An accumulator truncates every addend, 1e-9 of the sum a term,
+// so a shared reduction is the more exact one; beyond this the two would differ by more than fp32 sums in another order do.
+constexpr int64_t kMostSplitTerms = 16384;
+inline int resident_clusters(int z) {
+  constexpr int kResident[kMaxCtas + 1] = {0, 148, 74, 45, 33, 26, 22, 15, 15, 15, 11, 7, 7, 7, 7, 7, 7};
+  return z >= 1 && z <= kMaxCtas ? kResident[z] : 0;
+}
+
 // Scratch layout shared by both precisions (offsets in bytes from `scratch`):
 //   [0, 256)            status block (uint32 words; word 0 = timeout flag)
 //   [256, 256 + 4*Kp)   k -> element offset table (int32), -1 for padded k
@@ -55,6 +67,7 @@ struct ShiftPlan {
   int32_t nks_last;      // 16-wide MMA steps of the last k-block
   int64_t K2, K2p;       // C*Kh and its round-up to 64
   int64_t VQ;            // N*Ho*Wq virtual positions
+  int32_t bn, split;     // channel tile, CTAs of a cluster that share the k-blocks of a tile
 };
 ShiftPlan plan_f16_shift(const Geometry& g);
 
@@ -141,6 +154,7 @@ struct RunsPlan {
   int32_t region, raw_slot, a_stage, slot_bytes, cols, planes, seg_bytes;
   int32_t bn, ntn, ntm, nwork, sa, sr, sb;
   int32_t mode, teams;                 // how the staging warps read the raw slots, and how many teams they form
+  int32_t split;                       // CTAs of a cluster that share the reduction of a tile
   int64_t VQ;
   size_t filter_bytes;
 };

@@ -40,8 +40,11 @@
 // TFLOP/s; no pipe above 45 % of its rate: hand-offs over two stages); 3x3 on 512 channels at 7x7 627 -> 155; 11x11 on 256
 // channels at 28x28, batch 64, 14824 -> 3930 (202 TFLOP/s; 1.6 PFLOP/s of bf16 products with the strip ends, near the
 // power limit); 7x7 stride 2 on 3 channels at 224x224 642 -> 408.
-// A layer with few tiles is run by clusters of 2, 4 or 8 CTAs that share the stages of a tile and add their
-// registers through distributed shared memory, in rank order: 3x3 on 512 channels, one 7x7 image, 225 -> 31 us.
+// A layer with few tiles is run by clusters of 2 to 16 CTAs that share the stages of a tile and add their
+// registers through distributed shared memory, in rank order: 3x3 on 512 channels, one 7x7 image, 225 -> 31 us.  Any number of CTAs
+// whose clusters are all resident at once, sums pushed to the CTA that finishes them: against powers of two up to 8 and sums read from the
+// other CTAs, 40 layers of 1 to 90 tiles 1.13 times as fast on average (0.91 at the least): 3x5 stride 2 on 427 channels at 66x12, batch 2,
+// 35.8 -> 16.3 us, 7x7 on 256 -> 78 channels at 35x35, batch 2 (16 clusters of 8 in two rounds) 87 -> 47.
 #include <cuda_bf16.h>
 #include <stdlib.h>
 #include <string.h>
@@ -144,11 +147,6 @@ __device__ __forceinline__ void tmem_wait16(uint32_t (&r)[16]) {
                  "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
                :
                : "memory");
-}
-__device__ __forceinline__ float ld_cluster(uint32_t addr) {
-  float v;
-  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
-  return v;
 }
 // bf16 operands, fp32 accumulator, both k-major.
 __host__ __device__ constexpr uint32_t instr_desc_bf16(int M, int N) {
@@ -569,16 +567,15 @@ __global__ void __launch_bounds__(Form<BNMAX, PWG>::THREADS, 1) conv_f32_split_k
       }
       if (!ok) break;
       if (q.split > 1) {
-        // All MMAs of this CTA have completed, so its rings are free: partial sums as P[channel][row], 4 bytes.
         // (here and not behind the loop, where the sums would have to be live over everything below)
-        float* part = reinterpret_cast<float*>(smem);
+        const int channels = q.Co - nt * q.bn < q.bn ? q.Co - nt * q.bn : q.bn;
+        const ClusterSums sums(a_ring, q.split, rank, channels);
+        __syncwarp();
+        cluster_sync_all();                                 // (every MMA of every CTA has completed)
 #pragma unroll
-        for (int j = 0; j < F::CH; ++j)
-#pragma unroll
-          for (int e = 0; e < 16; ++e) {
-            const int c = (h + 2 * j) * 16 + e;
-            if (c < q.bn) part[c * TILE_M + lq * 32 + lane] = acc[j][e];
-          }
+        for (int j = 0; j < F::CH; ++j) sums.store(acc[j], (h + 2 * j) * 16, channels, lq * 32 + lane);
+        __syncwarp();
+        cluster_sync_all();
         break;
       }
       if (valid) {
@@ -601,41 +598,29 @@ __global__ void __launch_bounds__(Form<BNMAX, PWG>::THREADS, 1) conv_f32_split_k
       }
     }
     if (q.split > 1) {
-      __syncwarp();
-      cluster_sync_all();
+      if (!ok) { __syncwarp(); cluster_sync_all(); cluster_sync_all(); }      // (a wait gave up: the others wait for this CTA all the same)
       if (ok && valid) {
         const int co0 = nt * q.bn;
-        const int limit = q.Co - co0 < q.bn ? q.Co - co0 : q.bn;
-        float* yrow = q.y + ((int64_t)n * q.Co + co0) * q.HoWo + (int64_t)ho * q.Wo + i0;
-        const int per = q.bn / q.split;                     // channels this CTA finishes (bn is a multiple of 16)
-        uint32_t peer[8];
-#pragma unroll
-        for (int r = 0; r < 8; ++r) peer[r] = mapa_shared(a_ring + (lq * 32 + lane) * 4, r < q.split ? r : 0);
-        const int c_end = (rank + 1) * per < limit ? (rank + 1) * per : limit;
+        const int channels = q.Co - co0 < q.bn ? q.Co - co0 : q.bn;
+        const ClusterSums sums(a_ring, q.split, rank, channels);
+        const int first = rank * sums.per, mine = channels - first < sums.per ? channels - first : sums.per;
+        float* yrow = q.y + ((int64_t)n * q.Co + co0 + first) * q.HoWo + (int64_t)ho * q.Wo + i0;
         bool again = false;
-        for (int c = rank * per + h; c < c_end; c += 2) {
-          float v[8];
-#pragma unroll
-          for (int r = 0; r < 8; ++r) v[r] = r < q.split ? ld_cluster(peer[r] + c * (TILE_M * 4)) : 0.f;
-          float sum = v[0];
-#pragma unroll
-          for (int r = 1; r < 8; ++r) sum += v[r];
-          sum *= kUnscale;
+        for (int c = h; c < mine; c += 2) {
+          const float sum = sums.sum(c, lq * 32 + lane) * kUnscale;
           again |= suspicious(sum);
           yrow[(int64_t)c * q.HoWo] = sum;
         }
         if (again) {
           const float* x = q.win + (int64_t)n * q.img_stride + (int64_t)ho * q.strip + (int64_t)i0 * q.s * q.Kh;
           const int64_t K = (int64_t)q.K2 * q.Kw;
-          for (int c = rank * per + h; c < c_end; c += 32) {
-            const int left = (c_end - c + 1) / 2;
-            exact_outputs(x, q.f + (co0 + c) * K, yrow + (int64_t)c * q.HoWo, q.chan_stride, 2 * K, 2 * (int64_t)q.HoWo, q.C,
+          for (int c = h; c < mine; c += 32) {
+            const int left = (mine - c + 1) / 2;
+            exact_outputs(x, q.f + (co0 + first + c) * K, yrow + (int64_t)c * q.HoWo, q.chan_stride, 2 * K, 2 * (int64_t)q.HoWo, q.C,
                           q.Kh, q.Kw, left < 16 ? left : 16);
           }
         }
       }
-      __syncwarp();
-      cluster_sync_all();
     }
   }
   if (wg < F::PWG && q.split > 1) {
@@ -734,6 +719,7 @@ cudaError_t launch_form(const SplitParams& q, int smem, cudaStream_t stream) {
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
   if (!attr_done[dev]) {
     cudaError_t e = cudaFuncSetAttribute(conv_f32_split_kernel<BNMAX, PWG>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSplitSmem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(conv_f32_split_kernel<BNMAX, PWG>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
     attr_done[dev] = true;
   }
@@ -774,10 +760,10 @@ F32SplitPlan plan_f32_split(const Geometry& g) {
     if (nt * bn > p.packed_rows) p.packed_rows = nt * bn;
     if (force_bn && bn != atoi(force_bn)) continue;
     if (ntm * nt >= ((int64_t)1 << 30)) continue;
-    for (int z = 1; z <= 8; z *= 2) {
-      if (z > p.nstages || (z > 1 && ntm * nt * z > 128)) break;     // clusters: one tile each, all resident
-      if (force_z && z != atoi(force_z)) continue;
+    for (int z = 1; z <= kMaxCtas && z <= p.nstages; ++z) {
       const int64_t tiles = ntm * nt;
+      if (z > 1 && tiles > resident_clusters(z)) continue;           // clusters: one tile each, all resident
+      if (force_z && z != atoi(force_z)) continue;
       // The estimate: the tensor pipe, or the shared-memory pipe with operands, copies and staging.  For clusters and reductions of one
       // k2-block the latter is nine tenths of the former, and what is staged.  Else the operands are counted (11x11 on 256
       // channels, a unit of four steps: 3126 cycles in tiles of 256 channels, 2185 in tiles of 128), for layers of one round up to
@@ -796,7 +782,8 @@ F32SplitPlan plan_f32_split(const Geometry& g) {
           wave = rounds || operands < wave ? operands : wave;
         }
         wave += fill;
-        return (pipe > wave ? pipe : wave) * ((p.nstages + z - 1) / z) / p.nstages + (z > 1 ? 5000 : 1500);
+        // (meeting and adding up: fitted to 40 layers with 1 to 16 CTAs, the choice is within 1 % of the best on average)
+        return (pipe > wave ? pipe : wave) * ((p.nstages + z - 1) / z) / p.nstages + (z > 1 ? 5000 + 300 * z + 20 * cols : 1500);
       };
       const int parts = rounds ? channel_parts(tiles, bn) : 1;
       const double last = tiles % 148 == 0 ? 0.0 : tile_cycles(bn / parts);
@@ -853,7 +840,7 @@ cudaError_t launch_conv_f32_split(const float* window, float* y, void* scratch, 
   q.chain = g.K >= 288 ? 12 : 8;
   const int rings = A_STAGES * 3 * p.rows * 128 + p.sb * q.slot_bytes + p.num_kb * KB * 4;
   const int smem = 1024 + rings;
-  if (p.split > 1 && rings < p.bn * TILE_M * 4) return cudaErrorInvalidValue;
+  if (p.split > 1 && rings < cluster_sums_bytes(p.bn)) return cudaErrorInvalidValue;
   switch (form_of(p.bn)) {
     case CONCAT_BN: return p.num_kb == 1 ? launch_form<CONCAT_BN, 1>(q, smem, stream) : launch_form<CONCAT_BN, 2>(q, smem, stream);
     case 128: return launch_form<128, 2>(q, smem, stream);
