@@ -308,6 +308,15 @@ int32_t im2win_f16_runs_form(const im2win_shape* shape, int32_t form[12]) {
   return p.eligible;
 }
 
+// The same: CTAs that share the reduction of a tile in the kernel that an fp16 layer takes.
+int32_t im2win_f16_tile_ctas(const im2win_shape* shape) {
+  Geometry g;
+  ScratchLayout l;
+  if (derive_geometry(shape, &g) != IM2WIN_OK || scratch_layout(g, IM2WIN_F16, &l) != IM2WIN_OK) return 0;
+  if (l.f16_runs) return plan_f16_runs(g).split;
+  return l.f16_shift && !l.f16_stem && !l.f16_mat && !l.f16_raw ? plan_f16_shift(g).split : 1;
+}
+
 // The same for the fp32 tensor-core kernel: channel tile, CTAs of a tile, parts of the last round's tiles.
 int32_t im2win_f32_split_form(const im2win_shape* shape, int32_t form[3]) {
   Geometry g;

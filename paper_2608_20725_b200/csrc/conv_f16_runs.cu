@@ -26,6 +26,9 @@
 // Above 128 channels two CTAs form a pair (M = 256, cta_group::2): each stages its own position tile and half of the filter,
 // and the second CTA's MMA warp tells the leader that its half of a filter slot has arrived.
 //
+// Where tiles are so few that SMs would be left over, the CTAs of a cluster share a tile's k2-blocks and add their accumulators up
+// (SPLIT; see choose_split for when and what it gives).  A part may begin and end within a raw slot, which then two CTAs copy.
+//
 // What bounds it: no single pipe.  With the read-back, the S stores, the MMAs and the output stores all left out, what remains
 // (copies, hand-offs, the staging warps' arithmetic) still takes four fifths of the time: 86 of 109 us for 3x3 on 64 channels at
 // 56x56, batch 128.  Measured: 3x3 stride 2 on 256 -> 512 channels at 28x28, batch 128, 140 us with the gathering kernel,
@@ -87,6 +90,7 @@ struct alignas(64) RunsParams {
   int32_t ntm;                                // position tiles
   int32_t planes;                             // the least number of channel planes that is a multiple of 16 bytes; 0: bulk copies
   int32_t seg_bytes;                          // tiled copies: from image to image of a tile in a raw slot
+  int32_t split;                              // CTAs of a cluster that share the k2-blocks of a tile
 };
 
 __device__ __forceinline__ uint32_t ld_shared_u16(uint32_t addr) {
@@ -129,16 +133,18 @@ __device__ __forceinline__ TileRuns tile_runs(const RunsParams& q, uint32_t q0) 
   return r;
 }
 
-// The outputs y[i * ystride], i < count <= 16, that came out infinite or NaN although a zero filter element may have met an
+// The outputs y[i * ystride], i < which <= 16 (MASK: those whose bit i of `which` is set), that came out infinite or NaN although a zero filter element may have met an
 // infinity or NaN from outside their window (RunsParams::foreign): in fp32 FMAs, k ascending, from the window at x and
 // rows i of the filter image at f.  Sixteen sums at a time keep the loads of the filter (the same address in every lane) in
 // flight; they end early once all are NaN.  (A function of its own: expanded beside the epilogue it costs spills.)
+template <bool MASK>
 __device__ __noinline__ void exact_outputs(const unsigned char* __restrict__ x, const unsigned char* __restrict__ f, float* y,
                                            int64_t ystride, int64_t chan_bytes, int C, int Kh, int Kw, int s, int E, int g_step,
-                                           int j_step, int quad, int count) {
+                                           int j_step, int quad, int which) {
   auto not_finite = [](float v) { return !(fabsf(v) <= 3.4028234663852886e38f); };
   bool any = false;
-  for (int i = 0; i < count; ++i) any |= not_finite(y[i * ystride]);
+  auto mine = [&](int i) { return MASK ? (which >> i & 1) != 0 : i < which; };
+  for (int i = 0; MASK ? i < 16 : i < which; ++i) any |= mine(i) && not_finite(y[i * ystride]);
   if (!any) return;
   float acc[16];
 #pragma unroll
@@ -168,7 +174,7 @@ __device__ __noinline__ void exact_outputs(const unsigned char* __restrict__ x, 
 #pragma unroll
   for (int i = 0; i < 16; ++i) {
     float* p = y + i * ystride;
-    if (i < count && not_finite(*p)) *p = acc[i];
+    if (mine(i) && not_finite(*p)) *p = acc[i];
   }
 }
 
@@ -220,6 +226,22 @@ __device__ __forceinline__ int slot_row(const RunsParams& q, int x) {
 enum StagingMode { HALVES, WORDS, ROW_PAIRS, UNITS };
 constexpr int group_of(int mode) { return mode == WORDS ? 6 : 3; }
 
+// The part of the reduction a CTA does: k2-blocks, units and raw slots (of the first and the last slot maybe not every unit).
+struct Part {
+  int kb0, kb1, j0, j1, slot0, slot1;
+};
+__device__ __forceinline__ Part part_of(const RunsParams& q, int rank) {
+  const int per_slot = q.quad ? q.units : q.octs * q.E;
+  Part p;
+  p.kb0 = q.num_kb * rank / q.split;
+  p.kb1 = q.num_kb * (rank + 1) / q.split;
+  p.j0 = 8 * p.kb0;
+  p.j1 = 8 * p.kb1 < q.units ? 8 * p.kb1 : q.units;
+  p.slot0 = p.j0 / per_slot;
+  p.slot1 = (p.j1 + per_slot - 1) / per_slot;
+  return p;
+}
+
 struct StagingBarriers {
   uint32_t a_full0, a_empty0, raw_full0, raw_empty0;        // (a_full0 in a pair: the leader's, wherever it lies)
 };
@@ -249,8 +271,8 @@ __device__ __forceinline__ void locate_row(const RunsParams& q, const TileRuns& 
 // are in flight together, and the slot is given back before the wait for a free S stage.  (A unit at a time, both
 // warpgroups on every slot, took 87 instructions and 560 cycles a unit: 3x3 stride 2 on 256 -> 512 channels at 28x28, batch
 // 128, 121 us.)
-template <int MODE, bool PAIR>
-__device__ __forceinline__ void stage_tiles(const RunsParams& q, const Walk& walk, uint32_t a_ring, uint32_t raw_ring,
+template <int MODE, bool PAIR, bool SPLIT>
+__device__ __forceinline__ void stage_tiles(const RunsParams& q, const Walk& walk, const Part& part, uint32_t a_ring, uint32_t raw_ring,
                                             const StagingBarriers& b, int warp, int lane, volatile uint32_t* abort_flag) {
   auto arrive_full = [&](int stage) {
     if (PAIR) mbar_arrive_cluster(b.a_full0 + 8 * stage);
@@ -262,7 +284,7 @@ __device__ __forceinline__ void stage_tiles(const RunsParams& q, const Walk& wal
   const int team = warp / TEAM, row = ((warp % TEAM) * 32 + lane) * ROWS;
   const int plane = (q.Ho * q.Wp + q.Wq * q.s - q.Wp) * q.Kh;     // (up to the end of the last virtual column)
   const int per_oct = q.E, nocts = q.units / q.E, octs = q.octs;
-  const int nslots = (nocts + octs - 1) / octs;
+  const int nslots = SPLIT ? part.slot1 - part.slot0 : (nocts + octs - 1) / octs;      // (`next` counts from the part's first slot)
   auto swizzled = [](int r) { return (uint32_t)(r * 128 + ((r & 7) << 4)); };
   // (lanes 4 to 7 of eight store the second row of a pair first: the eight meet eight bank groups)
   const int second = ROWS == 2 ? (lane >> 2) & 1 : 0;
@@ -312,8 +334,9 @@ __device__ __forceinline__ void stage_tiles(const RunsParams& q, const Walk& wal
       if (!ok) break;
       uint32_t src = raw_ring + sr * q.raw_slot;
       const bool halo_turn = q.halo > 0 && (int)(turn % TEAM) == warp % TEAM;
-      const int here = nocts - next * octs < octs ? nocts - next * octs : octs;
-      int j = next * octs * per_oct;                         // unit
+      const int slot = SPLIT ? part.slot0 + next : next;
+      const int here = nocts - slot * octs < octs ? nocts - slot * octs : octs;
+      int j = slot * octs * per_oct;                                // unit
       for (int o = 0; o < here && ok; ++o, src += 8u * q.region) {
         for (int e0 = 0; e0 < per_oct && ok; e0 += GROUP) {
           const int n = per_oct - e0 < GROUP ? per_oct - e0 : GROUP;
@@ -357,7 +380,8 @@ __device__ __forceinline__ void stage_tiles(const RunsParams& q, const Walk& wal
 #pragma unroll
           for (int i = 0; i < GROUP; ++i) {
             if (i >= n) break;
-            go_to((j + i) >> 3);
+            if (SPLIT && (j + i < part.j0 || j + i >= part.j1)) continue;      // (another CTA's)
+            go_to(((j + i) >> 3) - part.kb0);
             if (!ok) break;
             const uint32_t stage = a_ring + sa * q.a_stage, ch = (uint32_t)((j + i) & 7) << 4;
             if constexpr (ROWS == 2) {
@@ -376,9 +400,9 @@ __device__ __forceinline__ void stage_tiles(const RunsParams& q, const Walk& wal
       if (sr >= q.sr) { sr -= q.sr; pr ^= 1u; }
     }
     if (team < teams) next -= nslots;
-    go_to(q.num_kb - 1);
+    go_to(part.kb1 - part.kb0 - 1);
     if (!ok) break;
-    if ((q.units & 1) != 0 && team == 0) {                   // zeros up to the end of the MMA's last step
+    if ((q.units & 1) != 0 && part.kb1 == q.num_kb && team == 0) {                   // zeros up to the end of the MMA's last step
       const uint32_t stage = a_ring + sa * q.a_stage, ch = (uint32_t)(q.units & 7) << 4;
       st_shared16(stage + (dst0 ^ ch), 0u, 0u, 0u, 0u);
       if (ROWS == 2) st_shared16(stage + (dst1 ^ ch), 0u, 0u, 0u, 0u);
@@ -394,8 +418,8 @@ __device__ __forceinline__ void stage_tiles(const RunsParams& q, const Walk& wal
 // The form for layers that give the teams too little to share out (see plan_f16_runs) or have more rows below a tile than a warp
 // can read for a group of units.  Warpgroup wg takes every second unit; every warp passes every stage and every slot in order, so no wait by phase
 // parity can run ahead.
-template <bool PAIR>
-__device__ __forceinline__ void stage_units(const RunsParams& q, const Walk& walk, uint32_t a_ring, uint32_t raw_ring,
+template <bool PAIR, bool SPLIT>
+__device__ __forceinline__ void stage_units(const RunsParams& q, const Walk& walk, const Part& part, uint32_t a_ring, uint32_t raw_ring,
                                             const StagingBarriers& b, int warp, int lane, volatile uint32_t* abort_flag) {
   const int wg = warp >> 2, row = (warp & 3) * 32 + lane;
   const int plane = (q.Ho * q.Wp + q.Wq * q.s - q.Wp) * q.Kh;     // (up to the end of the last virtual column)
@@ -411,20 +435,27 @@ __device__ __forceinline__ void stage_units(const RunsParams& q, const Walk& wal
     locate_row(q, tr, plane, q0 + row, q.quad, rb);
     if (lane < q.halo) locate_row(q, tr, plane, q0 + TILE_M + lane, q.quad, hb);
     uint32_t src = 0;                                        // of the current unit; inside the slot: its number, and its e
-    int in_slot = 0, e = 0;
-    for (int kb = 0; kb < q.num_kb && ok; ++kb) {
+    int in_slot = SPLIT ? part.j0 - part.slot0 * per_slot : 0, e = 0;
+    bool enter = true;                                       // the next unit is the first one of a slot
+    for (int kb = part.kb0; kb < part.kb1 && ok; ++kb) {
       ok = mbar_wait(b.a_empty0 + 8 * sa, pa ^ 1u, abort_flag, q.status);
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
       const uint32_t stage = a_ring + sa * q.a_stage;
       const int n_units = q.units - 8 * kb < 8 ? q.units - 8 * kb : 8;
       for (int ch = 0; ch < n_units; ++ch) {
-        if (in_slot == 0) {
+        if (enter) {
           ok = mbar_wait(b.raw_full0 + 8 * sr, pr, abort_flag, q.status);
           ok = __all_sync(0xffffffffu, ok);
           if (!ok) break;
           src = raw_ring + sr * q.raw_slot;
           e = 0;
+          if (SPLIT && in_slot > 0) {                        // (the part starts within a slot)
+            const int o = q.quad ? 0 : in_slot / q.E;
+            e = in_slot - o * q.E;
+            src += 8u * q.region * o + unit_step * e;
+          }
+          enter = false;
         }
         if ((ch & 1) == wg) {
           auto unit = [&](const uint32_t (&at)[8], int srow) {
@@ -438,11 +469,12 @@ __device__ __forceinline__ void stage_units(const RunsParams& q, const Walk& wal
           // the rows below the tile: lanes of one of the warpgroup's warps, another one from unit to unit
           if ((ch >> 1) == (warp & 3) && lane < q.halo) unit(hb, TILE_M + lane);
         }
-        if (++in_slot == per_slot || 8 * kb + ch == q.units - 1) {
+        if (++in_slot == per_slot || 8 * kb + ch == part.j1 - 1) {
           __syncwarp();
           if (lane == 0) mbar_arrive(b.raw_empty0 + 8 * sr);
           if (++sr == q.sr) { sr = 0; pr ^= 1u; }
           in_slot = 0;
+          enter = true;
         }
         ++e;
         src += e == q.E ? oct_step : unit_step;
@@ -464,7 +496,7 @@ __device__ __forceinline__ void stage_units(const RunsParams& q, const Walk& wal
   }
 }
 
-template <int BNMAX, bool PAIR, int MODE>
+template <int BNMAX, bool PAIR, int MODE, bool SPLIT>
 __global__ void __launch_bounds__(THREADS, 1) conv_f16_runs_kernel(const __grid_constant__ RunsParams q) {
   constexpr int NACC = 512 / BNMAX, ACC_LOG = NACC == 2 ? 1 : (NACC == 4 ? 2 : 3);      // ring of accumulators in tensor memory
   extern __shared__ unsigned char smem_dyn[];
@@ -482,11 +514,16 @@ __global__ void __launch_bounds__(THREADS, 1) conv_f16_runs_kernel(const __grid_
   const uint32_t b_full0 = raw_empty0 + 8 * MAX_RAW, b_empty0 = b_full0 + 8 * MAX_B;
   const uint32_t acc_full0 = b_empty0 + 8 * MAX_B, acc_empty0 = acc_full0 + 8 * MAX_ACC;
   const int rank = PAIR ? (int)cluster_ctarank() : 0;
-  const Walk walk = {PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x, PAIR ? (int)(gridDim.x >> 1) : (int)gridDim.x, rank, PAIR};
+  // (SPLIT: the cluster has one item, this CTA that part of its reduction)
+  const int share = SPLIT ? (int)cluster_ctarank() : 0;
+  const Walk walk = {SPLIT ? (int)blockIdx.x / q.split : (PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x),
+                     SPLIT ? q.nwork : (PAIR ? (int)(gridDim.x >> 1) : (int)gridDim.x), rank, PAIR};
+  const Part part = SPLIT ? part_of(q, share) : Part{0, q.num_kb, 0, q.units, 0, 0};   // (unsplit the slots are counted where they are used)
   // the leader's barriers that both CTAs of a pair arrive on
   const uint32_t a_full_dst = PAIR ? mapa_shared(a_full0, 0) : a_full0;
   const uint32_t b_full_dst = PAIR ? mapa_shared(b_full0, 0) : b_full0;
   const uint32_t acc_empty_dst = PAIR ? mapa_shared(acc_empty0, 0) : acc_empty0;
+  bool met = false;                                        // SPLIT: this warp has been at the cluster's barriers
   const int b_rows = PAIR ? q.bn / 2 : q.bn;               // filter rows (channels) this CTA holds of a kernel column
 
   if (threadIdx.x == 0) {
@@ -517,8 +554,8 @@ __global__ void __launch_bounds__(THREADS, 1) conv_f16_runs_kernel(const __grid_
     // ---------------- staging: raw runs -> S ------------------------------------------------------------
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_STAGING));
     const StagingBarriers b = {a_full_dst, a_empty0, raw_full0, raw_empty0};
-    if constexpr (MODE == UNITS) stage_units<PAIR>(q, walk, a_ring, raw_ring, b, warp, lane, &abort_flag);
-    else stage_tiles<MODE, PAIR>(q, walk, a_ring, raw_ring, b, warp, lane, &abort_flag);
+    if constexpr (MODE == UNITS) stage_units<PAIR, SPLIT>(q, walk, part, a_ring, raw_ring, b, warp, lane, &abort_flag);
+    else stage_tiles<MODE, PAIR, SPLIT>(q, walk, part, a_ring, raw_ring, b, warp, lane, &abort_flag);
   } else if (warp < STAGING_WARPS + 4) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_MISC));
     if (warp == STAGING_WARPS && rank == 0) {
@@ -552,7 +589,7 @@ __global__ void __launch_bounds__(THREADS, 1) conv_f16_runs_kernel(const __grid_
         uint32_t more = 0u;                                  // the tile's first instruction clears the accumulator
         const bool fetch_b = !q.resident || w == walk.first;          // (a resident filter is complete after the first tile)
         if (q.resident) slot = 0;
-        for (int kb = 0; kb < q.num_kb && ok; ++kb) {
+        for (int kb = part.kb0; kb < part.kb1 && ok; ++kb) {
           const int nks = kb == q.num_kb - 1 ? q.nks_last : KB / 16;
           ok = need(a_full0 + 8 * sa, pa, a_seen);
           if (!ok) break;
@@ -562,7 +599,7 @@ __global__ void __launch_bounds__(THREADS, 1) conv_f16_runs_kernel(const __grid_
           uint32_t npa = pa;
           if (nsa == q.sa) { nsa = 0; npa ^= 1u; }
           for (int g = 0; g < q.G; g += q.cols, a_view += 8u * q.cols) {
-            const bool last_unit = g + q.cols == q.G, last = kb + 1 == q.num_kb && last_unit;
+            const bool last_unit = g + q.cols == q.G, last = kb + 1 == part.kb1 && last_unit;
             int nslot = slot + 1;
             uint32_t npb = pb;
             if (nslot == q.sb) { nslot = 0; if (!q.resident) npb ^= 1u; }
@@ -615,9 +652,10 @@ __global__ void __launch_bounds__(THREADS, 1) conv_f16_runs_kernel(const __grid_
       bool ok = true;
       int slot = 0;
       uint32_t pb = 0;
-      const int slots = q.num_kb * q.G / q.cols, column = q.bn * 128;       // bytes of a kernel column's image
+      const int slots = (part.kb1 - part.kb0) * q.G / q.cols, column = q.bn * 128;       // bytes of a kernel column's image
       for (int w = walk.first; w < q.nwork && ok; w += walk.step) {
         const unsigned char* src = q.fp + (int64_t)(w % q.ntn) * slots * q.cols * column + rank * b_rows * 128;
+        if (SPLIT) src = q.fp + ((int64_t)(w % q.ntn) * q.num_kb + part.kb0) * q.G * column;
         for (int u = 0; u < slots; ++u, src += q.cols * column) {
           ok = mbar_wait(b_empty0 + 8 * slot, pb ^ 1u, &abort_flag, q.status);
           ok = __all_sync(0xffffffffu, ok);
@@ -643,7 +681,7 @@ __global__ void __launch_bounds__(THREADS, 1) conv_f16_runs_kernel(const __grid_
       int sr = 0;
       uint32_t pr = 0, sc = warp & 1;
       const int plane = (q.Ho * q.Wp + q.Wq * q.s - q.Wp) * q.Kh;
-      const int per_slot = q.quad ? 4 : 8 * q.octs, nslots = q.quad ? 1 : (q.C + per_slot - 1) / per_slot;
+      const int per_slot = q.quad ? 4 : 8 * q.octs, slot1 = SPLIT ? part.slot1 : (q.quad ? 1 : (q.C + per_slot - 1) / per_slot);
       for (int w = walk.first; w < q.nwork && ok; w += walk.step) {
         const TileRuns tr = tile_runs(q, walk.start(q, w));
         const int nseg = (int)(tr.n1 - tr.n0) + 1;
@@ -684,7 +722,7 @@ __global__ void __launch_bounds__(THREADS, 1) conv_f16_runs_kernel(const __grid_
         }
         // bytes behind the first slot's last run, up to the next 16-byte boundary, that are still of the tensor
         const int64_t spare = q.win_bytes - 15 - ((int64_t)tr.n1 * q.img_bytes + (per_slot - 1) * q.chan_bytes + (int64_t)tr.end1 * ES);
-        for (int sl = 0; sl < nslots; ++sl, ++sc) {
+        for (int sl = part.slot0; sl < slot1; ++sl, ++sc) {
           if (sc & 1) {
             if (++sr == q.sr) { sr = 0; pr ^= 1u; }
             continue;
@@ -782,6 +820,47 @@ __global__ void __launch_bounds__(THREADS, 1) conv_f16_runs_kernel(const __grid_
       ++ac;
       tc_fence_after();
       const uint32_t d = tmem_acc + ((uint32_t)(lq * 32) << 16) + ab * BNMAX;
+      if constexpr (SPLIT) {
+        // the parts of the cluster's tile added up: each CTA finishes its share of the channels
+        const ClusterSums sums(a_ring, q.split, share, limit);
+        const int position = lq * 32 + lane;
+        met = true;
+        __syncwarp();
+        cluster_sync_all();                                  // (every MMA of every CTA has completed)
+#pragma unroll 1
+        for (int c0 = h * (BNMAX / 2); c0 < (h + 1) * (BNMAX / 2) && c0 < limit; c0 += 32) {
+          uint32_t v[32];
+          float f[32];
+          tmem_ld32(d + c0, v);
+#pragma unroll
+          for (int e = 0; e < 32; ++e) f[e] = __uint_as_float(v[e]);
+          sums.store(f, c0, limit, position);
+        }
+        __syncwarp();
+        cluster_sync_all();
+        if (valid) {
+          const int first = share * sums.per, end = first + sums.per < limit ? first + sums.per : limit;
+          float zero = 0.f;
+          for (int c = first + h; c < end; c += 2) {
+            const float sum = sums.sum(c - first, position);
+            zero = fmaf(sum, 0.f, zero);
+            yrow[(int64_t)c * q.HoWo] = sum;
+          }
+          if (q.foreign && zero != 0.f) {                    // (a NaN: one of them is not finite)
+            const unsigned char* x = q.win + (int64_t)n * q.img_bytes + ((int64_t)ho * q.Wp + (int64_t)i0 * q.s) * q.Kh * ES;
+            const int column = q.bn * 128;
+            const unsigned char* f = q.fp + (int64_t)nt * q.num_kb * q.G * column;
+            for (int c = first & ~15; c < end; c += 16) {
+              int which = 0;
+              for (int i = 0; i < 16; ++i)
+                if (c + i >= first && c + i < end && ((c + i - first) & 1) == h) which |= 1 << i;
+              exact_outputs<true>(x, f + c * 128, yrow + (int64_t)c * q.HoWo, q.HoWo, q.chan_bytes, q.C, q.Kh, q.Kw, q.s, q.E, column,
+                            q.G * column, q.quad, which);
+            }
+          }
+        }
+        break;
+      }
 #pragma unroll 1
       for (int c0 = h * (BNMAX / 2); c0 < (h + 1) * (BNMAX / 2) && c0 < limit; c0 += 32) {
         uint32_t v[32];
@@ -803,7 +882,7 @@ __global__ void __launch_bounds__(THREADS, 1) conv_f16_runs_kernel(const __grid_
             const int column = q.bn * 128;                 // bytes of a filter column's image
             const unsigned char* f = q.fp + (int64_t)nt * q.num_kb * q.G * column;
             for (int c = c0; c < c0 + 32 && c < limit; c += 16)
-              exact_outputs(x, f + c * 128, yrow + (int64_t)c * q.HoWo, q.HoWo, q.chan_bytes, q.C, q.Kh, q.Kw, q.s, q.E,
+              exact_outputs<false>(x, f + c * 128, yrow + (int64_t)c * q.HoWo, q.HoWo, q.chan_bytes, q.C, q.Kh, q.Kw, q.s, q.E,
                             column, q.G * column, q.quad, limit - c < 16 ? limit - c : 16);
           }
         }
@@ -812,6 +891,14 @@ __global__ void __launch_bounds__(THREADS, 1) conv_f16_runs_kernel(const __grid_
         __syncwarp();
         if (lane == 0) arrive_empty(ab);
       }
+    }
+  }
+
+  if constexpr (SPLIT) {                                     // (the epilogue warps have met theirs, unless a wait gave up)
+    if (warp < STAGING_WARPS + 4 || !met) {
+      __syncwarp();
+      cluster_sync_all();
+      cluster_sync_all();
     }
   }
 
@@ -872,26 +959,34 @@ __global__ void __launch_bounds__(256) pack_f16_runs_kernel(const uint16_t* __re
   }
 }
 
-template <int BNMAX, bool PAIR, int MODE>
+template <int BNMAX, bool PAIR, int MODE, bool SPLIT>
 cudaError_t launch_mode(const RunsParams& q, int smem, cudaStream_t stream) {
+  constexpr auto kernel = conv_f16_runs_kernel<BNMAX, PAIR, MODE, SPLIT>;
   static bool attr_done[64] = {};
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
   if (!attr_done[dev]) {
-    cudaError_t e = cudaFuncSetAttribute(conv_f16_runs_kernel<BNMAX, PAIR, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRunsSmem);
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kRunsSmem);
+    if (e == cudaSuccess && SPLIT) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
     attr_done[dev] = true;
   }
+  if (SPLIT) return launch_after_previous(kernel, q.nwork * q.split, q.split, THREADS, smem, stream, q);
   const int most = PAIR ? 74 : 148, grid = (q.nwork < most ? q.nwork : most) * (PAIR ? 2 : 1);
-  return launch_after_previous(conv_f16_runs_kernel<BNMAX, PAIR, MODE>, grid, PAIR ? 2 : 1, THREADS, smem, stream, q);
+  return launch_after_previous(kernel, grid, PAIR ? 2 : 1, THREADS, smem, stream, q);
 }
 
-template <int BNMAX, bool PAIR>
+template <int BNMAX, bool PAIR, bool SPLIT>
 cudaError_t launch_form(int mode, const RunsParams& q, int smem, cudaStream_t stream) {
-  if (mode == HALVES) return launch_mode<BNMAX, PAIR, HALVES>(q, smem, stream);
-  if (mode == WORDS) return launch_mode<BNMAX, PAIR, WORDS>(q, smem, stream);
-  if (mode == ROW_PAIRS) return launch_mode<BNMAX, PAIR, ROW_PAIRS>(q, smem, stream);
-  return launch_mode<BNMAX, PAIR, UNITS>(q, smem, stream);
+  if (mode == HALVES) return launch_mode<BNMAX, PAIR, HALVES, SPLIT>(q, smem, stream);
+  if (mode == WORDS) return launch_mode<BNMAX, PAIR, WORDS, SPLIT>(q, smem, stream);
+  if (mode == ROW_PAIRS) return launch_mode<BNMAX, PAIR, ROW_PAIRS, SPLIT>(q, smem, stream);
+  return launch_mode<BNMAX, PAIR, UNITS, SPLIT>(q, smem, stream);
+}
+
+template <int BNMAX>
+cudaError_t launch_single(int mode, const RunsParams& q, int smem, cudaStream_t stream) {
+  return q.split > 1 ? launch_form<BNMAX, false, true>(mode, q, smem, stream) : launch_form<BNMAX, false, false>(mode, q, smem, stream);
 }
 
 }  // namespace
@@ -922,6 +1017,27 @@ static bool encode_window_rows(CUtensorMap* map, const uint16_t* window, const G
 static int64_t pack_channels(int64_t E, int C) {
   const int64_t n = ((8 + E - 2) / E + 1) * 8;
   return n < C ? n : C;
+}
+
+// CTAs of a cluster that share the k2-blocks of a tile, where there are so few tiles that an SM each is left for them: a k2-block
+// takes 1 us, meeting and adding up 1 us and 0.02 for each channel of a tile (fitted to 33 such layers with 1 to 16 CTAs; the choice is
+// within 0.7 % of the best on average, 9 % at the most).  Alone / split, us: 3x3 stride 2 on 512 -> 128 channels at 15x15, batch 27, 57 /
+// 20; 5x5 stride 2 on 128 channels at 39x39 29 / 12; 3x3 on 64 -> 104 channels at 50x50 (5 k2-blocks) 9.2 either way.
+// The tiles are those of the batch these images belong to: they decide the order of the sums.
+static int choose_split(const Geometry& g, const RunsPlan& p) {
+  // testing aid: CTAs per tile (1 where the kernel is forced and this is not)
+  if (const char* v = debug_getenv("IM2WIN_F16_SPLIT")) return atoi(v) < p.num_kb ? atoi(v) : p.num_kb;
+  if (debug_getenv("IM2WIN_F16_KERNEL")) return 1;
+  const int64_t tiles = ((int64_t)g.plan_N * g.Ho * p.Wq + TILE_M - 1) / TILE_M * p.ntn;
+  if (tiles > 74 || g.K > kMostSplitTerms) return 1;
+  int split = 1;
+  double best = p.num_kb;
+  for (int z = 2; z <= kMaxCtas && z <= p.num_kb; ++z) {
+    if (tiles * z > 148 || tiles > resident_clusters(z)) continue;
+    const double cost = 1.0 + 0.02 * p.bn + (p.num_kb + z - 1) / z + 0.05 * z;
+    if (cost < best) { best = cost; split = z; }
+  }
+  return split;
 }
 
 RunsPlan plan_f16_runs(const Geometry& g) {
@@ -966,6 +1082,8 @@ RunsPlan plan_f16_runs(const Geometry& g) {
   // 0.92 to 1.15 with up to 256 on 13.  N of a pair's instruction: a multiple of 32.  Wider tiles for the others would want more scratch)
   p.pair = p.bn > 128 && p.bn % 32 == 0 && ntm > 1 && p.num_kb * p.G >= 8;
   if (const char* v = debug_getenv("IM2WIN_F16_PAIR")) p.pair = p.pair && v[0] != '0';     // testing aid
+  p.split = choose_split(g, p);
+  p.pair = p.pair && p.split == 1;
   p.ntm = (int32_t)ntm;
   p.nwork = (int32_t)((p.pair ? (ntm + 1) / 2 : ntm) * p.ntn);
   const int budget = kRunsSmem - 1024;
@@ -1073,10 +1191,12 @@ cudaError_t launch_conv_f16_runs(const uint16_t* window, float* y, void* scratch
     if (!encode_window_rows(&q.map, window, g, p)) return cudaErrorInvalidValue;
   }
   q.slot_bytes = p.slot_bytes; q.cols = p.cols; q.ntm = p.ntm; q.resident = p.resident ? 1 : 0;
-  const int smem = 1024 + p.sa * p.a_stage + p.sb * p.slot_bytes + p.sr * p.raw_slot;
-  if (p.bn <= 64) return launch_form<64, false>(p.mode, q, smem, stream);
-  if (p.bn <= 128) return launch_form<128, false>(p.mode, q, smem, stream);
-  return p.pair ? launch_form<256, true>(p.mode, q, smem, stream) : launch_form<256, false>(p.mode, q, smem, stream);
+  q.split = p.split;
+  int smem = 1024 + p.sa * p.a_stage + p.sb * p.slot_bytes + p.sr * p.raw_slot;
+  if (p.split > 1 && smem < 1024 + cluster_sums_bytes(p.bn)) smem = 1024 + cluster_sums_bytes(p.bn);
+  if (p.bn <= 64) return launch_single<64>(p.mode, q, smem, stream);
+  if (p.bn <= 128) return launch_single<128>(p.mode, q, smem, stream);
+  return p.pair ? launch_form<256, true, false>(p.mode, q, smem, stream) : launch_single<256>(p.mode, q, smem, stream);
 }
 
 }  // namespace im2win

@@ -34,6 +34,9 @@
 // producer warps read the accumulator from tensor memory and store the real
 // outputs.  Two rings of stages: S tiles (each used by Kw MMA groups) and
 // filter tiles (each used by one).  All mbarrier waits are bounded.
+//
+// Where tiles are so few that SMs would be left over, the CTAs of a cluster share a tile's k-blocks and add their accumulators up
+// (SPLIT; see choose_split for when and what it gives).
 #include <cuda.h>
 #include <stdlib.h>
 
@@ -67,11 +70,12 @@ struct ShiftParams {
   int32_t halo8;          // halo rows of a sub-tile, rounded up to 8
   int32_t nbig;           // the first nbig tiles are 256 positions tall (two MMA halves), the rest 128
   int32_t a_stage_bytes, sa, sb;
+  int32_t split;          // CTAs of a cluster that share the k-blocks of a tile
 };
 
 
-template <int BN, int ITEMS>
-__global__ void __launch_bounds__(NUM_THREADS, (BN <= 128 ? 2 : 1))
+template <int BN, int ITEMS, bool SPLIT>
+__global__ void __launch_bounds__(NUM_THREADS, (BN <= 128 && !SPLIT ? 2 : 1))
 conv_f16_shift_kernel(const __grid_constant__ CUtensorMap fmap, ShiftParams q) {
   constexpr int B_STAGE_BYTES = BN * KB * 2;
 
@@ -92,10 +96,13 @@ conv_f16_shift_kernel(const __grid_constant__ CUtensorMap fmap, ShiftParams q) {
   const uint32_t acc_bar = smem_u32(&bars[4 * MAX_STAGES]);
 
   // Tall tiles (two 128-row MMA halves sharing every filter stage) come first in the grid.
-  const bool big = (int)blockIdx.x < q.nbig;
+  const int tile = SPLIT ? (int)blockIdx.x / q.split : (int)blockIdx.x;
+  const bool big = !SPLIT && tile < q.nbig;
   const int mt = big ? 2 : 1;
-  const int64_t q0 = big ? (int64_t)blockIdx.x * (2 * TILE_M)
-                         : (int64_t)q.nbig * (2 * TILE_M) + (int64_t)((int)blockIdx.x - q.nbig) * TILE_M;
+  const int64_t q0 = big ? (int64_t)tile * (2 * TILE_M) : (int64_t)q.nbig * (2 * TILE_M) + (int64_t)(tile - q.nbig) * TILE_M;
+  // k-blocks of this CTA: all, or its share of them in a cluster
+  const int rank = SPLIT ? (int)blockIdx.x - tile * q.split : 0;
+  const int kb0 = SPLIT ? q.num_kb * rank / q.split : 0, kb1 = SPLIT ? q.num_kb * (rank + 1) / q.split : q.num_kb;
   const int n0 = blockIdx.y * BN;
   const int rows = TILE_M * mt + q.halo8;          // rows of one sub-tile
   const int total_rows = q.s * rows;
@@ -174,7 +181,7 @@ conv_f16_shift_kernel(const __grid_constant__ CUtensorMap fmap, ShiftParams q) {
     // Dead rows and padded k2 read a word of the status block that is always zero, so nothing
     // needs masking afterwards.  (Holding the next unit's loads in a second register buffer,
     // and L2 prefetches of the next k-blocks' runs, were measured and did not pay.)
-    constexpr int G = ITEM_GROUP;
+    constexpr int G = SPLIT && ITEMS <= 10 ? ITEMS : ITEM_GROUP;
     constexpr int NG = ITEMS / G;
     const uint16_t* __restrict__ zero16 = reinterpret_cast<const uint16_t*>(q.status + 2);
     auto issue = [&](int kb, int climit, int gidx, uint32_t (&h)[G][8]) {
@@ -208,7 +215,7 @@ conv_f16_shift_kernel(const __grid_constant__ CUtensorMap fmap, ShiftParams q) {
     int st = 0;                 // ring slot and its phase bit, advanced without divisions
     uint32_t ph = 0;
     uint32_t buf[G][8];
-    for (int kb = 0; kb < q.num_kb && ok; ++kb) {
+    for (int kb = kb0; kb < kb1 && ok; ++kb) {
       const uint32_t a_stage = a_ring + st * q.a_stage_bytes;
       const int climit = kb == q.num_kb - 1 ? q.chunks_last : 8;   // the MMAs skip the padded tail of k
 #pragma unroll
@@ -240,7 +247,7 @@ conv_f16_shift_kernel(const __grid_constant__ CUtensorMap fmap, ShiftParams q) {
     ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
     __syncwarp();   // lane 0 observed the barrier: orders the other lanes' accesses after it
     if (threadIdx.x == 0) TIMER_LAP(5);     // wait for the accumulator
-    if (ok) {
+    if (!SPLIT && ok) {
       tc_fence_after();
       const int lq = warp & 3;                 // tensor-memory lane quadrant this warp may read
       const int chalf = warp >> 2;             // which half of the channel tile
@@ -275,7 +282,7 @@ conv_f16_shift_kernel(const __grid_constant__ CUtensorMap fmap, ShiftParams q) {
     bool ok = true;
     int st = 0;
     uint32_t ph = 0;
-    for (int kb = 0; kb < q.num_kb && ok; ++kb) {
+    for (int kb = kb0; kb < kb1 && ok; ++kb) {
       for (int v = 0; v < q.Kw; ++v) {
         ok = mbar_wait(b_empty0 + 8 * st, ph ^ 1u, &abort_flag, q.status);
         ok = __all_sync(0xffffffffu, ok);
@@ -304,7 +311,7 @@ conv_f16_shift_kernel(const __grid_constant__ CUtensorMap fmap, ShiftParams q) {
     const uint32_t a_lo0 = smem_desc_lo(a_ring), b_lo0 = smem_desc_lo(b_ring);
     const uint32_t sub_lo = (uint32_t)sub_bytes >> 4;
     TIMER_DECL;
-    for (int kb = 0; kb < q.num_kb && ok; ++kb) {
+    for (int kb = kb0; kb < kb1 && ok; ++kb) {
       TIMER_LAP(8);
       ok = mbar_wait(a_full0 + 8 * sta, pha, &abort_flag, q.status);
       ok = __all_sync(0xffffffffu, ok);
@@ -364,6 +371,38 @@ conv_f16_shift_kernel(const __grid_constant__ CUtensorMap fmap, ShiftParams q) {
     }
   }
 
+  if constexpr (SPLIT) {
+    // ---------------- the parts of the cluster's tile added up ------------------------------------------
+    const int channels = q.Co - n0 < BN ? q.Co - n0 : BN, position = (warp & 3) * 32 + lane, h = warp >> 2;
+    const ClusterSums sums(a_ring, q.split, rank, channels);
+    __syncwarp();
+    cluster_sync_all();                                    // (every MMA of every CTA has completed)
+    if (warp < PRODUCER_WARPS) {
+      tc_fence_after();
+#pragma unroll 1
+      for (int c0 = h * (BN / 2); c0 < (h + 1) * (BN / 2) && c0 < channels; c0 += 32) {
+        uint32_t v[32];
+        float f[32];
+        tmem_ld32(tmem_acc + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)c0, v);
+#pragma unroll
+        for (int e = 0; e < 32; ++e) f[e] = __uint_as_float(v[e]);
+        sums.store(f, c0, channels, position);
+      }
+    }
+    __syncwarp();
+    cluster_sync_all();
+    const uint32_t vq = (uint32_t)q0 + (uint32_t)position;
+    if (warp < PRODUCER_WARPS && vq < (uint32_t)q.VQ) {
+      const uint32_t sg = vq / (uint32_t)q.Wq;
+      const int kq = (int)(vq - sg * (uint32_t)q.Wq);
+      const uint32_t n = sg / (uint32_t)q.Ho;
+      const int ho = (int)(sg - n * (uint32_t)q.Ho), first = rank * sums.per;
+      float* yrow = q.y + ((int64_t)n * q.Co + n0 + first) * q.HoWo + ho * q.Wo + kq;
+      if (kq < q.Wo)
+        for (int c = h; c < sums.per && first + c < channels; c += 2) yrow[(int64_t)c * q.HoWo] = sums.sum(c, position);
+    }
+  }
+
   // ---------------- teardown ---------------------------------------------------
   tc_fence_before();
   __syncthreads();
@@ -399,10 +438,10 @@ EncodeTiledFn get_encode_fn() {
 constexpr int kSmemBudget = 220 * 1024;
 
 template <int BN>
-void choose_stages(const ShiftPlan& plan, int a_bytes, int* sa, int* sb) {
+void choose_stages(const ShiftPlan& plan, int a_bytes, int split, int* sa, int* sb) {
   const int b_bytes = BN * KB * 2;
   // Narrow channel tiles leave room for two CTAs per SM: give each half of the budget.
-  const int budget = (BN <= 128 ? kSmemBudget / 2 : kSmemBudget) - 2048 - (int)plan.K2p * 4;
+  const int budget = (BN <= 128 && split == 1 ? kSmemBudget / 2 : kSmemBudget) - 2048 - (int)plan.K2p * 4;
   int a = 2, b = 2;
   // Filter stages turn over Kw (x2 for tall tiles) times faster than S stages and hide the
   // L2 latency of the TMA loads: grow them to 4 first, then S to 3, then both further.
@@ -415,22 +454,39 @@ void choose_stages(const ShiftPlan& plan, int a_bytes, int* sa, int* sb) {
   *sb = b;
 }
 
-template <int BN, int ITEMS>
+template <int BN, int ITEMS, bool SPLIT>
 cudaError_t launch_variant(const CUtensorMap& fmap, const ShiftParams& q0, const ShiftPlan& plan, int co,
                            cudaStream_t stream) {
   ShiftParams q = q0;
   int sa, sb;
-  choose_stages<BN>(plan, q.a_stage_bytes, &sa, &sb);
+  choose_stages<BN>(plan, q.a_stage_bytes, q.split, &sa, &sb);
   q.sa = sa;
   q.sb = sb;
-  const int smem_bytes = sa * q.a_stage_bytes + sb * BN * KB * 2 + (int)plan.K2p * 4 + 1024;
-  cudaError_t e = cudaFuncSetAttribute(conv_f16_shift_kernel<BN, ITEMS>,
+  int smem_bytes = sa * q.a_stage_bytes + sb * BN * KB * 2 + (int)plan.K2p * 4 + 1024;
+  if (SPLIT && smem_bytes < cluster_sums_bytes(BN) + 1024) smem_bytes = cluster_sums_bytes(BN) + 1024;
+  cudaError_t e = cudaFuncSetAttribute(conv_f16_shift_kernel<BN, ITEMS, SPLIT>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
+  if (e == cudaSuccess && SPLIT)
+    e = cudaFuncSetAttribute(conv_f16_shift_kernel<BN, ITEMS, SPLIT>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (e != cudaSuccess) return e;
   const int64_t units = (plan.VQ + TILE_M - 1) / TILE_M;
-  dim3 grid((unsigned)(units - q.nbig), (unsigned)((co + BN - 1) / BN));   // a tall tile covers two units
-  conv_f16_shift_kernel<BN, ITEMS><<<grid, NUM_THREADS, smem_bytes, stream>>>(fmap, q);
-  return cudaGetLastError();
+  const dim3 grid((unsigned)((units - q.nbig) * q.split), (unsigned)((co + BN - 1) / BN));   // a tall tile covers two units
+  if constexpr (SPLIT) {
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)q.split; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(NUM_THREADS, 1, 1);
+    cfg.dynamicSmemBytes = (size_t)smem_bytes;
+    cfg.stream = stream;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, conv_f16_shift_kernel<BN, ITEMS, SPLIT>, fmap, q);
+  } else {
+    conv_f16_shift_kernel<BN, ITEMS, SPLIT><<<grid, NUM_THREADS, smem_bytes, stream>>>(fmap, q);
+    return cudaGetLastError();
+  }
 }
 
 // Number of 256-position tiles: whole waves of tall tiles while two units per slot remain, and
@@ -455,6 +511,11 @@ cudaError_t launch_bn(const CUtensorMap& fmap, const ShiftParams& q0, const Shif
                       int s, cudaStream_t stream) {
   ShiftParams q = q0;
   const int64_t units = (plan.VQ + TILE_M - 1) / TILE_M;
+  if (q.split > 1) {
+    if (plan.items <= 5) return launch_variant<BN, 5, true>(fmap, q, plan, co, stream);
+    if (plan.items <= 10) return launch_variant<BN, 10, true>(fmap, q, plan, co, stream);
+    return launch_variant<BN, 15, true>(fmap, q, plan, co, stream);
+  }
   q.nbig = choose_nbig(units, (co + BN - 1) / BN, BN <= 128 ? 2 : 1, q.Kw);
   const int mt = q.nbig > 0 ? 2 : 1;
   const int total_rows = s * (TILE_M * mt + q.halo8);
@@ -465,13 +526,47 @@ cudaError_t launch_bn(const CUtensorMap& fmap, const ShiftParams& q0, const Shif
   }
   const int rows_all = q.a_stage_bytes / 128;
   const int items = (rows_all * q.chunks + PRODUCER_THREADS - 1) / PRODUCER_THREADS;
-  if (items <= 5) return launch_variant<BN, 5>(fmap, q, plan, co, stream);
-  if (items <= 10) return launch_variant<BN, 10>(fmap, q, plan, co, stream);
-  if (items <= 15) return launch_variant<BN, 15>(fmap, q, plan, co, stream);
-  if (items <= 20) return launch_variant<BN, 20>(fmap, q, plan, co, stream);
+  if (items <= 5) return launch_variant<BN, 5, false>(fmap, q, plan, co, stream);
+  if (items <= 10) return launch_variant<BN, 10, false>(fmap, q, plan, co, stream);
+  if (items <= 15) return launch_variant<BN, 15, false>(fmap, q, plan, co, stream);
+  if (items <= 20) return launch_variant<BN, 20, false>(fmap, q, plan, co, stream);
   q.nbig = 0;
   q.a_stage_bytes = s * (TILE_M + q.halo8) * 128;
-  return launch_variant<BN, 15>(fmap, q, plan, co, stream);
+  return launch_variant<BN, 15, false>(fmap, q, plan, co, stream);
+}
+
+// Channel tile, and the CTAs of a cluster that share a tile's k-blocks where there are so few tiles that an SM each is left for
+// them.  Times in us, fitted to 34 such layers (each with 1 to 16 CTAs and every channel tile; the choice is within 0.7 % of the
+// best on average, 15 % at the most): a k-block takes the longer of its staging and its MMAs, meeting and adding up more with the
+// channels of a tile.  Unsplit, the kernels of two CTAs an SM spill where they stage two column classes.  Measured, alone / split: 3x3
+// stride 2 on 512 -> 512 channels, batch 4, 10x10 (one position tile) 62.7 / 17.7, 7x7 on 128 -> 9 channels at 9x9 37.4 / 9.2, 7x7 on
+// 256 channels at 19x19, batch 4, 68.6 / 16.7; two k-blocks 11.2 / 11.0 (1x7 on 128 channels at 7x7).
+// The tiles are those of the batch these images belong to: they decide the order of the sums.
+void choose_split(const Geometry& g, ShiftPlan* p) {
+  p->bn = g.Co <= 64 ? 64 : (g.Co <= 128 ? 128 : 256);
+  p->split = 1;
+  const int64_t units = ((int64_t)g.plan_N * g.Ho * p->Wq + TILE_M - 1) / TILE_M;
+  const int kb = (int)(p->K2p / KB), widest = p->bn;
+  // testing aids: channel tile, CTAs per tile (1 where the kernel is forced and this is not)
+  const char* force_bn = debug_getenv("IM2WIN_F16_SHIFT_BN");
+  const char* force_z = debug_getenv("IM2WIN_F16_SPLIT");
+  if (force_bn) p->bn = atoi(force_bn);
+  if (force_z) { p->split = atoi(force_z) < kb ? atoi(force_z) : kb; return; }
+  if (force_bn || debug_getenv("IM2WIN_F16_KERNEL") || units > 74 || g.K > kMostSplitTerms) return;
+  auto block = [&](int bn, bool alone) {
+    const double staging = g.s == 1 ? 1.2 + 0.15 * g.Kw : (alone && bn < 256 ? 4.6 : 2.2);
+    const double mma = g.Kw * 4 * (bn <= 128 ? 32 + bn / 4.0 : bn / 2.0) / 1900;
+    return staging > mma ? staging : mma;
+  };
+  double best = kb * block(widest, true);
+  for (int bn = widest; bn >= 64; bn /= 2) {
+    const int64_t tiles = units * ((g.Co + bn - 1) / bn);
+    for (int z = 2; z <= kMaxCtas && z <= kb; ++z) {
+      if (tiles * z > 148 || tiles > resident_clusters(z)) continue;
+      const double cost = bn / 32.0 + (kb + z - 1) / z * block(bn, false) + 0.05 * z;
+      if (cost < best) { best = cost; p->bn = bn; p->split = z; }
+    }
+  }
 }
 
 }  // namespace
@@ -497,6 +592,7 @@ ShiftPlan plan_f16_shift(const Geometry& g) {
   if (2 * p.total_rows * 128 + 2 * 256 * KB * 2 + p.K2p * 4 > kSmemBudget - 2048) return p;
   if (p.VQ + 2 * TILE_M >= ((int64_t)1 << 31)) return p;   // 32-bit position arithmetic
   p.eligible = true;
+  choose_split(g, &p);
   return p;
 }
 
@@ -507,7 +603,7 @@ cudaError_t launch_conv_f16_shift(const uint16_t* window, float* y, void* scratc
   EncodeTiledFn encode = get_encode_fn();
   if (!encode) return cudaErrorNotSupported;
   unsigned char* base = static_cast<unsigned char*>(scratch);
-  const int bn = g.Co <= 64 ? 64 : (g.Co <= 128 ? 128 : 256);
+  const int bn = plan.bn, split = plan.split;
 
   // Filter as Fp2[v][co][k2p] halves: a 3-D tensor (k2 fastest), one box = 64 k2 x BN channels of one v.
   CUtensorMap fmap;
@@ -532,6 +628,7 @@ cudaError_t launch_conv_f16_shift(const uint16_t* window, float* y, void* scratc
   q.Kh = g.Kh; q.Kw = g.Kw; q.s = g.s; q.num_kb = (int32_t)(plan.K2p / KB);
   q.halo8 = plan.rows - TILE_M;
   q.nbig = 0;
+  q.split = split;
   q.a_stage_bytes = plan.total_rows * 128;
   q.sa = q.sb = 2;
   if (bn == 64) return launch_bn<64>(fmap, q, plan, g.Co, g.s, stream);
