@@ -62,7 +62,11 @@ struct EpiParams {
   int32_t relu, out16, y_nhwc, atomic;
   int32_t Ho, Wo, Co, HoWo;
   int32_t rows_total;        // N*Ho strips
+  uint32_t stage_off;        // rows that are stored through shared memory (see store_rows): place of the buffers behind the rings, or 0
 };
+
+constexpr int ROW_PITCH = 68;                  // bytes of a row in a warp's buffer: 16 words and one more (no bank conflicts)
+constexpr int kStageBytes = EPI_WARPS * 32 * ROW_PITCH;
 
 struct NhwcParams {
   EpiParams e;
@@ -111,10 +115,10 @@ __device__ __forceinline__ void store_chunk(const EpiParams& q, int64_t base, in
     float* p = reinterpret_cast<float*>(q.y) + base;
     if (!q.y_nhwc) {
       store_strided32(p, cs, v, cnt);
-    } else if (vec_ok && cnt == 32) {
+    } else if (vec_ok) {                                     // (then cnt is a multiple of four)
 #pragma unroll
       for (int j = 0; j < 32; j += 4)
-        *reinterpret_cast<uint4*>(p + j) = make_uint4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+        if (j < cnt) *reinterpret_cast<uint4*>(p + j) = make_uint4(v[j], v[j + 1], v[j + 2], v[j + 3]);
     } else {
 #pragma unroll
       for (int j = 0; j < 32; ++j)
@@ -132,9 +136,10 @@ __device__ __forceinline__ void store_chunk(const EpiParams& q, int64_t base, in
         if (j + 1 < cnt) *p1 = __float2half_rn(__uint_as_float(v[j + 1]));
         p0 += step; p1 += step;
       }
-    } else if (vec_ok && cnt == 32) {
+    } else if (vec_ok) {
 #pragma unroll
       for (int j = 0; j < 32; j += 8) {
+        if (j >= cnt) break;
         uint32_t w[4];
 #pragma unroll
         for (int t = 0; t < 4; ++t) {
@@ -151,9 +156,97 @@ __device__ __forceinline__ void store_chunk(const EpiParams& q, int64_t base, in
   }
 }
 
+// Channel-innermost rows of channels that are no whole number of 16-byte vectors: a warp's rows go through a buffer in shared memory
+// and leave with the lanes along a row's channels, 16 words of a row at a time.  Stored from the registers, an element at a time, every
+// instruction touches 32 rows: 32 sectors, all of them partly.  (3x3 on 8 -> 163 channels at 132x132, batch 64, binary16 rows: 1700 us,
+// 248 now; fp32 rows of 422, 3x3 on 64 channels at 37x37, batch 128, 560 -> 140.  A kernel of its own: taken at run time it cost the
+// smallest layers without such rows 2 to 7 %.)  The valid rows of a warp are consecutive positions (unless its tile is a part of strips: element by element then), so
+// that a lane's places in the buffer and in the output move by constant steps.
+// A row's words go to 4, 8 or 16 lanes, as many as they are, so that an instruction takes 8, 4 or 2 rows.  `at`, `from`: this lane's word of
+// its first row, in the output and the buffer; kind: 0 a word, 1 its lower half only, 2 nothing of it is of the row.
+struct RowLanes {
+  int log, col, first;                                       // lanes of a row, this lane's word, its first row
+  __device__ __forceinline__ RowLanes(int words) {
+    const int lane = threadIdx.x & 31;
+    log = words <= 4 ? 2 : (words <= 8 ? 3 : 4);
+    col = lane & ((1 << log) - 1);
+    first = lane >> log;
+  }
+};
+__device__ __forceinline__ void flush_rows(const RowLanes& l, unsigned char* at, int64_t row_bytes, uint32_t from, int rows, int kind) {
+  const int step = 32 >> l.log;
+#pragma unroll
+  for (int i0 = 0; i0 < 16; i0 += 4) {
+    if (i0 >= 1 << l.log) break;
+    uint32_t v[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v[i]) : "r"(from + (uint32_t)((i0 + i) * step * ROW_PITCH)));
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int r = (i0 + i) * step;
+      unsigned char* p = at + r * row_bytes;
+      const bool live = l.first + r < rows;
+      if (live && kind == 0) *reinterpret_cast<uint32_t*>(p) = v[i];
+      if (live && kind == 1) *reinterpret_cast<uint16_t*>(p) = (uint16_t)v[i];
+    }
+  }
+  __syncwarp();                                              // (the buffer is free again)
+}
+// `base`: element index of this lane's first of cnt <= 32 channels.
+__device__ __forceinline__ void store_rows(const EpiParams& e, int64_t base, const uint32_t (&v)[32], int cnt, bool valid, uint32_t buf) {
+  const int lane = threadIdx.x & 31;
+  const uint32_t mask = __ballot_sync(0xffffffffu, valid);
+  const int slot = __popc(mask & ((1u << lane) - 1u)), rows = __popc(mask);
+  const int64_t base0 = __shfl_sync(0xffffffffu, base, mask ? __ffs(mask) - 1 : 0);
+  if (!__all_sync(0xffffffffu, !valid || base == base0 + (int64_t)slot * e.Co)) {
+    if (valid) store_chunk(e, base, 1, v, cnt, false);
+    return;
+  }
+  const uint32_t mine = buf + slot * ROW_PITCH;
+  if (e.out16) {
+    // A row that starts on an odd half lies one half further on in the buffer, so that words of both have the same elements; its
+    // first element, and the last where 32 do not fit its 16 words, leave from the registers.
+    __half* y = reinterpret_cast<__half*>(e.y);
+    const bool odd = (base & 1) != 0;
+    if (valid) {
+#pragma unroll
+      for (int j = 0; j < 16; ++j) {
+        const float lo = __uint_as_float(odd ? v[j ? 2 * j - 1 : 0] : v[2 * j]), hi = __uint_as_float(odd ? v[2 * j] : v[2 * j + 1]);
+        const __half2 h = __floats2half2_rn(lo, hi);
+        asm volatile("st.shared.u32 [%0], %1;" ::"r"(mine + 4 * j), "r"(*reinterpret_cast<const uint32_t*>(&h)) : "memory");
+      }
+      if (odd) y[base] = __float2half_rn(__uint_as_float(v[0]));
+      if (odd && cnt == 32) y[base + 31] = __float2half_rn(__uint_as_float(v[31]));
+    }
+    __syncwarp();
+    const RowLanes l((e.Co & 1) ? cnt / 2 + 1 : (cnt + 1) / 2);
+    const int64_t b = base0 + (int64_t)l.first * e.Co;       // (the parity of this lane's rows is the same: they are an even number apart)
+    const int at = 2 * l.col - (int)(b & 1);
+    const int kind = at < 0 || at >= cnt ? 2 : (at + 1 < cnt ? 0 : 1);
+    flush_rows(l, reinterpret_cast<unsigned char*>(y + b + at), 2 * (int64_t)e.Co, buf + l.first * ROW_PITCH + 4 * l.col, rows, kind);
+  } else {
+#pragma unroll
+    for (int h = 0; h < 32; h += 16) {
+      if (h >= cnt) break;
+      if (valid) {
+#pragma unroll
+        for (int j = 0; j < 16; ++j)
+          asm volatile("st.shared.u32 [%0], %1;" ::"r"(mine + 4 * j), "r"(v[h + j]) : "memory");
+      }
+      __syncwarp();
+      const RowLanes l(cnt - h);
+      const int64_t b = base0 + (int64_t)l.first * e.Co + h + l.col;
+      flush_rows(l, reinterpret_cast<unsigned char*>(reinterpret_cast<float*>(e.y) + b), 4 * (int64_t)e.Co,
+                 buf + l.first * ROW_PITCH + 4 * l.col, rows, h + l.col < cnt ? 0 : 2);
+    }
+  }
+}
+
 // Bias (first K part only), ReLU and store of 32 channels from c0 on of one accumulator row.
+template <bool ROWS>
 __device__ __forceinline__ void finish_chunk(const EpiParams& e, uint32_t (&v)[32], int c0, int n0, bool first_part,
-                                             bool valid, int64_t base, int64_t cs, bool vec_ok, bool add = false,
+                                             bool valid, int64_t base, int64_t cs, bool vec_ok, uint32_t stage, bool add = false,
                                              const float* bias_regs = nullptr) {
   const int cnt = e.Co - n0 - c0;                // channels left from c0 on
   if (cnt <= 0) return;
@@ -186,6 +279,10 @@ __device__ __forceinline__ void finish_chunk(const EpiParams& e, uint32_t (&v)[3
 #pragma unroll
     for (int t = 0; t < 32; ++t) v[t] = __float_as_uint(fmaxf(__uint_as_float(v[t]), 0.0f));
   }
+  if (ROWS && !add) {
+    store_rows(e, base + c0, v, cnt < 32 ? cnt : 32, valid, stage);
+    return;
+  }
   if (valid) store_chunk(e, base + (int64_t)c0 * cs, cs, v, cnt < 32 ? cnt : 32, vec_ok, add);
 }
 
@@ -207,9 +304,10 @@ __device__ __forceinline__ bool hoist_bias(const EpiParams& e, int ntn, int warp
 // bias, ReLU, store.  The tensor-memory load of the next 32 channels is in flight while the current
 // ones are stored (two register sets, taken in turn).  `base` is the element index of the tile's first
 // channel at this lane's position, `cs` the element distance between channels.
+template <bool ROWS>
 __device__ __forceinline__ void drain_accumulator(const EpiParams& e, int cols, int warp, int lane, uint32_t lane_base,
                                                   bool valid, int64_t base, int64_t cs, int n0, bool first_part, bool vec_ok,
-                                                  bool add = false, const float* bias_regs = nullptr) {
+                                                  uint32_t stage, bool add = false, const float* bias_regs = nullptr) {
   const int CH = cols / 2;                       // a multiple of 32
   const int cbeg = ((warp - WARP_EPI0) >> 2) * CH;
   const int cend = cbeg + CH;
@@ -219,11 +317,11 @@ __device__ __forceinline__ void drain_accumulator(const EpiParams& e, int cols, 
   for (int c0 = cbeg; c0 < cend; c0 += 64) {
     tmem_ld_wait_for(va);
     if (c0 + 32 < cend) tmem_ld32_issue(lane_base + (uint32_t)(c0 + 32), vb);
-    finish_chunk(e, va, c0, n0, first_part, valid, base, cs, vec_ok, add, bias_regs);
+    finish_chunk<ROWS>(e, va, c0, n0, first_part, valid, base, cs, vec_ok, stage, add, bias_regs);
     if (c0 + 32 >= cend) break;
     tmem_ld_wait_for(vb);
     if (c0 + 64 < cend) tmem_ld32_issue(lane_base + (uint32_t)(c0 + 64), va);
-    finish_chunk(e, vb, c0 + 32, n0, first_part, valid, base, cs, vec_ok, add);
+    finish_chunk<ROWS>(e, vb, c0 + 32, n0, first_part, valid, base, cs, vec_ok, stage, add);
   }
 }
 
@@ -310,8 +408,9 @@ __device__ __forceinline__ void dump_partial(int cols, int warp, int lane, uint3
 
 // The owner's drain of a tile whose reduction other CTAs shared: accumulator + `count` partial tiles
 // (`stride` floats apart from slot0 on), then bias, ReLU and store as for any tile.
+template <bool ROWS>
 __device__ __forceinline__ void drain_with_partials(const EpiParams& e, int cols, int warp, int lane, uint32_t lane_base,
-                                                    bool valid, int64_t base, int64_t cs, int n0, bool vec_ok,
+                                                    bool valid, int64_t base, int64_t cs, int n0, bool vec_ok, uint32_t stage,
                                                     const float* slot0, size_t stride, int count) {
   const int CH = cols / 2;
   const int cbeg = ((warp - WARP_EPI0) >> 2) * CH;
@@ -334,7 +433,7 @@ __device__ __forceinline__ void drain_with_partials(const EpiParams& e, int cols
         v[4 * j + 3] = __float_as_uint(__uint_as_float(v[4 * j + 3]) + a.w);
       }
     }
-    finish_chunk(e, v, c0, n0, true, valid, base, cs, vec_ok);
+    finish_chunk<ROWS>(e, v, c0, n0, true, valid, base, cs, vec_ok, stage);
   }
 }
 
@@ -357,7 +456,7 @@ __device__ __forceinline__ void decode_item(const NhwcParams& q, int w, int* who
   else { const int t = w - q.n_main; *whole = q.n_main + (t >> 1); *half = t & 1; }
 }
 
-template <int BN, bool PAIR, int KSUB>
+template <int BN, bool PAIR, int KSUB, bool ROWS>
 __device__ __forceinline__ void conv_nhwc_body(const CUtensorMap& amap, const CUtensorMap& bmap, const CUtensorMap& bmap_h,
                                                const NhwcParams& q) {
   constexpr int B_ROWS = PAIR ? BN / 2 : BN;              // filter rows (output channels) this CTA stages
@@ -539,6 +638,7 @@ __device__ __forceinline__ void conv_nhwc_body(const CUtensorMap& amap, const CU
     const int lq = warp & 3;                     // tensor-memory lane quadrant this warp may read
     const EpiParams& e = q.e;
     const bool vec_ok = e.out16 ? (e.Co % 8 == 0) : (e.Co % 4 == 0);
+    const uint32_t stage = ROWS ? smem_u32(smem) + e.stage_off + (warp - WARP_EPI0) * (32 * ROW_PITCH) : 0u;
     wait_for_previous_kernel();                  // before the first store to y
     float breg[32];
     const bool hoisted = hoist_bias<BN>(e, q.ntn, warp, breg);
@@ -588,7 +688,7 @@ __device__ __forceinline__ void conv_nhwc_body(const CUtensorMap& amap, const CU
       tc_fence_after();
       const uint32_t lane_base = tmem_acc + buf * (uint32_t)BN + ((uint32_t)(lq * 32) << 16);
       if (BN < 128 || frag == 0) {
-        drain_accumulator(e, cols, warp, lane, lane_base, valid, base, cs, n0, ks == 0, vec_ok, false, hoisted ? breg : nullptr);
+        drain_accumulator<ROWS>(e, cols, warp, lane, lane_base, valid, base, cs, n0, ks == 0, vec_ok, stage, false, hoisted ? breg : nullptr);
       } else {
         constexpr int PER = PAIR ? 2 : 1;                    // slots and flag words per CTA (pair) of the grid
         constexpr size_t SLOT = (size_t)BN * TILE_M;         // floats of one CTA's partial tile
@@ -608,7 +708,7 @@ __device__ __forceinline__ void conv_nhwc_body(const CUtensorMap& amap, const CU
           __syncwarp();
           if (threadIdx.x == WARP_EPI0 * 32) TIMER_LAP(8);   // epilogue: wait for the other CTAs' partial sums
           if (ok)
-            drain_with_partials(e, cols, warp, lane, lane_base, valid, base, cs, n0, vec_ok,
+            drain_with_partials<ROWS>(e, cols, warp, lane, lane_base, valid, base, cs, n0, vec_ok, stage,
                                 q.partial + (size_t)(PER * (w_first + 1) + (int)rank) * SLOT, PER * SLOT, count);
         }
       }
@@ -640,18 +740,18 @@ __device__ __forceinline__ void conv_nhwc_body(const CUtensorMap& amap, const CU
   }
 }
 
-template <int BN, int KSUB>
+template <int BN, int KSUB, bool ROWS>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
 conv_f16_nhwc_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ CUtensorMap bmap,
                      const __grid_constant__ CUtensorMap bmap_h, NhwcParams q) {
-  conv_nhwc_body<BN, false, KSUB>(amap, bmap, bmap_h, q);
+  conv_nhwc_body<BN, false, KSUB, ROWS>(amap, bmap, bmap_h, q);
 }
 
-template <int BN, int KSUB>
+template <int BN, int KSUB, bool ROWS>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
 conv_f16_nhwc_pair_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ CUtensorMap bmap,
                           const __grid_constant__ CUtensorMap bmap_h, NhwcParams q) {
-  conv_nhwc_body<BN, true, KSUB>(amap, bmap, bmap_h, q);
+  conv_nhwc_body<BN, true, KSUB, ROWS>(amap, bmap, bmap_h, q);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -735,7 +835,7 @@ __device__ __forceinline__ void issue_k2_block(uint32_t acc, uint32_t a_stage, u
 // TAIL: the launch has items that are parts of a tile (a short last round, see decode_shift_item); without
 // them every item is a whole tile and the part handling drops out of the code (layers with very short
 // items, a 3x3 stem has six MMAs per item, pay for every instruction in the per-item paths).
-template <int BN, bool PAIR, bool TAIL, bool HOIST>
+template <int BN, bool PAIR, bool TAIL, bool HOIST, bool ROWS>
 __device__ __forceinline__ void conv_shift_body(const CUtensorMap& amap, const CUtensorMap& bmap, const CUtensorMap& bmap_h,
                                                 const CUtensorMap& bmap_q, const ShiftViewParams& q) {
   constexpr int B_ROWS = PAIR ? BN / 2 : BN;
@@ -1050,6 +1150,7 @@ __device__ __forceinline__ void conv_shift_body(const CUtensorMap& amap, const C
     const int lq = warp & 3;
     const EpiParams& e = q.e;
     const bool vec_ok = e.out16 ? (e.Co % 8 == 0) : (e.Co % 4 == 0);
+    const uint32_t stage = ROWS ? smem_u32(smem) + e.stage_off + (warp - WARP_EPI0) * (32 * ROW_PITCH) : 0u;
     wait_for_previous_kernel();
     // HOIST (64-channel tiles, one channel tile, a bias): the warp's 32 bias values stay in registers.  A
     // kernel of its own: the same choice taken at run time cost the stems without a bias 8-15 %.
@@ -1103,7 +1204,7 @@ __device__ __forceinline__ void conv_shift_body(const CUtensorMap& amap, const C
         ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
         __syncwarp();
       }
-      if (ok) drain_accumulator(e, cols, warp, lane, lane_base, valid, base, cs, n0, kpart ? part == 0 : ks == 0, vec_ok, adds,
+      if (ok) drain_accumulator<ROWS>(e, cols, warp, lane, lane_base, valid, base, cs, n0, kpart ? part == 0 : ks == 0, vec_ok, stage, adds,
                                 HOIST ? breg : nullptr);
       if (kpart && part == 0) {
         publish_when_all_stored(epi_bar, epi_phase, warp, lane, flag, q.epoch, &abort_flag, q.status);
@@ -1135,20 +1236,20 @@ __device__ __forceinline__ void conv_shift_body(const CUtensorMap& amap, const C
   }
 }
 
-template <int BN, bool TAIL, bool HOIST>
+template <int BN, bool TAIL, bool HOIST, bool ROWS>
 __global__ void __launch_bounds__(SHIFT_THREADS, 1)
 conv_f16_nhwc_shift_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ CUtensorMap bmap,
                            const __grid_constant__ CUtensorMap bmap_h, const __grid_constant__ CUtensorMap bmap_q,
                            ShiftViewParams q) {
-  conv_shift_body<BN, false, TAIL, HOIST>(amap, bmap, bmap_h, bmap_q, q);
+  conv_shift_body<BN, false, TAIL, HOIST, ROWS>(amap, bmap, bmap_h, bmap_q, q);
 }
 
-template <int BN, bool TAIL, bool HOIST>
+template <int BN, bool TAIL, bool HOIST, bool ROWS>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(SHIFT_THREADS, 1)
 conv_f16_nhwc_shift_pair_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ CUtensorMap bmap,
                                 const __grid_constant__ CUtensorMap bmap_h, const __grid_constant__ CUtensorMap bmap_q,
                                 ShiftViewParams q) {
-  conv_shift_body<BN, true, TAIL, HOIST>(amap, bmap, bmap_h, bmap_q, q);
+  conv_shift_body<BN, true, TAIL, HOIST, ROWS>(amap, bmap, bmap_h, bmap_q, q);
 }
 
 // Filter pack (paper Section "Im2win Convolution": height before width; here with the channel below
@@ -1642,12 +1743,16 @@ RunPlan plan_runs(int64_t nwork, int slots, int num_kc, int ksub, int bn) {
   return r;
 }
 
-template <int BN, bool PAIR, int KSUB>
+// Whether a layer's rows are stored through shared memory: channel-innermost ones that are no whole number of 16-byte vectors.
+bool stages_rows(const EpiParams& e) { return e.y_nhwc && !e.atomic && e.Co % (e.out16 ? 8 : 4) != 0; }
+
+template <int BN, bool PAIR, int KSUB, bool ROWS>
 cudaError_t launch_variant(const CUtensorMap& amap, const CUtensorMap& bmap, const CUtensorMap& bmap_h, NhwcParams q,
                            const NhwcPlan& plan, cudaStream_t stream) {
   constexpr int B_ROWS = PAIR ? BN / 2 : BN;
   constexpr int STAGE = KSUB * (A_SLOT_BYTES + B_ROWS * KB * 2);
-  int stages = (kSmemMax - 2048) / STAGE;
+  constexpr int row_buffers = ROWS ? kStageBytes : 0;
+  int stages = (kSmemMax - 2048 - row_buffers) / STAGE;
   if (stages > MAX_STAGES) stages = MAX_STAGES;
   if (stages < 2) return cudaErrorInvalidValue;
   if (const char* v = debug_getenv("IM2WIN_NHWC_STAGES")) { const int n = atoi(v); if (n >= 2 && n < stages) stages = n; }   // ablation: ring depth
@@ -1666,7 +1771,8 @@ cudaError_t launch_variant(const CUtensorMap& amap, const CUtensorMap& bmap, con
   q.nwork = (int32_t)nwork;
   q.n_main = q.nwork;
   int slots = PAIR ? 74 : 148;
-  const int smem_bytes = stages * STAGE + 1024;
+  const int smem_bytes = stages * STAGE + 1024 + row_buffers;
+  q.e.stage_off = (uint32_t)(stages * STAGE);
   // per device and kernel variant, done once: the shared-memory opt-in and the number of CTA pairs
   // that can be resident together (both are host-side queries that would otherwise sit between the
   // filter pack and this launch on every call)
@@ -1682,7 +1788,7 @@ cudaError_t launch_variant(const CUtensorMap& amap, const CUtensorMap& bmap, con
   if (PAIR) {
     cudaError_t e = cudaSuccess;
     if (!attr_done[dev]) {
-      e = cudaFuncSetAttribute(conv_f16_nhwc_pair_kernel<BN, KSUB>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
+      e = cudaFuncSetAttribute(conv_f16_nhwc_pair_kernel<BN, KSUB, ROWS>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax - 1024);
       if (e != cudaSuccess) return e;
       attr_done[dev] = true;
     }
@@ -1695,14 +1801,14 @@ cudaError_t launch_variant(const CUtensorMap& amap, const CUtensorMap& bmap, con
     cfg.numAttrs = 1;
     int clusters = cached_clusters[dev];        // as many pairs as can be resident at once
     if (clusters == 0) {
-      e = cudaOccupancyMaxActiveClusters(&clusters, conv_f16_nhwc_pair_kernel<BN, KSUB>, &cfg);
+      e = cudaOccupancyMaxActiveClusters(&clusters, conv_f16_nhwc_pair_kernel<BN, KSUB, ROWS>, &cfg);
       if (e != cudaSuccess) return e;
       if (clusters < 1) return cudaErrorInvalidValue;
       cached_clusters[dev] = clusters;
     }
     if (clusters < slots) slots = clusters;
   } else if (!attr_done[dev]) {
-    cudaError_t e = cudaFuncSetAttribute(conv_f16_nhwc_kernel<BN, KSUB>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
+    cudaError_t e = cudaFuncSetAttribute(conv_f16_nhwc_kernel<BN, KSUB, ROWS>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax - 1024);
     if (e != cudaSuccess) return e;
     attr_done[dev] = true;
   }
@@ -1730,27 +1836,27 @@ cudaError_t launch_variant(const CUtensorMap& amap, const CUtensorMap& bmap, con
   if (PAIR) {
     cfg.gridDim = dim3(2 * ctas, 1, 1);
     cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, conv_f16_nhwc_pair_kernel<BN, KSUB>, amap, bmap, bmap_h, q);
+    return cudaLaunchKernelEx(&cfg, conv_f16_nhwc_pair_kernel<BN, KSUB, ROWS>, amap, bmap, bmap_h, q);
   }
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   cfg.gridDim = dim3((unsigned)ctas, 1, 1);
-  return cudaLaunchKernelEx(&cfg, conv_f16_nhwc_kernel<BN, KSUB>, amap, bmap, bmap_h, q);
+  return cudaLaunchKernelEx(&cfg, conv_f16_nhwc_kernel<BN, KSUB, ROWS>, amap, bmap, bmap_h, q);
 }
 
-template <int KSUB>
+template <int KSUB, bool ROWS>
 cudaError_t launch_ksub(const CUtensorMap& amap, const CUtensorMap& bmap, const CUtensorMap& bmap_h, const NhwcParams& q,
                         const NhwcPlan& plan, cudaStream_t stream) {
   if (plan.pair) {
-    if (plan.bn == 256) return launch_variant<256, true, KSUB>(amap, bmap, bmap_h, q, plan, stream);
-    if (plan.bn == 128) return launch_variant<128, true, KSUB>(amap, bmap, bmap_h, q, plan, stream);
-    return launch_variant<64, true, KSUB>(amap, bmap, bmap_h, q, plan, stream);
+    if (plan.bn == 256) return launch_variant<256, true, KSUB, ROWS>(amap, bmap, bmap_h, q, plan, stream);
+    if (plan.bn == 128) return launch_variant<128, true, KSUB, ROWS>(amap, bmap, bmap_h, q, plan, stream);
+    return launch_variant<64, true, KSUB, ROWS>(amap, bmap, bmap_h, q, plan, stream);
   }
-  if (plan.bn == 64) return launch_variant<64, false, KSUB>(amap, bmap, bmap_h, q, plan, stream);
-  if (plan.bn == 128) return launch_variant<128, false, KSUB>(amap, bmap, bmap_h, q, plan, stream);
-  return launch_variant<256, false, KSUB>(amap, bmap, bmap_h, q, plan, stream);
+  if (plan.bn == 64) return launch_variant<64, false, KSUB, ROWS>(amap, bmap, bmap_h, q, plan, stream);
+  if (plan.bn == 128) return launch_variant<128, false, KSUB, ROWS>(amap, bmap, bmap_h, q, plan, stream);
+  return launch_variant<256, false, KSUB, ROWS>(amap, bmap, bmap_h, q, plan, stream);
 }
 
 // Geometry of the shifted-view kernel for a layer (host side).
@@ -1783,13 +1889,14 @@ ShiftViewPlan plan_shift_view(const Geometry& g, const NhwcPlan& plan) {
   return p;
 }
 
-template <int BN, bool PAIR>
+template <int BN, bool PAIR, bool ROWS>
 cudaError_t launch_shift_variant(const CUtensorMap& amap, const CUtensorMap& bmap, const CUtensorMap& bmap_h,
                                  const CUtensorMap& bmap_q, ShiftViewParams q, const NhwcPlan& plan,
                                  const ShiftViewPlan& sp, cudaStream_t stream) {
   constexpr int B_ROWS = PAIR ? BN / 2 : BN;
   constexpr int B_BYTES = B_ROWS * KB * 2;
-  const int budget = kSmemMax - 2048;
+  constexpr int row_buffers = ROWS ? kStageBytes : 0;
+  const int budget = kSmemMax - 2048 - row_buffers;
   // units per filter stage: all kernel columns of a k2-block when two such stages fit beside two
   // activation stages (the MMA warp then pays two waits and two commits per block); otherwise three,
   // or fewer when three stages of that size do not fit (wide tiles without pairing)
@@ -1829,7 +1936,8 @@ cudaError_t launch_shift_variant(const CUtensorMap& amap, const CUtensorMap& bma
   // and items of 24 MMAs or more (a 3x3 stem, six MMAs per item and bound by its output stores, lost a third)
   q.dual = (q.resident && q.bu == q.Kw && q.sa / 2 >= sp.nkb2 && q.nwork >= 2 && sp.nkb2 * q.Kw * (KB / 16) >= 24) ? 1 : 0;
   if (const char* v = debug_getenv("IM2WIN_NHWC_DUAL")) q.dual = (q.dual && v[0] != '0') ? 1 : 0;
-  const int smem_bytes = q.sa * (int)sp.a_stage_bytes + q.sb * b_stage + 1024;
+  const int smem_bytes = q.sa * (int)sp.a_stage_bytes + q.sb * b_stage + 1024 + row_buffers;
+  q.e.stage_off = (uint32_t)(q.sa * (int)sp.a_stage_bytes + q.sb * b_stage);
   static int cached_clusters[64] = {};
   static int attr_bytes[64] = {};
   int dev = 0;
@@ -1842,10 +1950,10 @@ cudaError_t launch_shift_variant(const CUtensorMap& amap, const CUtensorMap& bma
   using Kernel = void (*)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, ShiftViewParams);
   constexpr bool CAN_HOIST = BN == 64;
   const Kernel variants[2][2] = {
-      {PAIR ? (Kernel)conv_f16_nhwc_shift_pair_kernel<BN, false, false> : (Kernel)conv_f16_nhwc_shift_kernel<BN, false, false>,
-       PAIR ? (Kernel)conv_f16_nhwc_shift_pair_kernel<BN, false, CAN_HOIST> : (Kernel)conv_f16_nhwc_shift_kernel<BN, false, CAN_HOIST>},
-      {PAIR ? (Kernel)conv_f16_nhwc_shift_pair_kernel<BN, true, false> : (Kernel)conv_f16_nhwc_shift_kernel<BN, true, false>,
-       PAIR ? (Kernel)conv_f16_nhwc_shift_pair_kernel<BN, true, CAN_HOIST> : (Kernel)conv_f16_nhwc_shift_kernel<BN, true, CAN_HOIST>}};
+      {PAIR ? (Kernel)conv_f16_nhwc_shift_pair_kernel<BN, false, false, ROWS> : (Kernel)conv_f16_nhwc_shift_kernel<BN, false, false, ROWS>,
+       PAIR ? (Kernel)conv_f16_nhwc_shift_pair_kernel<BN, false, CAN_HOIST, ROWS> : (Kernel)conv_f16_nhwc_shift_kernel<BN, false, CAN_HOIST, ROWS>},
+      {PAIR ? (Kernel)conv_f16_nhwc_shift_pair_kernel<BN, true, false, ROWS> : (Kernel)conv_f16_nhwc_shift_kernel<BN, true, false, ROWS>,
+       PAIR ? (Kernel)conv_f16_nhwc_shift_pair_kernel<BN, true, CAN_HOIST, ROWS> : (Kernel)conv_f16_nhwc_shift_kernel<BN, true, CAN_HOIST, ROWS>}};
   const bool hoist = CAN_HOIST && q.e.bias != nullptr && q.ntn == 1;
   if (attr_bytes[dev] < smem_bytes) {
     for (int t = 0; t < 2; ++t)
@@ -1941,6 +2049,19 @@ cudaError_t launch_shift_variant(const CUtensorMap& amap, const CUtensorMap& bma
                 q.tail_log2 > 0 ? "launch (shifted view, parts)" : "launch (shifted view)");
 }
 
+template <bool ROWS>
+cudaError_t launch_shift_tile(const CUtensorMap& amap, const CUtensorMap& bmap, const CUtensorMap& bmap_h, const CUtensorMap& bmap_q,
+                              const ShiftViewParams& q, const NhwcPlan& plan, const ShiftViewPlan& sp, cudaStream_t stream) {
+  if (plan.pair) {
+    if (plan.bn == 256) return launch_shift_variant<256, true, ROWS>(amap, bmap, bmap_h, bmap_q, q, plan, sp, stream);
+    if (plan.bn == 128) return launch_shift_variant<128, true, ROWS>(amap, bmap, bmap_h, bmap_q, q, plan, sp, stream);
+    return launch_shift_variant<64, true, ROWS>(amap, bmap, bmap_h, bmap_q, q, plan, sp, stream);
+  }
+  if (plan.bn == 64) return launch_shift_variant<64, false, ROWS>(amap, bmap, bmap_h, bmap_q, q, plan, sp, stream);
+  if (plan.bn == 128) return launch_shift_variant<128, false, ROWS>(amap, bmap, bmap_h, bmap_q, q, plan, sp, stream);
+  return launch_shift_variant<256, false, ROWS>(amap, bmap, bmap_h, bmap_q, q, plan, sp, stream);
+}
+
 cudaError_t launch_shift_view(const uint16_t* window, const uint16_t* fp, void* y, uint32_t* status, uint32_t* flags,
                               const Geometry& g, const NhwcPlan& plan, const ShiftViewPlan& sp, const EpilogueArgs& epi,
                               bool split, EncodeTiledFn encode, cudaStream_t stream) {
@@ -1985,14 +2106,10 @@ cudaError_t launch_shift_view(const uint16_t* window, const uint16_t* fp, void* 
   q.epoch = next_epoch();
   q.flags = flags;
   if (const char* v = debug_getenv("IM2WIN_NHWC_BU")) { const int bu = atoi(v); if (bu >= 1 && bu <= 8) { q.bu = bu; q.bu_forced = 1; } }
-  if (plan.pair) {
-    if (plan.bn == 256) return launch_shift_variant<256, true>(amap, bmap, bmap_h, bmap_q, q, plan, sp, stream);
-    if (plan.bn == 128) return launch_shift_variant<128, true>(amap, bmap, bmap_h, bmap_q, q, plan, sp, stream);
-    return launch_shift_variant<64, true>(amap, bmap, bmap_h, bmap_q, q, plan, sp, stream);
-  }
-  if (plan.bn == 64) return launch_shift_variant<64, false>(amap, bmap, bmap_h, bmap_q, q, plan, sp, stream);
-  if (plan.bn == 128) return launch_shift_variant<128, false>(amap, bmap, bmap_h, bmap_q, q, plan, sp, stream);
-  return launch_shift_variant<256, false>(amap, bmap, bmap_h, bmap_q, q, plan, sp, stream);
+  // (buffers for rows where two activation stages and two of one filter unit still fit beside them)
+  if (stages_rows(q.e) && 2 * (int64_t)sp.a_stage_bytes + 2 * (int64_t)b_rows * KB * 2 <= kSmemMax - 2048 - kStageBytes)
+    return launch_shift_tile<true>(amap, bmap, bmap_h, bmap_q, q, plan, sp, stream);
+  return launch_shift_tile<false>(amap, bmap, bmap_h, bmap_q, q, plan, sp, stream);
 }
 
 }  // namespace
@@ -2361,8 +2478,9 @@ cudaError_t launch_conv_f16_nhwc(const uint16_t* window, void* y, void* scratch,
   q.flags = reinterpret_cast<uint32_t*>(base + plan.flags_off);
   q.partial = plan.partial_bytes > 0 ? reinterpret_cast<float*>(base + plan.partial_off) : nullptr;
   q.epoch = next_epoch();
-  if (ksub == 1) return launch_ksub<1>(amap, bmap, bmap_h, q, plan, stream);
-  return launch_ksub<2>(amap, bmap, bmap_h, q, plan, stream);
+  if (ksub != 1) return launch_ksub<2, false>(amap, bmap, bmap_h, q, plan, stream);
+  if (stages_rows(q.e)) return launch_ksub<1, true>(amap, bmap, bmap_h, q, plan, stream);
+  return launch_ksub<1, false>(amap, bmap, bmap_h, q, plan, stream);
 }
 
 }  // namespace im2win

@@ -1,0 +1,40 @@
+"""Channel-innermost rows stored through shared memory (channels that are no whole number of 16-byte vectors) and by ragged numbers of
+vectors: rows that start on odd halves, last chunks of 1 to 31 channels, tiles whose strips leave gaps, tiles of parts of strips, a split
+reduction, several channel tiles.  Integer-valued inputs exactly (the result is one fp32 sum, rounded once), guard bands around the output.
+"""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2608_20725_b200 import workloads
+from paper_2608_20725_b200.workloads import Layer
+from gpu_helpers import gpu_conv_nhwc
+
+pytestmark = pytest.mark.gpu
+
+
+def L(name, N, C, H, W, Co, Kh, Kw, s, p, seed):
+    return Layer(name, N, C, H, W, Co, Kh, Kw, s, p, seed, "normal01", "he_normal")
+
+
+@pytest.mark.parametrize("kernel", ["shift", "overlap"])
+@pytest.mark.parametrize("layer", [
+    L("c1", 3, 8, 9, 11, 1, 3, 3, 1, 1, 700), L("c7", 2, 8, 12, 9, 7, 3, 3, 1, 0, 701), L("c9", 2, 16, 10, 10, 9, 1, 1, 1, 0, 702),
+    L("c12", 2, 8, 10, 13, 12, 3, 3, 1, 1, 703), L("c20", 2, 8, 9, 13, 20, 3, 3, 1, 1, 704), L("c33", 2, 16, 7, 7, 33, 3, 3, 1, 1, 705),
+    L("c63", 3, 8, 12, 12, 63, 3, 3, 1, 1, 706), L("c74", 2, 24, 11, 9, 74, 3, 3, 2, 1, 707), L("c95", 2, 8, 8, 31, 95, 3, 3, 1, 1, 708),
+    L("c163", 3, 8, 13, 17, 163, 3, 3, 1, 1, 709), L("c301", 2, 16, 9, 9, 301, 3, 3, 1, 1, 710),
+    L("parts", 1, 8, 4, 201, 37, 3, 3, 1, 1, 711),          # strips wider than a tile
+    L("rounds", 40, 8, 24, 24, 99, 3, 3, 1, 1, 712)], ids=lambda l: l.name)     # more tiles than CTAs
+def test_rows_of_any_number_of_channels(layer, kernel, monkeypatch):
+    monkeypatch.setenv("IM2WIN_NHWC_KERNEL", kernel)
+    dims = layer.dims()
+    x, f = workloads.make_small_integer_inputs(layer)
+    yr, _ = oracle.conv_direct(x.numpy(), f.numpy(), dims)
+    bias = np.arange(layer.Co) % 7 - 3.0
+    want = yr.transpose(0, 2, 3, 1)
+    for out16 in (False, True):
+        assert np.array_equal(gpu_conv_nhwc(x, f, dims, out16=out16, y_nhwc=True), want.astype(np.float16) if out16 else want)
+        got = gpu_conv_nhwc(x, f, dims, bias=bias, relu=True, out16=out16, y_nhwc=True)
+        ref = np.maximum(want + bias, 0.0)
+        assert np.array_equal(got, ref.astype(np.float16) if out16 else ref)
+
