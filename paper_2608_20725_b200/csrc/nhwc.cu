@@ -1363,24 +1363,29 @@ __global__ void transform_nhwc_from_nhwc_kernel(const uint16_t* __restrict__ x, 
   }
 }
 
-// x given NHWC: one block per strip (n, ho).  A thread takes 16-byte chunk i of the padded row (column
+// x given NHWC: 2^lg threads of a block per strip (n, ho), gridDim.y blocks side by side.  A thread takes 16-byte chunk i of the padded row (column
 // k = i / c8n, channels 8 (i % c8n) ..) and copies it from each of the strip's Kh input rows to
 // window[(k*Kh + u)*Cp + ...]: along a row the reads of consecutive threads are contiguous, the Kh loads of a
 // thread are independent, and its Kh stores complete a run of Kh*Cp halves; the only index arithmetic per
 // chunk is the split of i (a shift when Cp/8 is a power of two).  The chunk-per-thread kernel above pays five
 // 64-bit divisions per chunk and reached 0.39-0.54 of the copy rate where this one is used now (C a multiple
 // of 8: 0.65-0.87 on layers of 80 MB and more).
-template <bool POW2>
+// VEC: halves of a load, the largest of 8, 4, 2 and 1 that divides C (a pixel's channels then start on such a boundary; groups beyond C are
+// zeros): 12 channels at 196x150, batch 32, 5x5 69 us a chunk a thread, 39 here; 310 channels at 108x59, batch 4, 24 and 12.  A strip's
+// chunks over several blocks: 11x11 on 256 channels, one 189x189 image, 140 -> 48.
+template <bool POW2, int VEC, bool SIDE>
 __global__ void __launch_bounds__(256)
 transform_nhwc_from_nhwc_strip_kernel(const uint16_t* __restrict__ x, uint4* __restrict__ win, int C, int c8n, int sh,
-                                      int H, int W, int Ho, int Wp, int Kh, int s, int p) {
-  const int strip = blockIdx.x;                  // n*Ho + ho
+                                      int H, int W, int Ho, int Wp, int Kh, int s, int p, int lg_, int strips) {
+  const int lg = SIDE ? lg_ : 8;                 // (a constant where a block has one strip: a run-time one cost 7 to 12 %)
+  const int strip = ((int)blockIdx.x << (8 - lg)) + ((int)threadIdx.x >> lg);      // n*Ho + ho
+  if (strip >= strips) return;
   const int n = strip / Ho, ho = strip - n * Ho;
   uint4* out = win + (int64_t)strip * Wp * Kh * c8n;
   const int row_chunks = Wp * c8n;
   const int h0 = ho * s - p;
   const uint16_t* ximg = x + (int64_t)n * H * W * C;
-  for (int i = threadIdx.x; i < row_chunks; i += 256) {
+  for (int i = ((int)blockIdx.y << lg) + ((int)threadIdx.x & ((1 << lg) - 1)); i < row_chunks; i += (int)gridDim.y << lg) {
     const int k = POW2 ? i >> sh : i / c8n;
     const int c8 = i - k * c8n;
     const int w = k - p;
@@ -1392,7 +1397,26 @@ transform_nhwc_from_nhwc_strip_kernel(const uint16_t* __restrict__ x, uint4* __r
       uint4 v = make_uint4(0u, 0u, 0u, 0u);
       if (colok && h >= 0 && h < H) {
         const uint16_t* src = ximg + ((int64_t)h * W + w) * C + c8 * 8;
-        v = __ldg(reinterpret_cast<const uint4*>(src));
+        if constexpr (VEC == 8) {
+          v = __ldg(reinterpret_cast<const uint4*>(src));
+        } else {
+          const int left = C - c8 * 8;
+          if constexpr (VEC == 4) {
+            const uint2 a = __ldg(reinterpret_cast<const uint2*>(src));
+            const uint2 b = left > 4 ? __ldg(reinterpret_cast<const uint2*>(src) + 1) : make_uint2(0u, 0u);
+            v = make_uint4(a.x, a.y, b.x, b.y);
+          } else if constexpr (VEC == 2) {
+            uint32_t e[4];
+#pragma unroll
+            for (int t = 0; t < 4; ++t) e[t] = 2 * t < left ? __ldg(reinterpret_cast<const uint32_t*>(src) + t) : 0u;
+            v = make_uint4(e[0], e[1], e[2], e[3]);
+          } else {
+            uint32_t e[8];
+#pragma unroll
+            for (int t = 0; t < 8; ++t) e[t] = t < left ? __ldg(src + t) : (uint16_t)0;
+            v = make_uint4(e[0] | (e[1] << 16), e[2] | (e[3] << 16), e[4] | (e[5] << 16), e[6] | (e[7] << 16));
+          }
+        }
       }
       o[u * c8n] = v;
     }
@@ -1403,24 +1427,30 @@ transform_nhwc_from_nhwc_strip_kernel(const uint16_t* __restrict__ x, uint4* __r
 // strip.  The strip's Kh input rows (W*C halves each, contiguous) are staged in shared memory with coalesced
 // 2-byte loads; then thread j builds chunk j = k*Kh + u of the strip from the C halves of pixel (u, k - p)
 // and the block writes the strip as one contiguous run.
+template <bool SIDE>
 __global__ void __launch_bounds__(256)
 transform_nhwc_from_nhwc_small_c_kernel(const uint16_t* __restrict__ x, uint4* __restrict__ win, int C, int H, int W,
-                                        int Ho, int Wp, int Kh, int s, int p) {
-  extern __shared__ __align__(16) uint16_t px_s[];        // [Kh][W*C]
-  const int strip = blockIdx.x;
+                                        int Ho, int Wp, int Kh, int s, int p, int lg_, int strips) {
+  const int lg = SIDE ? lg_ : 8;
+  extern __shared__ __align__(16) uint16_t px_all[];      // [strips of the block][Kh][W*C]
+  const int threads = 1 << lg, group = (int)threadIdx.x >> lg, tid = (int)threadIdx.x & (threads - 1);
+  const int strip = ((int)blockIdx.x << (8 - lg)) + group;
+  const bool live = strip < strips;
+  uint16_t* px_s = px_all + group * (Kh * W * C);
   const int n = strip / Ho, ho = strip - n * Ho;
   const int h0 = ho * s - p;
   const int row = W * C;
   for (int u = 0; u < Kh; ++u) {
     const int h = h0 + u;
-    if (h < 0 || h >= H) continue;                 // (uniform per block; such rows are never read below)
+    if (!live || h < 0 || h >= H) continue;        // (such rows are never read below)
     const uint16_t* src = x + ((int64_t)n * H + h) * row;
-    for (int i = threadIdx.x; i < row; i += 256) px_s[u * row + i] = __ldg(src + i);
+    for (int i = tid; i < row; i += threads) px_s[u * row + i] = __ldg(src + i);
   }
   __syncthreads();
+  if (!live) return;
   uint4* out = win + (int64_t)strip * Wp * Kh;
   const int chunks = Wp * Kh;
-  for (int j = threadIdx.x; j < chunks; j += 256) {
+  for (int j = tid; j < chunks; j += threads) {
     const int k = j / Kh, u = j - k * Kh;
     const int w = k - p, h = h0 + u;
     uint16_t e[8] = {0, 0, 0, 0, 0, 0, 0, 0};
@@ -1578,22 +1608,28 @@ transform_nhwc_from_nchw_kernel(const uint16_t* __restrict__ x, uint16_t* __rest
 // shared memory to S[k][u][c]; everything else (padding, channels C..7) stays zero.  A column of S is
 // PW = 4*Kh + 1 words apart, an odd number, so that the scatter and the read-out spread over the
 // banks.
+template <bool SIDE>
 __global__ void __launch_bounds__(256)
 transform_nhwc_strip_kernel(const uint16_t* __restrict__ x, uint16_t* __restrict__ win, int C, int H, int W, int Ho,
-                            int Wp, int Kh, int s, int p, int SP) {
-  extern __shared__ __align__(16) uint32_t strip_s[];     // [Wp][PW] words, then the staging area [C][SP] halves
+                            int Wp, int Kh, int s, int p, int SP, int lg_, int strips, int words) {
+  const int lg = SIDE ? lg_ : 8;
+  extern __shared__ __align__(16) uint32_t strips_s[];    // of each strip of the block `words` words: [Wp][PW], then the staging area [C][SP] halves
   const int PW = 4 * Kh + 1;
   const int strip_words = (Wp * PW + 3) & ~3;
+  const int threads = 1 << lg, group = (int)threadIdx.x >> lg, tid = (int)threadIdx.x & (threads - 1);
+  uint32_t* strip_s = strips_s + group * words;
   uint16_t* stage = reinterpret_cast<uint16_t*>(strip_s + strip_words);
-  const int64_t n = blockIdx.x / Ho;
-  const int ho = (int)(blockIdx.x - n * Ho);
+  const int strip = ((int)blockIdx.x << (8 - lg)) + group;
+  const bool live = strip < strips;
+  const int64_t n = strip / Ho;
+  const int ho = strip - (int)n * Ho;
   // rows of the image this strip holds: u_lo .. u_hi of its Kh rows
   const int h0 = ho * s - p;
   const int u_lo = h0 < 0 ? -h0 : 0;
   const int u_hi = h0 + Kh - 1 < H ? Kh - 1 : H - 1 - h0;
-  const int L = (u_hi - u_lo + 1) * W;                    // halves per channel run (<= 0: none)
+  const int L = live ? (u_hi - u_lo + 1) * W : 0;         // halves per channel run (<= 0: none)
   const int NV = L > 0 ? L / 8 + 1 : 0;                   // 16-byte pieces a run may span after its head
-  const int step = (int)blockDim.x;
+  const int step = threads;
   const uint16_t* run0 = x + ((n * C) * H + (h0 + u_lo)) * (int64_t)W;         // channel c: + c*H*W
   const int64_t cstride = (int64_t)H * W;
   // halves before the first 16-byte boundary of channel c's run
@@ -1601,7 +1637,7 @@ transform_nhwc_strip_kernel(const uint16_t* __restrict__ x, uint16_t* __restrict
   auto head_of = [&](int c) { return (8 - ((ph0 + c * cs7) & 7)) & 7; };
   if (L > 0) {
     // 16-byte pieces, four in flight per thread: item -> (c, piece)
-    for (int i0 = threadIdx.x; i0 < C * NV; i0 += 4 * step) {
+    for (int i0 = tid; i0 < C * NV; i0 += 4 * step) {
       uint4 r[4];
       int dsts[4];
 #pragma unroll
@@ -1623,7 +1659,7 @@ transform_nhwc_strip_kernel(const uint16_t* __restrict__ x, uint16_t* __restrict
         if (dsts[j] >= 0) *reinterpret_cast<uint4*>(stage + dsts[j]) = r[j];
     }
     // the ragged ends of every run, element by element: at most 7 + 7 halves per channel
-    for (int i = threadIdx.x; i < C * 16; i += step) {
+    for (int i = tid; i < C * 16; i += step) {
       const int c = i >> 4, e = i & 15;
       const uint16_t* src = run0 + c * cstride;
       const int head = head_of(c);
@@ -1636,15 +1672,15 @@ transform_nhwc_strip_kernel(const uint16_t* __restrict__ x, uint16_t* __restrict
   }
   {
     const int total = Wp * PW, quads = total / 4;
-    for (int i = threadIdx.x; i < quads; i += step) reinterpret_cast<uint4*>(strip_s)[i] = make_uint4(0u, 0u, 0u, 0u);
-    for (int i = 4 * quads + threadIdx.x; i < total; i += step) strip_s[i] = 0u;
+    for (int i = tid; i < quads; i += step) reinterpret_cast<uint4*>(strip_s)[i] = make_uint4(0u, 0u, 0u, 0u);
+    for (int i = 4 * quads + tid; i < total; i += step) strip_s[i] = 0u;
   }
   __syncthreads();
   // scatter inside shared memory: a warp takes the rows (c, u) in turn, its lanes walk the columns
   if (L > 0) {
     uint16_t* sh = reinterpret_cast<uint16_t*>(strip_s);
     const int rows = u_hi - u_lo + 1;
-    const int warp = (int)threadIdx.x >> 5, lane = (int)threadIdx.x & 31, nwarps = step >> 5;
+    const int warp = tid >> 5, lane = tid & 31, nwarps = step >> 5;
     for (int c = 0; c < C; ++c) {
       const uint16_t* src_c = stage + c * SP + 8 - head_of(c);       // element 0 of channel c's run
       for (int r = warp; r < rows; r += nwarps) {
@@ -1656,12 +1692,12 @@ transform_nhwc_strip_kernel(const uint16_t* __restrict__ x, uint16_t* __restrict
   }
   __syncthreads();
   // read-out: chunk j = k*Kh + u of the strip, consecutive threads consecutive chunks
-  {
+  if (live) {
     uint4* dst = reinterpret_cast<uint4*>(win + (n * Ho + ho) * (int64_t)Wp * Kh * 8);
     const int chunks = Wp * Kh;
     const int d_k = step / Kh, d_u = step - d_k * Kh;
-    int k = (int)threadIdx.x / Kh, u = (int)threadIdx.x - k * Kh;
-    for (int j = threadIdx.x; j < chunks; j += step) {
+    int k = tid / Kh, u = tid - k * Kh;
+    for (int j = tid; j < chunks; j += step) {
       const uint32_t* src = strip_s + k * PW + 4 * u;
       dst[j] = make_uint4(src[0], src[1], src[2], src[3]);
       u += d_u; k += d_k;
@@ -2175,6 +2211,16 @@ NhwcPlan plan_nhwc(const Geometry& g) {
   return p;
 }
 
+// Threads (their logarithm) that a strip of `items` pieces of work gets: as many as it can use, 256 or a half, a quarter or an eighth of them,
+// so that a block of 256 takes up to eight short strips side by side -- while the blocks still fill the GPU a few times.  (1x1 on 8 channels
+// at 11x11, batch 128, 7.6 -> 5.3 us; 3x3 on 3 channels at 10x10, batch 128, 6.2 -> 4.5.)
+static int strip_threads(int64_t items, int64_t strips) {
+  int lg = 8;
+  while (lg > 5 && 2 * items <= (1 << lg) && (strips << (lg - 1)) / 256 >= 4 * 148) --lg;
+  if (const char* v = debug_getenv("IM2WIN_NHWC_STRIP_THREADS")) for (lg = 5; lg < 8 && (1 << lg) < atoi(v);) ++lg;      // testing aid
+  return lg;
+}
+
 cudaError_t launch_transform_nhwc(const uint16_t* x, int x_is_nhwc, uint16_t* window, const Geometry& g,
                                   cudaStream_t stream) {
   const NhwcPlan plan = plan_nhwc(g);
@@ -2184,20 +2230,38 @@ cudaError_t launch_transform_nhwc(const uint16_t* x, int x_is_nhwc, uint16_t* wi
     bool by_strip = (int64_t)g.N * g.Ho < ((int64_t)1 << 31) && (int64_t)g.Wp * g.Kh * c8n < ((int64_t)1 << 30);
     if (const char* v = debug_getenv("IM2WIN_NHWC_TRANSFORM")) by_strip = by_strip && strcmp(v, "chunks") != 0;   // testing aid
     const unsigned strips = (unsigned)((int64_t)g.N * g.Ho);
-    if (by_strip && g.C % 8 == 0) {
+    // (few short strips of channels that are no multiple of eight: a chunk a thread, below)
+    if (by_strip && (g.C % 8 == 0 || (plan.Cp > 8 && (int64_t)strips * (((int64_t)g.Wp * c8n + 255) / 256) >= 2 * 148))) {
       uint4* w4 = reinterpret_cast<uint4*>(window);
       int sh = 0;
       while ((1 << sh) < c8n) ++sh;
-      if ((c8n & (c8n - 1)) == 0)
-        transform_nhwc_from_nhwc_strip_kernel<true><<<strips, 256, 0, stream>>>(x, w4, g.C, c8n, sh, g.H, g.W, g.Ho, g.Wp, g.Kh, g.s, g.p);
-      else
-        transform_nhwc_from_nhwc_strip_kernel<false><<<strips, 256, 0, stream>>>(x, w4, g.C, c8n, 0, g.H, g.W, g.Ho, g.Wp, g.Kh, g.s, g.p);
+      const bool pow2 = (c8n & (c8n - 1)) == 0;
+      const int64_t row_chunks = (int64_t)g.Wp * c8n;
+      const int lg = strip_threads(row_chunks, strips);
+      // a strip's chunks over several blocks where the strips alone do not fill the GPU
+      int64_t parts = (row_chunks + 255) / 256;
+      if (parts > 8 * 148 / (int64_t)strips) parts = 8 * 148 / (int64_t)strips;
+      if (parts < 1 || lg < 8) parts = 1;
+      const dim3 blocks((strips + (256 >> lg) - 1) >> (8 - lg), (unsigned)parts);
+      void (*kernel)(const uint16_t*, uint4*, int, int, int, int, int, int, int, int, int, int, int, int);
+#define IM2WIN_STRIP(V)                                                                                                          \
+  (lg < 8 ? (pow2 ? transform_nhwc_from_nhwc_strip_kernel<true, V, true> : transform_nhwc_from_nhwc_strip_kernel<false, V, true>) \
+          : (pow2 ? transform_nhwc_from_nhwc_strip_kernel<true, V, false> : transform_nhwc_from_nhwc_strip_kernel<false, V, false>))
+      if (g.C % 8 == 0) kernel = IM2WIN_STRIP(8);
+      else if (g.C % 4 == 0) kernel = IM2WIN_STRIP(4);
+      else if (g.C % 2 == 0) kernel = IM2WIN_STRIP(2);
+      else kernel = IM2WIN_STRIP(1);
+#undef IM2WIN_STRIP
+      kernel<<<blocks, 256, 0, stream>>>(x, w4, g.C, c8n, pow2 ? sh : 0, g.H, g.W, g.Ho, g.Wp, g.Kh, g.s, g.p, lg, (int)strips);
       return cudaGetLastError();
     }
     const size_t px_smem = (size_t)g.Kh * g.W * g.C * 2;
     if (by_strip && plan.Cp == 8 && px_smem <= 48 * 1024) {
-      transform_nhwc_from_nhwc_small_c_kernel<<<strips, 256, px_smem, stream>>>(x, reinterpret_cast<uint4*>(window), g.C, g.H, g.W,
-                                                                               g.Ho, g.Wp, g.Kh, g.s, g.p);
+      int lg = strip_threads((int64_t)g.Wp * g.Kh, strips);
+      while (lg < 8 && px_smem * (256 >> lg) > 48 * 1024) ++lg;
+      auto kernel = lg < 8 ? transform_nhwc_from_nhwc_small_c_kernel<true> : transform_nhwc_from_nhwc_small_c_kernel<false>;
+      kernel<<<(strips + (256 >> lg) - 1) >> (8 - lg), 256, px_smem * (256 >> lg), stream>>>(
+          x, reinterpret_cast<uint4*>(window), g.C, g.H, g.W, g.Ho, g.Wp, g.Kh, g.s, g.p, lg, (int)strips);
       return cudaGetLastError();
     }
     const int64_t chunks = plan.window_elems / 8;
@@ -2217,12 +2281,17 @@ cudaError_t launch_transform_nhwc(const uint16_t* x, int x_is_nhwc, uint16_t* wi
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
     if (strip_smem > 48 * 1024 && !attr_done[dev]) {
-      cudaError_t e = cudaFuncSetAttribute(transform_nhwc_strip_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
+      cudaError_t e = cudaFuncSetAttribute(transform_nhwc_strip_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
       if (e != cudaSuccess) return e;
       attr_done[dev] = true;
     }
-    transform_nhwc_strip_kernel<<<(unsigned)((int64_t)g.N * g.Ho), 256, (size_t)strip_smem, stream>>>(
-        x, window, g.C, g.H, g.W, g.Ho, g.Wp, g.Kh, g.s, g.p, SP);
+    const int64_t strips = (int64_t)g.N * g.Ho, region = (strip_smem + 15) & ~(int64_t)15;
+    int lg = strip_threads((int64_t)g.Wp * g.Kh, strips);
+    while (lg < 8 && region * (256 >> lg) > 48 * 1024) ++lg;
+    const int side = 256 >> lg;
+    auto kernel = lg < 8 ? transform_nhwc_strip_kernel<true> : transform_nhwc_strip_kernel<false>;
+    kernel<<<(unsigned)((strips + side - 1) / side), 256, (size_t)(region * side), stream>>>(
+        x, window, g.C, g.H, g.W, g.Ho, g.Wp, g.Kh, g.s, g.p, SP, lg, (int)strips, (int)(region / 4));
     return cudaGetLastError();
   }
   // columns per block: the whole row when it fits 48 KB of shared memory as T[w][Cp + 2]

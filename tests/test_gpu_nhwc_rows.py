@@ -38,3 +38,17 @@ def test_rows_of_any_number_of_channels(layer, kernel, monkeypatch):
         ref = np.maximum(want + bias, 0.0)
         assert np.array_equal(got, ref.astype(np.float16) if out16 else ref)
 
+
+# the transform's strips side by side in a block: short ones, a last block that is not full, channels by 8, 4, 2 and 1
+@pytest.mark.parametrize("threads", ["32", "64", "256"])
+@pytest.mark.parametrize("layer", [
+    L("t3", 3, 3, 9, 11, 8, 3, 3, 1, 1, 720), L("t8", 5, 8, 7, 14, 8, 3, 5, 1, 1, 721), L("t7", 2, 7, 13, 9, 8, 5, 3, 2, 2, 722),
+    L("t12", 3, 12, 9, 7, 8, 3, 3, 1, 1, 723), L("t18", 3, 18, 9, 8, 8, 3, 3, 2, 0, 724), L("t35", 2, 35, 11, 13, 8, 1, 1, 2, 0, 725),
+    L("t64", 3, 64, 5, 5, 8, 3, 3, 1, 1, 726)], ids=lambda l: l.name)
+@pytest.mark.parametrize("layout", ["nchw", "nhwc"])
+def test_short_strips_side_by_side(layer, layout, threads, monkeypatch):
+    monkeypatch.setenv("IM2WIN_NHWC_STRIP_THREADS", threads)
+    dims = layer.dims()
+    x, f = workloads.make_small_integer_inputs(layer)
+    yr, _ = oracle.conv_direct(x.numpy(), f.numpy(), dims)
+    assert np.array_equal(gpu_conv_nhwc(x, f, dims, x_layout=layout), yr)
