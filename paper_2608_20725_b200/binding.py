@@ -119,14 +119,16 @@ def _check(code: int, where: str) -> None:
         raise Im2winError(code, where)
 
 
-# The handle of the current stream without a Stream object around it (0.2 us instead of 3.3; a call's launches take 3.5).
+# The handle of the current stream without a Stream object around it (0.2 us instead of 3.3; a call's launches take 3), and the
+# current device without the look whether CUDA is initialised (there are CUDA tensors).
 _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_device = getattr(torch._C, "_cuda_getDevice", torch.cuda.current_device)
 
 
 def _stream(stream) -> int:
     if stream is None:
         if _raw_stream is not None:
-            return _raw_stream(torch.cuda.current_device())
+            return _raw_stream(_device())
         stream = torch.cuda.current_stream()
     return stream.cuda_stream
 
@@ -140,34 +142,35 @@ def _dtype_code(t: torch.dtype) -> int:
 
 
 _size_cache: dict = {}
+_nhwc_size_cache: dict = {}
 
 
 def im2win_workspace_size(shape, dtype: int) -> Tuple[int, int, int, int]:
     """Returns (window_bytes, scratch_bytes, Ho, Wo)."""
-    s = as_shape(shape)
-    key = (bytes(s), dtype)
+    return _sizes(as_shape(shape), dtype)[:4]
+
+
+def _sizes(s: Shape, dtype: int) -> Tuple[int, ...]:
+    """(window_bytes, scratch_bytes, Ho, Wo, elements of the input, the filter and the output)."""
+    key = bytes(s)
     hit = _size_cache.get(key)
-    if hit is not None:
-        return hit
-    out = _workspace_size_uncached(s, dtype)
-    _remember(key, out)
-    return out
-
-
-def _remember(key, sizes) -> None:
-    if _debug:
-        return
-    if len(_size_cache) >= 4096:
-        _size_cache.clear()
-    _size_cache[key] = sizes
-
-
-def _workspace_size_uncached(s: Shape, dtype: int) -> Tuple[int, int, int, int]:
+    if hit is not None and hit[dtype] is not None:
+        return hit[dtype]
     wb, sb = ctypes.c_size_t(), ctypes.c_size_t()
     ho, wo = ctypes.c_int32(), ctypes.c_int32()
     _check(lib().im2win_workspace_size(ctypes.byref(s), dtype, ctypes.byref(wb), ctypes.byref(sb),
                                        ctypes.byref(ho), ctypes.byref(wo)), "im2win_workspace_size")
-    return wb.value, sb.value, ho.value, wo.value
+    out = (wb.value, sb.value, ho.value, wo.value, s.N * s.C * s.H * s.W, s.Co * s.C * s.Kh * s.Kw, s.N * s.Co * ho.value * wo.value)
+    _remember(_size_cache, key, (out, hit[F16] if hit else None) if dtype == F32 else (hit[F32] if hit else None, out))
+    return out
+
+
+def _remember(cache, key, sizes) -> None:
+    if _debug:
+        return
+    if len(cache) >= 4096:
+        cache.clear()
+    cache[key] = sizes
 
 
 def im2win_conv_kernel_name(shape, dtype: int) -> str:
@@ -186,12 +189,14 @@ def im2win_transform(x: torch.Tensor, window: torch.Tensor, shape, stream=None) 
     """x [N,C,H,W] -> window (flat tensor of window_bytes), both CUDA tensors of the same 2/4-byte dtype."""
     s = as_shape(shape)
     assert x.is_cuda and window.is_cuda and x.is_contiguous() and window.is_contiguous()
-    assert x.dtype == window.dtype
-    code = _dtype_code(x.dtype)
-    wb, _, _, _ = im2win_workspace_size(s, code)
-    assert x.numel() == s.N * s.C * s.H * s.W and window.numel() * window.element_size() >= wb
-    _check(lib().im2win_transform(x.data_ptr(), window.data_ptr(), ctypes.byref(s), code, _stream(stream)),
-           "im2win_transform")
+    dtype = x.dtype
+    assert dtype == window.dtype
+    code = _dtype_code(dtype)
+    sizes = _sizes(s, code)
+    assert x.numel() == sizes[4] and window.nbytes >= sizes[0]
+    code = lib().im2win_transform(x.data_ptr(), window.data_ptr(), ctypes.byref(s), code, _stream(stream))
+    if code:
+        _check(code, "im2win_transform")
 
 
 def _conv(fn_name: str, dtype: torch.dtype, code: int, window, filt, y, scratch, shape, stream):
@@ -199,12 +204,12 @@ def _conv(fn_name: str, dtype: torch.dtype, code: int, window, filt, y, scratch,
     for t in (window, filt, y, scratch):
         assert t.is_cuda and t.is_contiguous()
     assert window.dtype == dtype and filt.dtype == dtype and y.dtype == torch.float32
-    wb, sb, ho, wo = im2win_workspace_size(s, code)
-    assert window.numel() * window.element_size() >= wb
-    assert filt.numel() == s.Co * s.C * s.Kh * s.Kw and y.numel() == s.N * s.Co * ho * wo
-    _check(getattr(lib(), fn_name)(window.data_ptr(), filt.data_ptr(), y.data_ptr(), scratch.data_ptr(),
-                                   scratch.numel() * scratch.element_size(), ctypes.byref(s), _stream(stream)),
-           fn_name)
+    sizes = _sizes(s, code)
+    assert window.nbytes >= sizes[0] and filt.numel() == sizes[5] and y.numel() == sizes[6]
+    code = getattr(lib(), fn_name)(window.data_ptr(), filt.data_ptr(), y.data_ptr(), scratch.data_ptr(), scratch.nbytes,
+                                   ctypes.byref(s), _stream(stream))
+    if code:
+        _check(code, fn_name)
 
 
 def im2win_conv_f32(window, filter_oihw, y, scratch, shape, stream=None) -> None:
@@ -230,7 +235,7 @@ def im2win_pack_filter(filter_oihw, scratch, shape, stream=None) -> None:
     """Packs the filter into `scratch` once (static weights); im2win_conv_packed then reuses it."""
     s = as_shape(shape)
     assert filter_oihw.is_cuda and filter_oihw.is_contiguous() and scratch.is_cuda
-    _check(lib().im2win_pack_filter(filter_oihw.data_ptr(), scratch.data_ptr(), scratch.numel() * scratch.element_size(),
+    _check(lib().im2win_pack_filter(filter_oihw.data_ptr(), scratch.data_ptr(), scratch.nbytes,
                                     ctypes.byref(s), _dtype_code(filter_oihw.dtype), _stream(stream)),
            "im2win_pack_filter")
 
@@ -240,7 +245,7 @@ def im2win_conv_packed(window, y, scratch, shape, stream=None) -> None:
     s = as_shape(shape)
     assert window.is_cuda and window.is_contiguous() and y.is_cuda and y.dtype == torch.float32 and scratch.is_cuda
     _check(lib().im2win_conv_packed(window.data_ptr(), y.data_ptr(), scratch.data_ptr(),
-                                    scratch.numel() * scratch.element_size(), ctypes.byref(s),
+                                    scratch.nbytes, ctypes.byref(s),
                                     _dtype_code(window.dtype), _stream(stream)),
            "im2win_conv_packed")
 
@@ -267,7 +272,7 @@ def im2win_layer_forward_host(x_host: torch.Tensor, filter_host: torch.Tensor, y
     code = _dtype_code(x_host.dtype)
     _check(lib().im2win_layer_forward_host(x_host.data_ptr(), filter_host.data_ptr(), y_host.data_ptr(),
                                            device_workspace.data_ptr(),
-                                           device_workspace.numel() * device_workspace.element_size(),
+                                           device_workspace.nbytes,
                                            ctypes.byref(s), code, _stream(stream)),
            "im2win_layer_forward_host")
 
@@ -282,9 +287,12 @@ def make_epilogue(bias: Optional[torch.Tensor] = None, relu: bool = False, out_d
 
 def im2win_nhwc_workspace_size(shape) -> Tuple[int, int, int, int, int]:
     """Returns (window_bytes, scratch_bytes, Ho, Wo, Cp) of the NHWC form."""
-    s = as_shape(shape)
-    key = (bytes(s), "nhwc")
-    hit = _size_cache.get(key)
+    return _nhwc_sizes(as_shape(shape))
+
+
+def _nhwc_sizes(s: Shape) -> Tuple[int, int, int, int, int]:
+    key = bytes(s)
+    hit = _nhwc_size_cache.get(key)
     if hit is not None:
         return hit
     wb, sb = ctypes.c_size_t(), ctypes.c_size_t()
@@ -292,7 +300,7 @@ def im2win_nhwc_workspace_size(shape) -> Tuple[int, int, int, int, int]:
     _check(lib().im2win_nhwc_workspace_size(ctypes.byref(s), ctypes.byref(wb), ctypes.byref(sb), ctypes.byref(ho),
                                             ctypes.byref(wo), ctypes.byref(cp)), "im2win_nhwc_workspace_size")
     out = (wb.value, sb.value, ho.value, wo.value, cp.value)
-    _remember(key, out)
+    _remember(_nhwc_size_cache, key, out)
     return out
 
 
@@ -301,10 +309,10 @@ def im2win_transform_nhwc(x: torch.Tensor, x_layout: int, window: torch.Tensor, 
     s = as_shape(shape)
     assert x.is_cuda and window.is_cuda and x.is_contiguous() and window.is_contiguous()
     assert x.dtype == torch.float16 and window.dtype == torch.float16
-    wb = im2win_nhwc_workspace_size(s)[0]
-    assert x.numel() == s.N * s.C * s.H * s.W and window.numel() * 2 >= wb
-    _check(lib().im2win_transform_nhwc(x.data_ptr(), int(x_layout), window.data_ptr(), ctypes.byref(s), _stream(stream)),
-           "im2win_transform_nhwc")
+    assert x.numel() == s.N * s.C * s.H * s.W and window.nbytes >= _nhwc_sizes(s)[0]
+    code = lib().im2win_transform_nhwc(x.data_ptr(), int(x_layout), window.data_ptr(), ctypes.byref(s), _stream(stream))
+    if code:
+        _check(code, "im2win_transform_nhwc")
 
 
 def _epi_ref(epilogue: Optional[Epilogue]):
@@ -319,7 +327,7 @@ def im2win_conv_f16_nhwc(window, filter_oihw, y, scratch, shape, epilogue: Optio
     want = torch.float32 if epilogue is None or epilogue.out_dtype == F32 else torch.float16
     assert y.dtype == want
     _check(lib().im2win_conv_f16_nhwc(window.data_ptr(), filter_oihw.data_ptr(), y.data_ptr(), _epi_ref(epilogue),
-                                      scratch.data_ptr(), scratch.numel() * scratch.element_size(), ctypes.byref(s),
+                                      scratch.data_ptr(), scratch.nbytes, ctypes.byref(s),
                                       _stream(stream)), "im2win_conv_f16_nhwc")
 
 
@@ -327,7 +335,7 @@ def im2win_pack_filter_nhwc(filter_oihw, scratch, shape, stream=None) -> None:
     s = as_shape(shape)
     assert filter_oihw.is_cuda and filter_oihw.is_contiguous() and filter_oihw.dtype == torch.float16 and scratch.is_cuda
     _check(lib().im2win_pack_filter_nhwc(filter_oihw.data_ptr(), scratch.data_ptr(),
-                                         scratch.numel() * scratch.element_size(), ctypes.byref(s), _stream(stream)),
+                                         scratch.nbytes, ctypes.byref(s), _stream(stream)),
            "im2win_pack_filter_nhwc")
 
 
@@ -335,7 +343,7 @@ def im2win_conv_packed_nhwc(window, y, scratch, shape, epilogue: Optional[Epilog
     s = as_shape(shape)
     assert window.is_cuda and window.dtype == torch.float16 and y.is_cuda and scratch.is_cuda
     _check(lib().im2win_conv_packed_nhwc(window.data_ptr(), y.data_ptr(), _epi_ref(epilogue), scratch.data_ptr(),
-                                         scratch.numel() * scratch.element_size(), ctypes.byref(s), _stream(stream)),
+                                         scratch.nbytes, ctypes.byref(s), _stream(stream)),
            "im2win_conv_packed_nhwc")
 
 
@@ -368,13 +376,19 @@ def conv2d_im2win(x: torch.Tensor, filter_oihw: torch.Tensor, stride: int, pad: 
     N, C, H, W = x.shape
     Co, C2, Kh, Kw = filter_oihw.shape
     assert C == C2
+    dtype = x.dtype
+    code = _dtype_code(dtype)
+    assert x.is_cuda and filter_oihw.is_cuda and filter_oihw.dtype == dtype
     s = make_shape(N, C, H, W, Co, Kh, Kw, stride, pad)
-    window, scratch, y = alloc_layer_buffers(s, x.dtype, x.device)
+    sizes = _sizes(s, code)
     x = x.contiguous()
     filter_oihw = filter_oihw.contiguous()
-    im2win_transform(x, window, s, stream)
-    if x.dtype == torch.float32:
-        im2win_conv_f32(window, filter_oihw, y, scratch, s, stream)
-    else:
-        im2win_conv_f16(window, filter_oihw, y, scratch, s, stream)
+    # window and scratch in one buffer (an allocation takes as long as half a launch)
+    scratch_at = (sizes[0] + 255) & ~255
+    buffer = x.new_empty((scratch_at + sizes[1],), dtype=torch.uint8)
+    y = x.new_empty((N, Co, sizes[2], sizes[3]), dtype=torch.float32)
+    L, window, shape, queue = lib(), buffer.data_ptr(), ctypes.byref(s), _stream(stream)
+    _check(L.im2win_transform(x.data_ptr(), window, shape, code, queue), "im2win_transform")
+    name = "im2win_conv_f32" if code == F32 else "im2win_conv_f16"
+    _check(getattr(L, name)(window, filter_oihw.data_ptr(), y.data_ptr(), window + scratch_at, sizes[1], shape, queue), name)
     return y
