@@ -42,6 +42,7 @@
 #include <stdlib.h>
 
 #include "common.cuh"
+#include "launch.cuh"
 #include "ptx_sm100.cuh"
 
 namespace im2win {
@@ -644,6 +645,7 @@ __global__ void pack_f16_mat_kernel(const uint16_t* __restrict__ f, uint16_t* __
                                     int C, int Co, int Kh, int Kw, int K2p, int ncog, int noct) {
   extern __shared__ __align__(16) uint16_t pack_s[];
   let_next_kernel_start();
+  wait_for_previous_kernel();
   const size_t f_total = (size_t)Co * C * Kh * Kw;
   if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < kStatusBytes / 4) status[threadIdx.x] = 0u;
   const int num_kb = K2p / KB;
@@ -916,9 +918,8 @@ cudaError_t launch_pack_f16_mat(const uint16_t* filter, void* scratch, const Geo
   const size_t smem = ((size_t)noct * 8 * g.T + 16) * sizeof(uint16_t);
   if (smem > 48 * 1024) return cudaErrorInvalidValue;
   dim3 grid((unsigned)((plan.Cp8 + noct - 1) / noct), (unsigned)(ncog * 64 < 32768 ? ncog * 64 : 32768));
-  pack_f16_mat_kernel<<<grid, 256, smem, stream>>>(filter, fp, reinterpret_cast<uint32_t*>(base), g.C, g.Co, g.Kh, g.Kw,
+  return launch_early(pack_f16_mat_kernel, grid, 256, smem, stream, filter, fp, reinterpret_cast<uint32_t*>(base), g.C, g.Co, g.Kh, g.Kw,
                                                    (int)plan.K2p, ncog, noct);
-  return cudaGetLastError();
 }
 
 cudaError_t launch_conv_f16_mat(const uint16_t* window, float* y, void* scratch, const Geometry& g,

@@ -926,6 +926,7 @@ __global__ void __launch_bounds__(256) pack_f16_runs_kernel(const uint16_t* __re
                                                         int Co, int bn, int num_kb, int rows, int pitch, int quad) {
   extern __shared__ uint16_t pack_h[];
   let_next_kernel_start();                                 // (the convolution sets itself up meanwhile)
+  wait_for_previous_kernel();
   if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < kStatusBytes / 4) status[threadIdx.x] = 0u;
   const int kb = blockIdx.y, row0 = blockIdx.x * rows;     // (channel blocks along x: any number of channels)
   const int c0 = quad ? 0 : kb * 8 / E * 8;
@@ -1160,9 +1161,8 @@ cudaError_t launch_pack_f16_runs(const uint16_t* filter, void* scratch, const Ge
   while (rows > 1 && (rows * pitch * ES > 40 * 1024 || (int64_t)p.ntn * p.bn / rows * p.num_kb < 2 * 148)) rows /= 2;
   const size_t smem = (size_t)(rows * pitch * ES);
   dim3 grid((unsigned)(p.ntn * p.bn / rows), (unsigned)p.num_kb);   // (num_kb <= 2^14: C * E <= 2^20)
-  pack_f16_runs_kernel<<<grid, 256, smem, stream>>>(filter, base + kStatusBytes, reinterpret_cast<uint32_t*>(base), g.C, g.Kh, g.Kw,
+  return launch_early(pack_f16_runs_kernel, grid, 256, smem, stream, filter, base + kStatusBytes, reinterpret_cast<uint32_t*>(base), g.C, g.Kh, g.Kw,
                                                     g.s, p.E, p.G, g.Co, p.bn, p.num_kb, rows, (int)pitch, p.quad);
-  return cudaGetLastError();
 }
 
 cudaError_t launch_conv_f16_runs(const uint16_t* window, float* y, void* scratch, const Geometry& g, cudaStream_t stream) {

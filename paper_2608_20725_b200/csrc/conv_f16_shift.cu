@@ -41,6 +41,7 @@
 #include <stdlib.h>
 
 #include "common.cuh"
+#include "launch.cuh"
 #include "ptx_sm100.cuh"
 
 namespace im2win {
@@ -122,6 +123,7 @@ conv_f16_shift_kernel(const __grid_constant__ CUtensorMap fmap, ShiftParams q) {
   if (warp == PRODUCER_WARPS + 1) tmem_alloc(smem_u32(&tmem_base_slot), 2 * BN);
   // k2 -> element offset table of the whole reduction, kept in shared memory
   int32_t* koff_s = reinterpret_cast<int32_t*>(smem + q.sa * q.a_stage_bytes + q.sb * B_STAGE_BYTES);
+  wait_for_previous_kernel();
   for (int i = threadIdx.x; i < q.num_kb * KB; i += NUM_THREADS) koff_s[i] = __ldg(q.koff2 + i);
   tc_fence_before();
   __syncthreads();
@@ -473,19 +475,20 @@ cudaError_t launch_variant(const CUtensorMap& fmap, const ShiftParams& q0, const
   const dim3 grid((unsigned)((units - q.nbig) * q.split), (unsigned)((co + BN - 1) / BN));   // a tall tile covers two units
   if constexpr (SPLIT) {
     cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = (unsigned)q.split; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.gridDim = grid;
     cfg.blockDim = dim3(NUM_THREADS, 1, 1);
     cfg.dynamicSmemBytes = (size_t)smem_bytes;
     cfg.stream = stream;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     return cudaLaunchKernelEx(&cfg, conv_f16_shift_kernel<BN, ITEMS, SPLIT>, fmap, q);
   } else {
-    conv_f16_shift_kernel<BN, ITEMS, SPLIT><<<grid, NUM_THREADS, smem_bytes, stream>>>(fmap, q);
-    return cudaGetLastError();
+    return launch_early(conv_f16_shift_kernel<BN, ITEMS, SPLIT>, grid, NUM_THREADS, (size_t)smem_bytes, stream, fmap, q);
   }
 }
 

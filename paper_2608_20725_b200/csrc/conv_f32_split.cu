@@ -653,6 +653,7 @@ __global__ void __launch_bounds__(256) pack_f32_split_kernel(const float* __rest
                                                              int num_kb, int rows, int concat) {
   extern __shared__ float pack_f[];
   let_next_kernel_start();                                 // (the convolution sets itself up meanwhile)
+  wait_for_previous_kernel();
   if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < kStatusBytes / 4) status[threadIdx.x] = 0u;
   const int kb = blockIdx.y, row0 = blockIdx.x * rows;     // (channel blocks along x: any number of channels)
   const int nreal = K2 - kb * KB < KB ? K2 - kb * KB : KB;
@@ -815,9 +816,9 @@ cudaError_t launch_pack_f32_split(const float* filter, void* scratch, const Geom
   while (rows > 1 && ((size_t)rows * KB * g.Kw * 4 > 40 * 1024 || (int64_t)p.ntn * p.bn / rows * p.num_kb < 2 * 148)) rows /= 2;
   const size_t smem = (size_t)rows * KB * g.Kw * 4;
   dim3 grid((unsigned)(p.ntn * p.bn / rows), (unsigned)p.num_kb);
-  pack_f32_split_kernel<<<grid, 256, smem, stream>>>(filter, base + kStatusBytes, reinterpret_cast<float*>(base + kStatusBytes + p.copy_off), reinterpret_cast<uint32_t*>(base), g.C * g.Kh,
-                                                     g.Kw, g.Co, p.bn, p.num_kb, rows, p.bn <= CONCAT_BN ? 1 : 0);
-  return cudaGetLastError();
+  return launch_early(pack_f32_split_kernel, grid, 256, smem, stream, filter, base + kStatusBytes,
+                      reinterpret_cast<float*>(base + kStatusBytes + p.copy_off), reinterpret_cast<uint32_t*>(base), g.C * g.Kh, g.Kw, g.Co,
+                      p.bn, p.num_kb, rows, p.bn <= CONCAT_BN ? 1 : 0);
 }
 
 cudaError_t launch_conv_f32_split(const float* window, float* y, void* scratch, const Geometry& g, cudaStream_t stream) {

@@ -29,6 +29,7 @@
 #include <atomic>
 
 #include "common.cuh"
+#include "launch.cuh"
 #include "ptx_sm100.cuh"
 
 namespace im2win {
@@ -1263,7 +1264,8 @@ pack_f16_nhwc_kernel(const uint16_t* __restrict__ f, uint16_t* __restrict__ fp, 
   extern __shared__ __align__(16) uint16_t pack_s[];   // [cb][T], after up to 8 halves of phase padding
   // the convolution that follows in the stream may be launched now: its set-up overlaps this kernel,
   // and every role of it that touches memory first waits for this grid to have completed
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  let_next_kernel_start();
+  wait_for_previous_kernel();
   if (blockIdx.x == 0 && blockIdx.y == 0) {
     if (threadIdx.x < kStatusBytes / 4) status[threadIdx.x] = 0u;
     for (int i = threadIdx.x; i < kTailFlagBytes / 4; i += blockDim.x) flags[i] = 0u;
@@ -1336,6 +1338,7 @@ template <> struct VecType<1> { typedef uint16_t type; };
 // (or zeros in the padding): 16-byte chunks, one per thread, consecutive threads along (k, u, c).
 __global__ void transform_nhwc_from_nhwc_kernel(const uint16_t* __restrict__ x, uint16_t* __restrict__ win, int C, int Cp,
                                                 int H, int W, int Ho, int Wp, int Kh, int s, int p, int64_t chunks) {
+  let_next_kernel_start();
   const int c8n = Cp / 8;
   const bool vec = (C % 8) == 0;
   for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < chunks; idx += (int64_t)gridDim.x * blockDim.x) {
@@ -1377,6 +1380,7 @@ template <bool POW2, int VEC, bool SIDE>
 __global__ void __launch_bounds__(256)
 transform_nhwc_from_nhwc_strip_kernel(const uint16_t* __restrict__ x, uint4* __restrict__ win, int C, int c8n, int sh,
                                       int H, int W, int Ho, int Wp, int Kh, int s, int p, int lg_, int strips) {
+  let_next_kernel_start();
   const int lg = SIDE ? lg_ : 8;                 // (a constant where a block has one strip: a run-time one cost 7 to 12 %)
   const int strip = ((int)blockIdx.x << (8 - lg)) + ((int)threadIdx.x >> lg);      // n*Ho + ho
   if (strip >= strips) return;
@@ -1431,6 +1435,7 @@ template <bool SIDE>
 __global__ void __launch_bounds__(256)
 transform_nhwc_from_nhwc_small_c_kernel(const uint16_t* __restrict__ x, uint4* __restrict__ win, int C, int H, int W,
                                         int Ho, int Wp, int Kh, int s, int p, int lg_, int strips) {
+  let_next_kernel_start();
   const int lg = SIDE ? lg_ : 8;
   extern __shared__ __align__(16) uint16_t px_all[];      // [strips of the block][Kh][W*C]
   const int threads = 1 << lg, group = (int)threadIdx.x >> lg, tid = (int)threadIdx.x & (threads - 1);
@@ -1481,6 +1486,7 @@ template <int VEC, bool SWZ>
 __global__ void __launch_bounds__(256)
 transform_nhwc_from_nchw_kernel(const uint16_t* __restrict__ x, uint16_t* __restrict__ win, int C, int Cp, int H, int W,
                                 int Ho, int Wp, int Kh, int s, int p, int kc, int kchunks, int R, int rgroups) {
+  let_next_kernel_start();
   extern __shared__ __align__(16) uint16_t rows_s[];     // T[kc][Cp + 2], or (SWZ) T[kc][Cp] with swizzled chunks
   const int PC = SWZ ? Cp : Cp + 2;
   const int smask = SWZ ? ((Cp / 8 < 8 ? Cp / 8 : 8) - 1) : 0;
@@ -1612,6 +1618,7 @@ template <bool SIDE>
 __global__ void __launch_bounds__(256)
 transform_nhwc_strip_kernel(const uint16_t* __restrict__ x, uint16_t* __restrict__ win, int C, int H, int W, int Ho,
                             int Wp, int Kh, int s, int p, int SP, int lg_, int strips, int words) {
+  let_next_kernel_start();
   const int lg = SIDE ? lg_ : 8;
   extern __shared__ __align__(16) uint32_t strips_s[];    // of each strip of the block `words` words: [Wp][PW], then the staging area [C][SP] halves
   const int PW = 4 * Kh + 1;
@@ -2350,11 +2357,9 @@ cudaError_t launch_pack_f16_nhwc(const uint16_t* filter, void* scratch, const Ge
     if (e != cudaSuccess) return e;
   }
   dim3 grid((unsigned)((plan.Cp + cb - 1) / cb), (unsigned)(g.Co < 32768 ? g.Co : 32768));
-  pack_f16_nhwc_kernel<<<grid, 256, smem, stream>>>(filter, reinterpret_cast<uint16_t*>(base + kStatusBytes),
-                                                     reinterpret_cast<uint32_t*>(base),
-                                                     reinterpret_cast<uint32_t*>(base + plan.flags_off), g.C, plan.Cp, g.Co,
-                                                     g.Kh, g.Kw, cb);
-  return cudaGetLastError();
+  return launch_early(pack_f16_nhwc_kernel, grid, 256, smem, stream, filter, reinterpret_cast<uint16_t*>(base + kStatusBytes),
+                      reinterpret_cast<uint32_t*>(base), reinterpret_cast<uint32_t*>(base + plan.flags_off), g.C, plan.Cp, g.Co, g.Kh,
+                      g.Kw, cb);
 }
 
 namespace {

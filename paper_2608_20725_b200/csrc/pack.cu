@@ -12,6 +12,8 @@
 //   fp16 gather kernel: Fp[co][Kp]     (k contiguous),  zero padded in k
 //   fp16 shifted-view kernel: Fp2[v][co][K2p] with k2 = c*Kh + u (see pack_f16_shift_kernel)
 #include "common.cuh"
+#include "launch.cuh"
+#include "ptx_sm100.cuh"
 
 namespace im2win {
 namespace {
@@ -31,6 +33,8 @@ __device__ __forceinline__ void split_k(const PackParams& q, int64_t k, int& c, 
 __global__ void pack_f32_kernel(const float* __restrict__ f, float* __restrict__ fk,
                                 int32_t* __restrict__ koff, uint32_t* __restrict__ status,
                                 PackParams q) {
+  ptx::let_next_kernel_start();
+  ptx::wait_for_previous_kernel();
   if (blockIdx.x == 0 && threadIdx.x < kStatusBytes / 4) status[threadIdx.x] = 0u;
   const int64_t total = q.Kp * q.Co_pad;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -59,6 +63,8 @@ __global__ void pack_f32_kernel(const float* __restrict__ f, float* __restrict__
 __global__ void pack_f16_kernel(const uint16_t* __restrict__ f, uint16_t* __restrict__ fp,
                                 int32_t* __restrict__ koff, uint32_t* __restrict__ status,
                                 PackParams q) {
+  ptx::let_next_kernel_start();
+  ptx::wait_for_previous_kernel();
   if (blockIdx.x == 0 && threadIdx.x < kStatusBytes / 4) status[threadIdx.x] = 0u;
   const int64_t total = q.Kp * q.Co;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -89,6 +95,8 @@ __global__ void pack_f16_shift_kernel(const uint16_t* __restrict__ f, uint16_t* 
                                       uint32_t* __restrict__ table, uint32_t* __restrict__ status,
                                       PackParams q, int raw_pitch, int nslot, int chunk) {
   extern __shared__ __align__(16) uint16_t pack_s[];
+  ptx::let_next_kernel_start();
+  ptx::wait_for_previous_kernel();
   if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < kStatusBytes / 4) status[threadIdx.x] = 0u;
   const int K2 = q.C * q.Kh;
   const int K2p = (int)q.Kp;
@@ -166,20 +174,18 @@ cudaError_t launch_pack_f32(const float* filter, void* scratch, const Geometry& 
                             const ScratchLayout& l, cudaStream_t stream) {
   unsigned char* base = static_cast<unsigned char*>(scratch);
   PackParams q = make_params(g, l);
-  pack_f32_kernel<<<grid_for(q.Kp * q.Co_pad), 256, 0, stream>>>(
+  return launch_early(pack_f32_kernel, grid_for(q.Kp * q.Co_pad), 256, 0, stream,
       filter, reinterpret_cast<float*>(base + l.filter_off),
       reinterpret_cast<int32_t*>(base + l.koff_off), reinterpret_cast<uint32_t*>(base), q);
-  return cudaGetLastError();
 }
 
 cudaError_t launch_pack_f16(const uint16_t* filter, void* scratch, const Geometry& g,
                             const ScratchLayout& l, cudaStream_t stream) {
   unsigned char* base = static_cast<unsigned char*>(scratch);
   PackParams q = make_params(g, l);
-  pack_f16_kernel<<<grid_for(q.Kp * q.Co), 256, 0, stream>>>(
+  return launch_early(pack_f16_kernel, grid_for(q.Kp * q.Co), 256, 0, stream,
       filter, reinterpret_cast<uint16_t*>(base + l.filter_off),
       reinterpret_cast<int32_t*>(base + l.koff_off), reinterpret_cast<uint32_t*>(base), q);
-  return cudaGetLastError();
 }
 
 static cudaError_t pack_shift_common(const uint16_t* filter, void* scratch, const Geometry& g,
@@ -191,10 +197,9 @@ static cudaError_t pack_shift_common(const uint16_t* filter, void* scratch, cons
   const size_t smem = ((size_t)chunk * g.Kw + 16) * sizeof(uint16_t);
   if (smem > 48 * 1024) return cudaErrorInvalidValue;
   dim3 grid((unsigned)((q.Kp + chunk - 1) / chunk), (unsigned)(g.Co < 32768 ? g.Co : 32768));
-  pack_f16_shift_kernel<<<grid, 256, smem, stream>>>(filter, reinterpret_cast<uint16_t*>(base + l.filter_off),
+  return launch_early(pack_f16_shift_kernel, grid, 256, smem, stream, filter, reinterpret_cast<uint16_t*>(base + l.filter_off),
                                                      reinterpret_cast<uint32_t*>(base + l.koff_off),
                                                      reinterpret_cast<uint32_t*>(base), q, raw_pitch, nslot, chunk);
-  return cudaGetLastError();
 }
 
 cudaError_t launch_pack_f16_shift(const uint16_t* filter, void* scratch, const Geometry& g,

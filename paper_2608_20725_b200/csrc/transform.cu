@@ -28,6 +28,7 @@
 #include <string.h>
 
 #include "common.cuh"
+#include "ptx_sm100.cuh"
 
 namespace im2win {
 namespace {
@@ -76,6 +77,7 @@ constexpr int kTransformThreads = 256;
 template <typename E, int KH>
 __global__ void __launch_bounds__(kTransformThreads)
 transform_kernel(const E* __restrict__ x, E* __restrict__ win, TransformParams q) {
+  ptx::let_next_kernel_start();                    // (the kernels of this library wait for this one's end before they touch memory)
   extern __shared__ __align__(16) unsigned char smem_raw[];
   E* stage = reinterpret_cast<E*>(smem_raw);
 
@@ -179,6 +181,7 @@ __device__ __forceinline__ uint32_t run_pair16(const uint32_t (&r)[KH][NW], int 
 template <typename E, int KH, int VB>
 __global__ void __launch_bounds__(kStripThreads, KH >= 7 ? 4 : 0)   // (tall kernels: four CTAs per SM; they would otherwise take 76-128 registers and run three)
 transform_strips_kernel(const E* __restrict__ x, E* __restrict__ win, StripParams q) {
+  ptx::let_next_kernel_start();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int ES = (int)sizeof(E);
   constexpr int CPL = 4 / ES;                     // columns per item: one 32-bit word per kernel row

@@ -167,3 +167,37 @@ def test_which_fp16_layers_are_shared(layer, ctas):
     ((1, 256, 8, 8, 103, 3, 3, 1, 0), (16, 12))])
 def test_which_fp32_layers_are_shared(layer, form):
     assert split_form(layer)[:2] == form
+
+
+# kernels that start before the one ahead of them has ended (transform, filter pack, convolution): passes queued back to back on the same
+# window and scratch, inputs and filters in turn, give what each gives alone
+@pytest.mark.gpu
+@pytest.mark.parametrize("layer,dtype,kernel", [
+    (L("b_split", 8, 64, 30, 30, 64, 3, 3, 1, 1, 660), torch.float32, "f32-split"), (L("b_ffma", 8, 3, 40, 40, 40, 3, 3, 1, 1, 661), torch.float32, "f32-ffma"),
+    (L("b_runs", 16, 64, 28, 28, 64, 3, 3, 1, 1, 662), torch.float16, "f16-runs"), (L("b_shift", 2, 128, 21, 21, 64, 7, 7, 1, 3, 663), torch.float16, "f16-shift"),
+    (L("b_stem", 16, 3, 60, 60, 64, 7, 7, 2, 3, 664), torch.float16, "f16-stem"), (L("b_mat", 8, 128, 28, 28, 256, 3, 3, 1, 1, 665), torch.float16, "f16-mat"),
+    (L("b_nhwc", 8, 40, 30, 30, 70, 3, 3, 1, 1, 666), torch.float16, None)], ids=lambda v: getattr(v, "name", str(v)))
+def test_passes_back_to_back(layer, dtype, kernel):
+    dims = layer.dims()
+    code = binding.F32 if dtype == torch.float32 else binding.F16
+    assert kernel is None or binding.im2win_conv_kernel_name(dims, code) == kernel
+    x, f = workloads.make_inputs(layer)
+    xs, fs = [x.to(dtype).cuda(), (x.flip(0) * 2).to(dtype).cuda()], [f.to(dtype).cuda(), f.flip(0).to(dtype).cuda()]
+    window, scratch, y = binding.alloc_layer_buffers(dims, dtype) if kernel else binding.alloc_nhwc_buffers(dims)
+    out = [torch.empty_like(y) for _ in range(12)]
+
+    def one(i, y):
+        if kernel is None:
+            binding.im2win_transform_nhwc(xs[i % 2], binding.NCHW, window, dims)
+            binding.im2win_conv_f16_nhwc(window, fs[i % 3 % 2], y, scratch, dims)
+        else:
+            binding.im2win_transform(xs[i % 2], window, dims)
+            (binding.im2win_conv_f32 if code == binding.F32 else binding.im2win_conv_f16)(window, fs[i % 3 % 2], y, scratch, dims)
+
+    for i in range(12):
+        one(i, out[i])
+    binding.im2win_check_status(scratch)
+    for i in range(12):
+        one(i, y)
+        binding.im2win_check_status(scratch)
+        assert torch.equal(out[i], y)
