@@ -116,9 +116,13 @@ __device__ __forceinline__ void store_chunk(const EpiParams& q, int64_t base, in
     float* p = reinterpret_cast<float*>(q.y) + base;
     if (!q.y_nhwc) {
       store_strided32(p, cs, v, cnt);
-    } else if (vec_ok) {                                     // (then cnt is a multiple of four)
+    } else if (vec_ok && cnt == 32) {
 #pragma unroll
       for (int j = 0; j < 32; j += 4)
+        *reinterpret_cast<uint4*>(p + j) = make_uint4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+    } else if (vec_ok) {                                     // (then cnt is a multiple of four)
+#pragma unroll
+      for (int j = 0; j < 28; j += 4)
         if (j < cnt) *reinterpret_cast<uint4*>(p + j) = make_uint4(v[j], v[j + 1], v[j + 2], v[j + 3]);
     } else {
 #pragma unroll
@@ -137,7 +141,7 @@ __device__ __forceinline__ void store_chunk(const EpiParams& q, int64_t base, in
         if (j + 1 < cnt) *p1 = __float2half_rn(__uint_as_float(v[j + 1]));
         p0 += step; p1 += step;
       }
-    } else if (vec_ok) {
+    } else if (vec_ok) {                                     // (then cnt is a multiple of eight)
 #pragma unroll
       for (int j = 0; j < 32; j += 8) {
         if (j >= cnt) break;
@@ -753,6 +757,163 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
 conv_f16_nhwc_pair_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ CUtensorMap bmap,
                           const __grid_constant__ CUtensorMap bmap_h, NhwcParams q) {
   conv_nhwc_body<BN, true, KSUB, ROWS>(amap, bmap, bmap_h, q);
+}
+
+// The overlapping-row kernel where tiles are so few that SMs would be left over: the q.ksplit CTAs of a cluster share a tile's k-blocks, push
+// their sums to the CTA that finishes a share of the channels (ClusterSums), and that one adds them in rank order and applies the epilogue,
+// so that any epilogue works and nothing leaves the chip in between.  One tile a cluster, one accumulator; the roles of conv_nhwc_body.
+template <int BN>
+__global__ void __launch_bounds__(NUM_THREADS, 1)
+conv_f16_nhwc_shared_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ CUtensorMap bmap, NhwcParams q) {
+  constexpr uint32_t B_BYTES = (uint32_t)BN * KB * 2, STAGE_BYTES = (uint32_t)A_SLOT_BYTES + B_BYTES;
+  extern __shared__ unsigned char smem_dyn[];
+  unsigned char* smem = reinterpret_cast<unsigned char*>(((uintptr_t)smem_dyn + 1023) & ~(uintptr_t)1023);
+  __shared__ __align__(8) uint64_t bars[2 * MAX_STAGES + 1];
+  __shared__ uint32_t tmem_base_slot;
+  __shared__ volatile uint32_t abort_flag;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
+  const uint32_t ring = smem_u32(smem), full0 = smem_u32(&bars[0]), empty0 = smem_u32(&bars[MAX_STAGES]), acc_full = smem_u32(&bars[2 * MAX_STAGES]);
+  const int rank = (int)cluster_ctarank(), tile = (int)blockIdx.x / q.ksplit;
+  const int mt = tile / q.ntn, n0 = (tile - mt * q.ntn) * BN, rg = mt / q.tw, wt = mt - rg * q.tw;
+  const int kb0 = (int)((int64_t)q.num_kc * rank / q.ksplit), kb1 = (int)((int64_t)q.num_kc * (rank + 1) / q.ksplit);
+  if (threadIdx.x == 0) {
+    abort_flag = 0u;
+    for (int i = 0; i < MAX_STAGES; ++i) { mbar_init(full0 + 8 * i, 1); mbar_init(empty0 + 8 * i, 1); }
+    mbar_init(acc_full, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == WARP_MMA) tmem_alloc(smem_u32(&tmem_base_slot), BN);
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_acc = tmem_base_slot;
+  wait_for_previous_kernel();
+
+  bool ok = true;
+  if (warp == WARP_TMA) {
+    const bool leader = elect_one();
+    int st = 0;
+    uint32_t ph = 0;
+    for (int kb = kb0; kb < kb1; ++kb) {
+      ok = mbar_wait(empty0 + 8 * st, ph ^ 1u, &abort_flag, q.status);
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) break;
+      if (leader) {
+        const uint32_t dst = ring + (uint32_t)st * STAGE_BYTES, bar = full0 + 8 * st;
+        mbar_arrive_expect_tx(bar, q.a_bytes + B_BYTES);
+        tma_load_3d(dst, &amap, kb * KB, wt * q.bw, rg * q.G, bar);
+        tma_load_2d(dst + (uint32_t)A_SLOT_BYTES, &bmap, kb * KB, n0, bar);
+      }
+      __syncwarp();
+      if (++st == q.stages) { st = 0; ph ^= 1u; }
+    }
+    if (!ok) for (int i = 0; i < 64; ++i) __nanosleep(1000);         // copies in flight must land first
+  } else if (warp == WARP_MMA) {
+    constexpr uint32_t idesc = instr_desc_f16(TILE_M, BN);
+    const bool leader = elect_one();
+    const uint32_t a_lo0 = smem_desc_lo(ring), b_lo0 = smem_desc_lo(ring + (uint32_t)A_SLOT_BYTES);
+    int st = 0;
+    uint32_t ph = 0;
+    for (int kb = kb0; kb < kb1; ++kb) {
+      ok = mbar_wait(full0 + 8 * st, ph, &abort_flag, q.status);
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) break;
+      tc_fence_after();
+      if (leader) {
+        const uint32_t at = (uint32_t)st * (STAGE_BYTES >> 4);
+        const int nks = kb != q.num_kc - 1 ? KB / 16 : q.nks_last;
+#pragma unroll
+        for (int j = 0; j < KB / 16; ++j)
+          if (j < nks) umma_f16_lohi(tmem_acc, a_lo0 + at + 2 * j, b_lo0 + at + 2 * j, idesc, kb > kb0 || j > 0 ? 1u : 0u);
+        umma_commit(empty0 + 8 * st);
+        if (kb == kb1 - 1) umma_commit(acc_full);
+      }
+      __syncwarp();
+      if (++st == q.stages) { st = 0; ph ^= 1u; }
+    }
+  } else {
+    ok = mbar_wait(acc_full, 0u, &abort_flag, q.status);
+    ok = __all_sync(0xffffffffu, ok);
+  }
+
+  const EpiParams& e = q.e;
+  const int channels = e.Co - n0 < BN ? e.Co - n0 : BN, lq = warp & 3, h = (warp - WARP_EPI0) >> 2, position = lq * 32 + lane;
+  const ClusterSums sums(ring, q.ksplit, rank, channels);
+  __syncwarp();
+  cluster_sync_all();                                        // (every MMA of every CTA has completed)
+  if (warp >= WARP_EPI0 && ok) {
+    tc_fence_after();
+#pragma unroll 1
+    for (int c0 = h * (BN / 2); c0 < (h + 1) * (BN / 2) && c0 < channels; c0 += 32) {
+      uint32_t v[32];
+      float f[32];
+      tmem_ld32(tmem_acc + ((uint32_t)(lq * 32) << 16) + (uint32_t)c0, v);
+#pragma unroll
+      for (int t = 0; t < 32; ++t) f[t] = __uint_as_float(v[t]);
+      sums.store(f, c0, channels, position);
+    }
+  }
+  __syncwarp();
+  cluster_sync_all();
+  if (warp >= WARP_EPI0) {
+    const int first = rank * sums.per, mine = channels - first < sums.per ? channels - first : sums.per;
+    // row r of the tile: its strip and output column
+    auto locate = [&](int r, int& strip, int& wo) {
+      const int j = r / q.bw;
+      strip = rg * q.G + j;
+      wo = wt * q.bw + r - j * q.bw;
+      return j < q.G && strip < e.rows_total && wo < e.Wo;
+    };
+    auto finish = [&](int c) {
+      float v = sums.sum(c, position);
+      if (e.bias != nullptr) v += __ldg(e.bias + n0 + first + c);
+      return e.relu ? fmaxf(v, 0.0f) : v;
+    };
+    auto put = [&](int64_t at, float v) {
+      if (e.out16) reinterpret_cast<__half*>(e.y)[at] = __float2half_rn(v);
+      else reinterpret_cast<float*>(e.y)[at] = v;
+    };
+    int strip, wo;
+    if (!e.y_nhwc) {
+      if (locate(position, strip, wo)) {
+        const int n = strip / e.Ho;
+        const int64_t base = ((int64_t)n * e.Co + n0 + first) * e.HoWo + (strip - n * e.Ho) * e.Wo + wo;
+        for (int c = h; c < mine; c += 2) put(base + (int64_t)c * e.HoWo, finish(c));
+      }
+    } else {
+      // through shared memory, so that the lanes lie along a row's channels (an element a lane and row: 8.1 -> 9.7 us on 3x3 stride 2, 82 -> 64
+      // channels at 95x95, and 17.6 -> 27.3 on 3x3 on 512 -> 512 at 16x16, batch 4)
+      float* rows = reinterpret_cast<float*>(smem + cluster_sums_bytes(BN));
+      const int pitch = sums.per | 1;
+      for (int c = h; c < mine; c += 2) rows[position * pitch + c] = finish(c);
+      asm volatile("bar.sync 1, %0;" ::"n"(EPI_WARPS * 32) : "memory");
+      // 16 rows a warp: lane l knows where row l & 15 goes; 4 to 32 lanes store a row's channels
+      const int row0 = (warp - WARP_EPI0) * 16;
+      const bool live = locate(row0 + (lane & 15), strip, wo);
+      const uint32_t live_rows = __ballot_sync(0xffffffffu, live);
+      const int64_t at = ((int64_t)strip * e.Wo + wo) * e.Co + n0 + first;
+      const int log = mine <= 4 ? 2 : (mine <= 8 ? 3 : (mine <= 16 ? 4 : 5)), col = lane & ((1 << log) - 1);
+#pragma unroll 4
+      for (int r = lane >> log; r < 16; r += 32 >> log) {
+        const int64_t base = __shfl_sync(0xffffffffu, at, r);
+        if (live_rows >> r & 1u)
+          for (int c = col; c < mine; c += 32) put(base + c, rows[(row0 + r) * pitch + c]);
+      }
+    }
+  }
+
+  // ---------------- teardown ---------------------------------------------------
+  tc_fence_before();
+  __syncthreads();
+  if (abort_flag) {
+    for (int i = 0; i < 64; ++i) __nanosleep(1000);
+    __syncthreads();
+  }
+  if (warp == WARP_MMA) {
+    __syncwarp();
+    tc_fence_after();
+    tmem_dealloc(tmem_acc, BN);
+  }
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -1889,6 +2050,41 @@ cudaError_t launch_variant(const CUtensorMap& amap, const CUtensorMap& bmap, con
   return cudaLaunchKernelEx(&cfg, conv_f16_nhwc_kernel<BN, KSUB, ROWS>, amap, bmap, bmap_h, q);
 }
 
+template <int BN>
+cudaError_t launch_shared(const CUtensorMap& amap, const CUtensorMap& bmap, NhwcParams q, const NhwcPlan& plan, cudaStream_t stream) {
+  constexpr int STAGE = A_SLOT_BYTES + BN * KB * 2;
+  int stages = (kSmemMax - 2048) / STAGE;
+  if (stages > MAX_STAGES) stages = MAX_STAGES;
+  q.stages = stages;
+  q.num_kc = plan.num_kb;
+  q.nks_last = (int32_t)((plan.K - (int64_t)(plan.num_kb - 1) * KB + 15) / 16);
+  int smem_bytes = stages * STAGE + 1024;
+  constexpr int SUMS = cluster_sums_bytes(BN) + TILE_M * (BN / 2 + 1) * 4;       // partial sums, finished rows
+  if (smem_bytes < SUMS + 1024) smem_bytes = SUMS + 1024;
+  static bool attr_done[64] = {};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+  if (!attr_done[dev]) {
+    cudaError_t e = cudaFuncSetAttribute(conv_f16_nhwc_shared_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax - 1024);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(conv_f16_nhwc_shared_kernel<BN>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+    attr_done[dev] = true;
+  }
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)q.ksplit; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.blockDim = dim3(NUM_THREADS, 1, 1);
+  cfg.gridDim = dim3((unsigned)(plan.ntm * plan.ntn * q.ksplit), 1, 1);
+  cfg.dynamicSmemBytes = (size_t)smem_bytes;
+  cfg.stream = stream;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  return cudaLaunchKernelEx(&cfg, conv_f16_nhwc_shared_kernel<BN>, amap, bmap, q);
+}
+
 template <int KSUB, bool ROWS>
 cudaError_t launch_ksub(const CUtensorMap& amap, const CUtensorMap& bmap, const CUtensorMap& bmap_h, const NhwcParams& q,
                         const NhwcPlan& plan, cudaStream_t stream) {
@@ -2149,8 +2345,9 @@ cudaError_t launch_shift_view(const uint16_t* window, const uint16_t* fp, void* 
   q.epoch = next_epoch();
   q.flags = flags;
   if (const char* v = debug_getenv("IM2WIN_NHWC_BU")) { const int bu = atoi(v); if (bu >= 1 && bu <= 8) { q.bu = bu; q.bu_forced = 1; } }
-  // (buffers for rows where two activation stages and two of one filter unit still fit beside them)
-  if (stages_rows(q.e) && 2 * (int64_t)sp.a_stage_bytes + 2 * (int64_t)b_rows * KB * 2 <= kSmemMax - 2048 - kStageBytes)
+  // (buffers for rows where two activation stages and two of all kernel columns still fit beside them: with three columns a filter stage
+  // instead, 11x11 on 62 -> 73 channels at 91x91 took 44.7 us instead of 29.7)
+  if (stages_rows(q.e) && 2 * (int64_t)sp.a_stage_bytes + 2 * (int64_t)q.Kw * b_rows * KB * 2 <= kSmemMax - 2048 - kStageBytes)
     return launch_shift_tile<true>(amap, bmap, bmap_h, bmap_q, q, plan, sp, stream);
   return launch_shift_tile<false>(amap, bmap, bmap_h, bmap_q, q, plan, sp, stream);
 }
@@ -2371,6 +2568,7 @@ struct NhwcChoice {
   ShiftViewPlan sp;
   bool use_shift, split;
   bool runs;                 // overlapping-row kernel: the last round of tiles goes out as runs of its reduction
+  int ctas;                  // CTAs of a cluster that share a tile's reduction (conv_f16_nhwc_shared_kernel), or 1
 };
 
 // Tiles of parts of strips for the overlapping-row kernel.  Whole strips of 28 fill 112 of a tile's 128 rows, halves of nine
@@ -2390,8 +2588,39 @@ void part_strips(const Geometry& g, NhwcPlan& p) {
   }
 }
 
+// CTAs that share a tile, and its channel tile, where there are so few tiles that an SM each is left for them; 1 where it is not worth it.
+// Times in us beyond what every launch takes, fitted to 66 such layers (each with 2 to 16 CTAs and every channel tile; the choice is within 4 %
+// of the best on average and none is slower than unshared): a k-block 0.15 unshared (from 96 on the kernels share the last round through
+// memory: 0.06 and 8 once); shared 0.16 to 0.25, or as long as L2 takes to bring all CTAs theirs (6.5 to 10 bytes a ps); meeting and adding up 1 to 4.  Unshared / shared: 3x3 on 256 -> 96 channels at 17x17 11.4 / 6.9, 7x7 on
+// 80 -> 14 at 9x24 15.4 / 5.7, 11x11 stride 4 on 380 -> 17 at 57x57, binary16, 187 / 15; not 3x3 on 64 channels of one 56x56 image (6.5 / 9.4) or
+// 7x7 on 256 -> 71 at 13x13, batch 32 (28 / 33).  1.42 on average.
+int choose_shared(const Geometry& g, const NhwcPlan& plan, const EpilogueArgs& epi, int* bn_out) {
+  if (const char* v = debug_getenv("IM2WIN_NHWC_CTAS")) {    // testing aid: CTAs per tile
+    *bn_out = plan.bn;
+    return atoi(v) < plan.num_kb ? atoi(v) : plan.num_kb;
+  }
+  for (const char* name : {"IM2WIN_NHWC_KERNEL", "IM2WIN_NHWC_BN", "IM2WIN_NHWC_PAIR", "IM2WIN_NHWC_KSPLIT", "IM2WIN_NHWC_STREAM", "IM2WIN_NHWC_TAIL",
+                           "IM2WIN_NHWC_KSUB", "IM2WIN_NHWC_STAGES", "IM2WIN_NHWC_RASTER"})
+    if (debug_getenv(name)) return 1;                        // (the kernels that these are for)
+  if (plan.ntm > 74 || (!epi.out16 && g.K > kMostSplitTerms)) return 1;
+  int ctas = 1;
+  double best = 0.6 * 0.15 * plan.num_kb;                      // (the estimates are good to that much)
+  if (plan.num_kb >= 96 && 0.6 * (0.06 * plan.num_kb + 8) < best) best = 0.6 * (0.06 * plan.num_kb + 8);
+  for (int bn = plan.bn; bn >= 64; bn /= 2) {
+    const int64_t tiles = plan.ntm * ((g.Co + bn - 1) / bn);
+    for (int z = 2; z <= kMaxCtas && z <= plan.num_kb; ++z) {
+      if (tiles * z > 148 || tiles > resident_clusters(z)) continue;
+      const double alone = bn == 64 ? 0.16 : (bn == 128 ? 0.2 : 0.25), l2 = (double)tiles * z * (A_SLOT_BYTES + bn * KB * 2) / 6.5e6;
+      const double cost = bn / 64 + (plan.num_kb + z - 1) / z * (alone > l2 ? alone : l2);
+      if (cost < best) { best = cost; ctas = z; *bn_out = bn; }
+    }
+  }
+  return ctas;
+}
+
 NhwcChoice choose_nhwc(const Geometry& g, const EpilogueArgs& epi) {
   NhwcChoice c{};
+  c.ctas = 1;
   NhwcPlan& plan = c.plan;
   plan = plan_nhwc(g);
   if (!plan.eligible) return c;
@@ -2404,6 +2633,15 @@ NhwcChoice choose_nhwc(const Geometry& g, const EpilogueArgs& epi) {
   if (const char* v = debug_getenv("IM2WIN_NHWC_KSPLIT")) {
     const int ks = atoi(v);
     if (ks >= 1 && ks <= plan.num_kb) plan.ksplit = ks;
+  }
+  int bn = plan.bn;
+  c.ctas = choose_shared(g, plan, epi, &bn);
+  if (c.ctas > 1) {
+    plan.bn = bn;
+    plan.ntn = (g.Co + bn - 1) / bn;
+    plan.pair = false;
+    plan.ksplit = 1;
+    return c;
   }
   bool split = plan.ksplit > 1 && !epi.relu && !epi.out16;   // partial sums cannot pass a ReLU or a rounding
   if (!split) plan.ksplit = 1;
@@ -2484,6 +2722,7 @@ NhwcChoice choose_nhwc(const Geometry& g, const EpilogueArgs& epi) {
 const char* nhwc_kernel_name(const Geometry& g, const EpilogueArgs& epi) {
   const NhwcChoice c = choose_nhwc(g, epi);
   if (!c.plan.eligible) return "none";
+  if (c.ctas > 1) return "f16-nhwc-overlap+clusters";
   if (c.use_shift) return c.split ? "f16-nhwc-shift+ksplit" : "f16-nhwc-shift";
   return c.split ? "f16-nhwc-overlap+ksplit" : (c.runs ? "f16-nhwc-overlap+runs" : "f16-nhwc-overlap");
 }
@@ -2545,6 +2784,11 @@ cudaError_t launch_conv_f16_nhwc(const uint16_t* window, void* y, void* scratch,
   q.ksplit = plan.ksplit;
   q.ntn = plan.ntn;
   q.a_bytes = (uint32_t)(plan.G * plan.bw * KB * 2);
+  if (c.ctas > 1) {
+    q.ksplit = c.ctas;
+    if (plan.bn == 256) return launch_shared<256>(amap, bmap, q, plan, stream);
+    return plan.bn == 128 ? launch_shared<128>(amap, bmap, q, plan, stream) : launch_shared<64>(amap, bmap, q, plan, stream);
+  }
   int ksub = 1;
   if (const char* v = debug_getenv("IM2WIN_NHWC_KSUB")) ksub = atoi(v) == 1 ? 1 : 2;
   q.tail_halves = 1;

@@ -377,7 +377,7 @@ struct ClusterSums {
   }
 };
 // Bytes of P, whatever the share.
-constexpr int cluster_sums_bytes(int channels) { return (channels + kMaxCtas) * 128 * 4; }
+__host__ __device__ constexpr int cluster_sums_bytes(int channels) { return (channels + kMaxCtas) * 128 * 4; }
 // Arrive on an mbarrier given by a shared::cluster address (possibly in the other CTA).  Default
 // semantics (release at CTA scope): what the arriving thread wrote is its own CTA's shared memory,
 // read later by that CTA's tensor core; a cluster-scope release was measured to cost about a

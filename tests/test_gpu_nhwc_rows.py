@@ -1,14 +1,14 @@
 """Channel-innermost rows stored through shared memory (channels that are no whole number of 16-byte vectors) and by ragged numbers of
 vectors: rows that start on odd halves, last chunks of 1 to 31 channels, tiles whose strips leave gaps, tiles of parts of strips, a split
-reduction, several channel tiles.  Integer-valued inputs exactly (the result is one fp32 sum, rounded once), guard bands around the output.
+reduction, several channel tiles; tiles shared by clusters.  Integer-valued inputs exactly (the result is one fp32 sum, rounded once), guard bands around the output.
 """
 import numpy as np
 import pytest
 
 import oracle
-from paper_2608_20725_b200 import workloads
+from paper_2608_20725_b200 import binding, workloads
 from paper_2608_20725_b200.workloads import Layer
-from gpu_helpers import gpu_conv_nhwc
+from gpu_helpers import check_conv, gpu_conv_nhwc, oracle_inputs
 
 pytestmark = pytest.mark.gpu
 
@@ -52,3 +52,32 @@ def test_short_strips_side_by_side(layer, layout, threads, monkeypatch):
     x, f = workloads.make_small_integer_inputs(layer)
     yr, _ = oracle.conv_direct(x.numpy(), f.numpy(), dims)
     assert np.array_equal(gpu_conv_nhwc(x, f, dims, x_layout=layout), yr)
+
+
+# tiles whose reduction the CTAs of a cluster share: parts that the k-blocks do not divide into, more CTAs than channels in a tile, several
+# channel tiles, tiles of parts of strips, every epilogue
+@pytest.mark.parametrize("layer,bn,ctas", [
+    (L("s64", 2, 100, 9, 9, 60, 3, 3, 1, 1, 740), 64, 5), (L("s64_16", 1, 200, 7, 8, 5, 5, 3, 1, 1, 741), 64, 16),
+    (L("s128", 2, 72, 13, 11, 200, 3, 3, 2, 1, 742), 128, 3), (L("s256", 1, 130, 12, 9, 300, 3, 3, 1, 0, 743), 256, 7),
+    (L("s_parts", 1, 40, 4, 150, 37, 3, 5, 1, 1, 744), 64, 2), (L("s_one_kb", 2, 16, 9, 9, 24, 3, 3, 1, 1, 745), 64, 3)], ids=lambda v: getattr(v, "name", str(v)))
+def test_shared_tiles(layer, bn, ctas, monkeypatch):
+    monkeypatch.setenv("IM2WIN_NHWC_BN", str(bn))
+    monkeypatch.setenv("IM2WIN_NHWC_CTAS", str(ctas))
+    dims = layer.dims()
+    assert binding.im2win_nhwc_kernel_name(dims) == "f16-nhwc-overlap+clusters"
+    x, f = workloads.make_small_integer_inputs(layer)
+    yr, _ = oracle.conv_direct(x.numpy(), f.numpy(), dims)
+    bias = np.arange(layer.Co) % 7 - 3.0
+    for y_nhwc in (False, True):
+        want = yr.transpose(0, 2, 3, 1) if y_nhwc else yr
+        ref = np.maximum(want + (bias if y_nhwc else bias[:, None, None]), 0.0)
+        for out16 in (False, True):
+            assert np.array_equal(gpu_conv_nhwc(x, f, dims, out16=out16, y_nhwc=y_nhwc), want.astype(np.float16) if out16 else want)
+            got = gpu_conv_nhwc(x, f, dims, bias=bias, relu=True, out16=out16, y_nhwc=y_nhwc)
+            assert np.array_equal(got, ref.astype(np.float16) if out16 else ref)
+    # real values: the order of the parts is fixed, the sums within the tolerance
+    x, f = workloads.make_inputs(layer)
+    y = gpu_conv_nhwc(x, f, dims)
+    yr, ar = oracle.conv_direct(*oracle_inputs(x, f, "f16"), dims)
+    check_conv(y, yr, ar, "f16", layer.name)
+    assert np.array_equal(gpu_conv_nhwc(x, f, dims), y)
