@@ -296,7 +296,8 @@ im2win_status im2win_conv_packed_nhwc(const uint16_t* window, void* y, const im2
  * "f16-nhwc-overlap" (a tensor map with overlapping rows), with "+ksplit" when
  * every tile's reduction is split over several CTAs or "+runs" when the tiles
  * of a short last round are shared by runs of the reduction (decided for the
- * nominal 148 SMs; the launch decides for the device); "none" for a shape the
+ * nominal 148 SMs; the launch decides for the device) or "+clusters" when there
+ * are so few tiles that the CTAs of a cluster share each; "none" for a shape the
  * NHWC form does not take.  For reports and tests; the choice is an
  * implementation detail.
  */

@@ -881,8 +881,8 @@ conv_f16_nhwc_shared_kernel(const __grid_constant__ CUtensorMap amap, const __gr
         for (int c = h; c < mine; c += 2) put(base + (int64_t)c * e.HoWo, finish(c));
       }
     } else {
-      // through shared memory, so that the lanes lie along a row's channels (an element a lane and row: 8.1 -> 9.7 us on 3x3 stride 2, 82 -> 64
-      // channels at 95x95, and 17.6 -> 27.3 on 3x3 on 512 -> 512 at 16x16, batch 4)
+      // through shared memory, so that the lanes lie along a row's channels (3x3 on 512 -> 512 channels at 16x16, batch 4, shared by 8 CTAs:
+      // 22.3 us; an element a lane and row 27.3)
       float* rows = reinterpret_cast<float*>(smem + cluster_sums_bytes(BN));
       const int pitch = sums.per | 1;
       for (int c = h; c < mine; c += 2) rows[position * pitch + c] = finish(c);
@@ -2589,11 +2589,13 @@ void part_strips(const Geometry& g, NhwcPlan& p) {
 }
 
 // CTAs that share a tile, and its channel tile, where there are so few tiles that an SM each is left for them; 1 where it is not worth it.
-// Times in us beyond what every launch takes, fitted to 66 such layers (each with 2 to 16 CTAs and every channel tile; the choice is within 4 %
-// of the best on average and none is slower than unshared): a k-block 0.15 unshared (from 96 on the kernels share the last round through
-// memory: 0.06 and 8 once); shared 0.16 to 0.25, or as long as L2 takes to bring all CTAs theirs (6.5 to 10 bytes a ps); meeting and adding up 1 to 4.  Unshared / shared: 3x3 on 256 -> 96 channels at 17x17 11.4 / 6.9, 7x7 on
-// 80 -> 14 at 9x24 15.4 / 5.7, 11x11 stride 4 on 380 -> 17 at 57x57, binary16, 187 / 15; not 3x3 on 64 channels of one 56x56 image (6.5 / 9.4) or
-// 7x7 on 256 -> 71 at 13x13, batch 32 (28 / 33).  1.42 on average.
+// Times in us beyond what every launch takes, fitted to 66 such layers (each with 2 to 16 CTAs and every channel tile): a k-block 0.15 unshared
+// (from 96 on the kernels share the last round through memory: 0.06 and 8 once); shared 0.16 to 0.25, or as long as L2 takes to bring all CTAs
+// theirs (6.5 bytes a ps); meeting and adding up 1 to 4.  With 20 to 40 tiles, where L2 decides, and for channel-innermost outputs the estimate
+// is up to 1.6 times too good, so that it has to be 0.6 of the unshared one: without that margin 11 of 200 drawn layers lost 5 to 20 % (7x7 on
+// 128 -> 16 channels at 10x37, batch 8, 13.5 / 16.6, 11x11 on 64 -> 77 at 19x19, batch 32, 20.8 / 23.1), with it none of 300 more than 3 %.
+// Unshared / shared: 7x7 stride 4 on 163 -> 32 channels at 28x28, batch 2, 35.9 / 7.5, 3x3 stride 2 on 512 -> 28 at 15x15 22.5 / 6.4, 7x7 on
+// 512 -> 64 at 33x33, batch 8, 103 / 17.8.  3x3 on 64 channels of one 56x56 image stays unshared (6.5 / 9.4).
 int choose_shared(const Geometry& g, const NhwcPlan& plan, const EpilogueArgs& epi, int* bn_out) {
   if (const char* v = debug_getenv("IM2WIN_NHWC_CTAS")) {    // testing aid: CTAs per tile
     *bn_out = plan.bn;
