@@ -86,6 +86,22 @@ def test_unsupported_and_bad_dtype():
     assert e.value.code == 1
 
 
+@pytest.mark.parametrize("dtype", [-2, -1, 2, 7])
+def test_bad_dtype_of_a_layer_looked_up_before(dtype, monkeypatch):
+    """The sizes kept from earlier calls answer for the two precisions only."""
+    binding.lib()
+    monkeypatch.setattr(binding, "_debug", False)      # (with the testing aids on nothing is kept)
+    monkeypatch.setattr(binding, "_size_cache", {})
+    layer = dict(N=1, C=16, H=14, W=14, Co=16, Kh=3, Kw=3, stride=1, pad=1)
+    sizes = [binding.im2win_workspace_size(layer, code) for code in (binding.F32, binding.F16)]
+    assert len(binding._size_cache) == 1
+    for _ in range(2):
+        with pytest.raises(binding.Im2winError) as e:
+            binding.im2win_workspace_size(layer, dtype)
+        assert e.value.code == 1
+    assert [binding.im2win_workspace_size(layer, code) for code in (binding.F32, binding.F16)] == sizes
+
+
 def test_null_and_misaligned_pointers_rejected_before_launch():
     """These return before any CUDA call, so they are safe without a device."""
     lib = binding.lib()
