@@ -96,9 +96,10 @@ struct Segment {            // the part of a tile that lies in one image
 };
 
 // Programmatic dependent launch: the convolution kernel is launched so that it may start while
-// the filter pack (the kernel before it in the stream) is still running; its barrier setup, tensor
-// memory allocation and descriptor fetches overlap the pack.  Every role that touches global memory
-// first waits for the preceding kernel to have completed (and its writes to be visible).
+// the filter pack (the kernel before it in the stream) is still running; its barrier setup and tensor
+// memory allocation overlap the pack.  Then every thread waits for the preceding kernel to have completed
+// (and its writes to be visible).  (The MMA and re-layout warps too, which touch no tensor: a bounded wait
+// that is not over at once reads its limit from the status block, and that is cleared by the pack.)
 // (let_next_kernel_start in the pack, wait_for_previous_kernel here.)
 
 // Splits the rows of the tile starting at virtual position q0 by image: within an image the
@@ -204,6 +205,7 @@ __device__ __forceinline__ void conv_f16_mat_body(const CUtensorMap& fmap, const
   if (PAIR) cluster_sync_all();               // the peer's barriers exist before anything arrives on them
   tc_fence_after();
   const uint32_t tmem_acc = tmem_base_slot;
+  wait_for_previous_kernel();
   // where this CTA's arrivals for the MMA issuer go: the leader's barriers
   const uint32_t a_full_dst = PAIR ? mapa_shared(a_full0, 0) : a_full0;
   const uint32_t b_full_dst = PAIR ? mapa_shared(b_full0, 0) : b_full0;
@@ -396,7 +398,6 @@ __device__ __forceinline__ void conv_f16_mat_body(const CUtensorMap& fmap, const
     if (threadIdx.x == 0) TIMER_FLUSH();
   } else if (warp == WARP_TMA) {
     // ---------------- TMA loader of the filter tiles ---------------------------
-    wait_for_previous_kernel();
     const bool leader = elect_one();
     bool ok = true;
     int st = 0;
@@ -520,7 +521,6 @@ __device__ __forceinline__ void conv_f16_mat_body(const CUtensorMap& fmap, const
     // two warps share the boxes of a stage (even / odd): issuing a copy costs a few hundred
     // cycles and the stage is only complete when its last box has been requested
     const int half = warp - WARP_RAW;
-    wait_for_previous_kernel();
     const bool leader = elect_one();
     bool ok = true;
     int rst = 0;
@@ -558,7 +558,6 @@ __device__ __forceinline__ void conv_f16_mat_body(const CUtensorMap& fmap, const
   } else if (warp >= WARP_EPI0) {
     // ---------------- epilogue: tensor memory -> NCHW output --------------------
     const int lq = warp & 3;                     // tensor-memory lane quadrant this warp may read
-    wait_for_previous_kernel();                  // before the first store to y
     bool ok = true;
     uint32_t it = 0;
     for (int w = w_first; w < q.nwork && ok; w += w_step, ++it) {

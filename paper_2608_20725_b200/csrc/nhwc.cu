@@ -93,10 +93,11 @@ struct NhwcParams {
   uint32_t epoch;
 };
 
-// Programmatic dependent launch: the convolution may start while the kernel before it in the stream
-// (the filter pack) is still running, so that its barrier set-up, tensor-memory allocation and
-// descriptor fetches overlap that kernel; every role that touches global memory first waits for the
-// preceding kernel to have completed.
+// Programmatic dependent launch: the convolution may start while the kernels before it in the stream
+// (the filter pack, which itself waits for the transform) are still running, so that its barrier set-up and
+// tensor-memory allocation overlap them; then every thread waits for the preceding kernel to have completed.
+// (The MMA warps too, which touch no tensor: a bounded wait that is not over at once reads its limit from the
+// status block, and that is cleared by the pack.)
 
 __device__ __forceinline__ void red_add_f32(float* p, float v) {
   asm volatile("red.global.add.f32 [%0], %1;" ::"l"(p), "f"(v) : "memory");
@@ -510,6 +511,7 @@ __device__ __forceinline__ void conv_nhwc_body(const CUtensorMap& amap, const CU
   if (PAIR) cluster_sync_all();               // the peer's barriers exist before anything arrives on them
   tc_fence_after();
   const uint32_t tmem_acc = tmem_base_slot;
+  wait_for_previous_kernel();
   const uint32_t full_dst = PAIR ? mapa_shared(full0, 0) : full0;          // the leader's barriers
   const uint32_t acc_empty_dst = PAIR ? mapa_shared(acc_empty0, 0) : acc_empty0;
 
@@ -520,7 +522,6 @@ __device__ __forceinline__ void conv_nhwc_body(const CUtensorMap& amap, const CU
     // ---------------- copies of both operands ------------------------------------
     {
       const bool leader = elect_one();
-      wait_for_previous_kernel();                // the filter pack (and everything before it) is complete
       int st = 0;
       uint32_t ph = 0;
       bool ok = true;
@@ -644,7 +645,6 @@ __device__ __forceinline__ void conv_nhwc_body(const CUtensorMap& amap, const CU
     const EpiParams& e = q.e;
     const bool vec_ok = e.out16 ? (e.Co % 8 == 0) : (e.Co % 4 == 0);
     const uint32_t stage = ROWS ? smem_u32(smem) + e.stage_off + (warp - WARP_EPI0) * (32 * ROW_PITCH) : 0u;
-    wait_for_previous_kernel();                  // before the first store to y
     float breg[32];
     const bool hoisted = hoist_bias<BN>(e, q.ntn, warp, breg);
     bool ok = true;
@@ -1049,6 +1049,7 @@ __device__ __forceinline__ void conv_shift_body(const CUtensorMap& amap, const C
   if (PAIR) cluster_sync_all();
   tc_fence_after();
   const uint32_t tmem_acc = tmem_base_slot;
+  wait_for_previous_kernel();
   const uint32_t a_full_dst = PAIR ? mapa_shared(a_full0, 0) : a_full0;     // the leader's barriers
   const uint32_t b_full_dst = PAIR ? mapa_shared(b_full0, 0) : b_full0;
   const uint32_t acc_empty_dst = PAIR ? mapa_shared(acc_empty0, 0) : acc_empty0;
@@ -1060,7 +1061,6 @@ __device__ __forceinline__ void conv_shift_body(const CUtensorMap& amap, const C
     {
       const bool leader = elect_one();
       const int ncls = q.s < q.Kw ? q.s : q.Kw;   // column classes some kernel column reads
-      wait_for_previous_kernel();
       // with two issuing warps the ring is two rings of half the stages: even items fill one, odd items the other
       const int nst = q.dual ? q.sa / 2 : q.sa;
       int st_even = 0, st_odd = 0;             // (scalars, not an array indexed by the ring: that would live in local memory)
@@ -1107,7 +1107,6 @@ __device__ __forceinline__ void conv_shift_body(const CUtensorMap& amap, const C
     // ---------------- filter copies: bu (k2-block, kernel column) units per stage ----
     {
       const bool leader = elect_one();
-      wait_for_previous_kernel();
       int st = 0;
       uint32_t ph = 0;
       bool ok = true;
@@ -1313,7 +1312,6 @@ __device__ __forceinline__ void conv_shift_body(const CUtensorMap& amap, const C
     const EpiParams& e = q.e;
     const bool vec_ok = e.out16 ? (e.Co % 8 == 0) : (e.Co % 4 == 0);
     const uint32_t stage = ROWS ? smem_u32(smem) + e.stage_off + (warp - WARP_EPI0) * (32 * ROW_PITCH) : 0u;
-    wait_for_previous_kernel();
     // HOIST (64-channel tiles, one channel tile, a bias): the warp's 32 bias values stay in registers.  A
     // kernel of its own: the same choice taken at run time cost the stems without a bias 8-15 %.
     float breg[HOIST ? 32 : 1];

@@ -1,0 +1,52 @@
+"""Kernels that may start before the one ahead of them in the stream has ended (launch_early, launch_after_previous, or the launch
+attribute itself): every thread waits for that one before anything else that reads what it wrote.  A bounded barrier wait counts: its
+slow path takes its limit from the status block, which the filter pack clears, so that a wait that came first could give up on a
+word left over from whatever the memory held before, and the pack would then clear the status that says so.
+
+Read from the sources: the outcome of such a wait depends on what happens to be in memory.  No GPU needed."""
+import os
+import re
+
+import pytest
+
+from paper_2608_20725_b200 import build
+
+EARLY = re.compile(r"launch_early\(|launch_after_previous\(|cudaLaunchAttributeProgrammaticStreamSerialization")
+HEAD = re.compile(r"^(?:__global__ void\b.*|__device__ __forceinline__ void \w+_body\(.*|conv_\w+_kernel\(.*)$", re.M)
+
+
+def bodies(code):
+    """(head, body) of every kernel and of every function that is one in all but its launch."""
+    at = 0
+    while (m := HEAD.search(code, at)) is not None:
+        start = code.index("{", m.start())
+        depth, end = 1, start + 1
+        while depth:
+            depth += {"{": 1, "}": -1}.get(code[end], 0)
+            end += 1
+        yield code[m.start():start], code[start + 1:end - 1]
+        at = end
+
+
+def kernels_that_wait():
+    for path in build.sources():
+        code = re.sub(r"//[^\n]*", "", open(path).read())
+        if EARLY.search(code):
+            for head, body in bodies(code):
+                if "mbar_wait" in body or "wait_flag(" in body or "wait_for_previous_kernel()" in body:
+                    yield pytest.param(body, id=f"{os.path.basename(path)}:{re.findall(r'(\w+)\s*[(]', head.replace('__launch_bounds__', ''))[-1]}")
+
+
+@pytest.mark.parametrize("body", list(kernels_that_wait()))
+def test_every_thread_waits_first(body):
+    at = body.find("wait_for_previous_kernel()")
+    assert at >= 0, "no wait for the kernel ahead"
+    before = body[:at]
+    assert "mbar_wait" not in before and "wait_flag(" not in before, "a bounded wait comes first"
+    assert before.count("{") == before.count("}"), "inside a branch or a loop: not every thread comes by"
+
+
+def test_the_kernels_are_found():
+    """The ones that start early and have waits: seven convolutions and seven filter packs."""
+    ids = [p.id for p in kernels_that_wait()]
+    assert len(ids) == len(set(ids)) == 14, ids
