@@ -317,6 +317,11 @@ int32_t im2win_f16_tile_ctas(const im2win_shape* shape) {
   return l.f16_shift && !l.f16_stem && !l.f16_mat && !l.f16_raw ? plan_f16_shift(g).split : 1;
 }
 
+// The same: CTAs of a cluster that a launcher takes for `want`, on a device that holds resident[z] clusters of z CTAs.
+int32_t im2win_widest_cluster(int32_t want, const int32_t resident[17]) {
+  return widest_cluster(want, [&](int z) { return resident[z] > 0; });
+}
+
 // The same for the fp32 tensor-core kernel: channel tile, CTAs of a tile, parts of the last round's tiles.
 int32_t im2win_f32_split_form(const im2win_shape* shape, int32_t form[3]) {
   Geometry g;

@@ -30,6 +30,7 @@ struct Geometry {
 // Clusters of z CTAs, each CTA an SM to itself, that a B200 holds at once: they lie within a GPC, so that wide ones leave SMs over.
 // (What cudaOccupancyMaxActiveClusters says of 226 KB of shared memory a CTA; 16 clusters of 8 CTAs run in two rounds: 7x7 on
 // 256 -> 78 channels at 35x35, batch 2, 87 us in clusters of 8, 47 in clusters of 4.)
+// The plans go by this table, so that they do not depend on the machine; the launchers ask the device (ctas_that_fit).
 constexpr int kMaxCtas = 16;       // of a cluster (above 8: the non-portable sizes)
 // Longest reduction of an fp16 layer whose tiles are shared.  An accumulator truncates every addend, 1e-9 of the sum a term,
 // so a shared reduction is the more exact one; beyond this the two would differ by more than fp32 sums in another order do.
@@ -37,6 +38,14 @@ constexpr int64_t kMostSplitTerms = 16384;
 inline int resident_clusters(int z) {
   constexpr int kResident[kMaxCtas + 1] = {0, 148, 74, 45, 33, 26, 22, 15, 15, 15, 11, 7, 7, 7, 7, 7, 7};
   return z >= 1 && z <= kMaxCtas ? kResident[z] : 0;
+}
+
+// The most CTAs up to `want` whose cluster fits (a function of their number), 1 where none of two or more does.
+template <typename Fits>
+int widest_cluster(int want, const Fits& fits) {
+  for (int z = want; z > 1; --z)
+    if (fits(z)) return z;
+  return 1;
 }
 
 // Scratch layout shared by both precisions (offsets in bytes from `scratch`):

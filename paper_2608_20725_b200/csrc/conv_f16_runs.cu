@@ -972,7 +972,13 @@ cudaError_t launch_mode(const RunsParams& q, int smem, cudaStream_t stream) {
     if (e != cudaSuccess) return e;
     attr_done[dev] = true;
   }
-  if (SPLIT) return launch_after_previous(kernel, q.nwork * q.split, q.split, THREADS, smem, stream, q);
+  if constexpr (SPLIT) {
+    static KnownClusters known;
+    RunsParams shared = q;
+    shared.split = ctas_that_fit(kernel, q.split, THREADS, kRunsSmem, known);
+    if (shared.split == 1) return launch_mode<BNMAX, PAIR, MODE, false>(shared, smem, stream);
+    return launch_after_previous(kernel, shared.nwork * shared.split, shared.split, THREADS, smem, stream, shared);
+  }
   const int most = PAIR ? 74 : 148, grid = (q.nwork < most ? q.nwork : most) * (PAIR ? 2 : 1);
   return launch_after_previous(kernel, grid, PAIR ? 2 : 1, THREADS, smem, stream, q);
 }

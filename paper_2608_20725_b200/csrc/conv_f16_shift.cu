@@ -466,11 +466,11 @@ cudaError_t launch_variant(const CUtensorMap& fmap, const ShiftParams& q0, const
   q.sb = sb;
   int smem_bytes = sa * q.a_stage_bytes + sb * BN * KB * 2 + (int)plan.K2p * 4 + 1024;
   if (SPLIT && smem_bytes < cluster_sums_bytes(BN) + 1024) smem_bytes = cluster_sums_bytes(BN) + 1024;
-  cudaError_t e = cudaFuncSetAttribute(conv_f16_shift_kernel<BN, ITEMS, SPLIT>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
-  if (e == cudaSuccess && SPLIT)
-    e = cudaFuncSetAttribute(conv_f16_shift_kernel<BN, ITEMS, SPLIT>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-  if (e != cudaSuccess) return e;
+  if constexpr (!SPLIT) {
+    const cudaError_t e = cudaFuncSetAttribute(conv_f16_shift_kernel<BN, ITEMS, SPLIT>,
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
+    if (e != cudaSuccess) return e;
+  }
   const int64_t units = (plan.VQ + TILE_M - 1) / TILE_M;
   const dim3 grid((unsigned)((units - q.nbig) * q.split), (unsigned)((co + BN - 1) / BN));   // a tall tile covers two units
   if constexpr (SPLIT) {
@@ -490,6 +490,26 @@ cudaError_t launch_variant(const CUtensorMap& fmap, const ShiftParams& q0, const
   } else {
     return launch_early(conv_f16_shift_kernel<BN, ITEMS, SPLIT>, grid, NUM_THREADS, (size_t)smem_bytes, stream, fmap, q);
   }
+}
+
+// The shared form, in clusters of q.split CTAs or as many as fit; *alone: not even two do, and nothing was launched.
+template <int BN, int ITEMS>
+cudaError_t launch_shared(const CUtensorMap& fmap, ShiftParams q, const ShiftPlan& plan, int co, cudaStream_t stream, bool* alone) {
+  constexpr auto kernel = conv_f16_shift_kernel<BN, ITEMS, true>;
+  static_assert(cluster_sums_bytes(256) + 1024 <= kSmemBudget, "kSmemBudget is the most a launch takes");
+  static bool attr_done[64] = {};
+  static KnownClusters known;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+  if (!attr_done[dev]) {
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+    attr_done[dev] = true;
+  }
+  q.split = ctas_that_fit(kernel, q.split, NUM_THREADS, kSmemBudget, known);
+  *alone = q.split == 1;
+  return *alone ? cudaSuccess : launch_variant<BN, ITEMS, true>(fmap, q, plan, co, stream);
 }
 
 // Number of 256-position tiles: whole waves of tall tiles while two units per slot remain, and
@@ -515,9 +535,12 @@ cudaError_t launch_bn(const CUtensorMap& fmap, const ShiftParams& q0, const Shif
   ShiftParams q = q0;
   const int64_t units = (plan.VQ + TILE_M - 1) / TILE_M;
   if (q.split > 1) {
-    if (plan.items <= 5) return launch_variant<BN, 5, true>(fmap, q, plan, co, stream);
-    if (plan.items <= 10) return launch_variant<BN, 10, true>(fmap, q, plan, co, stream);
-    return launch_variant<BN, 15, true>(fmap, q, plan, co, stream);
+    bool alone = false;
+    const cudaError_t e = plan.items <= 5    ? launch_shared<BN, 5>(fmap, q, plan, co, stream, &alone)
+                          : plan.items <= 10 ? launch_shared<BN, 10>(fmap, q, plan, co, stream, &alone)
+                                             : launch_shared<BN, 15>(fmap, q, plan, co, stream, &alone);
+    if (!alone) return e;
+    q.split = 1;
   }
   q.nbig = choose_nbig(units, (co + BN - 1) / BN, BN <= 128 ? 2 : 1, q.Kw);
   const int mt = q.nbig > 0 ? 2 : 1;

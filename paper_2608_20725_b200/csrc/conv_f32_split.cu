@@ -714,8 +714,9 @@ int channel_parts(int64_t tiles, int bn) {
 }
 
 template <int BNMAX, int PWG>
-cudaError_t launch_form(const SplitParams& q, int smem, cudaStream_t stream) {
+cudaError_t launch_form(SplitParams q, int smem, cudaStream_t stream) {
   static bool attr_done[64] = {};
+  static KnownClusters known;
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
   if (!attr_done[dev]) {
@@ -724,6 +725,7 @@ cudaError_t launch_form(const SplitParams& q, int smem, cudaStream_t stream) {
     if (e != cudaSuccess) return e;
     attr_done[dev] = true;
   }
+  if (q.split > 1) q.split = ctas_that_fit(conv_f32_split_kernel<BNMAX, PWG>, q.split, Form<BNMAX, PWG>::THREADS, kSplitSmem, known);
   const int grid = q.split > 1 ? q.nwork * q.split : (q.nwork < 148 ? q.nwork : 148);
   return launch_after_previous(conv_f32_split_kernel<BNMAX, PWG>, grid, q.split, Form<BNMAX, PWG>::THREADS, smem, stream, q);
 }

@@ -2048,8 +2048,26 @@ cudaError_t launch_variant(const CUtensorMap& amap, const CUtensorMap& bmap, con
   return cudaLaunchKernelEx(&cfg, conv_f16_nhwc_kernel<BN, KSUB, ROWS>, amap, bmap, bmap_h, q);
 }
 
+// CTAs of a cluster that may share a tile on this device, for the `want` of the plan (1: none).
+template <int BN>
+cudaError_t shared_ctas(int want, int* ctas) {
+  static bool attr_done[64] = {};
+  static KnownClusters known;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+  if (!attr_done[dev]) {
+    cudaError_t e = cudaFuncSetAttribute(conv_f16_nhwc_shared_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax - 1024);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(conv_f16_nhwc_shared_kernel<BN>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+    attr_done[dev] = true;
+  }
+  *ctas = ctas_that_fit(conv_f16_nhwc_shared_kernel<BN>, want, NUM_THREADS, kSmemMax - 1024, known);
+  return cudaSuccess;
+}
+
 template <int BN>
 cudaError_t launch_shared(const CUtensorMap& amap, const CUtensorMap& bmap, NhwcParams q, const NhwcPlan& plan, cudaStream_t stream) {
+  // (the device holds clusters of q.ksplit CTAs: shared_ctas)
   constexpr int STAGE = A_SLOT_BYTES + BN * KB * 2;
   int stages = (kSmemMax - 2048) / STAGE;
   if (stages > MAX_STAGES) stages = MAX_STAGES;
@@ -2059,15 +2077,6 @@ cudaError_t launch_shared(const CUtensorMap& amap, const CUtensorMap& bmap, Nhwc
   int smem_bytes = stages * STAGE + 1024;
   constexpr int SUMS = cluster_sums_bytes(BN) + TILE_M * (BN / 2 + 1) * 4;       // partial sums, finished rows
   if (smem_bytes < SUMS + 1024) smem_bytes = SUMS + 1024;
-  static bool attr_done[64] = {};
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-  if (!attr_done[dev]) {
-    cudaError_t e = cudaFuncSetAttribute(conv_f16_nhwc_shared_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax - 1024);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(conv_f16_nhwc_shared_kernel<BN>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess) return e;
-    attr_done[dev] = true;
-  }
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -2618,7 +2627,8 @@ int choose_shared(const Geometry& g, const NhwcPlan& plan, const EpilogueArgs& e
   return ctas;
 }
 
-NhwcChoice choose_nhwc(const Geometry& g, const EpilogueArgs& epi) {
+// (may_share: whether the device holds the clusters that choose_shared asks for)
+NhwcChoice choose_nhwc(const Geometry& g, const EpilogueArgs& epi, bool may_share = true) {
   NhwcChoice c{};
   c.ctas = 1;
   NhwcPlan& plan = c.plan;
@@ -2635,7 +2645,7 @@ NhwcChoice choose_nhwc(const Geometry& g, const EpilogueArgs& epi) {
     if (ks >= 1 && ks <= plan.num_kb) plan.ksplit = ks;
   }
   int bn = plan.bn;
-  c.ctas = choose_shared(g, plan, epi, &bn);
+  if (may_share) c.ctas = choose_shared(g, plan, epi, &bn);
   if (c.ctas > 1) {
     plan.bn = bn;
     plan.ntn = (g.Co + bn - 1) / bn;
@@ -2729,8 +2739,14 @@ const char* nhwc_kernel_name(const Geometry& g, const EpilogueArgs& epi) {
 
 cudaError_t launch_conv_f16_nhwc(const uint16_t* window, void* y, void* scratch, const Geometry& g,
                                  const EpilogueArgs& epi, cudaStream_t stream) {
-  const NhwcChoice c = choose_nhwc(g, epi);
+  NhwcChoice c = choose_nhwc(g, epi);
   if (!c.plan.eligible) return cudaErrorInvalidValue;
+  if (c.ctas > 1) {
+    const int bn = c.plan.bn;
+    const cudaError_t e = bn == 256 ? shared_ctas<256>(c.ctas, &c.ctas) : (bn == 128 ? shared_ctas<128>(c.ctas, &c.ctas) : shared_ctas<64>(c.ctas, &c.ctas));
+    if (e != cudaSuccess) return e;
+    if (c.ctas == 1) c = choose_nhwc(g, epi, false);
+  }
   const NhwcPlan& plan = c.plan;
   const ShiftViewPlan& sp = c.sp;
   const bool use_shift = c.use_shift, split = c.split;
