@@ -1,7 +1,10 @@
 """Channel-innermost rows stored through shared memory (channels that are no whole number of 16-byte vectors) and by ragged numbers of
-vectors: rows that start on odd halves, last chunks of 1 to 31 channels, tiles whose strips leave gaps, tiles of parts of strips, a split
-reduction, several channel tiles; tiles shared by clusters.  Integer-valued inputs exactly (the result is one fp32 sum, rounded once), guard bands around the output.
+vectors: rows that start on odd halves, last chunks of 1 to 31 channels, tiles whose strips leave gaps, tiles of parts of strips, several
+channel tiles, a short last round whose tiles several CTAs share; tiles shared by clusters.  Integer-valued inputs exactly (the result is one
+fp32 sum, rounded once), guard bands around the output.
 """
+import functools
+
 import numpy as np
 import pytest
 
@@ -37,6 +40,40 @@ def test_rows_of_any_number_of_channels(layer, kernel, monkeypatch):
         got = gpu_conv_nhwc(x, f, dims, bias=bias, relu=True, out16=out16, y_nhwc=True)
         ref = np.maximum(want + bias, 0.0)
         assert np.array_equal(got, ref.astype(np.float16) if out16 else ref)
+
+
+# Rows that meet other CTAs: 78 tile items on 74 CTA pairs, with a reduction long enough that the four tiles of the last round are shared
+# between CTAs.  Overlapping rows (98 k-blocks): runs of the reduction, whose partial sums the storing CTA adds up, or halves of the
+# channels; shifted views (32 k2-blocks x 3 kernel columns, streamed): K parts, of which the first stores its rows and the others add to
+# them (fp32 outputs without ReLU), or quarters of the channels.
+SHORT_LAST_ROUND = {"overlap": L("last_overlap", 13, 128, 24, 26, 301, 7, 7, 1, 3, 713), "shift": L("last_shift", 13, 285, 28, 30, 301, 7, 3, 1, 1, 714)}
+
+
+@functools.lru_cache(maxsize=None)
+def short_last_round(kernel):
+    layer = SHORT_LAST_ROUND[kernel]
+    x, f = workloads.make_small_integer_inputs(layer)
+    yr, _ = oracle.conv_direct(x.numpy(), f.numpy(), layer.dims())
+    return x, f, yr.transpose(0, 2, 3, 1)
+
+
+@pytest.mark.parametrize("kernel,switches", [
+    ("overlap", {}), ("overlap", {"IM2WIN_NHWC_STREAM": "0"}), ("overlap", {"IM2WIN_NHWC_TAIL": "0"}),
+    ("shift", {}), ("shift", {"IM2WIN_NHWC_TAIL_K": "0"}), ("shift", {"IM2WIN_NHWC_TAIL": "0"})],
+    ids=["runs", "halves", "overlap_whole", "k_parts", "channel_parts", "shift_whole"])
+def test_rows_of_a_short_last_round(kernel, switches, monkeypatch):
+    monkeypatch.setenv("IM2WIN_NHWC_KERNEL", kernel)
+    monkeypatch.setenv("IM2WIN_NHWC_KSPLIT", "1")
+    for k, v in switches.items():
+        monkeypatch.setenv(k, v)
+    x, f, want = short_last_round(kernel)
+    dims = SHORT_LAST_ROUND[kernel].dims()
+    bias = np.arange(dims["Co"]) % 7 - 3.0
+    assert np.abs(want).max() + 3 < 2048                     # (whole numbers that binary16 holds)
+    for out16 in (False, True):
+        assert np.array_equal(gpu_conv_nhwc(x, f, dims, out16=out16, y_nhwc=True, packed=True, repeat=3), want)
+        assert np.array_equal(gpu_conv_nhwc(x, f, dims, bias=bias, out16=out16, y_nhwc=True), want + bias)
+        assert np.array_equal(gpu_conv_nhwc(x, f, dims, bias=bias, relu=True, out16=out16, y_nhwc=True), np.maximum(want + bias, 0.0))
 
 
 # the transform's strips side by side in a block: short ones, a last block that is not full, channels by 8, 4, 2 and 1
