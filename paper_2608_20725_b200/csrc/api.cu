@@ -322,6 +322,9 @@ int32_t im2win_widest_cluster(int32_t want, const int32_t resident[17]) {
   return widest_cluster(want, [&](int z) { return resident[z] > 0; });
 }
 
+// The same: shared memory of a block of `threads` that an early launch of `blocks` asks for, which needs `smem`.
+int64_t im2win_spread_smem(int64_t blocks, int32_t threads, int64_t smem) { return (int64_t)spread_smem(blocks, threads, (size_t)smem); }
+
 // The same for the fp32 tensor-core kernel: channel tile, CTAs of a tile, parts of the last round's tiles.
 int32_t im2win_f32_split_form(const im2win_shape* shape, int32_t form[3]) {
   Geometry g;

@@ -48,6 +48,17 @@ int widest_cluster(int want, const Fits& fits) {
   return 1;
 }
 
+// Shared memory with which an SM takes no more of `blocks` blocks than its share.  Blocks that are launched early go to the SMs that the kernel
+// ahead leaves first, as many to an SM as it holds, and crowd there while others idle.  (226 KB of an SM, 1 KB a block is the system's.)
+constexpr int kMostSpread = 200 * 1024;
+inline size_t spread_smem(int64_t blocks, int threads, size_t smem) {
+  const int64_t share = (blocks + 147) / 148;
+  if (share >= 2048 / threads) return smem;
+  int64_t spread = (226 * 1024 / share - 1024) / 128 * 128;
+  if (spread > kMostSpread) spread = kMostSpread;
+  return (int64_t)smem < spread ? (size_t)spread : smem;
+}
+
 // Scratch layout shared by both precisions (offsets in bytes from `scratch`):
 //   [0, 256)            status block (uint32 words; word 0 = timeout flag)
 //   [256, 256 + 4*Kp)   k -> element offset table (int32), -1 for padded k

@@ -466,13 +466,17 @@ cudaError_t launch_variant(const CUtensorMap& fmap, const ShiftParams& q0, const
   q.sb = sb;
   int smem_bytes = sa * q.a_stage_bytes + sb * BN * KB * 2 + (int)plan.K2p * 4 + 1024;
   if (SPLIT && smem_bytes < cluster_sums_bytes(BN) + 1024) smem_bytes = cluster_sums_bytes(BN) + 1024;
+  const int64_t units = (plan.VQ + TILE_M - 1) / TILE_M;
+  const dim3 grid((unsigned)((units - q.nbig) * q.split), (unsigned)((co + BN - 1) / BN));   // a tall tile covers two units
+  // An SM each where there is one for every tile, also where an SM could take two (spread_smem): 7x7 on 512 -> 116 channels, one 112x112 image,
+  // 221 us in twos, 169 alone; 7x5 on 128 -> 40 at 117x117 57.5 and 47.2.
+  const int64_t ctas = (int64_t)grid.x * grid.y;
+  if (!SPLIT && ctas <= 148) smem_bytes = (int)spread_smem(ctas, NUM_THREADS, (size_t)smem_bytes);
   if constexpr (!SPLIT) {
     const cudaError_t e = cudaFuncSetAttribute(conv_f16_shift_kernel<BN, ITEMS, SPLIT>,
                                                cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
     if (e != cudaSuccess) return e;
   }
-  const int64_t units = (plan.VQ + TILE_M - 1) / TILE_M;
-  const dim3 grid((unsigned)((units - q.nbig) * q.split), (unsigned)((co + BN - 1) / BN));   // a tall tile covers two units
   if constexpr (SPLIT) {
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[2];

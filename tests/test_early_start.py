@@ -4,12 +4,13 @@ slow path takes its limit from the status block, which the filter pack clears, s
 word left over from whatever the memory held before, and the pack would then clear the status that says so.
 
 Read from the sources: the outcome of such a wait depends on what happens to be in memory.  No GPU needed."""
+import ctypes
 import os
 import re
 
 import pytest
 
-from paper_2608_20725_b200 import build
+from paper_2608_20725_b200 import binding, build
 
 EARLY = re.compile(r"launch_early\(|launch_after_previous\(|cudaLaunchAttributeProgrammaticStreamSerialization")
 HEAD = re.compile(r"^(?:__global__ void\b.*|__device__ __forceinline__ void \w+_body\(.*|conv_\w+_kernel\(.*)$", re.M)
@@ -50,3 +51,16 @@ def test_the_kernels_are_found():
     """The ones that start early and have waits: seven convolutions and seven filter packs."""
     ids = [p.id for p in kernels_that_wait()]
     assert len(ids) == len(set(ids)) == 14, ids
+
+
+@pytest.mark.parametrize("threads,smem", [(256, 0), (256, 5000), (256, 47000), (256, 190000), (320, 90000)])
+def test_early_blocks_are_spread_over_the_sms(threads, smem):
+    """An SM (228 KB, 1 KB of them for each block) takes its share of the blocks and no more, or what it took anyway if that is less."""
+    fn = binding.lib().im2win_spread_smem
+    fn.argtypes, fn.restype = [ctypes.c_int64, ctypes.c_int32, ctypes.c_int64], ctypes.c_int64
+    anyway = min(2048 // threads, 228 * 1024 // (smem + 1024))
+    for blocks in [1, 2, 74, 147, 148, 149, 296, 297, 443, 444, 592, 740, 741, 888, 1036, 1037, 1184, 1185, 5000]:
+        asked = fn(blocks, threads, smem)
+        share = (blocks + 147) // 148
+        assert smem <= asked <= max(smem, 200 * 1024)
+        assert min(2048 // threads, 228 * 1024 // (asked + 1024)) == min(share, anyway)
