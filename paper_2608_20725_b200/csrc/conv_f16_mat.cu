@@ -917,7 +917,7 @@ cudaError_t launch_pack_f16_mat(const uint16_t* filter, void* scratch, const Geo
   const size_t smem = ((size_t)noct * 8 * g.T + 16) * sizeof(uint16_t);
   if (smem > 48 * 1024) return cudaErrorInvalidValue;
   dim3 grid((unsigned)((plan.Cp8 + noct - 1) / noct), (unsigned)(ncog * 64 < 32768 ? ncog * 64 : 32768));
-  return launch_early(pack_f16_mat_kernel, grid, 256, smem, stream, filter, fp, reinterpret_cast<uint32_t*>(base), g.C, g.Co, g.Kh, g.Kw,
+  return launch_pack<pack_f16_mat_kernel>(grid, 256, smem, stream, filter, fp, reinterpret_cast<uint32_t*>(base), g.C, g.Co, g.Kh, g.Kw,
                                                    (int)plan.K2p, ncog, noct);
 }
 

@@ -1167,7 +1167,7 @@ cudaError_t launch_pack_f16_runs(const uint16_t* filter, void* scratch, const Ge
   while (rows > 1 && (rows * pitch * ES > 40 * 1024 || (int64_t)p.ntn * p.bn / rows * p.num_kb < 2 * 148)) rows /= 2;
   const size_t smem = (size_t)(rows * pitch * ES);
   dim3 grid((unsigned)(p.ntn * p.bn / rows), (unsigned)p.num_kb);   // (num_kb <= 2^14: C * E <= 2^20)
-  return launch_early(pack_f16_runs_kernel, grid, 256, smem, stream, filter, base + kStatusBytes, reinterpret_cast<uint32_t*>(base), g.C, g.Kh, g.Kw,
+  return launch_pack<pack_f16_runs_kernel>(grid, 256, smem, stream, filter, base + kStatusBytes, reinterpret_cast<uint32_t*>(base), g.C, g.Kh, g.Kw,
                                                     g.s, p.E, p.G, g.Co, p.bn, p.num_kb, rows, (int)pitch, p.quad);
 }
 

@@ -818,7 +818,7 @@ cudaError_t launch_pack_f32_split(const float* filter, void* scratch, const Geom
   while (rows > 1 && ((size_t)rows * KB * g.Kw * 4 > 40 * 1024 || (int64_t)p.ntn * p.bn / rows * p.num_kb < 2 * 148)) rows /= 2;
   const size_t smem = (size_t)rows * KB * g.Kw * 4;
   dim3 grid((unsigned)(p.ntn * p.bn / rows), (unsigned)p.num_kb);
-  return launch_early(pack_f32_split_kernel, grid, 256, smem, stream, filter, base + kStatusBytes,
+  return launch_pack<pack_f32_split_kernel>(grid, 256, smem, stream, filter, base + kStatusBytes,
                       reinterpret_cast<float*>(base + kStatusBytes + p.copy_off), reinterpret_cast<uint32_t*>(base), g.C * g.Kh, g.Kw, g.Co,
                       p.bn, p.num_kb, rows, p.bn <= CONCAT_BN ? 1 : 0);
 }

@@ -2556,12 +2556,8 @@ cudaError_t launch_pack_f16_nhwc(const uint16_t* filter, void* scratch, const Ge
   if (cb > plan.Cp) cb = plan.Cp;
   const size_t smem = (size_t)cb * g.T * 2 + 32;
   if (smem > 200 * 1024) return cudaErrorInvalidValue;
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(pack_f16_nhwc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
   dim3 grid((unsigned)((plan.Cp + cb - 1) / cb), (unsigned)(g.Co < 32768 ? g.Co : 32768));
-  return launch_early(pack_f16_nhwc_kernel, grid, 256, smem, stream, filter, reinterpret_cast<uint16_t*>(base + kStatusBytes),
+  return launch_pack<pack_f16_nhwc_kernel>(grid, 256, smem, stream, filter, reinterpret_cast<uint16_t*>(base + kStatusBytes),
                       reinterpret_cast<uint32_t*>(base), reinterpret_cast<uint32_t*>(base + plan.flags_off), g.C, plan.Cp, g.Co, g.Kh,
                       g.Kw, cb);
 }

@@ -174,7 +174,7 @@ cudaError_t launch_pack_f32(const float* filter, void* scratch, const Geometry& 
                             const ScratchLayout& l, cudaStream_t stream) {
   unsigned char* base = static_cast<unsigned char*>(scratch);
   PackParams q = make_params(g, l);
-  return launch_early(pack_f32_kernel, grid_for(q.Kp * q.Co_pad), 256, 0, stream,
+  return launch_pack<pack_f32_kernel>(grid_for(q.Kp * q.Co_pad), 256, 0, stream,
       filter, reinterpret_cast<float*>(base + l.filter_off),
       reinterpret_cast<int32_t*>(base + l.koff_off), reinterpret_cast<uint32_t*>(base), q);
 }
@@ -183,7 +183,7 @@ cudaError_t launch_pack_f16(const uint16_t* filter, void* scratch, const Geometr
                             const ScratchLayout& l, cudaStream_t stream) {
   unsigned char* base = static_cast<unsigned char*>(scratch);
   PackParams q = make_params(g, l);
-  return launch_early(pack_f16_kernel, grid_for(q.Kp * q.Co), 256, 0, stream,
+  return launch_pack<pack_f16_kernel>(grid_for(q.Kp * q.Co), 256, 0, stream,
       filter, reinterpret_cast<uint16_t*>(base + l.filter_off),
       reinterpret_cast<int32_t*>(base + l.koff_off), reinterpret_cast<uint32_t*>(base), q);
 }
@@ -197,7 +197,7 @@ static cudaError_t pack_shift_common(const uint16_t* filter, void* scratch, cons
   const size_t smem = ((size_t)chunk * g.Kw + 16) * sizeof(uint16_t);
   if (smem > 48 * 1024) return cudaErrorInvalidValue;
   dim3 grid((unsigned)((q.Kp + chunk - 1) / chunk), (unsigned)(g.Co < 32768 ? g.Co : 32768));
-  return launch_early(pack_f16_shift_kernel, grid, 256, smem, stream, filter, reinterpret_cast<uint16_t*>(base + l.filter_off),
+  return launch_pack<pack_f16_shift_kernel>(grid, 256, smem, stream, filter, reinterpret_cast<uint16_t*>(base + l.filter_off),
                                                      reinterpret_cast<uint32_t*>(base + l.koff_off),
                                                      reinterpret_cast<uint32_t*>(base), q, raw_pitch, nslot, chunk);
 }

@@ -1,4 +1,4 @@
-"""Kernels that may start before the one ahead of them in the stream has ended (launch_early, launch_after_previous, or the launch
+"""Kernels that may start before the one ahead of them in the stream has ended (launch_early, launch_pack, launch_after_previous, or the launch
 attribute itself): every thread waits for that one before anything else that reads what it wrote.  A bounded barrier wait counts: its
 slow path takes its limit from the status block, which the filter pack clears, so that a wait that came first could give up on a
 word left over from whatever the memory held before, and the pack would then clear the status that says so.
@@ -12,7 +12,7 @@ import pytest
 
 from paper_2608_20725_b200 import binding, build
 
-EARLY = re.compile(r"launch_early\(|launch_after_previous\(|cudaLaunchAttributeProgrammaticStreamSerialization")
+EARLY = re.compile(r"launch_early\(|launch_pack<|launch_after_previous\(|cudaLaunchAttributeProgrammaticStreamSerialization")
 HEAD = re.compile(r"^(?:__global__ void\b.*|__device__ __forceinline__ void \w+_body\(.*|conv_\w+_kernel\(.*)$", re.M)
 
 
