@@ -250,7 +250,7 @@ __device__ __forceinline__ void issue_steps(uint32_t d, uint32_t bn, uint32_t a,
   }
 }
 
-template <int BNMAX, int PWG>
+template <int BNMAX, int PWG, bool SHARED>
 __global__ void __launch_bounds__(Form<BNMAX, PWG>::THREADS, 1) conv_f32_split_kernel(SplitParams q) {
   using F = Form<BNMAX, PWG>;
   extern __shared__ unsigned char smem_dyn[];
@@ -288,12 +288,13 @@ __global__ void __launch_bounds__(Form<BNMAX, PWG>::THREADS, 1) conv_f32_split_k
   const uint32_t tmem_acc = tmem_base_slot;
   wait_for_previous_kernel();
 
-  // Work: tile w = position tile * channel tiles + channel tile.  split = 1: the CTA walks tiles w, w + grid, ...;
+  // Work: tile w = position tile * channel tiles + channel tile.  Not SHARED: the CTA walks tiles w, w + grid, ...;
   // otherwise the cluster has one tile and its CTA r the stages [S r / split, S (r + 1) / split).
-  const int rank = q.split > 1 ? (int)cluster_ctarank() : 0;
-  const int w_first = q.split > 1 ? (int)blockIdx.x / q.split : (int)blockIdx.x;
-  const int w_step = q.split > 1 ? q.nwork : (int)gridDim.x;
-  const int st0 = (int)((int64_t)q.nstages * rank / q.split), st1 = (int)((int64_t)q.nstages * (rank + 1) / q.split);
+  const int rank = SHARED ? (int)cluster_ctarank() : 0;
+  const int w_first = SHARED ? (int)blockIdx.x / q.split : (int)blockIdx.x;
+  const int w_step = SHARED ? q.nwork : (int)gridDim.x;
+  const int st0 = SHARED ? (int)((int64_t)q.nstages * rank / q.split) : 0;
+  const int st1 = SHARED ? (int)((int64_t)q.nstages * (rank + 1) / q.split) : q.nstages;
   const int kb0 = st0 / q.nsub, t0 = st0 - kb0 * q.nsub;
 
   if (wg < F::PWG) {
@@ -486,7 +487,7 @@ __global__ void __launch_bounds__(Form<BNMAX, PWG>::THREADS, 1) conv_f32_split_k
       if (!ok) for (int i = 0; i < 64; ++i) __nanosleep(1000);
     }
     __syncwarp();
-    if (q.split > 1) { cluster_sync_all(); cluster_sync_all(); }
+    if (SHARED) { cluster_sync_all(); cluster_sync_all(); }
   } else {
     // ---------------- epilogue: fp32 sums of the tile in registers -------------------------------------
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(F::REGS_EPILOGUE));
@@ -566,7 +567,7 @@ __global__ void __launch_bounds__(Form<BNMAX, PWG>::THREADS, 1) conv_f32_split_k
         if (++t == q.nsub) { t = 0; ++kb; }
       }
       if (!ok) break;
-      if (q.split > 1) {
+      if constexpr (SHARED) {
         // (here and not behind the loop, where the sums would have to be live over everything below)
         const int channels = q.Co - nt * q.bn < q.bn ? q.Co - nt * q.bn : q.bn;
         const ClusterSums sums(a_ring, q.split, rank, channels);
@@ -597,7 +598,7 @@ __global__ void __launch_bounds__(Form<BNMAX, PWG>::THREADS, 1) conv_f32_split_k
         }
       }
     }
-    if (q.split > 1) {
+    if constexpr (SHARED) {
       if (!ok) { __syncwarp(); cluster_sync_all(); cluster_sync_all(); }      // (a wait gave up: the others wait for this CTA all the same)
       if (ok && valid) {
         const int co0 = nt * q.bn;
@@ -623,7 +624,7 @@ __global__ void __launch_bounds__(Form<BNMAX, PWG>::THREADS, 1) conv_f32_split_k
       }
     }
   }
-  if (wg < F::PWG && q.split > 1) {
+  if (wg < F::PWG && SHARED) {
     __syncwarp();
     cluster_sync_all();
     cluster_sync_all();
@@ -713,21 +714,32 @@ int channel_parts(int64_t tiles, int bn) {
   return 1;
 }
 
-template <int BNMAX, int PWG>
-cudaError_t launch_form(SplitParams q, int smem, cudaStream_t stream) {
+// SHARED: tiles shared by the CTAs of a cluster.  A kernel of its own: decided at run time, meeting and adding up sixteen parts cost the layers
+// that share nothing up to 9 % (5x5 on 4 -> 13 channels at 148x148, batch 128, 436 -> 461 us, 3x3 on 8 -> 50 at 195x195, batch 64, 363 -> 396).
+template <int BNMAX, int PWG, bool SHARED>
+cudaError_t launch_kernel(SplitParams q, int smem, cudaStream_t stream) {
+  constexpr auto kernel = conv_f32_split_kernel<BNMAX, PWG, SHARED>;
   static bool attr_done[64] = {};
-  static KnownClusters known;
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
   if (!attr_done[dev]) {
-    cudaError_t e = cudaFuncSetAttribute(conv_f32_split_kernel<BNMAX, PWG>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSplitSmem);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(conv_f32_split_kernel<BNMAX, PWG>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSplitSmem);
+    if (e == cudaSuccess && SHARED) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
     attr_done[dev] = true;
   }
-  if (q.split > 1) q.split = ctas_that_fit(conv_f32_split_kernel<BNMAX, PWG>, q.split, Form<BNMAX, PWG>::THREADS, kSplitSmem, known);
-  const int grid = q.split > 1 ? q.nwork * q.split : (q.nwork < 148 ? q.nwork : 148);
-  return launch_after_previous(conv_f32_split_kernel<BNMAX, PWG>, grid, q.split, Form<BNMAX, PWG>::THREADS, smem, stream, q);
+  if constexpr (SHARED) {
+    static KnownClusters known;
+    q.split = ctas_that_fit(kernel, q.split, Form<BNMAX, PWG>::THREADS, kSplitSmem, known);
+    if (q.split == 1) return launch_kernel<BNMAX, PWG, false>(q, smem, stream);
+    return launch_after_previous(kernel, q.nwork * q.split, q.split, Form<BNMAX, PWG>::THREADS, smem, stream, q);
+  }
+  return launch_after_previous(kernel, q.nwork < 148 ? q.nwork : 148, 1, Form<BNMAX, PWG>::THREADS, smem, stream, q);
+}
+
+template <int BNMAX, int PWG>
+cudaError_t launch_form(const SplitParams& q, int smem, cudaStream_t stream) {
+  return q.split > 1 ? launch_kernel<BNMAX, PWG, true>(q, smem, stream) : launch_kernel<BNMAX, PWG, false>(q, smem, stream);
 }
 
 }  // namespace
