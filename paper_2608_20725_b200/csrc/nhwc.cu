@@ -121,10 +121,6 @@ __device__ __forceinline__ void store_chunk(const EpiParams& q, int64_t base, in
 #pragma unroll
       for (int j = 0; j < 32; j += 4)
         *reinterpret_cast<uint4*>(p + j) = make_uint4(v[j], v[j + 1], v[j + 2], v[j + 3]);
-    } else if (vec_ok) {                                     // (then cnt is a multiple of four)
-#pragma unroll
-      for (int j = 0; j < 28; j += 4)
-        if (j < cnt) *reinterpret_cast<uint4*>(p + j) = make_uint4(v[j], v[j + 1], v[j + 2], v[j + 3]);
     } else {
 #pragma unroll
       for (int j = 0; j < 32; ++j)
@@ -142,10 +138,9 @@ __device__ __forceinline__ void store_chunk(const EpiParams& q, int64_t base, in
         if (j + 1 < cnt) *p1 = __float2half_rn(__uint_as_float(v[j + 1]));
         p0 += step; p1 += step;
       }
-    } else if (vec_ok) {                                     // (then cnt is a multiple of eight)
+    } else if (vec_ok && cnt == 32) {
 #pragma unroll
       for (int j = 0; j < 32; j += 8) {
-        if (j >= cnt) break;
         uint32_t w[4];
 #pragma unroll
         for (int t = 0; t < 4; ++t) {
@@ -159,6 +154,32 @@ __device__ __forceinline__ void store_chunk(const EpiParams& q, int64_t base, in
       for (int j = 0; j < 32; ++j)
         if (j < cnt) p[j] = __float2half_rn(__uint_as_float(v[j]));
     }
+  }
+}
+
+// Channel-innermost rows of a whole number of 16-byte vectors, the last 32 channels of which may be fewer: cnt is a multiple of a vector's.
+// (Beside the element-wise stores above, for rows of any length, this cost rows of whole 32 channels up to 14 %: 1x1 on 3 -> 64 channels at 160x160,
+// batch 128, binary16 rows, 203 -> 230 us.  In the ROWS kernels, which only rows that are no whole number of 32 channels take; stored an element at a
+// time those took up to 3.5 times as long: 3x3 on 3 -> 56 channels at 112x112, batch 64, binary16 rows, 218 -> 62.)
+__device__ __forceinline__ void store_vectors(const EpiParams& e, int64_t base, const uint32_t (&v)[32], int cnt) {
+  if (e.out16) {
+    __half* p = reinterpret_cast<__half*>(e.y) + base;
+#pragma unroll
+    for (int j = 0; j < 32; j += 8) {
+      if (j >= cnt) break;
+      uint32_t w[4];
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        const __half2 h = __floats2half2_rn(__uint_as_float(v[j + 2 * t]), __uint_as_float(v[j + 2 * t + 1]));
+        w[t] = *reinterpret_cast<const uint32_t*>(&h);
+      }
+      *reinterpret_cast<uint4*>(p + j) = make_uint4(w[0], w[1], w[2], w[3]);
+    }
+  } else {
+    float* p = reinterpret_cast<float*>(e.y) + base;
+#pragma unroll
+    for (int j = 0; j < 32; j += 4)
+      if (j < cnt) *reinterpret_cast<uint4*>(p + j) = make_uint4(v[j], v[j + 1], v[j + 2], v[j + 3]);
   }
 }
 
@@ -286,7 +307,8 @@ __device__ __forceinline__ void finish_chunk(const EpiParams& e, uint32_t (&v)[3
     for (int t = 0; t < 32; ++t) v[t] = __float_as_uint(fmaxf(__uint_as_float(v[t]), 0.0f));
   }
   if (ROWS && !add) {
-    store_rows(e, base + c0, v, cnt < 32 ? cnt : 32, valid, stage);
+    if (!vec_ok) store_rows(e, base + c0, v, cnt < 32 ? cnt : 32, valid, stage);
+    else if (valid) store_vectors(e, base + c0, v, cnt < 32 ? cnt : 32);
     return;
   }
   if (valid) store_chunk(e, base + (int64_t)c0 * cs, cs, v, cnt < 32 ? cnt : 32, vec_ok, add);
@@ -1945,15 +1967,17 @@ RunPlan plan_runs(int64_t nwork, int slots, int num_kc, int ksub, int bn) {
   return r;
 }
 
-// Whether a layer's rows are stored through shared memory: channel-innermost ones that are no whole number of 16-byte vectors.
-bool stages_rows(const EpiParams& e) { return e.y_nhwc && !e.atomic && e.Co % (e.out16 ? 8 : 4) != 0; }
+// Channel-innermost rows that are no whole number of 32 channels (the ROWS kernels), and bytes of the buffers through which they are stored if they
+// are no whole number of 16-byte vectors either.
+bool ragged_rows(const EpiParams& e) { return e.y_nhwc && !e.atomic && e.Co % 32 != 0; }
+int row_buffer_bytes(const EpiParams& e) { return ragged_rows(e) && e.Co % (e.out16 ? 8 : 4) != 0 ? kStageBytes : 0; }
 
 template <int BN, bool PAIR, int KSUB, bool ROWS>
 cudaError_t launch_variant(const CUtensorMap& amap, const CUtensorMap& bmap, const CUtensorMap& bmap_h, NhwcParams q,
                            const NhwcPlan& plan, cudaStream_t stream) {
   constexpr int B_ROWS = PAIR ? BN / 2 : BN;
   constexpr int STAGE = KSUB * (A_SLOT_BYTES + B_ROWS * KB * 2);
-  constexpr int row_buffers = ROWS ? kStageBytes : 0;
+  const int row_buffers = ROWS ? row_buffer_bytes(q.e) : 0;
   int stages = (kSmemMax - 2048 - row_buffers) / STAGE;
   if (stages > MAX_STAGES) stages = MAX_STAGES;
   if (stages < 2) return cudaErrorInvalidValue;
@@ -2141,7 +2165,7 @@ cudaError_t launch_shift_variant(const CUtensorMap& amap, const CUtensorMap& bma
                                  const ShiftViewPlan& sp, cudaStream_t stream) {
   constexpr int B_ROWS = PAIR ? BN / 2 : BN;
   constexpr int B_BYTES = B_ROWS * KB * 2;
-  constexpr int row_buffers = ROWS ? kStageBytes : 0;
+  const int row_buffers = ROWS ? row_buffer_bytes(q.e) : 0;
   const int budget = kSmemMax - 2048 - row_buffers;
   // units per filter stage: all kernel columns of a k2-block when two such stages fit beside two
   // activation stages (the MMA warp then pays two waits and two commits per block); otherwise three,
@@ -2354,7 +2378,7 @@ cudaError_t launch_shift_view(const uint16_t* window, const uint16_t* fp, void* 
   if (const char* v = debug_getenv("IM2WIN_NHWC_BU")) { const int bu = atoi(v); if (bu >= 1 && bu <= 8) { q.bu = bu; q.bu_forced = 1; } }
   // (buffers for rows where two activation stages and two of all kernel columns still fit beside them: with three columns a filter stage
   // instead, 11x11 on 62 -> 73 channels at 91x91 took 44.7 us instead of 29.7)
-  if (stages_rows(q.e) && 2 * (int64_t)sp.a_stage_bytes + 2 * (int64_t)q.Kw * b_rows * KB * 2 <= kSmemMax - 2048 - kStageBytes)
+  if (ragged_rows(q.e) && 2 * (int64_t)sp.a_stage_bytes + 2 * (int64_t)q.Kw * b_rows * KB * 2 <= kSmemMax - 2048 - row_buffer_bytes(q.e))
     return launch_shift_tile<true>(amap, bmap, bmap_h, bmap_q, q, plan, sp, stream);
   return launch_shift_tile<false>(amap, bmap, bmap_h, bmap_q, q, plan, sp, stream);
 }
@@ -2809,7 +2833,7 @@ cudaError_t launch_conv_f16_nhwc(const uint16_t* window, void* y, void* scratch,
   q.partial = plan.partial_bytes > 0 ? reinterpret_cast<float*>(base + plan.partial_off) : nullptr;
   q.epoch = next_epoch();
   if (ksub != 1) return launch_ksub<2, false>(amap, bmap, bmap_h, q, plan, stream);
-  if (stages_rows(q.e)) return launch_ksub<1, true>(amap, bmap, bmap_h, q, plan, stream);
+  if (ragged_rows(q.e)) return launch_ksub<1, true>(amap, bmap, bmap_h, q, plan, stream);
   return launch_ksub<1, false>(amap, bmap, bmap_h, q, plan, stream);
 }
 

@@ -25,6 +25,7 @@ def L(name, N, C, H, W, Co, Kh, Kw, s, p, seed):
     L("c1", 3, 8, 9, 11, 1, 3, 3, 1, 1, 700), L("c7", 2, 8, 12, 9, 7, 3, 3, 1, 0, 701), L("c9", 2, 16, 10, 10, 9, 1, 1, 1, 0, 702),
     L("c12", 2, 8, 10, 13, 12, 3, 3, 1, 1, 703), L("c20", 2, 8, 9, 13, 20, 3, 3, 1, 1, 704), L("c33", 2, 16, 7, 7, 33, 3, 3, 1, 1, 705),
     L("c63", 3, 8, 12, 12, 63, 3, 3, 1, 1, 706), L("c74", 2, 24, 11, 9, 74, 3, 3, 2, 1, 707), L("c95", 2, 8, 8, 31, 95, 3, 3, 1, 1, 708),
+    L("c24", 2, 8, 9, 11, 24, 3, 3, 1, 1, 715), L("c40", 2, 16, 10, 9, 40, 3, 3, 2, 1, 716), L("c104", 2, 8, 9, 9, 104, 3, 3, 1, 1, 717),   # whole vectors
     L("c163", 3, 8, 13, 17, 163, 3, 3, 1, 1, 709), L("c301", 2, 16, 9, 9, 301, 3, 3, 1, 1, 710),
     L("parts", 1, 8, 4, 201, 37, 3, 3, 1, 1, 711),          # strips wider than a tile
     L("rounds", 40, 8, 24, 24, 99, 3, 3, 1, 1, 712)], ids=lambda l: l.name)     # more tiles than CTAs
