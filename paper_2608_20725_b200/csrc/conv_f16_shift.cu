@@ -468,10 +468,11 @@ cudaError_t launch_variant(const CUtensorMap& fmap, const ShiftParams& q0, const
   if (SPLIT && smem_bytes < cluster_sums_bytes(BN) + 1024) smem_bytes = cluster_sums_bytes(BN) + 1024;
   const int64_t units = (plan.VQ + TILE_M - 1) / TILE_M;
   const dim3 grid((unsigned)((units - q.nbig) * q.split), (unsigned)((co + BN - 1) / BN));   // a tall tile covers two units
-  // An SM each where there is one for every tile, also where an SM could take two (spread_smem): 7x7 on 512 -> 116 channels, one 112x112 image,
-  // 221 us in twos, 169 alone; 7x5 on 128 -> 40 at 117x117 57.5 and 47.2.
-  const int64_t ctas = (int64_t)grid.x * grid.y;
-  if (!SPLIT && ctas <= 148) smem_bytes = (int)spread_smem(ctas, NUM_THREADS, (size_t)smem_bytes);
+  // An SM each where there is one for every tile, also where an SM could take two (see spread_smem): 7x7 on 512 -> 116 channels, one 112x112 image,
+  // 221 us in twos, 169 alone; 7x5 on 128 -> 40 at 117x117 57.5 and 47.2.  No more than it takes, half of an SM and a little: the gathering loads
+  // live on the cache that is left (11x11 stride 2 on 512 -> 128, one 53x53 image, 385 us, with 200 KB 460).
+  constexpr int kAlone = 115 * 1024;
+  if (!SPLIT && (int64_t)grid.x * grid.y <= 148 && smem_bytes < kAlone) smem_bytes = kAlone;
   if constexpr (!SPLIT) {
     const cudaError_t e = cudaFuncSetAttribute(conv_f16_shift_kernel<BN, ITEMS, SPLIT>,
                                                cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
