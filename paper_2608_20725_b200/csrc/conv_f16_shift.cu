@@ -493,6 +493,12 @@ cudaError_t launch_variant(const CUtensorMap& fmap, const ShiftParams& q0, const
     cfg.numAttrs = 2;
     return cudaLaunchKernelEx(&cfg, conv_f16_shift_kernel<BN, ITEMS, SPLIT>, fmap, q);
   } else {
+    // Not early where tall tiles and others share the SMs by twos: the tall ones, first in the grid, would go two to an SM (11x11 on 128 -> 64 channels at
+    // 34x12, batch 64, 78 tall of 296: 259 us early, 228 so, static weights; 7x7 on 135 -> 8 at 16x132, batch 35, 181 and 168).
+    if (BN <= 128 && q.nbig > 0 && q.nbig < (int)grid.x && (int64_t)grid.x * grid.y > 148) {
+      conv_f16_shift_kernel<BN, ITEMS, SPLIT><<<grid, NUM_THREADS, smem_bytes, stream>>>(fmap, q);
+      return cudaGetLastError();
+    }
     return launch_early(conv_f16_shift_kernel<BN, ITEMS, SPLIT>, grid, NUM_THREADS, (size_t)smem_bytes, stream, fmap, q);
   }
 }
