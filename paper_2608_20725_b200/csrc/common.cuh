@@ -28,7 +28,10 @@ struct Geometry {
 };
 
 // Clusters of z CTAs, each CTA an SM to itself, that a B200 holds at once: they lie within a GPC, so that wide ones leave SMs over.
-// (What cudaOccupancyMaxActiveClusters says of 226 KB of shared memory a CTA; 16 clusters of 8 CTAs run in two rounds: 7x7 on
+// (What cudaOccupancyMaxActiveClusters says of 226 KB of shared memory a CTA, but for threes and fives, of which it says 45 and 26: started while
+// the kernel ahead still leaves its SMs, they take those that are free, not those that fit best, and 42 and 25 are the most that never leave one for
+// a second round.  3x3 on 512 -> 64 channels, 128 positions a tile, shared by three: a pass of 42 tiles 27.2 us, of 44 32.8, of 45 37.8; by
+// five: 25 tiles 21.3, 26 27.5.  All other sizes up to their full number take the same.  16 clusters of 8 CTAs run in two rounds: 7x7 on
 // 256 -> 78 channels at 35x35, batch 2, 87 us in clusters of 8, 47 in clusters of 4.)
 // The plans go by this table, so that they do not depend on the machine; the launchers ask the device (ctas_that_fit).
 constexpr int kMaxCtas = 16;       // of a cluster (above 8: the non-portable sizes)
@@ -36,7 +39,7 @@ constexpr int kMaxCtas = 16;       // of a cluster (above 8: the non-portable si
 // so a shared reduction is the more exact one; beyond this the two would differ by more than fp32 sums in another order do.
 constexpr int64_t kMostSplitTerms = 16384;
 inline int resident_clusters(int z) {
-  constexpr int kResident[kMaxCtas + 1] = {0, 148, 74, 45, 33, 26, 22, 15, 15, 15, 11, 7, 7, 7, 7, 7, 7};
+  constexpr int kResident[kMaxCtas + 1] = {0, 148, 74, 42, 33, 25, 22, 15, 15, 15, 11, 7, 7, 7, 7, 7, 7};
   return z >= 1 && z <= kMaxCtas ? kResident[z] : 0;
 }
 

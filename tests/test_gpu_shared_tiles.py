@@ -154,6 +154,8 @@ def test_host_call_in_parts(layer):
 @pytest.mark.parametrize("layer,ctas", [
     ((27, 512, 15, 15, 128, 3, 3, 2, 1), 6),         # run-staged, 16 tiles of 24 k-blocks
     ((4, 256, 18, 18, 256, 7, 7, 2, 3), 10),         # shifted views
+    ((16, 256, 115, 10, 80, 3, 5, 2, 1), 2),         # 44 tiles: 45 clusters of three fit an idle GPU, 42 one that is being left
+    ((8, 86, 36, 36, 128, 11, 11, 2, 5), 4),         # 26 tiles, likewise 26 and 25 clusters of five
     ((1, 64, 50, 50, 104, 3, 3, 1, 0), 1),           # too little to share
     ((128, 64, 56, 56, 64, 3, 3, 1, 1), 1),          # tiles enough
     ((8, 393, 9, 20, 128, 11, 11, 2, 5), 1)])        # 47553 terms
@@ -163,6 +165,7 @@ def test_which_fp16_layers_are_shared(layer, ctas):
 
 @pytest.mark.parametrize("layer,form", [
     ((2, 256, 35, 35, 78, 7, 7, 1, 0), (48, 4)),     # 16 tiles: only 15 clusters of 8 are resident at once
+    ((2, 256, 36, 36, 23, 11, 11, 1, 5), (32, 4)),   # 26 tiles: no fives
     ((4, 512, 14, 14, 90, 11, 11, 4, 5), (16, 16)),
     ((1, 256, 8, 8, 103, 3, 3, 1, 0), (16, 12))])
 def test_which_fp32_layers_are_shared(layer, form):
