@@ -2621,8 +2621,8 @@ void part_strips(const Geometry& g, NhwcPlan& p) {
 // theirs (6.5 bytes a ps); meeting and adding up 1 to 4.  With 20 to 40 tiles, where L2 decides, and for channel-innermost outputs the estimate
 // is up to 1.6 times too good, so that it has to be 0.6 of the unshared one: without that margin 11 of 200 drawn layers lost 5 to 20 % (7x7 on
 // 128 -> 16 channels at 10x37, batch 8, 13.5 / 16.6, 11x11 on 64 -> 77 at 19x19, batch 32, 20.8 / 23.1), with it none of 300 more than 3 %.
-// Unshared / shared: 7x7 stride 4 on 163 -> 32 channels at 28x28, batch 2, 35.9 / 7.5, 3x3 stride 2 on 512 -> 28 at 15x15 22.5 / 6.4, 7x7 on
-// 512 -> 64 at 33x33, batch 8, 103 / 17.8.  3x3 on 64 channels of one 56x56 image stays unshared (6.5 / 9.4).
+// Unshared / shared: 7x7 stride 4 on 163 -> 32 channels at 28x28, batch 2, 35.9 / 7.5, 3x3 stride 2 on 512 -> 28 at 15x15 22.5 / 6.4, 7x7 stride 4
+// on 512 -> 64 at 33x33, batch 8, binary16 outputs, 103 / 16.6.  3x3 on 64 channels of one 56x56 image stays unshared (6.5 / 9.4).
 int choose_shared(const Geometry& g, const NhwcPlan& plan, const EpilogueArgs& epi, int* bn_out) {
   if (const char* v = debug_getenv("IM2WIN_NHWC_CTAS")) {    // testing aid: CTAs per tile
     *bn_out = plan.bn;
