@@ -36,12 +36,12 @@
 // Roles (one persistent CTA per SM): one or two warpgroups of producers (thread = row; 32 loads in flight,
 // split, 16-byte stores), an MMA warp, a filter-copy warp (one untiled bulk copy per piece: the pack kernel
 // writes shared-memory images), eight epilogue warps that keep the tile's fp32 sums in registers.
-// Measured against the FFMA kernel (us, filter packed beforehand): 3x3 on 64 channels at 56x56, batch 128, 543 -> 201 (147
-// TFLOP/s; no pipe above 45 % of its rate: hand-offs over two stages); 3x3 on 512 channels at 7x7 627 -> 155; 11x11 on 256
-// channels at 28x28, batch 64, 14824 -> 3930 (202 TFLOP/s; 1.6 PFLOP/s of bf16 products with the strip ends, near the
-// power limit); 7x7 stride 2 on 3 channels at 224x224 642 -> 408.
+// Measured against the FFMA kernel (us, filter packed beforehand): 3x3 on 64 channels at 56x56, batch 128, 543 -> 195 (152
+// TFLOP/s; no pipe above 45 % of its rate: hand-offs over two stages); 3x3 on 512 channels at 7x7 627 -> 158; 11x11 on 256
+// channels at 28x28, batch 64, 14824 -> 4143 in a long row, where the power limit decides (192 TFLOP/s; 1.5 PFLOP/s of bf16 products with
+// the strip ends); 7x7 stride 2 on 3 channels at 224x224 642 -> 385.
 // A layer with few tiles is run by clusters of 2 to 16 CTAs that share the stages of a tile and add their
-// registers through distributed shared memory, in rank order: 3x3 on 512 channels, one 7x7 image, 225 -> 31 us.  Any number of CTAs
+// registers through distributed shared memory, in rank order: 3x3 on 512 channels, one 7x7 image, 225 -> 16 us.  Any number of CTAs
 // whose clusters are all resident at once, sums pushed to the CTA that finishes them: against powers of two up to 8 and sums read from the
 // other CTAs, 40 layers of 1 to 90 tiles 1.13 times as fast on average (0.91 at the least): 3x5 stride 2 on 427 channels at 66x12, batch 2,
 // 35.8 -> 16.3 us, 7x7 on 256 -> 78 channels at 35x35, batch 2 (16 clusters of 8 in two rounds) 87 -> 47.
