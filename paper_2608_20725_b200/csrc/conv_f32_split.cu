@@ -37,7 +37,7 @@
 // split, 16-byte stores), an MMA warp, a filter-copy warp (one untiled bulk copy per piece: the pack kernel
 // writes shared-memory images), eight epilogue warps that keep the tile's fp32 sums in registers.
 // Measured against the FFMA kernel (us, filter packed beforehand): 3x3 on 64 channels at 56x56, batch 128, 543 -> 195 (152
-// TFLOP/s; no pipe above 45 % of its rate: hand-offs over two stages); 3x3 on 512 channels at 7x7 627 -> 158; 11x11 on 256
+// TFLOP/s; no pipe above half of its rate: hand-offs over two stages); 3x3 on 512 channels at 7x7 627 -> 158; 11x11 on 256
 // channels at 28x28, batch 64, 14824 -> 4143 in a long row, where the power limit decides (192 TFLOP/s; 1.5 PFLOP/s of bf16 products with
 // the strip ends); 7x7 stride 2 on 3 channels at 224x224 642 -> 385.
 // A layer with few tiles is run by clusters of 2 to 16 CTAs that share the stages of a tile and add their
